@@ -49,8 +49,7 @@ NCU_LIMITER = {
     "fine_fwd": "L2 -> SM read rate: 12.9 TB/s against 11.8 TB/s sustained peak (tensor pipe 82 % active at the half rate of M = 64)",
     "fine_bwd_dq": "shared-memory data pipe: tensor-core operand fetches 64 % + thread loads/stores 37 % (tensor pipe 43 %)",
     "fine_bwd_dkv": "shared-memory data pipe: tensor-core operand fetches 67 % + thread loads/stores 32 % (tensor pipe 47 %)",
-    "router_lse": "exponential unit 81 %, instruction issue 65 %",
-    "router_pool": "exponential unit 77 %, instruction issue 69 %",
+    "router_pool": "exponential unit (one ex2 per score): about three quarters busy",
 }
 # L2 -> SM read rate that ncu reports as the sustained peak of this part (derived__lts__lts2xbar_bytes.sum.peak_sustained
 # in the 8-head capture of profiles/kernels_720p_8heads_ncu_full.md, where the fine forward itself reads 12.0 TB/s).
@@ -433,10 +432,9 @@ def run_ours(args):
     value = replicas.whole_job_throughput(flops["dense_equiv_fwd_bwd"], world, ms_step * 1e-3) / 1e12
     value_e2e = replicas.whole_job_throughput(flops["dense_equiv_fwd_bwd"], world, ms_step_e2e * 1e-3) / 1e12
     pk, pk_kind = peaks()
-    executed = flops["fine_fwd"] + flops["fine_bwd_dq_executed"] + flops["fine_bwd_dkv_executed"] + 2 * flops["router_per_pass"]
+    executed = flops["fine_fwd"] + flops["fine_bwd_dq_executed"] + flops["fine_bwd_dkv_executed"] + flops["router_per_pass"]
     kernel_flops = {"fine_fwd": flops["fine_fwd"], "fine_bwd_dq": flops["fine_bwd_dq_executed"],
-                    "fine_bwd_dkv": flops["fine_bwd_dkv_executed"], "router_lse": flops["router_per_pass"],
-                    "router_pool": flops["router_per_pass"]}
+                    "fine_bwd_dkv": flops["fine_bwd_dkv_executed"], "router_pool": flops["router_per_pass"]}
     tensor_kernels = {k: kernel_ms[k] for k in kernel_flops}
     dominant = max(tensor_kernels, key=tensor_kernels.get)
     peak_tf = pk["bf16_tflops_sustained"]

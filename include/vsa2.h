@@ -283,8 +283,8 @@ int vsa2_device_status(const void* workspace, void* cuda_stream, int32_t* status
 /* Kernel groups, for timing from outside (e.g. a benchmark) without a profiler. */
 enum {
   VSA2_KERNEL_POOL = 0,         /* vsa2_attn_fwd: cube means of Q, K, V (Eq. 1) */
-  VSA2_KERNEL_ROUTER_LSE = 1,   /* router pass 1: row log-sum-exp (Eq. 6) */
-  VSA2_KERNEL_ROUTER_POOL = 2,  /* router pass 2: softmax + G x G pooling (Eq. 6-7) */
+  VSA2_KERNEL_ROUTER_LSE = 1,   /* router pass 1: row log-sum-exp (Eq. 6); empty when the router takes one pass */
+  VSA2_KERNEL_ROUTER_POOL = 2,  /* router pass 2, or its one pass: softmax + G x G pooling (Eq. 6-7) */
   VSA2_KERNEL_SELECT = 3,       /* TopK + CSR/CSC (Eq. 8-9) */
   VSA2_KERNEL_COARSE_FWD = 4,   /* Eq. 2-3 */
   VSA2_KERNEL_FINE_FWD = 5,     /* Eq. 12 + Eq. 14 */

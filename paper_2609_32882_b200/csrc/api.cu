@@ -347,12 +347,14 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
     ProfScope ps(VSA2_KERNEL_POOL_ROUTER, st, 1);
     VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, st));
   }
-  float* pr = at<float>(workspace, rl.pr);
+  // (half-cubes of 8 sub-cubes: the kernel folds its scores itself)
+  const bool folded = wide && r.G == 8;
+  float* pr = folded ? at<float>(sel_base, lay.pr) : at<float>(workspace, rl.pr);
   if (router_tc_supported(r))
-    VSA2_CUDA(launch_router_scores_tc(r, qr, kr, at<float>(workspace, rl.lse_r), pr, status, st));
+    VSA2_CUDA(launch_router_scores_tc(r, folded, qr, kr, pr, status, st));
   else   // sub-cube counts the tensor-core kernel has no layout for (G = 1 is the VSA router of Sec. 2.1)
     VSA2_CUDA(launch_router_scores(r, qr, kr, at<float>(workspace, rl.lse_r), pr, st));
-  if (wide) {
+  if (wide && !folded) {
     g_launches += 1;
     float* pr_cube = at<float>(sel_base, lay.pr);
     VSA2_CUDA(launch_fold_scores(r, pr, pr_cube, st));

@@ -185,10 +185,11 @@ cudaError_t launch_permute(const Geo& g, const bf16* src, int heads, bool invers
 cudaError_t launch_router_scores(const Geo& g, const bf16* qr, const bf16* kr, float* lse_r, float* pr,
                                  cudaStream_t st);
 
-// tensor-core router (router_tc.cu): lse_r holds log2-domain row statistics between its two passes
+// tensor-core router (router_tc.cu), both passes in one launch; with `fold` (half-cubes of 8 sub-cubes, N even) the scores
+// come out at the level of the 128-token cubes, bit for bit what launch_fold_scores makes of the others
 bool router_tc_supported(const Geo& g);
-cudaError_t launch_router_scores_tc(const Geo& g, const bf16* qr, const bf16* kr, float* lse_r, float* pr,
-                                    StatusBlock* status, cudaStream_t st);
+cudaError_t launch_router_scores_tc(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, StatusBlock* status,
+                                    cudaStream_t st);
 
 struct SelectScratch {
   unsigned* hist;        // [BH][3][2048]

@@ -3,11 +3,15 @@
 // Q_r K_r^T * scale, pass 2 recomputes the scores, applies the softmax and pools G x G sub-blocks on chip.
 //
 // A CTA owns 128 consecutive pooled queries (128/G query cubes) of one head and streams the head's pooled
-// keys in tiles of 128 through a TMA ring; S [128 q, 128 keys] lands in tensor memory (four buffers).
+// keys twice, in tiles of 128 through a TMA ring; S [128 q, 128 keys] lands in tensor memory (four buffers).
+// Both passes over an item run in one launch: the row statistics stay in shared memory, and a problem of a few items pays the
+// start of one kernel instead of two.
 // Four compute threads own each query row, 32 key columns of every tile each (a single warp per scheduler keeps
 // the exponential unit only half busy); pass 1 merges their running (max, sum) pairs once per item.  The G
 // rows of a query cube sit in G adjacent lanes: their pooled sums are combined with warp shuffles.
-// Both passes are bound by the exponential unit (one ex2 per score), not by the tensor pipe.
+// Both passes are bound by the exponential unit (one ex2 per score: 1024 cycles per tile of ~1250), not by the tensor pipe.
+// A buffer of scores is given back as soon as they are in registers (720p, 40 heads: 3.27 -> 3.22 ms; fetching the next tile's
+// scores before a tile is worked on made it 3.58).
 #include "tc_attn.cuh"
 
 namespace vsa2 {
@@ -33,10 +37,11 @@ struct RouterMisc {
   uint64_t q_full, q_empty;
   uint64_t k_full[kRtSlots], k_empty[kRtSlots];
   uint64_t s_full[kRtBufs], s_free[kRtBufs];
-  uint64_t part_ready, part_free;   // pass 1: hand-over of part_stats
+  uint64_t part_ready, lse_ready;   // between the passes: part_stats written, row_lse2 written
   uint32_t tmem_base;
   int abort_flag;
-  float2 part_stats[kRtParts - 1][128];   // pass 1: (running max, running sum) of the threads of parts 1 .. kRtParts-1
+  float2 part_stats[kRtParts - 1][128];   // (running max, running sum) of the threads of parts 1 .. kRtParts-1
+  float row_lse2[128];                    // log2 sum_{valid keys} 2^(s * scale * log2 e) of the item's rows
 };
 
 // tensor map over pooled operands [BH, N*G, D] bf16: box = 64 channels x 128 rows x 1
@@ -59,11 +64,72 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* m, uin
       : "memory");
 }
 
-// PASS 1 writes lse2[b, hq, row] = log2 sum_{valid keys} 2^(s * scale * log2 e);  PASS 2 writes P_r.
-template <int D, int PASS, int G>
+// Pass 1 on 32 scores of a row: running maximum (in the exponent's units) and sum.  The maximum is taken over the raw scores
+// (the scale is positive) and the scale folded into the exponent's multiply-add.
+__device__ __forceinline__ void rt_accumulate(uint32_t (&s)[32], uint32_t kbits, float c2, float& m_run, float& l_run) {
+  float cmax = -INFINITY;
+#pragma unroll
+  for (int c = 0; c < 32; ++c) {
+    if (kbits != 0xffffffffu && !((kbits >> c) & 1u)) s[c] = 0xff800000u;      // -inf
+    cmax = fmaxf(cmax, __uint_as_float(s[c]));
+  }
+  if (cmax > -INFINITY) {
+    const float m_new = fmaxf(m_run, cmax * c2);
+    float acc = 0.f;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) acc += ex2_approx(fmaf(__uint_as_float(s[c]), c2, -m_new));
+    l_run = l_run * ex2_approx(m_run - m_new) + acc;
+    m_run = m_new;
+  }
+}
+
+// Pass 2 on 32 scores of a row: softmax, column sums of the 32 / G key cubes, then the sum over the G rows of the query cube,
+// which sit in G adjacent lanes: a butterfly that halves the values a lane carries at every step (4 shuffles instead of
+// 3 per key cube) and leaves each total in one lane -- that of cube `mine` of the 32 / G.
+template <int G>
+__device__ __forceinline__ float rt_pool(const uint32_t (&s)[32], uint32_t kbits, float c2, float lse2, int lane, int& mine) {
+  static_assert(G == 8 || G == 16, "router pooling layout");
+  float p[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) {
+    p[c] = ex2_approx(fmaf(__uint_as_float(s[c]), c2, -lse2));
+    if (kbits != 0xffffffffu) p[c] = ((kbits >> c) & 1u) ? p[c] : 0.f;
+  }
+  float tv[32 / G];
+#pragma unroll
+  for (int cc = 0; cc < 32 / G; ++cc) {
+    float tot = 0.f;
+#pragma unroll
+    for (int c = 0; c < G; ++c) tot += p[cc * G + c];
+    tv[cc] = tot;
+  }
+  float t;
+  if constexpr (G == 8) {
+    const bool hi4 = lane & 4, hi2 = lane & 2;
+    const float k0 = hi4 ? tv[2] : tv[0], k1 = hi4 ? tv[3] : tv[1];
+    const float s0 = hi4 ? tv[0] : tv[2], s1 = hi4 ? tv[1] : tv[3];
+    const float u0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 4), u1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 4);
+    t = (hi2 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, hi2 ? u0 : u1, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    mine = (hi4 ? 2 : 0) + (hi2 ? 1 : 0);
+  } else {
+    const bool hi8 = lane & 8;
+    t = (hi8 ? tv[1] : tv[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? tv[0] : tv[1], 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 4);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    mine = hi8 ? 1 : 0;
+  }
+  return t;
+}
+
+// Writes P_r of the blocks of `g` or, with FOLD (G = 8), of the 128-token cubes whose half-cubes those blocks are: the scores of the
+// four pairs of halves, weighted with the valid query sub-cubes of each half (wide_cube.cu, fold_scores_kernel).
+template <int D, int G, bool FOLD>
 __global__ void __launch_bounds__(kRtThreads, 1)
 router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, Geo g,
-                 float* __restrict__ lse2, float* __restrict__ pr, StatusBlock* status) {
+                 float* __restrict__ pr, StatusBlock* status) {
+  static_assert(!FOLD || G == 8, "half-cubes of 8 sub-cubes");
   using C = RouterTc<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -79,13 +145,10 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   const float c2 = g.scale * 1.4426950408889634f;
 
   // validity of every pooled token of the sequence (a sub-cube that is padding only is invalid)
-  for (int w = tid; w < valid_words; w += blockDim.x) {
-    uint32_t bits = 0u;
-    for (int bit = 0; bit < 32; ++bit) {
-      const int r = w * 32 + bit;
-      if (r < NG && subcube_count(g, r / g.G, r % g.G) > 0) bits |= 1u << bit;
-    }
-    valid_bits[w] = bits;
+  for (int w = warp; w < valid_words; w += blockDim.x >> 5) {       // (a warp per word, a lane per token)
+    const int r = w * 32 + lane;
+    const uint32_t bits = __ballot_sync(0xffffffffu, r < NG && subcube_count(g, r / G, r % G) > 0);
+    if (lane == 0) valid_bits[w] = bits;
   }
   if (tid == 0) {
     misc->abort_flag = 0;
@@ -97,10 +160,10 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
     for (int s = 0; s < kRtBufs; ++s) {
       tc::mbar_init(&misc->s_full[s], 1);
-      tc::mbar_init(&misc->s_free[s], 128 * kRtParts);
+      tc::mbar_init(&misc->s_free[s], 4 * kRtParts);       // one arrival per compute warp
     }
     tc::mbar_init(&misc->part_ready, 128 * (kRtParts - 1));
-    tc::mbar_init(&misc->part_free, 128);
+    tc::mbar_init(&misc->lse_ready, 128);
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_k);
@@ -123,7 +186,8 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         VSA2_WAIT(&misc->q_empty, (n_items & 1) ^ 1);
         tc::mbar_expect_tx(&misc->q_full, C::TILE);
         for (int h = 0; h < C::DH; ++h) tma_load_3d(q_tile + h * C::HALF, &tm_q, &misc->q_full, h * 64, rt * kRtTile, bhq);
-        for (int kt = 0; kt < row_tiles; ++kt, ++seq) {
+        for (int step = 0; step < 2 * row_tiles; ++step, ++seq) {       // pass 1, then pass 2
+          const int kt = step < row_tiles ? step : step - row_tiles;
           const uint32_t slot = seq % kRtSlots, par = (seq / kRtSlots) & 1;
           VSA2_WAIT(&misc->k_empty[slot], par ^ 1);
           tc::mbar_expect_tx(&misc->k_full[slot], C::TILE);
@@ -139,7 +203,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       uint32_t seq = 0, n_items = 0;
       for (int item = blockIdx.x; item < total_items; item += gridDim.x, ++n_items) {
         VSA2_WAIT(&misc->q_full, n_items & 1);
-        for (int kt = 0; kt < row_tiles; ++kt, ++seq) {
+        for (int step = 0; step < 2 * row_tiles; ++step, ++seq) {
           const uint32_t slot = seq % kRtSlots, buf = seq % kRtBufs;
           VSA2_WAIT(&misc->k_full[slot], (seq / kRtSlots) & 1);
           VSA2_WAIT(&misc->s_free[buf], ((seq / kRtBufs) & 1) ^ 1);
@@ -154,124 +218,90 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           }
           tc::mma_commit(&misc->s_full[buf]);
           tc::mma_commit(&misc->k_empty[slot]);
-          if (kt == row_tiles - 1) tc::mma_commit(&misc->q_empty);
+          if (step == 2 * row_tiles - 1) tc::mma_commit(&misc->q_empty);
         }
       }
     }
   } else {
     const int quad = warp & 3;                   // tensor-memory lane quadrant of this warp
-    const int part = (warp - 2) >> 2;            // which 128 / kRtParts key columns of every tile
+    const int part = (warp - 2) >> 2;            // which 32 key columns of every tile
     const int row = (quad << 5) | lane;
-    const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + part * 32;
     uint32_t seq = 0, n_items = 0;
+    // this thread's 32 scores of tile `seq`
+    uint32_t s[32];
+    auto fetch = [&]() -> bool {
+      const uint32_t buf = seq % kRtBufs;
+      if (!tc::mbar_wait(&misc->s_full[buf], (seq / kRtBufs) & 1, &misc->abort_flag)) return false;
+      tc::tc_fence_after();
+      tc::tmem_ld32(lane_addr + buf * 128, s);
+      tc::tmem_ld_wait();
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&misc->s_free[buf]);
+      ++seq;
+      return true;
+    };
     for (int item = blockIdx.x; item < total_items; item += gridDim.x, ++n_items) {
       const int rt = item % row_tiles, bhq = item / row_tiles;
       const int r = rt * kRtTile + row;                          // pooled query index inside the head
       const bool q_valid = (valid_bits[r >> 5] >> (r & 31)) & 1u;
       float m_run = -INFINITY, l_run = 0.f;
-      float my_lse2 = 0.f, inv_norm = 0.f;
-      if (PASS == 2) {
-        my_lse2 = q_valid ? lse2[(size_t)bhq * NG + r] : INFINITY;          // +inf => p = 0 for padding rows
-        const uint32_t vb = __ballot_sync(0xffffffffu, q_valid);
-        const int gi = __popc((vb >> (lane & ~(G - 1))) & ((G == 32) ? 0xffffffffu : ((1u << G) - 1u)));
-        inv_norm = gi > 0 ? 1.f / ((float)gi * (float)G) : 0.f;
+      for (int kt = 0; kt < row_tiles; ++kt) {
+        if (!fetch()) goto done;
+        rt_accumulate(s, valid_bits[kt * 4 + part], c2, m_run, l_run);
       }
-      const int qi = r / G;                                       // query cube of this row
-      for (int kt = 0; kt < row_tiles; ++kt, ++seq) {
-        const uint32_t buf = seq % kRtBufs;
-        VSA2_WAIT(&misc->s_full[buf], (seq / kRtBufs) & 1);
-        tc::tc_fence_after();
+      // merge the four column quarters of the row
+      if (part > 0) {
+        misc->part_stats[part - 1][row] = make_float2(m_run, l_run);
+        tc::mbar_arrive(&misc->part_ready);
+      } else {
+        VSA2_WAIT(&misc->part_ready, n_items & 1);
+        float2 o[kRtParts - 1];
+        float m_new = m_run;
 #pragma unroll
-        for (int ch = part * (4 / kRtParts); ch < (part + 1) * (4 / kRtParts); ++ch) {
-          uint32_t s[32];
-          tc::tmem_ld32(lane_addr + buf * 128 + ch * 32, s);
-          tc::tmem_ld_wait();
-          const uint32_t kbits = valid_bits[kt * 4 + ch];
-          if (PASS == 1) {
-            // the maximum is taken over the raw scores (the scale is positive) and the scale folded into the exponent's
-            // multiply-add: four instructions per score instead of five (both passes are issue- and exponential-bound)
-            float cmax = -INFINITY;
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              if (kbits != 0xffffffffu && !((kbits >> c) & 1u)) s[c] = 0xff800000u;      // -inf
-              cmax = fmaxf(cmax, __uint_as_float(s[c]));
-            }
-            if (cmax > -INFINITY) {
-              const float m_new = fmaxf(m_run, cmax * c2);
-              float acc = 0.f;
-#pragma unroll
-              for (int c = 0; c < 32; ++c) acc += ex2_approx(fmaf(__uint_as_float(s[c]), c2, -m_new));
-              l_run = l_run * ex2_approx(m_run - m_new) + acc;
-              m_run = m_new;
-            }
-          } else {
-            // softmax, then G x G pooling: G columns in registers, G rows across adjacent lanes
-            float p[32];
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              p[c] = ex2_approx(fmaf(__uint_as_float(s[c]), c2, -my_lse2));
-              if (kbits != 0xffffffffu) p[c] = ((kbits >> c) & 1u) ? p[c] : 0.f;
-            }
-            // Column sums of the 32 / G key cubes of the chunk, then the sum over the G rows of the query cube, which sit in
-            // G adjacent lanes: a butterfly that halves the values a lane carries at every step (4 shuffles instead of
-            // 3 per key cube; the passes are bound by instruction issue) and leaves each total in one lane.
-            static_assert(G == 8 || G == 16, "router pooling layout");
-            float tv[32 / G];
-#pragma unroll
-            for (int cc = 0; cc < 32 / G; ++cc) {
-              float tot = 0.f;
-#pragma unroll
-              for (int c = 0; c < G; ++c) tot += p[cc * G + c];
-              tv[cc] = tot;
-            }
-            float t;
-            int cc_mine;
-            if constexpr (G == 8) {
-              const bool hi4 = lane & 4, hi2 = lane & 2;
-              const float k0 = hi4 ? tv[2] : tv[0], k1 = hi4 ? tv[3] : tv[1];
-              const float s0 = hi4 ? tv[0] : tv[2], s1 = hi4 ? tv[1] : tv[3];
-              const float u0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 4), u1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 4);
-              t = (hi2 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, hi2 ? u0 : u1, 2);
-              t += __shfl_xor_sync(0xffffffffu, t, 1);
-              cc_mine = (hi4 ? 2 : 0) + (hi2 ? 1 : 0);
-            } else {
-              const bool hi8 = lane & 8;
-              t = (hi8 ? tv[1] : tv[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? tv[0] : tv[1], 8);
-              t += __shfl_xor_sync(0xffffffffu, t, 4);
-              t += __shfl_xor_sync(0xffffffffu, t, 2);
-              t += __shfl_xor_sync(0xffffffffu, t, 1);
-              cc_mine = hi8 ? 1 : 0;
-            }
-            const int kj = (kt * kRtTile + ch * 32) / G + cc_mine;
-            const bool owner = G == 8 ? !(lane & 1) : !(lane & 7);
-            if (owner && qi < g.N && kj < g.N) pr[((size_t)bhq * g.N + qi) * g.N + kj] = t * inv_norm;
-          }
+        for (int pp = 0; pp < kRtParts - 1; ++pp) {
+          o[pp] = misc->part_stats[pp][row];
+          m_new = fmaxf(m_new, o[pp].x);
         }
-        tc::tc_fence_before();
-        tc::mbar_arrive(&misc->s_free[buf]);
+        if (m_new > -INFINITY) {
+          l_run *= ex2_approx(m_run - m_new);
+#pragma unroll
+          for (int pp = 0; pp < kRtParts - 1; ++pp) l_run += o[pp].y * ex2_approx(o[pp].x - m_new);
+        }
+        misc->row_lse2[row] = (l_run > 0.f) ? m_new + __log2f(l_run) : 0.f;
+        tc::mbar_arrive(&misc->lse_ready);
       }
-      if (PASS == 1) {
-        // merge the two column halves of the row
-        if (part > 0) {
-          VSA2_WAIT(&misc->part_free, (n_items & 1) ^ 1);
-          misc->part_stats[part - 1][row] = make_float2(m_run, l_run);
-          tc::mbar_arrive(&misc->part_ready);
+      VSA2_WAIT(&misc->lse_ready, n_items & 1);
+      // (part_stats and row_lse2 need no barrier of their own for their next item: parts 1.. write the former after this wait, which
+      //  part 0 has let pass after reading it; part 0 writes the latter after part_ready, on which every reader arrives later)
+      const float my_lse2 = q_valid ? misc->row_lse2[row] : INFINITY;          // +inf => p = 0 for padding rows
+      const uint32_t vb = __ballot_sync(0xffffffffu, q_valid);
+      const int gi = __popc((vb >> (lane & ~(G - 1))) & ((1u << G) - 1u));     // valid rows of the query block
+      const float inv_norm = gi > 0 ? 1.f / ((float)gi * (float)G) : 0.f;
+      const int qi = r / G;                                      // query block of this row
+      const int n_out = FOLD ? g.N / 2 : g.N;
+      float* out = pr + ((size_t)bhq * n_out + (FOLD ? qi >> 1 : qi)) * n_out;
+      float w0 = 0.f, w1 = 0.f;
+      if (FOLD) {
+        const int other = __shfl_xor_sync(0xffffffffu, gi, 8), vq0 = lane & 8 ? other : gi, vq1 = lane & 8 ? gi : other;
+        w0 = (float)vq0 / (float)(2 * (vq0 + vq1));
+        w1 = (float)vq1 / (float)(2 * (vq0 + vq1));
+      }
+      for (int kt = 0; kt < row_tiles; ++kt) {
+        if (!fetch()) goto done;
+        int mine;
+        const float t = rt_pool<G>(s, valid_bits[kt * 4 + part], c2, my_lse2, lane, mine);
+        const int kj = (kt * kRtTile + part * 32) / G + mine;
+        if constexpr (FOLD) {
+          // a lane holds one of the two key halves (lane bit 1) of one of the two query halves (lane bit 3) of a cube pair
+          const float v = t * inv_norm;
+          const float both = v + __shfl_xor_sync(0xffffffffu, v, 2);
+          const float low = __shfl_xor_sync(0xffffffffu, both, 8);
+          if (!(lane & 11) && qi < g.N && kj < g.N) out[kj >> 1] = w0 * both + w1 * low;
         } else {
-          VSA2_WAIT(&misc->part_ready, n_items & 1);
-          float2 o[kRtParts - 1];
-          float m_new = m_run;
-#pragma unroll
-          for (int pp = 0; pp < kRtParts - 1; ++pp) {
-            o[pp] = misc->part_stats[pp][row];
-            m_new = fmaxf(m_new, o[pp].x);
-          }
-          tc::mbar_arrive(&misc->part_free);
-          if (m_new > -INFINITY) {
-            l_run *= ex2_approx(m_run - m_new);
-#pragma unroll
-            for (int pp = 0; pp < kRtParts - 1; ++pp) l_run += o[pp].y * ex2_approx(o[pp].x - m_new);
-          }
-          if (r < NG) lse2[(size_t)bhq * NG + r] = (l_run > 0.f) ? m_new + __log2f(l_run) : 0.f;
+          const bool owner = G == 8 ? !(lane & 1) : !(lane & 7);
+          if (owner && qi < g.N && kj < g.N) out[kj] = t * inv_norm;
         }
       }
     }
@@ -294,42 +324,36 @@ done:
 
 bool router_tc_supported(const Geo& g) { return g.G == 8 || g.G == 16; }
 
-cudaError_t launch_router_scores_tc(const Geo& g, const bf16* qr, const bf16* kr, float* lse_r, float* pr,
-                                    StatusBlock* status, cudaStream_t st) {
-  const int NG = g.N * g.G;
-  CUtensorMap tq, tk;
-  if (!make_pooled_tmap(&tq, qr, g.D, NG, g.batch * g.Hq) || !make_pooled_tmap(&tk, kr, g.D, NG, g.batch * g.Hkv))
-    return cudaErrorInvalidValue;
+template <int D, int G, bool FOLD>
+static cudaError_t launch_router(const CUtensorMap& tq, const CUtensorMap& tk, const Geo& g, float* pr, StatusBlock* status,
+                                 cudaStream_t st) {
+  const int row_tiles = (g.N * G + kRtTile - 1) / kRtTile;
+  const size_t smb = RouterTc<D>::smem_bytes(row_tiles * kRtTile / 32);
+  if (smb > 227 * 1024) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const int row_tiles = (NG + kRtTile - 1) / kRtTile;
+  if ((e = cudaFuncSetAttribute(router_tc_kernel<D, G, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
   const int total = g.batch * g.Hq * row_tiles;
-  const int grid = total < sms ? total : sms;
-  const int valid_words = row_tiles * kRtTile / 32;
-#define VSA2_ROUTER_LAUNCH(DD, GG)                                                                                     \
-  do {                                                                                                               \
-    const size_t smb = RouterTc<DD>::smem_bytes(valid_words);                                                        \
-    if (smb > 227 * 1024) return cudaErrorInvalidValue;                                                              \
-    if ((e = cudaFuncSetAttribute(router_tc_kernel<DD, 1, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e; \
-    if ((e = cudaFuncSetAttribute(router_tc_kernel<DD, 2, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e; \
-    {                                                                                                                \
-      ProfScope ps(VSA2_KERNEL_ROUTER_LSE, st, 1);                                                                   \
-      router_tc_kernel<DD, 1, GG><<<grid, kRtThreads, smb, st>>>(tq, tk, g, lse_r, pr, status);                          \
-    }                                                                                                                \
-    {                                                                                                                \
-      ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);                                                                  \
-      router_tc_kernel<DD, 2, GG><<<grid, kRtThreads, smb, st>>>(tq, tk, g, lse_r, pr, status);                          \
-    }                                                                                                                \
-  } while (0)
-  if (g.D == 128 && g.G == 8) VSA2_ROUTER_LAUNCH(128, 8);
-  else if (g.D == 128 && g.G == 16) VSA2_ROUTER_LAUNCH(128, 16);
-  else if (g.D == 64 && g.G == 8) VSA2_ROUTER_LAUNCH(64, 8);
-  else if (g.D == 64 && g.G == 16) VSA2_ROUTER_LAUNCH(64, 16);
-  else return cudaErrorInvalidValue;
-#undef VSA2_ROUTER_LAUNCH
+  { ProfScope lse(VSA2_KERNEL_ROUTER_LSE, st, 0); }      // (both passes are timed as the second)
+  ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);
+  router_tc_kernel<D, G, FOLD><<<total < sms ? total : sms, kRtThreads, smb, st>>>(tq, tk, g, pr, status);
   return cudaGetLastError();
+}
+
+cudaError_t launch_router_scores_tc(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, StatusBlock* status,
+                                    cudaStream_t st) {
+  const int NG = g.N * g.G;
+  CUtensorMap tq, tk;
+  if (!make_pooled_tmap(&tq, qr, g.D, NG, g.batch * g.Hq) || !make_pooled_tmap(&tk, kr, g.D, NG, g.batch * g.Hkv))
+    return cudaErrorInvalidValue;
+  if (fold && g.G != 8) return cudaErrorInvalidValue;
+  if (g.D == 128 && g.G == 8) return fold ? launch_router<128, 8, true>(tq, tk, g, pr, status, st) : launch_router<128, 8, false>(tq, tk, g, pr, status, st);
+  if (g.D == 128 && g.G == 16) return launch_router<128, 16, false>(tq, tk, g, pr, status, st);
+  if (g.D == 64 && g.G == 8) return fold ? launch_router<64, 8, true>(tq, tk, g, pr, status, st) : launch_router<64, 8, false>(tq, tk, g, pr, status, st);
+  if (g.D == 64 && g.G == 16) return launch_router<64, 16, false>(tq, tk, g, pr, status, st);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace vsa2
