@@ -69,26 +69,16 @@ __global__ void __launch_bounds__(256) dkv_list_items_kernel(Geo g, const int* _
   if (in) list[1 + base + __popc(m & ((1u << lane) - 1u))] = item;
 }
 
-// scheduler of a launch that walks an item list: publish_ahead of tc_attn.cuh with the list in between
-__device__ __forceinline__ bool dkv_publish_listed(ItemQueue* q, uint32_t seq, uint32_t& published, int* counter,
-                                                   const int* list, volatile int* abort_flag) {
-  while (published <= seq + kItemAhead) {
-    const uint32_t slot = published % kItemSlots, par = ((published / kItemSlots) & 1) ^ 1;
-    if (!tc::mbar_wait_parked(&q->empty[slot], par, abort_flag)) return false;
-    const int it = atomicAdd(counter, 1);
-    q->item[slot] = it < list[0] ? list[1 + it] : -1;
-    tc::mbar_arrive(&q->full[slot]);
-    ++published;
-  }
-  return true;
-}
-
 // Roles: warp 0 = TMA producer of the Q pairs (ring A) and of the stationary K and V tiles, warp 1 = TMA producer of the
 // dO pairs (ring B), warp 2 = issuer of S = Q_pair K^T, warp 3 = issuer of dP = dO_pair V^T, warp 16 = issuer of
 // dV^T += dO_pair^T P (frees the dO slot), warp 17 = issuer of dK^T += Q_pair^T dS (frees the Q slot), warps 4..11 =
-// elementwise stage + epilogue (each half of the key columns): P is handed to the dV^T product before dS is formed;
+// elementwise stage (each half of the key columns): P is handed to the dV^T product before dS is formed;
 // warps 12..15 = one thread per query row of the tile: they look up the row's (head, block, token) and fetch its lse and
-// delta one tile ahead, so that the elementwise warps, which bound the pass, touch no global memory inside a tile.
+// delta one tile ahead, so that the elementwise warps, which bound the pass, touch no global memory inside a tile; warp 18 =
+// scheduler (BwdQueue); warps 20..23 = epilogue.  The accumulators of dK^T and dV^T exist twice (without SPLIT), so the
+// elementwise warps go from one KV block to the next while the epilogue warps read out and store the last one: with
+// the epilogue on the elementwise warps, 9200 of 85000 cycles of a 720p item (top-64) went by between its last tile and the
+// first of the next item (clock64 trace: 3900 epilogue, 3200 fetching the next item's record and lists, 2100 waits).
 // SPLIT: P and dS are handed to the dV^T and dK^T products as [bf16(X) | bf16(X - bf16(X))] (N = 128 products into two
 // accumulator halves that the epilogue adds), which removes their bf16 rounding from dV and dK: a KV block sums hundreds of
 // query blocks (times the query heads of a GQA group), and with plain bf16 operands that noise alone passes 2e-2.  The two
@@ -112,7 +102,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                        const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot, Geo g,
                        DkvArgs a) {
   constexpr int RA = SPLIT ? 2 : kRingA;                   // slots of the Q ring
-  constexpr uint32_t TM_DK = 256, TM_DV = SPLIT ? 384 : 320;
+  // accumulators: without SPLIT two sets of dK^T, dV^T (64 columns each), used by item parity
+  constexpr uint32_t TM_DK = 256, TM_DV = SPLIT ? 384 : 320, TM_SET = 128, SETS = SPLIT ? 1 : 2;
   using C = BwdTc<D, RA, SPLIT ? 4 : 2>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -123,7 +114,6 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   BwdMisc* misc = reinterpret_cast<BwdMisc*>(smem + C::OFF_MISC);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int total_items = g.batch * g.Hkv * g.N;
   const float c2 = g.scale * 1.4426950408889634f;
   const int rep = MHA ? 1 : g.rep;
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
@@ -134,8 +124,11 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   if (SPLIT && a.item_list != nullptr) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     bwd_init_barriers(misc);
-    tc::mbar_init(&misc->o_full, 2);                                          // two last-stage issuers
-    item_queue_init(&misc->items, 2 + 4 + 256 + 128);
+    for (int s = 0; s < 2; ++s) {
+      tc::mbar_init(&misc->o_full[s], 2);                                     // two last-stage issuers
+      tc::mbar_init(&misc->o_empty[s], 4);                                    // the epilogue warps
+    }
+    bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4);
     for (int s = 0; s < kRingB; ++s) tc::mbar_init(&misc->b_empty[s], 2);     // a dO slot is read by dP and by dV^T
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
@@ -151,47 +144,41 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
-  // tensor-memory columns: S buffers 0, 64; dP buffers 128, 192; dK^T 256; dV^T 320 (SPLIT: dK^T 256 + 320, dV^T 384 + 448)
+  // tensor-memory columns: S buffers 0, 64; dP buffers 128, 192; dK^T 256, dV^T 320 and 384, 448 (SPLIT: dK^T 256 + 320,
+  // dV^T 384 + 448)
 
-  // per item: prefix of the per-head column counts and the list starts (every role recomputes them)
+  // per item, for the roles that walk the list: prefix of the per-head column counts and the list starts
 #define VSA2_DKV_ITEM_SETUP()                                                            \
-  int j, bhk;                                                                            \
-  item_block(g, item, bhk, j);                                                           \
+  const int j = rec.x, bhk = rec.y, k = rec.z;                                           \
   const int b = bhk / g.Hkv, hk = bhk % g.Hkv;                                           \
   int cnt_prefix[(MHA ? 1 : kMaxRep) + 1], col_beg[MHA ? 1 : kMaxRep];                   \
   cnt_prefix[0] = 0;                                                                     \
-  for (int hh = 0; hh < rep; ++hh) {                                                     \
-    const size_t base_ = (size_t)(b * g.Hq + hk * rep + hh) * (g.N + 1) + j;             \
-    col_beg[hh] = a.col_ptr[base_];                                                      \
-    cnt_prefix[hh + 1] = cnt_prefix[hh] + (a.col_ptr[base_ + 1] - col_beg[hh]);          \
-  }                                                                                      \
-  const int k = cnt_prefix[rep];
+  col_beg[0] = rec.w;                                                                    \
+  if (MHA) {                                                                             \
+    cnt_prefix[1] = k;                                                                   \
+  } else {                                                                               \
+    for (int hh = 0; hh < rep; ++hh) {                                                   \
+      const size_t base_ = (size_t)(b * g.Hq + hk * rep + hh) * (g.N + 1) + j;           \
+      col_beg[hh] = a.col_ptr[base_];                                                    \
+      cnt_prefix[hh + 1] = cnt_prefix[hh] + (a.col_ptr[base_ + 1] - col_beg[hh]);        \
+    }                                                                                    \
+  }
 
-  if (warp < 2) {
+  // (registers: the launch allocates 80 a thread; the elementwise and epilogue warps take what the service warps leave)
+  if (warp < 4) {
+    tc::reg_dec<48>();
+    if (warp < 2) {
     // ------------------------------------------------------------------ TMA producers
     const int which = warp;                               // 0: Q pairs (ring A) + K, V tiles; 1: dO pairs (ring B)
     const CUtensorMap* tm = which == 0 ? &tm_q : &tm_do;
     const CUtensorMap* tm_text = which == 0 ? &tm_qt : &tm_dot;
     const int my_blk = lane & 1;
-    uint32_t tg = 0, n_items = 0, published = 0;
+    uint32_t tg = 0, n_items = 0;
     for (uint32_t seq = 0;; ++seq) {
-      // warp 0, lane 0 is the CTA's scheduler
-      int item = 0;
-      if (lane == 0) {
-        bool pub_ok = true;
-        if (which == 0) {
-          if (SPLIT && a.item_list != nullptr)
-            pub_ok = dkv_publish_listed(&misc->items, seq, published, a.item_counter, a.item_list, &misc->abort_flag);
-          else
-            pub_ok = item_publish_ahead(&misc->items, seq, published, a.item_counter, total_items, &misc->abort_flag);
-        }
-        item = pub_ok ? item_get(&misc->items, seq, &misc->abort_flag) : -2;
-      }
-      item = __shfl_sync(0xffffffffu, item, 0);
-      if (item == -2) goto done;
-      if (item < 0) break;
+      VSA2_NEXT_REC(rec, seq);
+      if (warp == 0 && lane == 0) tc::mbar_arrive(&misc->queue.taken);
+      if (rec.z == 0) continue;
       VSA2_DKV_ITEM_SETUP();
-      if (k == 0 || k < a.k_lo || k > a.k_hi) continue;
       if (which == 0) {
         int c1, c2, c3;
         block_box(g, j, c1, c2, c3);
@@ -222,7 +209,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         else VSA2_RING_LOAD(misc->b_full, misc->b_empty, kRingB, smem + C::OFF_RING_B, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
       }
     }
-  } else if (warp == 2 || warp == 3) {
+    } else {
     // ------------------------------------------------------------------ issuers of S = Q_pair K^T (warp 2) and
     // dP = dO_pair V^T (warp 3); whole warp in the loop, one elected lane issues (see the dQ pass)
     {
@@ -230,11 +217,9 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const uint32_t b_addr = tc::smem_u32(is_s ? k_tile : v_tile), base = tc::smem_u32(smem);
       uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        VSA2_NEXT_ITEM_WARP(item, seq);
-        VSA2_DKV_ITEM_SETUP();
-        (void)b; (void)hk; (void)j; (void)bhk; (void)col_beg;
-        if (k == 0 || k < a.k_lo || k > a.k_hi) continue;
-        const int nt = (k + 1) >> 1;
+        VSA2_NEXT_REC(rec, seq);
+        if (rec.z == 0) continue;
+        const int nt = (rec.z + 1) >> 1;
         VSA2_WAIT_PARKED(&misc->st_full, n_items & 1);
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t sb = tg & 1, pb = (tg >> 1) & 1;
@@ -264,7 +249,13 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         ++n_items;
       }
     }
-  } else if (warp == 16 || warp == 17) {
+    }
+  } else if (warp >= 16 && warp < 20) {
+    tc::reg_dec<48>();
+    if (warp == 18 && !bwd_schedule(&misc->queue, g, g.Hkv, rep, a.col_ptr, a.item_counter, SPLIT ? a.item_list : nullptr, a.k_lo,
+                                    a.k_hi, lane, &misc->abort_flag))
+      goto done;
+    if (warp < 18) {
     // ------------------------------------------------------------------ issuers of dV^T += dO_pair^T P (warp 16) and
     // dK^T += Q_pair^T dS (warp 17); whole warp in the loop, one elected lane issues
     {
@@ -272,12 +263,11 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const uint32_t b_addr = tc::smem_u32(is_v ? p_tile : ds_tile), base = tc::smem_u32(smem);
       uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        VSA2_NEXT_ITEM_WARP(item, seq);
-        VSA2_DKV_ITEM_SETUP();
-        (void)b; (void)hk; (void)j; (void)bhk; (void)col_beg;
-        if (k == 0 || k < a.k_lo || k > a.k_hi) continue;
-        const int nt = (k + 1) >> 1;
-        VSA2_WAIT_PARKED(&misc->o_empty, (n_items & 1) ^ 1);
+        VSA2_NEXT_REC(rec, seq);
+        if (rec.z == 0) continue;
+        const int nt = (rec.z + 1) >> 1;
+        const uint32_t set = n_items % SETS, acc = tmem_base + (is_v ? TM_DV : TM_DK) + set * TM_SET;
+        VSA2_WAIT_PARKED(&misc->o_empty[set], ((n_items / SETS) & 1) ^ 1);
         for (int t = 0; t < nt; ++t, ++tg) {
           if (is_v) {
             // P depends on S only, so it can be ready before the dO pair of the tile has landed: wait for that too
@@ -286,22 +276,22 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             VSA2_WAIT_PARKED(&misc->p_ready, tg & 1);
             tc::tc_fence_after();
             if (tc::elect_one()) {
-              if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(tmem_base + TM_DV, base + C::OFF_RING_B + sv * C::SLOT, b_addr, C::PBYTES, t > 0);
-              else mma_pairT_mnmajor<D, F16 == 2>(tmem_base + TM_DV, base + C::OFF_RING_B + sv * C::SLOT, b_addr, t > 0);
+              if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, C::PBYTES, t > 0);
+              else mma_pairT_mnmajor<D, F16 == 2>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, t > 0);
               tc::mma_commit(&misc->b_empty[sv]);
               tc::mma_commit(&misc->p_free);
-              if (t == nt - 1) tc::mma_commit(&misc->o_full);
+              if (t == nt - 1) tc::mma_commit(&misc->o_full[set]);
             }
           } else {
             const uint32_t sa = tg % RA;
             VSA2_WAIT_PARKED(&misc->ds_ready[0], tg & 1);
             tc::tc_fence_after();
             if (tc::elect_one()) {
-              if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(tmem_base + TM_DK, base + sa * C::SLOT, b_addr, C::PBYTES, t > 0);
-              else mma_pairT_mnmajor<D, F16 != 0>(tmem_base + TM_DK, base + sa * C::SLOT, b_addr, t > 0);
+              if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(acc, base + sa * C::SLOT, b_addr, C::PBYTES, t > 0);
+              else mma_pairT_mnmajor<D, F16 != 0>(acc, base + sa * C::SLOT, b_addr, t > 0);
               tc::mma_commit(&misc->a_empty[sa]);
               tc::mma_commit(&misc->ds_free[0]);
-              if (t == nt - 1) tc::mma_commit(&misc->o_full);
+              if (t == nt - 1) tc::mma_commit(&misc->o_full[set]);
             }
           }
           __syncwarp();
@@ -309,17 +299,19 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         ++n_items;
       }
     }
+    }
   } else if (warp >= 12 && warp < 16) {
+    tc::reg_dec<48>();
     // ------------------------------------------------------------------ row statistics of the tiles (128 threads)
     const int r = tid - 384;                 // query row of the tile
     const int blk = r >> 6;
     float2* rowstat = reinterpret_cast<float2*>(misc->stats);
     uint32_t tg = 0;
     for (uint32_t seq = 0;; ++seq) {
-      VSA2_NEXT_ITEM(item, seq);
+      VSA2_NEXT_REC(rec, seq);
+      if (rec.z == 0) continue;
       VSA2_DKV_ITEM_SETUP();
       (void)j; (void)bhk;
-      if (k == 0 || k < a.k_lo || k > a.k_hi) continue;
       const int nt = (k + 1) >> 1;
       int bhq_n, i_n;
       dkv_entry(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n);
@@ -334,44 +326,21 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         tc::mbar_arrive(&misc->stat_full);
       }
     }
-  } else if (warp >= 4 && warp < 12) {
-    // ------------------------------------------------------------------ elementwise stage + epilogue (256 threads):
+  } else if (warp < 12) {
+    tc::reg_inc<120>();
+    // ------------------------------------------------------------------ elementwise stage (256 threads):
     // warps 4..7 take key columns 0..31 of every tile, warps 8..11 columns 32..63
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
-    const int row = (quad << 5) | lane;      // query row of the tile (S, dP) / channel (dK^T, dV^T)
-    const int sm_tid = tid - 128;            // 0..255
+    const int row = (quad << 5) | lane;      // query row of the tile
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    uint32_t tg = 0, n_items = 0;
-    uint32_t n_mine = 0;                       // items of this launch so far (the group syncs and table parities count these)
-    for (uint32_t n_all = 0;; ++n_all) {
-      VSA2_NEXT_ITEM(item, n_all);
-      VSA2_DKV_ITEM_SETUP();
-      (void)col_beg;
-      if (k < a.k_lo || k > a.k_hi) continue;  // another launch's item (an empty list still gets its coarse-only output)
-      const int tb = n_mine & 1;
-      const uint32_t e_sync0 = n_mine * (g.out_f32 ? 1u : 3u);     // index of this item's first group sync
-      if (sm_tid < 64) misc->tok[tb][sm_tid] = block_token(g, j, sm_tid);
-      float coarse_k = 0.f, coarse_v = 0.f;
-      if (a.dkc != nullptr && row < D && !block_is_text(g, j)) {
-        for (int hh = 0; hh < rep; ++hh) {
-          const size_t cidx = ((size_t)(b * g.Hq + hk * rep + hh) * g.Nvid + j) * D + row;
-          coarse_k += a.dkc[cidx];
-          coarse_v += a.dvc[cidx];
-        }
-        const float inv_cnt = 1.f / (float)cube_count(g, j);
-        coarse_k *= inv_cnt;
-        coarse_v *= inv_cnt;
-      }
-      VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0);
-      uint32_t kvmask = 0xffffffffu;           // validity of this thread's 32 key columns, from the token table
-      if (k > 0 && block_count(g, j) < kBlockTokens) {
-        kvmask = 0u;
-#pragma unroll 1
-        for (int p = 0; p < 32; ++p)
-          if (misc->tok[tb][half * 32 + p] >= 0) kvmask |= 1u << p;
-      }
+    uint32_t tg = 0;
+    for (uint32_t seq = 0;; ++seq) {
+      VSA2_NEXT_REC(rec, seq);
+      const int j = rec.x, k = rec.z;
       if (k > 0) {
+        uint32_t kvmask = 0xffffffffu;         // validity of this thread's 32 key columns
+        if (block_count(g, j) < kBlockTokens) kvmask = __ballot_sync(0xffffffffu, block_token(g, j, half * 32 + lane) >= 0);
         const int nt = (k + 1) >> 1;
         const float2* rowstat = reinterpret_cast<const float2*>(misc->stats);
         for (int t = 0; t < nt; ++t, ++tg) {
@@ -450,71 +419,86 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             tc::mbar_arrive(&misc->ds_ready[0]);
           }
         }
-        VSA2_WAIT(&misc->o_full, n_items & 1);
-        tc::tc_fence_after();
       }
-      // epilogue: dK[l, d] = scale * dK^T[d, kv] + sum_heads dK_c[j, d] / count(j) (dS goes to its product without the
-      // softmax scale), dV the same without a scale; this thread owns 32 key columns
-      {
-        uint32_t kk[32], vv[32];
-        if (k > 0) {
-          tc::tmem_ld32(lane_addr + TM_DK + half * 32, kk);
-          tc::tmem_ld32(lane_addr + TM_DV + half * 32, vv);
+    }
+  } else {
+    tc::reg_inc<96>();
+    // ------------------------------------------------------------------ epilogue (128 threads, one per channel):
+    // dK[l, d] = scale * dK^T[d, kv] + sum_heads dK_c[j, d] / count(j) (dS goes to its product without the softmax scale),
+    // dV the same without a scale
+    const int row = tid - 640;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    uint32_t n_items = 0;
+    for (uint32_t seq = 0;; ++seq) {
+      VSA2_NEXT_REC(rec, seq);
+      const int j = rec.x, bhk = rec.y, k = rec.z;
+      const int b = bhk / g.Hkv, hk = bhk % g.Hkv;
+      const int tok0 = block_token(g, j, lane), tok1 = block_token(g, j, 32 + lane);
+      float coarse[2] = {0.f, 0.f};            // dK, dV
+      if (a.dkc != nullptr && row < D && !block_is_text(g, j)) {
+        for (int hh = 0; hh < rep; ++hh) {
+          const size_t cidx = ((size_t)(b * g.Hq + hk * rep + hh) * g.Nvid + j) * D + row;
+          coarse[0] += a.dkc[cidx];
+          coarse[1] += a.dvc[cidx];
+        }
+        const float inv_cnt = 1.f / (float)cube_count(g, j);
+        coarse[0] *= inv_cnt;
+        coarse[1] *= inv_cnt;
+      }
+      const size_t head = (size_t)bhk * g.S;
+      if (k == 0) {                            // nothing kept: the coarse gradients only
+        for (int c = 0; c < 64; ++c) {
+          const int l = __shfl_sync(0xffffffffu, c < 32 ? tok0 : tok1, c & 31);
+          if (l < 0 || row >= D) continue;
+          store_out(a.dk, (head + l) * D + row, coarse[0], g.out_f32);
+          store_out(a.dv, (head + l) * D + row, coarse[1], g.out_f32);
+        }
+        continue;
+      }
+      const uint32_t set = n_items % SETS;
+      VSA2_WAIT_PARKED(&misc->o_full[set], (n_items / SETS) & 1);
+      tc::tc_fence_after();
+      // The four warps write the same table.  Behind this wait every one of them is through with the item two before, whose
+      // table this was: its accumulators were given back after the last look at it (SETS = 2), or those of the item in between
+      // were (SETS = 1).
+      int* tok = misc->tok + (n_items & 1) * 64;
+      tok[lane] = tok0;
+      tok[32 + lane] = tok1;
+      __syncwarp();
+#pragma unroll 1
+      for (int part = 0; part < 4; ++part) {   // dK tokens 0..31, 32..63, dV the same
+        const bool is_v = part >= 2;
+        float v[32];
+        {
+          const uint32_t addr = lane_addr + set * TM_SET + (is_v ? TM_DV : TM_DK) + (part & 1) * 32;
+          uint32_t x[32];
+          tc::tmem_ld32(addr, x);
           tc::tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(x[c]);
           if constexpr (SPLIT) {
-            uint32_t lo[32];
-            tc::tmem_ld32(lane_addr + TM_DK + 64 + half * 32, lo);
+            tc::tmem_ld32(addr + 64, x);
             tc::tmem_ld_wait();
 #pragma unroll
-            for (int c = 0; c < 32; ++c) kk[c] = __float_as_uint(__uint_as_float(kk[c]) + __uint_as_float(lo[c]));
-            tc::tmem_ld32(lane_addr + TM_DV + 64 + half * 32, lo);
-            tc::tmem_ld_wait();
-#pragma unroll
-            for (int c = 0; c < 32; ++c) vv[c] = __float_as_uint(__uint_as_float(vv[c]) + __uint_as_float(lo[c]));
-          }
-          tc::tc_fence_before();
-          tc::mbar_arrive(&misc->o_empty);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) { kk[c] = 0u; vv[c] = 0u; }
-        }
-        if (g.out_f32) {
-          if (row < D) {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int l = misc->tok[tb][half * 32 + c];
-              if (l < 0) continue;
-              const size_t idx = ((size_t)bhk * g.S + l) * D + row;
-              store_out(a.dk, idx, fmaf(__uint_as_float(kk[c]), g.scale, coarse_k), 1);
-              store_out(a.dv, idx, __uint_as_float(vv[c]) + coarse_v, 1);
+            for (int c = 0; c < 32; ++c) v[c] += __uint_as_float(x[c]);
+            if (part == 3) {                   // everything has been read: the accumulators are free
+              tc::tc_fence_before();
+              __syncwarp();
+              if (lane == 0) tc::mbar_arrive(&misc->o_empty[0]);
             }
           }
-        } else {
-          // bf16: transpose through shared memory (the P and dS buffers are idle now), then 16-byte stores
-          bf16* st_k = reinterpret_cast<bf16*>(p_tile);       // [64 kv][D]
-          bf16* st_v = reinterpret_cast<bf16*>(ds_tile);      // [64 kv][D]
-          if (row < D) {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              st_k[(half * 32 + c) * D + row] = __float2bfloat16_rn(fmaf(__uint_as_float(kk[c]), g.scale, coarse_k));
-              st_v[(half * 32 + c) * D + row] = __float2bfloat16_rn(__uint_as_float(vv[c]) + coarse_v);
-            }
-          }
-          VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0 + 1);
-          constexpr int CH = D / 8;
-          for (int e = sm_tid; e < 64 * CH; e += 256) {
-            const int c = e / CH, ch = e % CH;
-            const int l = misc->tok[tb][c];
-            if (l < 0) continue;
-            const size_t idx = ((size_t)bhk * g.S + l) * D + ch * 8;
-            *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.dk) + idx) = *reinterpret_cast<const uint4*>(st_k + c * D + ch * 8);
-            *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.dv) + idx) = *reinterpret_cast<const uint4*>(st_v + c * D + ch * 8);
-          }
-          VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0 + 2);
         }
+        const float add = is_v ? coarse[1] : coarse[0];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) v[c] = is_v ? v[c] + add : fmaf(v[c], g.scale, add);
+        if (row < D) store_channels<D>(is_v ? a.dv : a.dk, g.out_f32, head, tok + (part & 1) * 32, v, row);
       }
-      if (k > 0) ++n_items;
-      ++n_mine;
+      if constexpr (!SPLIT) {
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&misc->o_empty[set]);
+      }
+      ++n_items;
     }
   }
 
@@ -585,6 +569,10 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                   (int)L_::smem_bytes)))                                                                         \
       return e;                                                                                                                  \
     cfg.dynamicSmemBytes = L_::smem_bytes;                                                                                       \
+    cudaFuncAttributes fa;                                                                                                       \
+    if ((e = cudaFuncGetAttributes(&fa, (const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F>)) != cudaSuccess) return e;           \
+    /* the warps that raise their register count wait for ever if the launch allocated less than their sum */                    \
+    if (fa.numRegs * kDkvThreads < 128 * (48 + 2 * 120 + 2 * 48 + 96)) return cudaErrorLaunchOutOfResources;                     \
     if ((e = cudaLaunchKernelEx(&cfg, fine_bwd_dkv_tc_kernel<DD, SP, MH, F>, TQ, TK, TV, TDO, TQT, TKT, TVT, TDOT, g, a)))       \
       return e;                                                                                                                  \
   } while (0)

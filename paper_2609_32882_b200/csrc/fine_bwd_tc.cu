@@ -243,7 +243,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const int k = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] - a.row_ptr[(size_t)bhq * (g.N + 1) + i];
         if (k == 0) continue;
         const int nt = (k + 1) >> 1;
-        VSA2_WAIT(&misc->o_empty, (n_items & 1) ^ 1);
+        VSA2_WAIT(&misc->o_empty[0], (n_items & 1) ^ 1);
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t sd = SPLIT ? 0u : (tg & 1), pd = SPLIT ? (tg & 1) : ((tg >> 1) & 1), sa = tg % kRingA;
           VSA2_WAIT(&misc->ds_ready[sd], pd);
@@ -256,7 +256,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                                            (F16 && t == nt - 1 && (k & 1)) ? 4 : 8);
             tc::mma_commit(&misc->a_empty[sa]);
             tc::mma_commit(&misc->ds_free[sd]);
-            if (t == nt - 1) tc::mma_commit(&misc->o_full);
+            if (t == nt - 1) tc::mma_commit(&misc->o_full[0]);
           }
           __syncwarp();
         }
@@ -285,7 +285,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
       const uint32_t e_sync0 = n_all * (g.out_f32 ? 1u : 3u);     // index of this item's first group sync
       if (sm_tid < 64) {
         const int l = block_token(g, i, sm_tid);
-        misc->tok[tb][sm_tid] = l;
+        misc->tok[tb * 64 + sm_tid] = l;
         misc->stats[tb * 64 + sm_tid] = l >= 0 ? a.lse[(size_t)bhq * g.S + l] * 1.4426950408889634f : INFINITY;
         misc->stats[128 + tb * 64 + sm_tid] = l >= 0 ? a.delta[(size_t)bhq * g.S + l] : 0.f;
       }
@@ -369,7 +369,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
           tc::fence_proxy_async_smem();
           tc::mbar_arrive(&misc->ds_ready[sd]);
         }
-        VSA2_WAIT(&misc->o_full, n_items & 1);
+        VSA2_WAIT(&misc->o_full[0], n_items & 1);
         tc::tc_fence_after();
       }
       // epilogue: dQ[l, d] = scale * dQ^T[d, q] + dQ_c[i, d] / count(i) (dS goes to its product without the softmax scale);
@@ -387,7 +387,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             for (int c = 0; c < 32; ++c) o0[c] = __float_as_uint(__uint_as_float(o0[c]) + __uint_as_float(o1[c]));
           }
           tc::tc_fence_before();
-          tc::mbar_arrive(&misc->o_empty);
+          tc::mbar_arrive(&misc->o_empty[0]);
           // F16: a dS that left the fp16 range went into the product as an infinity and has made every channel of its query
           // column non-finite: the result of this launch is not to be used, the fallback launch redoes it
           if constexpr (F16) {
@@ -401,7 +401,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
           if (row < D) {
 #pragma unroll
             for (int c = 0; c < 32; ++c) {
-              const int l = misc->tok[tb][half * 32 + c];
+              const int l = misc->tok[tb * 64 + half * 32 + c];
               if (l < 0) continue;
               store_out(a.dq, ((size_t)bhq * g.S + l) * D + row, fmaf(__uint_as_float(o0[c]), g.scale, coarse_d), 1);
             }
@@ -418,7 +418,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
           constexpr int CH = D / 8;
           for (int e = sm_tid; e < 64 * CH; e += 256) {
             const int qi = e / CH, ch = e % CH;
-            const int l = misc->tok[tb][qi];
+            const int l = misc->tok[tb * 64 + qi];
             if (l < 0) continue;
             *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.dq) + ((size_t)bhq * g.S + l) * D + ch * 8) =
                 *reinterpret_cast<const uint4*>(st + qi * D + ch * 8);

@@ -6,7 +6,8 @@
 namespace vsa2 {
 
 constexpr int kDqThreads = 416;    // dQ pass: 4 service warps, 2 x 4 elementwise warps, 1 more issuer warp
-constexpr int kDkvThreads = 576;   // dK/dV pass: 4 service warps, 2 x 4 elementwise warps, 4 row-statistics warps, 2 issuer warps
+constexpr int kDkvThreads = 768;   // dK/dV pass: 4 service warps, 2 x 4 elementwise warps, 4 row-statistics warps, 2 issuer warps,
+                                   // a scheduler warp (and an idle one), 4 epilogue warps
 constexpr int kRingA = 3;          // slots of the ring whose tiles are also an operand of the last product of a tile
 constexpr int kRingB = 2;          // (the ring-B slot of a tile is also the index of its tensor-memory buffers)
 static_assert(kRingB == 2, "ring B shares its slot index with the two accumulator buffers");
@@ -31,14 +32,104 @@ struct BwdTc {
   static constexpr size_t smem_bytes = OFF_MISC + MISC_BYTES + 1024;
 };
 
+// Work items of a persistent CTA with everything a role needs to know about one: {block, batch * heads index, entries of its
+// list, start of the list}, block -1 at the end.  A warp of its own (the scheduler) draws the items and looks the lists up, one
+// item ahead of the first producer: nothing of that -- an atomic and two dependent loads -- lies on another role's path,
+// and a CTA does not claim items that a CTA with less to do could start sooner.
+struct BwdQueue {
+  uint64_t full[kItemSlots], empty[kItemSlots], taken;
+  int4 rec[kItemSlots];
+};
+// `consumers`: warps that call bwd_queue_get for every item
+__device__ __forceinline__ void bwd_queue_init(BwdQueue* q, int consumers) {
+  for (int s = 0; s < kItemSlots; ++s) {
+    tc::mbar_init(&q->full[s], 1);
+    tc::mbar_init(&q->empty[s], consumers);
+  }
+  tc::mbar_init(&q->taken, 1);
+}
+// whole warp: record of the item with sequence number seq; false on a timed-out wait
+__device__ __forceinline__ bool bwd_queue_get(BwdQueue* q, uint32_t seq, int lane, int4& rec, volatile int* abort_flag) {
+  const uint32_t slot = seq % kItemSlots;
+  const bool ok = tc::mbar_wait_parked(&q->full[slot], (seq / kItemSlots) & 1, abort_flag);
+  rec = q->rec[slot];
+  __syncwarp();
+  if (lane == 0) tc::mbar_arrive(&q->empty[slot]);
+  return ok;
+}
+#define VSA2_NEXT_REC(REC, SEQ)                                                          \
+  int4 REC;                                                                              \
+  if (!bwd_queue_get(&misc->queue, (SEQ), lane, REC, &misc->abort_flag)) goto done;      \
+  if (REC.x < 0) break
+// scheduler warp: draws items until the counter (or the list) runs out.  `ptr`, `rep`: start pointers of the lists, an item has
+// those of `rep` consecutive heads; items with fewer than k_lo or more than k_hi entries are left out.
+__device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int heads, int rep, const int* ptr, int* counter,
+                                             const int* list, int k_lo, int k_hi, int lane, volatile int* abort_flag) {
+  const int total = list != nullptr ? list[0] : g.batch * heads * g.N;
+  uint32_t drawn = 0;
+  for (uint32_t p = 0;; ++p) {
+    const uint32_t slot = p % kItemSlots;
+    if (p > 0 && !tc::mbar_wait_parked(&q->taken, (p - 1) & 1, abort_flag)) return false;
+    if (!tc::mbar_wait_parked(&q->empty[slot], ((p / kItemSlots) & 1) ^ 1, abort_flag)) return false;
+    int4 rec;
+    for (;;) {
+      rec = make_int4(-1, 0, 0, 0);
+      int n = 0;
+      if (lane == 0) n = item_draw(drawn, counter);
+      n = __shfl_sync(0xffffffffu, n, 0);
+      ++drawn;
+      if (n >= total) break;
+      item_block(g, list != nullptr ? list[1 + n] : n, rec.y, rec.x);
+      int beg = 0, k = 0;
+      if (lane < rep) {      // (heads of a group are neighbours: b * Hq + hk * rep + hh)
+        const int* c = ptr + ((size_t)rec.y * rep + lane) * (g.N + 1) + rec.x;
+        beg = c[0];
+        k = c[1] - beg;
+      }
+      rec.z = __reduce_add_sync(0xffffffffu, k);
+      rec.w = __shfl_sync(0xffffffffu, beg, 0);
+      if (rec.z >= k_lo && rec.z <= k_hi) break;
+    }
+    if (lane == 0) {
+      q->rec[slot] = rec;
+      tc::mbar_arrive(&q->full[slot]);
+    }
+    if (rec.x < 0) return true;
+  }
+}
+
+// Stores 32 values per thread -- channel `row` of 32 tokens, the warp's lanes being 32 neighbouring channels -- to the token
+// rows named by tok[0 .. 31] (shared memory, -1 = no token).  No exchange between lanes: shuffles and a transpose in shared
+// memory both use the data pipe that bounds the passes, and a chain of them took the epilogue warps three times as long as
+// storing 64 bytes per warp and token.
+template <int D>
+__device__ __forceinline__ void store_channels(void* out, int out_f32, size_t head, const int* tok, const float (&v)[32], int row) {
+  if (out_f32) {
+    float* base = reinterpret_cast<float*>(out) + head * D + row;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const int l = tok[c];
+      if (l >= 0) base[(size_t)l * D] = v[c];
+    }
+  } else {
+    bf16* base = reinterpret_cast<bf16*>(out) + head * D + row;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const int l = tok[c];
+      if (l >= 0) base[(size_t)l * D] = __float2bfloat16_rn(v[c]);
+    }
+  }
+}
+
 struct BwdMisc {
-  uint64_t st_full, st_empty, o_full, o_empty;
+  uint64_t st_full, st_empty, o_full[2], o_empty[2];       // (the dQ pass uses one accumulator)
   uint64_t a_full[kRingA], a_empty[kRingA], b_full[kRingB], b_empty[kRingB];
   uint64_t s_full[2], s_free[2], dp_full[2], dp_free[2];   // the two score / dP accumulators in tensor memory
   uint64_t p_ready, p_free;                                 // dK/dV pass: the P operand buffer
   uint64_t ds_ready[2], ds_free[2];                         // dS operand buffers (the dK/dV pass has one)
   uint64_t stat_full, stat_free;                            // dK/dV pass: the per-row statistics of a tile
-  ItemQueue items;                                          // work items of this CTA (see tc_attn.cuh)
+  ItemQueue items;                                          // dQ pass: work items of this CTA (see tc_attn.cuh)
+  BwdQueue queue;                                           // dK/dV pass
   uint64_t e_sync;                                          // group barrier of the 256 elementwise threads
   uint32_t tmem_base;
   int abort_flag;
@@ -47,7 +138,7 @@ struct BwdMisc {
   // parity tb, lse * log2(e) (+inf for padding) and delta.  dK/dV pass: (lse * log2(e), delta) of the 128 query rows of
   // the current tile, interleaved.
   alignas(16) float stats[256];
-  int tok[2][64];
+  int tok[128];                    // raster tokens of the rows of an item's block, by parity (dK/dV pass: of the items with entries)
 };
 static_assert(sizeof(BwdMisc) <= 2048, "misc region too small");
 
@@ -55,8 +146,10 @@ __device__ __forceinline__ void bwd_init_barriers(BwdMisc* misc) {
   misc->abort_flag = 0;
   tc::mbar_init(&misc->st_full, 1);
   tc::mbar_init(&misc->st_empty, 2);     // both first-stage issuers
-  tc::mbar_init(&misc->o_full, 1);       // re-initialised to 2 by the dK/dV pass (two last-stage issuers)
-  tc::mbar_init(&misc->o_empty, 256);
+  for (int s = 0; s < 2; ++s) {
+    tc::mbar_init(&misc->o_full[s], 1);       // re-initialised by the dK/dV pass
+    tc::mbar_init(&misc->o_empty[s], 256);
+  }
   for (int s = 0; s < kRingA; ++s) {
     tc::mbar_init(&misc->a_full[s], 1);
     tc::mbar_init(&misc->a_empty[s], 1);

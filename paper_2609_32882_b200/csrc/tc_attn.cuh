@@ -201,8 +201,14 @@ __device__ __forceinline__ int warp_reduce_col(int lane) {
 // scheduler) draws item numbers from a global counter, a few items ahead, and publishes them through a small ring in
 // shared memory; every role of the CTA reads the same sequence from the ring.  All CTAs therefore advance through the
 // item sequence together (neighbouring items share operand tiles in L2) and finish together.  Item -1 ends the CTA.
+// The first item of a CTA is its block index: a problem of fewer items than SMs has one per CTA (drawn from the counter, three
+// at a time, they all went to the CTAs that started first: 30 items of the pooled backward ran on ten SMs).
 constexpr int kItemSlots = 4;       // ring depth
-constexpr int kItemAhead = 2;       // items published ahead of the scheduler's own position
+constexpr int kItemAhead = 2;       // items published ahead of the scheduler's own position (one less while it is at its first)
+// item number of the CTA's draw `n`
+__device__ __forceinline__ int item_draw(uint32_t n, int* counter) {
+  return n == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(counter, 1);
+}
 struct ItemQueue {
   uint64_t full[kItemSlots], empty[kItemSlots];
   int item[kItemSlots];
@@ -217,10 +223,10 @@ __device__ __forceinline__ void item_queue_init(ItemQueue* q, int consumers) {
 // scheduler: publishes every sequence number up to seq + kItemAhead that is not out yet; false on a timed-out wait
 __device__ __forceinline__ bool item_publish_ahead(ItemQueue* q, uint32_t seq, uint32_t& published, int* counter, int total,
                                                    volatile int* abort_flag) {
-  while (published <= seq + kItemAhead) {
+  while (published <= seq + (seq ? kItemAhead : 1)) {
     const uint32_t slot = published % kItemSlots, par = ((published / kItemSlots) & 1) ^ 1;
     if (!tc::mbar_wait_parked(&q->empty[slot], par, abort_flag)) return false;
-    const int it = atomicAdd(counter, 1);
+    const int it = item_draw(published, counter);
     q->item[slot] = it < total ? it : -1;
     tc::mbar_arrive(&q->full[slot]);
     ++published;
