@@ -245,6 +245,11 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
                   const void* d_o, void* dq, void* dk, void* dv, float* dgate,
                   void* workspace, size_t workspace_bytes, void* cuda_stream);
 
+/* Bytes of backward workspace with which vsa2_attn_bwd runs fastest (0 for invalid parameters): sizes.bwd_workspace_bytes is
+ * the least it accepts; what a caller hands it beyond that holds the score gradients of the dK/dV pass, so that the dQ pass
+ * need not recompute them (bounded: 7 GiB of them at most).  Both give the same results. */
+size_t vsa2_attn_bwd_preferred_workspace_bytes(const vsa2_params* p);
+
 /* Cube-major copy of a tensor (Sec. 2.2 "Permutation": (T, H, W) -> (N_t N_h N_w) x (B_t B_h B_w)), for callers whose
  * surrounding code works in that layout; the entry points above take the raster layout and never need it.
  *   inverse == 0: src [batch, heads, L, D] raster -> dst [batch, heads, N * B, D]; cube n occupies rows n*B .. n*B+B-1, its

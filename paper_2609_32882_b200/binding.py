@@ -31,7 +31,8 @@ ERR_STATIC_SCRATCH = -8
 
 EXPORTS = ("vsa2_query_sizes", "vsa2_route", "vsa2_route_scores", "vsa2_attn_fwd", "vsa2_attn_bwd",
            "vsa2_device_status", "vsa2_strerror", "vsa2_profile_events", "vsa2_launch_count", "vsa2_selftest_umma", "vsa2_route_noalloc", "vsa2_last_cuda_error",
-           "vsa2_gate_fwd", "vsa2_gate_bwd", "vsa2_gate_bwd_workspace_bytes", "vsa2_permute_cube_major",
+           "vsa2_gate_fwd", "vsa2_gate_bwd", "vsa2_gate_bwd_workspace_bytes",
+           "vsa2_attn_bwd_preferred_workspace_bytes", "vsa2_permute_cube_major",
            "vsa2_selftest_timeout", "vsa2_debug_rescue_capacity", "vsa2_selftest_divmod")
 
 KERNELS = ("pool", "router_lse", "router_pool", "select", "coarse_fwd", "fine_fwd", "bwd_pre", "coarse_bwd",
@@ -93,6 +94,8 @@ def _lib():
         lib.vsa2_route_noalloc.argtypes = [C.POINTER(Params), vp, vp, vp, C.POINTER(Map), vp, vp]
         lib.vsa2_permute_cube_major.argtypes = [C.POINTER(Params), C.c_int32, C.c_int32, vp, vp, vp]
         lib.vsa2_gate_fwd.argtypes = [C.POINTER(Params), C.c_int32, vp, vp, vp, vp]
+        lib.vsa2_attn_bwd_preferred_workspace_bytes.argtypes = [C.POINTER(Params)]
+        lib.vsa2_attn_bwd_preferred_workspace_bytes.restype = C.c_size_t
         lib.vsa2_gate_bwd_workspace_bytes.argtypes = [C.POINTER(Params), C.c_int32]
         lib.vsa2_gate_bwd_workspace_bytes.restype = C.c_size_t
         lib.vsa2_gate_bwd.argtypes = [C.POINTER(Params), C.c_int32, vp, vp, vp, vp, vp, vp, vp, sz, vp]
@@ -115,7 +118,8 @@ def _lib():
         lib.vsa2_selftest_divmod.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32]
         lib.vsa2_selftest_divmod.restype = C.c_int64
         for name in EXPORTS:
-            if name not in ("vsa2_strerror", "vsa2_route_scores", "vsa2_launch_count", "vsa2_last_cuda_error", "vsa2_selftest_divmod"):
+            if name not in ("vsa2_strerror", "vsa2_route_scores", "vsa2_launch_count", "vsa2_last_cuda_error", "vsa2_selftest_divmod",
+                            "vsa2_gate_bwd_workspace_bytes", "vsa2_attn_bwd_preferred_workspace_bytes"):
                 getattr(lib, name).restype = C.c_int
         _LIB = lib
     return _LIB
@@ -226,6 +230,11 @@ def vsa2_attn_bwd(p, q, k, v, gate, vmap: Map, o, lse, saved, d_o, dq, dk, dv, d
                                 _ptr(dv), _ptr(dgate), _ptr(workspace), nbytes, _stream(stream)), "vsa2_attn_bwd")
 
 
+def vsa2_attn_bwd_preferred_workspace_bytes(p) -> int:
+    """Bytes of backward workspace with which vsa2_attn_bwd runs fastest (at least sizes.bwd_workspace_bytes)."""
+    return int(_lib().vsa2_attn_bwd_preferred_workspace_bytes(C.byref(p)))
+
+
 def vsa2_profile_events(kernel_id: int, start_event, stop_event):
     """start/stop: torch.cuda.Event objects (already recorded once, so that their handles exist) or None."""
     a = None if start_event is None else start_event.cuda_event
@@ -280,7 +289,10 @@ class Vsa2Attention:
         u8 = dict(dtype=torch.uint8, device=dev)
         self.ws_route = torch.empty(s.route_workspace_bytes, **u8)
         self.ws_fwd = torch.empty(s.fwd_workspace_bytes, **u8)
-        self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
+        try:
+            self.ws_bwd = torch.empty(vsa2_attn_bwd_preferred_workspace_bytes(params), **u8)
+        except torch.cuda.OutOfMemoryError:     # the least the backward accepts: it recomputes what the rest would hold
+            self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
         for ws in (self.ws_route, self.ws_fwd, self.ws_bwd):
             ws[:256].zero_()          # status block
         self.out_torch_dtype = torch.float32 if params.out_dtype == F32 else torch.bfloat16

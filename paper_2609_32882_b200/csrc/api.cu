@@ -232,6 +232,37 @@ size_t bwd_workspace_bytes(const Geo& g) {
   return n;
 }
 
+// dS tiles that the dK/dV pass leaves for the dQ pass (fine_bwd_dq_ds_tc.cu), in what a caller's workspace holds beyond
+// bwd_workspace_bytes: 8 KB per kept pair of 64-token blocks, for as many KV groups at a time as fit.  Without room for one group
+// the dQ pass recomputes dS.  The preferred size stops at kStoredDsBytes of tiles (9 heads of 720p top-64, one group of the
+// 16..256-cube budget with four heads a group): a launch over fewer blocks loses more on its last, unevenly filled items
+// (one head of 720p at a time: 10 blocks per SM), more scratch gains nothing.
+constexpr size_t kStoredDsBytes = (size_t)7 << 30;
+struct DsLayout {
+  size_t counters, pos, tiles, total;
+  int groups;          // KV groups per chunk, 0: no stored dS
+};
+DsLayout ds_layout(const Geo& g, size_t avail_total, bool preferred) {
+  DsLayout r{};
+  if (!dq_pass_f16(g) || wide_cube(g)) return r;
+  const Geo x = g.Lt > 0 ? text_geo(g) : g;
+  const size_t all = (size_t)g.batch * g.Hkv, group = (size_t)x.rep * x.nnz_cap * kBlockTokens * kBlockTokens * sizeof(bf16);
+  if (group == 0) return r;
+  Carver c;
+  c.off = align_up(bwd_workspace_bytes(g), 256);
+  r.counters = c.take(2 * all * sizeof(int));
+  r.pos = c.take((size_t)g.batch * g.Hq * x.nnz_cap * sizeof(int));
+  r.tiles = c.off;
+  const size_t room = preferred ? kStoredDsBytes : avail_total > r.tiles ? avail_total - r.tiles : 0;
+  const size_t fit = room / group < all ? room / group : all;
+  // (row index of a tile in the tensor map: 32 bits)
+  if (fit == 0 || fit * group / 128 > 0x7fffffffULL) return r;
+  const size_t chunks = (all + fit - 1) / fit;
+  r.groups = (int)((all + chunks - 1) / chunks);
+  r.total = r.tiles + r.groups * group;
+  return r;
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 bool aligned256(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
 
@@ -312,6 +343,14 @@ int vsa2_query_sizes(const vsa2_params* p, vsa2_sizes* out) {
   out->fwd_workspace_bytes = fwd_workspace_bytes(g);
   out->bwd_workspace_bytes = bwd_workspace_bytes(g);
   return VSA2_OK;
+}
+
+size_t vsa2_attn_bwd_preferred_workspace_bytes(const vsa2_params* p) {
+  Geo g;
+  if (fill_geo(p, &g) != VSA2_OK) return 0;
+  const size_t least = bwd_workspace_bytes(g);
+  const DsLayout dl = ds_layout(g, 0, true);
+  return dl.groups > 0 ? dl.total : least;
 }
 
 int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets, const vsa2_map* map,
@@ -587,12 +626,24 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
       VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dvc_cube, dvc, st));
     }
   }
+  // dS kept from the dK/dV pass for the dQ pass, which then runs inside it; otherwise the dQ pass recomputes dS and runs first
+  const DsLayout dl = ds_layout(g, workspace_bytes, false);
+  const int ds_groups = dl.groups;
+  const StoredDs sd{at<unsigned char>(workspace, dl.tiles), at<int>(workspace, dl.pos), at<int>(workspace, dl.counters), ds_groups,
+                    row_ptr, col_idx, coarse ? dqc : nullptr, dq};
   // cubes of 128 tokens: both passes on 128 x 128 tiles
   const bool wide128 = wide && g.Lt == 0 && fine_bwd128_supported(n);
   {
     const bool f16 = dq_pass_f16(g);     // the copy, the fp16 form, the (idle) fallback
-    ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st, f16 ? 3 : 1);
-    if (wide128)
+    ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st, ds_groups > 0 ? 2 : f16 ? 3 : 1);
+    if (ds_groups > 0) {
+      VSA2_CUDA(launch_cast_bf16_to_f16(qb, at<unsigned char>(workspace, bwd_f16_offset(g)), (size_t)g.batch * g.Hq * g.S * g.D, kb,
+                                        at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)),
+                                        (size_t)g.batch * g.Hkv * g.S * g.D,
+                                        &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
+      VSA2_CUDA(launch_ds_positions(fx, row_ptr, col_idx, col_ptr, row_idx, at<int>(workspace, dl.pos), sd.counters,
+                                    2 * g.batch * g.Hkv, st));
+    } else if (wide128)
       VSA2_CUDA(launch_fine_bwd128_dq_tc(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
                                          reinterpret_cast<StatusBlock*>(workspace), st,
                                          f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
@@ -610,9 +661,11 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
     int* item_list = list_need <= list_have ? reinterpret_cast<int*>(d_oc_hat) : nullptr;
     const bool two = !dkv128 && fine_bwd_dkv_splits_long_columns(fx, true);
     const bool gqa16 = !dkv128 && dkv_pass_gqa_f16(g);    // (the copy of V and dO, the all-fp16 form, the pair form as its fallback)
-    const bool f16 = (two || gqa16) && dq_pass_f16(g);              // the dQ pass has left fp16 copies of Q and K
+    const bool f16 = (two || gqa16 || ds_groups > 0) && dq_pass_f16(g);      // fp16 copies of Q and K have been made
     ProfScope ps(VSA2_KERNEL_FINE_BWD_DKV, st, dkv128 ? (dq_pass_f16(g) ? 2 : 1)
                                                       : two ? (item_list ? 3 : 2) + (f16 ? 1 : 0) : (gqa16 ? 3 : 1));
+    const int chunks = ds_groups > 0 ? (g.batch * g.Hkv + ds_groups - 1) / ds_groups : 0;
+    if (chunks > 0) g_launches += 2 * chunks;      // (dQ per chunk and its fallback; the first dK/dV launch is counted above)
     unsigned char* v16 = gqa16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g) + bwd_k16_bytes(g)) : nullptr;
     if (dkv128)
       VSA2_CUDA(launch_fine_bwd128_dkv_tc(n, qb, kb, vb, dob, lse, delta, col_ptr, row_idx, coarse ? dkc : nullptr,
@@ -624,7 +677,7 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
                                        coarse ? dvc : nullptr, dk, dv, reinterpret_cast<StatusBlock*>(workspace), st, true,
                                        item_list, f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
                                        f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr, v16,
-                                       gqa16 ? v16 + bwd_k16_bytes(g) : nullptr));
+                                       gqa16 ? v16 + bwd_k16_bytes(g) : nullptr, ds_groups > 0 ? &sd : nullptr));
   }
   return VSA2_OK;
 }

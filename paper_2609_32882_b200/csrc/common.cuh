@@ -295,11 +295,30 @@ constexpr int kRangeFlagSlot = 8;
 // fp16 copies of two bf16 tensors (element counts multiples of 8); a finite value beyond the fp16 range sets *range_flag
 cudaError_t launch_cast_bf16_to_f16(const bf16* a, void* a16, size_t na, const bf16* b, void* b16, size_t nb, int* range_flag,
                                     cudaStream_t st);
+// dS kept between the two backward passes (fine_bwd_dq_ds_tc.cu): scratch for the pairs of `chunk_groups` KV groups at a time
+struct StoredDs {
+  void* scratch;        // chunk_groups * rep * nnz_cap tiles of 8 KB (64 queries x 64 keys, fp16)
+  const int* pos;       // [B, Hq, nnz_cap], filled by launch_ds_positions
+  int* counters;        // two words per chunk, cleared by launch_ds_positions
+  int chunk_groups;
+  const int* row_ptr;
+  const int* col_idx;
+  const float* dqc;
+  void* dq;
+};
+cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col_idx, const int* col_ptr, const int* row_idx, int* pos,
+                                int* counters, int n_counters, cudaStream_t st);
+cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
+                                  const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
+                                  int* item_counter, bool swizzled, cudaStream_t st);
+cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse,
+                                        const float* delta, const int* row_ptr, const int* col_idx, const float* dqc, void* dq,
+                                        StatusBlock* status, cudaStream_t st);
 cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, int* item_list, const void* q16,
-                                   const void* k16, void* v16, void* do16);
+                                   const void* k16, void* v16, void* do16, const StoredDs* sd);
 bool fine_bwd_dkv_gqa_uses_f16(const Geo& g);
 bool fine_bwd_dkv_splits_long_columns(const Geo& g, bool split_long_columns);
 

@@ -26,6 +26,10 @@ struct DkvArgs {
   int k_lo, k_hi;       // the launch handles the KV blocks whose column lists hold k_lo .. k_hi entries, and leaves the others alone
   int* range_flag;      // fp16 form and its fallback, as in DqArgs of the dQ pass (when = 0: the launch always runs)
   int when;
+  int first_item, items;  // work items of the launch (block lists of a range of KV heads)
+  unsigned char* ds;    // null, or the scratch for dS in fp16 (forms STORES_DS): [entry of the row lists of heads ds_head0 ..][8 chunks of 8 keys][64 q]
+  const int* ds_pos;    // [B, Hq, nnz_cap]: place of every entry of the column lists in the row lists
+  int ds_head0;
   const int* item_list; // null, or [count, item, item, ...]: the items with k_lo .. k_hi entries (the launch then walks this list
                         // instead of all items: a launch for the few long lists would spend most of its time skipping)
 };
@@ -35,12 +39,16 @@ constexpr int kMaxRep = 16;   // query heads per KV head the dK/dV pass supports
 // entry e of the concatenated column lists of the group's query heads -> (query head, query block)
 // (`cnt_prefix`, `col_beg`: per-head counts prefix and list starts of the item, read once per item so that this lookup
 // costs a single global load)
+// (`POS`: also its place in the row lists)
+template <bool POS = false>
 __device__ __forceinline__ void dkv_entry(const Geo& g, const DkvArgs& a, int rep, int b, int hk, const int* cnt_prefix,
-                                          const int* col_beg, int e, int& bhq, int& i) {
+                                          const int* col_beg, int e, int& bhq, int& i, int* pos = nullptr) {
   int hh = 0;
   while (hh + 1 < rep && e >= cnt_prefix[hh + 1]) ++hh;
   bhq = b * g.Hq + hk * rep + hh;
-  i = a.row_idx[(size_t)bhq * g.nnz_cap + col_beg[hh] + (e - cnt_prefix[hh])];
+  const size_t at = (size_t)bhq * g.nnz_cap + col_beg[hh] + (e - cnt_prefix[hh]);
+  i = a.row_idx[at];
+  if (POS && a.ds != nullptr) *pos = a.ds_pos[at];
 }
 
 // The work items whose column lists hold k_lo .. k_hi entries, appended to list[1 ...] with their count in list[0] (zero
@@ -92,6 +100,13 @@ __global__ void __launch_bounds__(256) dkv_list_items_kernel(Geo g, const int* _
 // with 11 bits in dS it stays below 1e-2 there, and the second launch for the long lists is not needed.  The launch stands
 // back when the range flag is up: the dQ pass, which runs first, forms the same dS values and raises it if one of them (or
 // a value of Q or K) leaves the fp16 range.
+// With `a.ds` (the fp16 forms, and SPLIT for GQA groups) dS also goes to memory, rounded to fp16 without a clamp, for the dQ pass of
+// fine_bwd_dq_ds_tc.cu: with SPLIT the elementwise threads
+// store a pair's tile as [chunk of 8 keys][query]; the fp16 forms have it in shared memory as the dK product's operand, and warp
+// 19 copies it as it stands, [query][64 keys] with the 128-byte swizzle (stored by the elementwise threads it cost the pass 14 %).  A dS beyond the fp16 range is an infinity there, which
+// that pass finds and turns into the range flag; the fp16 forms then also use it unclamped (their result is redone).
+// No key column is masked: the columns of positions without a token are accumulator columns that are never read out, and
+// in dQ they meet zero rows of K (fine_bwd_tc.cu).
 // F16 = 2: all four maps point at fp16 copies and P is rounded to fp16 as well (every product fp16 x fp16): the form for GQA
 // groups, where a KV block sums the query blocks of several heads and bf16 P leaves dV at 1.4e-2 (480p sample, |dV| = 11).
 template <int D, bool SPLIT, bool MHA, int F16>
@@ -116,6 +131,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float c2 = g.scale * 1.4426950408889634f;
   const int rep = MHA ? 1 : g.rep;
+  constexpr bool STORES_DS = F16 != 0 || (SPLIT && !MHA);
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
   if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
 
@@ -128,7 +144,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       tc::mbar_init(&misc->o_full[s], 2);                                     // two last-stage issuers
       tc::mbar_init(&misc->o_empty[s], 4);                                    // the epilogue warps
     }
-    bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4);
+    bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4 + (F16 != 0 && a.ds != nullptr ? 1 : 0));
+    if (F16 != 0 && a.ds != nullptr) tc::mbar_init(&misc->ds_free[0], 2);     // read by the dK product and by the copy
     for (int s = 0; s < kRingB; ++s) tc::mbar_init(&misc->b_empty[s], 2);     // a dO slot is read by dP and by dV^T
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
@@ -252,9 +269,30 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   } else if (warp >= 16 && warp < 20) {
     tc::reg_dec<48>();
-    if (warp == 18 && !bwd_schedule(&misc->queue, g, g.Hkv, rep, a.col_ptr, a.item_counter, SPLIT ? a.item_list : nullptr, a.k_lo,
+    if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, SPLIT ? a.item_list : nullptr, a.k_lo,
                                     a.k_hi, lane, &misc->abort_flag))
       goto done;
+    if (F16 != 0 && warp == 19 && a.ds != nullptr) {
+      // ---------------------------------------------------------------- copies the dS tiles to the scratch as they stand
+      uint32_t tg = 0;
+      for (uint32_t seq = 0;; ++seq) {
+        VSA2_NEXT_REC(rec, seq);
+        const int nt = (rec.z + 1) >> 1;
+        for (int t = 0; t < nt; ++t, ++tg) {
+          VSA2_WAIT_PARKED(&misc->ds_ready[0], tg & 1);
+          if (lane == 0) {
+            const int s0 = misc->ds_slot[tg & 3][0], s1 = misc->ds_slot[tg & 3][1];
+            if (s0 >= 0) tc::bulk_store(a.ds + (size_t)s0 * kSlab, ds_tile, kSlab);
+            if (s1 >= 0) tc::bulk_store(a.ds + (size_t)s1 * kSlab, ds_tile + kSlab, kSlab);
+            tc::bulk_store_commit();
+            tc::bulk_store_wait_read();
+            tc::mbar_arrive(&misc->ds_free[0]);
+          }
+          __syncwarp();
+        }
+      }
+      if (lane == 0) tc::bulk_store_wait();
+    }
     if (warp < 18) {
     // ------------------------------------------------------------------ issuers of dV^T += dO_pair^T P (warp 16) and
     // dK^T += Q_pair^T dS (warp 17); whole warp in the loop, one elected lane issues
@@ -313,15 +351,18 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       VSA2_DKV_ITEM_SETUP();
       (void)j; (void)bhk;
       const int nt = (k + 1) >> 1;
-      int bhq_n, i_n;
-      dkv_entry(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n);
+      int bhq_n, i_n, pos_n = 0;
+      dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n, &pos_n);
       for (int t = 0; t < nt; ++t, ++tg) {
+        const int slot = STORES_DS && a.ds != nullptr ? (bhq_n - a.ds_head0) * (int)g.nnz_cap + pos_n : -1;
         const bool dup = (blk == 1) && (2 * t + 1 >= k);
         const int l = dup ? -1 : block_token(g, i_n, r & 63);
         const size_t idx = l >= 0 ? (size_t)bhq_n * g.S + l : 0;
         const float lse_raw = a.lse[idx], dlt_raw = a.delta[idx];
-        if (t + 1 < nt) dkv_entry(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_n, i_n);
+        if (t + 1 < nt)
+          dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_n, i_n, &pos_n);
         VSA2_WAIT_PARKED(&misc->stat_free, (tg & 1) ^ 1);
+        if (STORES_DS && (r & 63) == 0) misc->ds_slot[tg & 3][blk] = dup ? -1 : slot;
         rowstat[r] = make_float2(l >= 0 ? lse_raw * 1.4426950408889634f : INFINITY, l >= 0 ? dlt_raw : 0.f);
         tc::mbar_arrive(&misc->stat_full);
       }
@@ -337,16 +378,15 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     uint32_t tg = 0;
     for (uint32_t seq = 0;; ++seq) {
       VSA2_NEXT_REC(rec, seq);
-      const int j = rec.x, k = rec.z;
+      const int k = rec.z;
       if (k > 0) {
-        uint32_t kvmask = 0xffffffffu;         // validity of this thread's 32 key columns
-        if (block_count(g, j) < kBlockTokens) kvmask = __ballot_sync(0xffffffffu, block_token(g, j, half * 32 + lane) >= 0);
         const int nt = (k + 1) >> 1;
         const float2* rowstat = reinterpret_cast<const float2*>(misc->stats);
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t s = tg & 1, par = (tg >> 1) & 1;
           VSA2_WAIT(&misc->stat_full, tg & 1);
           const float2 rs = rowstat[row];
+          const int ds_slot = SPLIT && STORES_DS ? misc->ds_slot[tg & 3][row >> 6] : -1;
           tc::mbar_arrive(&misc->stat_free);
           const float lse2 = rs.x, dlt = rs.y;
           uint32_t sv[32];      // S, then P
@@ -360,12 +400,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             uint32_t pp[16], pl[SPLIT ? 16 : 1];
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
-              float p0 = ex2_approx(fmaf(__uint_as_float(sv[c]), c2, -lse2));
-              float p1 = ex2_approx(fmaf(__uint_as_float(sv[c + 1]), c2, -lse2));
-              if (kvmask != 0xffffffffu) {
-                p0 = ((kvmask >> c) & 1u) ? p0 : 0.f;
-                p1 = ((kvmask >> (c + 1)) & 1u) ? p1 : 0.f;
-              }
+              const float p0 = ex2_approx(fmaf(__uint_as_float(sv[c]), c2, -lse2));
+              const float p1 = ex2_approx(fmaf(__uint_as_float(sv[c + 1]), c2, -lse2));
               sv[c] = __float_as_uint(p0);
               sv[c + 1] = __float_as_uint(p1);
               if constexpr (SPLIT) split_bf16x2(p0, p1, pp[c >> 1], pl[c >> 1]);
@@ -386,7 +422,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             tc::mbar_arrive(&misc->p_ready);
           }
           {
-            uint32_t dp[32], pd[16], pdl[SPLIT ? 16 : 1];
+            uint32_t dp[32], pd[16], pdl[SPLIT ? 16 : 1], ph[SPLIT && STORES_DS ? 16 : 1];
             VSA2_WAIT(&misc->dp_full[s], par);
             tc::tc_fence_after();
             tc::tmem_ld32(lane_addr + 128 + s * 64 + half * 32, dp);
@@ -399,10 +435,21 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               const float d1 = __uint_as_float(sv[c + 1]) * (__uint_as_float(dp[c + 1]) - dlt);
               if constexpr (SPLIT) {
                 split_bf16x2(d0, d1, pd[c >> 1], pdl[c >> 1]);
+                if constexpr (STORES_DS) ph[c >> 1] = pack_f16x2(d0, d1);
               } else if constexpr (F16 != 0) {
-                pd[c >> 1] = pack_f16x2_sat(d0, d1);     // (a dS at the clamp: the dQ pass has met the same value and raised the flag)
+                // (a dS beyond the range: the recomputing dQ pass, which runs first, has met the same value and raised the flag,
+                //  or the pass behind this one finds the infinity in the scratch)
+                pd[c >> 1] = pack_f16x2(d0, d1);
               } else {
                 pd[c >> 1] = pack_bf16x2(d0, d1);
+              }
+            }
+            if (SPLIT && STORES_DS && ds_slot >= 0) {
+              // [chunk of 8 keys][query row]: 512 contiguous bytes per warp and store
+              uint4* dst = reinterpret_cast<uint4*>(a.ds + (size_t)ds_slot * kSlab) + half * 256 + (row & 63);
+#pragma unroll
+              for (int ch = 0; ch < 4; ++ch) {
+                if constexpr (SPLIT && STORES_DS) dst[ch * 64] = make_uint4(ph[4 * ch], ph[4 * ch + 1], ph[4 * ch + 2], ph[4 * ch + 3]);
               }
             }
             VSA2_WAIT(&misc->ds_free[0], (tg & 1) ^ 1);
@@ -535,7 +582,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, int* item_list, const void* q16,
-                                   const void* k16, void* v16, void* do16) {
+                                   const void* k16, void* v16, void* do16, const StoredDs* sd) {
   if (g.rep > kMaxRep) return cudaErrorInvalidValue;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16;
   // GQA groups without a precision flag take the all-fp16 form when they are given scratch for fp16 copies of V and dO as
@@ -560,7 +607,6 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   cudaError_t e;
   if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
   const int total = g.batch * g.Hkv * g.N;
-  const int grid = total < sms ? total : sms;
   const bool mha = g.rep == 1;
 #define VSA2_LAUNCH_DKV(DD, SP, MH, F, TQ, TK, TQT, TKT, TV, TDO, TVT, TDOT)                                                                         \
   do {                                                                                                                           \
@@ -578,9 +624,12 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   } while (0)
   // `overlap`: the launch may start while the launch before it in the stream is still running (programmatic dependent
   // launch; that one releases it at its start and the two touch disjoint outputs).  `when`: see DkvArgs.
-  auto launch = [&](bool split, int counter_slot, int k_lo, int k_hi, const int* list, bool overlap, int when) -> cudaError_t {
+  // `group0`, `groups`: range of KV heads (batch * Hkv index); `ds`: the launch stores dS, counting on a counter of its own.
+  auto launch = [&](bool split, int* counter, int k_lo, int k_hi, const int* list, bool overlap, int when, int group0, int groups,
+                    bool ds) -> cudaError_t {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    const int items = groups * g.N;
+    cfg.gridDim = dim3(items < sms ? items : sms);
     cfg.blockDim = dim3(kDkvThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -588,8 +637,9 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    DkvArgs a{&status->pad[counter_slot], lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi,
-              &status->pad[kRangeFlagSlot], when, list};
+    DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
+              group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
+              group0 * g.rep, list};
     if (when == 1 && gqa16) {       // every product in fp16
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
       else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
@@ -611,26 +661,44 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   };
 #undef VSA2_LAUNCH_DKV
   constexpr int kAll = 0x7fffffff;
+  const int all = g.batch * g.Hkv;
+  int* range_flag = &status->pad[kRangeFlagSlot];
+  // Launches over all items; or, with `sd`, over as many KV groups at a time as the scratch holds, the dQ pass of these groups
+  // behind each
+  auto main_pass = [&](bool split, int when) -> cudaError_t {
+    if (sd == nullptr) return launch(split, &status->pad[3], 0, kAll, nullptr, false, when, 0, all, false);
+    cudaError_t r;
+    for (int c = 0, g0 = 0; g0 < all; ++c, g0 += sd->chunk_groups) {
+      const int n = all - g0 < sd->chunk_groups ? all - g0 : sd->chunk_groups;
+      if ((r = launch(split, sd->counters + 2 * c, 0, kAll, nullptr, false, when, g0, n, true)) != cudaSuccess) return r;
+      if ((r = launch_fine_bwd_dq_ds(g, k16, sd->scratch, g0 * g.rep, n * g.rep, sd->row_ptr, sd->col_idx, sd->dqc, sd->dq, status,
+                                     range_flag, sd->counters + 2 * c + 1, !split, st)) != cudaSuccess)
+        return r;
+    }
+    // dQ again, from bf16 pairs, if a value left the fp16 range
+    return launch_fine_bwd_dq_fallback(g, q, k, v, d_o, lse, delta, sd->row_ptr, sd->col_idx, sd->dqc, sd->dq, status, st);
+  };
   if (f16 && gqa16) {
     if ((e = launch_cast_bf16_to_f16(v, v16, (size_t)g.batch * g.Hkv * g.S * g.D, d_o, do16, (size_t)g.batch * g.Hq * g.S * g.D,
-                                     &status->pad[kRangeFlagSlot], st)) != cudaSuccess)
+                                     range_flag, st)) != cudaSuccess)
       return e;
-    if ((e = launch(false, 3, 0, kAll, nullptr, false, 1)) != cudaSuccess) return e;
-    return launch(true, 4, 0, kAll, nullptr, false, 2);
+    if ((e = main_pass(false, 1)) != cudaSuccess) return e;
+    return launch(true, &status->pad[4], 0, kAll, nullptr, false, 2, 0, all, false);
   }
-  if (fine_bwd_dkv_wants_pair(g)) return launch(true, 3, 0, kAll, nullptr, false, 0);
-  if (!fine_bwd_dkv_splits_long_columns(g, split_long_columns)) return launch(false, 3, 0, kAll, nullptr, false, 0);
+  if (fine_bwd_dkv_wants_pair(g)) return main_pass(true, 0);
+  if (!fine_bwd_dkv_splits_long_columns(g, split_long_columns))
+    return launch(false, &status->pad[3], 0, kAll, nullptr, false, 0, 0, all, false);
   // With the fp16 copies of Q and K: one launch in the fp16 form; the two launches below then run only if the range flag
   // came up (in the dQ pass or in this launch), on counters of their own.
   int when = 0, slot_plain = 3;
   if (f16) {
-    if ((e = launch(false, 3, 0, kAll, nullptr, false, 1)) != cudaSuccess) return e;
+    if ((e = main_pass(false, 1)) != cudaSuccess) return e;
     when = 2;
     slot_plain = 5;
   }
   if (item_list == nullptr) {
-    if ((e = launch(false, slot_plain, 0, kDkvLongColumn, nullptr, false, when)) != cudaSuccess) return e;
-    return launch(true, 4, kDkvLongColumn + 1, kAll, nullptr, false, when);
+    if ((e = launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, nullptr, false, when, 0, all, false)) != cudaSuccess) return e;
+    return launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, nullptr, false, when, 0, all, false);
   }
   // The long lists are a few hundred of the items: a small kernel collects them, the pair launch starts on them at once
   // (a handful of 0.3 ms items on 148 CTAs: it would end with most SMs idle), and the plain launch fills the SMs as the
@@ -638,8 +706,8 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   if ((e = cudaMemsetAsync(item_list, 0, sizeof(int), st)) != cudaSuccess) return e;
   dkv_list_items_kernel<<<(total + 255) / 256, 256, 0, st>>>(g, col_ptr, g.rep, total, kDkvLongColumn + 1, kAll, item_list);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch(true, 4, kDkvLongColumn + 1, kAll, item_list, false, when)) != cudaSuccess) return e;
-  return launch(false, slot_plain, 0, kDkvLongColumn, nullptr, true, when);
+  if ((e = launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, item_list, false, when, 0, all, false)) != cudaSuccess) return e;
+  return launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, nullptr, true, when, 0, all, false);
 }
 
 // Whether the dK/dV pass of a GQA problem takes its all-fp16 form when it is given the scratch for the four copies.  Rows that

@@ -457,13 +457,10 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
   const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr;
   const bf16* qa = f16 ? reinterpret_cast<const bf16*>(q16) : q;      // (same element size and layout: the maps only move bytes)
   const bf16* ka = f16 ? reinterpret_cast<const bf16*>(k16) : k;
-  CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq0, tk0, tqt0, tkt0;
+  CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot;
   if (!make_cube_tmap(&tq, qa, g, g.Hq) || !make_cube_tmap(&tk, ka, g, g.Hkv) || !make_cube_tmap(&tv, v, g, g.Hkv) ||
       !make_cube_tmap(&tdo, d_o, g, g.Hq) || !make_text_tmap(&tqt, qa, g, g.Hq) || !make_text_tmap(&tkt, ka, g, g.Hkv) ||
       !make_text_tmap(&tvt, v, g, g.Hkv) || !make_text_tmap(&tdot, d_o, g, g.Hq))
-    return cudaErrorInvalidValue;
-  if (f16 && (!make_cube_tmap(&tq0, q, g, g.Hq) || !make_cube_tmap(&tk0, k, g, g.Hkv) || !make_text_tmap(&tqt0, q, g, g.Hq) ||
-              !make_text_tmap(&tkt0, k, g, g.Hkv)))
     return cudaErrorInvalidValue;
   int sms = 0;
   cudaError_t e;
@@ -488,11 +485,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
     if (g.D == 128) VSA2_LAUNCH_DQ(128, false, true, tq, tk, tqt, tkt);
     else VSA2_LAUNCH_DQ(64, false, true, tq, tk, tqt, tkt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    a.when = 2;
-    a.item_counter = &status->pad[kRangeFlagSlot + 1];     // (its own counter: the fp16 launch has used the other)
-    if (g.D == 128) VSA2_LAUNCH_DQ(128, true, false, tq0, tk0, tqt0, tkt0);
-    else VSA2_LAUNCH_DQ(64, true, false, tq0, tk0, tqt0, tkt0);
-    return cudaGetLastError();
+    return launch_fine_bwd_dq_fallback(g, q, k, v, d_o, lse, delta, row_ptr, col_idx, dqc, dq, status, st);
   }
   if (g.D == 128) {
     if (split) VSA2_LAUNCH_DQ(128, true, false, tq, tk, tqt, tkt);
@@ -501,9 +494,29 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
     if (split) VSA2_LAUNCH_DQ(64, true, false, tq, tk, tqt, tkt);
     else VSA2_LAUNCH_DQ(64, false, false, tq, tk, tqt, tkt);
   }
-#undef VSA2_LAUNCH_DQ
   return cudaGetLastError();
 }
+
+// The pair form of the pass behind a range flag: returns at once unless the flag came up
+cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse,
+                                        const float* delta, const int* row_ptr, const int* col_idx, const float* dqc, void* dq,
+                                        StatusBlock* status, cudaStream_t st) {
+  CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot;
+  if (!make_cube_tmap(&tq, q, g, g.Hq) || !make_cube_tmap(&tk, k, g, g.Hkv) || !make_cube_tmap(&tv, v, g, g.Hkv) ||
+      !make_cube_tmap(&tdo, d_o, g, g.Hq) || !make_text_tmap(&tqt, q, g, g.Hq) || !make_text_tmap(&tkt, k, g, g.Hkv) ||
+      !make_text_tmap(&tvt, v, g, g.Hkv) || !make_text_tmap(&tdot, d_o, g, g.Hq))
+    return cudaErrorInvalidValue;
+  int sms = 0;
+  cudaError_t e;
+  if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
+  DqArgs a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, dq, status, &status->pad[kRangeFlagSlot], 2};
+  const int total = g.batch * g.Hq * g.N;
+  const int grid = total < sms ? total : sms;
+  if (g.D == 128) VSA2_LAUNCH_DQ(128, true, false, tq, tk, tqt, tkt);
+  else VSA2_LAUNCH_DQ(64, true, false, tq, tk, tqt, tkt);
+  return cudaGetLastError();
+}
+#undef VSA2_LAUNCH_DQ
 
 cudaError_t launch_cast_bf16_to_f16(const bf16* a, void* a16, size_t na, const bf16* b, void* b16, size_t nb, int* range_flag,
                                     cudaStream_t st) {

@@ -61,11 +61,12 @@ __device__ __forceinline__ bool bwd_queue_get(BwdQueue* q, uint32_t seq, int lan
   int4 REC;                                                                              \
   if (!bwd_queue_get(&misc->queue, (SEQ), lane, REC, &misc->abort_flag)) goto done;      \
   if (REC.x < 0) break
-// scheduler warp: draws items until the counter (or the list) runs out.  `ptr`, `rep`: start pointers of the lists, an item has
-// those of `rep` consecutive heads; items with fewer than k_lo or more than k_hi entries are left out.
-__device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int heads, int rep, const int* ptr, int* counter,
-                                             const int* list, int k_lo, int k_hi, int lane, volatile int* abort_flag) {
-  const int total = list != nullptr ? list[0] : g.batch * heads * g.N;
+// scheduler warp: draws the items first_item .. first_item + items - 1 (or those of a list) until the counter runs out.  `ptr`,
+// `rep`: start pointers of the lists, an item has those of `rep` consecutive heads; items with fewer than k_lo or more than k_hi
+// entries are left out.
+__device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int first_item, int items, int rep, const int* ptr,
+                                             int* counter, const int* list, int k_lo, int k_hi, int lane, volatile int* abort_flag) {
+  const int total = list != nullptr ? list[0] : items;
   uint32_t drawn = 0;
   for (uint32_t p = 0;; ++p) {
     const uint32_t slot = p % kItemSlots;
@@ -79,7 +80,7 @@ __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int head
       n = __shfl_sync(0xffffffffu, n, 0);
       ++drawn;
       if (n >= total) break;
-      item_block(g, list != nullptr ? list[1 + n] : n, rec.y, rec.x);
+      item_block(g, list != nullptr ? list[1 + n] : first_item + n, rec.y, rec.x);
       int beg = 0, k = 0;
       if (lane < rep) {      // (heads of a group are neighbours: b * Hq + hk * rep + hh)
         const int* c = ptr + ((size_t)rec.y * rep + lane) * (g.N + 1) + rec.x;
@@ -121,6 +122,20 @@ __device__ __forceinline__ void store_channels(void* out, int out_f32, size_t he
   }
 }
 
+struct DqDsArgs {
+  int* item_counter;    // global, zero before the launch
+  const int* row_ptr;
+  const int* col_idx;
+  const unsigned char* ds;
+  int ds_swizzled;      // layout of the tiles, see fine_bwd_dkv_tc.cu
+  const float* dqc;     // [B, Hq, N, D] or null
+  void* dq;
+  StatusBlock* status;
+  int* range_flag;      // the launch runs if it is clear, and sets it if a dS had left the fp16 range
+  int head0;            // (batch * Hq) index of the first head of the dS scratch
+  int first_item, items;
+};
+
 struct BwdMisc {
   uint64_t st_full, st_empty, o_full[2], o_empty[2];       // (the dQ pass uses one accumulator)
   uint64_t a_full[kRingA], a_empty[kRingA], b_full[kRingB], b_empty[kRingB];
@@ -128,8 +143,10 @@ struct BwdMisc {
   uint64_t p_ready, p_free;                                 // dK/dV pass: the P operand buffer
   uint64_t ds_ready[2], ds_free[2];                         // dS operand buffers (the dK/dV pass has one)
   uint64_t stat_full, stat_free;                            // dK/dV pass: the per-row statistics of a tile
-  ItemQueue items;                                          // dQ pass: work items of this CTA (see tc_attn.cuh)
-  BwdQueue queue;                                           // dK/dV pass
+  union {                                                   // work items of this CTA
+    ItemQueue items;                                        // dQ pass (see tc_attn.cuh)
+    BwdQueue queue;                                         // dK/dV pass
+  };
   uint64_t e_sync;                                          // group barrier of the 256 elementwise threads
   uint32_t tmem_base;
   int abort_flag;
@@ -138,6 +155,7 @@ struct BwdMisc {
   // parity tb, lse * log2(e) (+inf for padding) and delta.  dK/dV pass: (lse * log2(e), delta) of the 128 query rows of
   // the current tile, interleaved.
   alignas(16) float stats[256];
+  int ds_slot[4][2];               // dK/dV pass: places of a tile's two dS blocks in the scratch (-1: none), by tile index mod 4
   int tok[128];                    // raster tokens of the rows of an item's block, by parity (dK/dV pass: of the items with entries)
 };
 static_assert(sizeof(BwdMisc) <= 2048, "misc region too small");
