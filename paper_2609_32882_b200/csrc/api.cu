@@ -239,7 +239,7 @@ size_t bwd_workspace_bytes(const Geo& g) {
 // (one head of 720p at a time: 10 blocks per SM), more scratch gains nothing.
 constexpr size_t kStoredDsBytes = (size_t)7 << 30;
 struct DsLayout {
-  size_t counters, pos, tiles, total;
+  size_t counters, pos, order, tiles, total;
   int groups;          // KV groups per chunk, 0: no stored dS
 };
 DsLayout ds_layout(const Geo& g, size_t avail_total, bool preferred) {
@@ -252,6 +252,7 @@ DsLayout ds_layout(const Geo& g, size_t avail_total, bool preferred) {
   c.off = align_up(bwd_workspace_bytes(g), 256);
   r.counters = c.take(2 * all * sizeof(int));
   r.pos = c.take((size_t)g.batch * g.Hq * x.nnz_cap * sizeof(int));
+  r.order = c.take(all * x.N * sizeof(int));
   r.tiles = c.off;
   const size_t room = preferred ? kStoredDsBytes : avail_total > r.tiles ? avail_total - r.tiles : 0;
   const size_t fit = room / group < all ? room / group : all;
@@ -629,7 +630,9 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   // dS kept from the dK/dV pass for the dQ pass, which then runs inside it; otherwise the dQ pass recomputes dS and runs first
   const DsLayout dl = ds_layout(g, workspace_bytes, false);
   const int ds_groups = dl.groups;
-  const StoredDs sd{at<unsigned char>(workspace, dl.tiles), at<int>(workspace, dl.pos), at<int>(workspace, dl.counters), ds_groups,
+  // (a few items per SM end together whatever their order)
+  int* dkv_order = ds_groups > 0 && (long long)ds_groups * fx.N > 4 * 148 ? at<int>(workspace, dl.order) : nullptr;
+  const StoredDs sd{at<unsigned char>(workspace, dl.tiles), at<int>(workspace, dl.pos), at<int>(workspace, dl.counters), dkv_order, ds_groups,
                     row_ptr, col_idx, coarse ? dqc : nullptr, dq};
   // cubes of 128 tokens: both passes on 128 x 128 tiles
   const bool wide128 = wide && g.Lt == 0 && fine_bwd128_supported(n);
@@ -643,6 +646,10 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
                                         &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
       VSA2_CUDA(launch_ds_positions(fx, row_ptr, col_idx, col_ptr, row_idx, at<int>(workspace, dl.pos), sd.counters,
                                     2 * g.batch * g.Hkv, st));
+      if (dkv_order != nullptr) {
+        g_launches += 1;
+        VSA2_CUDA(launch_dkv_order(fx, col_ptr, dkv_order, st));
+      }
     } else if (wide128)
       VSA2_CUDA(launch_fine_bwd128_dq_tc(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
                                          reinterpret_cast<StatusBlock*>(workspace), st,

@@ -300,6 +300,7 @@ struct StoredDs {
   void* scratch;        // chunk_groups * rep * nnz_cap tiles of 8 KB (64 queries x 64 keys, fp16)
   const int* pos;       // [B, Hq, nnz_cap], filled by launch_ds_positions
   int* counters;        // two words per chunk, cleared by launch_ds_positions
+  int* order;           // null, or [B, Hkv, N]: items of the dK/dV pass, longest lists of a group first (launch_dkv_order)
   int chunk_groups;
   const int* row_ptr;
   const int* col_idx;
@@ -308,6 +309,7 @@ struct StoredDs {
 };
 cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col_idx, const int* col_ptr, const int* row_idx, int* pos,
                                 int* counters, int n_counters, cudaStream_t st);
+cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st);
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
                                   int* item_counter, bool swizzled, cudaStream_t st);

@@ -30,6 +30,7 @@ struct DkvArgs {
   unsigned char* ds;    // null, or the scratch for dS in fp16 (forms STORES_DS): [entry of the row lists of heads ds_head0 ..][8 chunks of 8 keys][64 q]
   const int* ds_pos;    // [B, Hq, nnz_cap]: place of every entry of the column lists in the row lists
   int ds_head0;
+  const int* order;     // null, or the order in which the items are drawn
   const int* item_list; // null, or [count, item, item, ...]: the items with k_lo .. k_hi entries (the launch then walks this list
                         // instead of all items: a launch for the few long lists would spend most of its time skipping)
 };
@@ -269,7 +270,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   } else if (warp >= 16 && warp < 20) {
     tc::reg_dec<48>();
-    if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, SPLIT ? a.item_list : nullptr, a.k_lo,
+    if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, SPLIT ? a.item_list : nullptr, a.order, a.k_lo,
                                     a.k_hi, lane, &misc->abort_flag))
       goto done;
     if (F16 != 0 && warp == 19 && a.ds != nullptr) {
@@ -639,7 +640,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     cfg.numAttrs = overlap ? 1 : 0;
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
-              group0 * g.rep, list};
+              group0 * g.rep, ds ? sd->order : nullptr, list};
     if (when == 1 && gqa16) {       // every product in fp16
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
       else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);

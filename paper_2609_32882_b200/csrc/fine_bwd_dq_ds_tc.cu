@@ -195,7 +195,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       if (lane == 0) tc::mbar_arrive(&misc->o_empty[set]);
     }
   } else {
-    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, lane,
+    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, nullptr, 0, 0x7fffffff, lane,
                       &misc->abort_flag))
       goto done;
   }
@@ -245,6 +245,53 @@ cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col
                                 int* counters, int n_counters, cudaStream_t st) {
   ds_positions_kernel<<<dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st>>>(g.N, g.nnz_cap, row_ptr, col_idx, col_ptr, row_idx, pos,
                                                                          counters, n_counters);
+  return cudaGetLastError();
+}
+
+// Items of the dK/dV pass in the order of their list lengths, longest first, group by group (groups stay in order: the CTAs work on
+// one group's tensors at a time, which L2 holds).  A KV block's list can be ten times the mean, and a launch that draws such
+// items last ends with most SMs idle (720p, budget of 16..256 cubes, four heads a group: 0.7 ms for the mean item of a
+// 6 ms launch).  Counting sort by one block per group; the order of equal lengths depends on the run, the results do not.
+__global__ void __launch_bounds__(1024) dkv_order_kernel(Geo g, const int* __restrict__ col_ptr, int* __restrict__ order) {
+  __shared__ int hist[1024], warp_sums[32], longest;
+  const int bhk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto length = [&](int r) {
+    int bh, j, k = 0;
+    item_block(g, bhk * g.N + r, bh, j);
+    for (int hh = 0; hh < g.rep; ++hh) {
+      const int* c = col_ptr + ((size_t)bhk * g.rep + hh) * (g.N + 1) + j;
+      k += c[1] - c[0];
+    }
+    return k;
+  };
+  hist[tid] = 0;
+  if (tid == 0) longest = 0;
+  __syncthreads();
+  int m = 0;
+  for (int r = tid; r < g.N; r += 1024) m = max(m, length(r));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) atomicMax(&longest, m);
+  __syncthreads();
+  const int shift = max(0, 22 - __clz(longest));          // bins of 2^shift entries: longest >> shift < 1024
+  for (int r = tid; r < g.N; r += 1024) atomicAdd(&hist[1023 - (length(r) >> shift)], 1);
+  __syncthreads();
+  const int mine = hist[tid];
+  int incl = mine;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) warp_sums[warp] = incl;
+  __syncthreads();
+  int before = 0;
+  for (int w = 0; w < warp; ++w) before += warp_sums[w];
+  hist[tid] = before + incl - mine;
+  __syncthreads();
+  for (int r = tid; r < g.N; r += 1024) order[bhk * g.N + atomicAdd(&hist[1023 - (length(r) >> shift)], 1)] = bhk * g.N + r;
+}
+
+cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st) {
+  dkv_order_kernel<<<g.batch * g.Hkv, 1024, 0, st>>>(g, col_ptr, order);
   return cudaGetLastError();
 }
 
