@@ -20,7 +20,7 @@ constexpr int kGtTok = 64;        // tokens per CTA tile
 constexpr int kGtCh = 128;        // channels per chunk
 constexpr int kGtThreads = 128;   // four warps
 constexpr int kGtSplits = 16;     // token ranges per batch entry in the dW_g pass
-constexpr int kDxCh = 64;         // channels per chunk of the dX pass (its fp32 staging tile has to fit beside the operands)
+constexpr int kDxCh = 128;        // channels per chunk of the dX pass
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
@@ -39,14 +39,26 @@ __device__ __forceinline__ void ldmatrix_x2_trans(uint32_t& r0, uint32_t& r1, co
 }
 __device__ __forceinline__ uint32_t lds32(const bf16* p) { return *reinterpret_cast<const uint32_t*>(p); }
 
-// X tile: rows l0 .. l0 + 63 of one batch entry, channels c0 .. c0 + 127 -> xs[64][LDX] (zero outside L x C)
 constexpr int kLdx = kGtCh + 8;   // 272-byte rows: 16-byte aligned, and eight consecutive rows cover all 32 banks
-__device__ __forceinline__ void load_x_tile(bf16* xs, const bf16* x, int l0, int L, int c0, int C) {
-  for (int e = threadIdx.x; e < kGtTok * (kGtCh / 8); e += kGtThreads) {
-    const int r = e / (kGtCh / 8), ch = e % (kGtCh / 8);
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (l0 + r < L && c0 + ch * 8 < C) v = __ldg(reinterpret_cast<const uint4*>(x + (size_t)(l0 + r) * C + c0 + ch * 8));
-    *reinterpret_cast<uint4*>(xs + r * kLdx + ch * 8) = v;
+
+// Eight consecutive elements of W, the first of them element i of a chunk whose rows (channels) have Hq heads, into the rows
+// row_of(channel) of a tile of LD elements a row.
+template <int LD, typename RowOf>
+__device__ __forceinline__ void scatter_w(bf16* ws, uint4 v, int i, int Hq, RowOf row_of) {
+  const bf16* e = reinterpret_cast<const bf16*>(&v);
+  int c = i / Hq, h = i - c * Hq;
+  bf16* row = ws + row_of(c) * LD;
+  if (Hq % 8 == 0) {
+    *reinterpret_cast<uint4*>(row + h) = v;
+    return;
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    row[h] = e[u];
+    if (++h == Hq) {
+      h = 0;
+      row = ws + row_of(++c) * LD;
+    }
   }
 }
 
@@ -82,54 +94,107 @@ __global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* __rest
 }
 
 // ---------------------------------------------------------------------------------------------- forward
-// grid (ceil(L / 64), batch); NT = head tiles of 8
-template <int NT>
-__global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, int L,
-                                                              int C, int Hq, float* __restrict__ gate) {
+// MW warps of 16 tokens x KW warps of CH channels each; grid (ceil(L / (16 MW)), batch); NT = head tiles of 8.
+// X goes from global memory straight into the A fragments: the order of the contraction is free, so a thread takes the 16
+// contiguous bytes of channels 8t .. 8t+7 of a group of 32 as its elements of two k-steps (logical k = 2t, 2t+1, 2t+8, 2t+9
+// of step s is channel 8t + 4s + 0 .. 3), and the rows of W lie in that order in shared memory, for ldmatrix.  The loads of the next
+// chunk are in flight while a chunk is multiplied.  Few tokens: KW warps share a token tile and add up at the end.
+template <int NT, int MW, int KW, int CH>
+__global__ void __launch_bounds__(32 * MW * KW) gate_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, int L,
+                                                                int C, int Hq, float* __restrict__ gate) {
   constexpr int LDW = NT * 8 + 8;                           // 16-byte aligned rows, eight rows on different banks
-  __shared__ __align__(16) bf16 xs[kGtTok * kLdx];
-  __shared__ __align__(16) bf16 ws[kGtCh * LDW];            // W chunk as stored: [channel][head]; read by ldmatrix.trans
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int l0 = blockIdx.x * kGtTok, b = blockIdx.y;
-  const bf16* xb = x + (size_t)b * L * C;
-  const bool w_vec = Hq % 8 == 0 && (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
+  constexpr int THREADS = 32 * MW * KW, STEP = KW * CH, GROUPS = CH / 32;
+  __shared__ __align__(16) bf16 ws[STEP * LDW];             // W chunk as stored: [channel][head]; read by ldmatrix.trans
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int mw = warp % MW, kw = warp / MW;
+  const int l0 = blockIdx.x * (16 * MW) + mw * 16, b = blockIdx.y;
+  const bf16* xa = x + ((size_t)b * L + min(l0 + g, L - 1)) * C + kw * CH + t * 8;       // (rows behind the last token repeat it)
+  const bf16* xc = x + ((size_t)b * L + min(l0 + g + 8, L - 1)) * C + kw * CH + t * 8;
+  // (the rows of a chunk of W are contiguous: read as 16-byte vectors whatever the number of heads)
+  const bool w_vec = (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
+  // channel of a chunk -> its row in ws (inside its group of 32: step, upper half, t, parity)
+  auto w_row = [](int c) { return (c & ~31) + ((c >> 2) & 1) * 16 + ((c >> 1) & 1) * 8 + ((c >> 3) & 3) * 2 + (c & 1); };
   float acc[NT][4];
 #pragma unroll
   for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-  for (int c0 = 0; c0 < C; c0 += kGtCh) {
+  constexpr int WV = STEP * NT / THREADS;                   // vectors of a W chunk per thread
+  uint4 ra[GROUPS], rc[GROUPS], rw[WV];
+  for (int e = tid; e < STEP * LDW / 8; e += THREADS) reinterpret_cast<uint4*>(ws)[e] = make_uint4(0, 0, 0, 0);   // (padding heads)
+  auto load = [&](int c0) {
+    if (w_vec) {
+#pragma unroll
+      for (int u = 0; u < WV; ++u) {
+        const int e = tid + u * THREADS;
+        rw[u] = e * 8 < STEP * Hq && c0 * Hq + e * 8 < C * Hq ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq) + e)
+                                                             : make_uint4(0, 0, 0, 0);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < GROUPS; ++q) {
+      const bool in = c0 + kw * CH + q * 32 + t * 8 < C;
+      ra[q] = in ? __ldg(reinterpret_cast<const uint4*>(xa + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
+      rc[q] = in ? __ldg(reinterpret_cast<const uint4*>(xc + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  load(0);
+  for (int c0 = 0; c0 < C; c0 += STEP) {
     __syncthreads();
-    load_x_tile(xs, xb, l0, L, c0, C);
-    if (w_vec && c0 + kGtCh <= C) {
-      // rows of W are whole 16-byte vectors and the chunk is contiguous: copy as such, then clear the padding heads
-      const int vec = Hq / 8;
-      const uint4* src = reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq);
-      for (int e = threadIdx.x; e < kGtCh * vec; e += kGtThreads)
-        *reinterpret_cast<uint4*>(ws + (e / vec) * LDW + (e % vec) * 8) = __ldg(src + e);
-      for (int e = threadIdx.x; e < kGtCh * (NT * 8 - Hq); e += kGtThreads)
-        ws[(e / (NT * 8 - Hq)) * LDW + Hq + e % (NT * 8 - Hq)] = __float2bfloat16_rn(0.f);
+    if (w_vec) {
+#pragma unroll
+      for (int u = 0; u < WV; ++u) {
+        const int e = tid + u * THREADS;
+        if (e * 8 < STEP * Hq) scatter_w<LDW>(ws, rw[u], e * 8, Hq, w_row);
+      }
     } else {
-      for (int e = threadIdx.x; e < kGtCh * NT * 8; e += kGtThreads) {
+      for (int e = tid; e < STEP * NT * 8; e += THREADS) {
         const int c = e / (NT * 8), h = e % (NT * 8);
-        ws[c * LDW + h] = (h < Hq && c0 + c < C) ? w[(size_t)(c0 + c) * Hq + h] : __float2bfloat16_rn(0.f);
+        ws[w_row(c) * LDW + h] = (h < Hq && c0 + c < C) ? w[(size_t)(c0 + c) * Hq + h] : __float2bfloat16_rn(0.f);
       }
     }
     __syncthreads();
-    const bf16* xr = xs + (warp * 16 + g) * kLdx + 2 * t;
+    uint4 ca[GROUPS], cc[GROUPS];
 #pragma unroll
-    for (int ks = 0; ks < kGtCh / 16; ++ks) {
-      uint32_t a[4] = {lds32(xr + ks * 16), lds32(xr + 8 * kLdx + ks * 16), lds32(xr + ks * 16 + 8),
-                       lds32(xr + 8 * kLdx + ks * 16 + 8)};
+    for (int q = 0; q < GROUPS; ++q) {
+      ca[q] = ra[q];
+      cc[q] = rc[q];
+    }
+    if (c0 + STEP < C) load(c0 + STEP);
 #pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        // B fragment (k = channels, n = heads) from the [channel][head] tile: two stored 8 x 8 blocks, transposed
-        uint32_t b0, b1;
-        ldmatrix_x2_trans(b0, b1, ws + (ks * 16 + (lane & 15)) * LDW + n * 8);
-        mma_bf16(acc[n], a, b0, b1);
+    for (int q = 0; q < GROUPS; ++q) {
+#pragma unroll
+      for (int st = 0; st < 2; ++st) {
+        const uint32_t a[4] = {st ? ca[q].z : ca[q].x, st ? cc[q].z : cc[q].x, st ? ca[q].w : ca[q].y, st ? cc[q].w : cc[q].y};
+        const bf16* row = ws + (kw * CH + q * 32 + st * 16 + (lane & 15)) * LDW;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          uint32_t b0, b1;
+          ldmatrix_x2_trans(b0, b1, row + n * 8);
+          mma_bf16(acc[n], a, b0, b1);
+        }
       }
     }
   }
+  if constexpr (KW > 1) {
+    // the KW partial sums of a tile, added in a fixed order by its first warp
+    __syncthreads();
+    float* red = reinterpret_cast<float*>(ws);              // [KW - 1][MW][32 lanes][NT * 4], within the W chunk's space
+    static_assert((KW - 1) * MW * 32 * NT * 4 * 4 <= STEP * LDW * 2, "reduction space");
+    if (kw > 0) {
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) red[(((kw - 1) * MW + mw) * (NT * 4) + n * 4 + e) * 32 + lane] = acc[n][e];
+    }
+    __syncthreads();
+    if (kw > 0) return;
+    for (int o = 0; o < KW - 1; ++o)
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[n][e] += red[((o * MW + mw) * (NT * 4) + n * 4 + e) * 32 + lane];
+  }
   float* gb = gate + (size_t)b * Hq * L;
-  const int tok = l0 + warp * 16 + g;
+  const int tok = l0 + g;
 #pragma unroll
   for (int n = 0; n < NT; ++n) {
     const int h = n * 8 + 2 * t;
@@ -145,18 +210,19 @@ __global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __rest
 }
 
 // ---------------------------------------------------------------------------------------------- dX
-// grid (ceil(L / 64), batch); KT = head tiles of 16 (the contraction)
+// grid (ceil(L / 64), batch, channel slices); KT = head tiles of 16 (the contraction).  Four column tiles of a group of 32
+// channels are interleaved (column n of tile u is channel 8 (n / 2) + 2 u + n % 2), so that a thread's accumulators of the four
+// are 8 neighbouring channels of a token and go to memory as one 16-byte store; no tile is staged for coalescing.
 template <int KT>
 __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __restrict__ w, const bf16* __restrict__ dz_tm,
-                                                                 int L, int Lp, int C, int Hq, int out_f32,
+                                                                 int L, int Lp, int C, int Hq, int per_slice, int out_f32,
                                                                  void* __restrict__ dx) {
   constexpr int LDZ = KT * 16 + 8;
-  constexpr int LDO = kDxCh + 4;
   __shared__ __align__(16) bf16 az[kGtTok * LDZ];            // dz^T: [token][head]
   __shared__ __align__(16) bf16 ws[kDxCh * LDZ];             // W chunk: [channel][head]
-  __shared__ __align__(16) float st[kGtTok * LDO];           // output tile, for coalesced stores
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int l0 = blockIdx.x * kGtTok, b = blockIdx.y;
+  const int c_beg = blockIdx.z * per_slice, c_end = min(C, c_beg + per_slice);
   {
     // the tile's 64 rows of dz_tm are contiguous: 16-byte loads
     const uint4* src = reinterpret_cast<const uint4*>(dz_tm + ((size_t)b * Lp + l0) * (KT * 16));
@@ -165,6 +231,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __r
       *reinterpret_cast<uint4*>(az + tl * LDZ + ch * 8) = __ldg(src + e);
     }
   }
+  for (int e = threadIdx.x; e < kDxCh * LDZ / 8; e += kGtThreads) reinterpret_cast<uint4*>(ws)[e] = make_uint4(0, 0, 0, 0);   // (padding heads)
   __syncthreads();
   uint32_t a[KT][4];
   {
@@ -177,53 +244,50 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __r
       a[ks][3] = lds32(ar + 8 * LDZ + ks * 16 + 8);
     }
   }
-  for (int c0 = 0; c0 < C; c0 += kDxCh) {
-    __syncthreads();                                           // previous chunk's stores have read st, its products ws
-    if (Hq % 8 == 0 && c0 + kDxCh <= C && (reinterpret_cast<uintptr_t>(w) & 15u) == 0) {
-      // rows of W are whole 16-byte vectors: copy them as such, then clear the padding heads
-      const int vec = Hq / 8;
+  const int la = l0 + warp * 16 + g, lb = la + 8;
+  // channel of a chunk -> its row in ws: the eight channels of a column tile lie together
+  auto w_row = [](int c) { return (c & ~31) + ((c >> 1) & 3) * 8 + ((c >> 3) & 3) * 2 + (c & 1); };
+  for (int c0 = c_beg; c0 < c_end; c0 += kDxCh) {
+    __syncthreads();                                           // the previous chunk's products have read ws
+    if ((reinterpret_cast<uintptr_t>(w) & 15u) == 0) {
       const uint4* src = reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq);
-      for (int e = threadIdx.x; e < kDxCh * vec; e += kGtThreads) {
-        const int c = e / vec, v = e % vec;
-        *reinterpret_cast<uint4*>(ws + c * LDZ + v * 8) = __ldg(src + e);
-      }
-      for (int e = threadIdx.x; e < kDxCh * (KT * 16 - Hq); e += kGtThreads) {
-        const int c = e / (KT * 16 - Hq), h = Hq + e % (KT * 16 - Hq);
-        ws[c * LDZ + h] = __float2bfloat16_rn(0.f);
-      }
+      for (int e = threadIdx.x; e * 8 < kDxCh * Hq; e += kGtThreads)
+        scatter_w<LDZ>(ws, c0 * Hq + e * 8 < C * Hq ? __ldg(src + e) : make_uint4(0, 0, 0, 0), e * 8, Hq, w_row);
     } else {
       for (int e = threadIdx.x; e < kDxCh * KT * 16; e += kGtThreads) {
         const int c = e / (KT * 16), h = e % (KT * 16);
-        ws[c * LDZ + h] = (h < Hq && c0 + c < C) ? w[(size_t)(c0 + c) * Hq + h] : __float2bfloat16_rn(0.f);
+        ws[w_row(c) * LDZ + h] = (h < Hq && c0 + c < C) ? w[(size_t)(c0 + c) * Hq + h] : __float2bfloat16_rn(0.f);
       }
     }
     __syncthreads();
-#pragma unroll 4
-    for (int n = 0; n < kDxCh / 8; ++n) {
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const bf16* wr = ws + (n * 8 + g) * LDZ + 2 * t;
+#pragma unroll 2
+    for (int q = 0; q < kDxCh / 32; ++q) {
+      float acc[4][4];
 #pragma unroll
-      for (int ks = 0; ks < KT; ++ks) mma_bf16(acc, a[ks], lds32(wr + ks * 16), lds32(wr + ks * 16 + 8));
-      *reinterpret_cast<float2*>(st + (warp * 16 + g) * LDO + n * 8 + 2 * t) = make_float2(acc[0], acc[1]);
-      *reinterpret_cast<float2*>(st + (warp * 16 + g + 8) * LDO + n * 8 + 2 * t) = make_float2(acc[2], acc[3]);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < kGtTok * (kDxCh / 8); e += kGtThreads) {
-      const int r = e / (kDxCh / 8), ch = e % (kDxCh / 8);
-      if (l0 + r >= L || c0 + ch * 8 >= C) continue;
-      const float4 v0 = *reinterpret_cast<const float4*>(st + r * LDO + ch * 8);
-      const float4 v1 = *reinterpret_cast<const float4*>(st + r * LDO + ch * 8 + 4);
-      const size_t idx = ((size_t)b * L + l0 + r) * C + c0 + ch * 8;
-      if (out_f32) {
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(dx) + idx) = v0;
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(dx) + idx + 4) = v1;
-      } else {
-        __nv_bfloat162 p0 = __floats2bfloat162_rn(v0.x, v0.y), p1 = __floats2bfloat162_rn(v0.z, v0.w);
-        __nv_bfloat162 p2 = __floats2bfloat162_rn(v1.x, v1.y), p3 = __floats2bfloat162_rn(v1.z, v1.w);
-        uint4 o;
-        o.x = *reinterpret_cast<uint32_t*>(&p0); o.y = *reinterpret_cast<uint32_t*>(&p1);
-        o.z = *reinterpret_cast<uint32_t*>(&p2); o.w = *reinterpret_cast<uint32_t*>(&p3);
-        *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(dx) + idx) = o;
+      for (int u = 0; u < 4; ++u) {
+        acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.f;
+        const bf16* wr = ws + (q * 32 + u * 8 + g) * LDZ + 2 * t;
+#pragma unroll
+        for (int ks = 0; ks < KT; ++ks) mma_bf16(acc[u], a[ks], lds32(wr + ks * 16), lds32(wr + ks * 16 + 8));
+      }
+      const int c = c0 + q * 32 + t * 8;                       // (C is a multiple of 8)
+      if (c >= c_end) continue;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const int l = half ? lb : la;
+        if (l >= L) continue;
+        const size_t idx = ((size_t)b * L + l) * C + c;
+        const float* v[4] = {acc[0] + 2 * half, acc[1] + 2 * half, acc[2] + 2 * half, acc[3] + 2 * half};
+        if (out_f32) {
+          float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(dx) + idx);
+          dst[0] = make_float4(v[0][0], v[0][1], v[1][0], v[1][1]);
+          dst[1] = make_float4(v[2][0], v[2][1], v[3][0], v[3][1]);
+        } else {
+          __nv_bfloat162 p[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) p[u] = __floats2bfloat162_rn(v[u][0], v[u][1]);
+          *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(dx) + idx) = *reinterpret_cast<const uint4*>(p);
+        }
       }
     }
   }
@@ -249,16 +313,37 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* __r
   for (int m = 0; m < 2; ++m)
 #pragma unroll
     for (int n = 0; n < NT; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+  // the next tile's loads are in flight while a tile is multiplied
+  constexpr int XV = kGtTok * (kGtCh / 8) / kGtThreads, ZV = (NT * 8 * (kGtTok / 8) + kGtThreads - 1) / kGtThreads;
+  uint4 rx[XV], rz[ZV];
+  auto load = [&](int l0) {
+#pragma unroll
+    for (int u = 0; u < XV; ++u) {
+      const int e = threadIdx.x + u * kGtThreads, r = e / (kGtCh / 8), ch = e % (kGtCh / 8);
+      rx[u] = (l0 + r < L && c0 + ch * 8 < C) ? __ldg(reinterpret_cast<const uint4*>(xb + (size_t)(l0 + r) * C + c0 + ch * 8))
+                                              : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < ZV; ++u) {
+      const int e = threadIdx.x + u * kGtThreads, h = e / (kGtTok / 8), ch = e % (kGtTok / 8);
+      rz[u] = h < HP ? __ldg(reinterpret_cast<const uint4*>(zb + (size_t)h * Lp + l0 + ch * 8)) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  if (l_beg < l_end) load(l_beg);
   for (int l0 = l_beg; l0 < l_end; l0 += kGtTok) {
     __syncthreads();
-    load_x_tile(xs, xb, l0, L, c0, C);
-    for (int e = threadIdx.x; e < NT * 8 * (kGtTok / 8); e += kGtThreads) {
-      const int h = e / (kGtTok / 8), ch = e % (kGtTok / 8);
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (h < HP) v = __ldg(reinterpret_cast<const uint4*>(zb + (size_t)h * Lp + l0 + ch * 8));
-      *reinterpret_cast<uint4*>(dz + h * LDZ + ch * 8) = v;
+#pragma unroll
+    for (int u = 0; u < XV; ++u) {
+      const int e = threadIdx.x + u * kGtThreads;
+      *reinterpret_cast<uint4*>(xs + (e / (kGtCh / 8)) * kLdx + (e % (kGtCh / 8)) * 8) = rx[u];
+    }
+#pragma unroll
+    for (int u = 0; u < ZV; ++u) {
+      const int e = threadIdx.x + u * kGtThreads, h = e / (kGtTok / 8), ch = e % (kGtTok / 8);
+      if (h < NT * 8) *reinterpret_cast<uint4*>(dz + h * LDZ + ch * 8) = rz[u];
     }
     __syncthreads();
+    if (l0 + kGtTok < l_end) load(l0 + kGtTok);
 #pragma unroll
     for (int ks = 0; ks < kGtTok / 16; ++ks) {
       uint32_t a[2][4];
@@ -320,9 +405,16 @@ size_t gate_bwd_workspace_bytes(int batch, int L, int hidden, int heads) {
 }
 
 cudaError_t launch_gate_fwd(int batch, int L, int C, int Hq, const bf16* x, const bf16* w, float* gate, cudaStream_t st) {
-  dim3 grid((L + kGtTok - 1) / kGtTok, batch);
+  // 64 tokens a CTA; with fewer than two such CTAs per SM, 16 tokens and the channels split over four warps (2048 tokens of 1536
+  // channels: 37 us with 64-token CTAs, which leave 116 of 148 SMs without one)
+  const bool few = (long long)batch * ((L + 63) / 64) < 2 * 148;
+  dim3 grid((L + (few ? 15 : 63)) / (few ? 16 : 64), batch);
   const int nt = (Hq + 7) / 8;
-#define VSA2_GATE_FWD(NT_) gate_fwd_kernel<NT_><<<grid, kGtThreads, 0, st>>>(x, w, L, C, Hq, gate)
+#define VSA2_GATE_FWD(NT_)                                                                            \
+  do {                                                                                                \
+    if (few) gate_fwd_kernel<NT_, 1, 4, 64><<<grid, 128, 0, st>>>(x, w, L, C, Hq, gate);              \
+    else gate_fwd_kernel<NT_, 4, 1, 128><<<grid, 128, 0, st>>>(x, w, L, C, Hq, gate);                 \
+  } while (0)
   if (nt <= 1) VSA2_GATE_FWD(1);
   else if (nt <= 2) VSA2_GATE_FWD(2);
   else if (nt <= 4) VSA2_GATE_FWD(4);
@@ -343,9 +435,14 @@ cudaError_t launch_gate_bwd(int batch, int L, int C, int Hq, int out_f32, const 
   gate_dz_kernel<<<dim3(Lp / kGtTok, batch), kGtThreads, (size_t)HP * (kGtTok + 8) * sizeof(bf16), st>>>(gate, dgate, L, Lp, Hq,
                                                                                                    HP, dz_hm, dz_tm);
   {
-    dim3 grid((L + kGtTok - 1) / kGtTok, batch);
+    // channel slices until there are eight CTAs per SM (a chunk is the least a CTA takes)
+    const int tiles = (L + kGtTok - 1) / kGtTok * batch, chunks = (C + kDxCh - 1) / kDxCh;
+    int slices = (8 * 148 + tiles - 1) / tiles;
+    if (slices > chunks) slices = chunks;
+    const int per_slice = (chunks + slices - 1) / slices * kDxCh;
+    dim3 grid((L + kGtTok - 1) / kGtTok, batch, (C + per_slice - 1) / per_slice);
     const int kt = (Hq + 15) / 16;
-#define VSA2_GATE_DX(KT_) gate_bwd_dx_kernel<KT_><<<grid, kGtThreads, 0, st>>>(w, dz_tm, L, Lp, C, Hq, out_f32, dx)
+#define VSA2_GATE_DX(KT_) gate_bwd_dx_kernel<KT_><<<grid, kGtThreads, 0, st>>>(w, dz_tm, L, Lp, C, Hq, per_slice, out_f32, dx)
     if (kt <= 1) VSA2_GATE_DX(1);
     else if (kt <= 2) VSA2_GATE_DX(2);
     else if (kt <= 3) VSA2_GATE_DX(3);

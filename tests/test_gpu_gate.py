@@ -99,3 +99,14 @@ def test_gate_feeds_the_attention_forward():
     geo = orc.Geometry(wl.grid, wl.cube, wl.rpool)
     O_ref, _ = orc.forward(a["q"], a["k"], a["v"], gate_ref, gmask, geo, 1.0 / np.sqrt(wl.head_dim))
     assert_close("O with the projected gate", O, O_ref, bf16_storage=True)
+
+
+@pytest.mark.parametrize("batch,heads,grid,hidden,out_dtype", [
+    (1, 3, (1, 1, 17), 8, vb.F32),             # one group of channels, one token beyond a tile of 16
+    (1, 24, (3, 5, 7), 1000, vb.BF16),         # channels split over warps (few tokens), the last chunk partial
+    (3, 11, (13, 23, 22), 328, vb.F32),        # 64-token tiles (312 of them), rows of W of 22 bytes
+    (1, 64, (19, 32, 32), 136, vb.BF16),       # the same with the most heads
+])
+def test_gate_projection_on_few_and_on_many_tokens(batch, heads, grid, hidden, out_dtype):
+    got, ref, _ = run_gate(batch, heads, grid, hidden, seed=11 * heads + hidden, out_dtype=out_dtype)
+    check(got, ref, out_dtype == vb.BF16)
