@@ -6,43 +6,46 @@
 
 namespace vsa2 {
 
-// One thread per (64-token block, 16-byte channel chunk): it walks the block's tokens four at a time (12 loads in flight),
-// keeps its 8 channels of sum_l gate_l dO_l and of O_c in registers, and the D / 8 threads of a block reduce the two row sums
-// of a token with shuffles -- no shared memory, and a warp's loads cover whole token rows.
+// One CTA of 256 threads per 64-token block: a thread has a 16-byte channel chunk of one token in 256 / (D / 8), two tokens at a time
+// (six loads in flight; four CTAs per SM); the D / 8 threads of a token reduce its two row sums with shuffles.  The sum
+// gate_l dO_l runs over the tokens in order, so the dO rows are left in shared memory for one thread per channel.  (With
+// one thread per chunk walking the block's tokens a small problem waited for sixteen rounds of loads, 21 us.)
 template <int D>
-__global__ void __launch_bounds__(128) bwd_preprocess_kernel(const bf16* __restrict__ d_o, const void* __restrict__ o,
+__global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __restrict__ d_o, const void* __restrict__ o,
                                                              const bf16* __restrict__ o_res,
                                                              const float* __restrict__ gate,
                                                              const float* __restrict__ oc_hat, Geo g,
                                                              float* __restrict__ delta, float* __restrict__ dgate,
                                                              float* __restrict__ d_oc_hat) {
-  constexpr int CH = D / 8;            // threads per block = 16-byte chunks of a token row
-  constexpr int BLOCKS = 128 / CH;     // 64-token blocks per CTA
-  constexpr int TOK = 4;               // tokens in flight per thread
-  const int i = blockIdx.x * BLOCKS + threadIdx.x / CH, ch = threadIdx.x % CH, hq = blockIdx.y, b = blockIdx.z;
-  if (i >= g.N) return;                // (whole shuffle groups leave together)
+  constexpr int CH = D / 8;                // threads per token = 16-byte chunks of a token row
+  constexpr int PAR = 256 / CH;            // tokens at a time
+  constexpr int TOK = 2;                   // tokens in flight per thread
+  __shared__ __align__(16) bf16 rows[kBlockTokens * D];
+  __shared__ float gates[kBlockTokens];
+  const int i = blockIdx.x, ch = threadIdx.x % CH, hq = blockIdx.y, b = blockIdx.z;
   const int lane = threadIdx.x & 31;
   const unsigned group_mask = (CH == 16 ? 0xffffu : 0xffu) << (lane & ~(CH - 1));
   const size_t bhq = (size_t)b * g.Hq + hq;
   // text blocks (i >= Nvid) take no part in the coarse branch or the gate: only delta is formed for them
   const bool coarse = !(g.flags & VSA2_FLAG_NO_COARSE) && gate != nullptr && !block_is_text(g, i);
-  float ocv[8], acc[8];
+  float ocv[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) ocv[e] = acc[e] = 0.f;
+  for (int e = 0; e < 8; ++e) ocv[e] = 0.f;
   if (coarse) {
     const float4* p4 = reinterpret_cast<const float4*>(oc_hat + (bhq * g.Nvid + i) * D + ch * 8);
     const float4 x = __ldg(p4), y = __ldg(p4 + 1);
     ocv[0] = x.x; ocv[1] = x.y; ocv[2] = x.z; ocv[3] = x.w;
     ocv[4] = y.x; ocv[5] = y.y; ocv[6] = y.z; ocv[7] = y.w;
   }
-  for (int p0 = 0; p0 < kBlockTokens; p0 += TOK) {
+#pragma unroll 1
+  for (int p0 = threadIdx.x / CH; p0 < kBlockTokens; p0 += TOK * PAR) {
     int l[TOK];
     float gt[TOK];
     uint4 dv[TOK], ob[TOK], rb[TOK];
     float4 of[TOK][2];
 #pragma unroll
     for (int u = 0; u < TOK; ++u) {
-      l[u] = block_token(g, i, p0 + u);
+      l[u] = block_token(g, i, p0 + u * PAR);
       gt[u] = 0.f;
       dv[u] = ob[u] = rb[u] = make_uint4(0, 0, 0, 0);
       of[u][0] = of[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -61,6 +64,11 @@ __global__ void __launch_bounds__(128) bwd_preprocess_kernel(const bf16* __restr
     }
 #pragma unroll
     for (int u = 0; u < TOK; ++u) {
+      const int p = p0 + u * PAR;
+      if (coarse) {
+        *reinterpret_cast<uint4*>(rows + p * D + ch * 8) = dv[u];
+        if (ch == 0) gates[p] = gt[u];
+      }
       float ov[8], dd[8];
       const __nv_bfloat162* d2 = reinterpret_cast<const __nv_bfloat162*>(&dv[u]);
 #pragma unroll
@@ -85,7 +93,6 @@ __global__ void __launch_bounds__(128) bwd_preprocess_kernel(const bf16* __restr
       for (int e = 0; e < 8; ++e) {
         s_oo = fmaf(dd[e], ov[e], s_oo);
         s_oc = fmaf(dd[e], ocv[e], s_oc);
-        acc[e] = fmaf(gt[u], dd[e], acc[e]);
       }
 #pragma unroll
       for (int off = CH / 2; off >= 1; off >>= 1) {
@@ -98,19 +105,21 @@ __global__ void __launch_bounds__(128) bwd_preprocess_kernel(const bf16* __restr
       }
     }
   }
-  if (coarse) {
-    float4* dst = reinterpret_cast<float4*>(d_oc_hat + (bhq * g.Nvid + i) * D + ch * 8);
-    dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+  if (!coarse) return;
+  __syncthreads();
+  if (threadIdx.x < D) {
+    float acc = 0.f;
+#pragma unroll 16
+    for (int p = 0; p < kBlockTokens; ++p) acc = fmaf(gates[p], __bfloat162float(rows[p * D + threadIdx.x]), acc);
+    d_oc_hat[(bhq * g.Nvid + i) * D + threadIdx.x] = acc;
   }
 }
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
                                   const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, cudaStream_t st) {
-  const int blocks = 128 / (g.D / 8);
-  dim3 grid((g.N + blocks - 1) / blocks, g.Hq, g.batch);
-  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 128, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat);
-  else bwd_preprocess_kernel<64><<<grid, 128, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat);
+  dim3 grid(g.N, g.Hq, g.batch);
+  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat);
+  else bwd_preprocess_kernel<64><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat);
   return cudaGetLastError();
 }
 

@@ -6,8 +6,8 @@
 
 namespace vsa2 {
 
-// One thread per (cube, 16-byte channel chunk): it reads the cube's tokens sub-cube by sub-cube (8 loads in flight for the
-// 2 x 2 x 2 router pool), so no tile is staged in shared memory and a warp's loads cover whole 256-byte token rows.
+// Any router pool other than 2 x 2 x 2: one thread per (cube, 16-byte channel chunk) reads the cube's tokens sub-cube by
+// sub-cube, so no tile is staged in shared memory and a warp's loads cover whole 256-byte token rows.
 //   xr [b, h, N*G, D] bf16 : fp32 sum along w, then h, then t (each left to right; padding positions add +0), IEEE fp32
 //                            division by the valid count, rounded to bf16 (nearest even).
 //   xc [b, h, N, D]   fp32 : sum of the sub-cube sums / count.
@@ -39,7 +39,7 @@ __device__ __forceinline__ void load8(const bf16* base, int t, int h, int w, con
   }
 }
 
-template <int D, bool R222>
+template <int D>
 __global__ void __launch_bounds__(128) pool_kernel(PoolJobs jobs, Geo g) {
   constexpr int CH = D / 8;            // 16-byte chunks of a token row
   constexpr int CUBES = 128 / CH;      // cubes per CTA
@@ -64,28 +64,18 @@ __global__ void __launch_bounds__(128) pool_kernel(PoolJobs jobs, Geo g) {
     const int gw = gsub % g.Gw, r = gsub / g.Gw, gh = r % g.Gh, gt = r / g.Gh;
     const int t0 = nt * g.Bt + gt * g.Rt, h0 = nh * g.Bh + gh * g.Rh, w0 = nw * g.Bw + gw * g.Rw;
     float ts[8];
-    if (R222) {
-      float v[8][8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) load8(base, t0 + (k >> 2), h0 + ((k >> 1) & 1), w0 + (k & 1), g, D, v[k]);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        ts[i] = __fadd_rn(__fadd_rn(__fadd_rn(v[0][i], v[1][i]), __fadd_rn(v[2][i], v[3][i])),
-                          __fadd_rn(__fadd_rn(v[4][i], v[5][i]), __fadd_rn(v[6][i], v[7][i])));
-    } else {
-      for (int it = 0; it < g.Rt; ++it) {
-        float hs[8];
-        for (int ih = 0; ih < g.Rh; ++ih) {
-          float ws[8];
-          for (int iw = 0; iw < g.Rw; ++iw) {
-            float v[8];
-            load8(base, t0 + it, h0 + ih, w0 + iw, g, D, v);
-            add8(ws, v, iw == 0);
-          }
-          add8(hs, ws, ih == 0);
+    for (int it = 0; it < g.Rt; ++it) {
+      float hs[8];
+      for (int ih = 0; ih < g.Rh; ++ih) {
+        float ws[8];
+        for (int iw = 0; iw < g.Rw; ++iw) {
+          float v[8];
+          load8(base, t0 + it, h0 + ih, w0 + iw, g, D, v);
+          add8(ws, v, iw == 0);
         }
-        add8(ts, hs, it == 0);
+        add8(hs, ws, ih == 0);
       }
+      add8(ts, hs, it == 0);
     }
     add8(tot, ts, gsub == 0);
     if (jb.xr != nullptr) {
@@ -108,6 +98,73 @@ __global__ void __launch_bounds__(128) pool_kernel(PoolJobs jobs, Geo g) {
     for (int i = 0; i < 8; ++i) m[i] = cnt > 0.f ? tot[i] / cnt : 0.f;
     *reinterpret_cast<float4*>(dst) = make_float4(m[0], m[1], m[2], m[3]);
     *reinterpret_cast<float4*>(dst + 4) = make_float4(m[4], m[5], m[6], m[7]);
+  }
+}
+
+// The same for the 2 x 2 x 2 router pool with one thread per (sub-cube, 16-byte chunk), for cubes of G = 8 sub-cubes: a CTA has
+// kSubThreads / (D / 8) sub-cubes, whole cubes, whose sub-cube sums meet in shared memory and are added in order.
+// Every load of a thread is in flight at once.  (One thread per cube walks eight sub-cubes one after another, 9 us on
+// the smallest grids.)
+constexpr int kSubThreads = 128;
+template <int D>
+__global__ void __launch_bounds__(kSubThreads) pool_subcube_kernel(PoolJobs jobs, Geo g) {
+  constexpr int CH = D / 8, SUB = kSubThreads / CH, CUBES = SUB / 8;
+  __shared__ __align__(16) float sums[SUB * D];
+  int h = blockIdx.y;
+  PoolJob jb = jobs.job[0];
+  if (jobs.n > 1 && h >= jb.heads) {
+    h -= jb.heads;
+    jb = jobs.job[1];
+    if (jobs.n > 2 && h >= jb.heads) {
+      h -= jb.heads;
+      jb = jobs.job[2];
+    }
+  }
+  const int sub = threadIdx.x / CH, ch = threadIdx.x % CH, b = blockIdx.z;
+  const int n = blockIdx.x * CUBES + (sub >> 3), gsub = sub & 7;
+  const size_t bh = (size_t)b * jb.heads + h;
+  if (n < g.N) {
+    const bf16* base = jb.x + bh * (size_t)g.S * D + ch * 8;
+    int nt, nh, nw;
+    cube_coords(g, n, nt, nh, nw);
+    const int gw = gsub % g.Gw, r = gsub / g.Gw, gh = r % g.Gh, gt = r / g.Gh;
+    const int t0 = nt * g.Bt + gt * 2, h0 = nh * g.Bh + gh * 2, w0 = nw * g.Bw + gw * 2;
+    float v[8][8], ts[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) load8(base, t0 + (k >> 2), h0 + ((k >> 1) & 1), w0 + (k & 1), g, D, v[k]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      ts[i] = __fadd_rn(__fadd_rn(__fadd_rn(v[0][i], v[1][i]), __fadd_rn(v[2][i], v[3][i])),
+                        __fadd_rn(__fadd_rn(v[4][i], v[5][i]), __fadd_rn(v[6][i], v[7][i])));
+    if (jb.xr != nullptr) {
+      const int cnt = max(0, min(2, g.T - t0)) * max(0, min(2, g.H - h0)) * max(0, min(2, g.W - w0));
+      uint4 o = make_uint4(0, 0, 0, 0);
+      if (cnt > 0) {
+        const float c = (float)cnt;
+        __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o2[i] = __floats2bfloat162_rn(__fdiv_rn(ts[2 * i], c), __fdiv_rn(ts[2 * i + 1], c));
+      }
+      *reinterpret_cast<uint4*>(jb.xr + ((bh * g.N + n) * 8 + gsub) * D + ch * 8) = o;
+    }
+    if (jb.xc != nullptr) {
+      float4* dst = reinterpret_cast<float4*>(sums + sub * D + ch * 8);
+      dst[0] = make_float4(ts[0], ts[1], ts[2], ts[3]);
+      dst[1] = make_float4(ts[4], ts[5], ts[6], ts[7]);
+    }
+  }
+  if (jb.xc == nullptr) return;            // (the same for every thread of the CTA)
+  __syncthreads();
+  if (n < g.N) {
+    // kSubThreads threads, CUBES * D means: one each
+    const int cube = threadIdx.x / D, d = threadIdx.x % D, nn = blockIdx.x * CUBES + cube;
+    if (nn < g.N) {
+      float tot = sums[cube * 8 * D + d];
+#pragma unroll
+      for (int q = 1; q < 8; ++q) tot = __fadd_rn(tot, sums[(cube * 8 + q) * D + d]);
+      const float cnt = (float)cube_count(g, nn);
+      jb.xc[(bh * g.N + nn) * D + d] = cnt > 0.f ? tot / cnt : 0.f;
+    }
   }
 }
 
@@ -153,13 +210,15 @@ static cudaError_t launch_pool_jobs(const Geo& g, const PoolJobs& jobs, cudaStre
   const int cubes = 128 / (g.D / 8);
   dim3 grid((g.N + cubes - 1) / cubes, heads, g.batch);
   const bool r222 = g.Rt == 2 && g.Rh == 2 && g.Rw == 2;
-  if (g.D == 128) {
-    if (r222) pool_kernel<128, true><<<grid, 128, 0, st>>>(jobs, g);
-    else pool_kernel<128, false><<<grid, 128, 0, st>>>(jobs, g);
-  } else {
-    if (r222) pool_kernel<64, true><<<grid, 128, 0, st>>>(jobs, g);
-    else pool_kernel<64, false><<<grid, 128, 0, st>>>(jobs, g);
+  if (r222 && g.G == 8) {          // (blocks of 64 tokens have eight such sub-cubes whatever the cube's shape)
+    const int per_cta = kSubThreads / g.D;
+    dim3 sub_grid((g.N + per_cta - 1) / per_cta, heads, g.batch);
+    if (g.D == 128) pool_subcube_kernel<128><<<sub_grid, kSubThreads, 0, st>>>(jobs, g);
+    else pool_subcube_kernel<64><<<sub_grid, kSubThreads, 0, st>>>(jobs, g);
+    return cudaGetLastError();
   }
+  if (g.D == 128) pool_kernel<128><<<grid, 128, 0, st>>>(jobs, g);
+  else pool_kernel<64><<<grid, 128, 0, st>>>(jobs, g);
   return cudaGetLastError();
 }
 

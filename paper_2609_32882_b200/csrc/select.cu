@@ -212,7 +212,55 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
   }
 }
 
-// per-row modes: radix select of the k_i-th largest of row i.  grid (N, BH), 256 threads
+// per-row modes: the k_i-th largest of row i by bisection over the bits of the threshold, a warp per row with the row in registers
+// (U a lane): rounds of U compares and a warp sum until the kept entries are apart from the others (about 20; 32 with ties), no
+// shared memory, no atomics, no block barrier.  grid (ceil(N / 8), BH)
+// (a block per row with 8-bit histograms: 104 us for 7,488 rows of 624, most of it one thread walking the bins)
+template <int U>
+__global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __restrict__ pr, int N, int K,
+                                                                const int* __restrict__ budgets, float* row_tau,
+                                                                int* row_eq_take, int* row_cnt) {
+  const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y;
+  if (i >= N) return;
+  const unsigned* src = reinterpret_cast<const unsigned*>(pr) + ((size_t)bh * N + i) * N;
+  const size_t o = (size_t)bh * N + i;
+  unsigned v[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) v[u] = u * 32 + lane < N ? __ldg(src + u * 32 + lane) : 0u;      // (0 is never above a candidate)
+  int k = budgets ? budgets[o] : K;
+  k = max(0, min(k, N));
+  if (k == 0) {
+    if (lane == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
+    return;
+  }
+  unsigned tau = 0u;            // the largest value with at least k entries >= it
+  for (int bit = 31; bit >= 0; --bit) {
+    const unsigned cand = tau | (1u << bit);
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) c += v[u] >= cand;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (c >= k) tau = cand;
+    if (c == k) {               // exactly the kept entries: the threshold is the smallest of them
+      unsigned m = 0xffffffffu;
+#pragma unroll
+      for (int u = 0; u < U; ++u) m = v[u] >= cand ? min(m, v[u]) : m;
+      tau = __reduce_min_sync(0xffffffffu, m);
+      break;
+    }
+  }
+  int gt = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) gt += v[u] > tau;
+  gt = __reduce_add_sync(0xffffffffu, gt);
+  if (lane == 0) {
+    row_tau[o] = __uint_as_float(tau);
+    row_eq_take[o] = k - gt;
+    row_cnt[o] = k;
+  }
+}
+
+// per-row modes, rows of more than 2048 entries: radix select of the k_i-th largest of row i.  grid (N, BH), 256 threads
 __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restrict__ pr, int N, int K,
                                                            const int* __restrict__ budgets, float* row_tau,
                                                            int* row_eq_take, int* row_cnt) {
@@ -457,8 +505,14 @@ cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, con
     // counts and bitmaps in one read of P_r (the bitmap of the entries equal to tau borrows the transposed bitmap's space)
     sel_row_bits_kernel<<<dim3((N + 7) / 8, BH), 256, 0, st>>>(pr, N, s.words, s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq);
   } else {
-    sel_row_topk_kernel<<<dim3(N, BH), 256, 0, st>>>(pr, N, g.K, g.mode == VSA2_PER_QUERY_BUDGET ? budgets : nullptr,
-                                                     s.row_tau, s.row_eq_take, s.row_cnt);
+    const int* bud = g.mode == VSA2_PER_QUERY_BUDGET ? budgets : nullptr;
+    const dim3 grid((N + 7) / 8, BH);
+    if (N <= 256) sel_row_topk_warp_kernel<8><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+    else if (N <= 640) sel_row_topk_warp_kernel<20><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+    else if (N <= 1024) sel_row_topk_warp_kernel<32><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+    else if (N <= 1536) sel_row_topk_warp_kernel<48><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+    else if (N <= 2048) sel_row_topk_warp_kernel<64><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+    else sel_row_topk_kernel<<<dim3(N, BH), 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
   }
   sel_scan_rows_kernel<<<BH, 1024, 0, st>>>(N, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
                                             s.row_eq_take, s.row_cnt, row_ptr, g.nnz_cap, status);

@@ -1,0 +1,40 @@
+"""Per-query TopK at the row lengths where the kernel takes another form (row held in 8, 20, 32, 48 or 64 registers a lane, or
+histograms of a whole block), with and without ties: the map must be exactly the k largest of the block scores the
+library computed, ties to the lower column, in both its CSR and its CSC form."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_32882_b200 import binding as vb
+from vsa2_testlib import csr_to_mask
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 31, 256, 257, 640, 641, 1024, 1025, 1536, 1537, 2048, 2049])
+@pytest.mark.parametrize("budget", [False, True])
+def test_rows_of_every_register_count(n, budget):
+    torch.manual_seed(n)
+    k = min(n, 13)
+    grid = (4, 4, 4 * n)
+    p = vb.make_params(1, 1, 1, 64, grid, select_mode=vb.PER_QUERY_BUDGET if budget else vb.PER_QUERY, topk=0 if budget else k,
+                       nnz_cap=n * (n // 2 + 1) if budget else 0)
+    attn = vb.Vsa2Attention(p)
+    q = torch.randn(1, 1, 16 * 4 * n, 64, device="cuda", dtype=torch.bfloat16)
+    kk = torch.randn_like(q)
+    if n > 1:
+        kk[:, :, : 16 * 4 * n // 2] = 0.0        # equal scores in half of the sub-cube columns: ties in every row
+        kk = kk.contiguous()
+    budgets = torch.randint(0, n // 2 + 1, (1, 1, n), dtype=torch.int32, device="cuda") if budget else None
+    attn.route(q, kk, budgets)
+    attn.check_status()
+    score = attn.scores()[0, 0].cpu().numpy()
+    rp, ci, cp, ri = (t[0, 0].cpu().numpy() for t in attn.map_views())
+    got = csr_to_mask(rp, ci, n)
+    assert np.array_equal(got, csr_to_mask(cp, ri, n).T)
+    take = budgets[0, 0].cpu().numpy() if budget else np.full(n, k)
+    order = np.argsort(-score, axis=1, kind="stable")
+    want = np.zeros_like(got)
+    for i in range(n):
+        want[i, order[i, : take[i]]] = True
+    assert np.array_equal(got, want)
