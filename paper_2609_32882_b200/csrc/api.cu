@@ -267,11 +267,16 @@ DsLayout ds_layout(const Geo& g, size_t avail_total, bool preferred) {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 bool aligned256(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
 
-// The kernels are built for sm_100a only.
+// The kernels are built for sm_100a only.  (A device's answer does not change: it is asked once.)
 int check_device() {
+  static std::atomic<int> known[kMaxDevices];      // compute capability major
   int dev = 0, major = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return VSA2_ERR_CUDA;
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return VSA2_ERR_CUDA;
+  if (dev < kMaxDevices) major = known[dev].load(std::memory_order_relaxed);
+  if (major == 0) {
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return VSA2_ERR_CUDA;
+    if (dev < kMaxDevices) known[dev].store(major, std::memory_order_relaxed);
+  }
   return major == 10 ? VSA2_OK : VSA2_ERR_UNSUPPORTED;
 }
 
@@ -292,6 +297,38 @@ cudaError_t g_last_cuda_error = cudaSuccess;
 }  // namespace
 
 namespace vsa2 {
+cudaError_t sm_count(int* sms) {
+  static std::atomic<int> known[kMaxDevices];
+  int dev = 0, n = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < kMaxDevices) n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (dev < kMaxDevices) known[dev].store(n, std::memory_order_relaxed);
+  }
+  *sms = n;
+  return cudaSuccess;
+}
+
+cudaError_t prepare_kernel(const void* kernel, KernelAttr& attr, size_t smem, int threads, int least_registers) {
+  int dev = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  const bool known = dev < kMaxDevices;
+  if (known && attr.smem[dev].load(std::memory_order_acquire) >= (int)smem) return cudaSuccess;
+  std::lock_guard<std::mutex> lock(attr.lock);        // (the limit only grows: two threads must not lower it for each other)
+  if (known && attr.smem[dev].load(std::memory_order_relaxed) >= (int)smem) return cudaSuccess;
+  if (least_registers > 0) {
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
+    if (fa.numRegs * threads < least_registers) return cudaErrorLaunchOutOfResources;
+  }
+  if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if (known) attr.smem[dev].store((int)smem, std::memory_order_release);
+  return cudaSuccess;
+}
+
 ProfScope::ProfScope(int kernel_id, cudaStream_t stream, int launches) : id(kernel_id), st(stream) {
   g_launches += launches;
   if (g_prof_start[id] != nullptr) cudaEventRecord(g_prof_start[id], st);
@@ -380,12 +417,11 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
     sel_base += wl.cube_base;
   }
   StatusBlock* status = at<StatusBlock>(workspace, rl.status);
-  VSA2_CUDA(cudaMemsetAsync(status, 0, sizeof(StatusBlock), st));
   bf16* qr = at<bf16>(workspace, rl.qr);
   bf16* kr = at<bf16>(workspace, rl.kr);
   {
     ProfScope ps(VSA2_KERNEL_POOL_ROUTER, st, 1);
-    VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, st));
+    VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, status, st));
   }
   // (half-cubes of 8 sub-cubes: the kernel folds its scores itself)
   const bool folded = wide && r.G == 8;
@@ -417,7 +453,7 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
   s.bitmap_t = at<unsigned>(workspace, lay.bitmap_t);
   s.words = lay.words;
   {
-    ProfScope ps(VSA2_KERNEL_SELECT, st, g.mode == VSA2_PER_SEQUENCE ? 14 : 7);
+    ProfScope ps(VSA2_KERNEL_SELECT, st, (g.mode == VSA2_PER_SEQUENCE ? 14 : 7) - (g.N <= kSelOneBlockN ? 5 : 0));
     VSA2_CUDA(launch_select(g, pr, budgets, s, map->row_ptr, map->col_idx, map->col_ptr, map->row_idx, status, st));
   }
   return VSA2_OK;
@@ -450,7 +486,8 @@ int vsa2_attn_fwd(const vsa2_params* p, const void* q, const void* k, const void
   if (workspace_bytes < fwd_workspace_bytes(g)) return VSA2_ERR_WORKSPACE_TOO_SMALL;
   if ((rc = check_device()) != VSA2_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-  VSA2_CUDA(cudaMemsetAsync(workspace, 0, sizeof(StatusBlock), st));
+  StatusBlock* status = reinterpret_cast<StatusBlock*>(workspace);      // cleared by the first launch
+  if (!coarse) VSA2_CUDA(cudaMemsetAsync(status, 0, sizeof(StatusBlock), st));
   const bf16* qb = reinterpret_cast<const bf16*>(q);
   const bf16* kb = reinterpret_cast<const bf16*>(k);
   const bf16* vb = reinterpret_cast<const bf16*>(v);
@@ -467,14 +504,14 @@ int vsa2_attn_fwd(const vsa2_params* p, const void* q, const void* k, const void
     {
       ProfScope ps(VSA2_KERNEL_POOL, st, wide ? 6 : 1);
       if (!wide) {
-        VSA2_CUDA(launch_pool_coarse(g, qb, kb, vb, saved->qc, saved->kc, saved->vc, st));
+        VSA2_CUDA(launch_pool_coarse(g, qb, kb, vb, saved->qc, saved->kc, saved->vc, status, st));
       } else {
         float* x64 = at<float>(workspace, wl.x64);
-        VSA2_CUDA(launch_pool(n, qb, n.Hq, nullptr, x64, st));
+        VSA2_CUDA(launch_pool(n, qb, n.Hq, nullptr, x64, status, st));
         VSA2_CUDA(launch_fold_mean(n, n.Hq, x64, saved->qc, st));
-        VSA2_CUDA(launch_pool(n, kb, n.Hkv, nullptr, x64, st));
+        VSA2_CUDA(launch_pool(n, kb, n.Hkv, nullptr, x64, nullptr, st));
         VSA2_CUDA(launch_fold_mean(n, n.Hkv, x64, saved->kc, st));
-        VSA2_CUDA(launch_pool(n, vb, n.Hkv, nullptr, x64, st));
+        VSA2_CUDA(launch_pool(n, vb, n.Hkv, nullptr, x64, nullptr, st));
         VSA2_CUDA(launch_fold_mean(n, n.Hkv, x64, saved->vc, st));
       }
     }
@@ -550,7 +587,7 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   if (workspace_bytes < bwd_workspace_bytes(g)) return VSA2_ERR_WORKSPACE_TOO_SMALL;
   if ((rc = check_device()) != VSA2_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-  VSA2_CUDA(cudaMemsetAsync(workspace, 0, sizeof(StatusBlock), st));
+  // (the status block is cleared by the preprocess: the first kernel that could write it comes after)
   // 128-token cubes: preprocess and the fine passes run on the half-cube problem `n` (regions `lay`), the coarse
   // backward at cube level (regions `cl` behind `cube_ws`); folds and expansions link the two
   const bool wide = wide_cube(g);
@@ -612,11 +649,11 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   {
     ProfScope ps(VSA2_KERNEL_BWD_PRE, st, 1);
     VSA2_CUDA(launch_bwd_preprocess(fx, dob, o, o_res, coarse ? gate : nullptr, oc_hat, delta, coarse ? dgate : nullptr,
-                                    d_oc_hat, st));
+                                    d_oc_hat, reinterpret_cast<StatusBlock*>(workspace), st));
   }
   if (coarse) {
-    // pooled grid: four casts, the dense map, the pooled preprocess, dQ, dK/dV (+ two group spreads)
-    ProfScope ps(VSA2_KERNEL_COARSE_BWD, st, 9 + (g.rep > 1 ? 2 : 0) + (wide ? 4 : 0));
+    // pooled grid: the bf16 copies with the dense map, the pooled preprocess, dQ, dK/dV (+ two group spreads)
+    ProfScope ps(VSA2_KERNEL_COARSE_BWD, st, 5 + (g.rep > 1 ? 2 : 0) + (wide ? 4 : 0));
     if (wide) VSA2_CUDA(launch_fold_sum(n, n.Hq, d_oc_hat, d_oc_hat_cube, st));
     VSA2_CUDA(launch_coarse_bwd_pooled(g, saved->qc, saved->kc, saved->vc, saved->oc_hat, saved->lse_c, d_oc_hat_cube,
                                        dqc_cube, dkc_cube, dvc_cube, at<unsigned char>(cube_ws, cl.pooled),
@@ -663,14 +700,11 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   }
   {
     const bool dkv128 = wide128 && !fine_bwd_dkv_wants_pair(n);
-    // scratch for the list of the long column lists (two-launch form): d_oc_hat is dead once the coarse backward has run
-    const size_t list_need = (size_t)fx.batch * fx.Hkv * fx.N + 1, list_have = (size_t)n.batch * n.Hq * n.N * n.D;
-    int* item_list = list_need <= list_have ? reinterpret_cast<int*>(d_oc_hat) : nullptr;
     const bool two = !dkv128 && fine_bwd_dkv_splits_long_columns(fx, true);
     const bool gqa16 = !dkv128 && dkv_pass_gqa_f16(g);    // (the copy of V and dO, the all-fp16 form, the pair form as its fallback)
     const bool f16 = (two || gqa16 || ds_groups > 0) && dq_pass_f16(g);      // fp16 copies of Q and K have been made
     ProfScope ps(VSA2_KERNEL_FINE_BWD_DKV, st, dkv128 ? (dq_pass_f16(g) ? 2 : 1)
-                                                      : two ? (item_list ? 3 : 2) + (f16 ? 1 : 0) : (gqa16 ? 3 : 1));
+                                                      : two ? 2 + (f16 ? 1 : 0) : (gqa16 ? 3 : 1));
     const int chunks = ds_groups > 0 ? (g.batch * g.Hkv + ds_groups - 1) / ds_groups : 0;
     if (chunks > 0) g_launches += 2 * chunks;      // (dQ per chunk and its fallback; the first dK/dV launch is counted above)
     unsigned char* v16 = gqa16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g) + bwd_k16_bytes(g)) : nullptr;
@@ -682,7 +716,7 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
     else
       VSA2_CUDA(launch_fine_bwd_dkv_tc(fx, qb, kb, vb, dob, lse, delta, col_ptr, row_idx, coarse ? dkc : nullptr,
                                        coarse ? dvc : nullptr, dk, dv, reinterpret_cast<StatusBlock*>(workspace), st, true,
-                                       item_list, f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
+                                       f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
                                        f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr, v16,
                                        gqa16 ? v16 + bwd_k16_bytes(g) : nullptr, ds_groups > 0 ? &sd : nullptr));
   }

@@ -16,12 +16,14 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
                                                              const float* __restrict__ gate,
                                                              const float* __restrict__ oc_hat, Geo g,
                                                              float* __restrict__ delta, float* __restrict__ dgate,
-                                                             float* __restrict__ d_oc_hat) {
+                                                             float* __restrict__ d_oc_hat, StatusBlock* clear) {
   constexpr int CH = D / 8;                // threads per token = 16-byte chunks of a token row
   constexpr int PAR = 256 / CH;            // tokens at a time
   constexpr int TOK = 2;                   // tokens in flight per thread
   __shared__ __align__(16) bf16 rows[kBlockTokens * D];
   __shared__ float gates[kBlockTokens];
+  if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(StatusBlock) / 4)
+    reinterpret_cast<int*>(clear)[threadIdx.x] = 0;      // (for the kernels behind this one)
   const int i = blockIdx.x, ch = threadIdx.x % CH, hq = blockIdx.y, b = blockIdx.z;
   const int lane = threadIdx.x & 31;
   const unsigned group_mask = (CH == 16 ? 0xffffu : 0xffu) << (lane & ~(CH - 1));
@@ -116,10 +118,11 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
 }
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
-                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, cudaStream_t st) {
+                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat,
+                                  StatusBlock* clear, cudaStream_t st) {
   dim3 grid(g.N, g.Hq, g.batch);
-  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat);
-  else bwd_preprocess_kernel<64><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat);
+  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, clear);
+  else bwd_preprocess_kernel<64><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, clear);
   return cudaGetLastError();
 }
 

@@ -211,11 +211,13 @@ cudaError_t launch_coarse_fwd_mma(const Geo& g, const float* qc, const float* kc
   cudaError_t e;
   if (g.D == 128) {
     const size_t smb = CoarseFwdSmem<128>::bytes;
-    if ((e = cudaFuncSetAttribute(coarse_fwd_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)coarse_fwd_mma_kernel<128>, attr, smb))) return e;
     coarse_fwd_mma_kernel<128><<<grid, kCfThreads, smb, st>>>(qc, kc, vc, g, oc_hat, lse_c);
   } else {
     const size_t smb = CoarseFwdSmem<64>::bytes;
-    if ((e = cudaFuncSetAttribute(coarse_fwd_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)coarse_fwd_mma_kernel<64>, attr, smb))) return e;
     coarse_fwd_mma_kernel<64><<<grid, kCfThreads, smb, st>>>(qc, kc, vc, g, oc_hat, lse_c);
   }
   return cudaGetLastError();

@@ -47,29 +47,45 @@ PooledLayout pooled_layout(const Geo& g, bool backward) {
   return r;
 }
 
-__global__ void cast_f32_to_bf16_kernel(const float* __restrict__ x, bf16* __restrict__ y, size_t n4) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n4) return;
-  const float4 v = __ldg(reinterpret_cast<const float4*>(x) + i);
-  __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-  uint2 o;
-  o.x = *reinterpret_cast<uint32_t*>(&a);
-  o.y = *reinterpret_cast<uint32_t*>(&b);
-  reinterpret_cast<uint2*>(y)[i] = o;
-}
-
-static cudaError_t cast_to_bf16(const float* x, bf16* y, size_t n, cudaStream_t st) {
-  const size_t n4 = n / 4;      // n is a multiple of the head dimension
-  cast_f32_to_bf16_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(x, y, n4);
-  return cudaGetLastError();
-}
-
 // dense map of np blocks for `heads` lists: ptr[h][i] = i * np, idx[h][i * np + j] = j (its transpose is the same map)
-__global__ void dense_map_kernel(int* __restrict__ ptr, int* __restrict__ idx, int np, int heads) {
-  const int h = blockIdx.x;
-  if (h >= heads) return;
-  for (int i = threadIdx.x; i <= np; i += blockDim.x) ptr[(size_t)h * (np + 1) + i] = i * np;
-  for (int e = threadIdx.x; e < np * np; e += blockDim.x) idx[(size_t)h * np * np + e] = e % np;
+__device__ __forceinline__ void dense_map_entry(int* ptr, int* idx, int np, size_t e) {
+  const size_t per = (size_t)np * np + np + 1, h = e / per;
+  const int r = (int)(e - h * per);
+  if (r <= np) ptr[h * (np + 1) + r] = r * np;
+  else idx[h * np * np + r - np - 1] = (r - np - 1) % np;
+}
+// What the pooled kernels read, in one launch: bf16 copies of up to four fp32 tensors, the dense map, a cleared status block
+struct PooledInputs {
+  const float* x[4];
+  bf16* y[4];
+  size_t n4[4];            // 16-byte groups of each tensor
+  int* ptr;
+  int* idx;
+  int np;
+  size_t map_words;        // heads * (np * np + np + 1)
+  StatusBlock* status;
+};
+__global__ void __launch_bounds__(256) pooled_inputs_kernel(PooledInputs p) {
+  if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
+  const size_t stride = (size_t)gridDim.x * blockDim.x, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    for (size_t i = first; i < p.n4[t]; i += stride) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(p.x[t]) + i);
+      __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+      uint2 o;
+      o.x = *reinterpret_cast<uint32_t*>(&a);
+      o.y = *reinterpret_cast<uint32_t*>(&b);
+      reinterpret_cast<uint2*>(p.y[t])[i] = o;
+    }
+  for (size_t i = first; i < p.map_words; i += stride) dense_map_entry(p.ptr, p.idx, p.np, i);
+}
+static cudaError_t launch_pooled_inputs(const PooledInputs& p, cudaStream_t st) {
+  size_t most = p.map_words;
+  for (size_t n : p.n4) most = n > most ? n : most;
+  const size_t blocks = (most + 255) / 256;
+  pooled_inputs_kernel<<<(unsigned)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st>>>(p);
+  return cudaGetLastError();
 }
 
 // the recursive dK/dV pass returns one gradient per KV head; the epilogues of the main passes sum dK_c, dV_c over the
@@ -104,12 +120,9 @@ cudaError_t launch_coarse_fwd_pooled(const Geo& g, const float* qc, const float*
   int* ptr = reinterpret_cast<int*>(ws + lay.ptr);
   int* idx = reinterpret_cast<int*>(ws + lay.idx);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(ws + lay.status, 0, sizeof(StatusBlock), st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(qc, q16, BHq * g.N * g.D, st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(kc, k16, BHk * g.N * g.D, st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(vc, v16, BHk * g.N * g.D, st)) != cudaSuccess) return e;
-  dense_map_kernel<<<(unsigned)BHq, 256, 0, st>>>(ptr, idx, p.N, (int)BHq);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const PooledInputs in{{qc, kc, vc, nullptr}, {q16, k16, v16, nullptr}, {BHq * g.N * g.D / 4, BHk * g.N * g.D / 4, BHk * g.N * g.D / 4, 0},
+                        ptr, idx, p.N, BHq * ((size_t)p.N * p.N + p.N + 1), reinterpret_cast<StatusBlock*>(ws + lay.status)};
+  if ((e = launch_pooled_inputs(in, st)) != cudaSuccess) return e;
   if ((e = launch_fine_fwd_tc(p, q16, k16, v16, nullptr, ptr, idx, nullptr, oc_hat, nullptr, lse_c,
                               reinterpret_cast<StatusBlock*>(ws + lay.status), st)) != cudaSuccess)
     return e;
@@ -135,19 +148,16 @@ cudaError_t launch_coarse_bwd_pooled(const Geo& g, const float* qc, const float*
   float* dv_kv = reinterpret_cast<float*>(ws + lay.dv_kv);
   StatusBlock* status = reinterpret_cast<StatusBlock*>(ws + lay.status);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(status, 0, sizeof(StatusBlock), st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(qc, q16, BHq * g.N * g.D, st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(kc, k16, BHk * g.N * g.D, st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(vc, v16, BHk * g.N * g.D, st)) != cudaSuccess) return e;
-  if ((e = cast_to_bf16(d_oc_hat, do16, BHq * g.N * g.D, st)) != cudaSuccess) return e;
-  dense_map_kernel<<<(unsigned)BHq, 256, 0, st>>>(ptr, idx, p.N, (int)BHq);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const size_t nq = BHq * g.N * g.D / 4, nk = BHk * g.N * g.D / 4;      // (multiples of the head dimension)
+  const PooledInputs in{{qc, kc, vc, d_oc_hat}, {q16, k16, v16, do16}, {nq, nk, nk, nq},
+                        ptr, idx, p.N, BHq * ((size_t)p.N * p.N + p.N + 1), status};
+  if ((e = launch_pooled_inputs(in, st)) != cudaSuccess) return e;
   // delta_c = rowsum(dO_c * O_c) through the preprocess kernel of the pooled problem (no gate: only delta is written)
-  if ((e = launch_bwd_preprocess(p, do16, oc_hat, nullptr, nullptr, nullptr, delta, nullptr, nullptr, st)) != cudaSuccess) return e;
+  if ((e = launch_bwd_preprocess(p, do16, oc_hat, nullptr, nullptr, nullptr, delta, nullptr, nullptr, nullptr, st)) != cudaSuccess) return e;
   if ((e = launch_fine_bwd_dq_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, dqc, status, st, nullptr, nullptr)) != cudaSuccess) return e;
   const bool grouped = g.rep > 1;
   if ((e = launch_fine_bwd_dkv_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, nullptr, grouped ? dk_kv : dkc,
-                                  grouped ? dv_kv : dvc, status, st, false, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr)) != cudaSuccess)
+                                  grouped ? dv_kv : dvc, status, st, false, nullptr, nullptr, nullptr, nullptr, nullptr)) != cudaSuccess)
     return e;
   if (grouped) {
     const size_t per_head4 = (size_t)g.N * g.D / 4;

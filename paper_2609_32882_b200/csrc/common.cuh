@@ -5,6 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <mutex>
+
 #include "vsa2.h"
 
 namespace vsa2 {
@@ -57,6 +60,19 @@ struct ProfScope {
   ProfScope(int kernel_id, cudaStream_t stream, int launches);
   ~ProfScope();
 };
+
+// Per kernel and device: the dynamic shared memory it has been allowed so far.  A launch asks the driver only when it needs more
+// (each such call costs the host as much as half a launch, and the kernels' needs are constants or grow with the problem).
+constexpr int kMaxDevices = 64;
+struct KernelAttr {
+  std::mutex lock;
+  std::atomic<int> smem[kMaxDevices] = {};
+};
+// `least_registers`: registers the launch has to allocate over all its threads (kernels that redistribute them wait for ever
+// otherwise), checked with `threads` on the first call
+cudaError_t prepare_kernel(const void* kernel, KernelAttr& attr, size_t smem, int threads = 0, int least_registers = 0);
+// number of SMs of the current device (looked up once per device)
+cudaError_t sm_count(int* sms);
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -174,10 +190,11 @@ __device__ __forceinline__ void store_out(void* base, size_t idx, float v, int o
 // ---------------------------------------------------------------------------------------------
 // launchers implemented in the .cu files (all enqueue on `st`, return cudaGetLastError())
 // ---------------------------------------------------------------------------------------------
-cudaError_t launch_pool(const Geo& g, const bf16* x, int heads, bf16* xr, float* xc, cudaStream_t st);
-cudaError_t launch_pool_router(const Geo& g, const bf16* q, const bf16* k, bf16* qr, bf16* kr, cudaStream_t st);
+// (`clear`: null, or a status block that the launch sets to zero for the kernels behind it)
+cudaError_t launch_pool(const Geo& g, const bf16* x, int heads, bf16* xr, float* xc, StatusBlock* clear, cudaStream_t st);
+cudaError_t launch_pool_router(const Geo& g, const bf16* q, const bf16* k, bf16* qr, bf16* kr, StatusBlock* clear, cudaStream_t st);
 cudaError_t launch_pool_coarse(const Geo& g, const bf16* q, const bf16* k, const bf16* v, float* qc, float* kc, float* vc,
-                               cudaStream_t st);
+                               StatusBlock* clear, cudaStream_t st);
 
 // raster <-> cube-major copy of a [batch, heads, L or N*B, D] bf16 tensor (pool.cu)
 cudaError_t launch_permute(const Geo& g, const bf16* src, int heads, bool inverse, bf16* dst, cudaStream_t st);
@@ -191,6 +208,9 @@ bool router_tc_supported(const Geo& g);
 cudaError_t launch_router_scores_tc(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, StatusBlock* status,
                                     cudaStream_t st);
 
+// up to this many cubes one block per head turns the selection into both maps (select.cu): 128 cubes 4.7 us against 12 us and
+// five more launches; at 288 cubes the block takes 40 us and the six launches 18
+constexpr int kSelOneBlockN = 128;
 struct SelectScratch {
   unsigned* hist;        // [BH][3][2048]
   unsigned* state;       // [BH][8]
@@ -319,12 +339,12 @@ cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16*
 cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
-                                   cudaStream_t st, bool split_long_columns, int* item_list, const void* q16,
+                                   cudaStream_t st, bool split_long_columns, const void* q16,
                                    const void* k16, void* v16, void* do16, const StoredDs* sd);
 bool fine_bwd_dkv_gqa_uses_f16(const Geo& g);
 bool fine_bwd_dkv_splits_long_columns(const Geo& g, bool split_long_columns);
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
                                   const float* oc_hat, float* delta, float* dgate, float* d_oc_hat,
-                                  cudaStream_t st);
+                                  StatusBlock* clear, cudaStream_t st);
 }  // namespace vsa2

@@ -761,11 +761,9 @@ template <int D, int PASS, bool SPLIT, bool F16 = false>
 static cudaError_t launch_bwd128(const CUtensorMap& x0, const CUtensorMap& x1, const CUtensorMap& y0, const CUtensorMap& y1,
                                  const Geo& g, const Bwd128Args& a, int grid, cudaStream_t st) {
   cudaError_t e;
-  cudaFuncAttributes fa;
-  if ((e = cudaFuncGetAttributes(&fa, fine_bwd128_tc_kernel<D, PASS, SPLIT, F16>)) != cudaSuccess) return e;
-  if (fa.numRegs * kW2Threads < 256 * 56 + 256 * 200) return cudaErrorLaunchOutOfResources;
-  if ((e = cudaFuncSetAttribute(fine_bwd128_tc_kernel<D, PASS, SPLIT, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)Bwd128<D>::smem_bytes)))
+  static KernelAttr attr;
+  if ((e = prepare_kernel((const void*)fine_bwd128_tc_kernel<D, PASS, SPLIT, F16>, attr, Bwd128<D>::smem_bytes, kW2Threads,
+                          256 * 56 + 256 * 200)))
     return e;
   fine_bwd128_tc_kernel<D, PASS, SPLIT, F16><<<grid, kW2Threads, Bwd128<D>::smem_bytes, st>>>(x0, x1, y0, y1, g, a);
   return cudaGetLastError();
@@ -785,10 +783,9 @@ cudaError_t launch_fine_bwd128_dq_tc(const Geo& g, const bf16* q, const bf16* k,
   if (f16 && (!make_cube_tmap(&tq16, reinterpret_cast<const bf16*>(q16), g, g.Hq) ||      // (same element size and layout)
               !make_cube_tmap(&tk16, reinterpret_cast<const bf16*>(k16), g, g.Hkv)))
     return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
   Bwd128Args a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, nullptr, dq, nullptr, status, flag, 0};
   const int total = g.batch * g.Hq * (g.N / 2);
@@ -827,10 +824,9 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
   if (f16 && (!make_cube_tmap(&tq16, reinterpret_cast<const bf16*>(q16), g, g.Hq) ||
               !make_cube_tmap(&tk16, reinterpret_cast<const bf16*>(k16), g, g.Hkv)))
     return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   Bwd128Args a{&status->pad[3], lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, &status->pad[kRangeFlagSlot], 0};
   const int total = g.batch * g.Hkv * (g.N / 2);
   const int grid = total < sms ? total : sms;

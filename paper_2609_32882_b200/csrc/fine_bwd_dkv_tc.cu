@@ -31,8 +31,6 @@ struct DkvArgs {
   const int* ds_pos;    // [B, Hq, nnz_cap]: place of every entry of the column lists in the row lists
   int ds_head0;
   const int* order;     // null, or the order in which the items are drawn
-  const int* item_list; // null, or [count, item, item, ...]: the items with k_lo .. k_hi entries (the launch then walks this list
-                        // instead of all items: a launch for the few long lists would spend most of its time skipping)
 };
 
 constexpr int kMaxRep = 16;   // query heads per KV head the dK/dV pass supports
@@ -50,32 +48,6 @@ __device__ __forceinline__ void dkv_entry(const Geo& g, const DkvArgs& a, int re
   const size_t at = (size_t)bhq * g.nnz_cap + col_beg[hh] + (e - cnt_prefix[hh]);
   i = a.row_idx[at];
   if (POS && a.ds != nullptr) *pos = a.ds_pos[at];
-}
-
-// The work items whose column lists hold k_lo .. k_hi entries, appended to list[1 ...] with their count in list[0] (zero
-// before the launch).  The order of the list depends on the run; the results do not (an item is a whole KV block).
-__global__ void __launch_bounds__(256) dkv_list_items_kernel(Geo g, const int* __restrict__ col_ptr, int rep, int total,
-                                                             int k_lo, int k_hi, int* list) {
-  const int item = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
-  bool in = false;
-  if (item < total) {
-    int j, bhk;
-    item_block(g, item, bhk, j);
-    const int b = bhk / g.Hkv, hk = bhk % g.Hkv;
-    int kk = 0;
-    for (int hh = 0; hh < rep; ++hh) {
-      const size_t base = (size_t)(b * g.Hq + hk * rep + hh) * (g.N + 1) + j;
-      kk += col_ptr[base + 1] - col_ptr[base];
-    }
-    in = kk >= k_lo && kk <= k_hi;
-  }
-  const unsigned m = __ballot_sync(0xffffffffu, in);
-  if (m == 0u) return;
-  const int leader = __ffs(m) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(&list[0], __popc(m));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if (in) list[1 + base + __popc(m & ((1u << lane) - 1u))] = item;
 }
 
 // Roles: warp 0 = TMA producer of the Q pairs (ring A) and of the stationary K and V tiles, warp 1 = TMA producer of the
@@ -136,9 +108,6 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
   if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
 
-  // the launch of the few long lists lets the launch behind it in the stream (the other lists: disjoint outputs, nothing
-  // read from this one) take the SMs as its CTAs leave them
-  if (SPLIT && a.item_list != nullptr) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     bwd_init_barriers(misc);
     for (int s = 0; s < 2; ++s) {
@@ -270,7 +239,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   } else if (warp >= 16 && warp < 20) {
     tc::reg_dec<48>();
-    if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, SPLIT ? a.item_list : nullptr, a.order, a.k_lo,
+    if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
                                     a.k_hi, lane, &misc->abort_flag))
       goto done;
     if (F16 != 0 && warp == 19 && a.ds != nullptr) {
@@ -577,12 +546,11 @@ constexpr int kDkvLongColumn = 256;
 // the list length (720p sample, fp32 outputs: 6.5e-3 at |dK| = 5.5 with 200 query blocks, 6.3e-3 at 3.0 with 260); the
 // few blocks that nearly every query keeps reach |dK| = 15 and then 1.5e-2 .. 2.7e-2 depending on nothing but where the
 // roundings fall (e.g. whether the softmax scale is applied before or after dS is rounded), i.e. across the stated 2e-2.
-// As pairs they come out at 6e-3.  The first launch walks all items and skips the long lists; the second walks the list of
-// them that a small kernel collects into `item_list` (1 + batch * Hkv * N ints of scratch; null: it walks all items too).
+// As pairs they come out at 6e-3.  Each launch walks all items and skips the other's.
 cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
-                                   cudaStream_t st, bool split_long_columns, int* item_list, const void* q16,
+                                   cudaStream_t st, bool split_long_columns, const void* q16,
                                    const void* k16, void* v16, void* do16, const StoredDs* sd) {
   if (g.rep > kMaxRep) return cudaErrorInvalidValue;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16;
@@ -606,41 +574,31 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     return cudaErrorInvalidValue;
   int sms = 0;
   cudaError_t e;
-  if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
-  const int total = g.batch * g.Hkv * g.N;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   const bool mha = g.rep == 1;
 #define VSA2_LAUNCH_DKV(DD, SP, MH, F, TQ, TK, TQT, TKT, TV, TDO, TVT, TDOT)                                                                         \
   do {                                                                                                                           \
     using L_ = BwdTc<DD, SP ? 2 : kRingA, SP ? 4 : 2>;                                                                           \
-    if ((e = cudaFuncSetAttribute(fine_bwd_dkv_tc_kernel<DD, SP, MH, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
-                                  (int)L_::smem_bytes)))                                                                         \
-      return e;                                                                                                                  \
     cfg.dynamicSmemBytes = L_::smem_bytes;                                                                                       \
-    cudaFuncAttributes fa;                                                                                                       \
-    if ((e = cudaFuncGetAttributes(&fa, (const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F>)) != cudaSuccess) return e;           \
-    /* the warps that raise their register count wait for ever if the launch allocated less than their sum */                    \
-    if (fa.numRegs * kDkvThreads < 128 * (48 + 2 * 120 + 2 * 48 + 96)) return cudaErrorLaunchOutOfResources;                     \
+    static KernelAttr attr_;                                                                                                     \
+    if ((e = prepare_kernel((const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F>, attr_, L_::smem_bytes, kDkvThreads,               \
+                            128 * (48 + 2 * 120 + 2 * 48 + 96))))                                                                \
+      return e;                                                                                                                  \
     if ((e = cudaLaunchKernelEx(&cfg, fine_bwd_dkv_tc_kernel<DD, SP, MH, F>, TQ, TK, TV, TDO, TQT, TKT, TVT, TDOT, g, a)))       \
       return e;                                                                                                                  \
   } while (0)
-  // `overlap`: the launch may start while the launch before it in the stream is still running (programmatic dependent
-  // launch; that one releases it at its start and the two touch disjoint outputs).  `when`: see DkvArgs.
+  // `when`: see DkvArgs.
   // `group0`, `groups`: range of KV heads (batch * Hkv index); `ds`: the launch stores dS, counting on a counter of its own.
-  auto launch = [&](bool split, int* counter, int k_lo, int k_hi, const int* list, bool overlap, int when, int group0, int groups,
+  auto launch = [&](bool split, int* counter, int k_lo, int k_hi, int when, int group0, int groups,
                     bool ds) -> cudaError_t {
     cudaLaunchConfig_t cfg = {};
     const int items = groups * g.N;
     cfg.gridDim = dim3(items < sms ? items : sms);
     cfg.blockDim = dim3(kDkvThreads);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = overlap ? 1 : 0;
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
-              group0 * g.rep, ds ? sd->order : nullptr, list};
+              group0 * g.rep, ds ? sd->order : nullptr};
     if (when == 1 && gqa16) {       // every product in fp16
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
       else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
@@ -667,11 +625,11 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   // Launches over all items; or, with `sd`, over as many KV groups at a time as the scratch holds, the dQ pass of these groups
   // behind each
   auto main_pass = [&](bool split, int when) -> cudaError_t {
-    if (sd == nullptr) return launch(split, &status->pad[3], 0, kAll, nullptr, false, when, 0, all, false);
+    if (sd == nullptr) return launch(split, &status->pad[3], 0, kAll, when, 0, all, false);
     cudaError_t r;
     for (int c = 0, g0 = 0; g0 < all; ++c, g0 += sd->chunk_groups) {
       const int n = all - g0 < sd->chunk_groups ? all - g0 : sd->chunk_groups;
-      if ((r = launch(split, sd->counters + 2 * c, 0, kAll, nullptr, false, when, g0, n, true)) != cudaSuccess) return r;
+      if ((r = launch(split, sd->counters + 2 * c, 0, kAll, when, g0, n, true)) != cudaSuccess) return r;
       if ((r = launch_fine_bwd_dq_ds(g, k16, sd->scratch, g0 * g.rep, n * g.rep, sd->row_ptr, sd->col_idx, sd->dqc, sd->dq, status,
                                      range_flag, sd->counters + 2 * c + 1, !split, st)) != cudaSuccess)
         return r;
@@ -684,11 +642,11 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                      range_flag, st)) != cudaSuccess)
       return e;
     if ((e = main_pass(false, 1)) != cudaSuccess) return e;
-    return launch(true, &status->pad[4], 0, kAll, nullptr, false, 2, 0, all, false);
+    return launch(true, &status->pad[4], 0, kAll, 2, 0, all, false);
   }
   if (fine_bwd_dkv_wants_pair(g)) return main_pass(true, 0);
   if (!fine_bwd_dkv_splits_long_columns(g, split_long_columns))
-    return launch(false, &status->pad[3], 0, kAll, nullptr, false, 0, 0, all, false);
+    return launch(false, &status->pad[3], 0, kAll, 0, 0, all, false);
   // With the fp16 copies of Q and K: one launch in the fp16 form; the two launches below then run only if the range flag
   // came up (in the dQ pass or in this launch), on counters of their own.
   int when = 0, slot_plain = 3;
@@ -697,18 +655,8 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     when = 2;
     slot_plain = 5;
   }
-  if (item_list == nullptr) {
-    if ((e = launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, nullptr, false, when, 0, all, false)) != cudaSuccess) return e;
-    return launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, nullptr, false, when, 0, all, false);
-  }
-  // The long lists are a few hundred of the items: a small kernel collects them, the pair launch starts on them at once
-  // (a handful of 0.3 ms items on 148 CTAs: it would end with most SMs idle), and the plain launch fills the SMs as the
-  // pair launch's CTAs leave them.
-  if ((e = cudaMemsetAsync(item_list, 0, sizeof(int), st)) != cudaSuccess) return e;
-  dkv_list_items_kernel<<<(total + 255) / 256, 256, 0, st>>>(g, col_ptr, g.rep, total, kDkvLongColumn + 1, kAll, item_list);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, item_list, false, when, 0, all, false)) != cudaSuccess) return e;
-  return launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, nullptr, true, when, 0, all, false);
+  if ((e = launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, when, 0, all, false)) != cudaSuccess) return e;
+  return launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, when, 0, all, false);
 }
 
 // Whether the dK/dV pass of a GQA problem takes its all-fp16 form when it is given the scratch for the four copies.  Rows that

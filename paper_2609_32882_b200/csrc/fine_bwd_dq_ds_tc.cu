@@ -195,7 +195,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       if (lane == 0) tc::mbar_arrive(&misc->o_empty[set]);
     }
   } else {
-    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, nullptr, 0, 0x7fffffff, lane,
+    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, lane,
                       &misc->abort_flag))
       goto done;
   }
@@ -305,14 +305,13 @@ cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds,
     return cudaErrorInvalidValue;
   int sms = 0;
   cudaError_t e;
-  if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), swizzled ? 1 : 0, dqc, dq, status, range_flag, head0, head0 * g.N, heads * g.N};
   const int grid = a.items < sms ? a.items : sms;
 #define VSA2_LAUNCH_DQ_DS(DD)                                                                                                    \
   do {                                                                                                                           \
-    if ((e = cudaFuncSetAttribute(fine_bwd_dq_ds_kernel<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize,                        \
-                                  (int)DqDs<DD>::smem_bytes)))                                                                   \
-      return e;                                                                                                                  \
+    static KernelAttr attr_;                                                                                                     \
+    if ((e = prepare_kernel((const void*)fine_bwd_dq_ds_kernel<DD>, attr_, DqDs<DD>::smem_bytes))) return e;                     \
     fine_bwd_dq_ds_kernel<DD><<<grid, kDsThreads, DqDs<DD>::smem_bytes, st>>>(tk, tkt, g, a);                               \
   } while (0)
   if (g.D == 128) VSA2_LAUNCH_DQ_DS(128);

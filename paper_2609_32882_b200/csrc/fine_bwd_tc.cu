@@ -464,7 +464,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
     return cudaErrorInvalidValue;
   int sms = 0;
   cudaError_t e;
-  if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
   DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, status, flag, 0};
   const int total = g.batch * g.Hq * g.N;
@@ -472,9 +472,8 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
   const bool split = !(g.flags & VSA2_FLAG_FAST_BWD);
 #define VSA2_LAUNCH_DQ(DD, SP, F, TQ, TK, TQT, TKT)                                                                              \
   do {                                                                                                                           \
-    if ((e = cudaFuncSetAttribute(fine_bwd_dq_tc_kernel<DD, SP, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,                 \
-                                  (int)BwdTc<DD>::smem_bytes)))                                                                  \
-      return e;                                                                                                                  \
+    static KernelAttr attr_;                                                                                                     \
+    if ((e = prepare_kernel((const void*)fine_bwd_dq_tc_kernel<DD, SP, F>, attr_, BwdTc<DD>::smem_bytes))) return e;             \
     fine_bwd_dq_tc_kernel<DD, SP, F><<<grid, kDqThreads, BwdTc<DD>::smem_bytes, st>>>(TQ, TK, tv, tdo, TQT, TKT, tvt, tdot, g, a); \
   } while (0)
   if (f16) {
@@ -508,7 +507,7 @@ cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16*
     return cudaErrorInvalidValue;
   int sms = 0;
   cudaError_t e;
-  if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   DqArgs a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, dq, status, &status->pad[kRangeFlagSlot], 2};
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
@@ -522,7 +521,7 @@ cudaError_t launch_cast_bf16_to_f16(const bf16* a, void* a16, size_t na, const b
                                     cudaStream_t st) {
   int sms = 0;
   cudaError_t e;
-  if ((e = bwd_sm_count(&sms)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   if ((na | nb) & 7) return cudaErrorInvalidValue;
   cast_bf16_to_f16_kernel<<<sms * 16, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
                                                      reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8,

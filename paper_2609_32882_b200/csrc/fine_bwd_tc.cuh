@@ -61,14 +61,13 @@ __device__ __forceinline__ bool bwd_queue_get(BwdQueue* q, uint32_t seq, int lan
   int4 REC;                                                                              \
   if (!bwd_queue_get(&misc->queue, (SEQ), lane, REC, &misc->abort_flag)) goto done;      \
   if (REC.x < 0) break
-// scheduler warp: draws the items first_item .. first_item + items - 1 (in the order of `order`, if there is one), or those of a
-// list, until the counter runs out.  `ptr`,
+// scheduler warp: draws the items first_item .. first_item + items - 1 (in the order of `order`, if there is one) until the
+// counter runs out.  `ptr`,
 // `rep`: start pointers of the lists, an item has those of `rep` consecutive heads; items with fewer than k_lo or more than k_hi
 // entries are left out.
 __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int first_item, int items, int rep, const int* ptr,
-                                             int* counter, const int* list, const int* order, int k_lo, int k_hi, int lane,
+                                             int* counter, const int* order, int k_lo, int k_hi, int lane,
                                              volatile int* abort_flag) {
-  const int total = list != nullptr ? list[0] : items;
   uint32_t drawn = 0;
   for (uint32_t p = 0;; ++p) {
     const uint32_t slot = p % kItemSlots;
@@ -81,8 +80,8 @@ __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int firs
       if (lane == 0) n = item_draw(drawn, counter);
       n = __shfl_sync(0xffffffffu, n, 0);
       ++drawn;
-      if (n >= total) break;
-      item_block(g, list != nullptr ? list[1 + n] : order != nullptr ? order[first_item + n] : first_item + n, rec.y, rec.x);
+      if (n >= items) break;
+      item_block(g, order != nullptr ? order[first_item + n] : first_item + n, rec.y, rec.x);
       int beg = 0, k = 0;
       if (lane < rep) {      // (heads of a group are neighbours: b * Hq + hk * rep + hh)
         const int* c = ptr + ((size_t)rec.y * rep + lane) * (g.N + 1) + rec.x;
@@ -212,12 +211,5 @@ __device__ __forceinline__ void bwd_init_barriers(BwdMisc* misc) {
       tc::tma_load_5d((RING_BASE) + slot_ * C::SLOT + (2 * (lane >> 1) + (lane & 1)) * kSlab, (TMAP), &(FULL)[slot_], \
                       (lane >> 1) * 64, (CW), (CH), (CT), (BH));                                                  \
   } while (0)
-
-static inline cudaError_t bwd_sm_count(int* sms) {
-  int dev = 0;
-  cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-}
 
 }  // namespace vsa2

@@ -157,11 +157,13 @@ cudaError_t launch_fine_fwd_list(const Geo& g, const int* count, int cap, const 
   cudaError_t e;
   if (g.D == 128) {
     size_t smb = FineFwdSmem<128>::bytes;
-    if ((e = cudaFuncSetAttribute(fine_fwd_list_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_list_kernel<128>, attr, smb))) return e;
     fine_fwd_list_kernel<128><<<64, 256, smb, st>>>(count, cap, items, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   } else {
     size_t smb = FineFwdSmem<64>::bytes;
-    if ((e = cudaFuncSetAttribute(fine_fwd_list_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_list_kernel<64>, attr, smb))) return e;
     fine_fwd_list_kernel<64><<<64, 256, smb, st>>>(count, cap, items, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   }
   return cudaGetLastError();
@@ -174,11 +176,13 @@ cudaError_t launch_fine_fwd(const Geo& g, const bf16* q, const bf16* k, const bf
   cudaError_t e;
   if (g.D == 128) {
     size_t smb = FineFwdSmem<128>::bytes;
-    if ((e = cudaFuncSetAttribute(fine_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_kernel<128>, attr, smb))) return e;
     fine_fwd_kernel<128><<<grid, 256, smb, st>>>(q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   } else {
     size_t smb = FineFwdSmem<64>::bytes;
-    if ((e = cudaFuncSetAttribute(fine_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_kernel<64>, attr, smb))) return e;
     fine_fwd_kernel<64><<<grid, 256, smb, st>>>(q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   }
   return cudaGetLastError();

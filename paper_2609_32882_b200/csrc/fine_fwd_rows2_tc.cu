@@ -529,10 +529,9 @@ cudaError_t launch_fine_fwd_rows2_tc(const Geo& g, bool pair_heads, const bf16* 
   CUtensorMap tq, tk, tv;
   if (!make_cube_tmap(&tq, q, g, g.Hq) || !make_cube_tmap(&tk, k, g, g.Hkv) || !make_cube_tmap(&tv, v, g, g.Hkv))
     return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   FwdRows2Args a;
   a.pair_heads = pair_heads ? 1 : 0;
   a.gate = gate; a.row_ptr = row_ptr; a.col_idx = col_idx; a.oc_hat = oc_hat; a.o = o; a.o_res = o_res; a.lse = lse;
@@ -543,19 +542,16 @@ cudaError_t launch_fine_fwd_rows2_tc(const Geo& g, bool pair_heads, const bf16* 
   a.rescue_cap = fwd_rescue_capacity();
   const int total = g.batch * g.Hq * g.N / 2;
   const int grid = total < sms ? total : sms;
-  {
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, g.D == 128 ? (const void*)fine_fwd_rows2_tc_kernel<128> : (const void*)fine_fwd_rows2_tc_kernel<64>)) != cudaSuccess) return e;
-    if (fa.numRegs * kF2Threads < 256 * 56 + 256 * 200) return cudaErrorLaunchOutOfResources;
-  }
   if (g.D == 128) {
     const size_t smb = FwdRows2<128>::smem_bytes(g.N);
     if (smb > 227 * 1024) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(fine_fwd_rows2_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<128>, attr, smb, kF2Threads, 256 * 56 + 256 * 200))) return e;
     fine_fwd_rows2_tc_kernel<128><<<grid, kF2Threads, smb, st>>>(tq, tk, tv, g, a);
   } else {
     const size_t smb = FwdRows2<64>::smem_bytes(g.N);
-    if ((e = cudaFuncSetAttribute(fine_fwd_rows2_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<64>, attr, smb, kF2Threads, 256 * 56 + 256 * 200))) return e;
     fine_fwd_rows2_tc_kernel<64><<<grid, kF2Threads, smb, st>>>(tq, tk, tv, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

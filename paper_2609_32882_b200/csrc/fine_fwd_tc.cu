@@ -537,10 +537,9 @@ cudaError_t launch_fine_fwd_tc(const Geo& g, const bf16* q, const bf16* k, const
   CUtensorMap tq, tk, tv;
   if (!make_cube_tmap(&tq, q, g, g.Hq) || !make_cube_tmap(&tk, k, g, g.Hkv) || !make_cube_tmap(&tv, v, g, g.Hkv))
     return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   FwdArgs a;
   a.gate = gate; a.row_ptr = row_ptr; a.col_idx = col_idx; a.oc_hat = oc_hat; a.o = o; a.o_res = o_res; a.lse = lse;
   a.status = status;
@@ -553,18 +552,15 @@ cudaError_t launch_fine_fwd_tc(const Geo& g, const bf16* q, const bf16* k, const
   if (g.N > kFwdMaxCubes) return cudaErrorInvalidValue;
   // The softmax warpgroups raise their register count to 200 with the registers the service warpgroups give up
   // (setmaxnreg); that request would block for ever if the launch allocation were smaller than 128 per thread.
-  {
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, g.D == 128 ? (const void*)fine_fwd_tc_kernel<128> : (const void*)fine_fwd_tc_kernel<64>)) != cudaSuccess) return e;
-    if (fa.numRegs * kFwdThreads < 256 * 56 + 256 * 200) return cudaErrorLaunchOutOfResources;
-  }
   if (g.D == 128) {
     const size_t smb = FwdTc<128>::smem_bytes(g.N);
-    if ((e = cudaFuncSetAttribute(fine_fwd_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_tc_kernel<128>, attr, smb, kFwdThreads, 256 * 56 + 256 * 200))) return e;
     fine_fwd_tc_kernel<128><<<grid, kFwdThreads, smb, st>>>(tq, tk, tv, g, a);
   } else {
     const size_t smb = FwdTc<64>::smem_bytes(g.N);
-    if ((e = cudaFuncSetAttribute(fine_fwd_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+    static KernelAttr attr;
+    if ((e = prepare_kernel((const void*)fine_fwd_tc_kernel<64>, attr, smb, kFwdThreads, 256 * 56 + 256 * 200))) return e;
     fine_fwd_tc_kernel<64><<<grid, kFwdThreads, smb, st>>>(tq, tk, tv, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

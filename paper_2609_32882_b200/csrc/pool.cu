@@ -21,7 +21,12 @@ struct PoolJob {
 struct PoolJobs {
   PoolJob job[3];
   int n;
+  StatusBlock* clear;       // null, or a status block to set to zero for the kernels behind this one
 };
+__device__ __forceinline__ void clear_status(const PoolJobs& jobs) {
+  if (jobs.clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(StatusBlock) / 4)
+    reinterpret_cast<int*>(jobs.clear)[threadIdx.x] = 0;
+}
 
 __device__ __forceinline__ void add8(float (&acc)[8], const float (&v)[8], bool first) {
 #pragma unroll
@@ -43,6 +48,7 @@ template <int D>
 __global__ void __launch_bounds__(128) pool_kernel(PoolJobs jobs, Geo g) {
   constexpr int CH = D / 8;            // 16-byte chunks of a token row
   constexpr int CUBES = 128 / CH;      // cubes per CTA
+  clear_status(jobs);
   int h = blockIdx.y;
   PoolJob jb = jobs.job[0];
   if (jobs.n > 1 && h >= jb.heads) {
@@ -110,6 +116,7 @@ template <int D>
 __global__ void __launch_bounds__(kSubThreads) pool_subcube_kernel(PoolJobs jobs, Geo g) {
   constexpr int CH = D / 8, SUB = kSubThreads / CH, CUBES = SUB / 8;
   __shared__ __align__(16) float sums[SUB * D];
+  clear_status(jobs);
   int h = blockIdx.y;
   PoolJob jb = jobs.job[0];
   if (jobs.n > 1 && h >= jb.heads) {
@@ -222,16 +229,18 @@ static cudaError_t launch_pool_jobs(const Geo& g, const PoolJobs& jobs, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t launch_pool(const Geo& g, const bf16* x, int heads, bf16* xr, float* xc, cudaStream_t st) {
+cudaError_t launch_pool(const Geo& g, const bf16* x, int heads, bf16* xr, float* xc, StatusBlock* clear, cudaStream_t st) {
   PoolJobs jobs{};
+  jobs.clear = clear;
   jobs.job[0] = PoolJob{x, xr, xc, heads};
   jobs.n = 1;
   return launch_pool_jobs(g, jobs, st);
 }
 
 // router means of Q and K (Eq. 5) in one launch
-cudaError_t launch_pool_router(const Geo& g, const bf16* q, const bf16* k, bf16* qr, bf16* kr, cudaStream_t st) {
+cudaError_t launch_pool_router(const Geo& g, const bf16* q, const bf16* k, bf16* qr, bf16* kr, StatusBlock* clear, cudaStream_t st) {
   PoolJobs jobs{};
+  jobs.clear = clear;
   jobs.job[0] = PoolJob{q, qr, nullptr, g.Hq};
   jobs.job[1] = PoolJob{k, kr, nullptr, g.Hkv};
   jobs.n = 2;
@@ -240,8 +249,9 @@ cudaError_t launch_pool_router(const Geo& g, const bf16* q, const bf16* k, bf16*
 
 // cube means of Q, K and V (Eq. 1) in one launch
 cudaError_t launch_pool_coarse(const Geo& g, const bf16* q, const bf16* k, const bf16* v, float* qc, float* kc, float* vc,
-                               cudaStream_t st) {
+                               StatusBlock* clear, cudaStream_t st) {
   PoolJobs jobs{};
+  jobs.clear = clear;
   jobs.job[0] = PoolJob{q, nullptr, qc, g.Hq};
   jobs.job[1] = PoolJob{k, nullptr, kc, g.Hkv};
   jobs.job[2] = PoolJob{v, nullptr, vc, g.Hkv};

@@ -330,11 +330,11 @@ static cudaError_t launch_router(const CUtensorMap& tq, const CUtensorMap& tk, c
   const int row_tiles = (g.N * G + kRtTile - 1) / kRtTile;
   const size_t smb = RouterTc<D>::smem_bytes(row_tiles * kRtTile / 32);
   if (smb > 227 * 1024) return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(router_tc_kernel<D, G, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb))) return e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
+  static KernelAttr attr;
+  if ((e = prepare_kernel((const void*)router_tc_kernel<D, G, FOLD>, attr, smb))) return e;
   const int total = g.batch * g.Hq * row_tiles;
   { ProfScope lse(VSA2_KERNEL_ROUTER_LSE, st, 0); }      // (both passes are timed as the second)
   ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);

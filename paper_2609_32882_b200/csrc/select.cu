@@ -488,6 +488,120 @@ __global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __re
   }
 }
 
+// Up to kSelOneBlockN cubes: everything behind the counts of the kept entries in one launch, a block per head with both bitmaps in
+// shared memory (the six launches below take 2 us and a gap each and keep a few SMs busy).  Same rules: rows in order, ties at the
+// threshold to the lower column, both maps cut at the capacity.
+__global__ void __launch_bounds__(1024) sel_maps_kernel(const float* __restrict__ pr, int N, int words, int per_sequence,
+                                                        const unsigned* __restrict__ state, const int* __restrict__ row_gt,
+                                                        const int* __restrict__ row_eq, const float* __restrict__ row_tau,
+                                                        const int* __restrict__ row_eq_take, const int* __restrict__ row_cnt,
+                                                        const unsigned* __restrict__ bits_gt, const unsigned* __restrict__ bits_eq,
+                                                        int* row_ptr, int* col_idx, int* col_ptr, int* row_idx, long long nnz_cap,
+                                                        StatusBlock* status) {
+  constexpr int W = kSelOneBlockN / 32;
+  __shared__ unsigned bm[kSelOneBlockN * W], bt[kSelOneBlockN * W];
+  __shared__ int take_s[kSelOneBlockN], ptr_s[kSelOneBlockN], ws[33];
+  const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const size_t base = (size_t)bh * N;
+  int cnt = 0, take = 0, tot;
+  if (per_sequence) {
+    const int eq = tid < N ? row_eq[base + tid] : 0;
+    const int before = block_excl_scan(eq, ws, tot);
+    if (tid < N) {
+      take = max(0, min(eq, (int)state[bh * 8 + 4] - before));
+      cnt = row_gt[base + tid] + take;
+    }
+  } else if (tid < N) {
+    take = row_eq_take[base + tid];
+    cnt = row_cnt[base + tid];
+  }
+  int pre = block_excl_scan(cnt, ws, tot);
+  if (tid < N) {
+    take_s[tid] = take;
+    ptr_s[tid] = pre;
+    row_ptr[(size_t)bh * (N + 1) + tid] = (int)min((long long)pre, nnz_cap);
+  }
+  if (tid == 0) {
+    row_ptr[(size_t)bh * (N + 1) + N] = (int)min((long long)tot, nnz_cap);
+    if ((long long)tot > nnz_cap) atomicExch(&status->status, VSA2_ERR_MAP_OVERFLOW);
+  }
+  __syncthreads();
+  int* out = col_idx + (size_t)bh * nnz_cap;
+  const unsigned lt = (1u << lane) - 1u;
+  for (int i = warp; i < N; i += 32) {
+    const unsigned* src = reinterpret_cast<const unsigned*>(pr) + (base + i) * N;
+    const unsigned tau = per_sequence ? 0u : __float_as_uint(row_tau[base + i]);
+    int pos = (int)min((long long)ptr_s[i], nnz_cap), left = take_s[i];
+    // (the whole row is read first: a row's words one after another waited for memory every time)
+    unsigned v[W], gw = 0u, ew = 0u;
+    if (per_sequence) {
+      if (lane < words) {
+        gw = __ldg(bits_gt + (base + i) * words + lane);
+        ew = __ldg(bits_eq + (base + i) * words + lane);
+      }
+    } else {
+#pragma unroll
+      for (int w = 0; w < W; ++w) v[w] = w * 32 + lane < N ? __ldg(src + w * 32 + lane) : 0u;
+    }
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      if (w >= words) break;
+      const int j = w * 32 + lane;
+      bool gt, eq;
+      if (per_sequence) {
+        gt = (__shfl_sync(0xffffffffu, gw, w) >> lane) & 1u;
+        eq = (__shfl_sync(0xffffffffu, ew, w) >> lane) & 1u;
+      } else {
+        gt = j < N && v[w] > tau;
+        eq = j < N && v[w] == tau;
+      }
+      const unsigned eqb = __ballot_sync(0xffffffffu, eq);
+      const bool sel = gt || (eq && __popc(eqb & lt) < left);
+      const unsigned selb = __ballot_sync(0xffffffffu, sel);
+      const int p = pos + __popc(selb & lt);
+      const bool emit = sel && p < nnz_cap;
+      if (emit) out[p] = j;
+      const unsigned keptb = __ballot_sync(0xffffffffu, emit);
+      pos += __popc(selb);
+      left -= __popc(eqb);
+      if (lane == 0) bm[i * W + w] = keptb;
+    }
+  }
+  __syncthreads();
+  for (int t = warp; t < words * words; t += 32) {
+    const int wi = t / words, wj = t - wi * words;
+    const unsigned v = wi * 32 + lane < N ? bm[(wi * 32 + lane) * W + wj] : 0u;
+    unsigned mine = 0u;
+#pragma unroll
+    for (int bit = 0; bit < 32; ++bit) {
+      const unsigned col_word = __ballot_sync(0xffffffffu, (v >> bit) & 1u);
+      if (lane == bit) mine = col_word;
+    }
+    if (wj * 32 + lane < N) bt[(wj * 32 + lane) * W + wi] = mine;
+  }
+  __syncthreads();
+  cnt = 0;
+  if (tid < N)
+    for (int w = 0; w < words; ++w) cnt += __popc(bt[tid * W + w]);
+  pre = block_excl_scan(cnt, ws, tot);
+  if (tid < N) {
+    ptr_s[tid] = (int)min((long long)pre, nnz_cap);
+    col_ptr[(size_t)bh * (N + 1) + tid] = ptr_s[tid];
+  }
+  if (tid == 0) col_ptr[(size_t)bh * (N + 1) + N] = (int)min((long long)tot, nnz_cap);
+  __syncthreads();
+  int* rows = row_idx + (size_t)bh * nnz_cap;
+  for (int j = warp; j < N; j += 32) {
+    int pos = ptr_s[j];
+    for (int w = 0; w < words; ++w) {
+      const unsigned word = bt[j * W + w];
+      const int p = pos + __popc(word & lt);
+      if (((word >> lane) & 1u) && p < nnz_cap) rows[p] = w * 32 + lane;
+      pos += __popc(word);
+    }
+  }
+}
+
 cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, int* row_ptr,
                           int* col_idx, int* col_ptr, int* row_idx, StatusBlock* status, cudaStream_t st) {
   const int BH = g.batch * g.Hq, N = g.N;
@@ -513,6 +627,12 @@ cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, con
     else if (N <= 1536) sel_row_topk_warp_kernel<48><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
     else if (N <= 2048) sel_row_topk_warp_kernel<64><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
     else sel_row_topk_kernel<<<dim3(N, BH), 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+  }
+  if (N <= kSelOneBlockN) {
+    sel_maps_kernel<<<BH, 1024, 0, st>>>(pr, N, s.words, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
+                                         s.row_eq_take, s.row_cnt, s.bitmap, s.bitmap_t, row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap,
+                                         status);
+    return cudaGetLastError();
   }
   sel_scan_rows_kernel<<<BH, 1024, 0, st>>>(N, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
                                             s.row_eq_take, s.row_cnt, row_ptr, g.nnz_cap, status);

@@ -42,13 +42,17 @@ inline bool make_cube_tmap(CUtensorMap* out, const void* base, const Geo& g, int
 
 // The text rows of the same tensor (rows L .. L + Lt - 1 of every head) as a 5-D map whose box is 64 rows x 64 channels, so
 // that the kernels fetch a text block with the same instruction and byte count as a cube; rows beyond Lt are zero-filled.
-// Without text tokens (Lt = 0) the map covers one row of the video part and is never used.
+// Without text tokens (Lt = 0) the map is never used and not encoded.
 inline bool make_text_tmap(CUtensorMap* out, const void* base, const Geo& g, int heads) {
+  if (g.Lt == 0) {
+    *out = CUtensorMap{};
+    return true;
+  }
   EncodeTiledFn fn = encode_tiled_fn();
   if (fn == nullptr) return false;
   const cuuint64_t D = (cuuint64_t)g.D;
-  const cuuint64_t rows = g.Lt > 0 ? (cuuint64_t)g.Lt : 1;
-  const unsigned char* first = reinterpret_cast<const unsigned char*>(base) + (g.Lt > 0 ? (size_t)g.L * g.D * 2 : 0);
+  const cuuint64_t rows = (cuuint64_t)g.Lt;
+  const unsigned char* first = reinterpret_cast<const unsigned char*>(base) + (size_t)g.L * g.D * 2;
   cuuint64_t dims[5] = {D, rows, 1, 1, (cuuint64_t)g.batch * heads};
   cuuint64_t strides[4] = {D * 2, rows * D * 2, rows * D * 2, (cuuint64_t)g.S * D * 2};
   cuuint32_t box[5] = {64, (cuuint32_t)kBlockTokens, 1, 1, 1};
