@@ -36,19 +36,16 @@ UNIT = "TFLOP/s dense-equivalent"
 ORACLE_HOW = "the oracle as it stands: fp64 numpy whose matrix products run on the multithreaded BLAS numpy links"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the 720p top-64 launch with 40 heads: an
-# 8-head ncu capture of the same kernels times 5 (every head streams its own tensors, so the traffic grows in
+# 8-head ncu capture of the same kernel times 5 (every head streams its own tensors, so the traffic grows in
 # proportion to the heads; the 40-head launch is too large for a full-set capture).
-NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.504200e9 + 0.295100e9),
-                                "fine_bwd_dq": 5 * (0.663200e9 + 0.147600e9 + 0.309700e9 + 0.262100e9),   # with the fp16 copy of Q, K
-                                "fine_bwd_dkv": 5 * (0.791600e9 + 0.304900e9)}
+NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.504200e9 + 0.295100e9)}
 
 
 # What ncu shows as the busiest unit of each tensor kernel at 64-token cubes (8-head capture, profiles/): the roofline
 # below is quoted against the tensor peak as the contract asks, these say what actually holds the kernel there.
 NCU_LIMITER = {
     "fine_fwd": "L2 -> SM read rate: 12.9 TB/s against 11.8 TB/s sustained peak (tensor pipe 82 % active at the half rate of M = 64)",
-    "fine_bwd_dq": "shared-memory data pipe: tensor-core operand fetches 64 % + thread loads/stores 37 % (tensor pipe 43 %)",
-    "fine_bwd_dkv": "shared-memory data pipe: tensor-core operand fetches 67 % + thread loads/stores 32 % (tensor pipe 47 %)",
+    "fine_bwd": "shared-memory data pipe (dK/dV: four products and the hand-over of dS) and the reads of the stored dS tiles (dQ)",
     "router_pool": "exponential unit (one ex2 per score): about three quarters busy",
 }
 # L2 -> SM read rate that ncu reports as the sustained peak of this part (derived__lts__lts2xbar_bytes.sum.peak_sustained
@@ -90,8 +87,6 @@ def flop_counts(wl: syn.Workload, nnz_total: int) -> dict:
         "dense_equiv_fwd_bwd": 3.5 * 4.0 * L * L * D * Hq,
         "fine_fwd": 4.0 * pair * nnz_total,
         "fine_bwd_algorithmic": 10.0 * pair * nnz_total,
-        "fine_bwd_dq_executed": 6.0 * pair * nnz_total,
-        "fine_bwd_dkv_executed": 8.0 * pair * nnz_total,
         "router_per_pass": 2.0 * (N * G) ** 2 * D * Hq,
         "coarse_fwd": 4.0 * N * N * D * Hq,
     }
@@ -426,24 +421,25 @@ def run_ours(args):
     flops = flop_counts(wl, nnz_total)
     if args.forward_only:
         flops["dense_equiv_fwd_bwd"] = flops["dense_equiv_fwd"]
-        flops["fine_bwd_dq_executed"] = flops["fine_bwd_dkv_executed"] = 0.0
+        flops["fine_bwd_algorithmic"] = 0.0
     ms_step = ms_total / args.steps
     ms_step_e2e = ms_e2e / args.steps
     value = replicas.whole_job_throughput(flops["dense_equiv_fwd_bwd"], world, ms_step * 1e-3) / 1e12
     value_e2e = replicas.whole_job_throughput(flops["dense_equiv_fwd_bwd"], world, ms_step_e2e * 1e-3) / 1e12
     pk, pk_kind = peaks()
-    executed = flops["fine_fwd"] + flops["fine_bwd_dq_executed"] + flops["fine_bwd_dkv_executed"] + flops["router_per_pass"]
-    kernel_flops = {"fine_fwd": flops["fine_fwd"], "fine_bwd_dq": flops["fine_bwd_dq_executed"],
-                    "fine_bwd_dkv": flops["fine_bwd_dkv_executed"], "router_pool": flops["router_per_pass"]}
-    tensor_kernels = {k: kernel_ms[k] for k in kernel_flops}
+    executed = flops["fine_fwd"] + flops["fine_bwd_algorithmic"] + 2.0 * flops["router_per_pass"]
+    kernel_flops = {"fine_fwd": flops["fine_fwd"], "fine_bwd": flops["fine_bwd_algorithmic"],
+                    "router_pool": 2.0 * flops["router_per_pass"]}
+    # dK/dV and dQ together: where dS is stored, dQ is formed inside the events of fine_bwd_dkv
+    tensor_kernels = {k: kernel_ms["fine_bwd_dq"] + kernel_ms["fine_bwd_dkv"] if k == "fine_bwd" else kernel_ms[k] for k in kernel_flops}
     dominant = max(tensor_kernels, key=tensor_kernels.get)
     peak_tf = pk["bf16_tflops_sustained"]
-    achieved = kernel_flops[dominant] / (kernel_ms[dominant] * 1e-3) / 1e12
+    achieved = kernel_flops[dominant] / (tensor_kernels[dominant] * 1e-3) / 1e12
     roofline = {"kernel": dominant, "bound": "tensor", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                 "frac": achieved / peak_tf,
                 "traffic": NCU_TRAFFIC_BYTES_720P_TOP64.get(dominant) if (args.config == 3 and not (args.heads or args.topk or args.grid or args.cube)) else None,
                 "peak_kind": pk_kind + " sustained bf16",
-                "flops_per_launch": kernel_flops[dominant], "ms_per_launch": kernel_ms[dominant],
+                "flops_per_launch": kernel_flops[dominant], "ms_per_launch": tensor_kernels[dominant],
                 "limiter_ncu": NCU_LIMITER.get(dominant) if wl.cube[0] * wl.cube[1] * wl.cube[2] == 64 else None}
     fine_fwd_tf = flops["fine_fwd"] / (kernel_ms["fine_fwd"] * 1e-3) / 1e12
     # operand bytes the fine forward has to bring into shared memory: a K and a V tile per selected (query block, KV block)

@@ -288,15 +288,15 @@ int vsa2_device_status(const void* workspace, void* cuda_stream, int32_t* status
 /* Kernel groups, for timing from outside (e.g. a benchmark) without a profiler. */
 enum {
   VSA2_KERNEL_POOL = 0,         /* vsa2_attn_fwd: cube means of Q, K, V (Eq. 1) */
-  VSA2_KERNEL_ROUTER_LSE = 1,   /* router pass 1: row log-sum-exp (Eq. 6); empty when the router takes one pass */
-  VSA2_KERNEL_ROUTER_POOL = 2,  /* router pass 2, or its one pass: softmax + G x G pooling (Eq. 6-7) */
+  VSA2_KERNEL_ROUTER_LSE = 1,   /* router pass 1 where it is a launch of its own (G other than 8, 16); else empty */
+  VSA2_KERNEL_ROUTER_POOL = 2,  /* softmax + G x G pooling (Eq. 6-7); both passes when one launch holds them */
   VSA2_KERNEL_SELECT = 3,       /* TopK + CSR/CSC (Eq. 8-9) */
   VSA2_KERNEL_COARSE_FWD = 4,   /* Eq. 2-3 */
   VSA2_KERNEL_FINE_FWD = 5,     /* Eq. 12 + Eq. 14 */
   VSA2_KERNEL_BWD_PRE = 6,      /* delta, dGate, dO_c_hat */
   VSA2_KERNEL_COARSE_BWD = 7,
-  VSA2_KERNEL_FINE_BWD_DQ = 8,
-  VSA2_KERNEL_FINE_BWD_DKV = 9,
+  VSA2_KERNEL_FINE_BWD_DQ = 8,  /* operand copies and, where dS is not stored, the dQ pass */
+  VSA2_KERNEL_FINE_BWD_DKV = 9, /* dK/dV pass, and dQ from the stored dS */
   VSA2_KERNEL_POOL_ROUTER = 10, /* vsa2_route: sub-cube means of Q, K (Eq. 5) */
   VSA2_KERNEL_COUNT = 11
 };
