@@ -1,0 +1,39 @@
+"""Backward with room for the stored score-gradient tiles of all KV heads, of all but one, and of none: the three routes form
+dQ from the same fp16 tiles and cubes in the same order, so the gradients must be the same bit for bit (the route without
+room is the one that the parity tests compare with the oracle)."""
+import pytest
+import torch
+
+from paper_2609_32882_b200 import binding as vb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads_q,heads_kv,dim,grid,topk,mode,text", [
+    (2, 2, 64, (4, 8, 8), 2, vb.PER_QUERY, 0),
+    (3, 3, 128, (5, 9, 13), 5, vb.PER_SEQUENCE, 0),          # ragged cubes, lists of any length, odd ones too
+    (4, 2, 128, (8, 16, 16), 9, vb.PER_QUERY, 0),            # grouped heads, fp16 form
+    (4, 2, 128, (8, 16, 16), 3, vb.PER_QUERY, 0),            # grouped heads, short lists: pair form
+    (2, 2, 128, (8, 12, 16), 4, vb.PER_SEQUENCE, 77),        # text blocks, the last one ragged
+    (8, 8, 64, (16, 20, 20), 3, vb.PER_SEQUENCE, 0),         # enough items for the pass to be drawn in order of length
+])
+def test_gradients_do_not_depend_on_the_scratch(heads_q, heads_kv, dim, grid, topk, mode, text):
+    p = vb.make_params(1, heads_q, heads_kv, dim, grid, select_mode=mode, topk=topk, text_len=text)
+    attn = vb.Vsa2Attention(p)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    rows = grid[0] * grid[1] * grid[2] + text
+    rnd = lambda h: torch.randn(1, h, rows, dim, device="cuda", generator=gen).bfloat16()
+    q, k, v, d_o = rnd(heads_q), rnd(heads_kv), rnd(heads_kv), rnd(heads_q)
+    gate = torch.rand(1, heads_q, rows - text, device="cuda", generator=gen)
+    attn.route(q, k)
+    o, lse = attn.forward(q, k, v, gate)
+    most, least = vb.vsa2_attn_bwd_preferred_workspace_bytes(p), attn.sizes.bwd_workspace_bytes
+    assert most > least
+    got = []
+    for size in (most, most - 256, least):
+        attn.ws_bwd = torch.empty(size, dtype=torch.uint8, device="cuda")
+        got.append(attn.backward(q, k, v, gate, o, lse, d_o))
+        attn.check_status()
+    for other in got[1:]:
+        for name, x, y in zip(("dq", "dk", "dv", "dgate"), got[0], other):
+            assert torch.equal(x, y), name
