@@ -94,59 +94,66 @@ __global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* __rest
 }
 
 // ---------------------------------------------------------------------------------------------- forward
-// MW warps of 16 tokens x KW warps of CH channels each; grid (ceil(L / (16 MW)), batch); NT = head tiles of 8.
-// X goes from global memory straight into the A fragments: the order of the contraction is free, so a thread takes the 16
-// contiguous bytes of channels 8t .. 8t+7 of a group of 32 as its elements of two k-steps (logical k = 2t, 2t+1, 2t+8, 2t+9
-// of step s is channel 8t + 4s + 0 .. 3), and the rows of W lie in that order in shared memory, for ldmatrix.  The loads of the next
-// chunk are in flight while a chunk is multiplied.  Few tokens: KW warps share a token tile and add up at the end.
-template <int NT, int MW, int KW, int CH>
-__global__ void __launch_bounds__(32 * MW * KW) gate_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, int L,
-                                                                int C, int Hq, float* __restrict__ gate) {
+// MW warp rows of 16 tokens, each of HW warps that take NT / HW head tiles of 8; grid (ceil(L / (16 MW)), batch).
+// X goes from global memory straight into the A fragments.  The k-steps run over the channels in order and one warp sums all of them,
+// so a gate does not depend on how many tokens share the launch; inside a step the order is free.  Of a group of 32 channels a
+// thread loads the 16 bytes of channels 8t .. 8t+7, trades 8 of them with thread t ^ 2 (the first two threads hold the first step's 16
+// channels, the others the second's) and then has 4 channels of each step as its logical k = 2t, 2t+1, 2t+8, 2t+9; the rows
+// of W lie in that order in shared memory, for ldmatrix.  (8-byte loads need no trade but twice the cache look-ups: 75,600 tokens of
+// 5,120 channels, 40 heads 345 us against 296; 10 heads 168 both ways.)  The loads of the next chunk are in flight while a chunk is multiplied; warps beyond MW HW only
+// stage W.
+template <int NT, int MW, int HW, int CH>
+__global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, int L,
+                                                              int C, int Hq, float* __restrict__ gate) {
+  static_assert(NT % HW == 0 && MW * HW * 32 <= kGtThreads, "warps of a CTA");
   constexpr int LDW = NT * 8 + 8;                           // 16-byte aligned rows, eight rows on different banks
-  constexpr int THREADS = 32 * MW * KW, STEP = KW * CH, GROUPS = CH / 32;
-  __shared__ __align__(16) bf16 ws[STEP * LDW];             // W chunk as stored: [channel][head]; read by ldmatrix.trans
+  constexpr int NTW = NT / HW, GROUPS = CH / 32;
+  __shared__ __align__(16) bf16 ws[CH * LDW];               // W chunk as stored: [channel][head]; read by ldmatrix.trans
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int mw = warp % MW, kw = warp / MW;
+  const int mw = warp % MW, hw = warp / MW, h0 = hw * NTW * 8;
+  const bool works = hw < HW;
   const int l0 = blockIdx.x * (16 * MW) + mw * 16, b = blockIdx.y;
-  const bf16* xa = x + ((size_t)b * L + min(l0 + g, L - 1)) * C + kw * CH + t * 8;       // (rows behind the last token repeat it)
-  const bf16* xc = x + ((size_t)b * L + min(l0 + g + 8, L - 1)) * C + kw * CH + t * 8;
+  const bf16* xa = x + ((size_t)b * L + min(l0 + g, L - 1)) * C + t * 8;       // (rows behind the last token repeat it)
+  const bf16* xc = x + ((size_t)b * L + min(l0 + g + 8, L - 1)) * C + t * 8;
   // (the rows of a chunk of W are contiguous: read as 16-byte vectors whatever the number of heads)
   const bool w_vec = (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
-  // channel of a chunk -> its row in ws (inside its group of 32: step, upper half, t, parity)
-  auto w_row = [](int c) { return (c & ~31) + ((c >> 2) & 1) * 16 + ((c >> 1) & 1) * 8 + ((c >> 3) & 3) * 2 + (c & 1); };
-  float acc[NT][4];
+  // channel of a chunk -> its row in ws (inside its step of 16: upper half, thread, parity)
+  auto w_row = [](int c) { return (c & ~15) + ((c >> 1) & 1) * 8 + (((c >> 3) & 1) + ((c >> 2) & 1) * 2) * 2 + (c & 1); };
+  float acc[NTW][4];
 #pragma unroll
-  for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-  constexpr int WV = STEP * NT / THREADS;                   // vectors of a W chunk per thread
+  for (int n = 0; n < NTW; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+  constexpr int WV = CH * NT / kGtThreads;                  // vectors of a W chunk per thread
   uint4 ra[GROUPS], rc[GROUPS], rw[WV];
-  for (int e = tid; e < STEP * LDW / 8; e += THREADS) reinterpret_cast<uint4*>(ws)[e] = make_uint4(0, 0, 0, 0);   // (padding heads)
+  for (int e = tid; e < CH * LDW / 8; e += kGtThreads) reinterpret_cast<uint4*>(ws)[e] = make_uint4(0, 0, 0, 0);   // (padding heads)
   auto load = [&](int c0) {
     if (w_vec) {
 #pragma unroll
       for (int u = 0; u < WV; ++u) {
-        const int e = tid + u * THREADS;
-        rw[u] = e * 8 < STEP * Hq && c0 * Hq + e * 8 < C * Hq ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq) + e)
-                                                             : make_uint4(0, 0, 0, 0);
+        const int e = tid + u * kGtThreads;
+        rw[u] = e * 8 < CH * Hq && c0 * Hq + e * 8 < C * Hq ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq) + e)
+                                                            : make_uint4(0, 0, 0, 0);
       }
     }
+    if (works) {
 #pragma unroll
-    for (int q = 0; q < GROUPS; ++q) {
-      const bool in = c0 + kw * CH + q * 32 + t * 8 < C;
-      ra[q] = in ? __ldg(reinterpret_cast<const uint4*>(xa + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
-      rc[q] = in ? __ldg(reinterpret_cast<const uint4*>(xc + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
+      for (int q = 0; q < GROUPS; ++q) {
+        const bool in = c0 + q * 32 + t * 8 < C;
+        ra[q] = in ? __ldg(reinterpret_cast<const uint4*>(xa + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
+        rc[q] = in ? __ldg(reinterpret_cast<const uint4*>(xc + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
+      }
     }
   };
   load(0);
-  for (int c0 = 0; c0 < C; c0 += STEP) {
+  for (int c0 = 0; c0 < C; c0 += CH) {
     __syncthreads();
     if (w_vec) {
 #pragma unroll
       for (int u = 0; u < WV; ++u) {
-        const int e = tid + u * THREADS;
-        if (e * 8 < STEP * Hq) scatter_w<LDW>(ws, rw[u], e * 8, Hq, w_row);
+        const int e = tid + u * kGtThreads;
+        if (e * 8 < CH * Hq) scatter_w<LDW>(ws, rw[u], e * 8, Hq, w_row);
       }
     } else {
-      for (int e = tid; e < STEP * NT * 8; e += THREADS) {
+      for (int e = tid; e < CH * NT * 8; e += kGtThreads) {
         const int c = e / (NT * 8), h = e % (NT * 8);
         ws[w_row(c) * LDW + h] = (h < Hq && c0 + c < C) ? w[(size_t)(c0 + c) * Hq + h] : __float2bfloat16_rn(0.f);
       }
@@ -158,46 +165,42 @@ __global__ void __launch_bounds__(32 * MW * KW) gate_fwd_kernel(const bf16* __re
       ca[q] = ra[q];
       cc[q] = rc[q];
     }
-    if (c0 + STEP < C) load(c0 + STEP);
+    if (c0 + CH < C) load(c0 + CH);
+    if (works) {
 #pragma unroll
-    for (int q = 0; q < GROUPS; ++q) {
+      for (int q = 0; q < GROUPS; ++q) {
+        // (x, y) = this thread's half for the first step of the group, (z, w) for the second
+        auto trade = [&](uint4 v) {
+          const uint32_t r0 = __shfl_xor_sync(0xffffffffu, t < 2 ? v.z : v.x, 2), r1 = __shfl_xor_sync(0xffffffffu, t < 2 ? v.w : v.y, 2);
+          return t < 2 ? make_uint4(v.x, v.y, r0, r1) : make_uint4(r0, r1, v.z, v.w);
+        };
+        const uint4 va = trade(ca[q]), vc = trade(cc[q]);
 #pragma unroll
-      for (int st = 0; st < 2; ++st) {
-        const uint32_t a[4] = {st ? ca[q].z : ca[q].x, st ? cc[q].z : cc[q].x, st ? ca[q].w : ca[q].y, st ? cc[q].w : cc[q].y};
-        const bf16* row = ws + (kw * CH + q * 32 + st * 16 + (lane & 15)) * LDW;
+        for (int st = 0; st < 2; ++st) {
+          const uint32_t a[4] = {st ? va.z : va.x, st ? vc.z : vc.x, st ? va.w : va.y, st ? vc.w : vc.y};
+          const bf16* row = ws + (q * 32 + st * 16 + (lane & 15)) * LDW + h0;
 #pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          uint32_t b0, b1;
-          ldmatrix_x2_trans(b0, b1, row + n * 8);
-          mma_bf16(acc[n], a, b0, b1);
+          for (int n = 0; n + 1 < NTW; n += 2) {
+            uint32_t bb[4];
+            ldmatrix_x4_trans(bb, row + n * 8 + (lane >> 4) * 8);
+            mma_bf16(acc[n], a, bb[0], bb[1]);
+            mma_bf16(acc[n + 1], a, bb[2], bb[3]);
+          }
+          if constexpr (NTW % 2 == 1) {
+            uint32_t b0, b1;
+            ldmatrix_x2_trans(b0, b1, row + (NTW - 1) * 8);
+            mma_bf16(acc[NTW - 1], a, b0, b1);
+          }
         }
       }
     }
   }
-  if constexpr (KW > 1) {
-    // the KW partial sums of a tile, added in a fixed order by its first warp
-    __syncthreads();
-    float* red = reinterpret_cast<float*>(ws);              // [KW - 1][MW][32 lanes][NT * 4], within the W chunk's space
-    static_assert((KW - 1) * MW * 32 * NT * 4 * 4 <= STEP * LDW * 2, "reduction space");
-    if (kw > 0) {
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) red[(((kw - 1) * MW + mw) * (NT * 4) + n * 4 + e) * 32 + lane] = acc[n][e];
-    }
-    __syncthreads();
-    if (kw > 0) return;
-    for (int o = 0; o < KW - 1; ++o)
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[n][e] += red[((o * MW + mw) * (NT * 4) + n * 4 + e) * 32 + lane];
-  }
+  if (!works) return;
   float* gb = gate + (size_t)b * Hq * L;
   const int tok = l0 + g;
 #pragma unroll
-  for (int n = 0; n < NT; ++n) {
-    const int h = n * 8 + 2 * t;
+  for (int n = 0; n < NTW; ++n) {
+    const int h = h0 + n * 8 + 2 * t;
     if (h < Hq) {
       if (tok < L) gb[(size_t)h * L + tok] = tanhf(acc[n][0]);
       if (tok + 8 < L) gb[(size_t)h * L + tok + 8] = tanhf(acc[n][2]);
@@ -405,22 +408,22 @@ size_t gate_bwd_workspace_bytes(int batch, int L, int hidden, int heads) {
 }
 
 cudaError_t launch_gate_fwd(int batch, int L, int C, int Hq, const bf16* x, const bf16* w, float* gate, cudaStream_t st) {
-  // 64 tokens a CTA; with fewer than two such CTAs per SM, 16 tokens and the channels split over four warps (2048 tokens of 1536
+  // 64 tokens a CTA; with fewer than two such CTAs per SM, 16 tokens and the head tiles split over the warps (2048 tokens of 1536
   // channels: 37 us with 64-token CTAs, which leave 116 of 148 SMs without one)
   const bool few = (long long)batch * ((L + 63) / 64) < 2 * 148;
   dim3 grid((L + (few ? 15 : 63)) / (few ? 16 : 64), batch);
   const int nt = (Hq + 7) / 8;
-#define VSA2_GATE_FWD(NT_)                                                                            \
-  do {                                                                                                \
-    if (few) gate_fwd_kernel<NT_, 1, 4, 64><<<grid, 128, 0, st>>>(x, w, L, C, Hq, gate);              \
-    else gate_fwd_kernel<NT_, 4, 1, 128><<<grid, 128, 0, st>>>(x, w, L, C, Hq, gate);                 \
+#define VSA2_GATE_FWD(NT_, HW_)                                                                                  \
+  do {                                                                                                           \
+    if (few) gate_fwd_kernel<NT_, 1, HW_, 256><<<grid, kGtThreads, 0, st>>>(x, w, L, C, Hq, gate);               \
+    else gate_fwd_kernel<NT_, 4, 1, 128><<<grid, kGtThreads, 0, st>>>(x, w, L, C, Hq, gate);                     \
   } while (0)
-  if (nt <= 1) VSA2_GATE_FWD(1);
-  else if (nt <= 2) VSA2_GATE_FWD(2);
-  else if (nt <= 4) VSA2_GATE_FWD(4);
-  else if (nt <= 5) VSA2_GATE_FWD(5);
-  else if (nt <= 6) VSA2_GATE_FWD(6);
-  else VSA2_GATE_FWD(8);
+  if (nt <= 1) VSA2_GATE_FWD(1, 1);
+  else if (nt <= 2) VSA2_GATE_FWD(2, 2);
+  else if (nt <= 4) VSA2_GATE_FWD(4, 4);
+  else if (nt <= 5) VSA2_GATE_FWD(5, 1);
+  else if (nt <= 6) VSA2_GATE_FWD(6, 3);
+  else VSA2_GATE_FWD(8, 4);
 #undef VSA2_GATE_FWD
   return cudaGetLastError();
 }

@@ -110,3 +110,20 @@ def test_gate_feeds_the_attention_forward():
 def test_gate_projection_on_few_and_on_many_tokens(batch, heads, grid, hidden, out_dtype):
     got, ref, _ = run_gate(batch, heads, grid, hidden, seed=11 * heads + hidden, out_dtype=out_dtype)
     check(got, ref, out_dtype == vb.BF16)
+
+
+@pytest.mark.parametrize("heads,hidden", [(5, 264), (12, 1536), (33, 1000), (64, 136)])
+def test_gate_of_a_token_does_not_depend_on_the_launch(heads, hidden):
+    """Few tokens take 16-token CTAs, many take 64-token CTAs: the sum over the channels runs in one order in both, so the gates of
+    the same rows of X are the same bit for bit."""
+    gen = torch.Generator(device="cuda").manual_seed(heads)
+    few, many = (3, 13, 17), (31, 33, 40)            # 663 tokens, 40,920 tokens
+    x = torch.randn(1, many[0] * many[1] * many[2], hidden, generator=gen, device="cuda").bfloat16()
+    w = (torch.randn(hidden, heads, generator=gen, device="cuda") / hidden ** 0.5).bfloat16()
+    gates = []
+    for grid in (many, few):
+        n = grid[0] * grid[1] * grid[2]
+        p = vb.make_params(batch=1, heads_q=heads, heads_kv=heads, head_dim=64, grid=grid, topk=1)
+        gates.append(torch.empty(1, heads, n, device="cuda"))
+        vb.vsa2_gate_fwd(p, hidden, x[:, :n].contiguous(), w, gates[-1])
+    assert torch.equal(gates[0][:, :, :gates[1].shape[2]], gates[1])
