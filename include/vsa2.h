@@ -70,14 +70,18 @@ enum { VSA2_FLAG_BF16_COARSE_FWD = 64 }; /* forward of the coarse branch on the 
 /* Precision of the backward passes.  P and dS are 16-bit operands of the dV, dK and dQ products; rounded once to bf16 (2^-9
  * relative) they alone push the worst elements of large gradients (|g| > 5) past max abs err 2e-2 (720p sample, fp32 outputs:
  * dQ 2.5e-2; with one query head per KV head the KV blocks that nearly every query keeps reach |dK| = 15 and 1.5 - 2.7e-2).
- * Default: the dQ pass works on fp16 copies of Q and K that it makes in the workspace (every bf16 value inside the fp16
- * range has an exact fp16 image, so S is unchanged) and rounds dS to fp16, 11 significant bits instead of 8, at the speed
- * of the once-rounded form; with one query head per KV head the dK/dV pass does the same for S, dS and its dK product (P and
+ * Default: the dQ pass works on fp16 copies of Q and K that it makes in the workspace (a bf16 value between 2^-17 and the
+ * fp16 range has an exact fp16 image, a smaller one is off by 2^-25 at most: S is unchanged) and rounds dS to fp16, 11 significant
+ * bits instead of 8, at the speed of the once-rounded form; with one query head per KV head the dK/dV pass does the same for S, dS and its dK product (P and
  * the dV product stay bf16: |dV| is small).  Measured against the oracle (fp32 outputs, 720p sample): dQ 8.7e-3, dK 3.5e-3.
  * A range flag guards the fp16 forms: a finite |Q| or |K| of 65520 or more, or a dS beyond the largest fp16 value, and the passes are
  * redone by the bf16-pair kernels described next (launched behind the fp16 ones, they return at once while the flag is clear).
+ * dS is scaled by a power of two per KV group, found from the largest |dO| and |O| of the group and taken out of the gradients
+ * again, so that the gradients of a mean over many elements (dO of 1e-7, say) do not end in the fp16 subnormals; heads of a
+ * group share the scale.
  * GQA groups (a KV block sums the query blocks of several heads) with TopK >= 8: the dK/dV pass makes fp16 copies of V and dO
- * as well and runs all four products in fp16, P included (480p sample: dK 9.4e-3, dV 2.7e-3; once-rounded bf16 2.2e-2 and
+ * as well (dO with the scale; where a group's |O| stays below 2^-16, V is taken to be too small for its copy and the flag goes
+ * up) and runs all four products in fp16, P included (480p sample: dK 9.4e-3, dV 2.7e-3; once-rounded bf16 2.2e-2 and
  * 1.4e-2), about 30 % faster than the pair form.
  * The pair form carries X as the bf16 value and the bf16 rounding of what that lost, in one product of twice the width: the
  * dK/dV pass of GQA groups uses it when rows keep fewer than 8 blocks or have per-row budgets (sharply peaked weights, where

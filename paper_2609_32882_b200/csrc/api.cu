@@ -19,7 +19,7 @@ struct RouteLayout {
   int words;
 };
 struct BwdLayout {
-  size_t status, delta, d_oc_hat, delta_c, dqc, dkc, dvc, pooled, total;
+  size_t status, delta, absmax, ds_exp, d_oc_hat, delta_c, dqc, dkc, dvc, pooled, total;
 };
 
 struct Carver {
@@ -144,6 +144,8 @@ BwdLayout bwd_layout(const Geo& g) {
   const size_t BHq = (size_t)g.batch * g.Hq;
   r.status = c.take(sizeof(StatusBlock));
   r.delta = c.take(BHq * g.S * sizeof(float));
+  r.absmax = c.take(BHq * (g.N + text_blocks(g)) * sizeof(float2));
+  r.ds_exp = c.take((size_t)g.batch * g.Hkv * sizeof(int));
   r.d_oc_hat = c.take(BHq * g.N * g.D * sizeof(float));
   r.delta_c = c.take(BHq * g.N * sizeof(float));
   r.dqc = c.take(BHq * g.N * g.D * sizeof(float));
@@ -646,10 +648,13 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   if (!coarse && dgate != nullptr)
     VSA2_CUDA(cudaMemsetAsync(dgate, 0, (size_t)g.batch * g.Hq * g.L * sizeof(float), st));
   const bf16* o_res = (saved != nullptr && !g.out_f32) ? reinterpret_cast<const bf16*>(saved->o_res) : nullptr;
+  // (V is copied to fp16 for GQA groups only; O is of V's size or, a mean of up to a few thousand rows, well below it)
+  const DsScale scale{at<float2>(workspace, lay.absmax), at<int>(workspace, lay.ds_exp), dkv_pass_gqa_f16(g) ? pow2i(-16) : 0.f};
   {
     ProfScope ps(VSA2_KERNEL_BWD_PRE, st, 1);
     VSA2_CUDA(launch_bwd_preprocess(fx, dob, o, o_res, coarse ? gate : nullptr, oc_hat, delta, coarse ? dgate : nullptr,
-                                    d_oc_hat, reinterpret_cast<StatusBlock*>(workspace), st));
+                                    d_oc_hat, dq_pass_f16(g) ? at<float2>(workspace, lay.absmax) : nullptr,
+                                    reinterpret_cast<StatusBlock*>(workspace), st));
   }
   if (coarse) {
     // pooled grid: the bf16 copies with the dense map, the pooled preprocess, dQ, dK/dV (+ two group spreads)
@@ -677,10 +682,9 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
     const bool f16 = dq_pass_f16(g);     // the copy, the fp16 form, the (idle) fallback
     ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st, ds_groups > 0 ? 2 : f16 ? 3 : 1);
     if (ds_groups > 0) {
-      VSA2_CUDA(launch_cast_bf16_to_f16(qb, at<unsigned char>(workspace, bwd_f16_offset(g)), (size_t)g.batch * g.Hq * g.S * g.D, kb,
-                                        at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)),
-                                        (size_t)g.batch * g.Hkv * g.S * g.D,
-                                        &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
+      VSA2_CUDA(launch_cast_qk(fx, qb, at<unsigned char>(workspace, bwd_f16_offset(g)), kb,
+                               at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale,
+                               &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
       VSA2_CUDA(launch_ds_positions(fx, row_ptr, col_idx, col_ptr, row_idx, at<int>(workspace, dl.pos), sd.counters,
                                     2 * g.batch * g.Hkv, st));
       if (dkv_order != nullptr) {
@@ -691,12 +695,12 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
       VSA2_CUDA(launch_fine_bwd128_dq_tc(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
                                          reinterpret_cast<StatusBlock*>(workspace), st,
                                          f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
-                                         f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr));
+                                         f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr, &scale));
     else
       VSA2_CUDA(launch_fine_bwd_dq_tc(fx, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
                                       reinterpret_cast<StatusBlock*>(workspace), st,
                                       f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
-                                      f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr));
+                                      f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr, &scale));
   }
   {
     const bool dkv128 = wide128 && !fine_bwd_dkv_wants_pair(n);
@@ -712,13 +716,14 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
       VSA2_CUDA(launch_fine_bwd128_dkv_tc(n, qb, kb, vb, dob, lse, delta, col_ptr, row_idx, coarse ? dkc : nullptr,
                                           coarse ? dvc : nullptr, dk, dv, reinterpret_cast<StatusBlock*>(workspace), st,
                                           dq_pass_f16(g) ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
-                                          dq_pass_f16(g) ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr));
+                                          dq_pass_f16(g) ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr,
+                                          scale.exp));
     else
       VSA2_CUDA(launch_fine_bwd_dkv_tc(fx, qb, kb, vb, dob, lse, delta, col_ptr, row_idx, coarse ? dkc : nullptr,
                                        coarse ? dvc : nullptr, dk, dv, reinterpret_cast<StatusBlock*>(workspace), st, true,
                                        f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
                                        f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr, v16,
-                                       gqa16 ? v16 + bwd_k16_bytes(g) : nullptr, ds_groups > 0 ? &sd : nullptr));
+                                       gqa16 ? v16 + bwd_k16_bytes(g) : nullptr, ds_groups > 0 ? &sd : nullptr, scale.exp));
   }
   return VSA2_OK;
 }

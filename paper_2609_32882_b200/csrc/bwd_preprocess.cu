@@ -1,6 +1,7 @@
 // First step of the backward pass: the per-token quantities of the gated merge (paper Eq. 14) and of the fine softmax
 // (Eq. 12) that the dQ and dK/dV passes (fine_bwd_tc.cu) and the coarse backward read:
 //   delta = rowsum(dO * O_f), dGate = rowsum(dO * O_c), dO_c_hat[n] = sum_{l in n} gate_l dO_l
+// and, for the scale of dS in the fp16 passes (DsScale in common.cuh), the largest |dO| and |O| of every block.
 // HBM-bound: one pass over dO, O (and the bf16 rounding residual of O).
 #include "common.cuh"
 
@@ -16,12 +17,14 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
                                                              const float* __restrict__ gate,
                                                              const float* __restrict__ oc_hat, Geo g,
                                                              float* __restrict__ delta, float* __restrict__ dgate,
-                                                             float* __restrict__ d_oc_hat, StatusBlock* clear) {
+                                                             float* __restrict__ d_oc_hat, float2* __restrict__ absmax,
+                                                             StatusBlock* clear) {
   constexpr int CH = D / 8;                // threads per token = 16-byte chunks of a token row
   constexpr int PAR = 256 / CH;            // tokens at a time
   constexpr int TOK = 2;                   // tokens in flight per thread
   __shared__ __align__(16) bf16 rows[kBlockTokens * D];
   __shared__ float gates[kBlockTokens];
+  __shared__ unsigned warp_max[2][8];
   if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(StatusBlock) / 4)
     reinterpret_cast<int*>(clear)[threadIdx.x] = 0;      // (for the kernels behind this one)
   const int i = blockIdx.x, ch = threadIdx.x % CH, hq = blockIdx.y, b = blockIdx.z;
@@ -39,6 +42,7 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
     ocv[0] = x.x; ocv[1] = x.y; ocv[2] = x.z; ocv[3] = x.w;
     ocv[4] = y.x; ocv[5] = y.y; ocv[6] = y.z; ocv[7] = y.w;
   }
+  unsigned most = 0u;                      // largest |O| (cut to bf16, upper half) and |dO|: bit patterns order like the numbers
 #pragma unroll 1
   for (int p0 = threadIdx.x / CH; p0 < kBlockTokens; p0 += TOK * PAR) {
     int l[TOK];
@@ -71,6 +75,9 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
         *reinterpret_cast<uint4*>(rows + p * D + ch * 8) = dv[u];
         if (ch == 0) gates[p] = gt[u];
       }
+      const unsigned d2_max = __vmaxu2(__vmaxu2(dv[u].x & 0x7fff7fffu, dv[u].y & 0x7fff7fffu),
+                                       __vmaxu2(dv[u].z & 0x7fff7fffu, dv[u].w & 0x7fff7fffu));
+      unsigned o_max = 0u;
       float ov[8], dd[8];
       const __nv_bfloat162* d2 = reinterpret_cast<const __nv_bfloat162*>(&dv[u]);
 #pragma unroll
@@ -95,7 +102,9 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
       for (int e = 0; e < 8; ++e) {
         s_oo = fmaf(dd[e], ov[e], s_oo);
         s_oc = fmaf(dd[e], ocv[e], s_oc);
+        o_max = max(o_max, __float_as_uint(ov[e]) & 0x7fff0000u);
       }
+      most = __vmaxu2(most, o_max | max(d2_max >> 16, d2_max & 0xffffu));
 #pragma unroll
       for (int off = CH / 2; off >= 1; off >>= 1) {
         s_oo += __shfl_xor_sync(group_mask, s_oo, off);
@@ -107,8 +116,17 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
       }
     }
   }
-  if (!coarse) return;
+  const unsigned d_max = __reduce_max_sync(0xffffffffu, most << 16), o_max = __reduce_max_sync(0xffffffffu, most & 0xffff0000u);
+  if (lane == 0) {
+    warp_max[0][threadIdx.x >> 5] = d_max;
+    warp_max[1][threadIdx.x >> 5] = o_max;
+  }
   __syncthreads();
+  if (absmax != nullptr && threadIdx.x < 8) {
+    const unsigned dm = __reduce_max_sync(0xffu, warp_max[0][threadIdx.x]), om = __reduce_max_sync(0xffu, warp_max[1][threadIdx.x]);
+    if (threadIdx.x == 0) absmax[bhq * g.N + i] = make_float2(__uint_as_float(dm), __uint_as_float(om));
+  }
+  if (!coarse) return;
   if (threadIdx.x < D) {
     float acc = 0.f;
 #pragma unroll 16
@@ -118,11 +136,11 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
 }
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
-                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat,
+                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, float2* absmax,
                                   StatusBlock* clear, cudaStream_t st) {
   dim3 grid(g.N, g.Hq, g.batch);
-  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, clear);
-  else bwd_preprocess_kernel<64><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, clear);
+  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  else bwd_preprocess_kernel<64><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
   return cudaGetLastError();
 }
 

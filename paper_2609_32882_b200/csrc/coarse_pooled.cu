@@ -153,11 +153,11 @@ cudaError_t launch_coarse_bwd_pooled(const Geo& g, const float* qc, const float*
                         ptr, idx, p.N, BHq * ((size_t)p.N * p.N + p.N + 1), status};
   if ((e = launch_pooled_inputs(in, st)) != cudaSuccess) return e;
   // delta_c = rowsum(dO_c * O_c) through the preprocess kernel of the pooled problem (no gate: only delta is written)
-  if ((e = launch_bwd_preprocess(p, do16, oc_hat, nullptr, nullptr, nullptr, delta, nullptr, nullptr, nullptr, st)) != cudaSuccess) return e;
-  if ((e = launch_fine_bwd_dq_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, dqc, status, st, nullptr, nullptr)) != cudaSuccess) return e;
+  if ((e = launch_bwd_preprocess(p, do16, oc_hat, nullptr, nullptr, nullptr, delta, nullptr, nullptr, nullptr, nullptr, st)) != cudaSuccess) return e;
+  if ((e = launch_fine_bwd_dq_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, dqc, status, st, nullptr, nullptr, nullptr)) != cudaSuccess) return e;
   const bool grouped = g.rep > 1;
   if ((e = launch_fine_bwd_dkv_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, nullptr, grouped ? dk_kv : dkc,
-                                  grouped ? dv_kv : dvc, status, st, false, nullptr, nullptr, nullptr, nullptr, nullptr)) != cudaSuccess)
+                                  grouped ? dv_kv : dvc, status, st, false, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr)) != cudaSuccess)
     return e;
   if (grouped) {
     const size_t per_head4 = (size_t)g.N * g.D / 4;

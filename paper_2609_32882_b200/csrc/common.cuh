@@ -294,27 +294,50 @@ cudaError_t launch_fine_fwd_rows2_tc(const Geo& g, bool pair_heads, const bf16* 
                                      const int* row_ptr, const int* col_idx, const float* oc_hat, void* o, bf16* o_res,
                                      float* lse, StatusBlock* status, cudaStream_t st);
 
+// Scale of dS in the passes that round it to fp16: 2^exp per KV group.  dS is a weight of about one over the kept keys times a
+// sum over dO V, so an unscaled fp16 dS has lost its bits to the subnormals long before dO is small (dO of 1e-4, 4096 keys: a
+// few per cent of dQ; of 1e-7: all of it).  The exponent lifts max|dO| max|O| of the group to 2^-3 (O is a mean of V rows, so it
+// is of V's size wherever a weight is large) and is never negative: gradients of ordinary size keep exponent 0, and a dS that
+// the scale takes beyond the fp16 range ends in the range fallback like any other.  It is folded into the row statistics
+// (lse, or delta where dO itself is a scaled copy) and taken out again by the epilogues, both exact.
+struct DsScale {
+  const float2* absmax;   // [B, Hq, N of the block problem]: max |dO|, max |O| of each block (launch_bwd_preprocess)
+  int* exp;               // [B, Hkv], written by launch_cast_qk
+  // 0, or (where dP is formed from an fp16 copy of V) the max |O| below which a group's V counts as too small for that copy and
+  // the range flag goes up: an element of it is then good to 2^-9 of V's size at worst
+  float least_o;
+};
+__host__ __device__ __forceinline__ float pow2i(int e) {      // 2^e, |e| <= 126
+  union { int i; float f; } u{(127 + e) << 23};
+  return u.f;
+}
+
 // tensor-core backward passes for cubes of 128 tokens (fine_bwd128_tc.cu): `g` and the maps are those of the half-cube problem
 bool fine_bwd128_supported(const Geo& g);
 bool fine_bwd_dkv_wants_pair(const Geo& g);
 cudaError_t launch_fine_bwd128_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                      const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
-                                     const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16);
+                                     const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
+                                     const DsScale* scale);
 cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                       const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                       const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
-                                      cudaStream_t st, const void* q16, const void* k16);
+                                      cudaStream_t st, const void* q16, const void* k16, const int* ds_exp);
 
 // tensor-core backward passes (fine_bwd_tc.cu)
 cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                   const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
-                                  const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16);
+                                  const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
+                                     const DsScale* scale);
 bool fine_bwd_dq_uses_f16(const Geo& g);
 // Slot of StatusBlock.pad that holds the range flag of the fp16 dQ passes (the slot behind it: the fallback launch's counter)
 constexpr int kRangeFlagSlot = 8;
-// fp16 copies of two bf16 tensors (element counts multiples of 8); a finite value beyond the fp16 range sets *range_flag
-cudaError_t launch_cast_bf16_to_f16(const bf16* a, void* a16, size_t na, const bf16* b, void* b16, size_t nb, int* range_flag,
-                                    cudaStream_t st);
+// fp16 copies of Q and K; a finite value beyond the fp16 range sets *range_flag.  Also forms scale->exp
+cudaError_t launch_cast_qk(const Geo& g, const bf16* q, void* q16, const bf16* k, void* k16, const DsScale& scale, int* range_flag,
+                           cudaStream_t st);
+// fp16 copies of V and of dO times 2^ds_exp of its KV group, with the same flag
+cudaError_t launch_cast_v_do(const Geo& g, const bf16* v, void* v16, const bf16* d_o, void* do16, const int* ds_exp, int* range_flag,
+                             cudaStream_t st);
 // dS kept between the two backward passes (fine_bwd_dq_ds_tc.cu): scratch for the pairs of `chunk_groups` KV groups at a time
 struct StoredDs {
   void* scratch;        // chunk_groups * rep * nnz_cap tiles of 8 KB (64 queries x 64 keys, fp16)
@@ -332,7 +355,7 @@ cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col
 cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st);
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
-                                  int* item_counter, bool swizzled, cudaStream_t st);
+                                  int* item_counter, bool swizzled, const int* ds_exp, cudaStream_t st);
 cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse,
                                         const float* delta, const int* row_ptr, const int* col_idx, const float* dqc, void* dq,
                                         StatusBlock* status, cudaStream_t st);
@@ -340,11 +363,11 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
-                                   const void* k16, void* v16, void* do16, const StoredDs* sd);
+                                   const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp);
 bool fine_bwd_dkv_gqa_uses_f16(const Geo& g);
 bool fine_bwd_dkv_splits_long_columns(const Geo& g, bool split_long_columns);
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
-                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat,
+                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, float2* absmax,
                                   StatusBlock* clear, cudaStream_t st);
 }  // namespace vsa2

@@ -67,6 +67,7 @@ struct Bwd128Args {
   StatusBlock* status;
   int* range_flag;      // fp16 form of the dQ pass and its fallback: as in DqArgs of the 64-token pass (when = 0: always runs)
   int when;
+  const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale; fp16 forms): the weights carry it
 };
 
 // The stationary cube of a work item and the lists of streamed cubes that meet it.
@@ -457,6 +458,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
         VSA2_NEXT_ITEM_WARP(item, seq);
         ItemLists<PASS> il;
         il.init(g, item);
+        const float lse_off = F16 && a.ds_exp != nullptr ? (float)a.ds_exp[il.bh_stat] : 0.f;
         for (int l_ = 0; l_ < il.nl; ++l_) {
           const int mh = il.bhq0 + l_;
           const int beg = a.ptr[(size_t)mh * (g.N + 1) + il.blk0];
@@ -512,7 +514,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
     }                                                                                                         \
     VSA2_WAIT_PARKED(&misc->stat_free, (tg & 1) ^ 1);                                                         \
     _Pragma("unroll") for (int u = 0; u < 4; ++u)                                                             \
-        misc->lse2[lane + 32 * u] = ((CUR##_ok >> u) & 1u) ? CUR##_ls[u] * 1.4426950408889634f : INFINITY;    \
+        misc->lse2[lane + 32 * u] = ((CUR##_ok >> u) & 1u) ? CUR##_ls[u] * 1.4426950408889634f - lse_off : INFINITY;    \
     tc::mbar_arrive(&misc->stat_full);                                                                        \
     VSA2_WAIT_PARKED(&misc->dlt_free, (tg & 1) ^ 1);                                                          \
     _Pragma("unroll") for (int u = 0; u < 4; ++u)                                                             \
@@ -555,9 +557,10 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
       const int nt_all = il.tiles(g, a);
       const int blk = il.blk0 + member;
       const int l_tok = block_token(g, blk, row & 63);
+      const int ds_exp = F16 && a.ds_exp != nullptr ? a.ds_exp[PASS == 0 ? il.bh_y0 : il.bh_stat] : 0;
       float lse2 = INFINITY, dlt = 0.f;
       if (PASS == 0 && l_tok >= 0) {
-        lse2 = a.lse[(size_t)il.bh_stat * g.S + l_tok] * 1.4426950408889634f;
+        lse2 = a.lse[(size_t)il.bh_stat * g.S + l_tok] * 1.4426950408889634f - (float)ds_exp;
         dlt = a.delta[(size_t)il.bh_stat * g.S + l_tok];
       }
       if (nt_all > 0) {
@@ -692,7 +695,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
             }
             if (l_tok < 0) continue;
             float val[32];
-            const float sc = (PASS == 0 || o == 0) ? g.scale : 1.f;      // dQ, dK = scale * (dS Y0); dV = P Y1
+            const float sc = ((PASS == 0 || o == 0) ? g.scale : 1.f) * pow2i(-ds_exp);      // dQ, dK = scale * (dS Y0); dV = P Y1
 #pragma unroll
             for (int e = 0; e < 32; ++e) val[e] = __uint_as_float(acc[e]) * sc;
             if (cterm != nullptr) {
@@ -773,9 +776,10 @@ static cudaError_t launch_bwd128(const CUtensorMap& x0, const CUtensorMap& x1, c
 // launch_fine_bwd_dq_tc
 cudaError_t launch_fine_bwd128_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                      const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
-                                     const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16) {
+                                     const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
+                                     const DsScale* scale) {
   if (!fine_bwd128_supported(g)) return cudaErrorInvalidValue;
-  const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr;
+  const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr && scale != nullptr;
   CUtensorMap tq, tk, tv, tdo, tq16, tk16;
   if (!make_cube_tmap(&tq, q, g, g.Hq) || !make_cube_tmap(&tk, k, g, g.Hkv) || !make_cube_tmap(&tv, v, g, g.Hkv) ||
       !make_cube_tmap(&tdo, d_o, g, g.Hq))
@@ -787,20 +791,19 @@ cudaError_t launch_fine_bwd128_dq_tc(const Geo& g, const bf16* q, const bf16* k,
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
-  Bwd128Args a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, nullptr, dq, nullptr, status, flag, 0};
+  Bwd128Args a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, nullptr, dq, nullptr, status, flag, 0, f16 ? scale->exp : nullptr};
   const int total = g.batch * g.Hq * (g.N / 2);
   const int grid = total < sms ? total : sms;
   const bool split = !(g.flags & VSA2_FLAG_FAST_BWD);
   if (f16) {
     // the copy, the fp16 form, and the pair form that runs only if the range flag came up (see launch_fine_bwd_dq_tc)
-    if ((e = launch_cast_bf16_to_f16(q, q16, (size_t)g.batch * g.Hq * g.S * g.D, k, k16, (size_t)g.batch * g.Hkv * g.S * g.D, flag,
-                                     st)) != cudaSuccess)
-      return e;
+    if ((e = launch_cast_qk(g, q, q16, k, k16, *scale, flag, st)) != cudaSuccess) return e;
     a.when = 1;
     e = g.D == 128 ? launch_bwd128<128, 0, false, true>(tq16, tdo, tk16, tv, g, a, grid, st)
                    : launch_bwd128<64, 0, false, true>(tq16, tdo, tk16, tv, g, a, grid, st);
     if (e != cudaSuccess) return e;
     a.when = 2;
+    a.ds_exp = nullptr;
     a.item_counter = &status->pad[kRangeFlagSlot + 1];
     return g.D == 128 ? launch_bwd128<128, 0, true>(tq, tdo, tk, tv, g, a, grid, st) : launch_bwd128<64, 0, true>(tq, tdo, tk, tv, g, a, grid, st);
   }
@@ -812,7 +815,7 @@ cudaError_t launch_fine_bwd128_dq_tc(const Geo& g, const bf16* q, const bf16* k,
 cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                       const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                       const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
-                                      cudaStream_t st, const void* q16, const void* k16) {
+                                      cudaStream_t st, const void* q16, const void* k16, const int* ds_exp) {
   if (!fine_bwd128_supported(g)) return cudaErrorInvalidValue;
   // `q16`, `k16`: null, or the fp16 copies of Q and K that the dQ pass of the same call has made (and whose range flag it has
   // settled): the pass then runs in its fp16 form, with the bf16 form behind the flag
@@ -827,7 +830,8 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  Bwd128Args a{&status->pad[3], lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, &status->pad[kRangeFlagSlot], 0};
+  Bwd128Args a{&status->pad[3], lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, &status->pad[kRangeFlagSlot], 0,
+               f16 ? ds_exp : nullptr};
   const int total = g.batch * g.Hkv * (g.N / 2);
   const int grid = total < sms ? total : sms;
   const bool split = fine_bwd_dkv_wants_pair(g);
@@ -838,6 +842,7 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
                    : launch_bwd128<64, 1, false, true>(tk16, tv, tq16, tdo, g, a, grid, st);
     if (e != cudaSuccess) return e;
     a.when = 2;
+    a.ds_exp = nullptr;
     a.item_counter = &status->pad[5];
   }
   if (g.D == 128) return launch_bwd128<128, 1, false>(tk, tv, tq, tdo, g, a, grid, st);

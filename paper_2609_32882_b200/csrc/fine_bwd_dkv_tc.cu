@@ -30,6 +30,7 @@ struct DkvArgs {
   unsigned char* ds;    // null, or the scratch for dS in fp16 (forms STORES_DS): [entry of the row lists of heads ds_head0 ..][8 chunks of 8 keys][64 q]
   const int* ds_pos;    // [B, Hq, nnz_cap]: place of every entry of the column lists in the row lists
   int ds_head0;
+  const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale; forms whose dS is rounded to fp16)
   const int* order;     // null, or the order in which the items are drawn
 };
 
@@ -80,6 +81,8 @@ __device__ __forceinline__ void dkv_entry(const Geo& g, const DkvArgs& a, int re
 // that pass finds and turns into the range flag; the fp16 forms then also use it unclamped (their result is redone).
 // No key column is masked: the columns of positions without a token are accumulator columns that are never read out, and
 // in dQ they meet zero rows of K (fine_bwd_tc.cu).
+// dS is scaled by 2^ds_exp (DsScale).  The weights carry the scale, through the lse of a row, so P and dV^T are scaled as well (P is
+// bf16 there, whose range has room); with F16 = 2 the copy of dO carries it and delta is multiplied.  The epilogue takes it out.
 // F16 = 2: all four maps point at fp16 copies and P is rounded to fp16 as well (every product fp16 x fp16): the form for GQA
 // groups, where a KV block sums the query blocks of several heads and bf16 P leaves dV at 1.4e-2 (480p sample, |dV| = 11).
 template <int D, bool SPLIT, bool MHA, int F16>
@@ -319,7 +322,9 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       VSA2_NEXT_REC(rec, seq);
       if (rec.z == 0) continue;
       VSA2_DKV_ITEM_SETUP();
-      (void)j; (void)bhk;
+      (void)j;
+      const int ds_exp = a.ds_exp != nullptr ? a.ds_exp[bhk] : 0;
+      const float lse_off = F16 == 2 ? 0.f : (float)ds_exp, dlt_scale = F16 == 2 ? pow2i(ds_exp) : 1.f;
       const int nt = (k + 1) >> 1;
       int bhq_n, i_n, pos_n = 0;
       dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n, &pos_n);
@@ -333,7 +338,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_n, i_n, &pos_n);
         VSA2_WAIT_PARKED(&misc->stat_free, (tg & 1) ^ 1);
         if (STORES_DS && (r & 63) == 0) misc->ds_slot[tg & 3][blk] = dup ? -1 : slot;
-        rowstat[r] = make_float2(l >= 0 ? lse_raw * 1.4426950408889634f : INFINITY, l >= 0 ? dlt_raw : 0.f);
+        rowstat[r] = make_float2(l >= 0 ? lse_raw * 1.4426950408889634f - lse_off : INFINITY, l >= 0 ? dlt_raw * dlt_scale : 0.f);
         tc::mbar_arrive(&misc->stat_full);
       }
     }
@@ -462,6 +467,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         coarse[0] *= inv_cnt;
         coarse[1] *= inv_cnt;
       }
+      const float inv_scale = a.ds_exp != nullptr ? pow2i(-a.ds_exp[bhk]) : 1.f, k_scale = g.scale * inv_scale;
       const size_t head = (size_t)bhk * g.S;
       if (k == 0) {                            // nothing kept: the coarse gradients only
         for (int c = 0; c < 64; ++c) {
@@ -507,7 +513,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         }
         const float add = is_v ? coarse[1] : coarse[0];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) v[c] = is_v ? v[c] + add : fmaf(v[c], g.scale, add);
+        for (int c = 0; c < 32; ++c) v[c] = fmaf(v[c], is_v ? inv_scale : k_scale, add);
         if (row < D) store_channels<D>(is_v ? a.dv : a.dk, g.out_f32, head, tok + (part & 1) * 32, v, row);
       }
       if constexpr (!SPLIT) {
@@ -551,7 +557,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
-                                   const void* k16, void* v16, void* do16, const StoredDs* sd) {
+                                   const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp) {
   if (g.rep > kMaxRep) return cudaErrorInvalidValue;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16;
   // GQA groups without a precision flag take the all-fp16 form when they are given scratch for fp16 copies of V and dO as
@@ -598,7 +604,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     cfg.stream = st;
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
-              group0 * g.rep, ds ? sd->order : nullptr};
+              group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr};
     if (when == 1 && gqa16) {       // every product in fp16
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
       else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
@@ -631,16 +637,14 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
       const int n = all - g0 < sd->chunk_groups ? all - g0 : sd->chunk_groups;
       if ((r = launch(split, sd->counters + 2 * c, 0, kAll, when, g0, n, true)) != cudaSuccess) return r;
       if ((r = launch_fine_bwd_dq_ds(g, k16, sd->scratch, g0 * g.rep, n * g.rep, sd->row_ptr, sd->col_idx, sd->dqc, sd->dq, status,
-                                     range_flag, sd->counters + 2 * c + 1, !split, st)) != cudaSuccess)
+                                     range_flag, sd->counters + 2 * c + 1, !split, ds_exp, st)) != cudaSuccess)
         return r;
     }
     // dQ again, from bf16 pairs, if a value left the fp16 range
     return launch_fine_bwd_dq_fallback(g, q, k, v, d_o, lse, delta, sd->row_ptr, sd->col_idx, sd->dqc, sd->dq, status, st);
   };
   if (f16 && gqa16) {
-    if ((e = launch_cast_bf16_to_f16(v, v16, (size_t)g.batch * g.Hkv * g.S * g.D, d_o, do16, (size_t)g.batch * g.Hq * g.S * g.D,
-                                     range_flag, st)) != cudaSuccess)
-      return e;
+    if ((e = launch_cast_v_do(g, v, v16, d_o, do16, ds_exp, range_flag, st)) != cudaSuccess) return e;
     if ((e = main_pass(false, 1)) != cudaSuccess) return e;
     return launch(true, &status->pad[4], 0, kAll, 2, 0, all, false);
   }

@@ -147,7 +147,8 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
     }
   } else if (warp < 12) {
     // ------------------------------------------------------------------ epilogue: two warpgroups take the items in turn, a thread
-    // has one channel: dQ[l, d] = scale * dQ^T[d, q] + dQ_c[i, d] / count(i) (dS comes without the softmax scale)
+    // has one channel: dQ[l, d] = scale * dQ^T[d, q] + dQ_c[i, d] / count(i) (dS comes without the softmax scale and
+    // with its own)
     const int wg = (warp - 4) >> 2;
     const int row = ((warp & 3) << 5) | lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
@@ -161,6 +162,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       const int tok0 = block_token(g, i, lane), tok1 = block_token(g, i, 32 + lane);
       const float coarse_d = (a.dqc != nullptr && row < D && !block_is_text(g, i))
                                  ? a.dqc[((size_t)rec.y * g.Nvid + i) * D + row] / (float)cube_count(g, i) : 0.f;
+      const float out_scale = g.scale * pow2i(-a.ds_exp[rec.y / g.rep]);      // (rec.y / rep: batch * Hkv + KV head)
       const size_t head = (size_t)rec.y * g.S;
       if (k == 0) {                            // nothing kept: the coarse gradient only
         for (int c = 0; c < 64; ++c) {
@@ -187,7 +189,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         if (row < D && any_non_finite32(x)) atomicExch(a.range_flag, 1);
         float v[32];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) v[c] = fmaf(__uint_as_float(x[c]), g.scale, coarse_d);
+        for (int c = 0; c < 32; ++c) v[c] = fmaf(__uint_as_float(x[c]), out_scale, coarse_d);
         if (row < D) store_channels<D>(a.dq, g.out_f32, head, tok + part * 32, v, row);
       }
       tc::tc_fence_before();
@@ -298,7 +300,7 @@ cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaS
 // dQ of the heads head0 .. head0 + heads - 1 (index batch * Hq) from their dS tiles
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
-                                  int* item_counter, bool swizzled, cudaStream_t st) {
+                                  int* item_counter, bool swizzled, const int* ds_exp, cudaStream_t st) {
   CUtensorMap tk, tkt;
   if (!make_cube_tmap(&tk, reinterpret_cast<const bf16*>(k16), g, g.Hkv) ||      // (same element size: the maps only move bytes)
       !make_text_tmap(&tkt, reinterpret_cast<const bf16*>(k16), g, g.Hkv))
@@ -306,7 +308,7 @@ cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds,
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), swizzled ? 1 : 0, dqc, dq, status, range_flag, head0, head0 * g.N, heads * g.N};
+  DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), swizzled ? 1 : 0, dqc, dq, status, range_flag, ds_exp, head0, head0 * g.N, heads * g.N};
   const int grid = a.items < sms ? a.items : sms;
 #define VSA2_LAUNCH_DQ_DS(DD)                                                                                                    \
   do {                                                                                                                           \

@@ -40,16 +40,53 @@ struct DqArgs {
   // always runs; 1: it runs if the flag is clear (and sets it if a dS saturates); 2: it runs only if the flag is set.
   int* range_flag;
   int when;
+  const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale)
 };
 
-// Copies of two bf16 tensors in fp16 (8 elements per thread and step).  Every finite bf16 below 65520 in magnitude has an
-// exact fp16 image down to 2^-24 granularity (fp16 keeps more mantissa bits), so products of the copies equal the products
-// of the originals; a finite value beyond that range sets `range_flag` and the caller's fp16 kernels stand back.
+// DsScale::exp of the groups blockIdx.x, blockIdx.x + gridDim.x, ... (the whole block calls it); true if one is below least_o
+__device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int per_group) {
+  __shared__ unsigned red[2][8];
+  bool small = false;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+    const uint2* m = reinterpret_cast<const uint2*>(s.absmax) + (size_t)grp * per_group;      // (bit patterns order like the numbers)
+    unsigned d = 0u, o = 0u;
+    for (int i = threadIdx.x; i < per_group; i += 256) {
+      const uint2 v = __ldg(m + i);
+      d = max(d, v.x);
+      o = max(o, v.y);
+    }
+    d = __reduce_max_sync(0xffffffffu, d);
+    o = __reduce_max_sync(0xffffffffu, o);
+    if (lane == 0) {
+      red[0][warp] = d;
+      red[1][warp] = o;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) {
+        d = max(d, red[0][w]);
+        o = max(o, red[1][w]);
+      }
+      const int e = (int)(d >> 23) - 127 + (int)(o >> 23) - 127;
+      s.exp[grp] = d == 0u || o == 0u ? 0 : max(0, min(-3 - e, 100));
+      small |= o != 0u && __uint_as_float(o) < s.least_o;
+    }
+    __syncthreads();
+  }
+  return small;
+}
+
+// Copies of two bf16 tensors in fp16 (8 elements per thread and step), b times 2^b_exp[its group of `b_group` steps] if there is one.
+// A finite bf16 below 65520 in magnitude has an exact fp16 image if it is a multiple of 2^-24 (all of 2^-17 and more are: fp16
+// keeps more mantissa bits), and one within 2^-25 otherwise; a finite value beyond that range sets `range_flag` and the caller's
+// fp16 kernels stand back.  With scale.absmax the launch also forms the exponents of dS.
 __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __restrict__ xa, uint4* __restrict__ ya, size_t na,
                                                                const uint4* __restrict__ xb, uint4* __restrict__ yb, size_t nb,
-                                                               int* range_flag) {
+                                                               const int* __restrict__ b_exp, unsigned b_group, int* range_flag,
+                                                               DsScale scale, int groups, int per_group) {
   const size_t stride = (size_t)gridDim.x * blockDim.x, n = na + nb;
-  bool bad = false;
+  bool bad = scale.absmax != nullptr && form_ds_exp(scale, groups, per_group);
   constexpr int U = 4;      // 16-byte loads in flight per thread (a pure streaming kernel)
   for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += U * stride) {
     uint4 v[U];
@@ -63,12 +100,15 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
       const size_t i = i0 + u * stride;
       if (i >= n) break;
       const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+      // (a scaled value stays finite: the exponent takes the largest of a group to 2^-2 / max |O| at most)
+      const float f = b_exp != nullptr && i >= na ? pow2i(__ldg(b_exp + (unsigned)(i - na) / b_group)) : 1.f;
       uint32_t r[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const uint32_t m0 = w[e] & 0x7fffu, m1 = (w[e] >> 16) & 0x7fffu;     // magnitudes as bf16 bit patterns (0x4780 = 65536)
-        bad |= (m0 >= 0x4780u && m0 < 0x7f80u) || (m1 >= 0x4780u && m1 < 0x7f80u);
-        const __half2 h = __floats2half2_rn(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
+        const float x0 = __uint_as_float(w[e] << 16) * f, x1 = __uint_as_float(w[e] & 0xffff0000u) * f;
+        const float m0 = fabsf(x0), m1 = fabsf(x1);
+        bad |= (m0 >= 65536.f && m0 < INFINITY) || (m1 >= 65536.f && m1 < INFINITY);
+        const __half2 h = __floats2half2_rn(x0, x1);
         r[e] = *reinterpret_cast<const uint32_t*>(&h);
       }
       const uint4 o = make_uint4(r[0], r[1], r[2], r[3]);
@@ -89,7 +129,7 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
 // F16 (without SPLIT): the maps of Q and K point at fp16 copies of the tensors and dS^T is rounded to fp16, so S^T and the
 // dQ^T product are fp16 x fp16 instructions (dP^T stays bf16 x bf16: V and dO are not copied).  S^T comes out as with the
 // bf16 originals (the copies are exact), dS keeps 11 significant bits instead of 8, which is what the pair form is for, at
-// the cost of the plain form.
+// the cost of the plain form.  dS is scaled by 2^ds_exp (DsScale): the weights are, through the lse of a row.
 template <int D, bool SPLIT, bool F16>
 __global__ void __launch_bounds__(kDqThreads, 1)
 fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -281,12 +321,14 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
       item_block(g, item, bhq, i);
       const int beg = a.row_ptr[(size_t)bhq * (g.N + 1) + i], end = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1];
       const int k = end - beg;
+      const int ds_exp = F16 && a.ds_exp != nullptr ? a.ds_exp[bhq / g.rep] : 0;      // (bhq / rep: batch * Hkv + KV head)
+      const float out_scale = g.scale * pow2i(-ds_exp);
       const int tb = n_all & 1;
       const uint32_t e_sync0 = n_all * (g.out_f32 ? 1u : 3u);     // index of this item's first group sync
       if (sm_tid < 64) {
         const int l = block_token(g, i, sm_tid);
         misc->tok[tb * 64 + sm_tid] = l;
-        misc->stats[tb * 64 + sm_tid] = l >= 0 ? a.lse[(size_t)bhq * g.S + l] * 1.4426950408889634f : INFINITY;
+        misc->stats[tb * 64 + sm_tid] = l >= 0 ? a.lse[(size_t)bhq * g.S + l] * 1.4426950408889634f - (float)ds_exp : INFINITY;
         misc->stats[128 + tb * 64 + sm_tid] = l >= 0 ? a.delta[(size_t)bhq * g.S + l] : 0.f;
       }
       const float coarse_d = (a.dqc != nullptr && row < D && !block_is_text(g, i))
@@ -403,7 +445,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             for (int c = 0; c < 32; ++c) {
               const int l = misc->tok[tb * 64 + half * 32 + c];
               if (l < 0) continue;
-              store_out(a.dq, ((size_t)bhq * g.S + l) * D + row, fmaf(__uint_as_float(o0[c]), g.scale, coarse_d), 1);
+              store_out(a.dq, ((size_t)bhq * g.S + l) * D + row, fmaf(__uint_as_float(o0[c]), out_scale, coarse_d), 1);
             }
           }
         } else {
@@ -412,7 +454,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
           if (row < D) {
 #pragma unroll
             for (int c = 0; c < 32; ++c)
-              st[(half * 32 + c) * D + row] = __float2bfloat16_rn(fmaf(__uint_as_float(o0[c]), g.scale, coarse_d));
+              st[(half * 32 + c) * D + row] = __float2bfloat16_rn(fmaf(__uint_as_float(o0[c]), out_scale, coarse_d));
           }
           VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0 + 1);
           constexpr int CH = D / 8;
@@ -448,13 +490,14 @@ done:
 // ================================================================================================
 // launcher
 // ================================================================================================
-// `q16`, `k16`: null, or scratch for fp16 copies of Q and K (as many elements as the tensors).  With them the default pass
+// `q16`, `k16`, `scale`: null, or scratch for fp16 copies of Q and K (as many elements as the tensors) and for the scale of dS.  With them the default pass
 // (no precision flag) is: the copy, the fp16 form of the kernel, and a launch of the pair form that does nothing unless the
 // range flag came up (a finite |Q|, |K| >= 65520 or a |dS| >= 65504: the pair form then computes dQ as before).
 cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                   const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
-                                  const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16) {
-  const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr;
+                                  const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
+                                  const DsScale* scale) {
+  const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr && scale != nullptr;
   const bf16* qa = f16 ? reinterpret_cast<const bf16*>(q16) : q;      // (same element size and layout: the maps only move bytes)
   const bf16* ka = f16 ? reinterpret_cast<const bf16*>(k16) : k;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot;
@@ -466,7 +509,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
-  DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, status, flag, 0};
+  DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, status, flag, 0, f16 ? scale->exp : nullptr};
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
   const bool split = !(g.flags & VSA2_FLAG_FAST_BWD);
@@ -477,9 +520,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
     fine_bwd_dq_tc_kernel<DD, SP, F><<<grid, kDqThreads, BwdTc<DD>::smem_bytes, st>>>(TQ, TK, tv, tdo, TQT, TKT, tvt, tdot, g, a); \
   } while (0)
   if (f16) {
-    if ((e = launch_cast_bf16_to_f16(q, q16, (size_t)g.batch * g.Hq * g.S * g.D, k, k16, (size_t)g.batch * g.Hkv * g.S * g.D, flag,
-                                     st)) != cudaSuccess)
-      return e;
+    if ((e = launch_cast_qk(g, q, q16, k, k16, *scale, flag, st)) != cudaSuccess) return e;
     a.when = 1;
     if (g.D == 128) VSA2_LAUNCH_DQ(128, false, true, tq, tk, tqt, tkt);
     else VSA2_LAUNCH_DQ(64, false, true, tq, tk, tqt, tkt);
@@ -508,7 +549,7 @@ cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16*
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  DqArgs a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, dq, status, &status->pad[kRangeFlagSlot], 2};
+  DqArgs a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, dq, status, &status->pad[kRangeFlagSlot], 2, nullptr};
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
   if (g.D == 128) VSA2_LAUNCH_DQ(128, true, false, tq, tk, tqt, tkt);
@@ -517,16 +558,30 @@ cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16*
 }
 #undef VSA2_LAUNCH_DQ
 
-cudaError_t launch_cast_bf16_to_f16(const bf16* a, void* a16, size_t na, const bf16* b, void* b16, size_t nb, int* range_flag,
-                                    cudaStream_t st) {
+static cudaError_t launch_cast(const bf16* a, void* a16, size_t na, const bf16* b, void* b16, size_t nb, const int* b_exp, size_t b_group,
+                               const DsScale& scale, int groups, int per_group, int* range_flag, cudaStream_t st) {
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  if ((na | nb) & 7) return cudaErrorInvalidValue;
+  // (element counts are multiples of the head dimension)
   cast_bf16_to_f16_kernel<<<sms * 16, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
-                                                     reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8,
-                                                     range_flag);
+                                                     reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8, b_exp,
+                                                     (unsigned)(b_group / 8), range_flag, scale, groups, per_group);
   return cudaGetLastError();
+}
+
+cudaError_t launch_cast_qk(const Geo& g, const bf16* q, void* q16, const bf16* k, void* k16, const DsScale& scale, int* range_flag,
+                           cudaStream_t st) {
+  const size_t head = (size_t)g.S * g.D;
+  return launch_cast(q, q16, (size_t)g.batch * g.Hq * head, k, k16, (size_t)g.batch * g.Hkv * head, nullptr, 8, scale, g.batch * g.Hkv,
+                     g.rep * g.N, range_flag, st);
+}
+
+cudaError_t launch_cast_v_do(const Geo& g, const bf16* v, void* v16, const bf16* d_o, void* do16, const int* ds_exp, int* range_flag,
+                             cudaStream_t st) {
+  const size_t head = (size_t)g.S * g.D;
+  return launch_cast(v, v16, (size_t)g.batch * g.Hkv * head, d_o, do16, (size_t)g.batch * g.Hq * head, ds_exp, g.rep * head, DsScale{}, 0, 0,
+                     range_flag, st);
 }
 
 // whether the dQ pass of this problem takes its fp16 form when it is given the scratch for the copies

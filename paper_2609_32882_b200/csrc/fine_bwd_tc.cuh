@@ -133,6 +133,7 @@ struct DqDsArgs {
   void* dq;
   StatusBlock* status;
   int* range_flag;      // the launch runs if it is clear, and sets it if a dS had left the fp16 range
+  const int* ds_exp;    // exponent of the scale of dS per KV group (DsScale)
   int head0;            // (batch * Hq) index of the first head of the dS scratch
   int first_item, items;
 };
