@@ -85,6 +85,8 @@ __device__ __forceinline__ void dkv_entry(const Geo& g, const DkvArgs& a, int re
 // bf16 there, whose range has room); with F16 = 2 the copy of dO carries it and delta is multiplied.  The epilogue takes it out.
 // F16 = 2: all four maps point at fp16 copies and P is rounded to fp16 as well (every product fp16 x fp16): the form for GQA
 // groups, where a KV block sums the query blocks of several heads and bf16 P leaves dV at 1.4e-2 (480p sample, |dV| = 11).
+// F16 = 3: the same without `a.ds`, dS clamped: the recomputing dQ pass forms dP from the bf16 originals, of which the copies of V and
+// dO can be 2^-25 off, so of a dS next to the limit one pass may have 65504 and the other an infinity that no flag tells of.
 template <int D, bool SPLIT, bool MHA, int F16>
 __global__ void __launch_bounds__(kDkvThreads, 1)
 fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -107,7 +109,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float c2 = g.scale * 1.4426950408889634f;
   const int rep = MHA ? 1 : g.rep;
-  constexpr bool STORES_DS = F16 != 0 || (SPLIT && !MHA);
+  constexpr bool STORES_DS = F16 == 1 || F16 == 2 || (SPLIT && !MHA);
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
   if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
 
@@ -117,8 +119,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       tc::mbar_init(&misc->o_full[s], 2);                                     // two last-stage issuers
       tc::mbar_init(&misc->o_empty[s], 4);                                    // the epilogue warps
     }
-    bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4 + (F16 != 0 && a.ds != nullptr ? 1 : 0));
-    if (F16 != 0 && a.ds != nullptr) tc::mbar_init(&misc->ds_free[0], 2);     // read by the dK product and by the copy
+    bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4 + (STORES_DS && !SPLIT && a.ds != nullptr ? 1 : 0));
+    if (STORES_DS && !SPLIT && a.ds != nullptr) tc::mbar_init(&misc->ds_free[0], 2);     // read by the dK product and by the copy
     for (int s = 0; s < kRingB; ++s) tc::mbar_init(&misc->b_empty[s], 2);     // a dO slot is read by dP and by dV^T
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
@@ -228,7 +230,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             VSA2_WAIT_PARKED(&misc->dp_free[sb], pb ^ 1);
             tc::tc_fence_after();
             if (tc::elect_one()) {
-              mma_pair_kmajor<D, F16 == 2>(tmem_base + 128 + sb * 64, base + C::OFF_RING_B + sb * C::SLOT, b_addr);
+              mma_pair_kmajor<D, F16 >= 2>(tmem_base + 128 + sb * 64, base + C::OFF_RING_B + sb * C::SLOT, b_addr);
               tc::mma_commit(&misc->dp_full[sb]);
               tc::mma_commit(&misc->b_empty[sb]);
               if (t == nt - 1) tc::mma_commit(&misc->st_empty);
@@ -245,7 +247,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
                                     a.k_hi, lane, &misc->abort_flag))
       goto done;
-    if (F16 != 0 && warp == 19 && a.ds != nullptr) {
+    if (STORES_DS && !SPLIT && warp == 19 && a.ds != nullptr) {
       // ---------------------------------------------------------------- copies the dS tiles to the scratch as they stand
       uint32_t tg = 0;
       for (uint32_t seq = 0;; ++seq) {
@@ -288,7 +290,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             tc::tc_fence_after();
             if (tc::elect_one()) {
               if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, C::PBYTES, t > 0);
-              else mma_pairT_mnmajor<D, F16 == 2>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, t > 0);
+              else mma_pairT_mnmajor<D, F16 >= 2>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, t > 0);
               tc::mma_commit(&misc->b_empty[sv]);
               tc::mma_commit(&misc->p_free);
               if (t == nt - 1) tc::mma_commit(&misc->o_full[set]);
@@ -324,7 +326,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       VSA2_DKV_ITEM_SETUP();
       (void)j;
       const int ds_exp = a.ds_exp != nullptr ? a.ds_exp[bhk] : 0;
-      const float lse_off = F16 == 2 ? 0.f : (float)ds_exp, dlt_scale = F16 == 2 ? pow2i(ds_exp) : 1.f;
+      const float lse_off = F16 >= 2 ? 0.f : (float)ds_exp, dlt_scale = F16 >= 2 ? pow2i(ds_exp) : 1.f;
       const int nt = (k + 1) >> 1;
       int bhq_n, i_n, pos_n = 0;
       dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n, &pos_n);
@@ -380,7 +382,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               sv[c] = __float_as_uint(p0);
               sv[c + 1] = __float_as_uint(p1);
               if constexpr (SPLIT) split_bf16x2(p0, p1, pp[c >> 1], pl[c >> 1]);
-              else if constexpr (F16 == 2) pp[c >> 1] = pack_f16x2_sat(p0, p1);
+              else if constexpr (F16 >= 2) pp[c >> 1] = pack_f16x2_sat(p0, p1);
               else pp[c >> 1] = pack_bf16x2(p0, p1);
             }
             VSA2_WAIT(&misc->p_free, (tg & 1) ^ 1);
@@ -411,6 +413,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               if constexpr (SPLIT) {
                 split_bf16x2(d0, d1, pd[c >> 1], pdl[c >> 1]);
                 if constexpr (STORES_DS) ph[c >> 1] = pack_f16x2(d0, d1);
+              } else if constexpr (F16 == 3) {
+                pd[c >> 1] = pack_f16x2_sat(d0, d1);
               } else if constexpr (F16 != 0) {
                 // (a dS beyond the range: the recomputing dQ pass, which runs first, has met the same value and raised the flag,
                 //  or the pass behind this one finds the infinity in the scratch)
@@ -605,9 +609,12 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
               group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr};
-    if (when == 1 && gqa16) {       // every product in fp16
+    if (when == 1 && gqa16 && ds) { // every product in fp16
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
       else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
+    } else if (when == 1 && gqa16) {
+      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 3, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
+      else VSA2_LAUNCH_DKV(64, false, false, 3, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
     } else if (when == 1) {         // S and the dK product in fp16 (one query head per KV head)
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, true, 1, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);
       else VSA2_LAUNCH_DKV(64, false, true, 1, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);

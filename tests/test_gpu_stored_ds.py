@@ -37,3 +37,33 @@ def test_gradients_do_not_depend_on_the_scratch(heads_q, heads_kv, dim, grid, to
     for other in got[1:]:
         for name, x, y in zip(("dq", "dk", "dv", "dgate"), got[0], other):
             assert torch.equal(x, y), name
+
+
+def test_a_score_gradient_at_the_fp16_limit_leaves_no_infinity_behind():
+    """GQA groups, every product on fp16 copies: dS = P (dP - delta) with P = 1 and delta = 0 (q, o and lse are zero) lies at 65519.99
+    with the bf16 tensors (fp16: 65504) and at 65520.01 with the copies, whose V elements of 1.0078 * 2^-25 have become 2^-24
+    (fp16: infinite).  Whichever pass meets which, dK (dS times q = 0) must come out as zero, not as 0 times infinity."""
+    heads_q, heads_kv, dim, grid = 4, 2, 64, (8, 8, 8)
+    p = vb.make_params(1, heads_q, heads_kv, dim, grid, select_mode=vb.PER_QUERY, topk=8, flags=vb.FLAG_NO_COARSE, out_dtype=vb.F32)
+    attn = vb.Vsa2Attention(p)
+    rows = grid[0] * grid[1] * grid[2]
+    q = torch.zeros(1, heads_q, rows, dim, device="cuda", dtype=torch.bfloat16)
+    k = torch.ones(1, heads_kv, rows, dim, device="cuda", dtype=torch.bfloat16)
+    v_row, do_row = torch.zeros(dim), torch.zeros(dim)
+    v_row[:32], do_row[:32] = 1.0078125 * 2.0 ** -25, 2.0 ** 14             # 0.0158 in bf16, 0.0313 as copies, summed first
+    v_row[32:46], do_row[32:46] = 1.0, 4096.0                                # 57344
+    v_row[46], do_row[46] = 1.9921875, 4096.0                                # 8160
+    v_row[47], do_row[47] = 1.0, 16.0
+    v_row[48], do_row[48] = 1.0, -3 * 2.0 ** -7                              # 65519.977 in all
+    v = v_row.expand(1, heads_kv, rows, dim).bfloat16().cuda().contiguous()
+    d_o = do_row.expand(1, heads_q, rows, dim).bfloat16().cuda().contiguous()
+    attn.route(q, k)
+    o = torch.zeros(1, heads_q, rows, dim, device="cuda")
+    lse = torch.zeros(1, heads_q, rows, device="cuda")
+    for size in (vb.vsa2_attn_bwd_preferred_workspace_bytes(p), attn.sizes.bwd_workspace_bytes):
+        attn.ws_bwd = torch.zeros(size, dtype=torch.uint8, device="cuda")
+        dq, dk, dv, _ = attn.backward(q, k, v, None, o, lse, d_o)
+        attn.check_status()
+        assert (dk == 0).all()
+        assert torch.isfinite(dq).all() and torch.isfinite(dv).all()
+        assert ((dq / (rows * 65520.0 / dim ** 0.5) - 1).abs() < 2.0 ** -10).all()
