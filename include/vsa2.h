@@ -249,9 +249,20 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
                   const void* d_o, void* dq, void* dk, void* dv, float* dgate,
                   void* workspace, size_t workspace_bytes, void* cuda_stream);
 
-/* Bytes of backward workspace with which vsa2_attn_bwd runs fastest (0 for invalid parameters): sizes.bwd_workspace_bytes is
- * the least it accepts; what a caller hands it beyond that holds the score gradients of the dK/dV pass, so that the dQ pass
- * need not recompute them (bounded: 7 GiB of them at most).  Both give the same results. */
+/* The same with a scratch region of its own beside the workspace (device, 256-byte aligned, any size, NULL = none), which holds
+ * the score gradients of the dK/dV pass so that the dQ pass need not recompute them.  Nothing in it is read after the call's
+ * kernels: one region may serve all calls that follow one another on a stream, whatever their parameters, while a workspace keeps
+ * the call's status word.  vsa2_attn_bwd is this call with what its workspace holds beyond sizes.bwd_workspace_bytes
+ * (rounded up to 256) as the scratch. */
+int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, const void* v, const float* gate,
+                          const vsa2_map* map, const void* o, const float* lse, const vsa2_saved* saved,
+                          const void* d_o, void* dq, void* dk, void* dv, float* dgate,
+                          void* workspace, size_t workspace_bytes, void* scratch, size_t scratch_bytes, void* cuda_stream);
+
+/* Bytes of scratch with which the backward runs fastest (bounded: 7 GiB of score gradients; 0 where none are kept, or for
+ * invalid parameters), and of a workspace that holds them too.  Less room is used as far as it goes, a KV group at a time; the
+ * results are the same. */
+size_t vsa2_attn_bwd_scratch_bytes(const vsa2_params* p);
 size_t vsa2_attn_bwd_preferred_workspace_bytes(const vsa2_params* p);
 
 /* Cube-major copy of a tensor (Sec. 2.2 "Permutation": (T, H, W) -> (N_t N_h N_w) x (B_t B_h B_w)), for callers whose

@@ -32,7 +32,8 @@ ERR_STATIC_SCRATCH = -8
 EXPORTS = ("vsa2_query_sizes", "vsa2_route", "vsa2_route_scores", "vsa2_attn_fwd", "vsa2_attn_bwd",
            "vsa2_device_status", "vsa2_strerror", "vsa2_profile_events", "vsa2_launch_count", "vsa2_selftest_umma", "vsa2_route_noalloc", "vsa2_last_cuda_error",
            "vsa2_gate_fwd", "vsa2_gate_bwd", "vsa2_gate_bwd_workspace_bytes",
-           "vsa2_attn_bwd_preferred_workspace_bytes", "vsa2_permute_cube_major",
+           "vsa2_attn_bwd_preferred_workspace_bytes", "vsa2_attn_bwd_scratch", "vsa2_attn_bwd_scratch_bytes",
+           "vsa2_permute_cube_major",
            "vsa2_selftest_timeout", "vsa2_debug_rescue_capacity", "vsa2_selftest_divmod")
 
 KERNELS = ("pool", "router_lse", "router_pool", "select", "coarse_fwd", "fine_fwd", "bwd_pre", "coarse_bwd",
@@ -94,8 +95,9 @@ def _lib():
         lib.vsa2_route_noalloc.argtypes = [C.POINTER(Params), vp, vp, vp, C.POINTER(Map), vp, vp]
         lib.vsa2_permute_cube_major.argtypes = [C.POINTER(Params), C.c_int32, C.c_int32, vp, vp, vp]
         lib.vsa2_gate_fwd.argtypes = [C.POINTER(Params), C.c_int32, vp, vp, vp, vp]
-        lib.vsa2_attn_bwd_preferred_workspace_bytes.argtypes = [C.POINTER(Params)]
-        lib.vsa2_attn_bwd_preferred_workspace_bytes.restype = C.c_size_t
+        for fn in (lib.vsa2_attn_bwd_preferred_workspace_bytes, lib.vsa2_attn_bwd_scratch_bytes):
+            fn.argtypes = [C.POINTER(Params)]
+            fn.restype = C.c_size_t
         lib.vsa2_gate_bwd_workspace_bytes.argtypes = [C.POINTER(Params), C.c_int32]
         lib.vsa2_gate_bwd_workspace_bytes.restype = C.c_size_t
         lib.vsa2_gate_bwd.argtypes = [C.POINTER(Params), C.c_int32, vp, vp, vp, vp, vp, vp, vp, sz, vp]
@@ -104,6 +106,7 @@ def _lib():
         lib.vsa2_attn_fwd.argtypes = [C.POINTER(Params), vp, vp, vp, vp, C.POINTER(Map), vp, vp, C.POINTER(Saved), vp, sz, vp]
         lib.vsa2_attn_bwd.argtypes = [C.POINTER(Params), vp, vp, vp, vp, C.POINTER(Map), vp, vp, C.POINTER(Saved), vp,
                                       vp, vp, vp, vp, vp, sz, vp]
+        lib.vsa2_attn_bwd_scratch.argtypes = lib.vsa2_attn_bwd.argtypes[:-1] + [vp, sz, vp]
         lib.vsa2_device_status.argtypes = [vp, vp, i32p]
         lib.vsa2_last_cuda_error.argtypes = []
         lib.vsa2_last_cuda_error.restype = C.c_char_p
@@ -119,7 +122,8 @@ def _lib():
         lib.vsa2_selftest_divmod.restype = C.c_int64
         for name in EXPORTS:
             if name not in ("vsa2_strerror", "vsa2_route_scores", "vsa2_launch_count", "vsa2_last_cuda_error", "vsa2_selftest_divmod",
-                            "vsa2_gate_bwd_workspace_bytes", "vsa2_attn_bwd_preferred_workspace_bytes"):
+                            "vsa2_gate_bwd_workspace_bytes", "vsa2_attn_bwd_preferred_workspace_bytes",
+                            "vsa2_attn_bwd_scratch_bytes"):
                 getattr(lib, name).restype = C.c_int
         _LIB = lib
     return _LIB
@@ -223,11 +227,21 @@ def vsa2_attn_fwd(p, q, k, v, gate, vmap: Map, o, lse, saved, workspace, workspa
 
 
 def vsa2_attn_bwd(p, q, k, v, gate, vmap: Map, o, lse, saved, d_o, dq, dk, dv, dgate, workspace,
-                  workspace_bytes=None, stream=None):
+                  workspace_bytes=None, stream=None, scratch=None):
+    """`scratch`: None (what `workspace` holds beyond the least serves as scratch) or a tensor of its own."""
     nbytes = workspace_bytes if workspace_bytes is not None else workspace.numel() * workspace.element_size()
-    _check(_lib().vsa2_attn_bwd(C.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), C.byref(vmap), _ptr(o), _ptr(lse),
-                                C.byref(saved) if saved is not None else None, _ptr(d_o), _ptr(dq), _ptr(dk),
-                                _ptr(dv), _ptr(dgate), _ptr(workspace), nbytes, _stream(stream)), "vsa2_attn_bwd")
+    args = (C.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(gate), C.byref(vmap), _ptr(o), _ptr(lse),
+            C.byref(saved) if saved is not None else None, _ptr(d_o), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dgate), _ptr(workspace), nbytes)
+    if scratch is None:
+        _check(_lib().vsa2_attn_bwd(*args, _stream(stream)), "vsa2_attn_bwd")
+    else:
+        _check(_lib().vsa2_attn_bwd_scratch(*args, _ptr(scratch), scratch.numel() * scratch.element_size(), _stream(stream)),
+               "vsa2_attn_bwd_scratch")
+
+
+def vsa2_attn_bwd_scratch_bytes(p) -> int:
+    """Bytes of scratch with which the backward runs fastest (0: it has no use for any)."""
+    return int(_lib().vsa2_attn_bwd_scratch_bytes(C.byref(p)))
 
 
 def vsa2_attn_bwd_preferred_workspace_bytes(p) -> int:
@@ -289,10 +303,10 @@ class Vsa2Attention:
         u8 = dict(dtype=torch.uint8, device=dev)
         self.ws_route = torch.empty(s.route_workspace_bytes, **u8)
         self.ws_fwd = torch.empty(s.fwd_workspace_bytes, **u8)
-        try:
-            self.ws_bwd = torch.empty(vsa2_attn_bwd_preferred_workspace_bytes(params), **u8)
-        except torch.cuda.OutOfMemoryError:     # the least the backward accepts: it recomputes what the rest would hold
-            self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
+        self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
+        # scratch of a backward call, up to 7 GiB: taken from torch's allocator for the call and given back, so the handles of a
+        # model share it and one that only runs forward has none; 0 = none (the dQ pass recomputes the score gradients)
+        self.bwd_scratch_bytes = vsa2_attn_bwd_scratch_bytes(params)
         for ws in (self.ws_route, self.ws_fwd, self.ws_bwd):
             ws[:256].zero_()          # status block
         self.out_torch_dtype = torch.float32 if params.out_dtype == F32 else torch.bfloat16
@@ -336,8 +350,25 @@ class Vsa2Attention:
             dv = torch.empty(v.shape, dtype=self.out_torch_dtype, device=q.device)
         if dgate is None:      # video tokens only (text tokens have no gate)
             dgate = torch.empty(q.shape[:-2] + (self.sizes.seq_len,), dtype=torch.float32, device=q.device)
-        vsa2_attn_bwd(p, q, k, v, gate, self.map, o, lse, self.saved, d_o, dq, dk, dv, dgate, self.ws_bwd, stream=stream)
+        vsa2_attn_bwd(p, q, k, v, gate, self.map, o, lse, self.saved, d_o, dq, dk, dv, dgate, self.ws_bwd, stream=stream,
+                      scratch=self._bwd_scratch(q.device, stream))
         return dq, dk, dv, dgate
+
+    def _bwd_scratch(self, device, stream):
+        """Scratch for one call, allocated on the stream the call runs on (its memory is then reused in that stream's order)."""
+        torch, n = self.torch, self.bwd_scratch_bytes
+        if n == 0:
+            return None
+        try:
+            if stream is None:
+                return torch.empty(n, dtype=torch.uint8, device=device)
+            if isinstance(stream, int):
+                stream = torch.cuda.ExternalStream(stream, device) if stream else torch.cuda.default_stream(device)
+            with torch.cuda.stream(stream):
+                return torch.empty(n, dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:     # not asked for again: a failing request makes the allocator empty its cache
+            self.bwd_scratch_bytes = 0
+            return None
 
     def check_status(self, stream=None):
         for name, ws in (("route", self.ws_route), ("fwd", self.ws_fwd), ("bwd", self.ws_bwd)):

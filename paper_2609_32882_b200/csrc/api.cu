@@ -234,8 +234,8 @@ size_t bwd_workspace_bytes(const Geo& g) {
   return n;
 }
 
-// dS tiles that the dK/dV pass leaves for the dQ pass (fine_bwd_dq_ds_tc.cu), in what a caller's workspace holds beyond
-// bwd_workspace_bytes: 8 KB per kept pair of 64-token blocks, for as many KV groups at a time as fit.  Without room for one group
+// dS tiles that the dK/dV pass leaves for the dQ pass (fine_bwd_dq_ds_tc.cu), in a scratch region of the caller's (offsets are
+// relative to it): 8 KB per kept pair of 64-token blocks, for as many KV groups at a time as fit.  Without room for one group
 // the dQ pass recomputes dS.  The preferred size stops at kStoredDsBytes of tiles (9 heads of 720p top-64, one group of the
 // 16..256-cube budget with four heads a group): a launch over fewer blocks loses more on its last, unevenly filled items
 // (one head of 720p at a time: 10 blocks per SM), more scratch gains nothing.
@@ -244,19 +244,18 @@ struct DsLayout {
   size_t counters, pos, order, tiles, total;
   int groups;          // KV groups per chunk, 0: no stored dS
 };
-DsLayout ds_layout(const Geo& g, size_t avail_total, bool preferred) {
+DsLayout ds_layout(const Geo& g, size_t avail, bool preferred) {
   DsLayout r{};
   if (!dq_pass_f16(g) || wide_cube(g)) return r;
   const Geo x = g.Lt > 0 ? text_geo(g) : g;
   const size_t all = (size_t)g.batch * g.Hkv, group = (size_t)x.rep * x.nnz_cap * kBlockTokens * kBlockTokens * sizeof(bf16);
   if (group == 0) return r;
   Carver c;
-  c.off = align_up(bwd_workspace_bytes(g), 256);
   r.counters = c.take(2 * all * sizeof(int));
   r.pos = c.take((size_t)g.batch * g.Hq * x.nnz_cap * sizeof(int));
   r.order = c.take(all * x.N * sizeof(int));
   r.tiles = c.off;
-  const size_t room = preferred ? kStoredDsBytes : avail_total > r.tiles ? avail_total - r.tiles : 0;
+  const size_t room = preferred ? kStoredDsBytes : avail > r.tiles ? avail - r.tiles : 0;
   const size_t fit = room / group < all ? room / group : all;
   // (row index of a tile in the tensor map: 32 bits)
   if (fit == 0 || fit * group / 128 > 0x7fffffffULL) return r;
@@ -385,12 +384,16 @@ int vsa2_query_sizes(const vsa2_params* p, vsa2_sizes* out) {
   return VSA2_OK;
 }
 
+size_t vsa2_attn_bwd_scratch_bytes(const vsa2_params* p) {
+  Geo g;
+  return fill_geo(p, &g) == VSA2_OK ? ds_layout(g, 0, true).total : 0;
+}
+
 size_t vsa2_attn_bwd_preferred_workspace_bytes(const vsa2_params* p) {
   Geo g;
   if (fill_geo(p, &g) != VSA2_OK) return 0;
-  const size_t least = bwd_workspace_bytes(g);
-  const DsLayout dl = ds_layout(g, 0, true);
-  return dl.groups > 0 ? dl.total : least;
+  const size_t least = bwd_workspace_bytes(g), scratch = ds_layout(g, 0, true).total;
+  return scratch > 0 ? align_up(least, 256) + scratch : least;
 }
 
 int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets, const vsa2_map* map,
@@ -577,6 +580,20 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   Geo g;
   int rc = fill_geo(p, &g);
   if (rc != VSA2_OK) return rc;
+  // (what the workspace holds beyond the least serves as the scratch; the checks of the call come first)
+  const size_t least = align_up(bwd_workspace_bytes(g), 256);
+  const bool more = workspace != nullptr && workspace_bytes > least;
+  return vsa2_attn_bwd_scratch(p, q, k, v, gate, map, o, lse, saved, d_o, dq, dk, dv, dgate, workspace, workspace_bytes,
+                               more ? at<unsigned char>(workspace, least) : nullptr, more ? workspace_bytes - least : 0, cuda_stream);
+}
+
+int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, const void* v, const float* gate,
+                          const vsa2_map* map, const void* o, const float* lse, const vsa2_saved* saved, const void* d_o,
+                          void* dq, void* dk, void* dv, float* dgate, void* workspace, size_t workspace_bytes, void* scratch,
+                          size_t scratch_bytes, void* cuda_stream) {
+  Geo g;
+  int rc = fill_geo(p, &g);
+  if (rc != VSA2_OK) return rc;
   if (!q || !k || !v || !map || !o || !lse || !d_o || !dq || !dk || !dv || !workspace || !map->row_ptr ||
       !map->col_idx || !map->col_ptr || !map->row_idx)
     return VSA2_ERR_INVALID_ARG;
@@ -584,7 +601,7 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
   if (coarse && (!saved || !saved->qc || !saved->kc || !saved->vc || !saved->oc_hat || !saved->lse_c))
     return VSA2_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(d_o) || !aligned16(dq) ||
-      !aligned16(dk) || !aligned16(dv) || !aligned256(workspace))
+      !aligned16(dk) || !aligned16(dv) || !aligned256(workspace) || !aligned256(scratch))
     return VSA2_ERR_MISALIGNED;
   if (workspace_bytes < bwd_workspace_bytes(g)) return VSA2_ERR_WORKSPACE_TOO_SMALL;
   if ((rc = check_device()) != VSA2_OK) return rc;
@@ -670,11 +687,11 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
     }
   }
   // dS kept from the dK/dV pass for the dQ pass, which then runs inside it; otherwise the dQ pass recomputes dS and runs first
-  const DsLayout dl = ds_layout(g, workspace_bytes, false);
+  const DsLayout dl = ds_layout(g, scratch != nullptr ? scratch_bytes : 0, false);
   const int ds_groups = dl.groups;
   // (a few items per SM end together whatever their order)
-  int* dkv_order = ds_groups > 0 && (long long)ds_groups * fx.N > 4 * 148 ? at<int>(workspace, dl.order) : nullptr;
-  const StoredDs sd{at<unsigned char>(workspace, dl.tiles), at<int>(workspace, dl.pos), at<int>(workspace, dl.counters), dkv_order, ds_groups,
+  int* dkv_order = ds_groups > 0 && (long long)ds_groups * fx.N > 4 * 148 ? at<int>(scratch, dl.order) : nullptr;
+  const StoredDs sd{at<unsigned char>(scratch, dl.tiles), at<int>(scratch, dl.pos), at<int>(scratch, dl.counters), dkv_order, ds_groups,
                     row_ptr, col_idx, coarse ? dqc : nullptr, dq};
   // cubes of 128 tokens: both passes on 128 x 128 tiles
   const bool wide128 = wide && g.Lt == 0 && fine_bwd128_supported(n);
@@ -685,7 +702,7 @@ int vsa2_attn_bwd(const vsa2_params* p, const void* q, const void* k, const void
       VSA2_CUDA(launch_cast_qk(fx, qb, at<unsigned char>(workspace, bwd_f16_offset(g)), kb,
                                at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale,
                                &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
-      VSA2_CUDA(launch_ds_positions(fx, row_ptr, col_idx, col_ptr, row_idx, at<int>(workspace, dl.pos), sd.counters,
+      VSA2_CUDA(launch_ds_positions(fx, row_ptr, col_idx, col_ptr, row_idx, at<int>(scratch, dl.pos), sd.counters,
                                     2 * g.batch * g.Hkv, st));
       if (dkv_order != nullptr) {
         g_launches += 1;

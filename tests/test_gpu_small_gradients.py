@@ -3,7 +3,6 @@ passes round dS to fp16, whose subnormals end at 2^-24; dQ, dK and dV scale with
 stated bounds scaled by the same factors -- with the score gradients kept between the passes and with them formed twice."""
 import numpy as np
 import pytest
-import torch
 
 from oracle import vsa2_oracle as orc
 from paper_2609_32882_b200 import binding as vb
@@ -34,7 +33,7 @@ def test_small_gradients_keep_their_bits(wl, tensor, factor, least):
         data["do"] = syn.f32_to_bf16_bits(d)
     run = CudaPath(wl, data, out_dtype=vb.F32, flags=vb.FLAG_NO_COARSE)
     if least:
-        run.attn.ws_bwd = torch.zeros(run.attn.sizes.bwd_workspace_bytes, dtype=torch.uint8, device="cuda")
+        run.attn.bwd_scratch_bytes = 0
     run.route()
     run.forward()
     run.backward()

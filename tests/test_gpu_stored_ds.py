@@ -1,6 +1,6 @@
-"""Backward with room for the stored score-gradient tiles of all KV heads, of all but one, and of none: the three routes form
-dQ from the same fp16 tiles and cubes in the same order, so the gradients must be the same bit for bit (the route without
-room is the one that the parity tests compare with the oracle)."""
+"""Backward with room for the stored score-gradient tiles of all KV groups, of some, and of none: the routes form
+dQ from the same fp16 tiles and cubes in the same order, so the gradients must be the same bit for bit (the parity tests compare
+the first with the oracle, through the scratch that a handle takes for the call)."""
 import pytest
 import torch
 
@@ -29,7 +29,10 @@ def test_gradients_do_not_depend_on_the_scratch(heads_q, heads_kv, dim, grid, to
     o, lse = attn.forward(q, k, v, gate)
     most, least = vb.vsa2_attn_bwd_preferred_workspace_bytes(p), attn.sizes.bwd_workspace_bytes
     assert most > least
-    got = []
+    assert most - least - vb.vsa2_attn_bwd_scratch_bytes(p) in range(256)
+    got = [attn.backward(q, k, v, gate, o, lse, d_o)]
+    attn.check_status()
+    attn.bwd_scratch_bytes = 0
     for size in (most, most - 256, least):
         attn.ws_bwd = torch.empty(size, dtype=torch.uint8, device="cuda")
         got.append(attn.backward(q, k, v, gate, o, lse, d_o))
@@ -61,7 +64,7 @@ def test_a_score_gradient_at_the_fp16_limit_leaves_no_infinity_behind():
     o = torch.zeros(1, heads_q, rows, dim, device="cuda")
     lse = torch.zeros(1, heads_q, rows, device="cuda")
     for size in (vb.vsa2_attn_bwd_preferred_workspace_bytes(p), attn.sizes.bwd_workspace_bytes):
-        attn.ws_bwd = torch.zeros(size, dtype=torch.uint8, device="cuda")
+        attn.ws_bwd, attn.bwd_scratch_bytes = torch.zeros(size, dtype=torch.uint8, device="cuda"), 0
         dq, dk, dv, _ = attn.backward(q, k, v, None, o, lse, d_o)
         attn.check_status()
         assert (dk == 0).all()

@@ -73,6 +73,23 @@ def test_backward_workspace_holds_the_fp16_copies_of_the_default_forms():
     assert bwd_bytes(wl, topk=4) == up(plain) + q16 + k16  # rows that keep few blocks: the dK/dV pass stays with its pairs
 
 
+def test_backward_scratch_is_checked_and_bounded():
+    lib = vb._lib()
+    p = vb.params_from_workload(syn.CONFIGS[3])                       # 720p, 40 heads, top-64
+    s = vb.vsa2_query_sizes(p)
+    extra = vb.vsa2_attn_bwd_scratch_bytes(p)
+    assert 5 << 30 < extra < 8 << 30                                  # 7 GiB of tiles at most, whole KV groups
+    assert vb.vsa2_attn_bwd_preferred_workspace_bytes(p) == (s.bwd_workspace_bytes + 255) // 256 * 256 + extra
+    precise = vb.params_from_workload(syn.CONFIGS[3], flags=vb.FLAG_PRECISE_BWD)
+    assert vb.vsa2_attn_bwd_scratch_bytes(precise) == 0
+    assert vb.vsa2_attn_bwd_preferred_workspace_bytes(precise) == vb.vsa2_query_sizes(precise).bwd_workspace_bytes
+    one, m = ctypes.c_void_p(256), vb.Map(256, 256, 256, 256)
+    saved = vb.Saved(256, 256, 256, 256, 256, 256)
+    args = [ctypes.byref(p)] + [one] * 4 + [ctypes.byref(m), one, one, ctypes.byref(saved)] + [one] * 6
+    assert lib.vsa2_attn_bwd_scratch(*args, s.bwd_workspace_bytes, ctypes.c_void_p(128), 1 << 30, None) == vb.ERR_MISALIGNED
+    assert lib.vsa2_attn_bwd_scratch(*args, s.bwd_workspace_bytes - 1, one, 1 << 30, None) == vb.ERR_WORKSPACE_TOO_SMALL
+
+
 def test_topk_is_clamped_and_keep_fraction_is_honoured():
     wl = syn.CONFIGS[1]
     assert vb.vsa2_query_sizes(vb.params_from_workload(wl, topk=1000)).topk_eff == 32
