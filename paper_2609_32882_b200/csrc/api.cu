@@ -1,4 +1,5 @@
 // C ABI of the VSA2 library: argument checks, workspace layout, kernel sequencing.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -312,21 +313,38 @@ cudaError_t sm_count(int* sms) {
   return cudaSuccess;
 }
 
+// the driver's number of the current context, never given twice in a process; 0 if there is none yet (or it cannot be had)
+static unsigned long long context_id() {
+  typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+  static const GetId get_id = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<GetId>(p) : nullptr;
+  }();
+  unsigned long long id = 0;
+  return get_id != nullptr && get_id(nullptr, &id) == CUDA_SUCCESS && id < 1ull << 44 ? id : 0;
+}
+
 cudaError_t prepare_kernel(const void* kernel, KernelAttr& attr, size_t smem, int threads, int least_registers) {
   int dev = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  const bool known = dev < kMaxDevices;
-  if (known && attr.smem[dev].load(std::memory_order_acquire) >= (int)smem) return cudaSuccess;
+  const unsigned long long ctx = dev < kMaxDevices ? context_id() : 0;      // 0: not known, ask the driver every time
+  auto allowed = [&] {
+    const unsigned long long k = attr.known[dev].load(std::memory_order_acquire);
+    return ctx != 0 && k >> 20 == ctx && (k & 0xfffffu) >= smem;
+  };
+  if (ctx != 0 && allowed()) return cudaSuccess;
   std::lock_guard<std::mutex> lock(attr.lock);        // (the limit only grows: two threads must not lower it for each other)
-  if (known && attr.smem[dev].load(std::memory_order_relaxed) >= (int)smem) return cudaSuccess;
+  if (ctx != 0 && allowed()) return cudaSuccess;
   if (least_registers > 0) {
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
     if (fa.numRegs * threads < least_registers) return cudaErrorLaunchOutOfResources;
   }
   if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if (known) attr.smem[dev].store((int)smem, std::memory_order_release);
+  if (ctx != 0) attr.known[dev].store(ctx << 20 | smem, std::memory_order_release);
   return cudaSuccess;
 }
 

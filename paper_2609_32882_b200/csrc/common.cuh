@@ -61,12 +61,14 @@ struct ProfScope {
   ~ProfScope();
 };
 
-// Per kernel and device: the dynamic shared memory it has been allowed so far.  A launch asks the driver only when it needs more
-// (each such call costs the host as much as half a launch, and the kernels' needs are constants or grow with the problem).
+// Per kernel and device: the dynamic shared memory it has been allowed so far, and the CUDA context in which that was (the limit is a
+// context's: another context of the device, or the primary one after a device reset, starts without it).  A launch asks the
+// driver only when it needs more or the context is another (each such call costs the host as much as half a launch, and the
+// kernels' needs are constants or grow with the problem).
 constexpr int kMaxDevices = 64;
 struct KernelAttr {
   std::mutex lock;
-  std::atomic<int> smem[kMaxDevices] = {};
+  std::atomic<unsigned long long> known[kMaxDevices] = {};      // context id << 20 | bytes
 };
 // `least_registers`: registers the launch has to allocate over all its threads (kernels that redistribute them wait for ever
 // otherwise), checked with `threads` on the first call
