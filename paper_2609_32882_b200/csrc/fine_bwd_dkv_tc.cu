@@ -32,6 +32,7 @@ struct DkvArgs {
   int ds_head0;
   const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale; forms whose dS is rounded to fp16)
   const int* order;     // null, or the order in which the items are drawn
+  int overlap;          // 1: the launch behind this one may start while this one runs; 2: this one may be running beside the one before it
 };
 
 constexpr int kMaxRep = 16;   // query heads per KV head the dK/dV pass supports
@@ -112,6 +113,9 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   constexpr bool STORES_DS = F16 == 1 || F16 == 2 || (SPLIT && !MHA);
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
   if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
+  // the launch of the few long lists lets the launch of the others (disjoint outputs, nothing read from this one) take the SMs as its
+  // CTAs leave them
+  if (SPLIT && a.overlap == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (tid == 0) {
     bwd_init_barriers(misc);
@@ -245,7 +249,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   } else if (warp >= 16 && warp < 20) {
     tc::reg_dec<48>();
     if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
-                                    a.k_hi, lane, &misc->abort_flag))
+                                    a.k_hi, SPLIT && MHA && a.k_lo > 1, nullptr, lane, &misc->abort_flag))
       goto done;
     if (STORES_DS && !SPLIT && warp == 19 && a.ds != nullptr) {
       // ---------------------------------------------------------------- copies the dS tiles to the scratch as they stand
@@ -542,6 +546,7 @@ done:
     __syncthreads();
   }
   if (warp == 2) tc::tmem_dealloc(tmem_base, 512);
+  if (!SPLIT && F16 == 0 && a.overlap == 2) asm volatile("griddepcontrol.wait;" ::: "memory");     // (what follows waits for both)
 }
 
 // ================================================================================================
@@ -556,7 +561,8 @@ constexpr int kDkvLongColumn = 256;
 // the list length (720p sample, fp32 outputs: 6.5e-3 at |dK| = 5.5 with 200 query blocks, 6.3e-3 at 3.0 with 260); the
 // few blocks that nearly every query keeps reach |dK| = 15 and then 1.5e-2 .. 2.7e-2 depending on nothing but where the
 // roundings fall (e.g. whether the softmax scale is applied before or after dS is rounded), i.e. across the stated 2e-2.
-// As pairs they come out at 6e-3.  Each launch walks all items and skips the other's.
+// As pairs they come out at 6e-3.  The pair launch comes first (a handful of 0.3 ms items on 148 CTAs: alone it would end with most
+// SMs idle) and the plain launch fills the SMs as its CTAs leave them; each skips the other's items.
 cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
@@ -599,16 +605,22 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   } while (0)
   // `when`: see DkvArgs.
   // `group0`, `groups`: range of KV heads (batch * Hkv index); `ds`: the launch stores dS, counting on a counter of its own.
+  // `overlap`: see DkvArgs.
   auto launch = [&](bool split, int* counter, int k_lo, int k_hi, int when, int group0, int groups,
-                    bool ds) -> cudaError_t {
+                    bool ds, int overlap = 0) -> cudaError_t {
     cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap == 2 ? 1 : 0;
     const int items = groups * g.N;
     cfg.gridDim = dim3(items < sms ? items : sms);
     cfg.blockDim = dim3(kDkvThreads);
     cfg.stream = st;
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
-              group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr};
+              group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr, overlap};
     if (when == 1 && gqa16 && ds) { // every product in fp16
       if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
       else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
@@ -666,8 +678,8 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     when = 2;
     slot_plain = 5;
   }
-  if ((e = launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, when, 0, all, false)) != cudaSuccess) return e;
-  return launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, when, 0, all, false);
+  if ((e = launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, when, 0, all, false, 1)) != cudaSuccess) return e;
+  return launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, when, 0, all, false, 2);
 }
 
 // Whether the dK/dV pass of a GQA problem takes its all-fp16 form when it is given the scratch for the four copies.  Rows that

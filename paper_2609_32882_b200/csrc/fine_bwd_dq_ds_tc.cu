@@ -185,8 +185,9 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         uint32_t x[32];
         tc::tmem_ld32(lane_addr + set * 64 + part * 32, x);
         tc::tmem_ld_wait();
-        // a dS that left the fp16 range is an infinity and has made every channel of its query column non-finite
-        if (row < D && any_non_finite32(x)) atomicExch(a.range_flag, 1);
+        // a dS that left the fp16 range is an infinity and has made every channel of its query column non-finite (one store per
+        // warp: with all rows out of range one per thread took 2.7 ms for 8 heads of 720p)
+        if (__any_sync(0xffffffffu, row < D && any_non_finite32(x)) && lane == 0) *a.range_flag = 1;
         float v[32];
 #pragma unroll
         for (int c = 0; c < 32; ++c) v[c] = fmaf(__uint_as_float(x[c]), out_scale, coarse_d);
@@ -197,7 +198,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       if (lane == 0) tc::mbar_arrive(&misc->o_empty[set]);
     }
   } else {
-    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, lane,
+    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, false, a.range_flag, lane,
                       &misc->abort_flag))
       goto done;
   }

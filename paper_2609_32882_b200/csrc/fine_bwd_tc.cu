@@ -43,12 +43,16 @@ struct DqArgs {
   const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale)
 };
 
-// DsScale::exp of the groups blockIdx.x, blockIdx.x + gridDim.x, ... (the whole block calls it); true if one is below least_o
-__device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int per_group) {
+// An exponent of max|dO| max|O| from which on a dS is taken to leave the fp16 range: a weight of 2^-8 in the row of the largest dO is
+// enough.  The flag then goes up before the fp16 passes have run for nothing (720p, 8 heads, dO of 3e6: 14.6 -> 7 ms).
+constexpr int kBeyondF16 = 22;
+// DsScale::exp of the groups blockIdx.x, blockIdx.x + step, ... (the whole block calls it); true if the fp16 forms are not to run:
+// O below least_o, or dS beyond the fp16 range
+__device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int per_group, int step) {
   __shared__ unsigned red[2][8];
-  bool small = false;
+  bool bad = false;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+  for (int grp = blockIdx.x; grp < groups; grp += step) {
     const uint2* m = reinterpret_cast<const uint2*>(s.absmax) + (size_t)grp * per_group;      // (bit patterns order like the numbers)
     unsigned d = 0u, o = 0u;
     for (int i = threadIdx.x; i < per_group; i += 256) {
@@ -70,25 +74,29 @@ __device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int pe
       }
       const int e = (int)(d >> 23) - 127 + (int)(o >> 23) - 127;
       s.exp[grp] = d == 0u || o == 0u ? 0 : max(0, min(-3 - e, 100));
-      small |= o != 0u && __uint_as_float(o) < s.least_o;
+      bad |= o != 0u && (__uint_as_float(o) < s.least_o || (d != 0u && e >= kBeyondF16));
     }
     __syncthreads();
   }
-  return small;
+  return bad;
 }
 
 // Copies of two bf16 tensors in fp16 (8 elements per thread and step), b times 2^b_exp[its group of `b_group` steps] if there is one.
 // A finite bf16 below 65520 in magnitude has an exact fp16 image if it is a multiple of 2^-24 (all of 2^-17 and more are: fp16
 // keeps more mantissa bits), and one within 2^-25 otherwise; a finite value beyond that range sets `range_flag` and the caller's
-// fp16 kernels stand back.  With scale.absmax the launch also forms the exponents of dS.
+// fp16 kernels stand back.  The first `reducers` blocks form the exponents of dS meanwhile.
 __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __restrict__ xa, uint4* __restrict__ ya, size_t na,
                                                                const uint4* __restrict__ xb, uint4* __restrict__ yb, size_t nb,
                                                                const int* __restrict__ b_exp, unsigned b_group, int* range_flag,
-                                                               DsScale scale, int groups, int per_group) {
-  const size_t stride = (size_t)gridDim.x * blockDim.x, n = na + nb;
-  bool bad = scale.absmax != nullptr && form_ds_exp(scale, groups, per_group);
+                                                               DsScale scale, int groups, int per_group, int reducers) {
+  const size_t stride = (size_t)(gridDim.x - reducers) * blockDim.x, n = na + nb;
+  bool bad = false;
+  if ((int)blockIdx.x < reducers) {
+    if (form_ds_exp(scale, groups, per_group, reducers)) atomicExch(range_flag, 1);
+    return;
+  }
   constexpr int U = 4;      // 16-byte loads in flight per thread (a pure streaming kernel)
-  for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += U * stride) {
+  for (size_t i0 = (size_t)(blockIdx.x - reducers) * blockDim.x + threadIdx.x; i0 < n; i0 += U * stride) {
     uint4 v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -564,9 +572,10 @@ static cudaError_t launch_cast(const bf16* a, void* a16, size_t na, const bf16* 
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   // (element counts are multiples of the head dimension)
-  cast_bf16_to_f16_kernel<<<sms * 16, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
+  const int reducers = groups < sms ? groups : sms;
+  cast_bf16_to_f16_kernel<<<sms * 16 + reducers, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
                                                      reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8, b_exp,
-                                                     (unsigned)(b_group / 8), range_flag, scale, groups, per_group);
+                                                     (unsigned)(b_group / 8), range_flag, scale, groups, per_group, reducers);
   return cudaGetLastError();
 }
 

@@ -62,13 +62,17 @@ __device__ __forceinline__ bool bwd_queue_get(BwdQueue* q, uint32_t seq, int lan
   if (!bwd_queue_get(&misc->queue, (SEQ), lane, REC, &misc->abort_flag)) goto done;      \
   if (REC.x < 0) break
 // scheduler warp: draws the items first_item .. first_item + items - 1 (in the order of `order`, if there is one) until the
-// counter runs out.  `ptr`,
-// `rep`: start pointers of the lists, an item has those of `rep` consecutive heads; items with fewer than k_lo or more than k_hi
-// entries are left out.
+// counter runs out or `stop` (null, or a flag in global memory, looked at every fourth draw) is up.  `ptr`, `rep`: start pointers of the lists, an item has those of
+// `rep` consecutive heads; items with fewer than k_lo or more than k_hi entries are left out.
+// `sparse`: few items are in that range.  A draw then stands for 32 of them, one per lane and far apart (their lists tend to be long
+// side by side), so that passing over the others costs a 32nd of the draws.
 __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int first_item, int items, int rep, const int* ptr,
-                                             int* counter, const int* order, int k_lo, int k_hi, int lane,
+                                             int* counter, const int* order, int k_lo, int k_hi, bool sparse, const int* stop, int lane,
                                              volatile int* abort_flag) {
+  const int draws = sparse ? (items + 31) / 32 : items;
   uint32_t drawn = 0;
+  unsigned left = 0u;             // sparse: lanes of the current draw whose items are still to be handed out
+  int4 mine;
   for (uint32_t p = 0;; ++p) {
     const uint32_t slot = p % kItemSlots;
     if (p > 0 && !tc::mbar_wait_parked(&q->taken, (p - 1) & 1, abort_flag)) return false;
@@ -76,11 +80,38 @@ __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int firs
     int4 rec;
     for (;;) {
       rec = make_int4(-1, 0, 0, 0);
+      if (left != 0u) {
+        const int src = __ffs(left) - 1;
+        left &= left - 1u;
+        rec.x = __shfl_sync(0xffffffffu, mine.x, src);
+        rec.y = __shfl_sync(0xffffffffu, mine.y, src);
+        rec.z = __shfl_sync(0xffffffffu, mine.z, src);
+        rec.w = __shfl_sync(0xffffffffu, mine.w, src);
+        break;
+      }
       int n = 0;
-      if (lane == 0) n = item_draw(drawn, counter);
+      if (lane == 0) {
+        n = item_draw(drawn, counter);
+        if ((drawn & 3u) == 1u && stop != nullptr && *reinterpret_cast<const volatile int*>(stop) != 0) n = draws;
+      }
       n = __shfl_sync(0xffffffffu, n, 0);
       ++drawn;
-      if (n >= items) break;
+      if (n >= draws) break;
+      if (sparse) {
+        const int item = n + lane * draws;
+        mine = make_int4(-1, 0, 0, 0);
+        if (item < items) {
+          item_block(g, first_item + item, mine.y, mine.x);
+          for (int hh = 0; hh < rep; ++hh) {
+            const int* c = ptr + ((size_t)mine.y * rep + hh) * (g.N + 1) + mine.x;
+            const int beg = c[0];
+            if (hh == 0) mine.w = beg;
+            mine.z += c[1] - beg;
+          }
+        }
+        left = __ballot_sync(0xffffffffu, item < items && mine.z >= k_lo && mine.z <= k_hi);
+        continue;
+      }
       item_block(g, order != nullptr ? order[first_item + n] : first_item + n, rec.y, rec.x);
       int beg = 0, k = 0;
       if (lane < rep) {      // (heads of a group are neighbours: b * Hq + hk * rep + hh)

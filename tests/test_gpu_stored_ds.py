@@ -70,3 +70,59 @@ def test_a_score_gradient_at_the_fp16_limit_leaves_no_infinity_behind():
         assert (dk == 0).all()
         assert torch.isfinite(dq).all() and torch.isfinite(dv).all()
         assert ((dq / (rows * 65520.0 / dim ** 0.5) - 1).abs() < 2.0 ** -10).all()
+
+
+@pytest.mark.parametrize("route", ["one_chunk", "group_by_group", "recomputed"])
+@pytest.mark.parametrize("where", ["everywhere", "last_head"])
+@pytest.mark.parametrize("batch,heads_q,heads_kv,dim,grid,topk,mode,factor", [
+    (2, 3, 3, 128, (5, 9, 13), 5, vb.PER_SEQUENCE, 2.5e5),
+    (2, 4, 2, 64, (8, 12, 12), 9, vb.PER_QUERY, 4e5),        # grouped heads: the fallback of dK/dV carries pairs for every list
+    (2, 4, 2, 64, (8, 12, 12), 9, vb.PER_QUERY, 1e8),        # so large that the flag is up before the first pass
+    (1, 2, 2, 64, (20, 32, 32), 256, vb.PER_QUERY, 3e6),     # lists on both sides of 256 entries: the fallback's two launches
+])
+def test_range_fallback_of_every_route(batch, heads_q, heads_kv, dim, grid, topk, mode, factor, where, route):
+    """Score gradients beyond the fp16 range everywhere, or in the last head alone (with a chunk per KV group only the last chunk
+    notices, when the others are through): all passes are redone by the forms that VSA2_FLAG_PRECISE_BWD and VSA2_FLAG_FAST_BWD run
+    directly, bit for bit."""
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    rows = grid[0] * grid[1] * grid[2]
+    rnd = lambda h: torch.randn(batch, h, rows, dim, device="cuda", generator=gen).bfloat16()
+    q, k, v, d_o = rnd(heads_q), rnd(heads_kv), rnd(heads_kv), rnd(heads_q).float()
+    d_o[(slice(None), slice(None)) if where == "everywhere" else (-1, -1)] *= factor
+    d_o = d_o.bfloat16()
+    gate = torch.rand(batch, heads_q, rows, device="cuda", generator=gen)
+
+    def run(flags, scratch=None):
+        attn = vb.Vsa2Attention(vb.make_params(batch, heads_q, heads_kv, dim, grid, select_mode=mode, topk=topk, flags=flags, out_dtype=vb.F32))
+        if scratch is not None:
+            attn.bwd_scratch_bytes = scratch(attn)
+        attn.route(q, k)
+        o, lse = attn.forward(q, k, v, gate)
+        out = attn.backward(q, k, v, gate, o, lse, d_o)
+        attn.check_status()
+        return attn, out
+
+    def one_group(attn):
+        # the whole, less all groups' tiles but one
+        tiles = heads_q // heads_kv * attn.sizes.nnz_cap * 64 * 64 * 2
+        return attn.bwd_scratch_bytes - (batch * heads_kv - 1) * tiles
+
+    attn, got = run(0, {"one_chunk": None, "group_by_group": one_group, "recomputed": lambda a: 0}[route])
+    _, pair = run(vb.FLAG_PRECISE_BWD)
+    assert all(torch.isfinite(t).all() for t in got)
+    assert torch.equal(got[0], pair[0]) and torch.equal(got[3], pair[3])
+    if heads_q != heads_kv:
+        assert torch.equal(got[1], pair[1]) and torch.equal(got[2], pair[2])
+        return
+    _, fast = run(vb.FLAG_FAST_BWD)
+    col_ptr = attn.map_views()[2]
+    long = ((col_ptr[..., 1:] - col_ptr[..., :-1]) > 256)                     # [B, H, N]
+    if topk == 256:
+        assert long.any() and not long.all()
+    # cube of every token: grids of whole cubes along each edge where lists can be long
+    t, h, w = (torch.arange(n, device="cuda") // 4 for n in grid)
+    n_h, n_w = -(-grid[1] // 4), -(-grid[2] // 4)
+    cube = ((t[:, None, None] * n_h + h[None, :, None]) * n_w + w[None, None, :]).reshape(-1)
+    is_long = long[:, :, cube][..., None]
+    for i in (1, 2):
+        assert torch.equal(got[i], torch.where(is_long, pair[i], fast[i]))
