@@ -303,10 +303,15 @@ class Vsa2Attention:
         u8 = dict(dtype=torch.uint8, device=dev)
         self.ws_route = torch.empty(s.route_workspace_bytes, **u8)
         self.ws_fwd = torch.empty(s.fwd_workspace_bytes, **u8)
-        self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
         # scratch of a backward call, up to 7 GiB: taken from torch's allocator for the call and given back, so the handles of a
-        # model share it and one that only runs forward has none; 0 = none (the dQ pass recomputes the score gradients)
+        # model share it and one that only runs forward has none; 0 = none (the dQ pass recomputes the score gradients).  Up to
+        # 1 MiB (a toy grid, whose passes wait for the host) is part of the workspace instead: asking takes 3 us
         self.bwd_scratch_bytes = vsa2_attn_bwd_scratch_bytes(params)
+        if self.bwd_scratch_bytes <= 1 << 20:
+            self.bwd_scratch_bytes = 0
+            self.ws_bwd = torch.empty(vsa2_attn_bwd_preferred_workspace_bytes(params), **u8)
+        else:
+            self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
         for ws in (self.ws_route, self.ws_fwd, self.ws_bwd):
             ws[:256].zero_()          # status block
         self.out_torch_dtype = torch.float32 if params.out_dtype == F32 else torch.bfloat16

@@ -42,7 +42,7 @@ def test_scratch_is_given_back_and_done_without_when_there_is_no_room():
     torch.cuda.synchronize()
     before = torch.cuda.memory_allocated()
     got = passes(attn, qkvg, d_o)
-    assert attn.bwd_scratch_bytes > 0
+    assert attn.bwd_scratch_bytes > 1 << 20
 
     assert torch.cuda.memory_allocated() - before <= sum(t.numel() * t.element_size() for t in got) + 16 * 512
     attn.bwd_scratch_bytes = 1 << 50                         # more than any GPU has
