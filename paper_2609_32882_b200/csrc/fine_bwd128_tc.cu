@@ -189,7 +189,12 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
   using C = Bwd128<D>;
   static_assert(PASS == 0 || !SPLIT, "the dK/dV pass has no room for the low-order parts of P and dS");
   static_assert(!F16 || !SPLIT, "the fp16 forms carry no pairs");
-  if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
+  if constexpr (F16 && PASS == 0) {
+    // one answer for the block: a CTA that starts late may find that another has just raised the flag
+    if (__syncthreads_or(threadIdx.x == 0 && *a.range_flag != 0)) return;
+  } else if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) {
+    return;     // (the flag is final before this launch starts)
+  }
   constexpr uint32_t NDP = PASS == 0 ? 2 : 1;                  // dP buffers
   // dQ pass: S 0; dP buffers 128, 256 (dS overwrites the dP it came from); dQ 384.
   // dK/dV pass: S^T and dP^T take turns in the staging columns 0..127 (each is pulled into registers as soon as it is

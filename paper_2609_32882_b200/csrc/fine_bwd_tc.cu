@@ -156,7 +156,12 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int total_items = g.batch * g.Hq * g.N;
   const float c2 = g.scale * 1.4426950408889634f;
-  if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
+  if constexpr (F16) {
+    // one answer for the block: a CTA that starts late may find that another has just raised the flag
+    if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) return;
+  } else if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) {
+    return;     // (the flag is final before this launch starts)
+  }
 
   if (tid == 0) {
     bwd_init_barriers(misc);
