@@ -274,24 +274,25 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __r
         for (int ks = 0; ks < KT; ++ks) mma_bf16(acc[u], a[ks], lds32(wr + ks * 16), lds32(wr + ks * 16 + 8));
       }
       const int c = c0 + q * 32 + t * 8;                       // (C is a multiple of 8)
-      if (c >= c_end) continue;
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         const int l = half ? lb : la;
-        if (l >= L) continue;
         const size_t idx = ((size_t)b * L + l) * C + c;
         const float* v[4] = {acc[0] + 2 * half, acc[1] + 2 * half, acc[2] + 2 * half, acc[3] + 2 * half};
-        if (out_f32) {
-          float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(dx) + idx);
-          dst[0] = make_float4(v[0][0], v[0][1], v[1][0], v[1][1]);
-          dst[1] = make_float4(v[2][0], v[2][1], v[3][0], v[3][1]);
-        } else {
-          __nv_bfloat162 p[4];
+        if (c < c_end && l < L) {
+          if (out_f32) {
+            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(dx) + idx);
+            dst[0] = make_float4(v[0][0], v[0][1], v[1][0], v[1][1]);
+            dst[1] = make_float4(v[2][0], v[2][1], v[3][0], v[3][1]);
+          } else {
+            __nv_bfloat162 p[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) p[u] = __floats2bfloat162_rn(v[u][0], v[u][1]);
-          *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(dx) + idx) = *reinterpret_cast<const uint4*>(p);
+            for (int u = 0; u < 4; ++u) p[u] = __floats2bfloat162_rn(v[u][0], v[u][1]);
+            *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(dx) + idx) = *reinterpret_cast<const uint4*>(p);
+          }
         }
       }
+      __syncwarp();                                            // (together again for the next group's products)
     }
   }
 }
