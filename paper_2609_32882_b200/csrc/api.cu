@@ -257,9 +257,11 @@ DsLayout ds_layout(const Geo& g, size_t avail, bool preferred) {
   r.order = c.take(all * x.N * sizeof(int));
   r.tiles = c.off;
   const size_t room = preferred ? kStoredDsBytes : avail > r.tiles ? avail - r.tiles : 0;
-  const size_t fit = room / group < all ? room / group : all;
-  // (row index of a tile in the tensor map: 32 bits)
-  if (fit == 0 || fit * group / 128 > 0x7fffffffULL) return r;
+  // (the dK/dV pass counts the tiles of a chunk in an int)
+  const size_t most = 0x7fffffffULL / ((size_t)x.rep * x.nnz_cap);
+  size_t fit = room / group < all ? room / group : all;
+  if (fit > most) fit = most;
+  if (fit == 0) return r;
   const size_t chunks = (all + fit - 1) / fit;
   r.groups = (int)((all + chunks - 1) / chunks);
   r.total = r.tiles + r.groups * group;
@@ -708,7 +710,9 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   const DsLayout dl = ds_layout(g, scratch != nullptr ? scratch_bytes : 0, false);
   const int ds_groups = dl.groups;
   // (a few items per SM end together whatever their order)
-  int* dkv_order = ds_groups > 0 && (long long)ds_groups * fx.N > 4 * 148 ? at<int>(scratch, dl.order) : nullptr;
+  int sms = 0;
+  VSA2_CUDA(sm_count(&sms));
+  int* dkv_order = ds_groups > 0 && (long long)ds_groups * fx.N > 4 * sms ? at<int>(scratch, dl.order) : nullptr;
   const StoredDs sd{at<unsigned char>(scratch, dl.tiles), at<int>(scratch, dl.pos), at<int>(scratch, dl.counters), dkv_order, ds_groups,
                     row_ptr, col_idx, coarse ? dqc : nullptr, dq};
   // cubes of 128 tokens: both passes on 128 x 128 tiles

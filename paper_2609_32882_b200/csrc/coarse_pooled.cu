@@ -83,8 +83,11 @@ __global__ void __launch_bounds__(256) pooled_inputs_kernel(PooledInputs p) {
 static cudaError_t launch_pooled_inputs(const PooledInputs& p, cudaStream_t st) {
   size_t most = p.map_words;
   for (size_t n : p.n4) most = n > most ? n : most;
+  int sms = 0;
+  cudaError_t e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
   const size_t blocks = (most + 255) / 256;
-  pooled_inputs_kernel<<<(unsigned)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st>>>(p);
+  pooled_inputs_kernel<<<(unsigned)(blocks < (size_t)sms * 8 ? blocks : (size_t)sms * 8), 256, 0, st>>>(p);
   return cudaGetLastError();
 }
 

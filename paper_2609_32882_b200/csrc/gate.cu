@@ -411,7 +411,10 @@ size_t gate_bwd_workspace_bytes(int batch, int L, int hidden, int heads) {
 cudaError_t launch_gate_fwd(int batch, int L, int C, int Hq, const bf16* x, const bf16* w, float* gate, cudaStream_t st) {
   // 64 tokens a CTA; with fewer than two such CTAs per SM, 16 tokens and the head tiles split over the warps (2048 tokens of 1536
   // channels: 37 us with 64-token CTAs, which leave 116 of 148 SMs without one)
-  const bool few = (long long)batch * ((L + 63) / 64) < 2 * 148;
+  int sms = 0;
+  cudaError_t e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
+  const bool few = (long long)batch * ((L + 63) / 64) < 2 * sms;
   dim3 grid((L + (few ? 15 : 63)) / (few ? 16 : 64), batch);
   const int nt = (Hq + 7) / 8;
 #define VSA2_GATE_FWD(NT_, HW_)                                                                                  \
@@ -441,7 +444,10 @@ cudaError_t launch_gate_bwd(int batch, int L, int C, int Hq, int out_f32, const 
   {
     // channel slices until there are eight CTAs per SM (a chunk is the least a CTA takes)
     const int tiles = (L + kGtTok - 1) / kGtTok * batch, chunks = (C + kDxCh - 1) / kDxCh;
-    int slices = (8 * 148 + tiles - 1) / tiles;
+    int sms = 0;
+    cudaError_t e;
+    if ((e = sm_count(&sms)) != cudaSuccess) return e;
+    int slices = (8 * sms + tiles - 1) / tiles;
     if (slices > chunks) slices = chunks;
     const int per_slice = (chunks + slices - 1) / slices * kDxCh;
     dim3 grid((L + kGtTok - 1) / kGtTok, batch, (C + per_slice - 1) / per_slice);
