@@ -116,7 +116,8 @@ TextMapLayout text_map_layout(const Geo& g, bool with_csc) {
   return r;
 }
 
-RouteLayout route_layout(const Geo& g) {
+// `folded`: g is a half-cube problem whose scores the router folds itself (its own block scores and selection never exist)
+RouteLayout route_layout(const Geo& g, bool folded = false) {
   RouteLayout r;
   Carver c;
   const size_t BHq = (size_t)g.batch * g.Hq, BHk = (size_t)g.batch * g.Hkv, NG = (size_t)g.N * g.G;
@@ -124,8 +125,8 @@ RouteLayout route_layout(const Geo& g) {
   r.status = c.take(sizeof(StatusBlock));
   r.qr = c.take(BHq * NG * g.D * sizeof(bf16));
   r.kr = c.take(BHk * NG * g.D * sizeof(bf16));
-  r.lse_r = c.take(BHq * NG * sizeof(float));
-  r.pr = c.take(BHq * (size_t)g.N * g.N * sizeof(float));
+  r.lse_r = c.take(router_tc_supported(g) ? 0 : BHq * NG * sizeof(float));      // (the tensor-core router keeps them on chip)
+  r.pr = c.take(folded ? 0 : BHq * (size_t)g.N * g.N * sizeof(float));
   r.hist = c.take(BHq * 3 * 2048 * sizeof(unsigned));
   r.state = c.take(BHq * 8 * sizeof(unsigned));
   r.row_tau = c.take(BHq * g.N * sizeof(float));
@@ -160,16 +161,19 @@ BwdLayout bwd_layout(const Geo& g) {
 // [StatusBlock + rescue list of the fine forward][scratch of the coarse branch on the pooled grid]
 size_t fwd_pooled_offset() { return align_up(fine_fwd_tc_workspace_bytes(), 256); }
 
+// 128-token cubes whose halves have eight sub-cubes: the router folds the scores itself
+bool router_folds(const Geo& g) { return wide_cube(g) && narrow_geo(g).G == 8; }
+
 // 128-token cubes: the regions above are laid out for the half-cube problem (`n` = narrow_geo), followed by what
 // links the two levels: cube-level router scores, half-cube copies of the coarse tensors and of the block map.
 struct WideRouteLayout {
-  RouteLayout narrow;      // status, qr, kr, lse_r, pr (half-cube scores); its selection scratch is unused
+  RouteLayout narrow;      // status, qr, kr, lse_r, pr (half-cube scores, unless folded); its selection scratch is unused
   RouteLayout cube;        // selection scratch and pr at cube level, offsets relative to `cube_base`
   size_t cube_base, total;
 };
 WideRouteLayout wide_route_layout(const Geo& g) {
   WideRouteLayout r;
-  r.narrow = route_layout(narrow_geo(g));
+  r.narrow = route_layout(narrow_geo(g), router_folds(g));
   r.cube = route_layout(g);
   r.cube_base = align_up(r.narrow.hist, 256);     // everything from the half-cube histograms on is not needed
   r.total = r.cube_base + r.cube.total;
@@ -433,7 +437,8 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
   // selection then runs on the cube-level matrix
   const bool wide = wide_cube(g);
   const Geo r = wide ? narrow_geo(g) : g;
-  const RouteLayout rl = route_layout(r);
+  const bool folded = router_folds(g);
+  const RouteLayout rl = route_layout(r, folded);
   RouteLayout lay = rl;
   unsigned char* sel_base = reinterpret_cast<unsigned char*>(workspace);
   if (wide) {
@@ -448,8 +453,6 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
     ProfScope ps(VSA2_KERNEL_POOL_ROUTER, st, 1);
     VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, status, st));
   }
-  // (half-cubes of 8 sub-cubes: the kernel folds its scores itself)
-  const bool folded = wide && r.G == 8;
   float* pr = folded ? at<float>(sel_base, lay.pr) : at<float>(workspace, rl.pr);
   if (router_tc_supported(r))
     VSA2_CUDA(launch_router_scores_tc(r, folded, qr, kr, pr, status, st));

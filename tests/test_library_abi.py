@@ -111,6 +111,19 @@ def test_query_sizes_for_cubes_of_128_tokens():
     assert s.route_workspace_bytes > 4 * 48 * 48 * 4 and s.bwd_workspace_bytes > narrow.bwd_workspace_bytes // 2
 
 
+def test_route_workspace_holds_no_scores_of_half_cubes():
+    """435,600 tokens in cubes of 128: the router folds the scores of the half-cubes itself, so the workspace holds the cubes' N x N
+    alone (0.5 GiB for 10 heads) and not the (2N) x (2N) of the halves as well (2.1 GiB)."""
+    p = vb.make_params(batch=1, heads_q=10, heads_kv=10, head_dim=128, grid=(121, 45, 80), cube=(4, 4, 8), topk=64)
+    s = vb.vsa2_query_sizes(p)
+    scores = 10 * s.n_cubes ** 2 * 4
+    rows = 20 * s.n_cubes * 16 * 128 * 2                       # pooled router operands of Q and K
+    assert scores + rows < s.route_workspace_bytes < 2 * scores + 2 * rows
+    # other sub-cube counts go through half-cube scores in memory
+    p4 = vb.make_params(batch=1, heads_q=10, heads_kv=10, head_dim=128, grid=(121, 45, 80), cube=(4, 4, 8), rpool=(2, 2, 4), topk=64)
+    assert vb.vsa2_query_sizes(p4).route_workspace_bytes > 5 * scores
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(heads_kv=5), vb.ERR_INVALID_ARG),                       # heads_q % heads_kv
     (dict(head_dim=96), vb.ERR_UNSUPPORTED),
