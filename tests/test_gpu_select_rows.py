@@ -38,3 +38,40 @@ def test_rows_of_every_register_count(n, budget):
     for i in range(n):
         want[i, order[i, : take[i]]] = True
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("n", [32, 33, 64, 65, 127, 128, 129, 160])
+@pytest.mark.parametrize("mode", ["row", "budget", "sequence"])
+def test_maps_around_the_one_block_form(n, mode):
+    """Up to 128 cubes one block per head builds both maps, in words of 32; ties in every row, one head whose scores all tie, and budgets
+    that are zero here and everything there."""
+    torch.manual_seed(n)
+    heads, k = 3, min(n, 7)
+    sel = {"row": vb.PER_QUERY, "budget": vb.PER_QUERY_BUDGET, "sequence": vb.PER_SEQUENCE}[mode]
+    budgets = None
+    if mode == "budget":
+        budgets = torch.randint(0, n + 1, (1, heads, n), dtype=torch.int32, device="cuda")
+        budgets[0, 0, ::3], budgets[0, 1, ::4] = 0, n
+    cap = int(budgets.sum(dim=-1).max()) if mode == "budget" else 0
+    p = vb.make_params(1, heads, heads, 64, (4, 4, 4 * n), select_mode=sel, topk=0 if mode == "budget" else k, nnz_cap=cap)
+    attn = vb.Vsa2Attention(p)
+    q = torch.randn(1, heads, 64 * n, 64, device="cuda", dtype=torch.bfloat16)
+    kk = torch.randn_like(q)
+    kk[:, :, : 32 * n] = 0.0                       # equal scores in half of the sub-cube columns
+    kk[:, 1] = 0.0                                 # and everywhere
+    attn.route(q, kk, budgets)
+    attn.check_status()
+    score = attn.scores()[0].cpu().numpy()
+    rp, ci, cp, ri = (t[0].cpu().numpy() for t in attn.map_views())
+    for h in range(heads):
+        got = csr_to_mask(rp[h], ci[h], n)
+        assert np.array_equal(got, csr_to_mask(cp[h], ri[h], n).T)
+        want = np.zeros_like(got)
+        if mode == "sequence":
+            want.reshape(-1)[np.argsort(-score[h].reshape(-1), kind="stable")[: n * k]] = True
+        else:
+            take = budgets[0, h].cpu().numpy() if mode == "budget" else np.full(n, k)
+            order = np.argsort(-score[h], axis=1, kind="stable")
+            for i in range(n):
+                want[i, order[i, : take[i]]] = True
+        assert np.array_equal(got, want), h
