@@ -85,6 +85,9 @@ __device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int pe
 // A finite bf16 below 65520 in magnitude has an exact fp16 image if it is a multiple of 2^-24 (all of 2^-17 and more are: fp16
 // keeps more mantissa bits), and one within 2^-25 otherwise; a finite value beyond that range sets `range_flag` and the caller's
 // fp16 kernels stand back.  The first `reducers` blocks form the exponents of dS meanwhile.
+// SCALED: there is a b_exp.  (Without it the magnitudes are compared as the integers they are; a thread walks its groups by adding
+// quotient and remainder of its stride: a division per step and products of 1 made the copies of 480p 30 us longer.)
+template <bool SCALED>
 __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __restrict__ xa, uint4* __restrict__ ya, size_t na,
                                                                const uint4* __restrict__ xb, uint4* __restrict__ yb, size_t nb,
                                                                const int* __restrict__ b_exp, unsigned b_group, int* range_flag,
@@ -96,7 +99,14 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
     return;
   }
   constexpr int U = 4;      // 16-byte loads in flight per thread (a pure streaming kernel)
-  for (size_t i0 = (size_t)(blockIdx.x - reducers) * blockDim.x + threadIdx.x; i0 < n; i0 += U * stride) {
+  const size_t first = (size_t)(blockIdx.x - reducers) * blockDim.x + threadIdx.x;
+  unsigned grp = 0u, in_grp = 0u, step_q = 0u, step_r = 0u;      // SCALED: group of element group i of b, place in it; the same of a stride
+  if (SCALED) {
+    step_q = (unsigned)(stride / b_group);
+    step_r = (unsigned)(stride % b_group);
+  }
+  bool in_b = false;
+  for (size_t i0 = first; i0 < n; i0 += U * stride) {
     uint4 v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -108,14 +118,34 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
       const size_t i = i0 + u * stride;
       if (i >= n) break;
       const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-      // (a scaled value stays finite: the exponent takes the largest of a group to 2^-2 / max |O| at most)
-      const float f = b_exp != nullptr && i >= na ? pow2i(__ldg(b_exp + (unsigned)(i - na) / b_group)) : 1.f;
+      float f = 1.f;
+      if (SCALED && i >= na) {
+        if (!in_b) {
+          in_b = true;
+          grp = (unsigned)((i - na) / b_group);
+          in_grp = (unsigned)((i - na) % b_group);
+        } else {
+          grp += step_q;
+          in_grp += step_r;
+          if (in_grp >= b_group) {
+            in_grp -= b_group;
+            ++grp;
+          }
+        }
+        // (a scaled value stays finite: the exponent takes the largest of a group to 2^-2 / max |O| at most)
+        f = pow2i(__ldg(b_exp + grp));
+      }
       uint32_t r[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float x0 = __uint_as_float(w[e] << 16) * f, x1 = __uint_as_float(w[e] & 0xffff0000u) * f;
-        const float m0 = fabsf(x0), m1 = fabsf(x1);
-        bad |= (m0 >= 65536.f && m0 < INFINITY) || (m1 >= 65536.f && m1 < INFINITY);
+        float x0 = __uint_as_float(w[e] << 16), x1 = __uint_as_float(w[e] & 0xffff0000u);
+        if (SCALED) {
+          x0 *= f;
+          x1 *= f;
+        }
+        // magnitudes as bit patterns (65536 <= |x| < infinity)
+        const uint32_t m0 = __float_as_uint(x0) & 0x7fffffffu, m1 = __float_as_uint(x1) & 0x7fffffffu;
+        bad |= m0 - 0x47800000u < 0x38000000u || m1 - 0x47800000u < 0x38000000u;
         const __half2 h = __floats2half2_rn(x0, x1);
         r[e] = *reinterpret_cast<const uint32_t*>(&h);
       }
@@ -578,7 +608,8 @@ static cudaError_t launch_cast(const bf16* a, void* a16, size_t na, const bf16* 
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   // (element counts are multiples of the head dimension)
   const int reducers = groups < sms ? groups : sms;
-  cast_bf16_to_f16_kernel<<<sms * 16 + reducers, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
+  auto* kernel = b_exp != nullptr ? cast_bf16_to_f16_kernel<true> : cast_bf16_to_f16_kernel<false>;
+  kernel<<<sms * 16 + reducers, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
                                                      reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8, b_exp,
                                                      (unsigned)(b_group / 8), range_flag, scale, groups, per_group, reducers);
   return cudaGetLastError();
