@@ -38,15 +38,19 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the 720p top-64 launch with 40 heads: an
 # 8-head ncu capture of the same kernel times 5 (every head streams its own tensors, so the traffic grows in
 # proportion to the heads; the 40-head launch is too large for a full-set capture).
-NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.504200e9 + 0.295100e9)}
+NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.501570e9 + 0.293740e9),
+                                # copies of Q and K + dK/dV with the stored dS + dQ from it
+                                "fine_bwd": 5 * ((0.309830e9 + 0.261202e9) + (2.446885e9 + 6.304944e9) + (6.611088e9 + 0.159028e9)),
+                                "router_pool": 5 * (0.047220e9 + 0.017765e9)}
 
 
 # What ncu shows as the busiest unit of each tensor kernel at 64-token cubes (8-head capture, profiles/): the roofline
 # below is quoted against the tensor peak as the contract asks, these say what actually holds the kernel there.
 NCU_LIMITER = {
     "fine_fwd": "L2 -> SM read rate: 12.9 TB/s against 11.8 TB/s sustained peak (tensor pipe 82 % active at the half rate of M = 64)",
-    "fine_bwd": "shared-memory data pipe (dK/dV: four products and the hand-over of dS) and the reads of the stored dS tiles (dQ)",
-    "router_pool": "exponential unit (one ex2 per score): about three quarters busy",
+    "fine_bwd": "dK/dV: shared-memory data pipe 99 % (tensor-core operand fetches 68 % + thread loads/stores 31 %; tensor pipe 46 %); "
+                "dQ from the stored dS: DRAM 68 % (tensor pipe 33 %)",
+    "router_pool": "exponential unit 80 % (two ex2 per score), instruction issue 64 %",
 }
 # L2 -> SM read rate that ncu reports as the sustained peak of this part (derived__lts__lts2xbar_bytes.sum.peak_sustained
 # in the 8-head capture of profiles/kernels_720p_8heads_ncu_full.md, where the fine forward itself reads 12.0 TB/s).

@@ -9,7 +9,8 @@
 // instead (fine_bwd_tc.cu) costs two more products, the exponentials and the V and dO tiles: 224 KB of shared-memory
 // traffic per tile against 96 KB, and under the power cap (all long cases) the work is the time.  The price is 8 KB per pair written to
 // and read from HBM; the passes run head group by head group so that the scratch stays bounded (kStoredDsBytes).
-// The tiles hold the values the recomputing pass would form (same operands, same order), so dQ is the same bit for bit.
+// The tiles hold the values the recomputing pass would form (same operands, same order), so dQ is the same bit for bit -- but for the
+// all-fp16 form of GQA groups, whose dP comes from fp16 copies of V and dO (an element below 2^-17 is 2^-25 off at most).
 #include "fine_bwd_tc.cuh"
 
 namespace vsa2 {
