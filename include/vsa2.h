@@ -205,7 +205,9 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
  *   - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that device
  *     current); make that first call at start-up, outside any stream capture: with CUDA's lazy module loading it is
  *     also the moment the driver loads the library's device code and backs the 8 MiB array, so it is the one call
- *     that can fail for lack of memory.  No call uses cudaMalloc, cudaFree or any allocating routine.
+ *     that can fail for lack of memory.  No call uses cudaMalloc, cudaFree or any allocating routine.  The address is one
+ *     context's: use this entry point in one CUDA context per device and not across a device reset (the other entry points may
+ *     be called in any context).
  *   - All calls on one device share the one array, and it keeps the last call's contents: the call clears what
  *     must start at zero itself, but two calls that overlap on the GPU (different streams, no ordering) race;
  *     order them on one stream or with events.  The address look-up is guarded by a mutex; the library's launch
