@@ -253,6 +253,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       goto done;
     if (STORES_DS && !SPLIT && warp == 19 && a.ds != nullptr) {
       // ---------------------------------------------------------------- copies the dS tiles to the scratch as they stand
+      const uint64_t policy = tc::evict_first_policy();
       uint32_t tg = 0;
       for (uint32_t seq = 0;; ++seq) {
         VSA2_NEXT_REC(rec, seq);
@@ -261,8 +262,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           VSA2_WAIT_PARKED(&misc->ds_ready[0], tg & 1);
           if (lane == 0) {
             const int s0 = misc->ds_slot[tg & 3][0], s1 = misc->ds_slot[tg & 3][1];
-            if (s0 >= 0) tc::bulk_store(a.ds + (size_t)s0 * kSlab, ds_tile, kSlab);
-            if (s1 >= 0) tc::bulk_store(a.ds + (size_t)s1 * kSlab, ds_tile + kSlab, kSlab);
+            if (s0 >= 0) tc::bulk_store(a.ds + (size_t)s0 * kSlab, ds_tile, kSlab, policy);
+            if (s1 >= 0) tc::bulk_store(a.ds + (size_t)s1 * kSlab, ds_tile + kSlab, kSlab, policy);
             tc::bulk_store_commit();
             tc::bulk_store_wait_read();
             tc::mbar_arrive(&misc->ds_free[0]);

@@ -75,6 +75,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
 
   if (warp < 3) {
     // ------------------------------------------------------------------ producers: first K block of a pair, second, dS pair
+    const uint64_t policy = tc::evict_first_policy();      // (the tiles pass through once, the K cubes stay)
     uint32_t tg = 0;
     for (uint32_t seq = 0;; ++seq) {
       VSA2_NEXT_REC(rec, seq);
@@ -106,7 +107,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
           if (lane < C::DH)
             tc::tma_load_5d(stage + (2 * lane + warp) * kSlab, text ? &tm_kt : &tm_k, &misc->full[slot], lane * 64, c1, c2, c3, bhk);
         } else if (lane == 0) {
-          tc::bulk_load(stage + C::KBYTES, tiles + (size_t)t * C::DSBYTES, ds_bytes, &misc->full[slot]);
+          tc::bulk_load(stage + C::KBYTES, tiles + (size_t)t * C::DSBYTES, ds_bytes, &misc->full[slot], policy);
         }
       }
     }
