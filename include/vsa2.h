@@ -261,7 +261,7 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
                           const void* d_o, void* dq, void* dk, void* dv, float* dgate,
                           void* workspace, size_t workspace_bytes, void* scratch, size_t scratch_bytes, void* cuda_stream);
 
-/* Bytes of scratch with which the backward runs fastest (bounded: 7 GiB of score gradients; 0 where none are kept, or for
+/* Bytes of scratch with which the backward runs fastest (bounded: 7 GiB of score gradients, with 128-token cubes 8; 0 where none are kept, or for
  * invalid parameters), and of a workspace that holds them too.  Less room is used as far as it goes, a KV group at a time; where
  * one group does not fit, or without scratch, the dQ pass recomputes.  The gradients are the same bit for bit, except that dQ of GQA
  * groups with all-fp16 passes (TopK >= 8) takes V and dO from their fp16 copies when its tiles were kept and from the bf16 tensors

@@ -303,7 +303,7 @@ class Vsa2Attention:
         u8 = dict(dtype=torch.uint8, device=dev)
         self.ws_route = torch.empty(s.route_workspace_bytes, **u8)
         self.ws_fwd = torch.empty(s.fwd_workspace_bytes, **u8)
-        # scratch of a backward call, up to 7 GiB: taken from torch's allocator for the call and given back, so the handles of a
+        # scratch of a backward call, up to 8 GiB: taken from torch's allocator for the call and given back, so the handles of a
         # model share it and one that only runs forward has none; 0 = none (the dQ pass recomputes the score gradients).  Up to
         # 1 MiB (a toy grid, whose passes wait for the host) is part of the workspace instead: asking takes 3 us
         self.bwd_scratch_bytes = vsa2_attn_bwd_scratch_bytes(params)

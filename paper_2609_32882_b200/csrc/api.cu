@@ -245,22 +245,28 @@ size_t bwd_workspace_bytes(const Geo& g) {
 // 16..256-cube budget with four heads a group): a launch over fewer blocks loses more on its last, unevenly filled items
 // (one head of 720p at a time: 10 blocks per SM), more scratch gains nothing.
 constexpr size_t kStoredDsBytes = (size_t)7 << 30;
+// 128-token cubes keep dS where both passes run on 128 x 128 tiles: a tile of 32 KB per pair of cubes, places and orders of the
+// cube map.  219,600 tokens, 10 heads, top-64, backward: 33.8 ms without, 31.9 with a head (4 GB) at a time, 31.8 with four
+constexpr size_t kStoredDsBytesWide = (size_t)8 << 30;      // two such heads
+bool wide_stored_ds(const Geo& g) { return g.Lt == 0 && g.rep == 1 && !fine_bwd_dkv_wants_pair(g) && fine_bwd128_supported(narrow_geo(g)); }
 struct DsLayout {
   size_t counters, pos, order, tiles, total;
   int groups;          // KV groups per chunk, 0: no stored dS
 };
 DsLayout ds_layout(const Geo& g, size_t avail, bool preferred) {
   DsLayout r{};
-  if (!dq_pass_f16(g) || wide_cube(g)) return r;
+  const bool wide = wide_cube(g);
+  if (!dq_pass_f16(g) || (wide && !wide_stored_ds(g))) return r;
   const Geo x = g.Lt > 0 ? text_geo(g) : g;
-  const size_t all = (size_t)g.batch * g.Hkv, group = (size_t)x.rep * x.nnz_cap * kBlockTokens * kBlockTokens * sizeof(bf16);
+  const size_t tokens = wide ? 2 * kBlockTokens : kBlockTokens;
+  const size_t all = (size_t)g.batch * g.Hkv, group = (size_t)x.rep * x.nnz_cap * tokens * tokens * sizeof(bf16);
   if (group == 0) return r;
   Carver c;
   r.counters = c.take(2 * all * sizeof(int));
   r.pos = c.take((size_t)g.batch * g.Hq * x.nnz_cap * sizeof(int));
   r.order = c.take(all * x.N * sizeof(int));
   r.tiles = c.off;
-  const size_t room = preferred ? kStoredDsBytes : avail > r.tiles ? avail - r.tiles : 0;
+  const size_t room = preferred ? (wide ? kStoredDsBytesWide : kStoredDsBytes) : avail > r.tiles ? avail - r.tiles : 0;
   // (the dK/dV pass counts the tiles of a chunk in an int)
   const size_t most = 0x7fffffffULL / ((size_t)x.rep * x.nnz_cap);
   size_t fit = room / group < all ? room / group : all;
@@ -715,9 +721,10 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   // (a few items per SM end together whatever their order)
   int sms = 0;
   VSA2_CUDA(sm_count(&sms));
-  int* dkv_order = ds_groups > 0 && (long long)ds_groups * fx.N > 4 * sms ? at<int>(scratch, dl.order) : nullptr;
+  const Geo& dg = wide ? g : fx;                // geometry of the lists by which the tiles of dS are placed
+  int* dkv_order = ds_groups > 0 && (long long)ds_groups * dg.N > 4 * sms ? at<int>(scratch, dl.order) : nullptr;
   const StoredDs sd{at<unsigned char>(scratch, dl.tiles), at<int>(scratch, dl.pos), at<int>(scratch, dl.counters), dkv_order, ds_groups,
-                    row_ptr, col_idx, coarse ? dqc : nullptr, dq};
+                    wide ? map->row_ptr : row_ptr, wide ? map->col_idx : col_idx, coarse ? dqc : nullptr, dq};
   // cubes of 128 tokens: both passes on 128 x 128 tiles
   const bool wide128 = wide && g.Lt == 0 && fine_bwd128_supported(n);
   {
@@ -727,11 +734,11 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
       VSA2_CUDA(launch_cast_qk(fx, qb, at<unsigned char>(workspace, bwd_f16_offset(g)), kb,
                                at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale,
                                &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
-      VSA2_CUDA(launch_ds_positions(fx, row_ptr, col_idx, col_ptr, row_idx, at<int>(scratch, dl.pos), sd.counters,
-                                    2 * g.batch * g.Hkv, st));
+      VSA2_CUDA(launch_ds_positions(dg, sd.row_ptr, sd.col_idx, wide ? map->col_ptr : col_ptr, wide ? map->row_idx : row_idx,
+                                    at<int>(scratch, dl.pos), sd.counters, 2 * g.batch * g.Hkv, st));
       if (dkv_order != nullptr) {
         g_launches += 1;
-        VSA2_CUDA(launch_dkv_order(fx, col_ptr, dkv_order, st));
+        VSA2_CUDA(launch_dkv_order(dg, wide ? map->col_ptr : col_ptr, dkv_order, st));
       }
     } else if (wide128)
       VSA2_CUDA(launch_fine_bwd128_dq_tc(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
@@ -754,7 +761,12 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
     const int chunks = ds_groups > 0 ? (g.batch * g.Hkv + ds_groups - 1) / ds_groups : 0;
     if (chunks > 0) g_launches += 2 * chunks;      // (dQ per chunk and its fallback; the first dK/dV launch is counted above)
     unsigned char* v16 = gqa16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g) + bwd_k16_bytes(g)) : nullptr;
-    if (dkv128)
+    if (dkv128 && ds_groups > 0)
+      VSA2_CUDA(launch_fine_bwd128_stored(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, col_ptr, row_idx, coarse ? dqc : nullptr,
+                                          coarse ? dkc : nullptr, coarse ? dvc : nullptr, dq, dk, dv,
+                                          reinterpret_cast<StatusBlock*>(workspace), st, at<unsigned char>(workspace, bwd_f16_offset(g)),
+                                          at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale.exp, sd));
+    else if (dkv128)
       VSA2_CUDA(launch_fine_bwd128_dkv_tc(n, qb, kb, vb, dob, lse, delta, col_ptr, row_idx, coarse ? dkc : nullptr,
                                           coarse ? dvc : nullptr, dk, dv, reinterpret_cast<StatusBlock*>(workspace), st,
                                           dq_pass_f16(g) ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,

@@ -340,9 +340,10 @@ cudaError_t launch_cast_qk(const Geo& g, const bf16* q, void* q16, const bf16* k
 // fp16 copies of V and of dO times 2^ds_exp of its KV group, with the same flag
 cudaError_t launch_cast_v_do(const Geo& g, const bf16* v, void* v16, const bf16* d_o, void* do16, const int* ds_exp, int* range_flag,
                              cudaStream_t st);
-// dS kept between the two backward passes (fine_bwd_dq_ds_tc.cu): scratch for the pairs of `chunk_groups` KV groups at a time
+// dS kept between the two backward passes (fine_bwd_dq_ds_tc.cu, fine_bwd128_dq_ds_tc.cu): scratch for the pairs of `chunk_groups`
+// KV groups at a time.  On 128 x 128 tiles every size and list below is that of the cube map.
 struct StoredDs {
-  void* scratch;        // chunk_groups * rep * nnz_cap tiles of 8 KB (64 queries x 64 keys, fp16)
+  void* scratch;        // chunk_groups * rep * nnz_cap tiles of 8 KB (64 queries x 64 keys, fp16), or of 32 KB (128 x 128)
   const int* pos;       // [B, Hq, nnz_cap], filled by launch_ds_positions
   int* counters;        // two words per chunk, cleared by launch_ds_positions
   int* order;           // null, or [B, Hkv, N]: items of the dK/dV pass, longest lists of a group first (launch_dkv_order)
@@ -358,6 +359,14 @@ cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaS
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
                                   int* item_counter, bool swizzled, const int* ds_exp, cudaStream_t st);
+cudaError_t launch_fine_bwd128_dq_ds(const Geo& g, long long cap, const void* k16, const void* ds, int head0, int heads,
+                                     const int* row_ptr, const int* col_idx, const float* dqc, void* dq, StatusBlock* status,
+                                     int* range_flag, int* item_counter, const int* ds_exp, cudaStream_t st);
+cudaError_t launch_fine_bwd128_stored(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse,
+                                      const float* delta, const int* row_ptr, const int* col_idx, const int* col_ptr,
+                                      const int* row_idx, const float* dqc, const float* dkc, const float* dvc, void* dq, void* dk,
+                                      void* dv, StatusBlock* status, cudaStream_t st, const void* q16, const void* k16,
+                                      const int* ds_exp, const StoredDs& sd);
 cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse,
                                         const float* delta, const int* row_ptr, const int* col_idx, const float* dqc, void* dq,
                                         StatusBlock* status, cudaStream_t st);

@@ -68,6 +68,13 @@ struct Bwd128Args {
   int* range_flag;      // fp16 form of the dQ pass and its fallback: as in DqArgs of the 64-token pass (when = 0: always runs)
   int when;
   const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale; fp16 forms): the weights carry it
+  int first_item, items;
+  // dK/dV pass that stores dS: the items in the order they are drawn in (or null); the tiles of the launch's heads and the first of
+  // these; places of the column lists' entries in the row lists, both of the CUBE map
+  const int* order;
+  unsigned char* ds;
+  int head0;
+  const int* pos;
 };
 
 // The stationary cube of a work item and the lists of streamed cubes that meet it.
@@ -181,7 +188,9 @@ __device__ __forceinline__ void store_operand_chunk_f16(uint32_t taddr, const fl
 // F16 (without SPLIT): the maps of X0 and Y0 (Q and K, in the order of the pass) point at fp16 copies and dS is rounded to fp16,
 // so S and the dQ (dK) product are fp16 x fp16 instructions; dP, P and the dV product stay bf16.  See the 64-token passes; as
 // there, only the dQ pass tracks the magnitude of dS.
-template <int D, int PASS, bool SPLIT, bool F16 = false>
+// STORE (dK/dV pass, F16): the launch also leaves every tile's dS for fine_bwd128_dq_ds_kernel, 16 coalesced bytes per thread at a
+// time; a dS beyond the fp16 range stays an infinity, which that kernel finds.
+template <int D, int PASS, bool SPLIT, bool F16 = false, bool STORE = false>
 __global__ void __launch_bounds__(kW2Threads, 1)
 fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_constant__ CUtensorMap tm_x1,
                       const __grid_constant__ CUtensorMap tm_y0, const __grid_constant__ CUtensorMap tm_y1, Geo g,
@@ -189,6 +198,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
   using C = Bwd128<D>;
   static_assert(PASS == 0 || !SPLIT, "the dK/dV pass has no room for the low-order parts of P and dS");
   static_assert(!F16 || !SPLIT, "the fp16 forms carry no pairs");
+  static_assert(!STORE || (PASS == 1 && F16), "the dK/dV pass stores fp16 tiles");
   if constexpr (F16 && PASS == 0) {
     // one answer for the block: a CTA that starts late may find that another has just raised the flag
     if (__syncthreads_or(threadIdx.x == 0 && *a.range_flag != 0)) return;
@@ -208,7 +218,6 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
   Bwd128Misc* misc = reinterpret_cast<Bwd128Misc*>(smem + C::OFF_MISC);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int total_items = g.batch * (PASS == 0 ? g.Hq : g.Hkv) * (g.N / 2);
   const float c2 = g.scale * 1.4426950408889634f;
 
   if (tid < 16) {
@@ -281,7 +290,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
       for (uint32_t seq = 0;; ++seq) {
         int item = 0;
         if (lane == 0) {
-          if (warp == 0 && !item_publish_ahead(&misc->items, seq, published, a.item_counter, total_items, &misc->abort_flag)) item = -2;
+          if (warp == 0 && !item_publish_ahead(&misc->items, seq, published, a.item_counter, a.items, &misc->abort_flag, a.first_item, STORE ? a.order : nullptr)) item = -2;
           else item = item_get(&misc->items, seq, &misc->abort_flag);
         }
         item = __shfl_sync(0xffffffffu, item, 0);
@@ -569,8 +578,24 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
         dlt = a.delta[(size_t)il.bh_stat * g.S + l_tok];
       }
       if (nt_all > 0) {
+        // STORE: places of the current tile and of the next one (loaded a tile ahead); one list per item (a head of its own per KV head)
+        int place = 0;
+        const int* place_next = nullptr;
+        unsigned char* ds_head = nullptr;
+        if constexpr (STORE) {
+          const int beg = a.ptr[(size_t)il.bhq0 * (g.N + 1) + il.blk0];
+          const size_t cap = (size_t)g.nnz_cap / 4;            // (the expanded lists hold every cube entry four times)
+          place_next = a.pos + (size_t)il.bhq0 * cap + beg / 4;
+          ds_head = a.ds + (size_t)(il.bhq0 - a.head0) * cap * (128 * 128 * 2) + (8 * half) * 2048 + row * 16;
+          place = __ldg(place_next);
+        }
         VSA2_W2_TILES_BEGIN
           const uint32_t dpb = (tg % NDP) * 128;
+          unsigned char* ds_tile = nullptr;
+          if constexpr (STORE) {
+            ds_tile = ds_head + (size_t)place * (128 * 128 * 2);
+            if (t + 1 < nt_l) place = __ldg(place_next + t + 1);
+          }
           uint32_t pf[64];                 // S, then P (as float bits) of this thread's 64 columns
           VSA2_WAIT(&misc->s_full, tg & 1);
           tc::tc_fence_after();
@@ -661,8 +686,17 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
               if constexpr (F16) {     // (a dS at the clamp: the dQ pass has met the same value and raised the flag)
                 uint32_t h[16];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) h[e] = pack_f16x2_sat(ds[2 * e], ds[2 * e + 1]);
+                for (int e = 0; e < 16; ++e) h[e] = STORE ? pack_f16x2(ds[2 * e], ds[2 * e + 1]) : pack_f16x2_sat(ds[2 * e], ds[2 * e + 1]);
                 tc::tmem_st_32x32b_x16(lane_addr + TM_DS + 32 * half + 16 * c, h);
+                if constexpr (STORE) {
+#pragma unroll
+                  for (int q = 0; q < 4; ++q) {
+                    // (a padding row's P is e^(0 - lse), its dS may be anything: the tile holds zeros there)
+                    uint4* dst = reinterpret_cast<uint4*>(ds_tile + (4 * c + q) * 2048);
+                    if (l_tok >= 0) __stcs(dst, make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]));
+                    else __stcs(dst, make_uint4(0u, 0u, 0u, 0u));
+                  }
+                }
               } else {
                 store_operand_chunk<false>(lane_addr + TM_DS + 32 * half + 16 * c, ds);
               }
@@ -765,15 +799,15 @@ bool fine_bwd128_supported(const Geo& g) {
   return g.Lt == 0 && g.N % 2 == 0 && g.rep <= 16 && (g.D == 64 || g.D == 128);
 }
 
-template <int D, int PASS, bool SPLIT, bool F16 = false>
+template <int D, int PASS, bool SPLIT, bool F16 = false, bool STORE = false>
 static cudaError_t launch_bwd128(const CUtensorMap& x0, const CUtensorMap& x1, const CUtensorMap& y0, const CUtensorMap& y1,
                                  const Geo& g, const Bwd128Args& a, int grid, cudaStream_t st) {
   cudaError_t e;
   static KernelAttr attr;
-  if ((e = prepare_kernel((const void*)fine_bwd128_tc_kernel<D, PASS, SPLIT, F16>, attr, Bwd128<D>::smem_bytes, kW2Threads,
+  if ((e = prepare_kernel((const void*)fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE>, attr, Bwd128<D>::smem_bytes, kW2Threads,
                           256 * 56 + 256 * 200)))
     return e;
-  fine_bwd128_tc_kernel<D, PASS, SPLIT, F16><<<grid, kW2Threads, Bwd128<D>::smem_bytes, st>>>(x0, x1, y0, y1, g, a);
+  fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE><<<grid, kW2Threads, Bwd128<D>::smem_bytes, st>>>(x0, x1, y0, y1, g, a);
   return cudaGetLastError();
 }
 
@@ -796,8 +830,8 @@ cudaError_t launch_fine_bwd128_dq_tc(const Geo& g, const bf16* q, const bf16* k,
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
-  Bwd128Args a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, nullptr, dq, nullptr, status, flag, 0, f16 ? scale->exp : nullptr};
-  const int total = g.batch * g.Hq * (g.N / 2);
+  Bwd128Args a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, nullptr, dq, nullptr, status, flag, 0, f16 ? scale->exp : nullptr, 0, g.batch * g.Hq * (g.N / 2)};
+  const int total = a.items;
   const int grid = total < sms ? total : sms;
   const bool split = !(g.flags & VSA2_FLAG_FAST_BWD);
   if (f16) {
@@ -836,8 +870,8 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   Bwd128Args a{&status->pad[3], lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, &status->pad[kRangeFlagSlot], 0,
-               f16 ? ds_exp : nullptr};
-  const int total = g.batch * g.Hkv * (g.N / 2);
+               f16 ? ds_exp : nullptr, 0, g.batch * g.Hkv * (g.N / 2)};
+  const int total = a.items;
   const int grid = total < sms ? total : sms;
   const bool split = fine_bwd_dkv_wants_pair(g);
   if (split) return cudaErrorInvalidValue;      // (the caller takes the 64-token kernels for that)
@@ -852,6 +886,45 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
   }
   if (g.D == 128) return launch_bwd128<128, 1, false>(tk, tv, tq, tdo, g, a, grid, st);
   return launch_bwd128<64, 1, false>(tk, tv, tq, tdo, g, a, grid, st);
+}
+
+// Both passes with dS kept between them (one query head per KV head, fp16 forms): KV heads in chunks that the scratch holds, the dQ
+// pass of a chunk behind its dK/dV pass; then, should a value have left the fp16 range, both passes again in the forms that
+// have no such limit.  `sd`: scratch, orders and places of the CUBE map; the other maps are expanded to 64-token blocks.
+cudaError_t launch_fine_bwd128_stored(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse,
+                                      const float* delta, const int* row_ptr, const int* col_idx, const int* col_ptr,
+                                      const int* row_idx, const float* dqc, const float* dkc, const float* dvc, void* dq, void* dk,
+                                      void* dv, StatusBlock* status, cudaStream_t st, const void* q16, const void* k16,
+                                      const int* ds_exp, const StoredDs& sd) {
+  if (!fine_bwd128_supported(g) || !fine_bwd_dq_uses_f16(g) || g.rep != 1) return cudaErrorInvalidValue;
+  CUtensorMap tq, tk, tv, tdo, tq16, tk16;
+  if (!make_cube_tmap(&tq, q, g, g.Hq) || !make_cube_tmap(&tk, k, g, g.Hkv) || !make_cube_tmap(&tv, v, g, g.Hkv) ||
+      !make_cube_tmap(&tdo, d_o, g, g.Hq) || !make_cube_tmap(&tq16, reinterpret_cast<const bf16*>(q16), g, g.Hq) ||
+      !make_cube_tmap(&tk16, reinterpret_cast<const bf16*>(k16), g, g.Hkv))
+    return cudaErrorInvalidValue;
+  int sms = 0;
+  cudaError_t e;
+  if ((e = sm_count(&sms)) != cudaSuccess) return e;
+  int* flag = &status->pad[kRangeFlagSlot];
+  const int cubes = g.N / 2, all = g.batch * g.Hkv;
+  for (int c = 0, g0 = 0; g0 < all; ++c, g0 += sd.chunk_groups) {
+    const int n = all - g0 < sd.chunk_groups ? all - g0 : sd.chunk_groups, items = n * cubes;
+    Bwd128Args a{sd.counters + 2 * c, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, flag, 1, ds_exp, g0 * cubes, items,
+                 sd.order, reinterpret_cast<unsigned char*>(sd.scratch), g0, sd.pos};
+    const int grid = items < sms ? items : sms;
+    e = g.D == 128 ? launch_bwd128<128, 1, false, true, true>(tk16, tv, tq16, tdo, g, a, grid, st)
+                   : launch_bwd128<64, 1, false, true, true>(tk16, tv, tq16, tdo, g, a, grid, st);
+    if (e != cudaSuccess) return e;
+    if ((e = launch_fine_bwd128_dq_ds(g, g.nnz_cap / 4, k16, sd.scratch, g0, n, sd.row_ptr, sd.col_idx, dqc, dq, status, flag,
+                                      sd.counters + 2 * c + 1, ds_exp, st)) != cudaSuccess)
+      return e;
+  }
+  const int items = all * cubes, grid = items < sms ? items : sms;
+  Bwd128Args a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, nullptr, dq, nullptr, status, flag, 2, nullptr, 0, items};
+  e = g.D == 128 ? launch_bwd128<128, 0, true>(tq, tdo, tk, tv, g, a, grid, st) : launch_bwd128<64, 0, true>(tq, tdo, tk, tv, g, a, grid, st);
+  if (e != cudaSuccess) return e;
+  Bwd128Args b{&status->pad[5], lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, flag, 2, nullptr, 0, items};
+  return g.D == 128 ? launch_bwd128<128, 1, false>(tk, tv, tq, tdo, g, b, grid, st) : launch_bwd128<64, 1, false>(tk, tv, tq, tdo, g, b, grid, st);
 }
 
 }  // namespace vsa2

@@ -220,14 +220,15 @@ __device__ __forceinline__ void item_queue_init(ItemQueue* q, int consumers) {
     tc::mbar_init(&q->empty[s], consumers);
   }
 }
-// scheduler: publishes every sequence number up to seq + kItemAhead that is not out yet; false on a timed-out wait
+// scheduler: publishes every sequence number up to seq + kItemAhead that is not out yet; false on a timed-out wait.
+// The items are first .. first + total - 1, in the order of `order` if there is one.
 __device__ __forceinline__ bool item_publish_ahead(ItemQueue* q, uint32_t seq, uint32_t& published, int* counter, int total,
-                                                   volatile int* abort_flag) {
+                                                   volatile int* abort_flag, int first = 0, const int* order = nullptr) {
   while (published <= seq + (seq ? kItemAhead : 1)) {
     const uint32_t slot = published % kItemSlots, par = ((published / kItemSlots) & 1) ^ 1;
     if (!tc::mbar_wait_parked(&q->empty[slot], par, abort_flag)) return false;
     const int it = item_draw(published, counter);
-    q->item[slot] = it < total ? it : -1;
+    q->item[slot] = it >= total ? -1 : order != nullptr ? order[first + it] : first + it;
     tc::mbar_arrive(&q->full[slot]);
     ++published;
   }

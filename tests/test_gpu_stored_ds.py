@@ -126,3 +126,37 @@ def test_range_fallback_of_every_route(batch, heads_q, heads_kv, dim, grid, topk
     is_long = long[:, :, cube][..., None]
     for i in (1, 2):
         assert torch.equal(got[i], torch.where(is_long, pair[i], fast[i]))
+
+
+@pytest.mark.parametrize("factor", [1.0, 2.5e5, 1e8])        # in range; found by the dQ pass; found before the first pass
+@pytest.mark.parametrize("heads,dim,grid,topk,mode", [
+    (2, 64, (4, 8, 16), 2, vb.PER_QUERY),
+    (3, 128, (5, 9, 9), 3, vb.PER_SEQUENCE),         # ragged cubes, trailing half-cubes without a token, lists of any length
+    (8, 64, (16, 20, 40), 3, vb.PER_SEQUENCE),       # enough items for the pass to be drawn in order of length
+    (2, 128, (8, 16, 32), 11, vb.PER_QUERY),
+])
+def test_gradients_of_128_token_cubes_do_not_depend_on_the_scratch(heads, dim, grid, topk, mode, factor):
+    """The same on 128 x 128 tiles: dQ from stored tiles (one chunk, a head at a time) against the pass that recomputes them; out of
+    range both end in the forms without fp16."""
+    p = vb.make_params(1, heads, heads, dim, grid, cube=(4, 4, 8), select_mode=mode, topk=topk)
+    attn = vb.Vsa2Attention(p)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    rows = grid[0] * grid[1] * grid[2]
+    rnd = lambda: torch.randn(1, heads, rows, dim, device="cuda", generator=gen).bfloat16()
+    q, k, v, d_o = rnd(), rnd(), rnd(), rnd().float()
+    d_o[:, -1] *= factor                             # (the last head alone: a head at a time, only the last chunk meets it)
+    d_o = d_o.bfloat16()
+    gate = torch.rand(1, heads, rows, device="cuda", generator=gen)
+    attn.route(q, k)
+    o, lse = attn.forward(q, k, v, gate)
+    all_heads, least = vb.vsa2_attn_bwd_scratch_bytes(p), attn.sizes.bwd_workspace_bytes
+    one_head = all_heads - (heads - 1) * attn.sizes.nnz_cap * 128 * 128 * 2
+    attn.bwd_scratch_bytes, attn.ws_bwd = 0, torch.empty(least, dtype=torch.uint8, device="cuda")
+    got = [attn.backward(q, k, v, gate, o, lse, d_o)]
+    for size in (all_heads, one_head):
+        attn.bwd_scratch_bytes = size
+        got.append(attn.backward(q, k, v, gate, o, lse, d_o))
+        attn.check_status()
+    for other in got[1:]:
+        for name, x, y in zip(("dq", "dk", "dv", "dgate"), got[0], other):
+            assert torch.isfinite(x.float()).all() and torch.equal(x, y), name
