@@ -191,6 +191,16 @@ int vsa2_query_sizes(const vsa2_params* p, vsa2_sizes* out);
 int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets,
                const vsa2_map* map_out, void* workspace, size_t workspace_bytes, void* cuda_stream);
 
+/* The same with a scratch region (device, 256-byte aligned, NULL = none).  With at least vsa2_route_scratch_bytes(p) bytes of it the
+ * router forms every exponential once and parks partial sums there; the maps are the same bit for bit, P_r differs in its last
+ * bits.  Nothing in it is read after the call's kernels: one region may serve all calls that follow one another on a stream.
+ * vsa2_route_scratch_bytes is 0 where the router has no use for any (small problems, other sub-cube counts than 8 per 64 tokens) and
+ * for invalid parameters; about 76 kB per cube otherwise (720p: 0.11 GB, 435,600 tokens in cubes of 128: 0.28 GB). */
+int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets,
+                       const vsa2_map* map_out, void* workspace, size_t workspace_bytes, void* scratch, size_t scratch_bytes,
+                       void* cuda_stream);
+size_t vsa2_route_scratch_bytes(const vsa2_params* p);
+
 /* Allocation-free variant of vsa2_route (the paper has no counterpart).
  *
  * For callers that cannot allocate device memory where they need a block map: code running where cudaMalloc is

@@ -33,7 +33,7 @@ EXPORTS = ("vsa2_query_sizes", "vsa2_route", "vsa2_route_scores", "vsa2_attn_fwd
            "vsa2_device_status", "vsa2_strerror", "vsa2_profile_events", "vsa2_launch_count", "vsa2_selftest_umma", "vsa2_route_noalloc", "vsa2_last_cuda_error",
            "vsa2_gate_fwd", "vsa2_gate_bwd", "vsa2_gate_bwd_workspace_bytes",
            "vsa2_attn_bwd_preferred_workspace_bytes", "vsa2_attn_bwd_scratch", "vsa2_attn_bwd_scratch_bytes",
-           "vsa2_permute_cube_major",
+           "vsa2_route_scratch", "vsa2_route_scratch_bytes", "vsa2_permute_cube_major",
            "vsa2_selftest_timeout", "vsa2_debug_rescue_capacity", "vsa2_selftest_divmod")
 
 KERNELS = ("pool", "router_lse", "router_pool", "select", "coarse_fwd", "fine_fwd", "bwd_pre", "coarse_bwd",
@@ -92,10 +92,11 @@ def _lib():
         vp, sz, i32p = C.c_void_p, C.c_size_t, C.POINTER(C.c_int32)
         lib.vsa2_query_sizes.argtypes = [C.POINTER(Params), C.POINTER(Sizes)]
         lib.vsa2_route.argtypes = [C.POINTER(Params), vp, vp, vp, C.POINTER(Map), vp, sz, vp]
+        lib.vsa2_route_scratch.argtypes = lib.vsa2_route.argtypes[:-1] + [vp, sz, vp]
         lib.vsa2_route_noalloc.argtypes = [C.POINTER(Params), vp, vp, vp, C.POINTER(Map), vp, vp]
         lib.vsa2_permute_cube_major.argtypes = [C.POINTER(Params), C.c_int32, C.c_int32, vp, vp, vp]
         lib.vsa2_gate_fwd.argtypes = [C.POINTER(Params), C.c_int32, vp, vp, vp, vp]
-        for fn in (lib.vsa2_attn_bwd_preferred_workspace_bytes, lib.vsa2_attn_bwd_scratch_bytes):
+        for fn in (lib.vsa2_attn_bwd_preferred_workspace_bytes, lib.vsa2_attn_bwd_scratch_bytes, lib.vsa2_route_scratch_bytes):
             fn.argtypes = [C.POINTER(Params)]
             fn.restype = C.c_size_t
         lib.vsa2_gate_bwd_workspace_bytes.argtypes = [C.POINTER(Params), C.c_int32]
@@ -123,7 +124,7 @@ def _lib():
         for name in EXPORTS:
             if name not in ("vsa2_strerror", "vsa2_route_scores", "vsa2_launch_count", "vsa2_last_cuda_error", "vsa2_selftest_divmod",
                             "vsa2_gate_bwd_workspace_bytes", "vsa2_attn_bwd_preferred_workspace_bytes",
-                            "vsa2_attn_bwd_scratch_bytes"):
+                            "vsa2_attn_bwd_scratch_bytes", "vsa2_route_scratch_bytes"):
                 getattr(lib, name).restype = C.c_int
         _LIB = lib
     return _LIB
@@ -178,10 +179,20 @@ def vsa2_query_sizes(p: Params) -> Sizes:
     return s
 
 
-def vsa2_route(p, q, k, budgets, vmap: Map, workspace, workspace_bytes=None, stream=None):
+def vsa2_route(p, q, k, budgets, vmap: Map, workspace, workspace_bytes=None, stream=None, scratch=None):
+    """`scratch`: None, or a tensor of at least vsa2_route_scratch_bytes(p) bytes (large problems run faster with it)."""
     nbytes = workspace_bytes if workspace_bytes is not None else workspace.numel() * workspace.element_size()
-    _check(_lib().vsa2_route(C.byref(p), _ptr(q), _ptr(k), _ptr(budgets), C.byref(vmap), _ptr(workspace), nbytes,
-                             _stream(stream)), "vsa2_route")
+    args = (C.byref(p), _ptr(q), _ptr(k), _ptr(budgets), C.byref(vmap), _ptr(workspace), nbytes)
+    if scratch is None:
+        _check(_lib().vsa2_route(*args, _stream(stream)), "vsa2_route")
+    else:
+        _check(_lib().vsa2_route_scratch(*args, _ptr(scratch), scratch.numel() * scratch.element_size(), _stream(stream)),
+               "vsa2_route_scratch")
+
+
+def vsa2_route_scratch_bytes(p) -> int:
+    """Bytes of scratch with which the router runs fastest (0: it has no use for any)."""
+    return int(_lib().vsa2_route_scratch_bytes(C.byref(p)))
 
 
 def vsa2_route_noalloc(p, q, k, budgets, vmap: Map, device_status=None, stream=None):
@@ -303,6 +314,8 @@ class Vsa2Attention:
         u8 = dict(dtype=torch.uint8, device=dev)
         self.ws_route = torch.empty(s.route_workspace_bytes, **u8)
         self.ws_fwd = torch.empty(s.fwd_workspace_bytes, **u8)
+        # scratch of a route call (large problems: 0.05 - 0.3 GB), like the one below
+        self.route_scratch_bytes = vsa2_route_scratch_bytes(params)
         # scratch of a backward call, up to 8 GiB: taken from torch's allocator for the call and given back, so the handles of a
         # model share it and one that only runs forward has none; 0 = none (the dQ pass recomputes the score gradients).  Up to
         # 1 MiB (a toy grid, whose passes wait for the host) is part of the workspace instead: asking takes 3 us
@@ -334,7 +347,8 @@ class Vsa2Attention:
 
     # calls ----------------------------------------------------------------------------------
     def route(self, q, k, budgets=None, stream=None):
-        vsa2_route(self.p, q, k, budgets, self.map, self.ws_route, stream=stream)
+        vsa2_route(self.p, q, k, budgets, self.map, self.ws_route, stream=stream,
+                   scratch=self._scratch("route_scratch_bytes", q.device, stream))
 
     def forward(self, q, k, v, gate, o=None, lse=None, stream=None):
         torch, p = self.torch, self.p
@@ -356,12 +370,13 @@ class Vsa2Attention:
         if dgate is None:      # video tokens only (text tokens have no gate)
             dgate = torch.empty(q.shape[:-2] + (self.sizes.seq_len,), dtype=torch.float32, device=q.device)
         vsa2_attn_bwd(p, q, k, v, gate, self.map, o, lse, self.saved, d_o, dq, dk, dv, dgate, self.ws_bwd, stream=stream,
-                      scratch=self._bwd_scratch(q.device, stream))
+                      scratch=self._scratch("bwd_scratch_bytes", q.device, stream))
         return dq, dk, dv, dgate
 
-    def _bwd_scratch(self, device, stream):
-        """Scratch for one call, allocated on the stream the call runs on (its memory is then reused in that stream's order)."""
-        torch, n = self.torch, self.bwd_scratch_bytes
+    def _scratch(self, size, device, stream):
+        """Scratch for one call of the bytes in attribute `size`, allocated on the stream the call runs on (its memory is then reused in
+        that stream's order)."""
+        torch, n = self.torch, getattr(self, size)
         if n == 0:
             return None
         try:
@@ -372,7 +387,7 @@ class Vsa2Attention:
             with torch.cuda.stream(stream):
                 return torch.empty(n, dtype=torch.uint8, device=device)
         except torch.cuda.OutOfMemoryError:     # not asked for again: a failing request makes the allocator empty its cache
-            self.bwd_scratch_bytes = 0
+            setattr(self, size, 0)
             return None
 
     def check_status(self, stream=None):

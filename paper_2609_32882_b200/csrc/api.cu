@@ -219,6 +219,29 @@ WideBwdLayout wide_bwd_layout(const Geo& g) {
   return r;
 }
 
+// One-pass router (router_tc.cu): half-cubes, or 64-token cubes, of eight sub-cubes.  Its scratch, from kRouterOneTiles key tiles on,
+// for the SMs of a B200.  Below, the launches that settle the map (4 per query, 11 per sequence) cost more than the exponentials:
+// whole route call, two-pass / one-pass, us: 7,056 tiles (336 cubes, 16 heads of 64 channels) 189 / 208; 7,776 tiles (288 cubes, 24
+// heads) 203 / 223; 18,252 tiles (624 cubes, 12 heads) 322 / 273; 81,000 tiles (1440 cubes, 10 heads) 1145 / 873.
+constexpr long long kRouterOneTiles = 12000;
+constexpr int kRouterOneSms = 148;
+constexpr int kSettlePairs = 1 << 17;      // pairs next to a threshold: about one in 10^5 of a problem's
+bool router_one_supported(const Geo& g) { return wide_cube(g) ? router_folds(g) && router_one_runs(narrow_geo(g)) : router_one_runs(g); }
+struct RouteOneLayout {
+  size_t park, lse2, pairs, rows, total;
+};
+RouteOneLayout route_one_layout(const Geo& g, int sms) {
+  const Geo r = wide_cube(g) ? narrow_geo(g) : g;
+  RouteOneLayout l;
+  Carver c;
+  l.park = c.take(router_one_park_bytes(r, router_folds(g), sms));
+  l.lse2 = c.take((size_t)g.batch * g.Hq * r.N * r.G * sizeof(float));
+  l.pairs = c.take((size_t)kSettlePairs * sizeof(int2));
+  l.rows = c.take((size_t)g.batch * g.Hq * g.N * sizeof(int));
+  l.total = c.off;
+  return l;
+}
+
 size_t route_workspace_bytes(const Geo& g) { return wide_cube(g) ? wide_route_layout(g).total : route_layout(g).total; }
 size_t fwd_base_bytes(const Geo& g) {
   return wide_cube(g) ? wide_fwd_layout(g).total : align_up(fwd_pooled_offset() + pooled_layout(g, false).total, 256);
@@ -428,6 +451,19 @@ size_t vsa2_attn_bwd_preferred_workspace_bytes(const vsa2_params* p) {
 
 int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets, const vsa2_map* map,
                void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  return vsa2_route_scratch(p, q, k, budgets, map, workspace, workspace_bytes, nullptr, 0, cuda_stream);
+}
+
+size_t vsa2_route_scratch_bytes(const vsa2_params* p) {
+  Geo g;
+  if (fill_geo(p, &g) != VSA2_OK || !router_one_supported(g)) return 0;
+  const Geo r = wide_cube(g) ? narrow_geo(g) : g;
+  const long long tiles = ((long long)r.N * r.G + 127) / 128;
+  return g.batch * g.Hq * tiles * tiles >= kRouterOneTiles ? route_one_layout(g, kRouterOneSms).total : 0;
+}
+
+int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets, const vsa2_map* map,
+                       void* workspace, size_t workspace_bytes, void* scratch, size_t scratch_bytes, void* cuda_stream) {
   Geo g;
   int rc = fill_geo(p, &g);
   if (rc != VSA2_OK) return rc;
@@ -435,7 +471,7 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
     return VSA2_ERR_INVALID_ARG;
   if (g.mode == VSA2_PER_QUERY_BUDGET && budgets == nullptr) return VSA2_ERR_INVALID_ARG;
   if (g.mode == VSA2_PER_QUERY_BUDGET && (g.flags & VSA2_FLAG_GROUP_ROUTING)) return VSA2_ERR_UNSUPPORTED;
-  if (!aligned16(q) || !aligned16(k) || !aligned256(workspace)) return VSA2_ERR_MISALIGNED;
+  if (!aligned16(q) || !aligned16(k) || !aligned256(workspace) || !aligned256(scratch)) return VSA2_ERR_MISALIGNED;
   if (workspace_bytes < route_workspace_bytes(g)) return VSA2_ERR_WORKSPACE_TOO_SMALL;
   if ((rc = check_device()) != VSA2_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
@@ -460,9 +496,19 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
     VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, status, st));
   }
   float* pr = folded ? at<float>(sel_base, lay.pr) : at<float>(workspace, rl.pr);
-  if (router_tc_supported(r))
-    VSA2_CUDA(launch_router_scores_tc(r, folded, qr, kr, pr, status, st));
-  else   // sub-cube counts the tensor-core kernel has no layout for (G = 1 is the VSA router of Sec. 2.1)
+  int sms = 0;
+  VSA2_CUDA(sm_count(&sms));
+  const bool group_sum = (g.flags & VSA2_FLAG_GROUP_ROUTING) && g.rep > 1;
+  const RouteOneLayout ol = router_one_supported(g) ? route_one_layout(g, sms) : RouteOneLayout{};
+  const bool one = router_one_supported(g) && scratch != nullptr && scratch_bytes >= ol.total;
+  int* redo = one ? &status->pad[0] : nullptr;      // (the status block is cleared by the pooling)
+  float* lse2 = one ? at<float>(scratch, ol.lse2) : nullptr;
+  if (router_tc_supported(r)) {
+    { ProfScope lse(VSA2_KERNEL_ROUTER_LSE, st, 0); }      // (both passes are timed as the second)
+    ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);
+    if (one) VSA2_CUDA(launch_router_one(r, folded, qr, kr, pr, at<unsigned char>(scratch, ol.park), lse2, redo, status, st));
+    else VSA2_CUDA(launch_router_scores_tc(r, folded, qr, kr, pr, nullptr, status, st));
+  } else   // sub-cube counts the tensor-core kernel has no layout for (G = 1 is the VSA router of Sec. 2.1)
     VSA2_CUDA(launch_router_scores(r, qr, kr, at<float>(workspace, rl.lse_r), pr, st));
   if (wide && !folded) {
     g_launches += 1;
@@ -470,9 +516,9 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
     VSA2_CUDA(launch_fold_scores(r, pr, pr_cube, st));
     pr = pr_cube;
   }
-  if ((g.flags & VSA2_FLAG_GROUP_ROUTING) && g.rep > 1) {
+  if (group_sum) {
     g_launches += 1;
-    VSA2_CUDA(launch_group_sum_scores(g, pr, st));
+    VSA2_CUDA(launch_group_sum_scores(g, pr, nullptr, st));
   }
   workspace = sel_base;
   SelectScratch s;
@@ -488,7 +534,17 @@ int vsa2_route(const vsa2_params* p, const void* q, const void* k, const int32_t
   s.words = lay.words;
   {
     ProfScope ps(VSA2_KERNEL_SELECT, st, (g.mode == VSA2_PER_SEQUENCE ? 14 : 7) - (g.N <= kSelOneBlockN ? 5 : 0));
-    VSA2_CUDA(launch_select(g, pr, budgets, s, map->row_ptr, map->col_idx, map->col_ptr, map->row_idx, status, st));
+    if (one) {
+      const Settle se{redo, &status->pad[1], at<int2>(scratch, ol.pairs), kSettlePairs, &status->pad[2], at<int>(scratch, ol.rows)};
+      g_launches += (g.mode == VSA2_PER_SEQUENCE ? 8 : 1) + 3 + (group_sum ? 1 : 0);
+      VSA2_CUDA(launch_select_band(g, pr, budgets, s, se, st));
+      VSA2_CUDA(launch_router_exact(r, folded, qr, kr, lse2, se.pairs, se.count, se.cap, group_sum ? g.rep : 1, redo, pr, status, st));
+      VSA2_CUDA(launch_select_settle(g, pr, budgets, s, se, st));
+      // (these and the thresholds of launch_select return at once unless the flag is up)
+      VSA2_CUDA(launch_router_scores_tc(r, folded, qr, kr, pr, redo, status, st));
+      if (group_sum) VSA2_CUDA(launch_group_sum_scores(g, pr, redo, st));
+    }
+    VSA2_CUDA(launch_select(g, pr, budgets, s, redo, map->row_ptr, map->col_idx, map->col_ptr, map->row_idx, status, st));
   }
   return VSA2_OK;
 }

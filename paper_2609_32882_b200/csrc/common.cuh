@@ -207,8 +207,16 @@ cudaError_t launch_router_scores(const Geo& g, const bf16* qr, const bf16* kr, f
 // tensor-core router (router_tc.cu), both passes in one launch; with `fold` (half-cubes of 8 sub-cubes, N even) the scores
 // come out at the level of the 128-token cubes, bit for bit what launch_fold_scores makes of the others
 bool router_tc_supported(const Geo& g);
-cudaError_t launch_router_scores_tc(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, StatusBlock* status,
+// (`redo`: null, or the flag without which the launch does nothing)
+cudaError_t launch_router_scores_tc(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, int* redo, StatusBlock* status,
                                     cudaStream_t st);
+// the one-pass form and the two-pass scores of listed pairs (router_tc.cu), where router_one_runs
+bool router_one_runs(const Geo& g);
+size_t router_one_park_bytes(const Geo& g, bool fold, int sms);
+cudaError_t launch_router_one(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, void* park, float* lse2, int* redo,
+                              StatusBlock* status, cudaStream_t st);
+cudaError_t launch_router_exact(const Geo& g, bool fold, const bf16* qr, const bf16* kr, const float* lse2, const int2* pairs,
+                                const int* count, int cap, int heads, const int* redo, float* pr, StatusBlock* status, cudaStream_t st);
 
 // up to this many cubes one block per head turns the selection into both maps (select.cu): 128 cubes 4.7 us against 12 us and
 // five more launches; at 288 cubes the block takes 40 us and the six launches 18
@@ -225,7 +233,21 @@ struct SelectScratch {
   unsigned* bitmap_t;    // [BH][N][words]   columns x row words
   int words;             // ceil(N/32)
 };
-cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s,
+// Selection on one-pass scores (select.cu): thresholds and the lists of what lies next to them (launch_select_band), the two-pass
+// scores of those (launch_router_exact), the decision (launch_select_settle); then launch_select with `redo`, which finds
+// everything in place or, should the flag be up, starts again from two-pass scores.
+struct Settle {
+  int* redo;           // raised when the two-pass form has to be run after all
+  int* count;          // listed pairs
+  int2* pairs;         // [cap] {(batch * Hq + head) * N + row, column}
+  int cap;
+  int* row_count;      // per-row modes: listed rows
+  int* rows;           // [B * Hq * N]
+};
+cudaError_t launch_select_band(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st);
+cudaError_t launch_select_settle(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se,
+                                 cudaStream_t st);
+cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const int* redo,
                           int* row_ptr, int* col_idx, int* col_ptr, int* row_idx, StatusBlock* status,
                           cudaStream_t st);
 
@@ -255,7 +277,7 @@ bool wide_cube(const Geo& g);
 Geo narrow_geo(const Geo& g);
 cudaError_t launch_fold_scores(const Geo& narrow, const float* pr64, float* pr, cudaStream_t st);
 // "group head" routing: replaces every block score by the sum over the query heads of its KV group (in place)
-cudaError_t launch_group_sum_scores(const Geo& g, float* pr, cudaStream_t st);
+cudaError_t launch_group_sum_scores(const Geo& g, float* pr, const int* redo, cudaStream_t st);      // (`redo`: null, or the flag without which nothing happens)
 cudaError_t launch_fold_mean(const Geo& narrow, int heads, const float* x64, float* x, cudaStream_t st);
 cudaError_t launch_fold_sum(const Geo& narrow, int heads, const float* x64, float* x, cudaStream_t st);
 cudaError_t launch_expand_rows(const Geo& narrow, int heads, bool by_count, const float* x, float* x64,

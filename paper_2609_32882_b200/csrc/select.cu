@@ -14,7 +14,8 @@ __device__ __forceinline__ int seq_shift(int pass) { return pass == 0 ? 21 : (pa
 __device__ __forceinline__ unsigned seq_mask(int pass) { return pass == 2 ? 0x3FFu : 0x7FFu; }
 
 // state[bh*8 + ..]: 0 prefix bits, 1 prefix mask, 2 remaining k, 3 tau bits, 4 eq_take
-__global__ void sel_init_kernel(unsigned* state, unsigned* hist, int BH, unsigned keep) {
+__global__ void sel_init_kernel(unsigned* state, unsigned* hist, int BH, unsigned keep, const int* redo) {
+  if (redo != nullptr && *redo == 0) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < BH * 3 * kHistBins) hist[i] = 0u;
   if (i < BH) {
@@ -27,8 +28,10 @@ __global__ void sel_init_kernel(unsigned* state, unsigned* hist, int BH, unsigne
 }
 
 __global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__ pr, long long n_elems,
-                                                       const unsigned* __restrict__ state, unsigned* hist, int pass) {
+                                                       const unsigned* __restrict__ state, unsigned* hist, int pass,
+                                                       const int* redo) {
   __shared__ unsigned sh[kHistBins];
+  if (redo != nullptr && *redo == 0) return;
   const int bh = blockIdx.y;
   for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) sh[i] = 0u;
   __syncthreads();
@@ -65,7 +68,8 @@ __global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__
 
 // One warp per (batch, head): finds the digit whose bin holds the `remaining`-th largest entry.  Lane l owns the bins
 // [l * nb/32, (l+1) * nb/32); a suffix sum over the lanes locates the lane, a short serial walk the bin.
-__global__ void __launch_bounds__(32) sel_pick_kernel(unsigned* state, const unsigned* hist, int pass) {
+__global__ void __launch_bounds__(32) sel_pick_kernel(unsigned* state, const unsigned* hist, int pass, const int* redo) {
+  if (redo != nullptr && *redo == 0) return;
   const int bh = blockIdx.x, lane = threadIdx.x;
   const unsigned* hsrc = hist + ((size_t)bh * 3 + pass) * kHistBins;
   const unsigned remaining0 = state[bh * 8 + 2];
@@ -111,16 +115,41 @@ __global__ void __launch_bounds__(32) sel_pick_kernel(unsigned* state, const uns
   }
 }
 
+// ---- scores of the one-pass router -----------------------------------------------------------------------------------------
+// A one-pass score x stands for a two-pass score within a factor 1 +- e.  With t the K-th largest x, entries above t (1 + 2e) are
+// among the K largest two-pass scores and entries below t (1 - 2e) are not, so only those between -- the band -- need their
+// two-pass scores, and only where the band holds more entries than are still wanted.
+// e: of a term that counts in a score of at least kBandLeast = 2^-60, either form rounds an exponent below 128 once (half an ulp,
+// 2^-18); the one-pass form also rounds the growth of the row's maximum, at most 64 (2^-19), while its reference against the
+// denominator keeps what rounding takes from it (router_tc.cu).  (2 2^-18 + 2^-19) ln 2 = 6.6e-6, and with five approximations of
+// ex2 (2^-22 each) and at most 40 additions of 2^-24 on either side less than 1.4e-5.  kBandUlps = 512 units of the last place of t
+// are at least 3.05e-5 of t, more than 2e.
+// Smaller thresholds go back to the two-pass form if their band matters.  About one entry in 10^5 lies in a band.
+constexpr unsigned kBandUlps = 512, kBandLeast = 0x21800000u, kBandMost = 0x7f000000u;
+__device__ __forceinline__ unsigned band_lo(unsigned tau) { return tau > kBandUlps ? tau - kBandUlps : 0u; }
+__device__ __forceinline__ unsigned band_hi(unsigned tau) { return tau < 0xffffffffu - kBandUlps ? tau + kBandUlps : 0xffffffffu; }
+__device__ __forceinline__ bool band_usable(unsigned tau) { return tau >= kBandLeast && tau <= kBandMost; }
+constexpr int kBandHead = 2048;      // entries of a head's band that sel_settle_kernel ranks
+__device__ __forceinline__ void settle_list(const Settle& se, int row, int column) {
+  const int at = atomicAdd(se.count, 1);
+  if (at < se.cap) se.pairs[at] = make_int2(row, column);
+  else atomicExch(se.redo, 1);
+}
+
 // per-sequence, one read of P_r for both the counts and the emission: one warp per row writes the row's bitmap words of the
 // entries above tau (`bits_gt`) and equal to tau (`bits_eq`) and the two counts.  grid (ceil(N/8), BH), 256 threads
+// BAND: entries above and in the band instead, the latter also listed for router_exact_kernel.
+template <bool BAND>
 __global__ void __launch_bounds__(256) sel_row_bits_kernel(const float* __restrict__ pr, int N, int words,
                                                            const unsigned* __restrict__ state, unsigned* bits_gt,
-                                                           unsigned* bits_eq, int* row_gt, int* row_eq) {
+                                                           unsigned* bits_eq, int* row_gt, int* row_eq, Settle se) {
+  if (!BAND && se.redo != nullptr && *se.redo == 0) return;
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int bh = blockIdx.y;
   if (i >= N) return;
   const unsigned tau = state[bh * 8 + 3];
+  const unsigned hi = BAND ? band_hi(tau) : tau, lo = BAND ? band_lo(tau) : tau;
   const unsigned* src = reinterpret_cast<const unsigned*>(pr) + ((size_t)bh * N + i) * N;
   int gt = 0, eq = 0;
   constexpr int U = 8;                 // words in flight per warp (the kernel is a pure streaming read)
@@ -135,11 +164,13 @@ __global__ void __launch_bounds__(256) sel_row_bits_kernel(const float* __restri
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = (w0 + u) * 32 + lane;
-      const unsigned gb = __ballot_sync(0xffffffffu, j < N && v[u] > tau);
-      const unsigned eb = __ballot_sync(0xffffffffu, j < N && v[u] == tau);
+      const bool in = j < N && v[u] >= lo && v[u] <= hi;
+      const unsigned gb = __ballot_sync(0xffffffffu, j < N && v[u] > hi);
+      const unsigned eb = __ballot_sync(0xffffffffu, in);
       if (lane == u) { mine_g = gb; mine_e = eb; }
       gt += __popc(gb);
       eq += __popc(eb);
+      if (BAND && in) settle_list(se, bh * N + i, j);
     }
     if (lane < U && w0 + lane < words) {       // lanes 0..U-1 write one word each: consecutive addresses
       bits_gt[((size_t)bh * N + i) * words + w0 + lane] = mine_g;
@@ -218,14 +249,18 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
 // (a block per row with 8-bit histograms: 104 us for 7,488 rows of 624, most of it one thread walking the bins)
 // U is the smallest of 8, 20, 32, 48, 64 that holds the row: a round costs U compares whatever the row's length, so the forms are
 // close enough together (1.3 - 1.6 times, below 640 entries 2.5) for the padding not to outweigh the launch.
-template <int U>
+// MODE kBand: a row whose band holds more entries than it still wants is listed (se.rows), and its band's entries (se.pairs).
+// MODE kListed: the listed rows alone, now with their two-pass scores (any grid).
+constexpr int kAllRows = 0, kBand = 1, kListed = 2;
+template <int U, int MODE>
 __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __restrict__ pr, int N, int K,
                                                                 const int* __restrict__ budgets, float* row_tau,
-                                                                int* row_eq_take, int* row_cnt) {
-  const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y;
-  if (i >= N) return;
-  const unsigned* src = reinterpret_cast<const unsigned*>(pr) + ((size_t)bh * N + i) * N;
-  const size_t o = (size_t)bh * N + i;
+                                                                int* row_eq_take, int* row_cnt, Settle se) {
+  if (MODE == kAllRows && se.redo != nullptr && *se.redo == 0) return;
+  const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= (MODE == kListed ? *se.row_count : N)) return;
+  const size_t o = MODE == kListed ? (size_t)se.rows[i] : (size_t)blockIdx.y * N + i;
+  const unsigned* src = reinterpret_cast<const unsigned*>(pr) + o * N;
   unsigned v[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) v[u] = u * 32 + lane < N ? __ldg(src + u * 32 + lane) : 0u;      // (0 is never above a candidate)
@@ -260,22 +295,42 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __r
     row_eq_take[o] = k - gt;
     row_cnt[o] = k;
   }
+  if constexpr (MODE == kBand) {
+    const unsigned lo = band_lo(tau), hi = band_hi(tau);
+    int from = 0;                     // entries above the lower end of the band: more than k, and the band matters
+#pragma unroll
+    for (int u = 0; u < U; ++u) from += u * 32 + lane < N && v[u] >= lo;
+    from = __reduce_add_sync(0xffffffffu, from);
+    if (from > k) {
+      if (lane == 0) {
+        if (band_usable(tau)) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
+        else atomicExch(se.redo, 1);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (u * 32 + lane < N && v[u] >= lo && v[u] <= hi) settle_list(se, (int)o, u * 32 + lane);
+    }
+  }
 }
 
 // per-row modes, rows of more than 2048 entries: radix select of the k_i-th largest of row i.  grid (N, BH), 256 threads
+// MODE as above
+template <int MODE>
 __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restrict__ pr, int N, int K,
                                                            const int* __restrict__ budgets, float* row_tau,
-                                                           int* row_eq_take, int* row_cnt) {
+                                                           int* row_eq_take, int* row_cnt, Settle se) {
   __shared__ unsigned sh[256];
   __shared__ unsigned s_prefix, s_mask, s_remaining;
-  const int i = blockIdx.x, bh = blockIdx.y;
-  const unsigned* src = reinterpret_cast<const unsigned*>(pr) + ((size_t)bh * N + i) * N;
-  int k = budgets ? budgets[(size_t)bh * N + i] : K;
+  if (MODE == kAllRows && se.redo != nullptr && *se.redo == 0) return;
+  const size_t listed = MODE == kListed ? (size_t)*se.row_count : 1;
+  for (size_t n = MODE == kListed ? blockIdx.x : 0; n < listed; n += gridDim.x) {
+  const size_t o = MODE == kListed ? (size_t)se.rows[n] : (size_t)blockIdx.y * N + blockIdx.x;
+  const unsigned* src = reinterpret_cast<const unsigned*>(pr) + o * N;
+  int k = budgets ? budgets[o] : K;
   k = max(0, min(k, N));
-  const size_t o = (size_t)bh * N + i;
   if (k == 0) {
     if (threadIdx.x == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
-    return;
+    continue;
   }
   if (threadIdx.x == 0) { s_prefix = 0u; s_mask = 0u; s_remaining = (unsigned)k; }
   for (int pass = 0; pass < 4; ++pass) {
@@ -302,10 +357,32 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restri
     }
     __syncthreads();
   }
+  const unsigned tau = s_prefix;
   if (threadIdx.x == 0) {
-    row_tau[o] = __uint_as_float(s_prefix);
+    row_tau[o] = __uint_as_float(tau);
     row_eq_take[o] = (int)s_remaining;
     row_cnt[o] = k;
+  }
+  if constexpr (MODE == kBand) {
+    const unsigned lo = band_lo(tau), hi = band_hi(tau);
+    int from = 0;
+    for (int j = threadIdx.x; j < N; j += blockDim.x) from += __ldg(src + j) >= lo;
+    if (threadIdx.x == 0) sh[0] = 0u;
+    __syncthreads();
+    if (from > 0) atomicAdd(&sh[0], (unsigned)from);
+    __syncthreads();
+    if (sh[0] > (unsigned)k) {
+      if (threadIdx.x == 0) {
+        if (band_usable(tau)) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
+        else atomicExch(se.redo, 1);
+      }
+      for (int j = threadIdx.x; j < N; j += blockDim.x) {
+        const unsigned v = __ldg(src + j);
+        if (v >= lo && v <= hi) settle_list(se, (int)o, j);
+      }
+    }
+  }
+  __syncthreads();
   }
 }
 
@@ -490,6 +567,69 @@ __global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __re
   }
 }
 
+// per-sequence, one-pass scores: of every head whose band holds more entries than are still wanted, ranks the band by its two-pass
+// scores (ties to the lower index) and takes what is not kept out of the bitmap and the counts.  One block per head.
+__global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restrict__ pr, int N, int words, unsigned keep, unsigned* state,
+                                                          const int* __restrict__ row_gt, int* row_eq, unsigned* bits_eq, Settle se) {
+  __shared__ int ws[33];
+  __shared__ int at[kBandHead], n_rows;
+  __shared__ unsigned val[kBandHead];
+  __shared__ int2 rows[kBandHead];          // (no more than entries)
+  const int bh = blockIdx.x, tid = threadIdx.x;
+  const size_t base = (size_t)bh * N;
+  int above = 0, band = 0, tot;
+  for (int i = tid; i < N; i += blockDim.x) {
+    above += row_gt[base + i];
+    band += row_eq[base + i];
+  }
+  block_excl_scan(above, ws, tot);
+  const int need = (int)keep - tot;
+  block_excl_scan(band, ws, band);
+  if (tid == 0) state[bh * 8 + 4] = (unsigned)need;
+  if (band == need) return;
+  if (band > kBandHead || !band_usable(state[bh * 8 + 3])) {
+    if (tid == 0) atomicExch(se.redo, 1);
+    return;
+  }
+  // the rows that have such entries and the place of their first; then a warp per row, a lane per word of its bitmap
+  if (tid == 0) n_rows = 0;
+  int carry = 0;
+  for (int i0 = 0; i0 < N; i0 += blockDim.x) {
+    const int i = i0 + tid, eq = i < N ? row_eq[base + i] : 0;
+    const int pos = carry + block_excl_scan(eq, ws, tot);
+    carry += tot;
+    if (eq > 0) rows[atomicAdd(&n_rows, 1)] = make_int2(i, pos);
+  }
+  __syncthreads();
+  const int lane = tid & 31;
+  for (int r = tid >> 5; r < n_rows; r += blockDim.x >> 5) {
+    const int i = rows[r].x;
+    int pos = rows[r].y;
+    for (int w0 = 0; w0 < words; w0 += 32) {
+      const unsigned bits = w0 + lane < words ? bits_eq[(base + i) * words + w0 + lane] : 0u;
+      const int c = __popc(bits), incl = warp_incl_scan(c, lane);
+      int p = pos + incl - c;
+      for (unsigned b = bits; b != 0u; b &= b - 1u, ++p) {
+        const int j = (w0 + lane) * 32 + (__ffs(b) - 1);
+        at[p] = i * N + j;
+        val[p] = __float_as_uint(pr[(base + i) * N + j]);
+      }
+      pos += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < band; e += blockDim.x) {
+    const unsigned v = val[e];
+    int rank = 0;
+    for (int f = 0; f < band; ++f) rank += val[f] > v || (val[f] == v && f < e);
+    if (rank >= need) {
+      const int i = at[e] / N, j = at[e] - i * N;
+      atomicAnd(&bits_eq[(base + i) * words + (j >> 5)], ~(1u << (j & 31)));
+      atomicSub(&row_eq[base + i], 1);
+    }
+  }
+}
+
 // Up to kSelOneBlockN cubes: everything behind the counts of the kept entries in one launch, a block per head with both bitmaps in
 // shared memory (the six launches below take 2 us and a gap each and keep a few SMs busy).  Same rules: rows in order, ties at the
 // threshold to the lower column, both maps cut at the capacity.
@@ -604,32 +744,66 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* __restrict_
   }
 }
 
-cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, int* row_ptr,
-                          int* col_idx, int* col_ptr, int* row_idx, StatusBlock* status, cudaStream_t st) {
+template <int MODE>
+static void launch_row_topk(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
   const int BH = g.batch * g.Hq, N = g.N;
-  const long long n_elems = (long long)N * N;
+  const int* bud = g.mode == VSA2_PER_QUERY_BUDGET ? budgets : nullptr;
+  const dim3 grid = MODE == kListed ? dim3((unsigned)(((long long)BH * N + 7) / 8)) : dim3((N + 7) / 8, BH);
+#define VSA2_ROW_TOPK(U) sel_row_topk_warp_kernel<U, MODE><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt, se)
+  if (N <= 256) VSA2_ROW_TOPK(8);
+  else if (N <= 640) VSA2_ROW_TOPK(20);
+  else if (N <= 1024) VSA2_ROW_TOPK(32);
+  else if (N <= 1536) VSA2_ROW_TOPK(48);
+  else if (N <= 2048) VSA2_ROW_TOPK(64);
+  else
+    sel_row_topk_kernel<MODE><<<MODE == kListed ? dim3(592) : dim3(N, BH), 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt, se);
+#undef VSA2_ROW_TOPK
+}
+
+// thresholds, counts and (per sequence) bitmaps of all heads; `se.redo`: null, or the flag without which nothing happens
+template <bool BAND>
+static void launch_thresholds(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
+  const int BH = g.batch * g.Hq, N = g.N;
   if (g.mode == VSA2_PER_SEQUENCE) {
+    const long long n_elems = (long long)N * N;
     const unsigned keep = (unsigned)((long long)N * g.K);
+    const int* redo = BAND ? nullptr : se.redo;
     int init_n = BH * 3 * kHistBins;
-    sel_init_kernel<<<(init_n + 255) / 256, 256, 0, st>>>(s.state, s.hist, BH, keep);
+    sel_init_kernel<<<(init_n + 255) / 256, 256, 0, st>>>(s.state, s.hist, BH, keep, redo);
     int chunks = (int)((n_elems + 256 * 16 - 1) / (256 * 16));
     if (chunks > 256) chunks = 256;
     for (int pass = 0; pass < 3; ++pass) {
-      sel_hist_kernel<<<dim3(chunks, BH), 256, 0, st>>>(pr, n_elems, s.state, s.hist, pass);
-      sel_pick_kernel<<<BH, 32, 0, st>>>(s.state, s.hist, pass);
+      sel_hist_kernel<<<dim3(chunks, BH), 256, 0, st>>>(pr, n_elems, s.state, s.hist, pass, redo);
+      sel_pick_kernel<<<BH, 32, 0, st>>>(s.state, s.hist, pass, redo);
     }
     // counts and bitmaps in one read of P_r (the bitmap of the entries equal to tau borrows the transposed bitmap's space)
-    sel_row_bits_kernel<<<dim3((N + 7) / 8, BH), 256, 0, st>>>(pr, N, s.words, s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq);
+    sel_row_bits_kernel<BAND><<<dim3((N + 7) / 8, BH), 256, 0, st>>>(pr, N, s.words, s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq, se);
   } else {
-    const int* bud = g.mode == VSA2_PER_QUERY_BUDGET ? budgets : nullptr;
-    const dim3 grid((N + 7) / 8, BH);
-    if (N <= 256) sel_row_topk_warp_kernel<8><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
-    else if (N <= 640) sel_row_topk_warp_kernel<20><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
-    else if (N <= 1024) sel_row_topk_warp_kernel<32><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
-    else if (N <= 1536) sel_row_topk_warp_kernel<48><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
-    else if (N <= 2048) sel_row_topk_warp_kernel<64><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
-    else sel_row_topk_kernel<<<dim3(N, BH), 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt);
+    launch_row_topk<BAND ? kBand : kAllRows>(g, pr, budgets, s, se, st);
   }
+}
+
+cudaError_t launch_select_band(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
+  launch_thresholds<true>(g, pr, budgets, s, se, st);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_select_settle(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se,
+                                 cudaStream_t st) {
+  const int BH = g.batch * g.Hq, N = g.N;
+  if (g.mode == VSA2_PER_SEQUENCE)
+    sel_settle_kernel<<<BH, 1024, 0, st>>>(pr, N, s.words, (unsigned)((long long)N * g.K), s.state, s.row_gt, s.row_eq, s.bitmap_t, se);
+  else
+    launch_row_topk<kListed>(g, pr, budgets, s, se, st);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const int* redo, int* row_ptr,
+                          int* col_idx, int* col_ptr, int* row_idx, StatusBlock* status, cudaStream_t st) {
+  const int BH = g.batch * g.Hq, N = g.N;
+  Settle se{};
+  se.redo = const_cast<int*>(redo);
+  launch_thresholds<false>(g, pr, budgets, s, se, st);
   if (N <= kSelOneBlockN) {
     sel_maps_kernel<<<BH, 1024, 0, st>>>(pr, N, s.words, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
                                          s.row_eq_take, s.row_cnt, s.bitmap, s.bitmap_t, row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap,

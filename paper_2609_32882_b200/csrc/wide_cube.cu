@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(128) extend_map_kernel(int Nvid, int NtB, int 
 
 // "group head" routing: the query heads of a KV group share one map.  pr [batch, Hq, N, N]: every entry is replaced by
 // the sum over the heads of its group (added in head order), so the selection that follows picks the same set for each
-__global__ void __launch_bounds__(256) group_sum_scores_kernel(float* __restrict__ pr, int rep, size_t per_head, size_t groups) {
+__global__ void __launch_bounds__(256) group_sum_scores_kernel(float* __restrict__ pr, int rep, size_t per_head, size_t groups,
+                                                               const int* redo) {
+  if (redo != nullptr && *redo == 0) return;
   const size_t total = groups * per_head;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const size_t grp = e / per_head, off = e % per_head;
@@ -176,9 +178,9 @@ int grid_for(size_t total) {
 
 }  // namespace
 
-cudaError_t launch_group_sum_scores(const Geo& g, float* pr, cudaStream_t st) {
+cudaError_t launch_group_sum_scores(const Geo& g, float* pr, const int* redo, cudaStream_t st) {
   const size_t per_head = (size_t)g.N * g.N, groups = (size_t)g.batch * g.Hkv;
-  group_sum_scores_kernel<<<grid_for(groups * per_head), 256, 0, st>>>(pr, g.rep, per_head, groups);
+  group_sum_scores_kernel<<<grid_for(groups * per_head), 256, 0, st>>>(pr, g.rep, per_head, groups, redo);
   return cudaGetLastError();
 }
 

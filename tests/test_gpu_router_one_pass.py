@@ -1,0 +1,93 @@
+"""The router that forms every exponential once (with scratch) against the one that forms them twice (without): the same maps bit
+for bit, the same scores but for their last bits, and at the thresholds the very scores -- for every way to select, shared maps,
+cubes of 128 tokens, grids that are ragged in every dimension, and inputs on which the one-pass form stands back (ties by the
+thousand, scores that climb beyond the range of a parked sum, thresholds next to zero)."""
+import pytest
+import torch
+
+from paper_2609_32882_b200 import binding as vb
+
+pytestmark = pytest.mark.gpu
+SEQ, ROW, BUDGET = vb.PER_SEQUENCE, vb.PER_QUERY, vb.PER_QUERY_BUDGET
+WIDE = dict(cube=(4, 4, 8))
+
+# heads_q, heads_kv, D, grid, cube, mode, topk, flags, kind of input
+CASES = [
+    (2, 1, 64, (4, 8, 8), {}, SEQ, 2, 0, "random"),                              # one tile, one block builds the map
+    (3, 3, 128, (9, 30, 45), {}, SEQ, 16, 0, "random"),                          # 288 cubes, ragged
+    (12, 4, 64, (13, 27, 47), {}, ROW, 24, 0, "random"),
+    (4, 2, 128, (21, 30, 52), {}, BUDGET, 0, 0, "random"),
+    (12, 3, 128, (13, 30, 33), {}, ROW, 9, vb.FLAG_GROUP_ROUTING, "random"),     # scores summed over the heads of a group
+    (4, 2, 128, (21, 30, 52), {}, SEQ, 40, vb.FLAG_GROUP_ROUTING, "random"),
+    (3, 3, 128, (20, 18, 68), WIDE, SEQ, 12, 0, "random"),                       # trailing half-cubes without a token
+    (2, 1, 64, (24, 44, 88), WIDE, ROW, 30, 0, "random"),
+    (1, 1, 64, (40, 60, 60), {}, ROW, 100, 0, "random"),                         # rows of more than 2048 entries
+    (2, 2, 64, (16, 32, 32), {}, SEQ, 10, 0, "constant"),                        # every score ties
+    (2, 2, 64, (16, 32, 32), {}, ROW, 10, 0, "constant"),
+    (2, 2, 64, (16, 32, 32), {}, ROW, 7, 0, "halves"),                           # ties by the row, some at the threshold
+    (2, 2, 64, (28, 28, 28), {}, SEQ, 20, 0, "growing"),
+    (2, 2, 128, (28, 28, 32), WIDE, ROW, 20, 0, "growing"),
+    (2, 2, 64, (16, 32, 32), {}, SEQ, 200, 0, "peaked"),                         # thresholds below 2^-60
+    (2, 2, 64, (16, 32, 32), {}, ROW, 256, 0, "random"),                         # everything is kept
+]
+
+
+def _inputs(heads_q, heads_kv, dim, grid, kind):
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rows = grid[0] * grid[1] * grid[2]
+    q = torch.randn(1, heads_q, rows, dim, device="cuda", generator=gen)
+    k = torch.randn(1, heads_kv, rows, dim, device="cuda", generator=gen)
+    if kind == "random":
+        return (2.0 * q).bfloat16(), (2.0 * k).bfloat16()
+    if kind == "constant":
+        k = torch.ones_like(k)
+    elif kind == "halves":       # the second half of the frames repeats the first
+        half = rows // 2
+        k[:, :, half:] = k[:, :, :half]
+        q, k = 2.0 * q, 2.0 * k
+    elif kind == "growing":      # scores climb by 60 nats from the first frame to the last
+        t = torch.arange(rows, device="cuda") // (grid[1] * grid[2]) / (grid[0] - 1)
+        q[..., 0] = 4.0
+        k[..., 0] = (60.0 * dim ** 0.5 / 4.0 * t)[None, None, :]
+    elif kind == "peaked":
+        q, k = 24.0 * q, 24.0 * k
+    return q.bfloat16(), k.bfloat16()
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[0]}x{c[1]}_d{c[2]}_{'x'.join(map(str, c[3]))}_mode{c[5]}_{c[8]}_{c[7]}")
+def test_one_pass_maps_are_the_two_pass_maps(case):
+    heads_q, heads_kv, dim, grid, cube, mode, topk, flags, kind = case
+    n = -(-grid[0] // 4) * -(-grid[1] // 4) * -(-grid[2] // (8 if cube else 4))
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    budgets = torch.randint(0, 120, (1, heads_q, n), device="cuda", generator=gen, dtype=torch.int32) if mode == BUDGET else None
+    cap = int(budgets.clamp(max=n).sum(-1).max()) if mode == BUDGET else 0
+    p = vb.make_params(1, heads_q, heads_kv, dim, grid, select_mode=mode, topk=topk, flags=flags, nnz_cap=cap, **cube)
+    q, k = _inputs(heads_q, heads_kv, dim, grid, kind)
+    attn = vb.Vsa2Attention(p)
+    sub = 8 * n * (2 if cube else 1)
+    tiles = -(-sub // 128)
+    scratch = torch.empty(148 * tiles * 8192 + heads_q * (4 * sub + 4 * n) + (1 << 20) + 4096, dtype=torch.uint8, device="cuda")
+    scratch.fill_(0xff)                                          # (NaN wherever something is read before it is written)
+    out = []
+    for s in (None, scratch):
+        vb.vsa2_route(p, q, k, budgets, attn.map, attn.ws_route, scratch=s)
+        attn.check_status()
+        views = attn.map_views()
+        nnz = int(views[0][..., -1].max())
+        out.append(([views[0].clone(), views[1][..., :nnz].clone(), views[2].clone(), views[3][..., :nnz].clone()], attn.scores()))
+    (two_map, two), (one_map, one) = out
+    for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), two_map, one_map):
+        if mode != BUDGET or "ptr" in name:
+            assert torch.equal(x, y), name
+    if mode == BUDGET:                                           # (heads keep different numbers of entries)
+        for h in range(heads_q):
+            e = int(two_map[0][0, h, -1])
+            assert torch.equal(two_map[1][0, h, :e], one_map[1][0, h, :e]) and torch.equal(two_map[3][0, h, :e], one_map[3][0, h, :e])
+    # the bound derived in select.cu (scores below 2^-60 have none there)
+    counted = two >= 2.0 ** -60
+    assert ((one - two).abs() <= 1.4e-5 * two)[counted].all()
+    if mode == SEQ and kind == "random":
+        # the band of a head: its two-pass scores
+        tau = two.flatten(2).topk(n * topk, dim=-1).values[..., -1].view(torch.int32)[..., None, None]
+        band = (two.view(torch.int32) - tau).abs() <= 128        # (well inside the 512 units of the one-pass threshold)
+        assert band.sum() >= heads_q and torch.equal(one[band], two[band])

@@ -196,3 +196,15 @@ def test_gate_entry_points_reject_unsupported_shapes_before_any_cuda_call():
     assert vb.vsa2_gate_bwd_workspace_bytes(many, 64) == 0
     assert vb.vsa2_gate_bwd_workspace_bytes(p, 64) == 16 * 64 * 8 * 4 + 2 * 64 * 16 * 2      # dW_g partials + dz in two layouts
     assert lib.vsa2_gate_bwd(ctypes.byref(p), 64, one, one, one, one, one, one, one, 100, None) == vb.ERR_WORKSPACE_TOO_SMALL
+
+
+def test_route_scratch_is_checked_and_asked_for_by_large_problems_only():
+    lib = vb._lib()
+    small, large = vb.params_from_workload(syn.CONFIGS[0]), vb.params_from_workload(syn.CONFIGS[3])
+    assert vb.vsa2_route_scratch_bytes(small) == 0
+    assert 100 << 20 < vb.vsa2_route_scratch_bytes(large) < 150 << 20
+    s = vb.vsa2_query_sizes(large)
+    one, m = ctypes.c_void_p(256), vb.Map(256, 256, 256, 256)
+    args = [ctypes.byref(large), one, one, None, ctypes.byref(m), one]
+    assert lib.vsa2_route_scratch(*args, s.route_workspace_bytes, ctypes.c_void_p(128), 1 << 30, None) == vb.ERR_MISALIGNED
+    assert lib.vsa2_route_scratch(*args, s.route_workspace_bytes - 1, one, 1 << 30, None) == vb.ERR_WORKSPACE_TOO_SMALL
