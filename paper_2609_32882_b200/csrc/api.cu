@@ -20,7 +20,7 @@ struct RouteLayout {
   int words;
 };
 struct BwdLayout {
-  size_t status, delta, absmax, ds_exp, d_oc_hat, delta_c, dqc, dkc, dvc, pooled, total;
+  size_t status, delta, absmax, ds_exp, full, d_oc_hat, delta_c, dqc, dkc, dvc, pooled, total;
 };
 
 struct Carver {
@@ -148,6 +148,7 @@ BwdLayout bwd_layout(const Geo& g) {
   r.delta = c.take(BHq * g.S * sizeof(float));
   r.absmax = c.take(BHq * (g.N + text_blocks(g)) * sizeof(float2));
   r.ds_exp = c.take((size_t)g.batch * g.Hkv * sizeof(int));
+  r.full = c.take(packed_cubes(g, nullptr).shift > 0 ? BHq * (g.N + text_blocks(g)) * sizeof(int) : 0);
   r.d_oc_hat = c.take(BHq * g.N * g.D * sizeof(float));
   r.delta_c = c.take(BHq * g.N * sizeof(float));
   r.dqc = c.take(BHq * g.N * g.D * sizeof(float));
@@ -779,6 +780,8 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   VSA2_CUDA(sm_count(&sms));
   const Geo& dg = wide ? g : fx;                // geometry of the lists by which the tiles of dS are placed
   int* dkv_order = ds_groups > 0 && (long long)ds_groups * dg.N > 4 * sms ? at<int>(scratch, dl.order) : nullptr;
+  // (64-token tiles; the dK/dV pass packs where it stores dS)
+  const PackedCubes pk = ds_groups > 0 && !wide ? packed_cubes(fx, at<int>(workspace, lay.full)) : PackedCubes{};
   const StoredDs sd{at<unsigned char>(scratch, dl.tiles), at<int>(scratch, dl.pos), at<int>(scratch, dl.counters), dkv_order, ds_groups,
                     wide ? map->row_ptr : row_ptr, wide ? map->col_idx : col_idx, coarse ? dqc : nullptr, dq};
   // cubes of 128 tokens: both passes on 128 x 128 tiles
@@ -792,6 +795,10 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
                                &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
       VSA2_CUDA(launch_ds_positions(dg, sd.row_ptr, sd.col_idx, wide ? map->col_ptr : col_ptr, wide ? map->row_idx : row_idx,
                                     at<int>(scratch, dl.pos), sd.counters, 2 * g.batch * g.Hkv, st));
+      if (pk.shift > 0) {
+        g_launches += 1;
+        VSA2_CUDA(launch_full_counts(fx, pk, col_ptr, row_idx, at<int>(workspace, lay.full), st));
+      }
       if (dkv_order != nullptr) {
         g_launches += 1;
         VSA2_CUDA(launch_dkv_order(dg, wide ? map->col_ptr : col_ptr, dkv_order, st));
@@ -833,7 +840,7 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
                                        coarse ? dvc : nullptr, dk, dv, reinterpret_cast<StatusBlock*>(workspace), st, true,
                                        f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,
                                        f16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)) : nullptr, v16,
-                                       gqa16 ? v16 + bwd_k16_bytes(g) : nullptr, ds_groups > 0 ? &sd : nullptr, scale.exp));
+                                       gqa16 ? v16 + bwd_k16_bytes(g) : nullptr, ds_groups > 0 ? &sd : nullptr, scale.exp, pk));
   }
   return VSA2_OK;
 }

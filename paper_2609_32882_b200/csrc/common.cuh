@@ -362,6 +362,16 @@ cudaError_t launch_cast_qk(const Geo& g, const bf16* q, void* q16, const bf16* k
 // fp16 copies of V and of dO times 2^ds_exp of its KV group, with the same flag
 cudaError_t launch_cast_v_do(const Geo& g, const bf16* v, void* v16, const bf16* d_o, void* do16, const int* ds_exp, int* range_flag,
                              cudaStream_t st);
+// Query cubes of a last layer of frames that the grid cuts, packed by the dK/dV pass: the tokens of such a cube are the first rows of
+// its 64-row tile (positions run frame by frame), so 2^shift of them share one tile.  Grids of 4n + 1 latent frames, which causal
+// video encoders make, leave one frame of four there: at 21 frames a sixth of all query blocks is a quarter of a tile.
+struct PackedCubes {
+  int shift;          // 1 or 2; 0: not packed
+  int first;          // first cube of the layer; its cubes are the last of the video, and of every (ascending) list
+  const int* full;    // [B, Hq, N]: entries of a column list in front of them
+};
+PackedCubes packed_cubes(const Geo& g, const int* full);
+cudaError_t launch_full_counts(const Geo& g, const PackedCubes& pk, const int* ptr, const int* idx, int* full, cudaStream_t st);
 // dS kept between the two backward passes (fine_bwd_dq_ds_tc.cu, fine_bwd128_dq_ds_tc.cu): scratch for the pairs of `chunk_groups`
 // KV groups at a time.  On 128 x 128 tiles every size and list below is that of the cube map.
 struct StoredDs {
@@ -380,7 +390,7 @@ cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col
 cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st);
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
-                                  int* item_counter, bool swizzled, const int* ds_exp, cudaStream_t st);
+                                  int* item_counter, bool swizzled, const int* ds_exp, const PackedCubes& pk, cudaStream_t st);
 cudaError_t launch_fine_bwd128_dq_ds(const Geo& g, long long cap, const void* k16, const void* ds, int head0, int heads,
                                      const int* row_ptr, const int* col_idx, const float* dqc, void* dq, StatusBlock* status,
                                      int* range_flag, int* item_counter, const int* ds_exp, cudaStream_t st);
@@ -396,7 +406,8 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
-                                   const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp);
+                                   const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp,
+                                   const PackedCubes& pk = PackedCubes{});
 bool fine_bwd_dkv_gqa_uses_f16(const Geo& g);
 bool fine_bwd_dkv_splits_long_columns(const Geo& g, bool split_long_columns);
 

@@ -236,7 +236,7 @@ cudaError_t launch_fine_bwd128_dq_ds(const Geo& g, long long cap, const void* k1
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), 0, dqc, dq, status, range_flag, ds_exp,
+  DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), 0, PackedCubes{}, dqc, dq, status, range_flag, ds_exp,
              head0, head0 * (g.N / 2), heads * (g.N / 2)};
   const int grid = a.items < sms ? a.items : sms;
   if (g.D == 128) {

@@ -32,6 +32,7 @@ struct DkvArgs {
   int ds_head0;
   const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale; forms whose dS is rounded to fp16)
   const int* order;     // null, or the order in which the items are drawn
+  PackedCubes pk;       // PACK
   int overlap;          // 1: the launch behind this one may start while this one runs; 2: this one may be running beside the one before it
 };
 
@@ -41,15 +42,31 @@ constexpr int kMaxRep = 16;   // query heads per KV head the dK/dV pass supports
 // (`cnt_prefix`, `col_beg`: per-head counts prefix and list starts of the item, read once per item so that this lookup
 // costs a single global load)
 // (`POS`: also its place in the row lists)
-template <bool POS = false>
-__device__ __forceinline__ void dkv_entry(const Geo& g, const DkvArgs& a, int rep, int b, int hk, const int* cnt_prefix,
-                                          const int* col_beg, int e, int& bhq, int& i, int* pos = nullptr) {
+// PACK: entry e is a tile of 64 rows, `sub` the packed cube of it that is asked for (the last one again beyond the list's end);
+// returns 0 for a block that fills the tile, 1 for a packed cube, 2 for one beyond the end.  `col_full`, `col_cnt`: entries of each
+// head's list in front of the cut layer, and of all of it.
+template <bool POS = false, bool PACK = false>
+__device__ __forceinline__ int dkv_entry(const Geo& g, const DkvArgs& a, int rep, int b, int hk, const int* cnt_prefix,
+                                         const int* col_beg, int e, int& bhq, int& i, int* pos = nullptr, int sub = 0,
+                                         const int* col_full = nullptr, const int* col_cnt = nullptr) {
   int hh = 0;
   while (hh + 1 < rep && e >= cnt_prefix[hh + 1]) ++hh;
   bhq = b * g.Hq + hk * rep + hh;
-  const size_t at = (size_t)bhq * g.nnz_cap + col_beg[hh] + (e - cnt_prefix[hh]);
+  int v = e - cnt_prefix[hh], kind = 0;
+  if (PACK && v >= col_full[hh]) {
+    const int full = col_full[hh], end = col_cnt[hh] - (g.N - g.Nvid), groups = (end - full + (1 << a.pk.shift) - 1) >> a.pk.shift;
+    if (v < full + groups) {
+      v = full + ((v - full) << a.pk.shift) + sub;
+      kind = v < end ? 1 : 2;
+      v = min(v, end - 1);
+    } else {
+      v += end - full - groups;                  // (a text block)
+    }
+  }
+  const size_t at = (size_t)bhq * g.nnz_cap + col_beg[hh] + v;
   i = a.row_idx[at];
   if (POS && a.ds != nullptr) *pos = a.ds_pos[at];
+  return kind;
 }
 
 // Roles: warp 0 = TMA producer of the Q pairs (ring A) and of the stationary K and V tiles, warp 1 = TMA producer of the
@@ -88,12 +105,19 @@ __device__ __forceinline__ void dkv_entry(const Geo& g, const DkvArgs& a, int re
 // groups, where a KV block sums the query blocks of several heads and bf16 P leaves dV at 1.4e-2 (480p sample, |dV| = 11).
 // F16 = 3: the same without `a.ds`, dS clamped: the recomputing dQ pass forms dP from the bf16 originals, of which the copies of V and
 // dO can be 2^-25 off, so of a dS next to the limit one pass may have 65504 and the other an infinity that no flag tells of.
-template <int D, bool SPLIT, bool MHA, int F16>
+// PACK: query cubes of a cut last layer (PackedCubes) share the 64-row halves of a tile: their boxes have fewer frames and lie one
+// behind the other, row statistics and dS places go by cube.  Every grid of 4n + 1 frames runs fewer tiles for it (21 frames: an
+// eighth); a form of its own, so that the others keep their code.  Backward, ms: 720p, 40 heads 26.3 -> 24.6, 8 heads on 2 with budgets
+// 15.1 -> 14.2; 480p, 12 heads on 3 4.33 -> 4.23; 13 frames, 16 heads of 64 channels 0.913 -> 0.875.  The packed cubes' rows are whole
+// steps of a contraction and stay in order, so the gradients are the same bit for bit.  (As KEYS such cubes are hardly ever
+// kept -- their block score is a mean over sub-cubes they do not have -- so nothing is packed there.)
+template <int D, bool SPLIT, bool MHA, int F16, bool PACK = false>
 __global__ void __launch_bounds__(kDkvThreads, 1)
 fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
                        const __grid_constant__ CUtensorMap tm_qt, const __grid_constant__ CUtensorMap tm_kt,
-                       const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot, Geo g,
+                       const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot,
+                       const __grid_constant__ CUtensorMap tm_qe, const __grid_constant__ CUtensorMap tm_doe, Geo g,
                        DkvArgs a) {
   constexpr int RA = SPLIT ? 2 : kRingA;                   // slots of the Q ring
   // accumulators: without SPLIT two sets of dK^T, dV^T (64 columns each), used by item parity
@@ -148,10 +172,25 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int j = rec.x, bhk = rec.y, k = rec.z;                                           \
   const int b = bhk / g.Hkv, hk = bhk % g.Hkv;                                           \
   int cnt_prefix[(MHA ? 1 : kMaxRep) + 1], col_beg[MHA ? 1 : kMaxRep];                   \
+  int col_full[MHA || !PACK ? 1 : kMaxRep], col_cnt[MHA || !PACK ? 1 : kMaxRep];         \
   cnt_prefix[0] = 0;                                                                     \
   col_beg[0] = rec.w;                                                                    \
   if (MHA) {                                                                             \
     cnt_prefix[1] = k;                                                                   \
+    if (PACK) {                                                                          \
+      col_full[0] = a.pk.full[(size_t)bhk * g.N + j];                                    \
+      col_cnt[0] = a.col_ptr[(size_t)bhk * (g.N + 1) + j + 1] - rec.w;                   \
+    }                                                                                    \
+  } else if (PACK) {                                                                     \
+    for (int hh = 0; hh < rep; ++hh) {                                                   \
+      const size_t head_ = (size_t)(b * g.Hq + hk * rep + hh), base_ = head_ * (g.N + 1) + j; \
+      col_beg[hh] = a.col_ptr[base_];                                                    \
+      col_cnt[hh] = a.col_ptr[base_ + 1] - col_beg[hh];                                  \
+      col_full[hh] = a.pk.full[head_ * g.N + j];                                         \
+      const int text_ = g.N - g.Nvid;                                                    \
+      cnt_prefix[hh + 1] = cnt_prefix[hh] + col_full[hh] + text_ +                       \
+                           ((col_cnt[hh] - text_ - col_full[hh] + (1 << a.pk.shift) - 1) >> a.pk.shift); \
+    }                                                                                    \
   } else {                                                                               \
     for (int hh = 0; hh < rep; ++hh) {                                                   \
       const size_t base_ = (size_t)(b * g.Hq + hk * rep + hh) * (g.N + 1) + j;           \
@@ -169,6 +208,9 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     const CUtensorMap* tm = which == 0 ? &tm_q : &tm_do;
     const CUtensorMap* tm_text = which == 0 ? &tm_qt : &tm_dot;
     const int my_blk = lane & 1;
+    const int my_h = (lane >> 1) % C::DH, my_sub = PACK ? ((lane >> 1) / C::DH) & ((1 << a.pk.shift) - 1) : 0;
+    const CUtensorMap* tm_cut = which == 0 ? &tm_qe : &tm_doe;
+    (void)my_h; (void)tm_cut;
     uint32_t tg = 0, n_items = 0;
     for (uint32_t seq = 0;; ++seq) {
       VSA2_NEXT_REC(rec, seq);
@@ -194,15 +236,32 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       ++n_items;
       const int nt = (k + 1) >> 1;
       int bhq_l, i_l;           // this lane's entry of the tile, fetched one tile ahead of the slot wait
-      dkv_entry(g, a, rep, b, hk, cnt_prefix, col_beg, (my_blk == 1 && k > 1) ? 1 : 0, bhq_l, i_l);
+      int kind_l = dkv_entry<false, PACK>(g, a, rep, b, hk, cnt_prefix, col_beg, (my_blk == 1 && k > 1) ? 1 : 0, bhq_l, i_l, nullptr, my_sub, col_full, col_cnt);
       for (int t = 0; t < nt; ++t, ++tg) {
         int c1, c2, c3;
         block_box(g, i_l, c1, c2, c3);
-        const CUtensorMap* tm_i = block_is_text(g, i_l) ? tm_text : tm;
-        const int bhq_t = bhq_l;
-        if (t + 1 < nt) dkv_entry(g, a, rep, b, hk, cnt_prefix, col_beg, (my_blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_l, i_l);
-        if (which == 0) VSA2_RING_LOAD(misc->a_full, misc->a_empty, RA, smem, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
-        else VSA2_RING_LOAD(misc->b_full, misc->b_empty, kRingB, smem + C::OFF_RING_B, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
+        const CUtensorMap* tm_i = PACK && kind_l > 0 ? tm_cut : block_is_text(g, i_l) ? tm_text : tm;
+        const int bhq_t = bhq_l, kind_t = kind_l;
+        if (t + 1 < nt)
+          kind_l = dkv_entry<false, PACK>(g, a, rep, b, hk, cnt_prefix, col_beg, (my_blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_l, i_l, nullptr,
+                                          my_sub, col_full, col_cnt);
+        if constexpr (PACK) {
+          const uint32_t nslots = which == 0 ? RA : kRingB, slot = tg % nslots, par = (tg / nslots) & 1;
+          uint64_t* full = which == 0 ? &misc->a_full[slot] : &misc->b_full[slot];
+          int ok = 1;
+          if (lane == 0) {
+            ok = tc::mbar_wait_parked(which == 0 ? &misc->a_empty[slot] : &misc->b_empty[slot], par ^ 1, &misc->abort_flag);
+            if (ok) tc::mbar_expect_tx(full, C::SLOT);
+          }
+          if (!__shfl_sync(0xffffffffu, ok, 0)) goto done;
+          if (lane < (kind_t > 0 ? 2 * C::DH << a.pk.shift : 2 * C::DH))
+            tc::tma_load_5d(smem + (which == 0 ? 0 : C::OFF_RING_B) + slot * C::SLOT + (2 * my_h + my_blk) * kSlab +
+                                (kind_t > 0 ? my_sub * (kSlab >> a.pk.shift) : 0),
+                            tm_i, full, my_h * 64, c1, c2, c3, bhq_t);
+        } else {
+          if (which == 0) VSA2_RING_LOAD(misc->a_full, misc->a_empty, RA, smem, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
+          else VSA2_RING_LOAD(misc->b_full, misc->b_empty, kRingB, smem + C::OFF_RING_B, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
+        }
       }
     }
     } else {
@@ -248,8 +307,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   } else if (warp >= 16 && warp < 20) {
     tc::reg_dec<48>();
-    if (warp == 18 && !bwd_schedule(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
-                                    a.k_hi, SPLIT && MHA && a.k_lo > 1, nullptr, lane, &misc->abort_flag))
+    if (warp == 18 && !bwd_schedule<PACK>(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
+                                    a.k_hi, SPLIT && MHA && a.k_lo > 1, nullptr, lane, &misc->abort_flag, a.pk))
       goto done;
     if (STORES_DS && !SPLIT && warp == 19 && a.ds != nullptr) {
       // ---------------------------------------------------------------- copies the dS tiles to the scratch as they stand
@@ -261,9 +320,17 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         for (int t = 0; t < nt; ++t, ++tg) {
           VSA2_WAIT_PARKED(&misc->ds_ready[0], tg & 1);
           if (lane == 0) {
-            const int s0 = misc->ds_slot[tg & 3][0], s1 = misc->ds_slot[tg & 3][1];
-            if (s0 >= 0) tc::bulk_store(a.ds + (size_t)s0 * kSlab, ds_tile, kSlab, policy);
-            if (s1 >= 0) tc::bulk_store(a.ds + (size_t)s1 * kSlab, ds_tile + kSlab, kSlab, policy);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int* at = misc->ds_slot[tg % 3][h];
+              if (!PACK || at[1] == kWholeBlock) {
+                if (at[0] >= 0) tc::bulk_store(a.ds + (size_t)at[0] * kSlab, ds_tile + h * kSlab, kSlab, policy);
+              } else {
+                const uint32_t bytes = kSlab >> a.pk.shift;
+                for (int c = 0; c < 1 << a.pk.shift; ++c)
+                  if (at[c] >= 0) tc::bulk_store(a.ds + (size_t)at[c] * kSlab, ds_tile + h * kSlab + c * bytes, bytes, policy);
+              }
+            }
             tc::bulk_store_commit();
             tc::bulk_store_wait_read();
             tc::mbar_arrive(&misc->ds_free[0]);
@@ -323,6 +390,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     // ------------------------------------------------------------------ row statistics of the tiles (128 threads)
     const int r = tid - 384;                 // query row of the tile
     const int blk = r >> 6;
+    const int sub = PACK ? (r & 63) >> (6 - a.pk.shift) : 0, cut_rows = PACK ? 64 >> a.pk.shift : 64;
     float2* rowstat = reinterpret_cast<float2*>(misc->stats);
     uint32_t tg = 0;
     for (uint32_t seq = 0;; ++seq) {
@@ -334,17 +402,22 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const float lse_off = F16 >= 2 ? 0.f : (float)ds_exp, dlt_scale = F16 >= 2 ? pow2i(ds_exp) : 1.f;
       const int nt = (k + 1) >> 1;
       int bhq_n, i_n, pos_n = 0;
-      dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n, &pos_n);
+      int kind_n = dkv_entry<STORES_DS, PACK>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && k > 1) ? 1 : 0, bhq_n, i_n, &pos_n, sub, col_full, col_cnt);
       for (int t = 0; t < nt; ++t, ++tg) {
         const int slot = STORES_DS && a.ds != nullptr ? (bhq_n - a.ds_head0) * (int)g.nnz_cap + pos_n : -1;
-        const bool dup = (blk == 1) && (2 * t + 1 >= k);
-        const int l = dup ? -1 : block_token(g, i_n, r & 63);
+        const bool dup = ((blk == 1) && (2 * t + 1 >= k)) || (PACK && kind_n == 2);
+        const int kind = kind_n, row_in = PACK && kind > 0 ? r & (cut_rows - 1) : r & 63;
+        const int l = dup ? -1 : block_token(g, i_n, row_in);
         const size_t idx = l >= 0 ? (size_t)bhq_n * g.S + l : 0;
         const float lse_raw = a.lse[idx], dlt_raw = a.delta[idx];
         if (t + 1 < nt)
-          dkv_entry<STORES_DS>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_n, i_n, &pos_n);
+          kind_n = dkv_entry<STORES_DS, PACK>(g, a, rep, b, hk, cnt_prefix, col_beg, (blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_n, i_n, &pos_n,
+                                              sub, col_full, col_cnt);
         VSA2_WAIT_PARKED(&misc->stat_free, (tg & 1) ^ 1);
-        if (STORES_DS && (r & 63) == 0) misc->ds_slot[tg & 3][blk] = dup ? -1 : slot;
+        if (STORES_DS && row_in == 0) {
+          misc->ds_slot[tg % 3][blk][PACK && kind > 0 ? sub : 0] = dup ? -1 : slot;
+          if (PACK && kind == 0) misc->ds_slot[tg % 3][blk][1] = kWholeBlock;
+        }
         rowstat[r] = make_float2(l >= 0 ? lse_raw * 1.4426950408889634f - lse_off : INFINITY, l >= 0 ? dlt_raw * dlt_scale : 0.f);
         tc::mbar_arrive(&misc->stat_full);
       }
@@ -368,7 +441,16 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const uint32_t s = tg & 1, par = (tg >> 1) & 1;
           VSA2_WAIT(&misc->stat_full, tg & 1);
           const float2 rs = rowstat[row];
-          const int ds_slot = SPLIT && STORES_DS ? misc->ds_slot[tg & 3][row >> 6] : -1;
+          int ds_slot = -1, ds_row = row & 63;
+          if (SPLIT && STORES_DS) {
+            const int* at = misc->ds_slot[tg % 3][row >> 6];
+            if (PACK && at[1] != kWholeBlock) {
+              ds_slot = at[ds_row >> (6 - a.pk.shift)];
+              ds_row &= (64 >> a.pk.shift) - 1;
+            } else {
+              ds_slot = at[0];
+            }
+          }
           tc::mbar_arrive(&misc->stat_free);
           const float lse2 = rs.x, dlt = rs.y;
           uint32_t sv[32];      // S, then P
@@ -430,7 +512,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             }
             if (SPLIT && STORES_DS && ds_slot >= 0) {
               // [chunk of 8 keys][query row]: 512 contiguous bytes per warp and store
-              uint4* dst = reinterpret_cast<uint4*>(a.ds + (size_t)ds_slot * kSlab) + half * 256 + (row & 63);
+              uint4* dst = reinterpret_cast<uint4*>(a.ds + (size_t)ds_slot * kSlab) + half * 256 + ds_row;
 #pragma unroll
               for (int ch = 0; ch < 4; ++ch) {
                 if constexpr (SPLIT && STORES_DS) dst[ch * 64] = make_uint4(ph[4 * ch], ph[4 * ch + 1], ph[4 * ch + 2], ph[4 * ch + 3]);
@@ -568,7 +650,8 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* lse, const float* delta, const int* col_ptr, const int* row_idx,
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
-                                   const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp) {
+                                   const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp,
+                                   const PackedCubes& pk) {
   if (g.rep > kMaxRep) return cudaErrorInvalidValue;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16;
   // GQA groups without a precision flag take the all-fp16 form when they are given scratch for fp16 copies of V and dO as
@@ -593,15 +676,24 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   const bool mha = g.rep == 1;
-#define VSA2_LAUNCH_DKV(DD, SP, MH, F, TQ, TK, TQT, TKT, TV, TDO, TVT, TDOT)                                                                         \
+  // the main forms with stored dS have a packed version
+  CUtensorMap tqe = {}, tdoe = {};
+  const bool pack = pk.shift > 0 && sd != nullptr;
+  if (pack) {
+    const int frames = g.T - (g.Nt - 1) * g.Bt;
+    if (!make_cube_tmap(&tqe, f16 ? reinterpret_cast<const bf16*>(q16) : q, g, g.Hq, frames) ||
+        !make_cube_tmap(&tdoe, f16 && gqa16 ? reinterpret_cast<const bf16*>(do16) : d_o, g, g.Hq, frames))
+      return cudaErrorInvalidValue;
+  }
+#define VSA2_LAUNCH_DKV(DD, SP, MH, F, PK, TQ, TK, TQT, TKT, TV, TDO, TVT, TDOT)                                                                         \
   do {                                                                                                                           \
     using L_ = BwdTc<DD, SP ? 2 : kRingA, SP ? 4 : 2>;                                                                           \
     cfg.dynamicSmemBytes = L_::smem_bytes;                                                                                       \
     static KernelAttr attr_;                                                                                                     \
-    if ((e = prepare_kernel((const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F>, attr_, L_::smem_bytes, kDkvThreads,               \
+    if ((e = prepare_kernel((const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F, PK>, attr_, L_::smem_bytes, kDkvThreads,               \
                             128 * (48 + 2 * 120 + 2 * 48 + 96))))                                                                \
       return e;                                                                                                                  \
-    if ((e = cudaLaunchKernelEx(&cfg, fine_bwd_dkv_tc_kernel<DD, SP, MH, F>, TQ, TK, TV, TDO, TQT, TKT, TVT, TDOT, g, a)))       \
+    if ((e = cudaLaunchKernelEx(&cfg, fine_bwd_dkv_tc_kernel<DD, SP, MH, F, PK>, TQ, TK, TV, TDO, TQT, TKT, TVT, TDOT, tqe, tdoe, g, a)))       \
       return e;                                                                                                                  \
   } while (0)
   // `when`: see DkvArgs.
@@ -621,26 +713,34 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     cfg.stream = st;
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
-              group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr, overlap};
-    if (when == 1 && gqa16 && ds) { // every product in fp16
-      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
-      else VSA2_LAUNCH_DKV(64, false, false, 2, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
+              group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr, pk, overlap};
+    if (ds && pack) {
+#define VSA2_LAUNCH_PACKED(DD)                                                                                  \
+      if (when == 1 && gqa16) VSA2_LAUNCH_DKV(DD, false, false, 2, true, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16); \
+      else if (when == 1) VSA2_LAUNCH_DKV(DD, false, true, 1, true, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);      \
+      else VSA2_LAUNCH_DKV(DD, true, false, 0, true, tq, tk, tqt, tkt, tv, tdo, tvt, tdot)
+      if (g.D == 128) { VSA2_LAUNCH_PACKED(128); }
+      else { VSA2_LAUNCH_PACKED(64); }
+#undef VSA2_LAUNCH_PACKED
+    } else if (when == 1 && gqa16 && ds) { // every product in fp16
+      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 2, false, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
+      else VSA2_LAUNCH_DKV(64, false, false, 2, false, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
     } else if (when == 1 && gqa16) {
-      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 3, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
-      else VSA2_LAUNCH_DKV(64, false, false, 3, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
+      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, false, 3, false, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
+      else VSA2_LAUNCH_DKV(64, false, false, 3, false, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16);
     } else if (when == 1) {         // S and the dK product in fp16 (one query head per KV head)
-      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, true, 1, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);
-      else VSA2_LAUNCH_DKV(64, false, true, 1, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);
+      if (g.D == 128) VSA2_LAUNCH_DKV(128, false, true, 1, false, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);
+      else VSA2_LAUNCH_DKV(64, false, true, 1, false, tq16, tk16, tqt16, tkt16, tv, tdo, tvt, tdot);
     } else if (g.D == 128) {
-      if (split && mha) VSA2_LAUNCH_DKV(128, true, true, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
-      else if (split) VSA2_LAUNCH_DKV(128, true, false, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
-      else if (mha) VSA2_LAUNCH_DKV(128, false, true, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
-      else VSA2_LAUNCH_DKV(128, false, false, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      if (split && mha) VSA2_LAUNCH_DKV(128, true, true, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      else if (split) VSA2_LAUNCH_DKV(128, true, false, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      else if (mha) VSA2_LAUNCH_DKV(128, false, true, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      else VSA2_LAUNCH_DKV(128, false, false, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
     } else {
-      if (split && mha) VSA2_LAUNCH_DKV(64, true, true, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
-      else if (split) VSA2_LAUNCH_DKV(64, true, false, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
-      else if (mha) VSA2_LAUNCH_DKV(64, false, true, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
-      else VSA2_LAUNCH_DKV(64, false, false, 0, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      if (split && mha) VSA2_LAUNCH_DKV(64, true, true, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      else if (split) VSA2_LAUNCH_DKV(64, true, false, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      else if (mha) VSA2_LAUNCH_DKV(64, false, true, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
+      else VSA2_LAUNCH_DKV(64, false, false, 0, false, tq, tk, tqt, tkt, tv, tdo, tvt, tdot);
     }
     return cudaGetLastError();
   };
@@ -657,7 +757,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
       const int n = all - g0 < sd->chunk_groups ? all - g0 : sd->chunk_groups;
       if ((r = launch(split, sd->counters + 2 * c, 0, kAll, when, g0, n, true)) != cudaSuccess) return r;
       if ((r = launch_fine_bwd_dq_ds(g, k16, sd->scratch, g0 * g.rep, n * g.rep, sd->row_ptr, sd->col_idx, sd->dqc, sd->dq, status,
-                                     range_flag, sd->counters + 2 * c + 1, !split, ds_exp, st)) != cudaSuccess)
+                                     range_flag, sd->counters + 2 * c + 1, !split, ds_exp, pack ? pk : PackedCubes{}, st)) != cudaSuccess)
         return r;
     }
     // dQ again, from bf16 pairs, if a value left the fp16 range
@@ -681,6 +781,37 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   }
   if ((e = launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, when, 0, all, false, 1)) != cudaSuccess) return e;
   return launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, when, 0, all, false, 2);
+}
+
+// Packed where two or four cubes fill a tile.  Below 128 cubes the counts are a launch for nothing.
+PackedCubes packed_cubes(const Geo& g, const int* full) {
+  const int rows = (g.T - (g.Nt - 1) * g.Bt) * g.Bh * g.Bw;
+  const int shift = rows == kBlockTokens / 4 ? 2 : rows == kBlockTokens / 2 ? 1 : 0;
+  return PackedCubes{g.Nvid >= 128 && g.Nt > 1 ? shift : 0, (g.Nt - 1) * g.Nh * g.Nw, full};
+}
+
+// One warp per list: the entries in front of the cubes of the last layer -- or, of a list that does not have them at its end, all
+// but the text blocks (nothing of it is packed then)
+__global__ void __launch_bounds__(256) full_counts_kernel(int N, int Nvid, int first, long long cap, const int* __restrict__ ptr,
+                                                          const int* __restrict__ idx, int* __restrict__ full) {
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (j >= N) return;
+  const size_t bh = blockIdx.y;
+  const int beg = ptr[bh * (N + 1) + j], k = ptr[bh * (N + 1) + j + 1] - beg - (N - Nvid);
+  const int* list = idx + bh * cap + beg;
+  int n = 0, last = -1;                      // entries before the layer, and the last of them
+  for (int e = lane; e < k; e += 32)
+    if (list[e] < first) {
+      ++n;
+      last = e;
+    }
+  n = __reduce_add_sync(0xffffffffu, n);
+  last = __reduce_max_sync(0xffffffffu, last);
+  if (lane == 0) full[bh * N + j] = last + 1 == n ? n : k;
+}
+cudaError_t launch_full_counts(const Geo& g, const PackedCubes& pk, const int* ptr, const int* idx, int* full, cudaStream_t st) {
+  full_counts_kernel<<<dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st>>>(g.N, g.Nvid, pk.first, g.nnz_cap, ptr, idx, full);
+  return cudaGetLastError();
 }
 
 // Whether the dK/dV pass of a GQA problem takes its all-fp16 form when it is given the scratch for the four copies.  Rows that

@@ -39,6 +39,8 @@ struct DqDsMisc {
 };
 static_assert(sizeof(DqDsMisc) <= 2048, "misc region too small");
 
+__device__ __forceinline__ bool packed_query(const Geo& g, const PackedCubes& pk, int i) { return pk.shift > 0 && i >= pk.first && i < g.Nvid; }
+
 template <int D>
 __global__ void __launch_bounds__(kDsThreads, 1)
 fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_kt, Geo g,
@@ -85,6 +87,8 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       const int b = rec.y / g.Hq, hq = rec.y % g.Hq, bhk = b * g.Hkv + hq / g.rep;
       const int* cols = a.col_idx + (size_t)rec.y * g.nnz_cap + rec.w;
       const unsigned char* tiles = a.ds + ((size_t)(rec.y - a.head0) * g.nnz_cap + rec.w) * kSlab;
+      // (rows of a packed cube are the first of its tiles as the fp16 forms leave them; the other form has them in every chunk)
+      const uint32_t tile_bytes = a.ds_swizzled && packed_query(g, a.pk, rec.x) ? kSlab >> a.pk.shift : kSlab;
       int j = warp < 2 ? cols[(warp == 1 && k > 1) ? 1 : 0] : 0;
       for (int t = 0; t < nt; ++t, ++tg) {
         int c1 = 0, c2 = 0, c3 = 0;
@@ -95,7 +99,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
           if (t + 1 < nt) j = cols[(warp == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2];   // next tile, fetched early
         }
         const uint32_t slot = tg % C::STAGES;
-        const uint32_t ds_bytes = (t == nt - 1 && (k & 1)) ? kSlab : C::DSBYTES;
+        const uint32_t ds_bytes = (t == nt - 1 && (k & 1)) ? tile_bytes : 2 * tile_bytes;
         int ok = 1;
         if (lane == 0) {
           ok = tc::mbar_wait_parked(&misc->empty[slot], ((tg / C::STAGES) & 1) ^ 1, &misc->abort_flag);
@@ -107,7 +111,9 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
           if (lane < C::DH)
             tc::tma_load_5d(stage + (2 * lane + warp) * kSlab, text ? &tm_kt : &tm_k, &misc->full[slot], lane * 64, c1, c2, c3, bhk);
         } else if (lane == 0) {
-          tc::bulk_load(stage + C::KBYTES, tiles + (size_t)t * C::DSBYTES, ds_bytes, &misc->full[slot], policy);
+          tc::bulk_load(stage + C::KBYTES, tiles + (size_t)t * C::DSBYTES, tile_bytes == kSlab ? ds_bytes : tile_bytes, &misc->full[slot], policy);
+          if (tile_bytes != kSlab && ds_bytes > tile_bytes)
+            tc::bulk_load(stage + C::KBYTES + kSlab, tiles + (size_t)t * C::DSBYTES + kSlab, tile_bytes, &misc->full[slot], policy);
         }
       }
     }
@@ -189,6 +195,10 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         tc::tmem_ld_wait();
         // a dS that left the fp16 range is an infinity and has made every channel of its query column non-finite (one store per
         // warp: with all rows out of range one per thread took 2.7 ms for 8 heads of 720p)
+        if (packed_query(g, a.pk, i)) {       // (what lies behind a packed cube's rows is nobody's dS)
+#pragma unroll
+          for (int c = 0; c < 32; ++c) x[c] = part * 32 + c < 64 >> a.pk.shift ? x[c] : 0u;
+        }
         if (__any_sync(0xffffffffu, row < D && any_non_finite32(x)) && lane == 0) *a.range_flag = 1;
         float v[32];
 #pragma unroll
@@ -303,7 +313,7 @@ cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaS
 // dQ of the heads head0 .. head0 + heads - 1 (index batch * Hq) from their dS tiles
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
-                                  int* item_counter, bool swizzled, const int* ds_exp, cudaStream_t st) {
+                                  int* item_counter, bool swizzled, const int* ds_exp, const PackedCubes& pk, cudaStream_t st) {
   CUtensorMap tk, tkt;
   if (!make_cube_tmap(&tk, reinterpret_cast<const bf16*>(k16), g, g.Hkv) ||      // (same element size: the maps only move bytes)
       !make_text_tmap(&tkt, reinterpret_cast<const bf16*>(k16), g, g.Hkv))
@@ -311,7 +321,7 @@ cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds,
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), swizzled ? 1 : 0, dqc, dq, status, range_flag, ds_exp, head0, head0 * g.N, heads * g.N};
+  DqDsArgs a{item_counter, row_ptr, col_idx, reinterpret_cast<const unsigned char*>(ds), swizzled ? 1 : 0, pk, dqc, dq, status, range_flag, ds_exp, head0, head0 * g.N, heads * g.N};
   const int grid = a.items < sms ? a.items : sms;
 #define VSA2_LAUNCH_DQ_DS(DD)                                                                                                    \
   do {                                                                                                                           \

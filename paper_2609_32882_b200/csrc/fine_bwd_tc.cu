@@ -376,7 +376,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
       }
       const float coarse_d = (a.dqc != nullptr && row < D && !block_is_text(g, i))
                                  ? a.dqc[((size_t)bhq * g.Nvid + i) * D + row] / (float)cube_count(g, i) : 0.f;
-      VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0);
+      VSA2_GROUP_SYNC_AT(&misc->p_ready, e_sync0);
       if (k > 0) {
         const int nt = (k + 1) >> 1;
         const float4* lse4 = reinterpret_cast<const float4*>(misc->stats + tb * 64) + half * 8;
@@ -499,7 +499,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             for (int c = 0; c < 32; ++c)
               st[(half * 32 + c) * D + row] = __float2bfloat16_rn(fmaf(__uint_as_float(o0[c]), out_scale, coarse_d));
           }
-          VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0 + 1);
+          VSA2_GROUP_SYNC_AT(&misc->p_ready, e_sync0 + 1);
           constexpr int CH = D / 8;
           for (int e = sm_tid; e < 64 * CH; e += 256) {
             const int qi = e / CH, ch = e % CH;
@@ -508,7 +508,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.dq) + ((size_t)bhq * g.S + l) * D + ch * 8) =
                 *reinterpret_cast<const uint4*>(st + qi * D + ch * 8);
           }
-          VSA2_GROUP_SYNC_AT(&misc->e_sync, e_sync0 + 2);
+          VSA2_GROUP_SYNC_AT(&misc->p_ready, e_sync0 + 2);
         }
       }
       if (k > 0) ++n_items;

@@ -66,9 +66,11 @@ __device__ __forceinline__ bool bwd_queue_get(BwdQueue* q, uint32_t seq, int lan
 // `rep` consecutive heads; items with fewer than k_lo or more than k_hi entries are left out.
 // `sparse`: few items are in that range.  A draw then stands for 32 of them, one per lane and far apart (their lists tend to be long
 // side by side), so that passing over the others costs a 32nd of the draws.
+// PACK: the entries counted are tiles of 64 rows (a list's cubes of the cut layer are packed).
+template <bool PACK = false>
 __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int first_item, int items, int rep, const int* ptr,
                                              int* counter, const int* order, int k_lo, int k_hi, bool sparse, const int* stop, int lane,
-                                             volatile int* abort_flag) {
+                                             volatile int* abort_flag, const PackedCubes& pk = PackedCubes{}) {
   const int draws = sparse ? (items + 31) / 32 : items;
   uint32_t drawn = 0;
   unsigned left = 0u;             // sparse: lanes of the current draw whose items are still to be handed out
@@ -118,6 +120,10 @@ __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int firs
         const int* c = ptr + ((size_t)rec.y * rep + lane) * (g.N + 1) + rec.x;
         beg = c[0];
         k = c[1] - beg;
+        if (PACK) {
+          const int full = pk.full[((size_t)rec.y * rep + lane) * g.N + rec.x], text = g.N - g.Nvid;
+          k = full + text + (k - text - full + (1 << pk.shift) - 1 >> pk.shift);
+        }
       }
       rec.z = __reduce_add_sync(0xffffffffu, k);
       rec.w = __shfl_sync(0xffffffffu, beg, 0);
@@ -160,6 +166,7 @@ struct DqDsArgs {
   const int* col_idx;
   const unsigned char* ds;
   int ds_swizzled;      // layout of the tiles, see fine_bwd_dkv_tc.cu
+  PackedCubes pk;       // as in the dK/dV pass: only the first rows of a tile of a packed query cube have been written
   const float* dqc;     // [B, Hq, N, D] or null
   void* dq;
   StatusBlock* status;
@@ -169,26 +176,31 @@ struct DqDsArgs {
   int first_item, items;
 };
 
+constexpr int kWholeBlock = -2;
 struct BwdMisc {
   uint64_t st_full, st_empty, o_full[2], o_empty[2];       // (the dQ pass uses one accumulator)
   uint64_t a_full[kRingA], a_empty[kRingA], b_full[kRingB], b_empty[kRingB];
   uint64_t s_full[2], s_free[2], dp_full[2], dp_free[2];   // the two score / dP accumulators in tensor memory
-  uint64_t p_ready, p_free;                                 // dK/dV pass: the P operand buffer
+  uint64_t p_ready, p_free;                                 // dK/dV pass: the P operand buffer; dQ pass: p_ready is the group barrier
+                                                            // of its 256 elementwise threads
   uint64_t ds_ready[2], ds_free[2];                         // dS operand buffers (the dK/dV pass has one)
   uint64_t stat_full, stat_free;                            // dK/dV pass: the per-row statistics of a tile
   union {                                                   // work items of this CTA
     ItemQueue items;                                        // dQ pass (see tc_attn.cuh)
     BwdQueue queue;                                         // dK/dV pass
   };
-  uint64_t e_sync;                                          // group barrier of the 256 elementwise threads
   uint32_t tmem_base;
   int abort_flag;
-  unsigned char edge[kRingA][2];   // dQ pass: edge flags of the two key cubes in each ring-A slot (written by its producer)
   // dQ pass: lse2[tb][c] = stats[tb * 64 + c], delta[tb][c] = stats[128 + tb * 64 + c]: per query column of the item with
   // parity tb, lse * log2(e) (+inf for padding) and delta.  dK/dV pass: (lse * log2(e), delta) of the 128 query rows of
   // the current tile, interleaved.
   alignas(16) float stats[256];
-  int ds_slot[4][2];               // dK/dV pass: places of a tile's two dS blocks in the scratch (-1: none), by tile index mod 4
+  union {
+    unsigned char edge[kRingA][2];   // dQ pass: edge flags of the two key cubes in each ring-A slot (written by its producer)
+    // dK/dV pass: places of the dS blocks of a tile's two halves in the scratch (-1: none), by tile index mod 3 (they are written at
+    // most two tiles ahead of their last reader); a half that is one block has kWholeBlock in its second word
+    int ds_slot[3][2][4];
+  };
   int tok[128];                    // raster tokens of the rows of an item's block, by parity (dK/dV pass: of the items with entries)
 };
 static_assert(sizeof(BwdMisc) <= 2048, "misc region too small");
@@ -218,7 +230,6 @@ __device__ __forceinline__ void bwd_init_barriers(BwdMisc* misc) {
     tc::mbar_init(&misc->ds_free[s], 1);
   }
   tc::mbar_init(&misc->p_ready, 256);
-  tc::mbar_init(&misc->e_sync, 256);
   tc::mbar_init(&misc->p_free, 1);
   tc::mbar_init(&misc->stat_full, 128);
   tc::mbar_init(&misc->stat_free, 256);

@@ -26,13 +26,14 @@ inline EncodeTiledFn encode_tiled_fn() {
 }
 
 // bf16 tensor [batch*heads, L, D] in raster token order -> tensor map whose box is one cube, 64 channels wide.
-inline bool make_cube_tmap(CUtensorMap* out, const void* base, const Geo& g, int heads) {
+// `frames`: 0, or the frames of the box (a cube of a cut last layer: its tokens are the first rows of its tile).
+inline bool make_cube_tmap(CUtensorMap* out, const void* base, const Geo& g, int heads, int frames = 0) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (fn == nullptr) return false;
   const cuuint64_t D = (cuuint64_t)g.D;
   cuuint64_t dims[5] = {D, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.T, (cuuint64_t)g.batch * heads};
   cuuint64_t strides[4] = {D * 2, (cuuint64_t)g.W * D * 2, (cuuint64_t)g.H * g.W * D * 2, (cuuint64_t)g.S * D * 2};
-  cuuint32_t box[5] = {64, (cuuint32_t)g.Bw, (cuuint32_t)g.Bh, (cuuint32_t)g.Bt, 1};
+  cuuint32_t box[5] = {64, (cuuint32_t)g.Bw, (cuuint32_t)g.Bh, (cuuint32_t)(frames > 0 ? frames : g.Bt), 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
