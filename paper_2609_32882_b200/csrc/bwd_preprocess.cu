@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
                                                              float* __restrict__ delta, float* __restrict__ dgate,
                                                              float* __restrict__ d_oc_hat, float2* __restrict__ absmax,
                                                              StatusBlock* clear) {
+  grid_enter();
   constexpr int CH = D / 8;                // threads per token = 16-byte chunks of a token row
   constexpr int PAR = 256 / CH;            // tokens at a time
   constexpr int TOK = 2;                   // tokens in flight per thread
@@ -139,8 +140,8 @@ cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, 
                                   const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, float2* absmax,
                                   StatusBlock* clear, cudaStream_t st) {
   dim3 grid(g.N, g.Hq, g.batch);
-  if (g.D == 128) bwd_preprocess_kernel<128><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
-  else bwd_preprocess_kernel<64><<<grid, 256, 0, st>>>(d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  if (g.D == 128) launch_kernel(bwd_preprocess_kernel<128>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  else launch_kernel(bwd_preprocess_kernel<64>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
   return cudaGetLastError();
 }
 

@@ -62,6 +62,7 @@ template <int D>
 __global__ void __launch_bounds__(kCfThreads, 2)
 coarse_fwd_mma_kernel(const float* __restrict__ qc, const float* __restrict__ kc, const float* __restrict__ vc, Geo g,
                       float* __restrict__ oc_hat, float* __restrict__ lse_c) {
+  grid_enter();
   using S = CoarseFwdSmem<D>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* kbuf = reinterpret_cast<float*>(smem_raw);                       // [2][32][LDK]
@@ -213,12 +214,12 @@ cudaError_t launch_coarse_fwd_mma(const Geo& g, const float* qc, const float* kc
     const size_t smb = CoarseFwdSmem<128>::bytes;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)coarse_fwd_mma_kernel<128>, attr, smb))) return e;
-    coarse_fwd_mma_kernel<128><<<grid, kCfThreads, smb, st>>>(qc, kc, vc, g, oc_hat, lse_c);
+    launch_kernel(coarse_fwd_mma_kernel<128>, grid, kCfThreads, smb, st, qc, kc, vc, g, oc_hat, lse_c);
   } else {
     const size_t smb = CoarseFwdSmem<64>::bytes;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)coarse_fwd_mma_kernel<64>, attr, smb))) return e;
-    coarse_fwd_mma_kernel<64><<<grid, kCfThreads, smb, st>>>(qc, kc, vc, g, oc_hat, lse_c);
+    launch_kernel(coarse_fwd_mma_kernel<64>, grid, kCfThreads, smb, st, qc, kc, vc, g, oc_hat, lse_c);
   }
   return cudaGetLastError();
 }

@@ -66,6 +66,7 @@ struct PooledInputs {
   StatusBlock* status;
 };
 __global__ void __launch_bounds__(256) pooled_inputs_kernel(PooledInputs p) {
+  grid_enter();
   if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
   const size_t stride = (size_t)gridDim.x * blockDim.x, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
 #pragma unroll
@@ -87,7 +88,7 @@ static cudaError_t launch_pooled_inputs(const PooledInputs& p, cudaStream_t st) 
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   const size_t blocks = (most + 255) / 256;
-  pooled_inputs_kernel<<<(unsigned)(blocks < (size_t)sms * 8 ? blocks : (size_t)sms * 8), 256, 0, st>>>(p);
+  launch_kernel(pooled_inputs_kernel, (unsigned)(blocks < (size_t)sms * 8 ? blocks : (size_t)sms * 8), 256, 0, st, p);
   return cudaGetLastError();
 }
 
@@ -95,6 +96,7 @@ static cudaError_t launch_pooled_inputs(const PooledInputs& p, cudaStream_t st) 
 // query heads of a group, so the result goes to the group's first query head and zeros to the others
 __global__ void spread_to_group_kernel(const float* __restrict__ x_kv, float* __restrict__ x_q, int rep, size_t per_head4,
                                        int heads_q) {
+  grid_enter();
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const int hq = blockIdx.y;            // b * Hq + hq (Hq = Hkv * rep, so b * Hq + hq = (b * Hkv + hk) * rep + hh)
   if (i >= per_head4 || hq >= heads_q) return;
@@ -107,6 +109,7 @@ __global__ void spread_to_group_kernel(const float* __restrict__ x_kv, float* __
 // status word there (a bounded wait that ran out, a rescue list that overflowed) is copied into the caller's status word,
 // which is the one vsa2_device_status reads.
 __global__ void merge_status_kernel(const StatusBlock* __restrict__ from, StatusBlock* __restrict__ into) {
+  grid_enter();
   const int s = from->status;
   if (s != 0) atomicCAS(&into->status, 0, s);
 }
@@ -129,7 +132,7 @@ cudaError_t launch_coarse_fwd_pooled(const Geo& g, const float* qc, const float*
   if ((e = launch_fine_fwd_tc(p, q16, k16, v16, nullptr, ptr, idx, nullptr, oc_hat, nullptr, lse_c,
                               reinterpret_cast<StatusBlock*>(ws + lay.status), st)) != cudaSuccess)
     return e;
-  merge_status_kernel<<<1, 1, 0, st>>>(reinterpret_cast<const StatusBlock*>(ws + lay.status), caller_status);
+  launch_kernel(merge_status_kernel, 1, 1, 0, st, reinterpret_cast<const StatusBlock*>(ws + lay.status), caller_status);
   return cudaGetLastError();
 }
 
@@ -165,11 +168,11 @@ cudaError_t launch_coarse_bwd_pooled(const Geo& g, const float* qc, const float*
   if (grouped) {
     const size_t per_head4 = (size_t)g.N * g.D / 4;
     dim3 grid((unsigned)((per_head4 + 255) / 256), (unsigned)BHq);
-    spread_to_group_kernel<<<grid, 256, 0, st>>>(dk_kv, dkc, g.rep, per_head4, (int)BHq);
-    spread_to_group_kernel<<<grid, 256, 0, st>>>(dv_kv, dvc, g.rep, per_head4, (int)BHq);
+    launch_kernel(spread_to_group_kernel, grid, 256, 0, st, dk_kv, dkc, g.rep, per_head4, (int)BHq);
+    launch_kernel(spread_to_group_kernel, grid, 256, 0, st, dv_kv, dvc, g.rep, per_head4, (int)BHq);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  merge_status_kernel<<<1, 1, 0, st>>>(status, caller_status);
+  launch_kernel(merge_status_kernel, 1, 1, 0, st, status, caller_status);
   return cudaGetLastError();
 }
 

@@ -53,6 +53,33 @@ struct StatusBlock {
   int pad[62];
 };
 
+// Kernels of a call follow one another on one stream, up to 40 of them, and on small problems most take a few microseconds.  Each is
+// launched so that its CTAs may be placed as soon as all CTAs of the kernel before it have started (and finds room), and waits
+// in grid_enter for that kernel's completion and its writes: what is left between two kernels is that wait instead of a launch.
+// Every kernel enters that way first of all, also one that has nothing to do: its completion then stands for all before it.
+template <typename T> struct NotDeduced { using type = T; };
+template <typename... P>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                 typename NotDeduced<P>::type... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+__device__ __forceinline__ void grid_enter(bool early = true) {
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Persistent kernels with many items per CTA keep the SMs to themselves until they end
+__device__ __forceinline__ void grid_enter_items(int items) { grid_enter(items <= 8 * (int)gridDim.x); }
+
 // Brackets the launches of one kernel group: counts them and records the caller's timing events.
 struct ProfScope {
   int id;

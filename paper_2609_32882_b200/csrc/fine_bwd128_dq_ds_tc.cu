@@ -40,6 +40,7 @@ static_assert(sizeof(DqDs128Misc) <= 1024, "misc region too small");
 template <int D>
 __global__ void __launch_bounds__(kW2DsThreads, 1)
 fine_bwd128_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, Geo g, long long cap, DqDsArgs a) {
+  grid_enter_items(a.items);
   using C = DqDs128<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -242,11 +243,11 @@ cudaError_t launch_fine_bwd128_dq_ds(const Geo& g, long long cap, const void* k1
   if (g.D == 128) {
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_bwd128_dq_ds_kernel<128>, attr, DqDs128<128>::smem_bytes))) return e;
-    fine_bwd128_dq_ds_kernel<128><<<grid, kW2DsThreads, DqDs128<128>::smem_bytes, st>>>(tk, g, cap, a);
+    launch_kernel(fine_bwd128_dq_ds_kernel<128>, grid, kW2DsThreads, DqDs128<128>::smem_bytes, st, tk, g, cap, a);
   } else {
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_bwd128_dq_ds_kernel<64>, attr, DqDs128<64>::smem_bytes))) return e;
-    fine_bwd128_dq_ds_kernel<64><<<grid, kW2DsThreads, DqDs128<64>::smem_bytes, st>>>(tk, g, cap, a);
+    launch_kernel(fine_bwd128_dq_ds_kernel<64>, grid, kW2DsThreads, DqDs128<64>::smem_bytes, st, tk, g, cap, a);
   }
   return cudaGetLastError();
 }

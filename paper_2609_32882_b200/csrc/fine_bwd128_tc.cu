@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(kW2Threads, 1)
 fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_constant__ CUtensorMap tm_x1,
                       const __grid_constant__ CUtensorMap tm_y0, const __grid_constant__ CUtensorMap tm_y1, Geo g,
                       Bwd128Args a) {
+  grid_enter_items(a.items);
   using C = Bwd128<D>;
   static_assert(PASS == 0 || !SPLIT, "the dK/dV pass has no room for the low-order parts of P and dS");
   static_assert(!F16 || !SPLIT, "the fp16 forms carry no pairs");
@@ -807,7 +808,7 @@ static cudaError_t launch_bwd128(const CUtensorMap& x0, const CUtensorMap& x1, c
   if ((e = prepare_kernel((const void*)fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE>, attr, Bwd128<D>::smem_bytes, kW2Threads,
                           256 * 56 + 256 * 200)))
     return e;
-  fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE><<<grid, kW2Threads, Bwd128<D>::smem_bytes, st>>>(x0, x1, y0, y1, g, a);
+  launch_kernel(fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE>, grid, kW2Threads, Bwd128<D>::smem_bytes, st, x0, x1, y0, y1, g, a);
   return cudaGetLastError();
 }
 

@@ -119,6 +119,16 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                        const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot,
                        const __grid_constant__ CUtensorMap tm_qe, const __grid_constant__ CUtensorMap tm_doe, Geo g,
                        DkvArgs a) {
+  // The launch of the few long lists lets the launch of the others (disjoint outputs, nothing read from this one) take the SMs as its
+  // CTAs leave them, once what both read is there; that one waits for this one at its end, so that what follows waits for both.
+  if (SPLIT && a.overlap == 1) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  } else if (!SPLIT && F16 == 0 && a.overlap == 2) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  } else {
+    grid_enter_items(a.items);
+  }
   constexpr int RA = SPLIT ? 2 : kRingA;                   // slots of the Q ring
   // accumulators: without SPLIT two sets of dK^T, dV^T (64 columns each), used by item parity
   constexpr uint32_t TM_DK = 256, TM_DV = SPLIT ? 384 : 320, TM_SET = 128, SETS = SPLIT ? 1 : 2;
@@ -136,10 +146,10 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int rep = MHA ? 1 : g.rep;
   constexpr bool STORES_DS = F16 == 1 || F16 == 2 || (SPLIT && !MHA);
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
-  if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) return;     // (the flag is final before this launch starts)
-  // the launch of the few long lists lets the launch of the others (disjoint outputs, nothing read from this one) take the SMs as its
-  // CTAs leave them
-  if (SPLIT && a.overlap == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) {     // (the flag is final before this launch starts)
+    if (!SPLIT && F16 == 0 && a.overlap == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
 
   if (tid == 0) {
     bwd_init_barriers(misc);
@@ -706,7 +716,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = overlap == 2 ? 1 : 0;
+    cfg.numAttrs = 1;
     const int items = groups * g.N;
     cfg.gridDim = dim3(items < sms ? items : sms);
     cfg.blockDim = dim3(kDkvThreads);
@@ -794,6 +804,7 @@ PackedCubes packed_cubes(const Geo& g, const int* full) {
 // but the text blocks (nothing of it is packed then)
 __global__ void __launch_bounds__(256) full_counts_kernel(int N, int Nvid, int first, long long cap, const int* __restrict__ ptr,
                                                           const int* __restrict__ idx, int* __restrict__ full) {
+  grid_enter();
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (j >= N) return;
   const size_t bh = blockIdx.y;
@@ -810,7 +821,7 @@ __global__ void __launch_bounds__(256) full_counts_kernel(int N, int Nvid, int f
   if (lane == 0) full[bh * N + j] = last + 1 == n ? n : k;
 }
 cudaError_t launch_full_counts(const Geo& g, const PackedCubes& pk, const int* ptr, const int* idx, int* full, cudaStream_t st) {
-  full_counts_kernel<<<dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st>>>(g.N, g.Nvid, pk.first, g.nnz_cap, ptr, idx, full);
+  launch_kernel(full_counts_kernel, dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st, g.N, g.Nvid, pk.first, g.nnz_cap, ptr, idx, full);
   return cudaGetLastError();
 }
 

@@ -45,6 +45,7 @@ template <int D>
 __global__ void __launch_bounds__(kDsThreads, 1)
 fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_kt, Geo g,
                       DqDsArgs a) {
+  grid_enter_items(a.items);
   using C = DqDs<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -236,6 +237,7 @@ __global__ void __launch_bounds__(256) ds_positions_kernel(int N, long long cap,
                                                            const int* __restrict__ col_idx, const int* __restrict__ col_ptr,
                                                            const int* __restrict__ row_idx, int* __restrict__ pos,
                                                            int* __restrict__ counters, int n_counters) {
+  grid_enter();
   if (blockIdx.x == 0 && blockIdx.y == 0)
     for (int c = threadIdx.x; c < n_counters; c += blockDim.x) counters[c] = 0;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -258,7 +260,7 @@ __global__ void __launch_bounds__(256) ds_positions_kernel(int N, long long cap,
 
 cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col_idx, const int* col_ptr, const int* row_idx, int* pos,
                                 int* counters, int n_counters, cudaStream_t st) {
-  ds_positions_kernel<<<dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st>>>(g.N, g.nnz_cap, row_ptr, col_idx, col_ptr, row_idx, pos,
+  launch_kernel(ds_positions_kernel, dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st, g.N, g.nnz_cap, row_ptr, col_idx, col_ptr, row_idx, pos,
                                                                          counters, n_counters);
   return cudaGetLastError();
 }
@@ -268,6 +270,7 @@ cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col
 // items last ends with most SMs idle (720p, budget of 16..256 cubes, four heads a group: 0.7 ms for the mean item of a
 // 6 ms launch).  Counting sort by one block per group; the order of equal lengths depends on the run, the results do not.
 __global__ void __launch_bounds__(1024) dkv_order_kernel(Geo g, const int* __restrict__ col_ptr, int* __restrict__ order) {
+  grid_enter();
   __shared__ int hist[1024], warp_sums[32], longest;
   const int bhk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   auto length = [&](int r) {
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(1024) dkv_order_kernel(Geo g, const int* __res
 }
 
 cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st) {
-  dkv_order_kernel<<<g.batch * g.Hkv, 1024, 0, st>>>(g, col_ptr, order);
+  launch_kernel(dkv_order_kernel, g.batch * g.Hkv, 1024, 0, st, g, col_ptr, order);
   return cudaGetLastError();
 }
 
@@ -327,7 +330,7 @@ cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds,
   do {                                                                                                                           \
     static KernelAttr attr_;                                                                                                     \
     if ((e = prepare_kernel((const void*)fine_bwd_dq_ds_kernel<DD>, attr_, DqDs<DD>::smem_bytes))) return e;                     \
-    fine_bwd_dq_ds_kernel<DD><<<grid, kDsThreads, DqDs<DD>::smem_bytes, st>>>(tk, tkt, g, a);                               \
+    launch_kernel(fine_bwd_dq_ds_kernel<DD>, grid, kDsThreads, DqDs<DD>::smem_bytes, st, tk, tkt, g, a);                               \
   } while (0)
   if (g.D == 128) VSA2_LAUNCH_DQ_DS(128);
   else VSA2_LAUNCH_DQ_DS(64);

@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
                                                                const uint4* __restrict__ xb, uint4* __restrict__ yb, size_t nb,
                                                                const int* __restrict__ b_exp, unsigned b_group, int* range_flag,
                                                                DsScale scale, int groups, int per_group, int reducers) {
+  grid_enter();
   const size_t stride = (size_t)(gridDim.x - reducers) * blockDim.x, n = na + nb;
   bool bad = false;
   if ((int)blockIdx.x < reducers) {
@@ -175,6 +176,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                       const __grid_constant__ CUtensorMap tm_qt, const __grid_constant__ CUtensorMap tm_kt,
                       const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot, Geo g,
                       DqArgs a) {
+  grid_enter_items(g.batch * g.Hq * g.N);
   using C = BwdTc<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -560,7 +562,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
   do {                                                                                                                           \
     static KernelAttr attr_;                                                                                                     \
     if ((e = prepare_kernel((const void*)fine_bwd_dq_tc_kernel<DD, SP, F>, attr_, BwdTc<DD>::smem_bytes))) return e;             \
-    fine_bwd_dq_tc_kernel<DD, SP, F><<<grid, kDqThreads, BwdTc<DD>::smem_bytes, st>>>(TQ, TK, tv, tdo, TQT, TKT, tvt, tdot, g, a); \
+    launch_kernel(fine_bwd_dq_tc_kernel<DD, SP, F>, grid, kDqThreads, BwdTc<DD>::smem_bytes, st, TQ, TK, tv, tdo, TQT, TKT, tvt, tdot, g, a); \
   } while (0)
   if (f16) {
     if ((e = launch_cast_qk(g, q, q16, k, k16, *scale, flag, st)) != cudaSuccess) return e;
@@ -609,7 +611,7 @@ static cudaError_t launch_cast(const bf16* a, void* a16, size_t na, const bf16* 
   // (element counts are multiples of the head dimension)
   const int reducers = groups < sms ? groups : sms;
   auto* kernel = b_exp != nullptr ? cast_bf16_to_f16_kernel<true> : cast_bf16_to_f16_kernel<false>;
-  kernel<<<sms * 16 + reducers, 256, 0, st>>>(reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
+  launch_kernel(kernel, sms * 16 + reducers, 256, 0, st, reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
                                                      reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8, b_exp,
                                                      (unsigned)(b_group / 8), range_flag, scale, groups, per_group, reducers);
   return cudaGetLastError();

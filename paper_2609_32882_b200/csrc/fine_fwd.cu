@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(256) fine_fwd_kernel(const bf16* __restrict__ 
                                                        const int* __restrict__ row_ptr, const int* __restrict__ col_idx,
                                                        const float* __restrict__ oc_hat, Geo g, void* __restrict__ o,
                                                        bf16* __restrict__ o_res, float* __restrict__ lse) {
+  grid_enter();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   fine_fwd_block<D>(smem_raw, blockIdx.x, blockIdx.y, blockIdx.z, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
 }
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(256) fine_fwd_list_kernel(const int* __restric
                                                             const int* __restrict__ row_ptr, const int* __restrict__ col_idx,
                                                             const float* __restrict__ oc_hat, Geo g, void* __restrict__ o,
                                                             bf16* __restrict__ o_res, float* __restrict__ lse) {
+  grid_enter();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int n = min(*count, cap);
   for (int e = blockIdx.x; e < n; e += gridDim.x) {
@@ -159,12 +161,12 @@ cudaError_t launch_fine_fwd_list(const Geo& g, const int* count, int cap, const 
     size_t smb = FineFwdSmem<128>::bytes;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_list_kernel<128>, attr, smb))) return e;
-    fine_fwd_list_kernel<128><<<64, 256, smb, st>>>(count, cap, items, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
+    launch_kernel(fine_fwd_list_kernel<128>, 64, 256, smb, st, count, cap, items, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   } else {
     size_t smb = FineFwdSmem<64>::bytes;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_list_kernel<64>, attr, smb))) return e;
-    fine_fwd_list_kernel<64><<<64, 256, smb, st>>>(count, cap, items, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
+    launch_kernel(fine_fwd_list_kernel<64>, 64, 256, smb, st, count, cap, items, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   }
   return cudaGetLastError();
 }
@@ -178,12 +180,12 @@ cudaError_t launch_fine_fwd(const Geo& g, const bf16* q, const bf16* k, const bf
     size_t smb = FineFwdSmem<128>::bytes;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_kernel<128>, attr, smb))) return e;
-    fine_fwd_kernel<128><<<grid, 256, smb, st>>>(q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
+    launch_kernel(fine_fwd_kernel<128>, grid, 256, smb, st, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   } else {
     size_t smb = FineFwdSmem<64>::bytes;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_kernel<64>, attr, smb))) return e;
-    fine_fwd_kernel<64><<<grid, 256, smb, st>>>(q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
+    launch_kernel(fine_fwd_kernel<64>, grid, 256, smb, st, q, k, v, gate, row_ptr, col_idx, oc_hat, g, o, o_res, lse);
   }
   return cudaGetLastError();
 }

@@ -100,6 +100,7 @@ template <int D>
 __global__ void __launch_bounds__(kF2Threads, 1)
 fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, Geo g, FwdRows2Args a) {
+  grid_enter_items(g.batch * g.Hq * g.N / 2);
   using C = FwdRows2<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -547,12 +548,12 @@ cudaError_t launch_fine_fwd_rows2_tc(const Geo& g, bool pair_heads, const bf16* 
     if (smb > 227 * 1024) return cudaErrorInvalidValue;
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<128>, attr, smb, kF2Threads, 256 * 56 + 256 * 200))) return e;
-    fine_fwd_rows2_tc_kernel<128><<<grid, kF2Threads, smb, st>>>(tq, tk, tv, g, a);
+    launch_kernel(fine_fwd_rows2_tc_kernel<128>, grid, kF2Threads, smb, st, tq, tk, tv, g, a);
   } else {
     const size_t smb = FwdRows2<64>::smem_bytes(g.N);
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<64>, attr, smb, kF2Threads, 256 * 56 + 256 * 200))) return e;
-    fine_fwd_rows2_tc_kernel<64><<<grid, kF2Threads, smb, st>>>(tq, tk, tv, g, a);
+    launch_kernel(fine_fwd_rows2_tc_kernel<64>, grid, kF2Threads, smb, st, tq, tk, tv, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_fine_fwd_list(g, a.rescue_count, a.rescue_cap, a.rescue_items, q, k, v, gate, row_ptr, col_idx, oc_hat, o, o_res, lse, st);

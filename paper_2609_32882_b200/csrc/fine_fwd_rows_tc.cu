@@ -106,6 +106,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                         const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_qt,
                         const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt, Geo g,
                         FwdRowsArgs a) {
+  grid_enter_items(g.batch * g.Hq * g.N);
   using C = FwdRows<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -655,12 +656,12 @@ cudaError_t launch_fine_fwd_rows_tc(const Geo& g, const bf16* q, const bf16* k, 
     const size_t smb = FwdRows<128>::smem_bytes(g.N);
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_rows_tc_kernel<128>, attr, smb, kFrThreads, 256 * 56 + 256 * 200))) return e;
-    fine_fwd_rows_tc_kernel<128><<<grid, kFrThreads, smb, st>>>(tq, tk, tv, tqt, tkt, tvt, g, a);
+    launch_kernel(fine_fwd_rows_tc_kernel<128>, grid, kFrThreads, smb, st, tq, tk, tv, tqt, tkt, tvt, g, a);
   } else {
     const size_t smb = FwdRows<64>::smem_bytes(g.N);
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_rows_tc_kernel<64>, attr, smb, kFrThreads, 256 * 56 + 256 * 200))) return e;
-    fine_fwd_rows_tc_kernel<64><<<grid, kFrThreads, smb, st>>>(tq, tk, tv, tqt, tkt, tvt, g, a);
+    launch_kernel(fine_fwd_rows_tc_kernel<64>, grid, kFrThreads, smb, st, tq, tk, tv, tqt, tkt, tvt, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // query blocks whose row sums left the safe range are redone with the exact running maximum

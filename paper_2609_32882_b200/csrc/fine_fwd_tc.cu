@@ -92,6 +92,7 @@ template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fine_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, Geo g, FwdArgs a) {
+  grid_enter();
   using C = FwdTc<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -556,12 +557,12 @@ cudaError_t launch_fine_fwd_tc(const Geo& g, const bf16* q, const bf16* k, const
     const size_t smb = FwdTc<128>::smem_bytes(g.N);
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_tc_kernel<128>, attr, smb, kFwdThreads, 256 * 56 + 256 * 200))) return e;
-    fine_fwd_tc_kernel<128><<<grid, kFwdThreads, smb, st>>>(tq, tk, tv, g, a);
+    launch_kernel(fine_fwd_tc_kernel<128>, grid, kFwdThreads, smb, st, tq, tk, tv, g, a);
   } else {
     const size_t smb = FwdTc<64>::smem_bytes(g.N);
     static KernelAttr attr;
     if ((e = prepare_kernel((const void*)fine_fwd_tc_kernel<64>, attr, smb, kFwdThreads, 256 * 56 + 256 * 200))) return e;
-    fine_fwd_tc_kernel<64><<<grid, kFwdThreads, smb, st>>>(tq, tk, tv, g, a);
+    launch_kernel(fine_fwd_tc_kernel<64>, grid, kFwdThreads, smb, st, tq, tk, tv, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // query blocks whose row sums left the safe range are redone with the exact running maximum

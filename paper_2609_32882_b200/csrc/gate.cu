@@ -69,6 +69,7 @@ __device__ __forceinline__ void scatter_w(bf16* ws, uint4 v, int i, int Hq, RowO
 __global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* __restrict__ gate, const float* __restrict__ dgate,
                                                              int L, int Lp, int Hq, int HP, bf16* __restrict__ dz_hm,
                                                              bf16* __restrict__ dz_tm) {
+  grid_enter();
   extern __shared__ __align__(16) unsigned char gate_dz_smem[];
   bf16* tile = reinterpret_cast<bf16*>(gate_dz_smem);          // [HP][64 + 8]
   constexpr int LD = kGtTok + 8;
@@ -105,6 +106,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* __rest
 template <int NT, int MW, int HW, int CH>
 __global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, int L,
                                                               int C, int Hq, float* __restrict__ gate) {
+  grid_enter();
   static_assert(NT % HW == 0 && MW * HW * 32 <= kGtThreads, "warps of a CTA");
   constexpr int LDW = NT * 8 + 8;                           // 16-byte aligned rows, eight rows on different banks
   constexpr int NTW = NT / HW, GROUPS = CH / 32;
@@ -220,6 +222,7 @@ template <int KT>
 __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __restrict__ w, const bf16* __restrict__ dz_tm,
                                                                  int L, int Lp, int C, int Hq, int per_slice, int out_f32,
                                                                  void* __restrict__ dx) {
+  grid_enter();
   constexpr int LDZ = KT * 16 + 8;
   __shared__ __align__(16) bf16 az[kGtTok * LDZ];            // dz^T: [token][head]
   __shared__ __align__(16) bf16 ws[kDxCh * LDZ];             // W chunk: [channel][head]
@@ -303,6 +306,7 @@ template <int NT>
 __global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dz_hm,
                                                                  int L, int Lp, int C, int Hq, int HP,
                                                                  float* __restrict__ partial) {
+  grid_enter();
   constexpr int LDZ = kGtTok + 8;
   __shared__ __align__(16) bf16 xs[kGtTok * kLdx];           // [token][channel]; read transposed by ldmatrix
   __shared__ __align__(16) bf16 dz[NT * 8 * LDZ];            // [head][token]
@@ -386,6 +390,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* __r
 }
 
 __global__ void gate_reduce_dw_kernel(const float* __restrict__ partial, int parts, size_t n, float* __restrict__ dw) {
+  grid_enter();
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   float acc = 0.f;
@@ -419,8 +424,8 @@ cudaError_t launch_gate_fwd(int batch, int L, int C, int Hq, const bf16* x, cons
   const int nt = (Hq + 7) / 8;
 #define VSA2_GATE_FWD(NT_, HW_)                                                                                  \
   do {                                                                                                           \
-    if (few) gate_fwd_kernel<NT_, 1, HW_, 256><<<grid, kGtThreads, 0, st>>>(x, w, L, C, Hq, gate);               \
-    else gate_fwd_kernel<NT_, 4, 1, 128><<<grid, kGtThreads, 0, st>>>(x, w, L, C, Hq, gate);                     \
+    if (few) launch_kernel(gate_fwd_kernel<NT_, 1, HW_, 256>, grid, kGtThreads, 0, st, x, w, L, C, Hq, gate);               \
+    else launch_kernel(gate_fwd_kernel<NT_, 4, 1, 128>, grid, kGtThreads, 0, st, x, w, L, C, Hq, gate);                     \
   } while (0)
   if (nt <= 1) VSA2_GATE_FWD(1, 1);
   else if (nt <= 2) VSA2_GATE_FWD(2, 2);
@@ -439,7 +444,7 @@ cudaError_t launch_gate_bwd(int batch, int L, int C, int Hq, int out_f32, const 
   unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace);
   bf16* dz_hm = reinterpret_cast<bf16*>(wsb + align_up((size_t)batch * kGtSplits * C * Hq * sizeof(float), 256));
   bf16* dz_tm = reinterpret_cast<bf16*>(reinterpret_cast<unsigned char*>(dz_hm) + dz_bytes(batch, L, Hq));
-  gate_dz_kernel<<<dim3(Lp / kGtTok, batch), kGtThreads, (size_t)HP * (kGtTok + 8) * sizeof(bf16), st>>>(gate, dgate, L, Lp, Hq,
+  launch_kernel(gate_dz_kernel, dim3(Lp / kGtTok, batch), kGtThreads, (size_t)HP * (kGtTok + 8) * sizeof(bf16), st, gate, dgate, L, Lp, Hq,
                                                                                                    HP, dz_hm, dz_tm);
   {
     // channel slices until there are eight CTAs per SM (a chunk is the least a CTA takes)
@@ -452,7 +457,7 @@ cudaError_t launch_gate_bwd(int batch, int L, int C, int Hq, int out_f32, const 
     const int per_slice = (chunks + slices - 1) / slices * kDxCh;
     dim3 grid((L + kGtTok - 1) / kGtTok, batch, (C + per_slice - 1) / per_slice);
     const int kt = (Hq + 15) / 16;
-#define VSA2_GATE_DX(KT_) gate_bwd_dx_kernel<KT_><<<grid, kGtThreads, 0, st>>>(w, dz_tm, L, Lp, C, Hq, per_slice, out_f32, dx)
+#define VSA2_GATE_DX(KT_) launch_kernel(gate_bwd_dx_kernel<KT_>, grid, kGtThreads, 0, st, w, dz_tm, L, Lp, C, Hq, per_slice, out_f32, dx)
     if (kt <= 1) VSA2_GATE_DX(1);
     else if (kt <= 2) VSA2_GATE_DX(2);
     else if (kt <= 3) VSA2_GATE_DX(3);
@@ -462,7 +467,7 @@ cudaError_t launch_gate_bwd(int batch, int L, int C, int Hq, int out_f32, const 
   {
     dim3 grid((C + kGtCh - 1) / kGtCh, kGtSplits, batch);
     const int nt = (Hq + 7) / 8;
-#define VSA2_GATE_DW(NT_) gate_bwd_dw_kernel<NT_><<<grid, kGtThreads, 0, st>>>(x, dz_hm, L, Lp, C, Hq, HP, partial)
+#define VSA2_GATE_DW(NT_) launch_kernel(gate_bwd_dw_kernel<NT_>, grid, kGtThreads, 0, st, x, dz_hm, L, Lp, C, Hq, HP, partial)
     if (nt <= 1) VSA2_GATE_DW(1);
     else if (nt <= 2) VSA2_GATE_DW(2);
     else if (nt <= 4) VSA2_GATE_DW(4);
@@ -472,7 +477,7 @@ cudaError_t launch_gate_bwd(int batch, int L, int C, int Hq, int out_f32, const 
 #undef VSA2_GATE_DW
   }
   const size_t n = (size_t)C * Hq;
-  gate_reduce_dw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(partial, batch * kGtSplits, n, d_w);
+  launch_kernel(gate_reduce_dw_kernel, (unsigned)((n + 255) / 256), 256, 0, st, partial, batch * kGtSplits, n, d_w);
   return cudaGetLastError();
 }
 

@@ -46,6 +46,7 @@ __device__ __forceinline__ void load8(const bf16* base, int t, int h, int w, con
 
 template <int D>
 __global__ void __launch_bounds__(128) pool_kernel(PoolJobs jobs, Geo g) {
+  grid_enter();
   constexpr int CH = D / 8;            // 16-byte chunks of a token row
   constexpr int CUBES = 128 / CH;      // cubes per CTA
   clear_status(jobs);
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(128) pool_kernel(PoolJobs jobs, Geo g) {
 constexpr int kSubThreads = 128;
 template <int D>
 __global__ void __launch_bounds__(kSubThreads) pool_subcube_kernel(PoolJobs jobs, Geo g) {
+  grid_enter();
   constexpr int CH = D / 8, SUB = kSubThreads / CH, CUBES = SUB / 8;
   __shared__ __align__(16) float sums[SUB * D];
   clear_status(jobs);
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(kSubThreads) pool_subcube_kernel(PoolJobs jobs
 template <int D>
 __global__ void __launch_bounds__(256) permute_kernel(const bf16* __restrict__ src, int heads, Geo g, int inverse,
                                                       bf16* __restrict__ dst) {
+  grid_enter();
   const int n = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const size_t bh = (size_t)b * heads + h;
   const int B = g.Bt * g.Bh * g.Bw;
@@ -206,8 +209,8 @@ __global__ void __launch_bounds__(256) permute_kernel(const bf16* __restrict__ s
 
 cudaError_t launch_permute(const Geo& g, const bf16* src, int heads, bool inverse, bf16* dst, cudaStream_t st) {
   dim3 grid(g.N, heads, g.batch);
-  if (g.D == 128) permute_kernel<128><<<grid, 256, 0, st>>>(src, heads, g, inverse ? 1 : 0, dst);
-  else permute_kernel<64><<<grid, 256, 0, st>>>(src, heads, g, inverse ? 1 : 0, dst);
+  if (g.D == 128) launch_kernel(permute_kernel<128>, grid, 256, 0, st, src, heads, g, inverse ? 1 : 0, dst);
+  else launch_kernel(permute_kernel<64>, grid, 256, 0, st, src, heads, g, inverse ? 1 : 0, dst);
   return cudaGetLastError();
 }
 
@@ -220,12 +223,12 @@ static cudaError_t launch_pool_jobs(const Geo& g, const PoolJobs& jobs, cudaStre
   if (r222 && g.G == 8) {          // (blocks of 64 tokens have eight such sub-cubes whatever the cube's shape)
     const int per_cta = kSubThreads / g.D;
     dim3 sub_grid((g.N + per_cta - 1) / per_cta, heads, g.batch);
-    if (g.D == 128) pool_subcube_kernel<128><<<sub_grid, kSubThreads, 0, st>>>(jobs, g);
-    else pool_subcube_kernel<64><<<sub_grid, kSubThreads, 0, st>>>(jobs, g);
+    if (g.D == 128) launch_kernel(pool_subcube_kernel<128>, sub_grid, kSubThreads, 0, st, jobs, g);
+    else launch_kernel(pool_subcube_kernel<64>, sub_grid, kSubThreads, 0, st, jobs, g);
     return cudaGetLastError();
   }
-  if (g.D == 128) pool_kernel<128><<<grid, 128, 0, st>>>(jobs, g);
-  else pool_kernel<64><<<grid, 128, 0, st>>>(jobs, g);
+  if (g.D == 128) launch_kernel(pool_kernel<128>, grid, 128, 0, st, jobs, g);
+  else launch_kernel(pool_kernel<64>, grid, 128, 0, st, jobs, g);
   return cudaGetLastError();
 }
 

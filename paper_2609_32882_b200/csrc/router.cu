@@ -21,6 +21,7 @@ struct RouterSmem {
 template <int D, int PASS>
 __global__ void __launch_bounds__(256) router_kernel(const bf16* __restrict__ qr, const bf16* __restrict__ kr, Geo g,
                                                      float* __restrict__ lse_r, float* __restrict__ pr) {
+  grid_enter();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using SM = RouterSmem<D>;
   bf16* Qs = reinterpret_cast<bf16*>(smem_raw);
@@ -130,20 +131,20 @@ cudaError_t launch_router_scores(const Geo& g, const bf16* qr, const bf16* kr, f
     if ((e = cudaFuncSetAttribute(router_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
     {
       ProfScope ps(VSA2_KERNEL_ROUTER_LSE, st, 1);
-      router_kernel<128, 1><<<grid, 256, sm, st>>>(qr, kr, g, lse_r, pr);
+      launch_kernel(router_kernel<128, 1>, grid, 256, sm, st, qr, kr, g, lse_r, pr);
     }
     ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);
-    router_kernel<128, 2><<<grid, 256, sm, st>>>(qr, kr, g, lse_r, pr);
+    launch_kernel(router_kernel<128, 2>, grid, 256, sm, st, qr, kr, g, lse_r, pr);
   } else {
     size_t sm = RouterSmem<64>::bytes;
     if ((e = cudaFuncSetAttribute(router_kernel<64, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
     if ((e = cudaFuncSetAttribute(router_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
     {
       ProfScope ps(VSA2_KERNEL_ROUTER_LSE, st, 1);
-      router_kernel<64, 1><<<grid, 256, sm, st>>>(qr, kr, g, lse_r, pr);
+      launch_kernel(router_kernel<64, 1>, grid, 256, sm, st, qr, kr, g, lse_r, pr);
     }
     ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);
-    router_kernel<64, 2><<<grid, 256, sm, st>>>(qr, kr, g, lse_r, pr);
+    launch_kernel(router_kernel<64, 2>, grid, 256, sm, st, qr, kr, g, lse_r, pr);
   }
   return cudaGetLastError();
 }

@@ -236,6 +236,7 @@ template <int D, int G, bool FOLD, bool ONE>
 __global__ void __launch_bounds__(kRtThreads, 1)
 router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, Geo g,
                  float* __restrict__ pr, RouterOne one, StatusBlock* status) {
+  grid_enter_items(g.batch * g.Hq * ((g.N * G + kRtTile - 1) / kRtTile));
   static_assert(!FOLD || G == 8, "half-cubes of 8 sub-cubes");
   static_assert(!ONE || G == 8, "a thread parks the sums of four cubes");
   constexpr int PASSES = ONE ? 1 : 2;
@@ -556,7 +557,7 @@ static cudaError_t launch_router(const CUtensorMap& tq, const CUtensorMap& tk, c
   static KernelAttr attr;
   if ((e = prepare_kernel((const void*)router_tc_kernel<D, G, FOLD, ONE>, attr, smb))) return e;
   const int total = g.batch * g.Hq * row_tiles;
-  router_tc_kernel<D, G, FOLD, ONE><<<total < sms ? total : sms, kRtThreads, smb, st>>>(tq, tk, g, pr, one, status);
+  launch_kernel(router_tc_kernel<D, G, FOLD, ONE>, total < sms ? total : sms, kRtThreads, smb, st, tq, tk, g, pr, one, status);
   return cudaGetLastError();
 }
 
@@ -618,6 +619,7 @@ struct RouterExactArgs {
 
 template <int D, bool FOLD>
 __global__ void __launch_bounds__(128) router_exact_kernel(Geo g, RouterExactArgs a) {
+  grid_enter();
   using C = RouterTc<D>;
   constexpr int ROWS = FOLD ? 16 : 8, PAIRS = kRtTile / ROWS;      // sub-cubes of a pair's side, pairs of a tile
   extern __shared__ unsigned char smem_raw[];
@@ -741,7 +743,7 @@ cudaError_t launch_router_exact(const Geo& g, bool fold, const bf16* qr, const b
     const size_t smb = 2 * RouterTc<DD>::TILE + 1024;                                                    \
     static KernelAttr attr_;                                                                             \
     if ((e = prepare_kernel((const void*)router_exact_kernel<DD, FF>, attr_, smb))) return e;            \
-    router_exact_kernel<DD, FF><<<sms, 128, smb, st>>>(g, a);                                            \
+    launch_kernel(router_exact_kernel<DD, FF>, sms, 128, smb, st, g, a);                                            \
   } while (0)
   if (g.D == 128 && fold) VSA2_LAUNCH_EXACT(128, true);
   else if (g.D == 128) VSA2_LAUNCH_EXACT(128, false);

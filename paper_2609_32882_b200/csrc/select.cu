@@ -15,6 +15,7 @@ __device__ __forceinline__ unsigned seq_mask(int pass) { return pass == 2 ? 0x3F
 
 // state[bh*8 + ..]: 0 prefix bits, 1 prefix mask, 2 remaining k, 3 tau bits, 4 eq_take
 __global__ void sel_init_kernel(unsigned* state, unsigned* hist, int BH, unsigned keep, const int* redo) {
+  grid_enter();
   if (redo != nullptr && *redo == 0) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < BH * 3 * kHistBins) hist[i] = 0u;
@@ -30,6 +31,7 @@ __global__ void sel_init_kernel(unsigned* state, unsigned* hist, int BH, unsigne
 __global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__ pr, long long n_elems,
                                                        const unsigned* __restrict__ state, unsigned* hist, int pass,
                                                        const int* redo) {
+  grid_enter();
   __shared__ unsigned sh[kHistBins];
   if (redo != nullptr && *redo == 0) return;
   const int bh = blockIdx.y;
@@ -69,6 +71,7 @@ __global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__
 // One warp per (batch, head): finds the digit whose bin holds the `remaining`-th largest entry.  Lane l owns the bins
 // [l * nb/32, (l+1) * nb/32); a suffix sum over the lanes locates the lane, a short serial walk the bin.
 __global__ void __launch_bounds__(32) sel_pick_kernel(unsigned* state, const unsigned* hist, int pass, const int* redo) {
+  grid_enter();
   if (redo != nullptr && *redo == 0) return;
   const int bh = blockIdx.x, lane = threadIdx.x;
   const unsigned* hsrc = hist + ((size_t)bh * 3 + pass) * kHistBins;
@@ -143,6 +146,7 @@ template <bool BAND>
 __global__ void __launch_bounds__(256) sel_row_bits_kernel(const float* __restrict__ pr, int N, int words,
                                                            const unsigned* __restrict__ state, unsigned* bits_gt,
                                                            unsigned* bits_eq, int* row_gt, int* row_eq, Settle se) {
+  grid_enter();
   if (!BAND && se.redo != nullptr && *se.redo == 0) return;
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -202,6 +206,7 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
                                                                  const int* __restrict__ row_eq_take,
                                                                  const int* __restrict__ row_ptr, int* col_idx,
                                                                  unsigned* bitmap, long long nnz_cap) {
+  grid_enter();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int bh = blockIdx.y;
@@ -256,6 +261,7 @@ template <int U, int MODE>
 __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __restrict__ pr, int N, int K,
                                                                 const int* __restrict__ budgets, float* row_tau,
                                                                 int* row_eq_take, int* row_cnt, Settle se) {
+  grid_enter();
   if (MODE == kAllRows && se.redo != nullptr && *se.redo == 0) return;
   const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= (MODE == kListed ? *se.row_count : N)) return;
@@ -319,6 +325,7 @@ template <int MODE>
 __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restrict__ pr, int N, int K,
                                                            const int* __restrict__ budgets, float* row_tau,
                                                            int* row_eq_take, int* row_cnt, Settle se) {
+  grid_enter();
   __shared__ unsigned sh[256];
   __shared__ unsigned s_prefix, s_mask, s_remaining;
   if (MODE == kAllRows && se.redo != nullptr && *se.redo == 0) return;
@@ -418,6 +425,7 @@ __global__ void __launch_bounds__(1024) sel_scan_rows_kernel(int N, int per_sequ
                                                              const int* __restrict__ row_gt, const int* __restrict__ row_eq,
                                                              float* row_tau, int* row_eq_take, int* row_cnt, int* row_ptr,
                                                              long long nnz_cap, StatusBlock* status) {
+  grid_enter();
   __shared__ int ws[33];
   const int bh = blockIdx.x;
   const size_t base = (size_t)bh * N;
@@ -463,6 +471,7 @@ __global__ void __launch_bounds__(256) sel_emit_rows_kernel(const float* __restr
                                                             const int* __restrict__ row_eq_take,
                                                             const int* __restrict__ row_ptr, int* col_idx,
                                                             unsigned* bitmap, long long nnz_cap) {
+  grid_enter();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int bh = blockIdx.y;
@@ -496,6 +505,7 @@ __global__ void __launch_bounds__(256) sel_emit_rows_kernel(const float* __restr
 // one warp per 32 x 32 bit tile, transposed with 32 ballots.  grid (words, ceil(words/8), BH), 256 threads
 __global__ void __launch_bounds__(256) sel_transpose_bitmap_kernel(const unsigned* __restrict__ bitmap, int N, int words,
                                                                    unsigned* __restrict__ bitmap_t) {
+  grid_enter();
   const int lane = threadIdx.x & 31;
   const int wj = blockIdx.x;                                   // word column of the source: columns 32 wj .. 32 wj + 31
   const int wi = blockIdx.y * 8 + (threadIdx.x >> 5);          // word row of the source: rows 32 wi .. 32 wi + 31
@@ -516,6 +526,7 @@ __global__ void __launch_bounds__(256) sel_transpose_bitmap_kernel(const unsigne
 // one warp per column: number of kept rows.  grid (ceil(N/8), BH), 256 threads
 __global__ void __launch_bounds__(256) sel_col_count_kernel(const unsigned* __restrict__ bitmap_t, int N, int words,
                                                             int* col_cnt) {
+  grid_enter();
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y;
   if (j >= N) return;
@@ -528,6 +539,7 @@ __global__ void __launch_bounds__(256) sel_col_count_kernel(const unsigned* __re
 
 __global__ void __launch_bounds__(1024) sel_scan_cols_kernel(int N, const int* __restrict__ col_cnt, int* col_ptr,
                                                              long long nnz_cap) {
+  grid_enter();
   __shared__ int ws[33];
   const int bh = blockIdx.x;
   int carry = 0;
@@ -546,6 +558,7 @@ __global__ void __launch_bounds__(1024) sel_scan_cols_kernel(int N, const int* _
 __global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __restrict__ bitmap_t, int N, int words,
                                                             const int* __restrict__ col_ptr, int* row_idx,
                                                             long long nnz_cap) {
+  grid_enter();
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y;
   if (j >= N) return;
@@ -571,6 +584,7 @@ __global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __re
 // scores (ties to the lower index) and takes what is not kept out of the bitmap and the counts.  One block per head.
 __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restrict__ pr, int N, int words, unsigned keep, unsigned* state,
                                                           const int* __restrict__ row_gt, int* row_eq, unsigned* bits_eq, Settle se) {
+  grid_enter();
   __shared__ int ws[33];
   __shared__ int at[kBandHead], n_rows;
   __shared__ unsigned val[kBandHead];
@@ -640,6 +654,7 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* __restrict_
                                                         const unsigned* __restrict__ bits_gt, const unsigned* __restrict__ bits_eq,
                                                         int* row_ptr, int* col_idx, int* col_ptr, int* row_idx, long long nnz_cap,
                                                         StatusBlock* status) {
+  grid_enter();
   constexpr int W = kSelOneBlockN / 32;
   __shared__ unsigned bm[kSelOneBlockN * W], bt[kSelOneBlockN * W];
   __shared__ int take_s[kSelOneBlockN], ptr_s[kSelOneBlockN], ws[33];
@@ -749,14 +764,14 @@ static void launch_row_topk(const Geo& g, const float* pr, const int* budgets, c
   const int BH = g.batch * g.Hq, N = g.N;
   const int* bud = g.mode == VSA2_PER_QUERY_BUDGET ? budgets : nullptr;
   const dim3 grid = MODE == kListed ? dim3((unsigned)(((long long)BH * N + 7) / 8)) : dim3((N + 7) / 8, BH);
-#define VSA2_ROW_TOPK(U) sel_row_topk_warp_kernel<U, MODE><<<grid, 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt, se)
+#define VSA2_ROW_TOPK(U) launch_kernel(sel_row_topk_warp_kernel<U, MODE>, grid, 256, 0, st, pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt, se)
   if (N <= 256) VSA2_ROW_TOPK(8);
   else if (N <= 640) VSA2_ROW_TOPK(20);
   else if (N <= 1024) VSA2_ROW_TOPK(32);
   else if (N <= 1536) VSA2_ROW_TOPK(48);
   else if (N <= 2048) VSA2_ROW_TOPK(64);
   else
-    sel_row_topk_kernel<MODE><<<MODE == kListed ? dim3(592) : dim3(N, BH), 256, 0, st>>>(pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt, se);
+    launch_kernel(sel_row_topk_kernel<MODE>, MODE == kListed ? dim3(592) : dim3(N, BH), 256, 0, st, pr, N, g.K, bud, s.row_tau, s.row_eq_take, s.row_cnt, se);
 #undef VSA2_ROW_TOPK
 }
 
@@ -769,15 +784,15 @@ static void launch_thresholds(const Geo& g, const float* pr, const int* budgets,
     const unsigned keep = (unsigned)((long long)N * g.K);
     const int* redo = BAND ? nullptr : se.redo;
     int init_n = BH * 3 * kHistBins;
-    sel_init_kernel<<<(init_n + 255) / 256, 256, 0, st>>>(s.state, s.hist, BH, keep, redo);
+    launch_kernel(sel_init_kernel, (init_n + 255) / 256, 256, 0, st, s.state, s.hist, BH, keep, redo);
     int chunks = (int)((n_elems + 256 * 16 - 1) / (256 * 16));
     if (chunks > 256) chunks = 256;
     for (int pass = 0; pass < 3; ++pass) {
-      sel_hist_kernel<<<dim3(chunks, BH), 256, 0, st>>>(pr, n_elems, s.state, s.hist, pass, redo);
-      sel_pick_kernel<<<BH, 32, 0, st>>>(s.state, s.hist, pass, redo);
+      launch_kernel(sel_hist_kernel, dim3(chunks, BH), 256, 0, st, pr, n_elems, s.state, s.hist, pass, redo);
+      launch_kernel(sel_pick_kernel, BH, 32, 0, st, s.state, s.hist, pass, redo);
     }
     // counts and bitmaps in one read of P_r (the bitmap of the entries equal to tau borrows the transposed bitmap's space)
-    sel_row_bits_kernel<BAND><<<dim3((N + 7) / 8, BH), 256, 0, st>>>(pr, N, s.words, s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq, se);
+    launch_kernel(sel_row_bits_kernel<BAND>, dim3((N + 7) / 8, BH), 256, 0, st, pr, N, s.words, s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq, se);
   } else {
     launch_row_topk<BAND ? kBand : kAllRows>(g, pr, budgets, s, se, st);
   }
@@ -792,7 +807,7 @@ cudaError_t launch_select_settle(const Geo& g, const float* pr, const int* budge
                                  cudaStream_t st) {
   const int BH = g.batch * g.Hq, N = g.N;
   if (g.mode == VSA2_PER_SEQUENCE)
-    sel_settle_kernel<<<BH, 1024, 0, st>>>(pr, N, s.words, (unsigned)((long long)N * g.K), s.state, s.row_gt, s.row_eq, s.bitmap_t, se);
+    launch_kernel(sel_settle_kernel, BH, 1024, 0, st, pr, N, s.words, (unsigned)((long long)N * g.K), s.state, s.row_gt, s.row_eq, s.bitmap_t, se);
   else
     launch_row_topk<kListed>(g, pr, budgets, s, se, st);
   return cudaGetLastError();
@@ -805,24 +820,24 @@ cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, con
   se.redo = const_cast<int*>(redo);
   launch_thresholds<false>(g, pr, budgets, s, se, st);
   if (N <= kSelOneBlockN) {
-    sel_maps_kernel<<<BH, 1024, 0, st>>>(pr, N, s.words, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
+    launch_kernel(sel_maps_kernel, BH, 1024, 0, st, pr, N, s.words, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
                                          s.row_eq_take, s.row_cnt, s.bitmap, s.bitmap_t, row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap,
                                          status);
     return cudaGetLastError();
   }
-  sel_scan_rows_kernel<<<BH, 1024, 0, st>>>(N, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
+  launch_kernel(sel_scan_rows_kernel, BH, 1024, 0, st, N, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
                                             s.row_eq_take, s.row_cnt, row_ptr, g.nnz_cap, status);
   if (g.mode == VSA2_PER_SEQUENCE)
-    sel_emit_rows_bits_kernel<<<dim3((N + 7) / 8, BH), 256, 0, st>>>(N, s.words, s.bitmap_t, s.row_eq_take, row_ptr, col_idx,
+    launch_kernel(sel_emit_rows_bits_kernel, dim3((N + 7) / 8, BH), 256, 0, st, N, s.words, s.bitmap_t, s.row_eq_take, row_ptr, col_idx,
                                                                      s.bitmap, g.nnz_cap);
   else
-    sel_emit_rows_kernel<<<dim3((N + 7) / 8, BH), 256, 0, st>>>(pr, N, s.words, s.row_tau, s.row_eq_take, row_ptr,
+    launch_kernel(sel_emit_rows_kernel, dim3((N + 7) / 8, BH), 256, 0, st, pr, N, s.words, s.row_tau, s.row_eq_take, row_ptr,
                                                                 col_idx, s.bitmap, g.nnz_cap);
   // columns: transposed bitmap, then counts (row_gt reused as scratch), scan, ordered emission
-  sel_transpose_bitmap_kernel<<<dim3(s.words, (s.words + 7) / 8, BH), 256, 0, st>>>(s.bitmap, N, s.words, s.bitmap_t);
-  sel_col_count_kernel<<<dim3((N + 7) / 8, BH), 256, 0, st>>>(s.bitmap_t, N, s.words, s.row_gt);
-  sel_scan_cols_kernel<<<BH, 1024, 0, st>>>(N, s.row_gt, col_ptr, g.nnz_cap);
-  sel_emit_cols_kernel<<<dim3((N + 7) / 8, BH), 256, 0, st>>>(s.bitmap_t, N, s.words, col_ptr, row_idx, g.nnz_cap);
+  launch_kernel(sel_transpose_bitmap_kernel, dim3(s.words, (s.words + 7) / 8, BH), 256, 0, st, s.bitmap, N, s.words, s.bitmap_t);
+  launch_kernel(sel_col_count_kernel, dim3((N + 7) / 8, BH), 256, 0, st, s.bitmap_t, N, s.words, s.row_gt);
+  launch_kernel(sel_scan_cols_kernel, BH, 1024, 0, st, N, s.row_gt, col_ptr, g.nnz_cap);
+  launch_kernel(sel_emit_cols_kernel, dim3((N + 7) / 8, BH), 256, 0, st, s.bitmap_t, N, s.words, col_ptr, row_idx, g.nnz_cap);
   return cudaGetLastError();
 }
 

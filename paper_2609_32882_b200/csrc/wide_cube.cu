@@ -45,6 +45,7 @@ __device__ __forceinline__ int valid_subcubes(const Geo& n, int cube) {
 // pr [BH, 2N, 2N] half-cube scores -> out [BH, N, N].  Eq. 7 divides the sum over a cube pair's valid sub-cube
 // pairs by (valid query sub-cubes of the cube) * G; a half-cube score is the same with its own counts.
 __global__ void __launch_bounds__(256) fold_scores_kernel(Geo n, const float* __restrict__ pr, float* __restrict__ out) {
+  grid_enter();
   const int N = n.N / 2;
   const int c = blockIdx.x;
   const size_t bh = (size_t)blockIdx.z * n.Hq + blockIdx.y;
@@ -61,6 +62,7 @@ __global__ void __launch_bounds__(256) fold_scores_kernel(Geo n, const float* __
 // x64 [BH, 2N, D] half-cube means -> x [BH, N, D] cube means (count-weighted)
 __global__ void __launch_bounds__(256) fold_mean_kernel(Geo n, const float* __restrict__ x64, float* __restrict__ x,
                                                         size_t total) {
+  grid_enter();
   const int D = n.D;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const size_t row = e / D;          // bh * N + c
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(256) fold_mean_kernel(Geo n, const float* __re
 // x64 [BH, 2N, D] -> x [BH, N, D]: sum of the two halves
 __global__ void __launch_bounds__(256) fold_sum_kernel(int D, const float* __restrict__ x64, float* __restrict__ x,
                                                        size_t total) {
+  grid_enter();
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const size_t row = e / D;
     const int d = (int)(e % D);
@@ -87,6 +90,7 @@ __global__ void __launch_bounds__(256) fold_sum_kernel(int D, const float* __res
 // cube's tokens (the consumer divides by the half's own count, which leaves row / cube count as Eq. 1 requires)
 __global__ void __launch_bounds__(256) expand_rows_kernel(Geo n, int by_count, const float* __restrict__ x,
                                                           float* __restrict__ x64, size_t total64) {
+  grid_enter();
   const int D = n.D;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total64; e += (size_t)gridDim.x * blockDim.x) {
     const size_t row64 = e / D;        // bh * 2N + i
@@ -105,6 +109,7 @@ __global__ void __launch_bounds__(256) expand_rows_kernel(Geo n, int by_count, c
 __global__ void __launch_bounds__(128) expand_map_kernel(int N, int Hq, long long cap, const int* __restrict__ ptr,
                                                          const int* __restrict__ idx, int* __restrict__ ptr64,
                                                          int* __restrict__ idx64) {
+  grid_enter();
   const int c = blockIdx.x;
   const size_t bh = (size_t)blockIdx.z * Hq + blockIdx.y;
   const int* p = ptr + bh * (N + 1);
@@ -133,6 +138,7 @@ __global__ void __launch_bounds__(128) expand_map_kernel(int N, int Hq, long lon
 __global__ void __launch_bounds__(128) extend_map_kernel(int Nvid, int NtB, int Hq, long long cap, long long capx,
                                                          const int* __restrict__ ptr, const int* __restrict__ idx,
                                                          int* __restrict__ ptrx, int* __restrict__ idxx) {
+  grid_enter();
   const int r = blockIdx.x, Nx = Nvid + NtB;
   const size_t bh = (size_t)blockIdx.z * Hq + blockIdx.y;
   const int* p = ptr + bh * (Nvid + 1);
@@ -160,6 +166,7 @@ __global__ void __launch_bounds__(128) extend_map_kernel(int Nvid, int NtB, int 
 // the sum over the heads of its group (added in head order), so the selection that follows picks the same set for each
 __global__ void __launch_bounds__(256) group_sum_scores_kernel(float* __restrict__ pr, int rep, size_t per_head, size_t groups,
                                                                const int* redo) {
+  grid_enter();
   if (redo != nullptr && *redo == 0) return;
   const size_t total = groups * per_head;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -180,47 +187,47 @@ int grid_for(size_t total) {
 
 cudaError_t launch_group_sum_scores(const Geo& g, float* pr, const int* redo, cudaStream_t st) {
   const size_t per_head = (size_t)g.N * g.N, groups = (size_t)g.batch * g.Hkv;
-  group_sum_scores_kernel<<<grid_for(groups * per_head), 256, 0, st>>>(pr, g.rep, per_head, groups, redo);
+  launch_kernel(group_sum_scores_kernel, grid_for(groups * per_head), 256, 0, st, pr, g.rep, per_head, groups, redo);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fold_scores(const Geo& narrow, const float* pr64, float* pr, cudaStream_t st) {
   const int N = narrow.N / 2;
   dim3 grid(N, narrow.Hq, narrow.batch);
-  fold_scores_kernel<<<grid, 256, 0, st>>>(narrow, pr64, pr);
+  launch_kernel(fold_scores_kernel, grid, 256, 0, st, narrow, pr64, pr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fold_mean(const Geo& narrow, int heads, const float* x64, float* x, cudaStream_t st) {
   const size_t total = (size_t)narrow.batch * heads * (narrow.N / 2) * narrow.D;
-  fold_mean_kernel<<<grid_for(total), 256, 0, st>>>(narrow, x64, x, total);
+  launch_kernel(fold_mean_kernel, grid_for(total), 256, 0, st, narrow, x64, x, total);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fold_sum(const Geo& narrow, int heads, const float* x64, float* x, cudaStream_t st) {
   const size_t total = (size_t)narrow.batch * heads * (narrow.N / 2) * narrow.D;
-  fold_sum_kernel<<<grid_for(total), 256, 0, st>>>(narrow.D, x64, x, total);
+  launch_kernel(fold_sum_kernel, grid_for(total), 256, 0, st, narrow.D, x64, x, total);
   return cudaGetLastError();
 }
 
 cudaError_t launch_expand_rows(const Geo& narrow, int heads, bool by_count, const float* x, float* x64,
                                cudaStream_t st) {
   const size_t total = (size_t)narrow.batch * heads * narrow.N * narrow.D;
-  expand_rows_kernel<<<grid_for(total), 256, 0, st>>>(narrow, by_count ? 1 : 0, x, x64, total);
+  launch_kernel(expand_rows_kernel, grid_for(total), 256, 0, st, narrow, by_count ? 1 : 0, x, x64, total);
   return cudaGetLastError();
 }
 
 cudaError_t launch_expand_map(const Geo& narrow, const int* ptr, const int* idx, int* ptr64, int* idx64,
                               cudaStream_t st) {
   dim3 grid(narrow.N / 2, narrow.Hq, narrow.batch);
-  expand_map_kernel<<<grid, 128, 0, st>>>(narrow.N / 2, narrow.Hq, narrow.nnz_cap / 4, ptr, idx, ptr64, idx64);
+  launch_kernel(expand_map_kernel, grid, 128, 0, st, narrow.N / 2, narrow.Hq, narrow.nnz_cap / 4, ptr, idx, ptr64, idx64);
   return cudaGetLastError();
 }
 
 cudaError_t launch_extend_map(const Geo& g, int text_blocks, const int* ptr, const int* idx, int* ptrx, int* idxx, long long capx,
                               cudaStream_t st) {
   dim3 grid(g.Nvid + text_blocks, g.Hq, g.batch);
-  extend_map_kernel<<<grid, 128, 0, st>>>(g.Nvid, text_blocks, g.Hq, g.nnz_cap, capx, ptr, idx, ptrx, idxx);
+  launch_kernel(extend_map_kernel, grid, 128, 0, st, g.Nvid, text_blocks, g.Hq, g.nnz_cap, capx, ptr, idx, ptrx, idxx);
   return cudaGetLastError();
 }
 
