@@ -56,7 +56,10 @@ struct StatusBlock {
 // Kernels of a call follow one another on one stream, up to 40 of them, and on small problems most take a few microseconds.  Each is
 // launched so that its CTAs may be placed as soon as all CTAs of the kernel before it have started (and finds room), and waits
 // in grid_enter for that kernel's completion and its writes: what is left between two kernels is that wait instead of a launch.
-// Every kernel enters that way first of all, also one that has nothing to do: its completion then stands for all before it.
+// Every kernel enters that way before it reads or writes global memory, also one that has nothing to do: its completion then stands
+// for all before it.  A kernel with tensor memory lets its successor in only when it has allocated it (or exits): a successor
+// that allocated first would keep it from ending.  The large ones also wait behind their set-up (barriers, tensor memory, tables).
+// 2048-token clip, 12 heads, training: 216 us without, 189 with the wait at the top of every kernel, 183 so; ragged clip 733, 709, 702.
 template <typename T> struct NotDeduced { using type = T; };
 template <typename... P>
 inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -40,13 +40,11 @@ static_assert(sizeof(DqDs128Misc) <= 1024, "misc region too small");
 template <int D>
 __global__ void __launch_bounds__(kW2DsThreads, 1)
 fine_bwd128_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, Geo g, long long cap, DqDsArgs a) {
-  grid_enter_items(a.items);
   using C = DqDs128<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   DqDs128Misc* misc = reinterpret_cast<DqDs128Misc*>(smem + C::OFF_MISC);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) return;       // the fallback computes dQ
 
   if (tid == 0) {
     misc->abort_flag = 0;
@@ -70,6 +68,11 @@ fine_bwd128_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, Geo g, long l
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  grid_enter_items(a.items);
+  if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) {       // the fallback computes dQ
+    if (warp == 3) tc::tmem_dealloc(tmem_base, 128 * kW2DsSets);
+    return;
+  }
 
   if (warp < 3) {
     // ------------------------------------------------------------------ producers: first half of a key cube, second, dS tile

@@ -195,16 +195,17 @@ __global__ void __launch_bounds__(kW2Threads, 1)
 fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_constant__ CUtensorMap tm_x1,
                       const __grid_constant__ CUtensorMap tm_y0, const __grid_constant__ CUtensorMap tm_y1, Geo g,
                       Bwd128Args a) {
-  grid_enter_items(a.items);
   using C = Bwd128<D>;
   static_assert(PASS == 0 || !SPLIT, "the dK/dV pass has no room for the low-order parts of P and dS");
   static_assert(!F16 || !SPLIT, "the fp16 forms carry no pairs");
   static_assert(!STORE || (PASS == 1 && F16), "the dK/dV pass stores fp16 tiles");
   if constexpr (F16 && PASS == 0) {
     // one answer for the block: a CTA that starts late may find that another has just raised the flag
+    grid_enter(false);
     if (__syncthreads_or(threadIdx.x == 0 && *a.range_flag != 0)) return;
-  } else if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) {
-    return;     // (the flag is final before this launch starts)
+  } else if (a.when != 0) {
+    grid_enter(false);
+    if ((*a.range_flag != 0) != (a.when == 2)) return;     // (the flag is final before this launch starts)
   }
   constexpr uint32_t NDP = PASS == 0 ? 2 : 1;                  // dP buffers
   // dQ pass: S 0; dP buffers 128, 256 (dS overwrites the dP it came from); dQ 384.
@@ -275,6 +276,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  if (!(F16 && PASS == 0) && a.when == 0) grid_enter_items(a.items);
 
   if (warp < 8) {
     tc::reg_dec<56>();

@@ -119,16 +119,6 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                        const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot,
                        const __grid_constant__ CUtensorMap tm_qe, const __grid_constant__ CUtensorMap tm_doe, Geo g,
                        DkvArgs a) {
-  // The launch of the few long lists lets the launch of the others (disjoint outputs, nothing read from this one) take the SMs as its
-  // CTAs leave them, once what both read is there; that one waits for this one at its end, so that what follows waits for both.
-  if (SPLIT && a.overlap == 1) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  } else if (!SPLIT && F16 == 0 && a.overlap == 2) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  } else {
-    grid_enter_items(a.items);
-  }
   constexpr int RA = SPLIT ? 2 : kRingA;                   // slots of the Q ring
   // accumulators: without SPLIT two sets of dK^T, dV^T (64 columns each), used by item parity
   constexpr uint32_t TM_DK = 256, TM_DV = SPLIT ? 384 : 320, TM_SET = 128, SETS = SPLIT ? 1 : 2;
@@ -146,9 +136,17 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int rep = MHA ? 1 : g.rep;
   constexpr bool STORES_DS = F16 == 1 || F16 == 2 || (SPLIT && !MHA);
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
-  if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) {     // (the flag is final before this launch starts)
-    if (!SPLIT && F16 == 0 && a.overlap == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
-    return;
+  // The launch of the few long lists (overlap 1) lets the launch of the others (2; disjoint outputs, nothing read from the first) take
+  // the SMs as its CTAs leave them, once what both read is there; the second waits for the first at its end, so that what
+  // follows waits for both.
+  const bool second = !SPLIT && F16 == 0 && a.overlap == 2;
+  const bool fallback = a.when == 2;             // hardly ever does anything, and then it needs no set-up
+  if (fallback) {
+    if (!second) grid_enter(false);
+    if (*a.range_flag == 0) {                    // (final before this launch starts)
+      if (second) grid_enter(false);
+      return;
+    }
   }
 
   if (tid == 0) {
@@ -174,6 +172,16 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  if (SPLIT && a.overlap == 1) {
+    grid_enter(false);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  } else if (!second && !fallback) {
+    grid_enter_items(a.items);
+  }
+  if (a.when == 1 && __syncthreads_or(tid == 0 && *a.range_flag != 0)) {
+    if (warp == 2) tc::tmem_dealloc(tmem_base, 512);
+    return;
+  }
   // tensor-memory columns: S buffers 0, 64; dP buffers 128, 192; dK^T 256, dV^T 320 and 384, 448 (SPLIT: dK^T 256 + 320,
   // dV^T 384 + 448)
 
@@ -789,8 +797,10 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
     when = 2;
     slot_plain = 5;
   }
-  if ((e = launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, when, 0, all, false, 1)) != cudaSuccess) return e;
-  return launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, when, 0, all, false, 2);
+  // (no list is longer than the blocks of the problem)
+  const bool long_lists = g.N > kDkvLongColumn;
+  if (long_lists && (e = launch(true, &status->pad[4], kDkvLongColumn + 1, kAll, when, 0, all, false, 1)) != cudaSuccess) return e;
+  return launch(false, &status->pad[slot_plain], 0, kDkvLongColumn, when, 0, all, false, long_lists ? 2 : 0);
 }
 
 // Packed where two or four cubes fill a tile.  Below 128 cubes the counts are a launch for nothing.

@@ -45,13 +45,11 @@ template <int D>
 __global__ void __launch_bounds__(kDsThreads, 1)
 fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_kt, Geo g,
                       DqDsArgs a) {
-  grid_enter_items(a.items);
   using C = DqDs<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   DqDsMisc* misc = reinterpret_cast<DqDsMisc*>(smem + C::OFF_MISC);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) return;       // the fallback computes dQ
 
   if (tid == 0) {
     misc->abort_flag = 0;
@@ -75,6 +73,11 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  grid_enter_items(a.items);
+  if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) {       // the fallback computes dQ
+    if (warp == 3) tc::tmem_dealloc(tmem_base, 64 * kDsSets);
+    return;
+  }
 
   if (warp < 3) {
     // ------------------------------------------------------------------ producers: first K block of a pair, second, dS pair

@@ -176,7 +176,6 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                       const __grid_constant__ CUtensorMap tm_qt, const __grid_constant__ CUtensorMap tm_kt,
                       const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot, Geo g,
                       DqArgs a) {
-  grid_enter_items(g.batch * g.Hq * g.N);
   using C = BwdTc<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -190,9 +189,11 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   const float c2 = g.scale * 1.4426950408889634f;
   if constexpr (F16) {
     // one answer for the block: a CTA that starts late may find that another has just raised the flag
+    grid_enter(false);
     if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) return;
-  } else if (a.when != 0 && ((*a.range_flag != 0) != (a.when == 2))) {
-    return;     // (the flag is final before this launch starts)
+  } else if (a.when != 0) {
+    grid_enter(false);
+    if ((*a.range_flag != 0) != (a.when == 2)) return;     // (the flag is final before this launch starts)
   }
 
   if (tid == 0) {
@@ -212,6 +213,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  if (!F16 && a.when == 0) grid_enter_items(total_items);
   // tensor-memory columns: S^T buffers 0, 64; dP^T buffers 128, 192; dQ^T 256 (SPLIT: its low-order part at 320)
 
   if (warp < 2) {

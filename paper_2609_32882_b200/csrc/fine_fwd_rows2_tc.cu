@@ -100,7 +100,6 @@ template <int D>
 __global__ void __launch_bounds__(kF2Threads, 1)
 fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, Geo g, FwdRows2Args a) {
-  grid_enter_items(g.batch * g.Hq * g.N / 2);
   using C = FwdRows2<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -160,6 +159,7 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  grid_enter_items(g.batch * g.Hq * g.N / 2);
 
   if (warp < 8) {
     tc::reg_dec<56>();

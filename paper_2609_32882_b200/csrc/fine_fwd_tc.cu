@@ -92,7 +92,6 @@ template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fine_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, Geo g, FwdArgs a) {
-  grid_enter();
   using C = FwdTc<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -145,6 +144,7 @@ fine_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  grid_enter();
   // tensor-memory columns: S^T buffers 0, 64, 128, 192; O^T of the even tiles 256, of the odd tiles 320
 
   if (warp < 8) {

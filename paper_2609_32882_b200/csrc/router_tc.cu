@@ -236,11 +236,14 @@ template <int D, int G, bool FOLD, bool ONE>
 __global__ void __launch_bounds__(kRtThreads, 1)
 router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, Geo g,
                  float* __restrict__ pr, RouterOne one, StatusBlock* status) {
-  grid_enter_items(g.batch * g.Hq * ((g.N * G + kRtTile - 1) / kRtTile));
   static_assert(!FOLD || G == 8, "half-cubes of 8 sub-cubes");
   static_assert(!ONE || G == 8, "a thread parks the sums of four cubes");
   constexpr int PASSES = ONE ? 1 : 2;
-  if (!ONE && one.redo != nullptr && *one.redo == 0) return;       // (settled before this launch starts)
+  const bool redo = !ONE && one.redo != nullptr;
+  if (redo) {
+    grid_enter(false);
+    if (*one.redo == 0) return;                  // (settled before this launch starts)
+  }
   using C = RouterTc<D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -287,6 +290,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
+  if (!redo) grid_enter_items(total_items);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -619,7 +623,7 @@ struct RouterExactArgs {
 
 template <int D, bool FOLD>
 __global__ void __launch_bounds__(128) router_exact_kernel(Geo g, RouterExactArgs a) {
-  grid_enter();
+  grid_enter(false);
   using C = RouterTc<D>;
   constexpr int ROWS = FOLD ? 16 : 8, PAIRS = kRtTile / ROWS;      // sub-cubes of a pair's side, pairs of a tile
   extern __shared__ unsigned char smem_raw[];
