@@ -431,9 +431,10 @@ def run_ours(args):
     value = replicas.whole_job_throughput(flops["dense_equiv_fwd_bwd"], world, ms_step * 1e-3) / 1e12
     value_e2e = replicas.whole_job_throughput(flops["dense_equiv_fwd_bwd"], world, ms_step_e2e * 1e-3) / 1e12
     pk, pk_kind = peaks()
-    executed = flops["fine_fwd"] + flops["fine_bwd_algorithmic"] + 2.0 * flops["router_per_pass"]
+    router_passes = 1.0 if attn.route_scratch_bytes else 2.0       # (the one-pass form runs with scratch)
+    executed = flops["fine_fwd"] + flops["fine_bwd_algorithmic"] + router_passes * flops["router_per_pass"]
     kernel_flops = {"fine_fwd": flops["fine_fwd"], "fine_bwd": flops["fine_bwd_algorithmic"],
-                    "router_pool": 2.0 * flops["router_per_pass"]}
+                    "router_pool": router_passes * flops["router_per_pass"]}
     # dK/dV and dQ together: where dS is stored, dQ is formed inside the events of fine_bwd_dkv
     tensor_kernels = {k: kernel_ms["fine_bwd_dq"] + kernel_ms["fine_bwd_dkv"] if k == "fine_bwd" else kernel_ms[k] for k in kernel_flops}
     dominant = max(tensor_kernels, key=tensor_kernels.get)
