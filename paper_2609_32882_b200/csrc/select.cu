@@ -134,6 +134,7 @@ __device__ __forceinline__ unsigned band_hi(unsigned tau) { return tau < 0xfffff
 __device__ __forceinline__ bool band_usable(unsigned tau) { return tau >= kBandLeast && tau <= kBandMost; }
 constexpr int kBandHead = 2048;      // entries of a head's band that sel_settle_kernel ranks
 __device__ __forceinline__ void settle_list(const Settle& se, int row, int column) {
+  if (*reinterpret_cast<volatile int*>(se.redo) != 0) return;      // (a million ties would wait for one counter: the list is full, or not used)
   const int at = atomicAdd(se.count, 1);
   if (at < se.cap) se.pairs[at] = make_int2(row, column);
   else atomicExch(se.redo, 1);
