@@ -41,7 +41,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.501570e9 + 0.293740e9),
                                 # copies of Q and K + dK/dV with the stored dS + dQ from it
                                 "fine_bwd": 5 * ((0.309830e9 + 0.261202e9) + (2.446885e9 + 6.304944e9) + (6.611088e9 + 0.159028e9)),
-                                "router_pool": 5 * (0.047220e9 + 0.017765e9)}
+                                # one-pass router: the parked scores are written and read once (4-head capture)
+                                "router_pool": 10 * (0.229342e9 + 0.244402e9)}
 
 
 # What ncu shows as the busiest unit of each tensor kernel at 64-token cubes (8-head capture, profiles/): the roofline
@@ -50,7 +51,7 @@ NCU_LIMITER = {
     "fine_fwd": "L2 -> SM read rate: 12.9 TB/s against 11.8 TB/s sustained peak (tensor pipe 82 % active at the half rate of M = 64)",
     "fine_bwd": "dK/dV: shared-memory data pipe 99 % (tensor-core operand fetches 68 % + thread loads/stores 31 %; tensor pipe 46 %); "
                 "dQ from the stored dS: DRAM 68 % (tensor pipe 33 %)",
-    "router_pool": "exponential unit 80 % (two ex2 per score), instruction issue 64 %",
+    "router_pool": "instruction issue 69 %, exponential unit 63 % (one ex2 per score) of the cycles an SM is busy; 4-head capture",
 }
 # L2 -> SM read rate that ncu reports as the sustained peak of this part (derived__lts__lts2xbar_bytes.sum.peak_sustained
 # in the 8-head capture of profiles/kernels_720p_8heads_ncu_full.md, where the fine forward itself reads 12.0 TB/s).
