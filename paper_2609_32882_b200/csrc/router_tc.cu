@@ -513,6 +513,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
     if constexpr (ONE) {
       // the last item's, kRtAhead tiles side by side (one after the other: 390 cycles each)
+      __threadfence();      // (as in the loop: its last kRtAhead tiles have been parked since the fence there)
       for (int k0 = 0; k0 < row_tiles; k0 += kRtAhead) {
         rt_copy_wait<0>();
         Parked x[kRtAhead];

@@ -91,3 +91,27 @@ def test_one_pass_maps_are_the_two_pass_maps(case):
         tau = two.flatten(2).topk(n * topk, dim=-1).values[..., -1].view(torch.int32)[..., None, None]
         band = (two.view(torch.int32) - tau).abs() <= 128        # (well inside the 512 units of the one-pass threshold)
         assert band.sum() >= heads_q and torch.equal(one[band], two[band])
+
+
+@pytest.mark.parametrize("heads,dim,grid,cube", [
+    (1, 64, (16, 32, 32), {}),            # one item a CTA: every tile is fetched behind the loop
+    (2, 128, (20, 18, 68), WIDE),
+    (7, 128, (13, 30, 33), {}),           # two or three items a CTA
+])
+def test_parked_sums_come_back_whole(heads, dim, grid, cube):
+    """Every parked sum is read after it was written, those of a CTA's last item too: NaN wherever one is not, run after run."""
+    p = vb.make_params(1, heads, heads, dim, grid, topk=9, **cube)
+    q, k = _inputs(heads, heads, dim, grid, "random")
+    attn = vb.Vsa2Attention(p)
+    n = -(-grid[0] // 4) * -(-grid[1] // 4) * -(-grid[2] // (8 if cube else 4))
+    tiles = -(-8 * n * (2 if cube else 1) // 128)
+    scratch = torch.empty(148 * tiles * 8192 + heads * (4 * 128 * tiles + 4 * n) + (1 << 20) + 4096, dtype=torch.uint8, device="cuda")
+    first = None
+    for _ in range(12):
+        scratch.fill_(0xff)
+        vb.vsa2_route(p, q, k, None, attn.map, attn.ws_route, scratch=scratch)
+        attn.check_status()
+        scores = attn.scores().clone()
+        assert torch.isfinite(scores).all()
+        first = scores if first is None else first
+        assert torch.equal(scores, first)
