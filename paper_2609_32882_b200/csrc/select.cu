@@ -587,7 +587,8 @@ __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restric
                                                           const int* __restrict__ row_gt, int* row_eq, unsigned* bits_eq, Settle se) {
   grid_enter();
   __shared__ int ws[33];
-  __shared__ int at[kBandHead], n_rows;
+  __shared__ int n_rows;
+  __shared__ int2 at[kBandHead];            // {row, column}: their flat index need not fit an int (46,341 cubes and more)
   __shared__ unsigned val[kBandHead];
   __shared__ int2 rows[kBandHead];          // (no more than entries)
   const int bh = blockIdx.x, tid = threadIdx.x;
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restric
       int p = pos + incl - c;
       for (unsigned b = bits; b != 0u; b &= b - 1u, ++p) {
         const int j = (w0 + lane) * 32 + (__ffs(b) - 1);
-        at[p] = i * N + j;
+        at[p] = make_int2(i, j);
         val[p] = __float_as_uint(pr[(base + i) * N + j]);
       }
       pos += __shfl_sync(0xffffffffu, incl, 31);
@@ -638,7 +639,7 @@ __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restric
     int rank = 0;
     for (int f = 0; f < band; ++f) rank += val[f] > v || (val[f] == v && f < e);
     if (rank >= need) {
-      const int i = at[e] / N, j = at[e] - i * N;
+      const int i = at[e].x, j = at[e].y;
       atomicAnd(&bits_eq[(base + i) * words + (j >> 5)], ~(1u << (j & 31)));
       atomicSub(&row_eq[base + i], 1);
     }

@@ -54,6 +54,12 @@ def _inputs(heads_q, heads_kv, dim, grid, kind):
     return q.bfloat16(), k.bfloat16()
 
 
+def _state(attn):
+    """(flag that sends a call back to the two-pass form, pairs settled on two-pass scores) of the last route call."""
+    words = attn.ws_route[:256].view(torch.int32)
+    return int(words[2]), int(words[3])
+
+
 @pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[0]}x{c[1]}_d{c[2]}_{'x'.join(map(str, c[3]))}_mode{c[5]}_{c[8]}_{c[7]}")
 def test_one_pass_maps_are_the_two_pass_maps(case):
     heads_q, heads_kv, dim, grid, cube, mode, topk, flags, kind = case
@@ -115,3 +121,22 @@ def test_parked_sums_come_back_whole(heads, dim, grid, cube):
         assert torch.isfinite(scores).all()
         first = scores if first is None else first
         assert torch.equal(scores, first)
+
+
+def test_pairs_whose_flat_index_is_beyond_32_bits_are_settled():
+    """48,400 cubes: row * cubes + column passes 2^31 in the last rows, of which some entries lie in the band of the threshold."""
+    grid = (16, 440, 440)
+    p = vb.make_params(1, 1, 1, 64, grid, topk=4)
+    q, k = _inputs(1, 1, 64, grid, "random")
+    attn = vb.Vsa2Attention(p)
+    n, tiles = 48400, 3025
+    scratch = torch.empty(148 * tiles * 8192 + 4 * 128 * tiles + 4 * n + (1 << 20) + 4096, dtype=torch.uint8, device="cuda")
+    maps = []
+    for s in (None, scratch):
+        vb.vsa2_route(p, q, k, None, attn.map, attn.ws_route, scratch=s)
+        attn.check_status()
+        maps.append([x.clone() for x in attn.map_views()])
+    redo, pairs = _state(attn)
+    assert redo == 0 and pairs > 0
+    for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), *maps):
+        assert torch.equal(x, y), name
