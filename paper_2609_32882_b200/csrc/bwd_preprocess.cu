@@ -12,10 +12,10 @@ namespace vsa2 {
 // gate_l dO_l runs over the tokens in order, so the dO rows are left in shared memory for one thread per channel.  (With
 // one thread per chunk walking the block's tokens a small problem waited for sixteen rounds of loads, 21 us.)
 template <int D>
-__global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __restrict__ d_o, const void* __restrict__ o,
-                                                             const bf16* __restrict__ o_res,
-                                                             const float* __restrict__ gate,
-                                                             const float* __restrict__ oc_hat, Geo g,
+__global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o, const void* o,
+                                                             const bf16* o_res,
+                                                             const float* gate,
+                                                             const float* oc_hat, Geo g,
                                                              float* __restrict__ delta, float* __restrict__ dgate,
                                                              float* __restrict__ d_oc_hat, float2* __restrict__ absmax,
                                                              StatusBlock* clear) {
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
   for (int e = 0; e < 8; ++e) ocv[e] = 0.f;
   if (coarse) {
     const float4* p4 = reinterpret_cast<const float4*>(oc_hat + (bhq * g.Nvid + i) * D + ch * 8);
-    const float4 x = __ldg(p4), y = __ldg(p4 + 1);
+    const float4 x = *p4, y = p4[1];
     ocv[0] = x.x; ocv[1] = x.y; ocv[2] = x.z; ocv[3] = x.w;
     ocv[4] = y.x; ocv[5] = y.y; ocv[6] = y.z; ocv[7] = y.w;
   }
@@ -58,15 +58,15 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* __re
       of[u][0] = of[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (l[u] >= 0) {
         const size_t base = (bhq * g.S + l[u]) * D + ch * 8;
-        dv[u] = __ldg(reinterpret_cast<const uint4*>(d_o + base));
+        dv[u] = *reinterpret_cast<const uint4*>(d_o + base);
         if (g.out_f32) {
-          of[u][0] = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(o) + base));
-          of[u][1] = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(o) + base + 4));
+          of[u][0] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(o) + base);
+          of[u][1] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(o) + base + 4);
         } else {
-          ob[u] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(o) + base));
-          if (o_res != nullptr) rb[u] = __ldg(reinterpret_cast<const uint4*>(o_res + base));
+          ob[u] = *reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(o) + base);
+          if (o_res != nullptr) rb[u] = *reinterpret_cast<const uint4*>(o_res + base);
         }
-        if (coarse) gt[u] = __ldg(gate + bhq * g.L + l[u]);
+        if (coarse) gt[u] = gate[bhq * g.L + l[u]];
       }
     }
 #pragma unroll

@@ -60,7 +60,7 @@ __device__ __forceinline__ void issue_tile(float* ks, float* vs, const float* kc
 // grid (ceil(N / 64), Hq, batch), 128 threads
 template <int D>
 __global__ void __launch_bounds__(kCfThreads, 2)
-coarse_fwd_mma_kernel(const float* __restrict__ qc, const float* __restrict__ kc, const float* __restrict__ vc, Geo g,
+coarse_fwd_mma_kernel(const float* qc, const float* kc, const float* vc, Geo g,
                       float* __restrict__ oc_hat, float* __restrict__ lse_c) {
   grid_enter();
   using S = CoarseFwdSmem<D>;
@@ -88,10 +88,10 @@ coarse_fwd_mma_kernel(const float* __restrict__ qc, const float* __restrict__ kc
     const float* q_hi = qc + qoff + (size_t)min(row_hi, N - 1) * D;
 #pragma unroll
     for (int ks = 0; ks < D / 8; ++ks) {
-      qf[ks][0] = to_tf32(__ldg(q_lo + ks * 8 + tq));
-      qf[ks][1] = to_tf32(__ldg(q_hi + ks * 8 + tq));
-      qf[ks][2] = to_tf32(__ldg(q_lo + ks * 8 + tq + 4));
-      qf[ks][3] = to_tf32(__ldg(q_hi + ks * 8 + tq + 4));
+      qf[ks][0] = to_tf32(q_lo[ks * 8 + tq]);
+      qf[ks][1] = to_tf32(q_hi[ks * 8 + tq]);
+      qf[ks][2] = to_tf32(q_lo[ks * 8 + tq + 4]);
+      qf[ks][3] = to_tf32(q_hi[ks * 8 + tq + 4]);
     }
   }
   float o[D / 8][4];

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) pooled_inputs_kernel(PooledInputs p) {
 #pragma unroll
   for (int t = 0; t < 4; ++t)
     for (size_t i = first; i < p.n4[t]; i += stride) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(p.x[t]) + i);
+      const float4 v = reinterpret_cast<const float4*>(p.x[t])[i];
       __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
       uint2 o;
       o.x = *reinterpret_cast<uint32_t*>(&a);
@@ -94,21 +94,21 @@ static cudaError_t launch_pooled_inputs(const PooledInputs& p, cudaStream_t st) 
 
 // the recursive dK/dV pass returns one gradient per KV head; the epilogues of the main passes sum dK_c, dV_c over the
 // query heads of a group, so the result goes to the group's first query head and zeros to the others
-__global__ void spread_to_group_kernel(const float* __restrict__ x_kv, float* __restrict__ x_q, int rep, size_t per_head4,
+__global__ void spread_to_group_kernel(const float* x_kv, float* __restrict__ x_q, int rep, size_t per_head4,
                                        int heads_q) {
   grid_enter();
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const int hq = blockIdx.y;            // b * Hq + hq (Hq = Hkv * rep, so b * Hq + hq = (b * Hkv + hk) * rep + hh)
   if (i >= per_head4 || hq >= heads_q) return;
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (hq % rep == 0) v = __ldg(reinterpret_cast<const float4*>(x_kv) + (size_t)(hq / rep) * per_head4 + i);
+  if (hq % rep == 0) v = reinterpret_cast<const float4*>(x_kv)[(size_t)(hq / rep) * per_head4 + i];
   reinterpret_cast<float4*>(x_q)[(size_t)hq * per_head4 + i] = v;
 }
 
 // The pooled passes count their work items in a status block of their own (inside the scratch region); a non-zero
 // status word there (a bounded wait that ran out, a rescue list that overflowed) is copied into the caller's status word,
 // which is the one vsa2_device_status reads.
-__global__ void merge_status_kernel(const StatusBlock* __restrict__ from, StatusBlock* __restrict__ into) {
+__global__ void merge_status_kernel(const StatusBlock* from, StatusBlock* into) {
   grid_enter();
   const int s = from->status;
   if (s != 0) atomicCAS(&into->status, 0, s);

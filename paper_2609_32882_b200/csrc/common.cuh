@@ -59,6 +59,9 @@ struct StatusBlock {
 // Every kernel enters that way before it reads or writes global memory, also one that has nothing to do: its completion then stands
 // for all before it.  A kernel with tensor memory lets its successor in only when it has allocated it (or exits): a successor
 // that allocated first would keep it from ending.  The large ones also wait behind their set-up (barriers, tensor memory, tables).
+// What a kernel reads may be written while it is already there, waiting: so none of it is read-only for the kernel's lifetime, and no kernel
+// reads through __ldg or `const __restrict__` pointers (loads on the read-only path may be moved in front of the wait, and owe
+// nothing to it).  `__restrict__` stands only on pointers that a kernel writes and never reads.
 // 2048-token clip, 12 heads, training: 216 us without, 189 with the wait at the top of every kernel, 183 so; ragged clip 733, 709, 702.
 template <typename T> struct NotDeduced { using type = T; };
 template <typename... P>

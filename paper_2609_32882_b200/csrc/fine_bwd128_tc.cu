@@ -590,14 +590,14 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
           const size_t cap = (size_t)g.nnz_cap / 4;            // (the expanded lists hold every cube entry four times)
           place_next = a.pos + (size_t)il.bhq0 * cap + beg / 4;
           ds_head = a.ds + (size_t)(il.bhq0 - a.head0) * cap * (128 * 128 * 2) + (8 * half) * 2048 + row * 16;
-          place = __ldg(place_next);
+          place = *place_next;
         }
         VSA2_W2_TILES_BEGIN
           const uint32_t dpb = (tg % NDP) * 128;
           unsigned char* ds_tile = nullptr;
           if constexpr (STORE) {
             ds_tile = ds_head + (size_t)place * (128 * 128 * 2);
-            if (t + 1 < nt_l) place = __ldg(place_next + t + 1);
+            if (t + 1 < nt_l) place = place_next[t + 1];
           }
           uint32_t pf[64];                 // S, then P (as float bits) of this thread's 64 columns
           VSA2_WAIT(&misc->s_full, tg & 1);

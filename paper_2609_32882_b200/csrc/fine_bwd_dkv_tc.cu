@@ -812,8 +812,8 @@ PackedCubes packed_cubes(const Geo& g, const int* full) {
 
 // One warp per list: the entries in front of the cubes of the last layer -- or, of a list that does not have them at its end, all
 // but the text blocks (nothing of it is packed then)
-__global__ void __launch_bounds__(256) full_counts_kernel(int N, int Nvid, int first, long long cap, const int* __restrict__ ptr,
-                                                          const int* __restrict__ idx, int* __restrict__ full) {
+__global__ void __launch_bounds__(256) full_counts_kernel(int N, int Nvid, int first, long long cap, const int* ptr,
+                                                          const int* idx, int* __restrict__ full) {
   grid_enter();
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (j >= N) return;

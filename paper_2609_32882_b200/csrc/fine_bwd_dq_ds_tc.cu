@@ -236,9 +236,9 @@ done:
 
 // place of every entry of the column lists in the row lists of its head: pos[bh][e] for entry e of row_idx (both kinds of lists
 // ascend).  One warp per column; `counters`: n words to clear for the launches behind this one
-__global__ void __launch_bounds__(256) ds_positions_kernel(int N, long long cap, const int* __restrict__ row_ptr,
-                                                           const int* __restrict__ col_idx, const int* __restrict__ col_ptr,
-                                                           const int* __restrict__ row_idx, int* __restrict__ pos,
+__global__ void __launch_bounds__(256) ds_positions_kernel(int N, long long cap, const int* row_ptr,
+                                                           const int* col_idx, const int* col_ptr,
+                                                           const int* row_idx, int* __restrict__ pos,
                                                            int* __restrict__ counters, int n_counters) {
   grid_enter();
   if (blockIdx.x == 0 && blockIdx.y == 0)
@@ -272,7 +272,7 @@ cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col
 // one group's tensors at a time, which L2 holds).  A KV block's list can be ten times the mean, and a launch that draws such
 // items last ends with most SMs idle (720p, budget of 16..256 cubes, four heads a group: 0.7 ms for the mean item of a
 // 6 ms launch).  Counting sort by one block per group; the order of equal lengths depends on the run, the results do not.
-__global__ void __launch_bounds__(1024) dkv_order_kernel(Geo g, const int* __restrict__ col_ptr, int* __restrict__ order) {
+__global__ void __launch_bounds__(1024) dkv_order_kernel(Geo g, const int* col_ptr, int* __restrict__ order) {
   grid_enter();
   __shared__ int hist[1024], warp_sums[32], longest;
   const int bhk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -56,7 +56,7 @@ __device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int pe
     const uint2* m = reinterpret_cast<const uint2*>(s.absmax) + (size_t)grp * per_group;      // (bit patterns order like the numbers)
     unsigned d = 0u, o = 0u;
     for (int i = threadIdx.x; i < per_group; i += 256) {
-      const uint2 v = __ldg(m + i);
+      const uint2 v = m[i];
       d = max(d, v.x);
       o = max(o, v.y);
     }
@@ -88,9 +88,9 @@ __device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int pe
 // SCALED: there is a b_exp.  (Without it the magnitudes are compared as the integers they are; a thread walks its groups by adding
 // quotient and remainder of its stride: a division per step and products of 1 made the copies of 480p 30 us longer.)
 template <bool SCALED>
-__global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __restrict__ xa, uint4* __restrict__ ya, size_t na,
-                                                               const uint4* __restrict__ xb, uint4* __restrict__ yb, size_t nb,
-                                                               const int* __restrict__ b_exp, unsigned b_group, int* range_flag,
+__global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* xa, uint4* __restrict__ ya, size_t na,
+                                                               const uint4* xb, uint4* __restrict__ yb, size_t nb,
+                                                               const int* b_exp, unsigned b_group, int* range_flag,
                                                                DsScale scale, int groups, int per_group, int reducers) {
   grid_enter();
   const size_t stride = (size_t)(gridDim.x - reducers) * blockDim.x, n = na + nb;
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const size_t i = i0 + u * stride;
-      v[u] = i < n ? (i < na ? __ldg(xa + i) : __ldg(xb + (i - na))) : make_uint4(0, 0, 0, 0);
+      v[u] = i < n ? (i < na ? xa[i] : xb[i - na]) : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* __re
           }
         }
         // (a scaled value stays finite: the exponent takes the largest of a group to 2^-2 / max |O| at most)
-        f = pow2i(__ldg(b_exp + grp));
+        f = pow2i(b_exp[grp]);
       }
       uint32_t r[4];
 #pragma unroll

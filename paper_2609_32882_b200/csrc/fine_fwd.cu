@@ -19,10 +19,10 @@ struct FineFwdSmem {
 // One query block (i, hq, b) by a CTA of 256 threads: exact online softmax (running row maximum).
 template <int D>
 __device__ __forceinline__ void fine_fwd_block(unsigned char* smem_raw, int i, int hq, int b,
-                                               const bf16* __restrict__ q, const bf16* __restrict__ k,
-                                               const bf16* __restrict__ v, const float* __restrict__ gate,
-                                               const int* __restrict__ row_ptr, const int* __restrict__ col_idx,
-                                               const float* __restrict__ oc_hat, const Geo& g, void* __restrict__ o,
+                                               const bf16* q, const bf16* k,
+                                               const bf16* v, const float* gate,
+                                               const int* row_ptr, const int* col_idx,
+                                               const float* oc_hat, const Geo& g, void* __restrict__ o,
                                                bf16* __restrict__ o_res, float* __restrict__ lse) {
   using SM = FineFwdSmem<D>;
   bf16* Qs = reinterpret_cast<bf16*>(smem_raw);
@@ -121,10 +121,10 @@ __device__ __forceinline__ void fine_fwd_block(unsigned char* smem_raw, int i, i
 
 // grid (N, Hq, batch), 256 threads
 template <int D>
-__global__ void __launch_bounds__(256) fine_fwd_kernel(const bf16* __restrict__ q, const bf16* __restrict__ k,
-                                                       const bf16* __restrict__ v, const float* __restrict__ gate,
-                                                       const int* __restrict__ row_ptr, const int* __restrict__ col_idx,
-                                                       const float* __restrict__ oc_hat, Geo g, void* __restrict__ o,
+__global__ void __launch_bounds__(256) fine_fwd_kernel(const bf16* q, const bf16* k,
+                                                       const bf16* v, const float* gate,
+                                                       const int* row_ptr, const int* col_idx,
+                                                       const float* oc_hat, Geo g, void* __restrict__ o,
                                                        bf16* __restrict__ o_res, float* __restrict__ lse) {
   grid_enter();
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -135,11 +135,11 @@ __global__ void __launch_bounds__(256) fine_fwd_kernel(const bf16* __restrict__ 
 // list (its producers keep counting after the list is full and report that through the status word): only the `cap`
 // entries that were written are read.
 template <int D>
-__global__ void __launch_bounds__(256) fine_fwd_list_kernel(const int* __restrict__ count, int cap, const int* __restrict__ items,
-                                                            const bf16* __restrict__ q, const bf16* __restrict__ k,
-                                                            const bf16* __restrict__ v, const float* __restrict__ gate,
-                                                            const int* __restrict__ row_ptr, const int* __restrict__ col_idx,
-                                                            const float* __restrict__ oc_hat, Geo g, void* __restrict__ o,
+__global__ void __launch_bounds__(256) fine_fwd_list_kernel(const int* count, int cap, const int* items,
+                                                            const bf16* q, const bf16* k,
+                                                            const bf16* v, const float* gate,
+                                                            const int* row_ptr, const int* col_idx,
+                                                            const float* oc_hat, Geo g, void* __restrict__ o,
                                                             bf16* __restrict__ o_res, float* __restrict__ lse) {
   grid_enter();
   extern __shared__ __align__(128) unsigned char smem_raw[];

@@ -66,7 +66,7 @@ __device__ __forceinline__ void scatter_w(bf16* ws, uint4 v, int i, int Hq, RowO
 //   dz_hm [batch][HP][Lp]  head-major  (HP = heads rounded up to 16, Lp = tokens rounded up to 64; zero padding)
 //   dz_tm [batch][Lp][HP]  token-major
 // grid (Lp / 64, batch)
-__global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* __restrict__ gate, const float* __restrict__ dgate,
+__global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* gate, const float* dgate,
                                                              int L, int Lp, int Hq, int HP, bf16* __restrict__ dz_hm,
                                                              bf16* __restrict__ dz_tm) {
   grid_enter();
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* __rest
 // 5,120 channels, 40 heads 345 us against 296; 10 heads 168 both ways.)  The loads of the next chunk are in flight while a chunk is multiplied; warps beyond MW HW only
 // stage W.
 template <int NT, int MW, int HW, int CH>
-__global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, int L,
+__global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* x, const bf16* w, int L,
                                                               int C, int Hq, float* __restrict__ gate) {
   grid_enter();
   static_assert(NT % HW == 0 && MW * HW * 32 <= kGtThreads, "warps of a CTA");
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __rest
 #pragma unroll
       for (int u = 0; u < WV; ++u) {
         const int e = tid + u * kGtThreads;
-        rw[u] = e * 8 < CH * Hq && c0 * Hq + e * 8 < C * Hq ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq) + e)
+        rw[u] = e * 8 < CH * Hq && c0 * Hq + e * 8 < C * Hq ? reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq)[e]
                                                             : make_uint4(0, 0, 0, 0);
       }
     }
@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __rest
 #pragma unroll
       for (int q = 0; q < GROUPS; ++q) {
         const bool in = c0 + q * 32 + t * 8 < C;
-        ra[q] = in ? __ldg(reinterpret_cast<const uint4*>(xa + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
-        rc[q] = in ? __ldg(reinterpret_cast<const uint4*>(xc + c0 + q * 32)) : make_uint4(0, 0, 0, 0);
+        ra[q] = in ? *reinterpret_cast<const uint4*>(xa + c0 + q * 32) : make_uint4(0, 0, 0, 0);
+        rc[q] = in ? *reinterpret_cast<const uint4*>(xc + c0 + q * 32) : make_uint4(0, 0, 0, 0);
       }
     }
   };
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* __rest
 // channels are interleaved (column n of tile u is channel 8 (n / 2) + 2 u + n % 2), so that a thread's accumulators of the four
 // are 8 neighbouring channels of a token and go to memory as one 16-byte store; no tile is staged for coalescing.
 template <int KT>
-__global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __restrict__ w, const bf16* __restrict__ dz_tm,
+__global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* w, const bf16* dz_tm,
                                                                  int L, int Lp, int C, int Hq, int per_slice, int out_f32,
                                                                  void* __restrict__ dx) {
   grid_enter();
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __r
     const uint4* src = reinterpret_cast<const uint4*>(dz_tm + ((size_t)b * Lp + l0) * (KT * 16));
     for (int e = threadIdx.x; e < kGtTok * KT * 2; e += kGtThreads) {
       const int tl = e / (KT * 2), ch = e % (KT * 2);
-      *reinterpret_cast<uint4*>(az + tl * LDZ + ch * 8) = __ldg(src + e);
+      *reinterpret_cast<uint4*>(az + tl * LDZ + ch * 8) = src[e];
     }
   }
   for (int e = threadIdx.x; e < kDxCh * LDZ / 8; e += kGtThreads) reinterpret_cast<uint4*>(ws)[e] = make_uint4(0, 0, 0, 0);   // (padding heads)
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __r
     if ((reinterpret_cast<uintptr_t>(w) & 15u) == 0) {
       const uint4* src = reinterpret_cast<const uint4*>(w + (size_t)c0 * Hq);
       for (int e = threadIdx.x; e * 8 < kDxCh * Hq; e += kGtThreads)
-        scatter_w<LDZ>(ws, c0 * Hq + e * 8 < C * Hq ? __ldg(src + e) : make_uint4(0, 0, 0, 0), e * 8, Hq, w_row);
+        scatter_w<LDZ>(ws, c0 * Hq + e * 8 < C * Hq ? src[e] : make_uint4(0, 0, 0, 0), e * 8, Hq, w_row);
     } else {
       for (int e = threadIdx.x; e < kDxCh * KT * 16; e += kGtThreads) {
         const int c = e / (KT * 16), h = e % (KT * 16);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dx_kernel(const bf16* __r
 // ---------------------------------------------------------------------------------------------- dW_g
 // grid (ceil(C / 128), splits, batch): partial[(b * splits + s)][c][h] = sum over the split's tokens of X[l, c] dz[l, h]
 template <int NT>
-__global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dz_hm,
+__global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* x, const bf16* dz_hm,
                                                                  int L, int Lp, int C, int Hq, int HP,
                                                                  float* __restrict__ partial) {
   grid_enter();
@@ -328,13 +328,13 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* __r
 #pragma unroll
     for (int u = 0; u < XV; ++u) {
       const int e = threadIdx.x + u * kGtThreads, r = e / (kGtCh / 8), ch = e % (kGtCh / 8);
-      rx[u] = (l0 + r < L && c0 + ch * 8 < C) ? __ldg(reinterpret_cast<const uint4*>(xb + (size_t)(l0 + r) * C + c0 + ch * 8))
+      rx[u] = (l0 + r < L && c0 + ch * 8 < C) ? *reinterpret_cast<const uint4*>(xb + (size_t)(l0 + r) * C + c0 + ch * 8)
                                               : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int u = 0; u < ZV; ++u) {
       const int e = threadIdx.x + u * kGtThreads, h = e / (kGtTok / 8), ch = e % (kGtTok / 8);
-      rz[u] = h < HP ? __ldg(reinterpret_cast<const uint4*>(zb + (size_t)h * Lp + l0 + ch * 8)) : make_uint4(0, 0, 0, 0);
+      rz[u] = h < HP ? *reinterpret_cast<const uint4*>(zb + (size_t)h * Lp + l0 + ch * 8) : make_uint4(0, 0, 0, 0);
     }
   };
   if (l_beg < l_end) load(l_beg);
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kGtThreads) gate_bwd_dw_kernel(const bf16* __r
     }
 }
 
-__global__ void gate_reduce_dw_kernel(const float* __restrict__ partial, int parts, size_t n, float* __restrict__ dw) {
+__global__ void gate_reduce_dw_kernel(const float* partial, int parts, size_t n, float* __restrict__ dw) {
   grid_enter();
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= n) return;

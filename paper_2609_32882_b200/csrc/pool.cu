@@ -34,7 +34,7 @@ __device__ __forceinline__ void add8(float (&acc)[8], const float (&v)[8], bool 
 }
 __device__ __forceinline__ void load8(const bf16* base, int t, int h, int w, const Geo& g, int D, float (&f)[8]) {
   uint4 v = make_uint4(0, 0, 0, 0);
-  if (t < g.T && h < g.H && w < g.W) v = __ldg(reinterpret_cast<const uint4*>(base + (size_t)((t * g.H + h) * g.W + w) * D));
+  if (t < g.T && h < g.H && w < g.W) v = *reinterpret_cast<const uint4*>(base + (size_t)((t * g.H + h) * g.W + w) * D);
   const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&v);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kSubThreads) pool_subcube_kernel(PoolJobs jobs
 // The attention kernels never need this copy (they address cubes through tensor maps over the raster layout); it is for
 // callers whose surrounding code works in the cube-major layout.
 template <int D>
-__global__ void __launch_bounds__(256) permute_kernel(const bf16* __restrict__ src, int heads, Geo g, int inverse,
+__global__ void __launch_bounds__(256) permute_kernel(const bf16* src, int heads, Geo g, int inverse,
                                                       bf16* __restrict__ dst) {
   grid_enter();
   const int n = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
@@ -199,10 +199,10 @@ __global__ void __launch_bounds__(256) permute_kernel(const bf16* __restrict__ s
     const size_t cubed = ((bh * g.N + n) * B + p) * (size_t)D + ch * 8;
     if (!inverse) {
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (l >= 0) v = __ldg(reinterpret_cast<const uint4*>(src + raster));
+      if (l >= 0) v = *reinterpret_cast<const uint4*>(src + raster);
       *reinterpret_cast<uint4*>(dst + cubed) = v;
     } else if (l >= 0) {
-      *reinterpret_cast<uint4*>(dst + raster) = __ldg(reinterpret_cast<const uint4*>(src + cubed));
+      *reinterpret_cast<uint4*>(dst + raster) = *reinterpret_cast<const uint4*>(src + cubed);
     }
   }
 }

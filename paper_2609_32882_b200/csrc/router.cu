@@ -19,8 +19,8 @@ struct RouterSmem {
 // grid (ceil(N*G/128), Hq, batch), 256 threads.
 // PASS 1: lse_r[b,hq,row] = log sum_{valid keys} exp(s*scale).   PASS 2: writes P_r.
 template <int D, int PASS>
-__global__ void __launch_bounds__(256) router_kernel(const bf16* __restrict__ qr, const bf16* __restrict__ kr, Geo g,
-                                                     float* __restrict__ lse_r, float* __restrict__ pr) {
+__global__ void __launch_bounds__(256) router_kernel(const bf16* qr, const bf16* kr, Geo g,
+                                                     float* lse_r, float* pr) {
   grid_enter();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using SM = RouterSmem<D>;
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256) router_kernel(const bf16* __restrict__ qr
   for (int c = threadIdx.x; c < kRT * CH; c += blockDim.x) {
     int r = c / CH, ch = c % CH;
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (row0 + r < rows_total) v = __ldg(reinterpret_cast<const uint4*>(qbase + (size_t)(row0 + r) * D + ch * 8));
+    if (row0 + r < rows_total) v = *reinterpret_cast<const uint4*>(qbase + (size_t)(row0 + r) * D + ch * 8);
     *reinterpret_cast<uint4*>(Qs + r * SM::LDQ + ch * 8) = v;
   }
   if (threadIdx.x < kRT) {
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256) router_kernel(const bf16* __restrict__ qr
     for (int c = threadIdx.x; c < kRT * CH; c += blockDim.x) {
       int r = c / CH, ch = c % CH;
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (k0 + r < rows_total) v = __ldg(reinterpret_cast<const uint4*>(kbase + (size_t)(k0 + r) * D + ch * 8));
+      if (k0 + r < rows_total) v = *reinterpret_cast<const uint4*>(kbase + (size_t)(k0 + r) * D + ch * 8);
       *reinterpret_cast<uint4*>(Ks + r * SM::LDQ + ch * 8) = v;
     }
     if (threadIdx.x < kRT) {

@@ -235,7 +235,7 @@ __device__ __forceinline__ float rt_pool(const uint32_t (&s)[32], uint32_t kbits
 template <int D, int G, bool FOLD, bool ONE>
 __global__ void __launch_bounds__(kRtThreads, 1)
 router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, Geo g,
-                 float* __restrict__ pr, RouterOne one, StatusBlock* status) {
+                 float* pr, RouterOne one, StatusBlock* status) {
   static_assert(!FOLD || G == 8, "half-cubes of 8 sub-cubes");
   static_assert(!ONE || G == 8, "a thread parks the sums of four cubes");
   constexpr int PASSES = ONE ? 1 : 2;

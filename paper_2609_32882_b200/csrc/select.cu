@@ -28,8 +28,8 @@ __global__ void sel_init_kernel(unsigned* state, unsigned* hist, int BH, unsigne
   }
 }
 
-__global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__ pr, long long n_elems,
-                                                       const unsigned* __restrict__ state, unsigned* hist, int pass,
+__global__ void __launch_bounds__(256) sel_hist_kernel(const float* pr, long long n_elems,
+                                                       const unsigned* state, unsigned* hist, int pass,
                                                        const int* redo) {
   grid_enter();
   __shared__ unsigned sh[kHistBins];
@@ -48,9 +48,9 @@ __global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__
     const uint4* src4 = reinterpret_cast<const uint4*>(src);
     const long long n4 = n_elems >> 2;
     for (long long i = tid; i < n4; i += 2 * nthr) {
-      const uint4 a = __ldg(src4 + i);
+      const uint4 a = src4[i];
       const bool two = i + nthr < n4;
-      const uint4 b = two ? __ldg(src4 + i + nthr) : make_uint4(0, 0, 0, 0);
+      const uint4 b = two ? src4[i + nthr] : make_uint4(0, 0, 0, 0);
       const unsigned va[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
       for (int e = 0; e < 8; ++e)
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256) sel_hist_kernel(const float* __restrict__
     done = n_elems;
   }
   for (long long i = done + tid; i < n_elems; i += nthr) {
-    unsigned v = __ldg(src + i);
+    unsigned v = src[i];
     if ((v & pmask) == prefix) atomicAdd(&sh[(v >> shift) & dmask], 1u);
   }
   __syncthreads();
@@ -144,8 +144,8 @@ __device__ __forceinline__ void settle_list(const Settle& se, int row, int colum
 // entries above tau (`bits_gt`) and equal to tau (`bits_eq`) and the two counts.  grid (ceil(N/8), BH), 256 threads
 // BAND: entries above and in the band instead, the latter also listed for router_exact_kernel.
 template <bool BAND>
-__global__ void __launch_bounds__(256) sel_row_bits_kernel(const float* __restrict__ pr, int N, int words,
-                                                           const unsigned* __restrict__ state, unsigned* bits_gt,
+__global__ void __launch_bounds__(256) sel_row_bits_kernel(const float* pr, int N, int words,
+                                                           const unsigned* state, unsigned* bits_gt,
                                                            unsigned* bits_eq, int* row_gt, int* row_eq, Settle se) {
   grid_enter();
   if (!BAND && se.redo != nullptr && *se.redo == 0) return;
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(256) sel_row_bits_kernel(const float* __restri
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = (w0 + u) * 32 + lane;
-      v[u] = j < N ? __ldg(src + j) : 0u;      // (scores are non-negative: 0 is never above tau, and equal only if tau = 0
+      v[u] = j < N ? src[j] : 0u;      // (scores are non-negative: 0 is never above tau, and equal only if tau = 0
     }                                          //  -- excluded by the j < N test below)
     unsigned mine_g = 0u, mine_e = 0u;
 #pragma unroll
@@ -203,9 +203,9 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 // word its position in the row's list, and each lane writes its own few entries (a warp per word spent 30 instructions on
 // every word, 45 words a row).  Ties at tau go to the lower column: a lane keeps the equal entries whose rank in the row is
 // below the row's quota.  grid (ceil(N/8), BH), 256 threads
-__global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int words, const unsigned* __restrict__ bits_eq,
-                                                                 const int* __restrict__ row_eq_take,
-                                                                 const int* __restrict__ row_ptr, int* col_idx,
+__global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int words, const unsigned* bits_eq,
+                                                                 const int* row_eq_take,
+                                                                 const int* row_ptr, int* col_idx,
                                                                  unsigned* bitmap, long long nnz_cap) {
   grid_enter();
   const int lane = threadIdx.x & 31;
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
   for (int w0 = 0; w0 < words; w0 += 32) {
     const int w = w0 + lane;
     const unsigned gb = w < words ? bitmap[base + w] : 0u;
-    unsigned eb = w < words ? __ldg(bits_eq + base + w) : 0u;
+    unsigned eb = w < words ? bits_eq[base + w] : 0u;
     const int ce = __popc(eb);
     const int ce_incl = warp_incl_scan(ce, lane);
     int rank = eq_seen + ce_incl - ce;             // equal entries of the row before this word
@@ -259,8 +259,8 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
 // MODE kListed: the listed rows alone, now with their two-pass scores (any grid).
 constexpr int kAllRows = 0, kBand = 1, kListed = 2;
 template <int U, int MODE>
-__global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __restrict__ pr, int N, int K,
-                                                                const int* __restrict__ budgets, float* row_tau,
+__global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* pr, int N, int K,
+                                                                const int* budgets, float* row_tau,
                                                                 int* row_eq_take, int* row_cnt, Settle se) {
   grid_enter();
   if (MODE == kAllRows && se.redo != nullptr && *se.redo == 0) return;
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __r
   const unsigned* src = reinterpret_cast<const unsigned*>(pr) + o * N;
   unsigned v[U];
 #pragma unroll
-  for (int u = 0; u < U; ++u) v[u] = u * 32 + lane < N ? __ldg(src + u * 32 + lane) : 0u;      // (0 is never above a candidate)
+  for (int u = 0; u < U; ++u) v[u] = u * 32 + lane < N ? src[u * 32 + lane] : 0u;      // (0 is never above a candidate)
   int k = budgets ? budgets[o] : K;
   k = max(0, min(k, N));
   if (k == 0) {
@@ -323,8 +323,8 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* __r
 // per-row modes, rows of more than 2048 entries: radix select of the k_i-th largest of row i.  grid (N, BH), 256 threads
 // MODE as above
 template <int MODE>
-__global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restrict__ pr, int N, int K,
-                                                           const int* __restrict__ budgets, float* row_tau,
+__global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int N, int K,
+                                                           const int* budgets, float* row_tau,
                                                            int* row_eq_take, int* row_cnt, Settle se) {
   grid_enter();
   __shared__ unsigned sh[256];
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restri
     __syncthreads();
     const unsigned prefix = s_prefix, pmask = s_mask;
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
-      unsigned v = __ldg(src + j);
+      unsigned v = src[j];
       if ((v & pmask) == prefix) atomicAdd(&sh[(v >> shift) & 0xFFu], 1u);
     }
     __syncthreads();
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restri
   if constexpr (MODE == kBand) {
     const unsigned lo = band_lo(tau), hi = band_hi(tau);
     int from = 0;
-    for (int j = threadIdx.x; j < N; j += blockDim.x) from += __ldg(src + j) >= lo;
+    for (int j = threadIdx.x; j < N; j += blockDim.x) from += src[j] >= lo;
     if (threadIdx.x == 0) sh[0] = 0u;
     __syncthreads();
     if (from > 0) atomicAdd(&sh[0], (unsigned)from);
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* __restri
         else atomicExch(se.redo, 1);
       }
       for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        const unsigned v = __ldg(src + j);
+        const unsigned v = src[j];
         if (v >= lo && v <= hi) settle_list(se, (int)o, j);
       }
     }
@@ -422,8 +422,8 @@ __device__ __forceinline__ int block_excl_scan(int v, int* warp_sums, int& total
 }
 
 // one block per (batch, head): per-sequence tie quota per row, then row_ptr = exclusive scan of counts
-__global__ void __launch_bounds__(1024) sel_scan_rows_kernel(int N, int per_sequence, const unsigned* __restrict__ state,
-                                                             const int* __restrict__ row_gt, const int* __restrict__ row_eq,
+__global__ void __launch_bounds__(1024) sel_scan_rows_kernel(int N, int per_sequence, const unsigned* state,
+                                                             const int* row_gt, const int* row_eq,
                                                              float* row_tau, int* row_eq_take, int* row_cnt, int* row_ptr,
                                                              long long nnz_cap, StatusBlock* status) {
   grid_enter();
@@ -467,10 +467,10 @@ __global__ void __launch_bounds__(1024) sel_scan_rows_kernel(int N, int per_sequ
 }
 
 // one warp per row: ordered emission of the kept columns and of the row's bitmap words
-__global__ void __launch_bounds__(256) sel_emit_rows_kernel(const float* __restrict__ pr, int N, int words,
-                                                            const float* __restrict__ row_tau,
-                                                            const int* __restrict__ row_eq_take,
-                                                            const int* __restrict__ row_ptr, int* col_idx,
+__global__ void __launch_bounds__(256) sel_emit_rows_kernel(const float* pr, int N, int words,
+                                                            const float* row_tau,
+                                                            const int* row_eq_take,
+                                                            const int* row_ptr, int* col_idx,
                                                             unsigned* bitmap, long long nnz_cap) {
   grid_enter();
   const int lane = threadIdx.x & 31;
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(256) sel_emit_rows_kernel(const float* __restr
   const unsigned lt = (1u << lane) - 1u;
   for (int w = 0; w < words; ++w) {
     int j = w * 32 + lane;
-    unsigned v = j < N ? __ldg(src + j) : 0u;
+    unsigned v = j < N ? src[j] : 0u;
     bool gt = j < N && v > tau;
     bool eq = j < N && v == tau;
     unsigned eqb = __ballot_sync(0xffffffffu, eq);
@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(256) sel_emit_rows_kernel(const float* __restr
 
 // bitmap [BH][N rows][words] -> bitmap_t [BH][N columns][words] (bit i of row-word set <-> bit of column-word set):
 // one warp per 32 x 32 bit tile, transposed with 32 ballots.  grid (words, ceil(words/8), BH), 256 threads
-__global__ void __launch_bounds__(256) sel_transpose_bitmap_kernel(const unsigned* __restrict__ bitmap, int N, int words,
+__global__ void __launch_bounds__(256) sel_transpose_bitmap_kernel(const unsigned* bitmap, int N, int words,
                                                                    unsigned* __restrict__ bitmap_t) {
   grid_enter();
   const int lane = threadIdx.x & 31;
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(256) sel_transpose_bitmap_kernel(const unsigne
   const int bh = blockIdx.z;
   if (wi >= words) return;
   const int i = wi * 32 + lane;
-  const unsigned v = i < N ? __ldg(bitmap + ((size_t)bh * N + i) * words + wj) : 0u;
+  const unsigned v = i < N ? bitmap[((size_t)bh * N + i) * words + wj] : 0u;
   unsigned mine = 0u;
 #pragma unroll
   for (int bit = 0; bit < 32; ++bit) {
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(256) sel_transpose_bitmap_kernel(const unsigne
 }
 
 // one warp per column: number of kept rows.  grid (ceil(N/8), BH), 256 threads
-__global__ void __launch_bounds__(256) sel_col_count_kernel(const unsigned* __restrict__ bitmap_t, int N, int words,
+__global__ void __launch_bounds__(256) sel_col_count_kernel(const unsigned* bitmap_t, int N, int words,
                                                             int* col_cnt) {
   grid_enter();
   const int lane = threadIdx.x & 31;
@@ -533,12 +533,12 @@ __global__ void __launch_bounds__(256) sel_col_count_kernel(const unsigned* __re
   if (j >= N) return;
   const unsigned* bm = bitmap_t + ((size_t)bh * N + j) * words;
   int c = 0;
-  for (int w = lane; w < words; w += 32) c += __popc(__ldg(bm + w));
+  for (int w = lane; w < words; w += 32) c += __popc(bm[w]);
   for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (lane == 0) col_cnt[(size_t)bh * N + j] = c;
 }
 
-__global__ void __launch_bounds__(1024) sel_scan_cols_kernel(int N, const int* __restrict__ col_cnt, int* col_ptr,
+__global__ void __launch_bounds__(1024) sel_scan_cols_kernel(int N, const int* col_cnt, int* col_ptr,
                                                              long long nnz_cap) {
   grid_enter();
   __shared__ int ws[33];
@@ -556,8 +556,8 @@ __global__ void __launch_bounds__(1024) sel_scan_cols_kernel(int N, const int* _
 }
 
 // one warp per column, one lane per bitmap word: ordered emission of the rows that keep it.  grid (ceil(N/8), BH), 256 threads
-__global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __restrict__ bitmap_t, int N, int words,
-                                                            const int* __restrict__ col_ptr, int* row_idx,
+__global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* bitmap_t, int N, int words,
+                                                            const int* col_ptr, int* row_idx,
                                                             long long nnz_cap) {
   grid_enter();
   const int lane = threadIdx.x & 31;
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __re
   int* out = row_idx + (size_t)bh * nnz_cap;
   for (int w0 = 0; w0 < words; w0 += 32) {
     // one lane per word, as in sel_emit_rows_bits_kernel
-    unsigned word = w0 + lane < words ? __ldg(bm + w0 + lane) : 0u;
+    unsigned word = w0 + lane < words ? bm[w0 + lane] : 0u;
     const int c = __popc(word);
     const int c_incl = warp_incl_scan(c, lane);
     int p = pos + c_incl - c;
@@ -583,8 +583,8 @@ __global__ void __launch_bounds__(256) sel_emit_cols_kernel(const unsigned* __re
 
 // per-sequence, one-pass scores: of every head whose band holds more entries than are still wanted, ranks the band by its two-pass
 // scores (ties to the lower index) and takes what is not kept out of the bitmap and the counts.  One block per head.
-__global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restrict__ pr, int N, int words, unsigned keep, unsigned* state,
-                                                          const int* __restrict__ row_gt, int* row_eq, unsigned* bits_eq, Settle se) {
+__global__ void __launch_bounds__(1024) sel_settle_kernel(const float* pr, int N, int words, unsigned keep, unsigned* state,
+                                                          const int* row_gt, int* row_eq, unsigned* bits_eq, Settle se) {
   grid_enter();
   __shared__ int ws[33];
   __shared__ int n_rows;
@@ -649,11 +649,11 @@ __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* __restric
 // Up to kSelOneBlockN cubes: everything behind the counts of the kept entries in one launch, a block per head with both bitmaps in
 // shared memory (the six launches below take 2 us and a gap each and keep a few SMs busy).  Same rules: rows in order, ties at the
 // threshold to the lower column, both maps cut at the capacity.
-__global__ void __launch_bounds__(1024) sel_maps_kernel(const float* __restrict__ pr, int N, int words, int per_sequence,
-                                                        const unsigned* __restrict__ state, const int* __restrict__ row_gt,
-                                                        const int* __restrict__ row_eq, const float* __restrict__ row_tau,
-                                                        const int* __restrict__ row_eq_take, const int* __restrict__ row_cnt,
-                                                        const unsigned* __restrict__ bits_gt, const unsigned* __restrict__ bits_eq,
+__global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, int words, int per_sequence,
+                                                        const unsigned* state, const int* row_gt,
+                                                        const int* row_eq, const float* row_tau,
+                                                        const int* row_eq_take, const int* row_cnt,
+                                                        const unsigned* bits_gt, const unsigned* bits_eq,
                                                         int* row_ptr, int* col_idx, int* col_ptr, int* row_idx, long long nnz_cap,
                                                         StatusBlock* status) {
   grid_enter();
@@ -695,12 +695,12 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* __restrict_
     unsigned v[W], gw = 0u, ew = 0u;
     if (per_sequence) {
       if (lane < words) {
-        gw = __ldg(bits_gt + (base + i) * words + lane);
-        ew = __ldg(bits_eq + (base + i) * words + lane);
+        gw = bits_gt[(base + i) * words + lane];
+        ew = bits_eq[(base + i) * words + lane];
       }
     } else {
 #pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = w * 32 + lane < N ? __ldg(src + w * 32 + lane) : 0u;
+      for (int w = 0; w < W; ++w) v[w] = w * 32 + lane < N ? src[w * 32 + lane] : 0u;
     }
 #pragma unroll
     for (int w = 0; w < W; ++w) {

@@ -44,7 +44,7 @@ __device__ __forceinline__ int valid_subcubes(const Geo& n, int cube) {
 
 // pr [BH, 2N, 2N] half-cube scores -> out [BH, N, N].  Eq. 7 divides the sum over a cube pair's valid sub-cube
 // pairs by (valid query sub-cubes of the cube) * G; a half-cube score is the same with its own counts.
-__global__ void __launch_bounds__(256) fold_scores_kernel(Geo n, const float* __restrict__ pr, float* __restrict__ out) {
+__global__ void __launch_bounds__(256) fold_scores_kernel(Geo n, const float* pr, float* __restrict__ out) {
   grid_enter();
   const int N = n.N / 2;
   const int c = blockIdx.x;
@@ -54,13 +54,13 @@ __global__ void __launch_bounds__(256) fold_scores_kernel(Geo n, const float* __
   const float2* r0 = reinterpret_cast<const float2*>(pr + (bh * n.N + 2 * c) * (size_t)n.N);
   const float2* r1 = reinterpret_cast<const float2*>(pr + (bh * n.N + 2 * c + 1) * (size_t)n.N);
   for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    const float2 a = __ldg(r0 + j), b = __ldg(r1 + j);
+    const float2 a = r0[j], b = r1[j];
     out[(bh * N + c) * (size_t)N + j] = w0 * (a.x + a.y) + w1 * (b.x + b.y);
   }
 }
 
 // x64 [BH, 2N, D] half-cube means -> x [BH, N, D] cube means (count-weighted)
-__global__ void __launch_bounds__(256) fold_mean_kernel(Geo n, const float* __restrict__ x64, float* __restrict__ x,
+__global__ void __launch_bounds__(256) fold_mean_kernel(Geo n, const float* x64, float* __restrict__ x,
                                                         size_t total) {
   grid_enter();
   const int D = n.D;
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) fold_mean_kernel(Geo n, const float* __re
 }
 
 // x64 [BH, 2N, D] -> x [BH, N, D]: sum of the two halves
-__global__ void __launch_bounds__(256) fold_sum_kernel(int D, const float* __restrict__ x64, float* __restrict__ x,
+__global__ void __launch_bounds__(256) fold_sum_kernel(int D, const float* x64, float* __restrict__ x,
                                                        size_t total) {
   grid_enter();
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256) fold_sum_kernel(int D, const float* __res
 
 // x [BH, N, D] -> x64 [BH, 2N, D]: each half gets the cube's row; with `by_count` scaled by the half's share of the
 // cube's tokens (the consumer divides by the half's own count, which leaves row / cube count as Eq. 1 requires)
-__global__ void __launch_bounds__(256) expand_rows_kernel(Geo n, int by_count, const float* __restrict__ x,
+__global__ void __launch_bounds__(256) expand_rows_kernel(Geo n, int by_count, const float* x,
                                                           float* __restrict__ x64, size_t total64) {
   grid_enter();
   const int D = n.D;
@@ -106,8 +106,8 @@ __global__ void __launch_bounds__(256) expand_rows_kernel(Geo n, int by_count, c
 
 // Compressed rows (or columns) of the cube map -> those of the half-cube map: list (c; j0, j1, ...) becomes the two
 // lists (2c; 2j0, 2j0+1, 2j1, ...) and (2c+1; same).  ptr [BH, N+1], idx [BH, cap] -> ptr64 [BH, 2N+1], idx64 [BH, 4cap]
-__global__ void __launch_bounds__(128) expand_map_kernel(int N, int Hq, long long cap, const int* __restrict__ ptr,
-                                                         const int* __restrict__ idx, int* __restrict__ ptr64,
+__global__ void __launch_bounds__(128) expand_map_kernel(int N, int Hq, long long cap, const int* ptr,
+                                                         const int* idx, int* __restrict__ ptr64,
                                                          int* __restrict__ idx64) {
   grid_enter();
   const int c = blockIdx.x;
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(128) expand_map_kernel(int N, int Hq, long lon
 // ptr [BH, Nvid+1], idx [BH, cap] -> ptrx [BH, Nx+1], idxx [BH, capx] with Nx = Nvid + NtB, capx = cap + Nvid NtB + NtB Nx.
 // The same rule serves the CSR and the CSC map (the extension is symmetric).
 __global__ void __launch_bounds__(128) extend_map_kernel(int Nvid, int NtB, int Hq, long long cap, long long capx,
-                                                         const int* __restrict__ ptr, const int* __restrict__ idx,
+                                                         const int* ptr, const int* idx,
                                                          int* __restrict__ ptrx, int* __restrict__ idxx) {
   grid_enter();
   const int r = blockIdx.x, Nx = Nvid + NtB;
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(128) extend_map_kernel(int Nvid, int NtB, int 
 
 // "group head" routing: the query heads of a KV group share one map.  pr [batch, Hq, N, N]: every entry is replaced by
 // the sum over the heads of its group (added in head order), so the selection that follows picks the same set for each
-__global__ void __launch_bounds__(256) group_sum_scores_kernel(float* __restrict__ pr, int rep, size_t per_head, size_t groups,
+__global__ void __launch_bounds__(256) group_sum_scores_kernel(float* pr, int rep, size_t per_head, size_t groups,
                                                                const int* redo) {
   grid_enter();
   if (redo != nullptr && *redo == 0) return;

@@ -64,7 +64,7 @@ __device__ __forceinline__ void load_cube_tile(bf16* dst, int ld, const bf16* he
     int p = c / CH, ch = c % CH;
     int l = block_token(g, n, p);
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (l >= 0) v = __ldg(reinterpret_cast<const uint4*>(head_base + (size_t)l * D + ch * 8));
+    if (l >= 0) v = *reinterpret_cast<const uint4*>(head_base + (size_t)l * D + ch * 8);
     *reinterpret_cast<uint4*>(dst + (size_t)p * ld + ch * 8) = v;
   }
 }

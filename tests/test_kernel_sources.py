@@ -1,0 +1,33 @@
+"""Rules that the CUDA sources have to keep and that no output shows."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_32882_b200", "csrc")
+
+
+def _code(path):
+    with open(path) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_no_kernel_reads_as_constant_what_the_kernel_before_it_may_still_write():
+    """Kernels are placed while the one ahead of them runs and wait in grid_enter: loads on the read-only path (__ldg, ld.global.nc, and what
+    the compiler makes of `const __restrict__`) need not stay behind that wait.  (The self-tests are launched without overlap.)"""
+    files = [f for f in glob.glob(os.path.join(CSRC, "*.cu*")) if not f.endswith("selftest.cu")]
+    assert len(files) > 15
+    for path in files:
+        code = _code(path)
+        assert "__ldg" not in code and "ld.global.nc" not in code, path
+        assert not re.search(r"const\s+[\w:]+\s*\*\s*__restrict__", code), path
+
+
+def test_every_kernel_is_launched_to_overlap_and_waits_for_the_one_before_it():
+    for path in glob.glob(os.path.join(CSRC, "*.cu")):
+        if path.endswith("selftest.cu"):
+            continue
+        code = _code(path)
+        assert "<<<" not in code, path
+        kernels = re.findall(r"__global__[^;{]*?\b(\w+_kernel)\s*\([^{;]*\)\s*\{(.*?)\n\}", code, re.S)
+        for name, body in kernels:
+            assert "grid_enter" in body, (path, name)
