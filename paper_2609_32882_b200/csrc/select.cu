@@ -127,7 +127,9 @@ __global__ void __launch_bounds__(32) sel_pick_kernel(unsigned* state, const uns
 // denominator keeps what rounding takes from it (router_tc.cu).  (2 2^-18 + 2^-19) ln 2 = 6.6e-6, and with five approximations of
 // ex2 (2^-22 each) and at most 40 additions of 2^-24 on either side less than 1.4e-5.  kBandUlps = 512 units of the last place of t
 // are at least 3.05e-5 of t, more than 2e.
-// Smaller thresholds go back to the two-pass form if their band matters.  About one entry in 10^5 lies in a band.
+// Below kBandLeast the bound does not hold (a thread's sums may be lost altogether), so entries may lie anywhere: a head or row with
+// such a threshold goes back to the two-pass form whatever its band holds, unless everything is kept.  About one entry in 10^5 lies in a
+// band.
 constexpr unsigned kBandUlps = 512, kBandLeast = 0x21800000u, kBandMost = 0x7f000000u;
 __device__ __forceinline__ unsigned band_lo(unsigned tau) { return tau > kBandUlps ? tau - kBandUlps : 0u; }
 __device__ __forceinline__ unsigned band_hi(unsigned tau) { return tau < 0xffffffffu - kBandUlps ? tau + kBandUlps : 0xffffffffu; }
@@ -303,16 +305,18 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* pr,
     row_cnt[o] = k;
   }
   if constexpr (MODE == kBand) {
+    if (k == N) return;
+    if (!band_usable(tau)) {
+      if (lane == 0) atomicExch(se.redo, 1);
+      return;
+    }
     const unsigned lo = band_lo(tau), hi = band_hi(tau);
     int from = 0;                     // entries above the lower end of the band: more than k, and the band matters
 #pragma unroll
     for (int u = 0; u < U; ++u) from += u * 32 + lane < N && v[u] >= lo;
     from = __reduce_add_sync(0xffffffffu, from);
     if (from > k) {
-      if (lane == 0) {
-        if (band_usable(tau)) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
-        else atomicExch(se.redo, 1);
-      }
+      if (lane == 0) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (u * 32 + lane < N && v[u] >= lo && v[u] <= hi) settle_list(se, (int)o, u * 32 + lane);
@@ -372,6 +376,11 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
     row_cnt[o] = k;
   }
   if constexpr (MODE == kBand) {
+    if (k == N) return;                           // (one row a block)
+    if (!band_usable(tau)) {
+      if (threadIdx.x == 0) atomicExch(se.redo, 1);
+      return;
+    }
     const unsigned lo = band_lo(tau), hi = band_hi(tau);
     int from = 0;
     for (int j = threadIdx.x; j < N; j += blockDim.x) from += src[j] >= lo;
@@ -380,10 +389,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
     if (from > 0) atomicAdd(&sh[0], (unsigned)from);
     __syncthreads();
     if (sh[0] > (unsigned)k) {
-      if (threadIdx.x == 0) {
-        if (band_usable(tau)) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
-        else atomicExch(se.redo, 1);
-      }
+      if (threadIdx.x == 0) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
       for (int j = threadIdx.x; j < N; j += blockDim.x) {
         const unsigned v = src[j];
         if (v >= lo && v <= hi) settle_list(se, (int)o, j);
@@ -602,8 +608,9 @@ __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* pr, int N
   const int need = (int)keep - tot;
   block_excl_scan(band, ws, band);
   if (tid == 0) state[bh * 8 + 4] = (unsigned)need;
-  if (band == need) return;
-  if (band > kBandHead || !band_usable(state[bh * 8 + 3])) {
+  const bool usable = band_usable(state[bh * 8 + 3]);
+  if (band == need && (usable || keep == (unsigned)((size_t)N * N))) return;
+  if (band > kBandHead || !usable) {
     if (tid == 0) atomicExch(se.redo, 1);
     return;
   }

@@ -140,3 +140,53 @@ def test_pairs_whose_flat_index_is_beyond_32_bits_are_settled():
     assert redo == 0 and pairs > 0
     for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), *maps):
         assert torch.equal(x, y), name
+
+
+def _levels(kind):
+    """256 cubes, 16 key tiles of 16 cubes; a thread has the cubes 4 part .. 4 part + 3 of every tile.  Scores of the key cubes in nats below a
+    dominant key in cube 0, by query sub-cube (0; the others)."""
+    cube = torch.arange(256, device="cuda")
+    tile, part = cube // 16, cube % 16 // 4
+    if kind == "tail":          # parts 1 - 3: the first tile 130 octaves down, the later ones 69; part 0: from 101 octaves on, cube by cube
+        k0 = torch.where(tile == 0, -90.0, -48.0)
+        in0 = part == 0
+        k0[in0] = -70.0 - 0.5 * torch.arange(int(in0.sum()), device="cuda")
+        k1 = k0
+        k2 = torch.zeros(256, device="cuda")
+    else:                       # "rows": part 0 leads by a 16th of a nat where sub-cube 0 asks, parts 1 - 3 by a tenth with the other sub-cubes
+        k0 = torch.where((part > 0) & (tile == 0), -38.0, -37.0)
+        k1 = torch.where(part == 0, -100.0, torch.where(tile == 0, -85.5, -41.25))
+        k2 = torch.where(part == 0, 0.5, 0.0)
+    k0, k1, k2 = k0.clone(), k1.clone(), k2.clone()
+    k0[0] = k1[0] = k2[0] = 0.0
+    return k0, k1, k2
+
+
+@pytest.mark.parametrize("kind,mode", [("tail", ROW), ("tail", SEQ), ("tail", BUDGET)])
+def test_thresholds_far_below_the_row_maximum(kind, mode):
+    """A thread's parked sums are lost where its first scores lie 2^126 below the row's denominator, the scores it has later (up to 2^64
+    more) with them: a threshold so low must not be taken from one-pass scores, however clear of its neighbours it is."""
+    grid, topk = (16, 32, 32), 4
+    k0, k1, k2 = _levels(kind)
+    t, h, w = (x.reshape(-1) for x in torch.meshgrid(*(torch.arange(n, device="cuda") for n in grid), indexing="ij"))
+    of = (t // 4 * 8 + h // 4) * 8 + w // 4
+    first = ((t % 4 < 2) & (h % 4 < 2) & (w % 4 < 2)).float()                 # tokens of sub-cube 0
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    noise = 0.25 if kind == "tail" else 0.0
+    q = noise * torch.randn(1, 1, 16384, 64, device="cuda", generator=gen)
+    k = noise * 4 * torch.randn(1, 1, 16384, 64, device="cuda", generator=gen)
+    q[..., 0], q[..., 1], q[..., 2] = 8.0 * first, 8.0 * (1.0 - first), 1.0
+    k[..., 0], k[..., 1], k[..., 2] = k0[of], k1[of], k2[of]
+    q, k = q.bfloat16(), k.bfloat16()
+    budgets = torch.full((1, 1, 256), topk, device="cuda", dtype=torch.int32) if mode == BUDGET else None
+    p = vb.make_params(1, 1, 1, 64, grid, select_mode=mode, topk=0 if mode == BUDGET else topk, nnz_cap=256 * topk)
+    attn = vb.Vsa2Attention(p)
+    scratch = torch.empty(16 << 20, dtype=torch.uint8, device="cuda")
+    maps = []
+    for s in (None, scratch):
+        vb.vsa2_route(p, q, k, budgets, attn.map, attn.ws_route, scratch=s)
+        attn.check_status()
+        maps.append([x.clone() for x in attn.map_views()])
+    assert _state(attn)[0] == 1
+    for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), *maps):
+        assert torch.equal(x, y), name
