@@ -98,9 +98,10 @@ struct RouterOne {
   float* lse2;         // [BH, N * G]: log2 of the row denominators
   int* redo;           // raised when the scores of this launch are not to be used; two-pass launch: runs only if it is up (or null)
 };
-// The reference of a thread's parked sums is the maximum of its first 32 valid keys.  The maximum may grow by a factor 2^64 along
-// the row; terms 2^-126 below the reference are lost, of which no score of 2^-60 or more consists (select.cu)
-constexpr float kRtMostGrowth = 64.f;
+// The reference of a thread's parked sums is the maximum of its first 32 valid keys.  The maximum may grow by a factor 2^48 along
+// the row.  Where the reference lies more than 2^126 below the denominator all that a thread has of the row is lost: terms of less than
+// 2^-78 each, little of any score of 2^-52 or more even when the terms are summed over the 16 heads of a group (select.cu)
+constexpr float kRtMostGrowth = 48.f;
 // 2^(a - b) with the rounding of the difference put back (exponents of 16 to 32 would lose 7e-7)
 __device__ __forceinline__ float rt_exp2_diff(float a, float b) {
   const float d = a - b, t = d - a, lost = (a - (d - t)) - (b + t);

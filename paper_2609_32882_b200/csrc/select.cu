@@ -122,15 +122,16 @@ __global__ void __launch_bounds__(32) sel_pick_kernel(unsigned* state, const uns
 // A one-pass score x stands for a two-pass score within a factor 1 +- e.  With t the K-th largest x, entries above t (1 + 2e) are
 // among the K largest two-pass scores and entries below t (1 - 2e) are not, so only those between -- the band -- need their
 // two-pass scores, and only where the band holds more entries than are still wanted.
-// e: of a term that counts in a score of at least kBandLeast = 2^-60, either form rounds an exponent below 128 once (half an ulp,
-// 2^-18); the one-pass form also rounds the growth of the row's maximum, at most 64 (2^-19), while its reference against the
-// denominator keeps what rounding takes from it (router_tc.cu).  (2 2^-18 + 2^-19) ln 2 = 6.6e-6, and with five approximations of
-// ex2 (2^-22 each) and at most 40 additions of 2^-24 on either side less than 1.4e-5.  kBandUlps = 512 units of the last place of t
+// e: of a term that counts in a score of at least kBandLeast = 2^-52, either form rounds an exponent below 128 once (half an ulp,
+// 2^-18); the one-pass form also rounds the growth of the row's maximum, at most 48 (2^-19), while its reference against the
+// denominator keeps what rounding takes from it (router_tc.cu).  (2 2^-18 + 2^-19) ln 2 = 6.6e-6, with five approximations of
+// ex2 (2^-22 each) and at most 40 additions of 2^-24 on either side 1.26e-5.  A query cube's other rows, and other heads of a group, may
+// have lost terms of 2^-78 (router_tc.cu): 2^-74 of a sum over 16 heads, 2^-22 of kBandLeast.  Together less than 1.4e-5.  kBandUlps = 512 units of the last place of t
 // are at least 3.05e-5 of t, more than 2e.
 // Below kBandLeast the bound does not hold (a thread's sums may be lost altogether), so entries may lie anywhere: a head or row with
 // such a threshold goes back to the two-pass form whatever its band holds, unless everything is kept.  About one entry in 10^5 lies in a
 // band.
-constexpr unsigned kBandUlps = 512, kBandLeast = 0x21800000u, kBandMost = 0x7f000000u;
+constexpr unsigned kBandUlps = 512, kBandLeast = 0x25800000u, kBandMost = 0x7f000000u;
 __device__ __forceinline__ unsigned band_lo(unsigned tau) { return tau > kBandUlps ? tau - kBandUlps : 0u; }
 __device__ __forceinline__ unsigned band_hi(unsigned tau) { return tau < 0xffffffffu - kBandUlps ? tau + kBandUlps : 0xffffffffu; }
 __device__ __forceinline__ bool band_usable(unsigned tau) { return tau >= kBandLeast && tau <= kBandMost; }
