@@ -482,7 +482,8 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         misc->row_lse2[row] = lse2;
         if (ONE && r < NG) {
           one.lse2[(size_t)bhq * NG + r] = lse2;
-          if (q_valid && !(fabsf(lse2) < INFINITY)) atomicExch(one.redo, 1);
+          // (a denominator that is not a number leaves lse2 = 0, and the two-pass form then has the bare exponentials)
+          if (q_valid && !(l_run < INFINITY && fabsf(lse2) < INFINITY)) atomicExch(one.redo, 1);
         }
         tc::mbar_arrive(&misc->lse_ready);
       }

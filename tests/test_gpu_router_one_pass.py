@@ -190,3 +190,34 @@ def test_thresholds_far_below_the_row_maximum(kind, mode):
     assert _state(attn)[0] == 1
     for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), *maps):
         assert torch.equal(x, y), name
+
+
+@pytest.mark.parametrize("mode", [SEQ, ROW])
+@pytest.mark.parametrize("kind", ["key nan", "key inf", "key -inf", "query nan", "query inf"])
+def test_scores_that_are_not_finite(kind, mode):
+    """Rows whose denominator is not a number keep their scores as they are: 2^144 at the cubes of the first key tile of parts 1 - 3, 2^-86
+    at their others (beyond the fp32 range of what is parked against the first), 1 in part 0."""
+    grid, topk = (16, 32, 32), 200
+    cube = torch.arange(256, device="cuda")
+    level = torch.where(cube % 16 < 4, 0.0, torch.where(cube < 16, 100.0, -60.0))
+    t, h, w = (x.reshape(-1) for x in torch.meshgrid(*(torch.arange(n, device="cuda") for n in grid), indexing="ij"))
+    q, k = (x.float() * 0.1 for x in _inputs(1, 1, 64, grid, "random"))
+    q[..., 0], k[..., 0] = 8.0, level[(t // 4 * 8 + h // 4) * 8 + w // 4]
+    x, value = (q if kind.startswith("query") else k), float(kind.split()[1])
+    x[0, 0, 2048 + 128, 3] = value                       # (of cube 8, of part 2, or of query cube 8)
+    if kind == "key nan":
+        k[0, 0, 2048, 3] = value                         # (of cube 0, of part 0)
+    p = vb.make_params(1, 1, 1, 64, grid, select_mode=mode, topk=topk)
+    attn = vb.Vsa2Attention(p)
+    scratch = torch.empty(16 << 20, dtype=torch.uint8, device="cuda")
+    out = []
+    for s in (None, scratch):
+        vb.vsa2_route(p, q.bfloat16(), k.bfloat16(), None, attn.map, attn.ws_route, scratch=s)
+        attn.check_status()
+        out.append(([x.clone() for x in attn.map_views()], attn.scores()))
+    (two_map, two), (one_map, one) = out
+    for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), two_map, one_map):
+        assert torch.equal(x, y), name
+    assert torch.equal(one.isnan(), two.isnan())
+    counted = two >= 2.0 ** -40
+    assert (((one - two).abs() <= 1.4e-5 * two) | (one == two))[counted].all()
