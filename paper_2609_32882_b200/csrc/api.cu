@@ -384,8 +384,9 @@ cudaError_t prepare_kernel(const void* kernel, KernelAttr& attr, size_t smem, in
   return cudaSuccess;
 }
 
-ProfScope::ProfScope(int kernel_id, cudaStream_t stream, int launches) : id(kernel_id), st(stream) {
-  g_launches += launches;
+void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+
+ProfScope::ProfScope(int kernel_id, cudaStream_t stream) : id(kernel_id), st(stream) {
   if (g_prof_start[id] != nullptr) cudaEventRecord(g_prof_start[id], st);
 }
 ProfScope::~ProfScope() {
@@ -493,7 +494,7 @@ int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const
   bf16* qr = at<bf16>(workspace, rl.qr);
   bf16* kr = at<bf16>(workspace, rl.kr);
   {
-    ProfScope ps(VSA2_KERNEL_POOL_ROUTER, st, 1);
+    ProfScope ps(VSA2_KERNEL_POOL_ROUTER, st);
     VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, status, st));
   }
   float* pr = folded ? at<float>(sel_base, lay.pr) : at<float>(workspace, rl.pr);
@@ -505,22 +506,18 @@ int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const
   int* redo = one ? &status->pad[0] : nullptr;      // (the status block is cleared by the pooling)
   float* lse2 = one ? at<float>(scratch, ol.lse2) : nullptr;
   if (router_tc_supported(r)) {
-    { ProfScope lse(VSA2_KERNEL_ROUTER_LSE, st, 0); }      // (both passes are timed as the second)
-    ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st, 1);
+    { ProfScope lse(VSA2_KERNEL_ROUTER_LSE, st); }      // (both passes are timed as the second)
+    ProfScope ps(VSA2_KERNEL_ROUTER_POOL, st);
     if (one) VSA2_CUDA(launch_router_one(r, folded, qr, kr, pr, at<unsigned char>(scratch, ol.park), lse2, redo, status, st));
     else VSA2_CUDA(launch_router_scores_tc(r, folded, qr, kr, pr, nullptr, status, st));
   } else   // sub-cube counts the tensor-core kernel has no layout for (G = 1 is the VSA router of Sec. 2.1)
     VSA2_CUDA(launch_router_scores(r, qr, kr, at<float>(workspace, rl.lse_r), pr, st));
   if (wide && !folded) {
-    g_launches += 1;
     float* pr_cube = at<float>(sel_base, lay.pr);
     VSA2_CUDA(launch_fold_scores(r, pr, pr_cube, st));
     pr = pr_cube;
   }
-  if (group_sum) {
-    g_launches += 1;
-    VSA2_CUDA(launch_group_sum_scores(g, pr, nullptr, st));
-  }
+  if (group_sum) VSA2_CUDA(launch_group_sum_scores(g, pr, nullptr, st));
   workspace = sel_base;
   SelectScratch s;
   s.hist = at<unsigned>(workspace, lay.hist);
@@ -534,10 +531,9 @@ int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const
   s.bitmap_t = at<unsigned>(workspace, lay.bitmap_t);
   s.words = lay.words;
   {
-    ProfScope ps(VSA2_KERNEL_SELECT, st, (g.mode == VSA2_PER_SEQUENCE ? 14 : 7) - (g.N <= kSelOneBlockN ? 5 : 0));
+    ProfScope ps(VSA2_KERNEL_SELECT, st);
     if (one) {
       const Settle se{redo, &status->pad[1], at<int2>(scratch, ol.pairs), kSettlePairs, &status->pad[2], at<int>(scratch, ol.rows)};
-      g_launches += (g.mode == VSA2_PER_SEQUENCE ? 8 : 1) + 3 + (group_sum ? 1 : 0);
       VSA2_CUDA(launch_select_band(g, pr, budgets, s, se, st));
       VSA2_CUDA(launch_router_exact(r, folded, qr, kr, lse2, se.pairs, se.count, se.cap, group_sum ? g.rep : 1, redo, pr, status, st));
       VSA2_CUDA(launch_select_settle(g, pr, budgets, s, se, st));
@@ -593,7 +589,7 @@ int vsa2_attn_fwd(const vsa2_params* p, const void* q, const void* k, const void
   const float* oc_hat = coarse ? saved->oc_hat : nullptr;
   if (coarse) {
     {
-      ProfScope ps(VSA2_KERNEL_POOL, st, wide ? 6 : 1);
+      ProfScope ps(VSA2_KERNEL_POOL, st);
       if (!wide) {
         VSA2_CUDA(launch_pool_coarse(g, qb, kb, vb, saved->qc, saved->kc, saved->vc, status, st));
       } else {
@@ -607,7 +603,7 @@ int vsa2_attn_fwd(const vsa2_params* p, const void* q, const void* k, const void
       }
     }
     {
-      ProfScope ps(VSA2_KERNEL_COARSE_FWD, st, ((g.flags & VSA2_FLAG_BF16_COARSE_FWD) ? 7 : 1) + (wide ? 1 : 0));
+      ProfScope ps(VSA2_KERNEL_COARSE_FWD, st);
       if (!(g.flags & VSA2_FLAG_BF16_COARSE_FWD))
         VSA2_CUDA(launch_coarse_fwd_mma(g, saved->qc, saved->kc, saved->vc, saved->oc_hat, saved->lse_c, st));
       else
@@ -621,7 +617,6 @@ int vsa2_attn_fwd(const vsa2_params* p, const void* q, const void* k, const void
     }
   }
   if (wide) {
-    g_launches += 1;
     VSA2_CUDA(launch_expand_map(n, map->row_ptr, map->col_idx, at<int>(workspace, wl.ptr64), at<int>(workspace, wl.idx64), st));
     row_ptr = at<int>(workspace, wl.ptr64);
     col_idx = at<int>(workspace, wl.idx64);
@@ -635,14 +630,13 @@ int vsa2_attn_fwd(const vsa2_params* p, const void* q, const void* k, const void
     unsigned char* tbase = at<unsigned char>(workspace, fwd_base_bytes(g));
     fx = text_geo(n);
     if (!fine_fwd_rows_supported(fx)) return VSA2_ERR_UNSUPPORTED;
-    g_launches += 1;
     VSA2_CUDA(launch_extend_map(n, text_blocks(g), row_ptr, col_idx, at<int>(tbase, tl.ptr), at<int>(tbase, tl.idx),
                                 fx.nnz_cap, st));
     row_ptr = at<int>(tbase, tl.ptr);
     col_idx = at<int>(tbase, tl.idx);
   }
   {
-    ProfScope ps(VSA2_KERNEL_FINE_FWD, st, (g.flags & VSA2_FLAG_EXACT_MAX_FWD) ? 1 : 2);
+    ProfScope ps(VSA2_KERNEL_FINE_FWD, st);
     if (g.flags & VSA2_FLAG_EXACT_MAX_FWD)
       VSA2_CUDA(launch_fine_fwd(fx, qb, kb, vb, coarse ? gate : nullptr, row_ptr, col_idx, oc_hat, o, o_res, lse, st));
     else if ((wide || (g.flags & VSA2_FLAG_GROUP_ROUTING)) && fine_fwd_rows2_supported(n, !wide))
@@ -720,7 +714,6 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   const int* row_idx = map->row_idx;
   const float* oc_hat = coarse ? saved->oc_hat : nullptr;
   if (wide) {
-    g_launches += 2;
     VSA2_CUDA(launch_expand_map(n, map->row_ptr, map->col_idx, at<int>(workspace, wl.ptr64), at<int>(workspace, wl.idx64), st));
     VSA2_CUDA(launch_expand_map(n, map->col_ptr, map->row_idx, at<int>(workspace, wl.cptr64), at<int>(workspace, wl.ridx64), st));
     row_ptr = at<int>(workspace, wl.ptr64);
@@ -728,7 +721,6 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
     col_ptr = at<int>(workspace, wl.cptr64);
     row_idx = at<int>(workspace, wl.ridx64);
     if (coarse) {
-      g_launches += 1;
       VSA2_CUDA(launch_expand_rows(n, n.Hq, false, saved->oc_hat, at<float>(workspace, wl.oc_hat64), st));
       oc_hat = at<float>(workspace, wl.oc_hat64);
     }
@@ -738,7 +730,6 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
     const TextMapLayout tl = text_map_layout(g, true);
     unsigned char* tbase = at<unsigned char>(workspace, bwd_base_bytes(g));
     fx = text_geo(n);
-    g_launches += 2;
     VSA2_CUDA(launch_extend_map(n, text_blocks(g), row_ptr, col_idx, at<int>(tbase, tl.ptr), at<int>(tbase, tl.idx),
                                 fx.nnz_cap, st));
     VSA2_CUDA(launch_extend_map(n, text_blocks(g), col_ptr, row_idx, at<int>(tbase, tl.cptr), at<int>(tbase, tl.ridx),
@@ -754,14 +745,14 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   // (V is copied to fp16 for GQA groups only; O is of V's size or, a mean of up to a few thousand rows, well below it)
   const DsScale scale{at<float2>(workspace, lay.absmax), at<int>(workspace, lay.ds_exp), dkv_pass_gqa_f16(g) ? pow2i(-16) : 0.f};
   {
-    ProfScope ps(VSA2_KERNEL_BWD_PRE, st, 1);
+    ProfScope ps(VSA2_KERNEL_BWD_PRE, st);
     VSA2_CUDA(launch_bwd_preprocess(fx, dob, o, o_res, coarse ? gate : nullptr, oc_hat, delta, coarse ? dgate : nullptr,
                                     d_oc_hat, dq_pass_f16(g) ? at<float2>(workspace, lay.absmax) : nullptr,
                                     reinterpret_cast<StatusBlock*>(workspace), st));
   }
   if (coarse) {
     // pooled grid: the bf16 copies with the dense map, the pooled preprocess, dQ, dK/dV (+ two group spreads)
-    ProfScope ps(VSA2_KERNEL_COARSE_BWD, st, 5 + (g.rep > 1 ? 2 : 0) + (wide ? 4 : 0));
+    ProfScope ps(VSA2_KERNEL_COARSE_BWD, st);
     if (wide) VSA2_CUDA(launch_fold_sum(n, n.Hq, d_oc_hat, d_oc_hat_cube, st));
     VSA2_CUDA(launch_coarse_bwd_pooled(g, saved->qc, saved->kc, saved->vc, saved->oc_hat, saved->lse_c, d_oc_hat_cube,
                                        dqc_cube, dkc_cube, dvc_cube, at<unsigned char>(cube_ws, cl.pooled),
@@ -788,21 +779,15 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   const bool wide128 = wide && g.Lt == 0 && fine_bwd128_supported(n);
   {
     const bool f16 = dq_pass_f16(g);     // the copy, the fp16 form, the (idle) fallback
-    ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st, ds_groups > 0 ? 2 : f16 ? 3 : 1);
+    ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st);
     if (ds_groups > 0) {
       VSA2_CUDA(launch_cast_qk(fx, qb, at<unsigned char>(workspace, bwd_f16_offset(g)), kb,
                                at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale,
                                &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
       VSA2_CUDA(launch_ds_positions(dg, sd.row_ptr, sd.col_idx, wide ? map->col_ptr : col_ptr, wide ? map->row_idx : row_idx,
                                     at<int>(scratch, dl.pos), sd.counters, 2 * g.batch * g.Hkv, st));
-      if (pk.shift > 0) {
-        g_launches += 1;
-        VSA2_CUDA(launch_full_counts(fx, pk, col_ptr, row_idx, at<int>(workspace, lay.full), st));
-      }
-      if (dkv_order != nullptr) {
-        g_launches += 1;
-        VSA2_CUDA(launch_dkv_order(dg, wide ? map->col_ptr : col_ptr, dkv_order, st));
-      }
+      if (pk.shift > 0) VSA2_CUDA(launch_full_counts(fx, pk, col_ptr, row_idx, at<int>(workspace, lay.full), st));
+      if (dkv_order != nullptr) VSA2_CUDA(launch_dkv_order(dg, wide ? map->col_ptr : col_ptr, dkv_order, st));
     } else if (wide128)
       VSA2_CUDA(launch_fine_bwd128_dq_tc(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
                                          reinterpret_cast<StatusBlock*>(workspace), st,
@@ -819,10 +804,7 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
     const bool two = !dkv128 && fine_bwd_dkv_splits_long_columns(fx, true);
     const bool gqa16 = !dkv128 && dkv_pass_gqa_f16(g);    // (the copy of V and dO, the all-fp16 form, the pair form as its fallback)
     const bool f16 = (two || gqa16 || ds_groups > 0) && dq_pass_f16(g);      // fp16 copies of Q and K have been made
-    ProfScope ps(VSA2_KERNEL_FINE_BWD_DKV, st, dkv128 ? (dq_pass_f16(g) ? 2 : 1)
-                                                      : two ? 2 + (f16 ? 1 : 0) : (gqa16 ? 3 : 1));
-    const int chunks = ds_groups > 0 ? (g.batch * g.Hkv + ds_groups - 1) / ds_groups : 0;
-    if (chunks > 0) g_launches += 2 * chunks;      // (dQ per chunk and its fallback; the first dK/dV launch is counted above)
+    ProfScope ps(VSA2_KERNEL_FINE_BWD_DKV, st);
     unsigned char* v16 = gqa16 ? at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g) + bwd_k16_bytes(g)) : nullptr;
     if (dkv128 && ds_groups > 0)
       VSA2_CUDA(launch_fine_bwd128_stored(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, col_ptr, row_idx, coarse ? dqc : nullptr,
@@ -853,7 +835,6 @@ int vsa2_permute_cube_major(const vsa2_params* p, int32_t heads, int32_t inverse
   if (!src || !dst || heads <= 0 || heads > 65535) return VSA2_ERR_INVALID_ARG;
   if (!aligned16(src) || !aligned16(dst)) return VSA2_ERR_MISALIGNED;
   if ((rc = check_device()) != VSA2_OK) return rc;
-  g_launches += 1;
   VSA2_CUDA(launch_permute(g, reinterpret_cast<const bf16*>(src), heads, inverse != 0, reinterpret_cast<bf16*>(dst),
                            reinterpret_cast<cudaStream_t>(cuda_stream)));
   return VSA2_OK;
@@ -867,7 +848,6 @@ int vsa2_gate_fwd(const vsa2_params* p, int32_t hidden, const void* x, const voi
   if (!gate_supported(hidden, g.Hq)) return VSA2_ERR_UNSUPPORTED;
   if (!aligned16(x)) return VSA2_ERR_MISALIGNED;
   if ((rc = check_device()) != VSA2_OK) return rc;
-  g_launches += 1;
   VSA2_CUDA(launch_gate_fwd(g.batch, g.L, hidden, g.Hq, reinterpret_cast<const bf16*>(x), reinterpret_cast<const bf16*>(w_g),
                             gate, reinterpret_cast<cudaStream_t>(cuda_stream)));
   return VSA2_OK;
@@ -889,7 +869,6 @@ int vsa2_gate_bwd(const vsa2_params* p, int32_t hidden, const void* x, const voi
   if (!aligned16(x) || !aligned16(dx) || !aligned256(workspace)) return VSA2_ERR_MISALIGNED;
   if (workspace_bytes < gate_bwd_workspace_bytes(g.batch, g.L, hidden, g.Hq)) return VSA2_ERR_WORKSPACE_TOO_SMALL;
   if ((rc = check_device()) != VSA2_OK) return rc;
-  g_launches += 4;
   VSA2_CUDA(launch_gate_bwd(g.batch, g.L, hidden, g.Hq, g.out_f32, reinterpret_cast<const bf16*>(x),
                             reinterpret_cast<const bf16*>(w_g), gate, dgate, d_w_g, dx, workspace,
                             reinterpret_cast<cudaStream_t>(cuda_stream)));

@@ -63,6 +63,7 @@ struct StatusBlock {
 // reads through __ldg or `const __restrict__` pointers (loads on the read-only path may be moved in front of the wait, and owe
 // nothing to it).  `__restrict__` stands only on pointers that a kernel writes and never reads.
 // 2048-token clip, 12 heads, training: 216 us without, 189 with the wait at the top of every kernel, 183 so; ragged clip 733, 709, 702.
+void count_launch();      // (vsa2_launch_count)
 template <typename T> struct NotDeduced { using type = T; };
 template <typename... P>
 inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
@@ -77,7 +78,9 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e == cudaSuccess) count_launch();
+  return e;
 }
 __device__ __forceinline__ void grid_enter(bool early = true) {
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -86,11 +89,11 @@ __device__ __forceinline__ void grid_enter(bool early = true) {
 // Persistent kernels with many items per CTA keep the SMs to themselves until they end
 __device__ __forceinline__ void grid_enter_items(int items) { grid_enter(items <= 8 * (int)gridDim.x); }
 
-// Brackets the launches of one kernel group: counts them and records the caller's timing events.
+// Brackets the launches of one kernel group with the caller's timing events.
 struct ProfScope {
   int id;
   cudaStream_t st;
-  ProfScope(int kernel_id, cudaStream_t stream, int launches);
+  ProfScope(int kernel_id, cudaStream_t stream);
   ~ProfScope();
 };
 

@@ -706,12 +706,11 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
 #define VSA2_LAUNCH_DKV(DD, SP, MH, F, PK, TQ, TK, TQT, TKT, TV, TDO, TVT, TDOT)                                                                         \
   do {                                                                                                                           \
     using L_ = BwdTc<DD, SP ? 2 : kRingA, SP ? 4 : 2>;                                                                           \
-    cfg.dynamicSmemBytes = L_::smem_bytes;                                                                                       \
     static KernelAttr attr_;                                                                                                     \
     if ((e = prepare_kernel((const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F, PK>, attr_, L_::smem_bytes, kDkvThreads,               \
                             128 * (48 + 2 * 120 + 2 * 48 + 96))))                                                                \
       return e;                                                                                                                  \
-    if ((e = cudaLaunchKernelEx(&cfg, fine_bwd_dkv_tc_kernel<DD, SP, MH, F, PK>, TQ, TK, TV, TDO, TQT, TKT, TVT, TDOT, tqe, tdoe, g, a)))       \
+    if ((e = launch_kernel(fine_bwd_dkv_tc_kernel<DD, SP, MH, F, PK>, grid, kDkvThreads, L_::smem_bytes, st, TQ, TK, TV, TDO, TQT, TKT, TVT, TDOT, tqe, tdoe, g, a))) \
       return e;                                                                                                                  \
   } while (0)
   // `when`: see DkvArgs.
@@ -719,16 +718,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   // `overlap`: see DkvArgs.
   auto launch = [&](bool split, int* counter, int k_lo, int k_hi, int when, int group0, int groups,
                     bool ds, int overlap = 0) -> cudaError_t {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const int items = groups * g.N;
-    cfg.gridDim = dim3(items < sms ? items : sms);
-    cfg.blockDim = dim3(kDkvThreads);
-    cfg.stream = st;
+    const int items = groups * g.N, grid = items < sms ? items : sms;
     DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
               group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr, pk, overlap};
