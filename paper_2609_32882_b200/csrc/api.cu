@@ -220,22 +220,20 @@ WideBwdLayout wide_bwd_layout(const Geo& g) {
   return r;
 }
 
-// One-pass router (router_tc.cu): half-cubes, or 64-token cubes, of eight sub-cubes.  Its scratch, from kRouterOneTiles key tiles on,
-// for the SMs of a B200.  Below, the launches that settle the map (4 per query, 11 per sequence) cost more than the exponentials:
+// One-pass router (router_tc.cu): half-cubes, or 64-token cubes, of eight sub-cubes.  Asked for from kRouterOneTiles key tiles on.  Below, the launches that settle the map (4 per query, 11 per sequence) cost more than the exponentials:
 // whole route call, two-pass / one-pass, us: 7,056 tiles (336 cubes, 16 heads of 64 channels) 189 / 208; 7,776 tiles (288 cubes, 24
 // heads) 203 / 223; 18,252 tiles (624 cubes, 12 heads) 322 / 273; 81,000 tiles (1440 cubes, 10 heads) 1145 / 873.
 constexpr long long kRouterOneTiles = 12000;
-constexpr int kRouterOneSms = 148;
 constexpr int kSettlePairs = 1 << 17;      // pairs next to a threshold: about one in 10^5 of a problem's
 bool router_one_supported(const Geo& g) { return wide_cube(g) ? router_folds(g) && router_one_runs(narrow_geo(g)) : router_one_runs(g); }
 struct RouteOneLayout {
   size_t park, lse2, pairs, rows, total;
 };
-RouteOneLayout route_one_layout(const Geo& g, int sms) {
+RouteOneLayout route_one_layout(const Geo& g) {
   const Geo r = wide_cube(g) ? narrow_geo(g) : g;
   RouteOneLayout l;
   Carver c;
-  l.park = c.take(router_one_park_bytes(r, router_folds(g), sms));
+  l.park = c.take(router_one_park_bytes(r, router_folds(g)));
   l.lse2 = c.take((size_t)g.batch * g.Hq * r.N * r.G * sizeof(float));
   l.pairs = c.take((size_t)kSettlePairs * sizeof(int2));
   l.rows = c.take((size_t)g.batch * g.Hq * g.N * sizeof(int));
@@ -461,7 +459,7 @@ size_t vsa2_route_scratch_bytes(const vsa2_params* p) {
   if (fill_geo(p, &g) != VSA2_OK || !router_one_supported(g)) return 0;
   const Geo r = wide_cube(g) ? narrow_geo(g) : g;
   const long long tiles = ((long long)r.N * r.G + 127) / 128;
-  return g.batch * g.Hq * tiles * tiles >= kRouterOneTiles ? route_one_layout(g, kRouterOneSms).total : 0;
+  return g.batch * g.Hq * tiles * tiles >= kRouterOneTiles ? route_one_layout(g).total : 0;
 }
 
 int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const int32_t* budgets, const vsa2_map* map,
@@ -498,10 +496,8 @@ int vsa2_route_scratch(const vsa2_params* p, const void* q, const void* k, const
     VSA2_CUDA(launch_pool_router(r, reinterpret_cast<const bf16*>(q), reinterpret_cast<const bf16*>(k), qr, kr, status, st));
   }
   float* pr = folded ? at<float>(sel_base, lay.pr) : at<float>(workspace, rl.pr);
-  int sms = 0;
-  VSA2_CUDA(sm_count(&sms));
   const bool group_sum = (g.flags & VSA2_FLAG_GROUP_ROUTING) && g.rep > 1;
-  const RouteOneLayout ol = router_one_supported(g) ? route_one_layout(g, sms) : RouteOneLayout{};
+  const RouteOneLayout ol = router_one_supported(g) ? route_one_layout(g) : RouteOneLayout{};
   const bool one = router_one_supported(g) && scratch != nullptr && scratch_bytes >= ol.total;
   int* redo = one ? &status->pad[0] : nullptr;      // (the status block is cleared by the pooling)
   float* lse2 = one ? at<float>(scratch, ol.lse2) : nullptr;

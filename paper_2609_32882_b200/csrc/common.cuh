@@ -248,7 +248,7 @@ cudaError_t launch_router_scores_tc(const Geo& g, bool fold, const bf16* qr, con
                                     cudaStream_t st);
 // the one-pass form and the two-pass scores of listed pairs (router_tc.cu), where router_one_runs
 bool router_one_runs(const Geo& g);
-size_t router_one_park_bytes(const Geo& g, bool fold, int sms);
+size_t router_one_park_bytes(const Geo& g, bool fold);
 cudaError_t launch_router_one(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, void* park, float* lse2, int* redo,
                               StatusBlock* status, cudaStream_t st);
 cudaError_t launch_router_exact(const Geo& g, bool fold, const bf16* qr, const bf16* kr, const float* lse2, const int2* pairs,

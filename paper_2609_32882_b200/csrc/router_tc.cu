@@ -30,6 +30,9 @@ constexpr int kRtParts = 4;        // compute threads per pooled query row (each
 constexpr int kRtThreads = 64 + 128 * kRtParts;    // TMA warp, MMA warp, 4 * kRtParts compute warps
 constexpr int kRtSlots = 4;
 constexpr int kRtTile = 128;
+// one-pass form: at most so many CTAs, those of a B200, on whatever it runs -- a caller asks for the scratch, a region per CTA, without a
+// device at hand
+constexpr int kRtOneCtas = 148;
 constexpr int kRtAhead = 4;        // one-pass form: tiles of parked sums on their way
 constexpr int kRtBufs = 4;         // score tiles in tensor memory (4 x 128 columns = all of it)
 
@@ -564,6 +567,7 @@ static cudaError_t launch_router(const CUtensorMap& tq, const CUtensorMap& tk, c
   static KernelAttr attr;
   if ((e = prepare_kernel((const void*)router_tc_kernel<D, G, FOLD, ONE>, attr, smb))) return e;
   const int total = g.batch * g.Hq * row_tiles;
+  if (ONE && sms > kRtOneCtas) sms = kRtOneCtas;
   launch_kernel(router_tc_kernel<D, G, FOLD, ONE>, total < sms ? total : sms, kRtThreads, smb, st, tq, tk, g, pr, one, status);
   return cudaGetLastError();
 }
@@ -597,9 +601,9 @@ bool router_one_runs(const Geo& g) {
   return g.G == 8 && row_tiles >= 2 * kRtAhead && smb <= 227 * 1024;
 }
 
-size_t router_one_park_bytes(const Geo& g, bool fold, int sms) {
+size_t router_one_park_bytes(const Geo& g, bool fold) {
   const size_t row_tiles = ((size_t)g.N * g.G + kRtTile - 1) / kRtTile, items = (size_t)g.batch * g.Hq * row_tiles;
-  return (items < (size_t)sms ? items : (size_t)sms) * row_tiles * kRtParts * kRtTile * (fold ? sizeof(float2) : sizeof(float4));
+  return (items < (size_t)kRtOneCtas ? items : (size_t)kRtOneCtas) * row_tiles * kRtParts * kRtTile * (fold ? sizeof(float2) : sizeof(float4));
 }
 
 cudaError_t launch_router_one(const Geo& g, bool fold, const bf16* qr, const bf16* kr, float* pr, void* park, float* lse2, int* redo,

@@ -221,3 +221,26 @@ def test_scores_that_are_not_finite(kind, mode):
     assert torch.equal(one.isnan(), two.isnan())
     counted = two >= 2.0 ** -40
     assert (((one - two).abs() <= 1.4e-5 * two) | (one == two))[counted].all()
+
+
+@pytest.mark.parametrize("heads_q,heads_kv,dim,grid,cube,mode", [
+    (4, 4, 128, (21, 30, 52), {}, SEQ),
+    (12, 12, 64, (13, 27, 47), {}, ROW),
+    (2, 2, 128, (61, 30, 52), WIDE, ROW),
+])
+def test_scratch_of_the_size_asked_for_is_enough_and_one_byte_less_is_none(heads_q, heads_kv, dim, grid, cube, mode):
+    p = vb.make_params(1, heads_q, heads_kv, dim, grid, select_mode=mode, topk=16, **cube)
+    q, k = _inputs(heads_q, heads_kv, dim, grid, "random")
+    attn = vb.Vsa2Attention(p)
+    size = vb.vsa2_route_scratch_bytes(p)
+    assert size == attn.route_scratch_bytes > 0
+    guarded = torch.full((size + 4096,), 0xa5, dtype=torch.uint8, device="cuda")
+    scores, settled = [], []
+    for scratch in (None, guarded[:size - 1], guarded[:size]):
+        vb.vsa2_route(p, q, k, None, attn.map, attn.ws_route, scratch=scratch)
+        attn.check_status()
+        scores.append(attn.scores())
+        settled.append(_state(attn))
+    assert (guarded[size:] == 0xa5).all()
+    assert torch.equal(scores[0], scores[1]) and not torch.equal(scores[0], scores[2])
+    assert settled[1] == (0, 0) and settled[2][0] == 0 and settled[2][1] > 0
