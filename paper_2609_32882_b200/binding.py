@@ -327,6 +327,7 @@ class Vsa2Attention:
             self.ws_bwd = torch.empty(s.bwd_workspace_bytes, **u8)
         for ws in (self.ws_route, self.ws_fwd, self.ws_bwd):
             ws[:256].zero_()          # status block
+        self._refused = {}            # scratch there was no room for: {attribute: [bytes, calls it is done without, calls left]}
         self.out_torch_dtype = torch.float32 if params.out_dtype == F32 else torch.bfloat16
 
     # shapes ---------------------------------------------------------------------------------
@@ -375,20 +376,32 @@ class Vsa2Attention:
 
     def _scratch(self, size, device, stream):
         """Scratch for one call of the bytes in attribute `size`, allocated on the stream the call runs on (its memory is then reused in
-        that stream's order)."""
-        torch, n = self.torch, getattr(self, size)
+        that stream's order).  Where there is no room the call does without, and so do the next 16 calls, after a second refusal 32 and so
+        on up to 1024 (a failing request makes the allocator empty its cache); meanwhile the attribute is 0."""
+        torch, n, refused = self.torch, getattr(self, size), self._refused.get(size)
+        if n == 0 and refused is not None:
+            refused[2] -= 1
+            if refused[2] < 0 and not torch.cuda.is_current_stream_capturing():
+                n = refused[0]
         if n == 0:
             return None
         try:
             if stream is None:
-                return torch.empty(n, dtype=torch.uint8, device=device)
-            if isinstance(stream, int):
-                stream = torch.cuda.ExternalStream(stream, device) if stream else torch.cuda.default_stream(device)
-            with torch.cuda.stream(stream):
-                return torch.empty(n, dtype=torch.uint8, device=device)
-        except torch.cuda.OutOfMemoryError:     # not asked for again: a failing request makes the allocator empty its cache
+                scratch = torch.empty(n, dtype=torch.uint8, device=device)
+            else:
+                if isinstance(stream, int):
+                    stream = torch.cuda.ExternalStream(stream, device) if stream else torch.cuda.default_stream(device)
+                with torch.cuda.stream(stream):
+                    scratch = torch.empty(n, dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:
+            calls = min(2 * refused[1], 1024) if refused is not None else 16
+            self._refused[size] = [n, calls, calls]
             setattr(self, size, 0)
             return None
+        if refused is not None:
+            del self._refused[size]
+            setattr(self, size, n)
+        return scratch
 
     def check_status(self, stream=None):
         for name, ws in (("route", self.ws_route), ("fwd", self.ws_fwd), ("bwd", self.ws_bwd)):

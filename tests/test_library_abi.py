@@ -208,3 +208,35 @@ def test_route_scratch_is_checked_and_asked_for_by_large_problems_only():
     args = [ctypes.byref(large), one, one, None, ctypes.byref(m), one]
     assert lib.vsa2_route_scratch(*args, s.route_workspace_bytes, ctypes.c_void_p(128), 1 << 30, None) == vb.ERR_MISALIGNED
     assert lib.vsa2_route_scratch(*args, s.route_workspace_bytes - 1, one, 1 << 30, None) == vb.ERR_WORKSPACE_TOO_SMALL
+
+
+def test_scratch_is_asked_for_again_after_a_shortage():
+    """One refused request does not decide for the rest of a handle's life: it is repeated after 16 calls, 32, ... while there is no room."""
+    import torch
+
+    class Short:
+        """torch, but for its memory."""
+        room, asked = False, 0
+        uint8, cuda = torch.uint8, torch.cuda
+
+        def empty(self, n, **kw):
+            self.asked += 1
+            if not self.room:
+                raise torch.cuda.OutOfMemoryError("no room")
+            return torch.empty(n, **kw)
+
+    attn = object.__new__(vb.Vsa2Attention)
+    attn.torch, attn._refused, attn.route_scratch_bytes, attn.bwd_scratch_bytes = Short(), {}, 4096, 0
+    take = lambda name="route_scratch_bytes": attn._scratch(name, "cpu", None)
+    asked_at = []
+    for call in range(60):
+        before = attn.torch.asked
+        assert take() is None and attn.route_scratch_bytes == 0
+        if attn.torch.asked > before:
+            asked_at.append(call)
+    assert asked_at == [0, 17, 50]
+    attn.torch.room = True
+    got = [take() for _ in range(70)]
+    first = next(i for i, x in enumerate(got) if x is not None)
+    assert attn.route_scratch_bytes == 4096 and all(x.numel() == 4096 for x in got[first:]) and first < 65
+    assert take("bwd_scratch_bytes") is None                       # (0 from the start: none is wanted)
