@@ -274,8 +274,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* pr,
   unsigned v[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) v[u] = u * 32 + lane < N ? src[u * 32 + lane] : 0u;      // (0 is never above a candidate)
-  int k = budgets ? budgets[o] : K;
-  k = max(0, min(k, N));
+  const int asked = budgets ? budgets[o] : K, k = max(0, min(asked, N));
   if (k == 0) {
     if (lane == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
     return;
@@ -306,17 +305,15 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* pr,
     row_cnt[o] = k;
   }
   if constexpr (MODE == kBand) {
-    if (k == N) return;
-    if (!band_usable(tau)) {
-      if (lane == 0) atomicExch(se.redo, 1);
-      return;
-    }
     const unsigned lo = band_lo(tau), hi = band_hi(tau);
     int from = 0;                     // entries above the lower end of the band: more than k, and the band matters
 #pragma unroll
     for (int u = 0; u < U; ++u) from += u * 32 + lane < N && v[u] >= lo;
     from = __reduce_add_sync(0xffffffffu, from);
-    if (from > k) {
+    if (!band_usable(tau)) {
+      // (not `k < N` or `k == N`: nvcc 12.9.86 compiles the latter to true here, whatever the clamped k is)
+      if (lane == 0 && asked < N) atomicExch(se.redo, 1);
+    } else if (from > k) {
       if (lane == 0) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
 #pragma unroll
       for (int u = 0; u < U; ++u)
@@ -339,8 +336,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
   for (size_t n = MODE == kListed ? blockIdx.x : 0; n < listed; n += gridDim.x) {
   const size_t o = MODE == kListed ? (size_t)se.rows[n] : (size_t)blockIdx.y * N + blockIdx.x;
   const unsigned* src = reinterpret_cast<const unsigned*>(pr) + o * N;
-  int k = budgets ? budgets[o] : K;
-  k = max(0, min(k, N));
+  const int asked = budgets ? budgets[o] : K, k = max(0, min(asked, N));
   if (k == 0) {
     if (threadIdx.x == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
     continue;
@@ -377,11 +373,6 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
     row_cnt[o] = k;
   }
   if constexpr (MODE == kBand) {
-    if (k == N) return;                           // (one row a block)
-    if (!band_usable(tau)) {
-      if (threadIdx.x == 0) atomicExch(se.redo, 1);
-      return;
-    }
     const unsigned lo = band_lo(tau), hi = band_hi(tau);
     int from = 0;
     for (int j = threadIdx.x; j < N; j += blockDim.x) from += src[j] >= lo;
@@ -389,7 +380,9 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
     __syncthreads();
     if (from > 0) atomicAdd(&sh[0], (unsigned)from);
     __syncthreads();
-    if (sh[0] > (unsigned)k) {
+    if (!band_usable(tau)) {
+      if (threadIdx.x == 0 && asked < N) atomicExch(se.redo, 1);
+    } else if (sh[0] > (unsigned)k) {
       if (threadIdx.x == 0) se.rows[atomicAdd(se.row_count, 1)] = (int)o;
       for (int j = threadIdx.x; j < N; j += blockDim.x) {
         const unsigned v = src[j];
