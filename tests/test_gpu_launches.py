@@ -96,3 +96,67 @@ def test_launch_count_is_the_number_of_kernels(layer):
     with torch.cuda.graph(graph):
         layer()
     assert vb.vsa2_launch_count() - before == _kernels(graph)
+
+
+REPLAYED = [
+    dict(heads_q=9, heads_kv=9, dim=128, grid=(21, 30, 52), topk=16, mode=SEQ),              # one-pass router, packed query cubes, long lists
+    dict(heads_q=12, heads_kv=4, dim=64, grid=(21, 30, 52), topk=12, flags=vb.FLAG_GROUP_ROUTING),
+    dict(heads_q=3, heads_kv=3, dim=128, grid=(29, 30, 45), topk=9, cube=(4, 4, 8), one_pass=True),
+    dict(heads_q=2, heads_kv=2, dim=64, grid=(4, 8, 8), topk=2, hidden=64),
+]
+
+
+@pytest.mark.parametrize("layer", REPLAYED, ids=_name)
+def test_a_replayed_graph_gives_what_the_calls_give(layer):
+    """A whole pass captured once (the edges between kernels are programmatic there too) and replayed on other inputs."""
+    layer = Layer(**layer)
+    layer()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        captured = layer()
+    for seed in (1, 7, 8):
+        for x, y in zip((layer.q, layer.k, layer.v, layer.d_o, layer.gate), layer.inputs(seed)):
+            x.copy_(y)
+        for x in captured:
+            x.zero_()
+        graph.replay()
+        graph.replay()
+        got = [x.clone() for x in captured]
+        layer.attn.check_status()
+        want = layer()
+        torch.cuda.synchronize()
+        for i, (x, y) in enumerate(zip(got, want)):
+            assert torch.equal(x, y), (seed, i)
+    if layer.attn.route_scratch_bytes or layer.scratch is not None:
+        words = layer.attn.ws_route[:256].view(torch.int32)
+        assert int(words[2]) == 0 and int(words[3]) > 0               # (the one-pass form, with pairs to settle)
+
+
+def test_two_host_threads_on_two_streams():
+    """Each thread's kernels are placed beside the other's, some with tensor memory for the whole SM."""
+    layers = [Layer(**REPLAYED[0]), Layer(heads_q=4, heads_kv=2, dim=128, grid=(13, 30, 45), topk=9, one_pass=True, seed=2)]
+    want = [layer() for layer in layers]
+    torch.cuda.synchronize()
+    results, errors = [None, None], []
+
+    def work(i):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for _ in range(12):
+                    results[i] = layers[i]()
+            stream.synchronize()
+        except Exception as e:                                          # noqa: BLE001 (handed to the test's thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for layer, got, ref in zip(layers, results, want):
+        layer.attn.check_status()
+        for x, y in zip(got, ref):
+            assert torch.equal(x, y)

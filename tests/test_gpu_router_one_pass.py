@@ -29,6 +29,12 @@ CASES = [
     (2, 2, 128, (28, 28, 32), WIDE, ROW, 20, 0, "growing"),
     (2, 2, 64, (16, 32, 32), {}, SEQ, 200, 0, "peaked"),                         # thresholds below 2^-60
     (2, 2, 64, (16, 32, 32), {}, ROW, 256, 0, "random"),                         # everything is kept
+    (2, 1, 128, (8, 32, 32), {}, SEQ, 7, 0, "random"),                           # eight tiles, one block builds the map of what was settled
+    (3, 3, 64, (8, 32, 32), {}, ROW, 9, 0, "random"),
+    (2, 2, 128, (16, 16, 64), WIDE, SEQ, 11, 0, "random"),                       # the same with cubes of 128 tokens
+    (2, 2, 64, (16, 32, 32), {}, ROW, 7, 0, "few"),                              # ties by the row, few enough to be settled
+    (2, 2, 64, (16, 32, 32), {}, SEQ, 10, 0, "region"),                          # 4096 ties at the threshold
+    (2, 2, 64, (16, 32, 32), {}, ROW, 10, 0, "region"),
 ]
 
 
@@ -49,6 +55,13 @@ def _inputs(heads_q, heads_kv, dim, grid, kind):
         t = torch.arange(rows, device="cuda") // (grid[1] * grid[2]) / (grid[0] - 1)
         q[..., 0] = 4.0
         k[..., 0] = (60.0 * dim ** 0.5 / 4.0 * t)[None, None, :]
+    elif kind == "few":          # an eighth of the cubes repeat others
+        v = k.view(1, heads_kv, *grid, dim)
+        v[:, :, 12:, :16] = v[:, :, :4, :16]
+        q, k = 2.0 * q, 2.0 * k
+    elif kind == "region":       # a quarter of the rows without content
+        for x in (q, k):
+            x.view(1, -1, *grid, dim)[:, :, :, :grid[1] // 4] = 1.0
     elif kind == "peaked":
         q, k = 24.0 * q, 24.0 * k
     return q.bfloat16(), k.bfloat16()
@@ -82,6 +95,16 @@ def test_one_pass_maps_are_the_two_pass_maps(case):
         nnz = int(views[0][..., -1].max())
         out.append(([views[0].clone(), views[1][..., :nnz].clone(), views[2].clone(), views[3][..., :nnz].clone()], attn.scores()))
     (two_map, two), (one_map, one) = out
+    redo, pairs = _state(attn)
+    if tiles < 8:
+        assert torch.equal(one, two)
+    elif kind in ("growing", "peaked") and topk < n:             # seen by the router: nothing is listed
+        assert (redo, pairs) == (1, 0) and torch.equal(one, two)
+    elif mode == SEQ and kind in ("constant", "region"):         # a head has more ties at its threshold than are ranked
+        assert redo == 1 and pairs > 0 and torch.equal(one, two)
+    else:                        # the one-pass form's scores but for the pairs that are settled, and its map
+        assert redo == 0 and (kind == "constant" or not torch.equal(one, two))
+        assert pairs > 0 or topk == n or (mode != SEQ and kind == "random")
     for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), two_map, one_map):
         if mode != BUDGET or "ptr" in name:
             assert torch.equal(x, y), name
