@@ -53,6 +53,19 @@ def test_scratch_is_given_back_and_done_without_when_there_is_no_room():
         assert torch.equal(a, b) and torch.equal(a, c)
 
 
+def test_routes_without_scratch_when_there_is_no_room():
+    attn, qkvg, _ = make(6, heads_q=9, heads_kv=9, grid=(21, 30, 52), topk=16)
+    assert attn.route_scratch_bytes > 1 << 20
+    attn.route(*qkvg[:2])
+    want, scores = [x.clone() for x in attn.map_views()], attn.scores()
+    attn.route_scratch_bytes = 1 << 50                       # more than any GPU has
+    attn.route(*qkvg[:2])
+    attn.check_status()
+    assert attn.route_scratch_bytes == 0 and not torch.equal(attn.scores(), scores)
+    for x, y in zip(want, attn.map_views()):
+        assert torch.equal(x, y)
+
+
 def test_handles_on_two_streams_and_in_a_graph():
     """Two handles whose backwards overlap on two streams (one given as a torch stream, one as its handle), and one whose passes
     are captured and replayed while the other runs."""
