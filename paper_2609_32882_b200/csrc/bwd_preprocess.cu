@@ -11,7 +11,9 @@ namespace vsa2 {
 // (six loads in flight; four CTAs per SM); the D / 8 threads of a token reduce its two row sums with shuffles.  The sum
 // gate_l dO_l runs over the tokens in order, so the dO rows are left in shared memory for one thread per channel.  (With
 // one thread per chunk walking the block's tokens a small problem waited for sixteen rounds of loads, 21 us.)
-template <int D>
+// F32: the type of O.  (As a branch in the loop it cost the loads of a token their place ahead of the first use: 720p, 40 heads, 646 us
+// against 533 = 4.5 TB/s.)
+template <int D, bool F32>
 __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o, const void* o,
                                                              const bf16* o_res,
                                                              const float* gate,
@@ -48,23 +50,21 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
   for (int p0 = threadIdx.x / CH; p0 < kBlockTokens; p0 += TOK * PAR) {
     int l[TOK];
     float gt[TOK];
-    uint4 dv[TOK], ob[TOK], rb[TOK];
-    float4 of[TOK][2];
+    uint4 dv[TOK], ov4[TOK][2];            // (O in fp32, or in bf16 and its residual: the same registers)
 #pragma unroll
     for (int u = 0; u < TOK; ++u) {
       l[u] = block_token(g, i, p0 + u * PAR);
       gt[u] = 0.f;
-      dv[u] = ob[u] = rb[u] = make_uint4(0, 0, 0, 0);
-      of[u][0] = of[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      dv[u] = ov4[u][0] = ov4[u][1] = make_uint4(0, 0, 0, 0);
       if (l[u] >= 0) {
         const size_t base = (bhq * g.S + l[u]) * D + ch * 8;
         dv[u] = *reinterpret_cast<const uint4*>(d_o + base);
-        if (g.out_f32) {
-          of[u][0] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(o) + base);
-          of[u][1] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(o) + base + 4);
+        if constexpr (F32) {
+          ov4[u][0] = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(o) + base);
+          ov4[u][1] = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(o) + base + 4);
         } else {
-          ob[u] = *reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(o) + base);
-          if (o_res != nullptr) rb[u] = *reinterpret_cast<const uint4*>(o_res + base);
+          ov4[u][0] = *reinterpret_cast<const uint4*>(reinterpret_cast<const bf16*>(o) + base);
+          if (o_res != nullptr) ov4[u][1] = *reinterpret_cast<const uint4*>(o_res + base);
         }
         if (coarse) gt[u] = gate[bhq * g.L + l[u]];
       }
@@ -86,15 +86,18 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
         const float2 f = __bfloat1622float2(d2[e]);
         dd[2 * e] = f.x; dd[2 * e + 1] = f.y;
       }
-      if (g.out_f32) {
-        ov[0] = of[u][0].x; ov[1] = of[u][0].y; ov[2] = of[u][0].z; ov[3] = of[u][0].w;
-        ov[4] = of[u][1].x; ov[5] = of[u][1].y; ov[6] = of[u][1].z; ov[7] = of[u][1].w;
+      if constexpr (F32) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          ov[4 * e] = __uint_as_float(ov4[u][e].x); ov[4 * e + 1] = __uint_as_float(ov4[u][e].y);
+          ov[4 * e + 2] = __uint_as_float(ov4[u][e].z); ov[4 * e + 3] = __uint_as_float(ov4[u][e].w);
+        }
       } else {
-        const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&ob[u]);
-        const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&rb[u]);
+        const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&ov4[u][0]);
+        const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&ov4[u][1]);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float2 f = __bfloat1622float2(o2[e]), r = __bfloat1622float2(r2[e]);     // (no residual: rb is zero)
+          const float2 f = __bfloat1622float2(o2[e]), r = __bfloat1622float2(r2[e]);     // (no residual: zero)
           ov[2 * e] = f.x + r.x; ov[2 * e + 1] = f.y + r.y;
         }
       }
@@ -140,8 +143,10 @@ cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, 
                                   const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, float2* absmax,
                                   StatusBlock* clear, cudaStream_t st) {
   dim3 grid(g.N, g.Hq, g.batch);
-  if (g.D == 128) launch_kernel(bwd_preprocess_kernel<128>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
-  else launch_kernel(bwd_preprocess_kernel<64>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  if (g.D == 128 && g.out_f32) launch_kernel(bwd_preprocess_kernel<128, true>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  else if (g.D == 128) launch_kernel(bwd_preprocess_kernel<128, false>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  else if (g.out_f32) launch_kernel(bwd_preprocess_kernel<64, true>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  else launch_kernel(bwd_preprocess_kernel<64, false>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
   return cudaGetLastError();
 }
 

@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(kGtThreads) gate_dz_kernel(const float* gate, 
 // channels, the others the second's) and then has 4 channels of each step as its logical k = 2t, 2t+1, 2t+8, 2t+9; the rows
 // of W lie in that order in shared memory, for ldmatrix.  (8-byte loads need no trade but twice the cache look-ups: 75,600 tokens of
 // 5,120 channels, 40 heads 345 us against 296; 10 heads 168 both ways.)  The loads of the next chunk are in flight while a chunk is multiplied; warps beyond MW HW only
-// stage W.
+// stage W.  Least CTAs per SM where the compiler's own choice of registers is slower: 32 heads 213 us (240), 40 heads 293 (320).
 template <int NT, int MW, int HW, int CH>
-__global__ void __launch_bounds__(kGtThreads) gate_fwd_kernel(const bf16* x, const bf16* w, int L,
+__global__ void __launch_bounds__(kGtThreads, MW != 4 ? 0 : NT == 4 ? 4 : NT == 5 ? 3 : 0) gate_fwd_kernel(const bf16* x, const bf16* w, int L,
                                                               int C, int Hq, float* __restrict__ gate) {
   grid_enter();
   static_assert(NT % HW == 0 && MW * HW * 32 <= kGtThreads, "warps of a CTA");
