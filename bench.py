@@ -38,20 +38,20 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the 720p top-64 launch with 40 heads: an
 # 8-head ncu capture of the same kernel times 5 (every head streams its own tensors, so the traffic grows in
 # proportion to the heads; the 40-head launch is too large for a full-set capture).
-NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.501570e9 + 0.293740e9),
+NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.505465e9 + 0.293843e9),
                                 # copies of Q and K + dK/dV with the stored dS + dQ from it
-                                "fine_bwd": 5 * ((0.309830e9 + 0.261202e9) + (2.446885e9 + 6.304944e9) + (6.611088e9 + 0.159028e9)),
-                                # one-pass router: the parked scores are written and read once (4-head capture)
-                                "router_pool": 10 * (0.229342e9 + 0.244402e9)}
+                                "fine_bwd": 5 * ((0.309827e9 + 0.264207e9) + (1.562046e9 + 5.232290e9) + (5.133052e9 + 0.135355e9)),
+                                # one-pass router: the parked scores are written and read once
+                                "router_pool": 5 * (0.532343e9 + 0.564607e9)}
 
 
 # What ncu shows as the busiest unit of each tensor kernel at 64-token cubes (8-head capture, profiles/): the roofline
 # below is quoted against the tensor peak as the contract asks, these say what actually holds the kernel there.
 NCU_LIMITER = {
     "fine_fwd": "L2 -> SM read rate: 12.9 TB/s against 11.8 TB/s sustained peak (tensor pipe 82 % active at the half rate of M = 64)",
-    "fine_bwd": "dK/dV: shared-memory data pipe 99 % (tensor-core operand fetches 68 % + thread loads/stores 31 %; tensor pipe 46 %); "
-                "dQ from the stored dS: DRAM 68 % (tensor pipe 33 %)",
-    "router_pool": "instruction issue 69 %, exponential unit 63 % (one ex2 per score) of the cycles an SM is busy; 4-head capture",
+    "fine_bwd": "dK/dV: shared-memory data pipe 88 % (tensor-core operand fetches 61 % + thread loads/stores 27 %; tensor pipe 41 %); "
+                "dQ from the stored dS: DRAM 54 % (tensor pipe 33 %)",
+    "router_pool": "instruction issue 71 %, exponential unit 66 % (one ex2 per score)",
 }
 # L2 -> SM read rate that ncu reports as the sustained peak of this part (derived__lts__lts2xbar_bytes.sum.peak_sustained
 # in the 8-head capture of profiles/kernels_720p_8heads_ncu_full.md, where the fine forward itself reads 12.0 TB/s).
