@@ -185,11 +185,13 @@ def _levels(kind):
     return k0, k1, k2
 
 
-@pytest.mark.parametrize("kind,mode", [("tail", ROW), ("tail", SEQ), ("tail", BUDGET), ("rows", ROW)])
-def test_thresholds_far_below_the_row_maximum(kind, mode):
+@pytest.mark.parametrize("kind,mode,topk", [("tail", ROW, 4), ("tail", SEQ, 4), ("tail", BUDGET, 4), ("rows", ROW, 4),
+                                            ("tail", ROW, 256), ("tail", SEQ, 256), ("tail", BUDGET, 300)])
+def test_thresholds_far_below_the_row_maximum(kind, mode, topk):
     """A thread's parked sums are lost where its first scores lie 2^126 below the row's denominator, the scores it has later (up to 2^48
-    more) with them: a threshold so low must not be taken from one-pass scores, however clear of its neighbours it is."""
-    grid, topk = (16, 32, 32), 4
+    more) with them: a threshold so low must not be taken from one-pass scores, however clear of its neighbours it is -- unless
+    everything is kept."""
+    grid = (16, 32, 32)
     k0, k1, k2 = _levels(kind)
     t, h, w = (x.reshape(-1) for x in torch.meshgrid(*(torch.arange(n, device="cuda") for n in grid), indexing="ij"))
     of = (t // 4 * 8 + h // 4) * 8 + w // 4
@@ -202,7 +204,8 @@ def test_thresholds_far_below_the_row_maximum(kind, mode):
     k[..., 0], k[..., 1], k[..., 2] = k0[of], k1[of], k2[of]
     q, k = q.bfloat16(), k.bfloat16()
     budgets = torch.full((1, 1, 256), topk, device="cuda", dtype=torch.int32) if mode == BUDGET else None
-    p = vb.make_params(1, 1, 1, 64, grid, select_mode=mode, topk=0 if mode == BUDGET else topk, nnz_cap=256 * topk)
+    p = vb.make_params(1, 1, 1, 64, grid, select_mode=mode, topk=0 if mode == BUDGET else topk,
+                       nnz_cap=256 * min(topk, 256))
     attn = vb.Vsa2Attention(p)
     scratch = torch.empty(16 << 20, dtype=torch.uint8, device="cuda")
     maps = []
@@ -210,7 +213,7 @@ def test_thresholds_far_below_the_row_maximum(kind, mode):
         vb.vsa2_route(p, q, k, budgets, attn.map, attn.ws_route, scratch=s)
         attn.check_status()
         maps.append([x.clone() for x in attn.map_views()])
-    assert _state(attn)[0] == 1
+    assert _state(attn)[0] == (topk < 256)
     for name, x, y in zip(("row_ptr", "col_idx", "col_ptr", "row_idx"), *maps):
         assert torch.equal(x, y), name
 
