@@ -6,6 +6,8 @@
 // integer work only).
 #include "common.cuh"
 
+#include <cooperative_groups.h>
+
 namespace vsa2 {
 
 constexpr int kHistBins = 2048;
@@ -411,7 +413,8 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
   }
 }
 
-// exclusive scan of v over the block (1024 threads); returns the prefix, total in `total`
+// exclusive scan of v over the block (up to 1024 threads, whole warps); returns the prefix, total in `total`
+template <int THREADS = 1024>
 __device__ __forceinline__ int block_excl_scan(int v, int* warp_sums, int& total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int incl = v;
@@ -422,7 +425,7 @@ __device__ __forceinline__ int block_excl_scan(int v, int* warp_sums, int& total
   if (lane == 31) warp_sums[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    int w = warp_sums[lane];
+    int w = lane < THREADS / 32 ? warp_sums[lane] : 0;
     int wi = w;
     for (int o = 1; o < 32; o <<= 1) {
       int t = __shfl_up_sync(0xffffffffu, wi, o);
@@ -779,6 +782,312 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, 
   }
 }
 
+// ---- a head in one launch ----------------------------------------------------------------------------------------------------
+// Per sequence, mid sizes: a cluster of eight CTAs per head, each with an eighth of the rows.  Behind the router the steps above are 14
+// launches of a few microseconds of work each, every one of them a wait for the one before, and the scores are read four times; here a
+// head's scores are read once into the cluster's shared memory, the histograms and the counts of the parts meet through distributed
+// shared memory, and both maps are written at the end.  What bounds it is latency: nine cluster barriers with reads of the other parts' memory
+// behind them (about 10 of 22 us at 288 cubes).  Everything is counted in integers and placed by prefix sums in row and column
+// order, so the maps are those of the other form, ties and truncation included.
+// Route calls, us, the launches above / this: 180 cubes, 12 heads 84 / 59; 288 cubes, 2 heads 79 / 64, 24 heads 183 / 158; 336 cubes, 16
+// heads 180 / 163, 32 heads behind the one-pass router 270 / 229; 384 cubes, 16 heads 204 / 184; 480 cubes, 2 heads 99.6 / 96.3, 32
+// heads 409 / 407; 528 cubes, 2 heads 109 / 111, 32 heads 475 / 481: eight CTAs a head are too few from there on, hence kSelHeadN.
+// (One to 128 cubes have sel_maps_kernel.  For the maps of the per-row modes, and from bitmaps, a cluster was slower: 480p, 12 heads 264 / 279.)
+// MAPS: the maps are written.  Without: bitmaps, counts and threshold as sel_row_bits_kernel leaves them, for one-pass scores (BAND: as there).
+constexpr int kSelParts = 8, kSelHeadThreads = 512, kSelHeadN = 480;
+struct SelHead {
+  const float* pr;
+  int N, words;
+  unsigned keep;
+  unsigned* state;
+  unsigned *bits_gt, *bits_eq;
+  int *row_gt, *row_eq;
+  int *row_ptr, *col_idx, *col_ptr, *row_idx;
+  long long nnz_cap;
+  StatusBlock* status;
+};
+// shared memory in words: the part's scores (kScores); then two histograms, in whose place afterwards the part's kept bits by row and by
+// column, its counts by column and the places of its entries in the columns' lists lie; then per row the kept entries' position and the entries
+// taken at the threshold
+struct SelHeadSmem {
+  int rows, groups, hist, bm, eq, bt, cnt, col, pos, take, total;
+  __host__ __device__ SelHeadSmem(int N, int words) {
+    rows = (N + kSelParts - 1) / kSelParts;
+    groups = (rows + 31) / 32;
+    hist = (rows * N + 3) & ~3;
+    bm = hist;
+    eq = bm + rows * words;
+    bt = eq + rows * words;
+    cnt = bt + groups * N;
+    col = cnt + N;
+    pos = col + N;
+    if (pos < hist + 2 * kHistBins) pos = hist + 2 * kHistBins;
+    take = pos + rows;
+    total = take + rows;
+  }
+};
+
+template <bool BAND, bool MAPS>
+__global__ void __cluster_dims__(kSelParts, 1, 1) __launch_bounds__(kSelHeadThreads) sel_head_kernel(SelHead a, Settle se) {
+  grid_enter();
+  if (!BAND && !MAPS && *se.redo == 0) return;      // (the whole grid)
+  extern __shared__ unsigned sm[];
+  constexpr int T = kSelHeadThreads, WARPS = T / 32;
+  __shared__ int ws[33], part_tot[2], base[4];
+  __shared__ unsigned pick[2];
+  __shared__ alignas(16) unsigned slice[kHistBins / kSelParts];
+  const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int part = (int)cluster.block_rank(), bh = blockIdx.x / kSelParts;
+  const int N = a.N, words = a.words, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const SelHeadSmem L(N, words);
+  const int r0 = part * L.rows, rows = max(0, min(L.rows, N - r0));
+  const size_t row0 = (size_t)bh * N + r0;
+  const unsigned* src = reinterpret_cast<const unsigned*>(a.pr) + row0 * N;
+  unsigned tau = 0u;
+  int quota = 0;
+
+  {
+    // threshold: three digits, most significant first; the first histogram is taken while the scores come in
+    const int n = rows * N;
+    unsigned remaining = a.keep, mask = 0u;
+    for (int c = tid; c < 2 * kHistBins; c += T) sm[L.hist + c] = 0u;
+    __syncthreads();
+    for (int e = tid; e < n; e += 8 * T) {
+      unsigned v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = e + u * T < n ? src[e + u * T] : 0u;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (e + u * T < n) {
+          sm[e + u * T] = v[u];
+          atomicAdd(&sm[L.hist + (v[u] >> seq_shift(0))], 1u);
+        }
+    }
+    for (int pass = 0;; ++pass) {
+      // Every part adds up an eighth of the bins over all of them, then every part reads the sums, the highest digits in the first threads.
+      // (Each part reading all eight histograms: 11,500 cycles a pass.)
+      const int nb = (int)seq_mask(pass) + 1, per_part = nb / kSelParts;
+      unsigned* hist = sm + L.hist + (pass & 1) * kHistBins;
+      cluster.sync();
+      if (tid < per_part) {
+        unsigned c = 0u;
+#pragma unroll
+        for (int p = 0; p < kSelParts; ++p) c += cluster.map_shared_rank(hist, p)[part * per_part + tid];
+        slice[tid] = c;
+      }
+      cluster.sync();
+      const int per = nb / T, lo = nb - per * (tid + 1);          // this thread's bins: four, in the last pass two
+      const unsigned* sums = cluster.map_shared_rank(slice, lo / per_part) + lo % per_part;
+      uint4 c;
+      if (per == 4) {
+        c = *reinterpret_cast<const uint4*>(sums);
+      } else {
+        const uint2 two = *reinterpret_cast<const uint2*>(sums);
+        c = make_uint4(two.x, two.y, 0u, 0u);
+      }
+      const unsigned mine = c.x + c.y + c.z + c.w;
+      int tot;
+      const unsigned above = (unsigned)block_excl_scan<T>((int)mine, ws, tot);
+      if (above < remaining && remaining <= above + mine) {
+        const unsigned left = remaining - above;        // the left-th largest of this thread's entries
+        const unsigned a3 = c.w, a2 = a3 + c.z, a1 = a2 + c.y;
+        const int b = left <= a3 ? 3 : left <= a2 ? 2 : left <= a1 ? 1 : 0;
+        pick[0] = (unsigned)(lo + b);
+        pick[1] = left - (b == 3 ? 0u : b == 2 ? a3 : b == 1 ? a2 : a1);
+      }
+      __syncthreads();
+      tau |= pick[0] << seq_shift(pass);
+      mask |= seq_mask(pass) << seq_shift(pass);
+      remaining = pick[1];
+      if (pass == 2) break;
+      // (the first histogram is cleared for its second use behind the barriers that its readers have passed)
+      hist = sm + L.hist + ((pass + 1) & 1) * kHistBins;
+      if (pass == 1) {
+        for (int c_ = tid; c_ < kHistBins; c_ += T) hist[c_] = 0u;
+        __syncthreads();
+      }
+      const int shift = seq_shift(pass + 1);
+      const unsigned dmask = seq_mask(pass + 1);
+#pragma unroll 4
+      for (int e = tid; e < n; e += T) {
+        const unsigned v = sm[e];
+        if ((v & mask) == tau) atomicAdd(&hist[(v >> shift) & dmask], 1u);
+      }
+    }
+    quota = (int)remaining;
+    if (!MAPS && part == 0 && tid == 0) {
+      a.state[bh * 8 + 3] = tau;
+      a.state[bh * 8 + 4] = remaining;
+    }
+    cluster.sync();            // (the histograms have been read: their place is used again)
+  }
+
+  // entries above the threshold (or its band) and at it, by row
+  const unsigned hi = BAND ? band_hi(tau) : tau, lo = BAND ? band_lo(tau) : tau;
+  unsigned* gt_bits = MAPS ? sm + L.bm : a.bits_gt + row0 * words;
+  unsigned* eq_bits = MAPS ? sm + L.eq : a.bits_eq + row0 * words;
+  for (int r = warp; r < rows; r += WARPS) {
+    int gt = 0, eq = 0;
+    constexpr int U = 4;
+    for (int w0 = 0; w0 < words; w0 += U) {
+      unsigned mine_g = 0u, mine_e = 0u;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = (w0 + u) * 32 + lane;
+        const unsigned v = j < N ? sm[r * N + j] : 0u;
+        const bool in = j < N && v >= lo && v <= hi;
+        const unsigned gb = __ballot_sync(0xffffffffu, j < N && v > hi), eb = __ballot_sync(0xffffffffu, in);
+        if (lane == u) { mine_g = gb; mine_e = eb; }
+        gt += __popc(gb);
+        eq += __popc(eb);
+        if constexpr (BAND) settle_list_warp(se, in, (int)row0 + r, j);
+      }
+      if (lane < U && w0 + lane < words) {
+        gt_bits[r * words + w0 + lane] = mine_g;
+        eq_bits[r * words + w0 + lane] = mine_e;
+      }
+    }
+    if (lane == 0) {
+      if constexpr (MAPS) {
+        sm[L.pos + r] = (unsigned)gt;
+        sm[L.take + r] = (unsigned)eq;
+      } else {
+        a.row_gt[row0 + r] = gt;
+        a.row_eq[row0 + r] = eq;
+      }
+    }
+  }
+  if constexpr (MAPS) {
+    // positions of the rows: sums over the rows before, in this part and in the parts before.  Ties go to the lower row: of the
+    // entries at the threshold the first `quota` are kept, so the kept entries before a row are those above it and min(quota, those at it)
+    __syncthreads();
+    int gt = 0, eq = 0, gt_tot, eq_tot;
+    if (tid < rows) {
+      gt = (int)sm[L.pos + tid];
+      eq = (int)sm[L.take + tid];
+    }
+    int gt_before = block_excl_scan<T>(gt, ws, gt_tot), eq_before = block_excl_scan<T>(eq, ws, eq_tot);
+    if (tid == 0) {
+      part_tot[0] = gt_tot;
+      part_tot[1] = eq_tot;
+    }
+    cluster.sync();
+    if (warp == 0) {
+      const int* t = cluster.map_shared_rank(part_tot, lane % kSelParts);
+      const int tg = lane < kSelParts ? t[0] : 0, te = lane < kSelParts ? t[1] : 0;
+      const int bg = __reduce_add_sync(0xffffffffu, lane < part ? tg : 0), be = __reduce_add_sync(0xffffffffu, lane < part ? te : 0);
+      const int ag = __reduce_add_sync(0xffffffffu, tg), ae = __reduce_add_sync(0xffffffffu, te);
+      if (lane == 0) {
+        base[0] = bg;
+        base[1] = be;
+        base[2] = ag;
+        base[3] = ae;
+      }
+    }
+    __syncthreads();
+    gt_before += base[0];
+    eq_before += base[1];
+    const long long kept = (long long)base[2] + min(base[3], quota);
+    if (tid < rows) {
+      const int pre = gt_before + min(eq_before, quota);
+      sm[L.pos + tid] = (unsigned)min((long long)pre, a.nnz_cap);
+      sm[L.take + tid] = (unsigned)max(0, min(eq, quota - eq_before));
+    }
+    __syncthreads();
+    // the rows' kept bits (without entries beyond the capacity), a lane per word
+    for (int r = warp; r < rows; r += WARPS) {
+      int pos = (int)sm[L.pos + r], left = (int)sm[L.take + r];
+      for (int w0 = 0; w0 < words; w0 += 32) {
+        const int w = w0 + lane;
+        unsigned sel = w < words ? sm[L.bm + r * words + w] : 0u;
+        unsigned eb = w < words ? sm[L.eq + r * words + w] : 0u;
+        const int ce = __popc(eb), ce_incl = warp_incl_scan(ce, lane);
+        for (int rank = ce_incl - ce; eb != 0u && rank < left; ++rank) {
+          sel |= eb & (0u - eb);
+          eb &= eb - 1u;
+        }
+        const int c = __popc(sel), c_incl = warp_incl_scan(c, lane);
+        for (long long p = (long long)pos + c_incl; p > a.nnz_cap && sel != 0u; --p) sel &= ~(0x80000000u >> __clz(sel));
+        if (w < words) sm[L.bm + r * words + w] = sel;
+        pos += __shfl_sync(0xffffffffu, c_incl, 31);
+        left -= __shfl_sync(0xffffffffu, ce_incl, 31);
+      }
+    }
+    __syncthreads();
+    // the part's bits by column, 32 x 32 at a time, and their counts
+    for (int t = warp; t < L.groups * words; t += WARPS) {
+      const int rg = t / words, w = t - rg * words, r = rg * 32 + lane;
+      const unsigned v = r < rows ? sm[L.bm + r * words + w] : 0u;
+      unsigned mine = 0u;
+#pragma unroll
+      for (int bit = 0; bit < 32; ++bit) {
+        const unsigned col_word = __ballot_sync(0xffffffffu, (v >> bit) & 1u);
+        if (lane == bit) mine = col_word;
+      }
+      if (w * 32 + lane < N) sm[L.bt + rg * N + w * 32 + lane] = mine;
+    }
+    __syncthreads();
+    for (int j = tid; j < N; j += T) {
+      int c = 0;
+      for (int rg = 0; rg < L.groups; ++rg) c += __popc(sm[L.bt + rg * N + j]);
+      sm[L.cnt + j] = (unsigned)c;
+    }
+    cluster.sync();
+    // where this part's entries of a column begin: behind the columns before, the rows of the parts before first
+    int carry = 0;
+    for (int j0 = 0; j0 < N; j0 += T) {
+      const int j = j0 + tid;
+      int c = 0, before = 0, tot;
+      if (j < N) {
+#pragma unroll
+        for (int p = 0; p < kSelParts; ++p) {
+          const int cp = (int)cluster.map_shared_rank(sm + L.cnt, p)[j];
+          if (p < part) before += cp;
+          c += cp;
+        }
+      }
+      const int pre = carry + block_excl_scan<T>(c, ws, tot);
+      carry += tot;
+      if (j < N) {
+        sm[L.col + j] = (unsigned)(pre + before);
+      }
+    }
+    // (no part ends while another reads its counts.  Nothing is written to global memory before this last barrier, whose release would
+    // wait for it.)
+    cluster.sync();
+    // maps: the rows' lists with a lane per word, the columns' with a lane per row
+    const unsigned lt = (1u << lane) - 1u;
+    int* out = a.col_idx + (size_t)bh * a.nnz_cap;
+    for (int r = warp; r < rows; r += WARPS) {
+      int pos = (int)sm[L.pos + r];
+      if (lane == 0) a.row_ptr[(size_t)bh * (N + 1) + r0 + r] = pos;
+      for (int w0 = 0; w0 < words; w0 += 32) {
+        unsigned sel = w0 + lane < words ? sm[L.bm + r * words + w0 + lane] : 0u;
+        const int c = __popc(sel), c_incl = warp_incl_scan(c, lane);
+        for (int p = pos + c_incl - c; sel != 0u; sel &= sel - 1u, ++p) out[p] = (w0 + lane) * 32 + (__ffs(sel) - 1);
+        pos += __shfl_sync(0xffffffffu, c_incl, 31);
+      }
+    }
+    int* lists = a.row_idx + (size_t)bh * a.nnz_cap;
+#pragma unroll 4
+    for (int j = warp; j < N; j += WARPS) {
+      int p = (int)sm[L.col + j];
+      if (part == 0 && lane == 0) a.col_ptr[(size_t)bh * (N + 1) + j] = (int)min((long long)p, a.nnz_cap);
+      for (int rg = 0; rg < L.groups; ++rg) {
+        const unsigned b = sm[L.bt + rg * N + j];
+        const int at = p + __popc(b & lt);
+        if (((b >> lane) & 1u) && at < a.nnz_cap) lists[at] = r0 + rg * 32 + lane;
+        p += __popc(b);
+      }
+    }
+    if (part == 0 && tid == 0) {
+      a.col_ptr[(size_t)bh * (N + 1) + N] = (int)min((long long)carry, a.nnz_cap);
+      a.row_ptr[(size_t)bh * (N + 1) + N] = (int)min(kept, a.nnz_cap);
+      if (kept > a.nnz_cap) atomicExch(&a.status->status, VSA2_ERR_MAP_OVERFLOW);
+    }
+  }
+}
+
 template <int MODE>
 static void launch_row_topk(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
   const int BH = g.batch * g.Hq, N = g.N;
@@ -795,14 +1104,32 @@ static void launch_row_topk(const Geo& g, const float* pr, const int* budgets, c
 #undef VSA2_ROW_TOPK
 }
 
+// whether the selection of a head runs in a cluster
+static bool sel_head_runs(const Geo& g) {
+  return g.mode == VSA2_PER_SEQUENCE && g.N > kSelOneBlockN && g.N <= kSelHeadN;
+}
+template <bool BAND, bool MAPS>
+static cudaError_t launch_sel_head(const Geo& g, const float* pr, const SelectScratch& s, int* row_ptr, int* col_idx, int* col_ptr, int* row_idx,
+                                   StatusBlock* status, const Settle& se, cudaStream_t st) {
+  static KernelAttr attr;
+  const size_t smem = (size_t)SelHeadSmem(g.N, s.words).total * 4;
+  cudaError_t e;
+  if ((e = prepare_kernel((const void*)sel_head_kernel<BAND, MAPS>, attr, smem))) return e;
+  const SelHead a{pr, g.N, s.words, (unsigned)((long long)g.N * g.K), s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq,
+                  row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap, status};
+  return launch_kernel(sel_head_kernel<BAND, MAPS>, kSelParts * g.batch * g.Hq, kSelHeadThreads, smem, st, a, se);
+}
+
 // thresholds, counts and (per sequence) bitmaps of all heads; `se.redo`: null, or the flag without which nothing happens
 template <bool BAND>
-static void launch_thresholds(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
+static cudaError_t launch_thresholds(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
   const int BH = g.batch * g.Hq, N = g.N;
   if (g.mode == VSA2_PER_SEQUENCE) {
     const long long n_elems = (long long)N * N;
     const unsigned keep = (unsigned)((long long)N * g.K);
     const int* redo = BAND ? nullptr : se.redo;
+    if ((BAND || redo != nullptr) && sel_head_runs(g))
+      return launch_sel_head<BAND, false>(g, pr, s, nullptr, nullptr, nullptr, nullptr, nullptr, se, st);
     int init_n = BH * 3 * kHistBins;
     launch_kernel(sel_init_kernel, (init_n + 255) / 256, 256, 0, st, s.state, s.hist, BH, keep, redo);
     int chunks = (int)((n_elems + 256 * 16 - 1) / (256 * 16));
@@ -816,11 +1143,11 @@ static void launch_thresholds(const Geo& g, const float* pr, const int* budgets,
   } else {
     launch_row_topk<BAND ? kBand : kAllRows>(g, pr, budgets, s, se, st);
   }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_select_band(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se, cudaStream_t st) {
-  launch_thresholds<true>(g, pr, budgets, s, se, st);
-  return cudaGetLastError();
+  return launch_thresholds<true>(g, pr, budgets, s, se, st);
 }
 
 cudaError_t launch_select_settle(const Geo& g, const float* pr, const int* budgets, const SelectScratch& s, const Settle& se,
@@ -838,7 +1165,10 @@ cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, con
   const int BH = g.batch * g.Hq, N = g.N;
   Settle se{};
   se.redo = const_cast<int*>(redo);
-  launch_thresholds<false>(g, pr, budgets, s, se, st);
+  if (redo == nullptr && sel_head_runs(g))
+    return launch_sel_head<false, true>(g, pr, s, row_ptr, col_idx, col_ptr, row_idx, status, se, st);
+  cudaError_t e;
+  if ((e = launch_thresholds<false>(g, pr, budgets, s, se, st)) != cudaSuccess) return e;
   if (N <= kSelOneBlockN) {
     launch_kernel(sel_maps_kernel, BH, 1024, 0, st, pr, N, s.words, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
                                          s.row_eq_take, s.row_cnt, s.bitmap, s.bitmap_t, row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap,
