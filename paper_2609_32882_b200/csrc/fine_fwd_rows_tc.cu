@@ -2,18 +2,20 @@
 //
 // Formulation.  A query block has B = 64 tokens.  Both products keep the 64 queries in the rows of the accumulator (M = 64)
 // and stack two selected KV blocks per tile:
-//     S [64 q, 128 kv] = Q [64, D] * K_pair^T            (A = Q from shared memory,  B = K_pair, N = 128 keys)
+//     S [64 q, 128 kv] = Q [64, D] * K_pair^T            (A = Q from TENSOR MEMORY,  B = K_pair, N = 128 keys)
 //     O [64 q, D]     += P [64, 128 kv] * V_pair         (A = P from TENSOR MEMORY,  B = V_pair, N = D)
-// M = 64 runs the tensor pipe at half rate, but every K / V tile is fetched from shared memory exactly once per tile and P
-// never touches shared memory: per tile 64 KB of TMA writes + 64 KB of B fetches + 16 KB of Q, against 176 KB for the
-// transposed M = 128, N = 64 products, which were bound by that traffic.  K and V tiles arrive by 5-D TMA straight from the
+// M = 64 runs the tensor pipe at half rate (64 cycles per step, 1024 per tile), but every K / V tile is fetched from shared memory
+// exactly once per tile and neither P nor Q ever is: per tile 64 KB of TMA writes + 64 KB of B fetches, as many cycles of the
+// shared-memory pipe as of the tensor pipe (Q from shared memory: 16 KB and 128 cycles more), against 176 KB for the
+// transposed M = 128, N = 64 products.  K and V tiles arrive by 5-D TMA straight from the
 // raster tensors (one box = one cube, zero-filled outside the grid); the V tile that TMA wrote row-per-key is read as an
 // MN-major B operand, so nothing is transposed in memory.
 //
-// Tensor memory (512 columns): two S buffers (2 x 128 fp32 columns), two P buffers (2 x 64 columns of bf16 pairs) and the O
-// accumulator (D columns).  An M = 64 accumulator keeps row m in lane (m % 16) + 32 (m / 16); the softmax warps read S with
-// 16-lane loads that give a thread two query rows x 32 key columns, and the bf16 pairs it forms from neighbouring columns
-// are exactly the words its 16-lane store writes into the P operand.
+// Tensor memory (512 columns).  An M = 64 accumulator keeps row m in lane (m % 16) + 32 (m / 16), half of each quadrant's lanes, and an A
+// operand lies in the lanes of its accumulator.  The upper halves hold two S buffers (2 x 128 fp32 columns) and Q of two blocks
+// (2 x 64 columns of bf16 pairs), the lower ones two P buffers (2 x 64) and the O accumulators of two blocks (2 x D).  The
+// softmax warps read S with 16-lane loads that give a thread two query rows x 32 key columns, and the bf16 pairs it forms from
+// neighbouring columns are exactly the words its 16-lane store writes into the P operand.
 //
 // Softmax.  Four threads share a query row.  Each row keeps a fixed reference M (the exact row maximum of the block's first
 // tile, log2 units): P = 2^(s*scale*log2e - M); any reference gives the same softmax unless something overflows, the row
@@ -23,14 +25,25 @@
 // weights sum to one and the rounding of a dominant P cancels instead of scaling the whole output row (that scaling,
 // 2^-9 relative, reached the backward through delta = rowsum(dO * O) and was its largest error on sharply peaked rows).
 //
-// Roles (512 threads): warps 0..3 = TMA producers (K / V ring x first / second block of a pair; warp 0 also brings the Q
-// tile and schedules the CTA's work items), warp 4 = issuer of S, warp 5 = issuer of O, warps 8..15 = two softmax +
-// epilogue warpgroups that alternate tiles.  Persistent CTAs draw query blocks from a global counter.  Every wait is bounded.
+// Roles (640 threads): warps 0..3 = TMA producers (K / V ring x first / second block of a pair; warp 0 also brings the Q
+// tile and schedules the CTA's work items), warp 4 = issuer of S, warp 5 = issuer of O, warp 6 = per-item tables, warps 8..15 = two
+// softmax warpgroups that alternate tiles, warps 16..19 = Q of the next block into tensor memory, then the epilogue of the present one
+// while the softmax warps are at the next.  Persistent CTAs draw query blocks from a global counter.  Every wait is bounded.
+//
+// What the softmax warps execute is kept short, once and without alternatives: its tile loop is some 8 KB of straight code, and what else
+// ran in between (the epilogue, a masked form of the loop) made them wait for the instruction cache, up to 2500 cycles a tile.  So:
+// epilogue elsewhere, masking ahead of the one loop, the first tile's maximum inside it, two values per instruction.  Forward calls, us, before (epilogue
+// in the softmax warps, selects in a masked copy of the loop, Q from shared memory) -> after: 9 x 30 x 45 tokens, 24 heads, top-16 514 -> 436;
+// 13 x 27 x 47, 16 heads of 64 channels, top-24 484 -> 362; 480p, 12 heads on 3, top-78 1688 -> 1573; 720p, 5 heads with text 1899 -> 1772;
+// 10 heads, top-128 4958 -> 4654.  (Epilogue and Q alone: 573, 481, 1602, 1877, 4789: more code beside the loop.)
 #include "tc_attn.cuh"
 
 namespace vsa2 {
 
-constexpr int kFrThreads = 512;
+constexpr int kFrThreads = 640;
+// registers a thread: the launch allocates 96 (640 threads); the softmax warps take what the service warps leave
+constexpr int kFrServiceRegs = 48, kFrSoftmaxRegs = 144, kFrRegs = 256 * kFrServiceRegs + 256 * kFrSoftmaxRegs + 128 * 96;
+static_assert(kFrRegs == kFrThreads * 96, "the shares have to fit the launch");
 constexpr int kFrKSlots = 3;
 constexpr int kFrVSlots = 3;
 constexpr int kFrMaxCubes = 8192;      // edge-flag table in shared memory: one byte per cube
@@ -40,16 +53,20 @@ struct FwdRows {
   static constexpr int DH = D / 64;
   static constexpr uint32_t SLOT = 2 * DH * kSlab;     // a K pair or a V pair, [half][A | B]
   static constexpr uint32_t QBYTES = DH * kSlab;
-  static constexpr int NQ = 1;                                            // Q tiles (by item parity if 2)
   static constexpr uint32_t OFF_Q = (kFrKSlots + kFrVSlots) * SLOT;
-  static constexpr uint32_t OFF_MISC = OFF_Q + NQ * QBYTES;
-  static constexpr uint32_t MISC_BYTES = 4096;
-  static constexpr uint32_t TM_S = 0, TM_P = 256, TM_O = 384;
+  static constexpr uint32_t OFF_MISC = OFF_Q + QBYTES;
+  static constexpr uint32_t MISC_BYTES = 10240;
+  // tensor memory: the upper sixteen lanes of each quadrant hold S and its A operand Q, the lower ones O and its A operand P
+  static constexpr uint32_t TM_UP = 16u << 16, TM_S = TM_UP, TM_Q = TM_UP + 256, TM_P = 0, TM_O = 128;
   static size_t smem_bytes(int n_cubes) { return OFF_MISC + MISC_BYTES + ((size_t)n_cubes + 15) / 16 * 16 + 1024; }
 };
 
+constexpr int kFrTail = 16, kFrNone = 17;
 struct FwdRowsMisc {
-  uint64_t q_full[2], q_empty[2], o_full, o_empty;
+  uint64_t q_full, q_empty;            // the Q tile in shared memory
+  uint64_t qt_full[2], qt_empty[2];    // Q in tensor memory, and the O accumulators: by parity of the CTA's blocks that keep anything
+  uint64_t o_full[2], o_empty[2];
+  uint64_t sums_full[2];               // row sums of the item with that parity
   uint64_t tab_full[2], tab_free[2];   // per-item tables (tok, gate, oc) of the item with that parity
   uint64_t k_full[kFrKSlots], k_empty[kFrKSlots];
   uint64_t v_full[kFrVSlots], v_empty[kFrVSlots];
@@ -59,17 +76,19 @@ struct FwdRowsMisc {
   uint64_t all_sync;               // group barrier of the 256 softmax threads
   uint32_t tmem_base;
   int abort_flag;
-  int rescue_flag;
-  unsigned short vmask[17][4];     // [table row of the block][lane % 4]: which of a thread's 16 key columns are valid tokens
-  alignas(16) float m_ref[64];     // per query row: reference exponent (log2 units)
-  float red[2][2][64];             // [warpgroup][exact sum | sum of the bf16 roundings][query row]
+  uint32_t rescued;                // 1 + number of the last item that was handed to the exact kernel
+  // [validity row of a block][lane % 4]: 0 for key columns 8n + 2c + e (n = 0..7, e = 0, 1) that hold tokens, -infinity for the others; added
+  // to the exponents.  Row 0 is not looked at; kFrTail: the last text block if it is cut, kFrNone: no token (the block that an odd list repeats)
+  alignas(16) float2 bias[18][4][8];
+  float m_ref[2][64];              // by item parity, per query row: reference exponent (log2 units)
+  float red[2][2][2][64];          // [item parity][warpgroup][exact sum | sum of the bf16 roundings][query row]
   alignas(16) float oc[2][128];    // coarse output row of the query cube, by item parity
   int tok[2][64];                  // raster token of each query row (-1 = padding), by item parity
   float gate[2][64];
   int list_k[2], list_beg[2];      // length and start of the item's list of KV blocks
   int list_head[2][4];             // its first four entries (tiles 0 and 1)
 };
-static_assert(sizeof(FwdRowsMisc) <= 4096, "misc region too small");
+static_assert(sizeof(FwdRowsMisc) <= 10240, "misc region too small");
 
 struct FwdRowsArgs {
   int* item_counter;    // global, zero before the launch
@@ -117,35 +136,31 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
   const int total_items = g.batch * g.Hq * g.N;
   const float c2 = g.scale * 1.4426950408889634f;
 
-  // per block: the row of the validity table below -- the edge flags of a video cube (0 = nothing cut), 0 for a full text
-  // block, 16 for the ragged last text block
+  // per block: its row in the validity table -- the edge flags of a video cube (0 = nothing cut), 0 for a full text block
   for (int n = tid; n < g.N; n += blockDim.x)
-    edge[n] = (unsigned char)(n < g.Nvid ? cube_edge_flags(g, n) : (block_count(g, n) == kBlockTokens ? 0 : 16));
-  if (tid < 68) {
-    // validity of key columns 8n + 2c + e (n = 0..7, e = 0, 1) of a 64-token block, for lane % 4 == c: rows 0..15 by the
-    // edge flags of a video cube, row 16 for the last text block when it holds fewer than 64 tokens
-    const unsigned f = tid >> 2, c = tid & 3;
-    const int text_tail = g.Lt % kBlockTokens;
-    unsigned m = 0;
-    for (int n = 0; n < 8; ++n)
-      for (int e = 0; e < 2; ++e) {
-        const int pos = 8 * n + 2 * (int)c + e;
-        CubePos cp;
-        cp.init(g, pos);
-        if (f < 16 ? cp.valid(f, g) : pos < text_tail) m |= 1u << (2 * n + e);
-      }
-    misc->vmask[f][c] = (unsigned short)m;
+    edge[n] = (unsigned char)(n < g.Nvid ? cube_edge_flags(g, n) : (block_count(g, n) == kBlockTokens ? 0 : kFrTail));
+  for (int e = tid; e < 18 * 64; e += blockDim.x) {
+    const unsigned f = e >> 6;
+    const int pos = e & 63;
+    CubePos cp;
+    cp.init(g, pos);
+    const bool token = f < kFrTail ? cp.valid(f, g) : f == kFrTail && pos < g.Lt % kBlockTokens;
+    reinterpret_cast<float*>(&misc->bias[f][(pos >> 1) & 3][pos >> 3])[pos & 1] = token ? 0.f : -INFINITY;
   }
   if (tid == 0) {
     misc->abort_flag = 0;
+    misc->rescued = 0;
+    tc::mbar_init(&misc->q_full, 1);
+    tc::mbar_init(&misc->q_empty, 128);
     for (int s = 0; s < 2; ++s) {
-      tc::mbar_init(&misc->q_full[s], 1);
-      tc::mbar_init(&misc->q_empty[s], 1);
+      tc::mbar_init(&misc->qt_full[s], 128);
+      tc::mbar_init(&misc->qt_empty[s], 1);
+      tc::mbar_init(&misc->o_full[s], 1);
+      tc::mbar_init(&misc->o_empty[s], 128);
+      tc::mbar_init(&misc->sums_full[s], 256);
       tc::mbar_init(&misc->tab_full[s], 32);
-      tc::mbar_init(&misc->tab_free[s], 256);
+      tc::mbar_init(&misc->tab_free[s], 256 + 128);
     }
-    tc::mbar_init(&misc->o_full, 1);
-    tc::mbar_init(&misc->o_empty, 256);
     for (int s = 0; s < kFrKSlots; ++s) {
       tc::mbar_init(&misc->k_full[s], 2);    // the two producer warps of the ring
       tc::mbar_init(&misc->k_empty[s], 1);
@@ -161,7 +176,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       tc::mbar_init(&misc->p_free[s], 1);
     }
     tc::mbar_init(&misc->all_sync, 256);
-    item_queue_init(&misc->items, 4 + 2 + 1 + 256); // lane 0 of the producers, of the two issuers and of the table loader, the softmax threads
+    item_queue_init(&misc->items, 4 + 2 + 1 + 256 + 4); // lane 0 of the producers, of the issuers, of the table loader and of the epilogue warps; the softmax threads
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_k);
@@ -183,7 +198,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
   grid_enter_items(g.batch * g.Hq * g.N);
 
   if (warp < 8) {
-    tc::reg_dec<56>();
+    tc::reg_dec<kFrServiceRegs>();
     if (warp < 4) {
       // ---------------------------------------------------------------- TMA producers
       // One warp sustains only ~24 B/clk of 5-D boxes (the copy instructions of a warp issue one after the other), so every
@@ -220,15 +235,13 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
           int c1, c2, c3;
           block_box(g, i, c1, c2, c3);
           int ok = 1;
-          const uint32_t qb = n_items % C::NQ;
           if (lane == 0) {
-            ok = tc::mbar_wait(&misc->q_empty[qb], ((n_items / C::NQ) & 1) ^ 1, &misc->abort_flag);
-            if (ok) tc::mbar_expect_tx(&misc->q_full[qb], C::QBYTES);
+            ok = tc::mbar_wait(&misc->q_empty, (n_items & 1) ^ 1, &misc->abort_flag);
+            if (ok) tc::mbar_expect_tx(&misc->q_full, C::QBYTES);
           }
           if (!__shfl_sync(0xffffffffu, ok, 0)) goto done;
           if (lane < C::DH)
-            tc::tma_load_5d(q_tile + qb * C::QBYTES + lane * kSlab, block_is_text(g, i) ? &tm_qt : &tm_q, &misc->q_full[qb],
-                            lane * 64, c1, c2, c3, bhq);
+            tc::tma_load_5d(q_tile + lane * kSlab, block_is_text(g, i) ? &tm_qt : &tm_q, &misc->q_full, lane * 64, c1, c2, c3, bhq);
         }
         ++n_items;
         const int nt = (k + 1) >> 1;
@@ -267,9 +280,8 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const int k = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] - a.row_ptr[(size_t)bhq * (g.N + 1) + i];
         if (k == 0) continue;
         const int nt = (k + 1) >> 1;
-        const uint32_t qb = n_items % C::NQ;
-        const uint64_t dq = tc::smem_desc_sw128(tc::smem_u32(q_tile) + qb * C::QBYTES, 16, 1024);
-        VSA2_WAIT(&misc->q_full[qb], (n_items / C::NQ) & 1);
+        const uint32_t qb = n_items & 1, tm_q_op = tmem_base + C::TM_Q + qb * 64;
+        VSA2_WAIT(&misc->qt_full[qb], (n_items >> 1) & 1);
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t slot = tg % kFrKSlots, buf = tg & 1;
           VSA2_WAIT(&misc->k_full[slot], (tg / kFrKSlots) & 1);
@@ -279,13 +291,12 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             const uint64_t dk = tc::smem_desc_sw128(slot0 + slot * C::SLOT, 16, 1024);
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
-              const uint64_t oa = (uint64_t)(((ks / 4) * kSlab + (ks % 4) * 32) >> 4);
               const uint64_t ob = (uint64_t)(((ks / 4) * 2 * kSlab + (ks % 4) * 32) >> 4);
-              tc::mma_ss(tmem_base + C::TM_S + buf * 128, dq + oa, dk + ob, idesc, ks > 0);
+              tc::mma_ts(tmem_base + C::TM_S + buf * 128, tm_q_op + ks * 8, dk + ob, idesc, ks > 0);
             }
             tc::mma_commit(&misc->s_full[buf]);
             tc::mma_commit(&misc->k_empty[slot]);
-            if (t == nt - 1) tc::mma_commit(&misc->q_empty[qb]);   // the Q tile may be replaced once the last S of the block is done
+            if (t == nt - 1) tc::mma_commit(&misc->qt_empty[qb]);  // Q may be replaced once the last S of the block is done
           }
           __syncwarp();
         }
@@ -308,7 +319,8 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const int k = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] - a.row_ptr[(size_t)bhq * (g.N + 1) + i];
         if (k == 0) continue;
         const int nt = (k + 1) >> 1;
-        VSA2_WAIT(&misc->o_empty, (n_items & 1) ^ 1);      // the previous query block's accumulator was read out
+        const uint32_t ob_ = n_items & 1, acc = tmem_base + C::TM_O + ob_ * 128;
+        VSA2_WAIT(&misc->o_empty[ob_], ((n_items >> 1) & 1) ^ 1);      // the accumulator of the block before the last was read out
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t slot = tg % kFrVSlots, buf = tg & 1;
           VSA2_WAIT(&misc->v_full[slot], (tg / kFrVSlots) & 1);
@@ -319,11 +331,11 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
               const uint64_t ob = (uint64_t)(((ks / 4) * kSlab + (ks % 4) * 2048) >> 4);
-              tc::mma_ts(tmem_base + C::TM_O, tmem_base + C::TM_P + buf * 64 + ks * 8, dv + ob, idesc, t > 0 || ks > 0);
+              tc::mma_ts(acc, tmem_base + C::TM_P + buf * 64 + ks * 8, dv + ob, idesc, t > 0 || ks > 0);
             }
             tc::mma_commit(&misc->v_empty[slot]);
             tc::mma_commit(&misc->p_free[buf]);
-            if (t == nt - 1) tc::mma_commit(&misc->o_full);
+            if (t == nt - 1) tc::mma_commit(&misc->o_full[ob_]);
           }
           __syncwarp();
         }
@@ -371,17 +383,15 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         tc::mbar_arrive(&misc->tab_full[tb]);
       }
     }
-  } else {
-    // ------------------------------------------------------------------ softmax + epilogue (2 x 128 threads)
-    tc::reg_inc<200>();
+  } else if (warp < 16) {
+    // ------------------------------------------------------------------ softmax (2 x 128 threads)
+    tc::reg_inc<kFrSoftmaxRegs>();
     const int wg = (warp >> 2) - 2;              // 0 or 1: the tiles with (global tile index & 1) == wg
     const int quad = warp & 3;
     const int cq = lane & 3;
     const int row_a = quad * 16 + (lane >> 2), row_b = row_a + 8;     // the two query rows of this thread
-    const int sm_tid = tid & 127;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    constexpr int COLS = D / 2;                  // output columns per warpgroup in the epilogue
-    uint32_t tg = 0, n_items = 0, all_phase = 0;
+    uint32_t tg = 0, all_phase = 0;
     for (uint32_t n_all = 0;; ++n_all) {
       VSA2_NEXT_ITEM(item, n_all);
       int i, bhq;
@@ -392,164 +402,198 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       const int* cols = a.col_idx + (size_t)bhq * g.nnz_cap + misc->list_beg[tb];
       const int* head = misc->list_head[tb];
       (void)i;
-      if (wg == 0 && sm_tid == 0) misc->rescue_flag = 0;
-
       const int nt = (k + 1) >> 1;
       const uint32_t tg0 = tg;
-      uint32_t sv[64];
-      bool have_first = false;
-      if (k > 0 && (tg & 1) == (uint32_t)wg) {
-        // this warpgroup owns tile 0: reference exponent of every query row = exact row maximum of that tile
-        const uint32_t buf = tg & 1;
-        VSA2_WAIT(&misc->s_full[buf], (tg >> 1) & 1);
+      // Tiles with (global tile index & 1) == wg.  The owner of tile 0 takes the exact row maximum of that tile as the reference exponent of
+      // every query row; both warpgroups pick it up in front of their first tile's weights.
+      float2 l_a = make_float2(0.f, 0.f), l_b = l_a;       // exact sums of the two rows, even and odd columns apart
+      float r_a = 0.f, r_b = 0.f;                          // and sums of the bf16 roundings
+      float m_a = 0.f, m_b = 0.f;
+      const int t_first = (tg0 & 1) == (uint32_t)wg ? 0 : 1;
+      // KV blocks of this warpgroup's tiles: the first from the item's table, the others fetched one own tile ahead
+      int ja = head[2 * t_first < k ? 2 * t_first : 0], jb = head[2 * t_first + 1 < k ? 2 * t_first + 1 : 0];
+      if (t_first >= nt) VSA2_GROUP_SYNC(&misc->all_sync, all_phase);      // (no tile of its own)
+      for (int t = t_first; t < nt; t += 2) {
+        const uint32_t tgt = tg0 + t, buf = tgt & 1;
+        const int fa = edge[ja], fb = 2 * t + 1 >= k ? kFrNone : edge[jb];
+        if (t + 2 < nt) {
+          ja = cols[2 * t + 4];
+          jb = cols[2 * t + 5 < k ? 2 * t + 5 : 2 * t + 4];
+        }
+        uint32_t sv[64];
+        VSA2_WAIT(&misc->s_full[buf], (tgt >> 1) & 1);
         tc::tc_fence_after();
         tc::tmem_ld_16x256b_x16(lane_addr + C::TM_S + buf * 128, sv);
         tc::tmem_ld_wait();
         tc::tc_fence_before();
         tc::mbar_arrive(&misc->s_free[buf]);
-        have_first = true;
-        const unsigned ma = misc->vmask[edge[head[0]]][cq];
-        const unsigned mb = k > 1 ? misc->vmask[edge[head[1]]][cq] : 0u;
-        float mx_a = -INFINITY, mx_b = -INFINITY;
+        if ((fa | fb) != 0) {
+          // scores of key columns without a token become -infinity, so their weights 0 (a test that is the same for all lanes; by the
+          // tokens of a lane's own columns, warps ran a masked and an unmasked form one after the other)
+          const float2 *ba = misc->bias[fa][cq], *bb = misc->bias[fb][cq];
+#pragma unroll
+          for (int n = 0; n < 16; ++n) {
+            const float2 bn = n < 8 ? ba[n] : bb[n - 8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float2 x = __fadd2_rn(make_float2(__uint_as_float(sv[4 * n + 2 * h]), __uint_as_float(sv[4 * n + 2 * h + 1])), bn);
+              sv[4 * n + 2 * h] = __float_as_uint(x.x);
+              sv[4 * n + 2 * h + 1] = __float_as_uint(x.y);
+            }
+          }
+        }
+        if (t == t_first) {
+          if (t == 0) {
+            float mx_a = -INFINITY, mx_b = -INFINITY;
+#pragma unroll
+            for (int n = 0; n < 16; ++n) {
+              mx_a = fmaxf(mx_a, fmaxf(__uint_as_float(sv[4 * n]), __uint_as_float(sv[4 * n + 1])));
+              mx_b = fmaxf(mx_b, fmaxf(__uint_as_float(sv[4 * n + 2]), __uint_as_float(sv[4 * n + 3])));
+            }
+            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 1));
+            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 1));
+            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 2));
+            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 2));
+            if (cq == 0) {
+              misc->m_ref[tb][row_a] = (mx_a > -INFINITY) ? mx_a * c2 : 0.f;
+              misc->m_ref[tb][row_b] = (mx_b > -INFINITY) ? mx_b * c2 : 0.f;
+            }
+          }
+          VSA2_GROUP_SYNC(&misc->all_sync, all_phase);
+          m_a = misc->m_ref[tb][row_a];
+          m_b = misc->m_ref[tb][row_b];
+        }
+        uint32_t pk[32];
 #pragma unroll
         for (int n = 0; n < 16; ++n) {
-          const unsigned m = (n < 8 ? ma : mb) >> (2 * (n & 7));
-          if (m & 1u) { mx_a = fmaxf(mx_a, __uint_as_float(sv[4 * n])); mx_b = fmaxf(mx_b, __uint_as_float(sv[4 * n + 2])); }
-          if (m & 2u) { mx_a = fmaxf(mx_a, __uint_as_float(sv[4 * n + 1])); mx_b = fmaxf(mx_b, __uint_as_float(sv[4 * n + 3])); }
+          const float2 xa = fma_bits2(sv[4 * n], sv[4 * n + 1], c2, -m_a, -m_a), xb = fma_bits2(sv[4 * n + 2], sv[4 * n + 3], c2, -m_b, -m_b);
+          const float p0 = ex2_approx(xa.x), p1 = ex2_approx(xa.y), p2 = ex2_approx(xb.x), p3 = ex2_approx(xb.y);
+          l_a = __fadd2_rn(l_a, make_float2(p0, p1));
+          l_b = __fadd2_rn(l_b, make_float2(p2, p3));
+          const uint32_t wa = pack_bf16x2(p0, p1), wb = pack_bf16x2(p2, p3);
+          r_a += __uint_as_float(wa << 16) + __uint_as_float(wa & 0xffff0000u);
+          r_b += __uint_as_float(wb << 16) + __uint_as_float(wb & 0xffff0000u);
+          pk[2 * n] = wa;
+          pk[2 * n + 1] = wb;
         }
-        mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 1));
-        mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 1));
-        mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 2));
-        mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 2));
-        if (cq == 0) {
-          misc->m_ref[row_a] = (mx_a > -INFINITY) ? mx_a * c2 : 0.f;
-          misc->m_ref[row_b] = (mx_b > -INFINITY) ? mx_b * c2 : 0.f;
-        }
+        VSA2_WAIT(&misc->p_free[buf], ((tgt >> 1) & 1) ^ 1);
+        tc::tmem_st_16x128b_x16(lane_addr + C::TM_P + buf * 64, pk);
+        tc::tmem_st_wait();
+        tc::tc_fence_before();
+        tc::mbar_arrive(&misc->p_ready[buf]);
       }
-      VSA2_GROUP_SYNC(&misc->all_sync, all_phase);       // reference exponents visible to both warpgroups
-
-      float l_a = 0.f, l_b = 0.f, r_a = 0.f, r_b = 0.f;   // exact sums and sums of the bf16 roundings of the two rows
-      float m_a = 0.f, m_b = 0.f;
-      if (k > 0) {
-        m_a = misc->m_ref[row_a];
-        m_b = misc->m_ref[row_b];
-        const int t_first = ((tg0 & 1) == (uint32_t)wg) ? 0 : 1;
-        // KV blocks of this warpgroup's tiles: the first from the item's table, the others fetched one own tile ahead
-        int ja = head[2 * t_first < k ? 2 * t_first : 0], jb = head[2 * t_first + 1 < k ? 2 * t_first + 1 : 0];
-        for (int t = t_first; t < nt; t += 2) {
-          const uint32_t tgt = tg0 + t, buf = tgt & 1;
-          const bool dup = 2 * t + 1 >= k;
-          const unsigned ma = misc->vmask[edge[ja]][cq];
-          const unsigned mb = dup ? 0u : misc->vmask[edge[jb]][cq];
-          if (t + 2 < nt) {
-            ja = cols[2 * t + 4];
-            jb = cols[2 * t + 5 < k ? 2 * t + 5 : 2 * t + 4];
-          }
-          if (!(have_first && t == 0)) {
-            VSA2_WAIT(&misc->s_full[buf], (tgt >> 1) & 1);
-            tc::tc_fence_after();
-            tc::tmem_ld_16x256b_x16(lane_addr + C::TM_S + buf * 128, sv);
-            tc::tmem_ld_wait();
-            tc::tc_fence_before();
-            tc::mbar_arrive(&misc->s_free[buf]);
-          }
-          uint32_t pk[32];
-          if ((ma & mb) == 0xffffu) {
+      tg += nt;
+      // row sums: over the four threads of a row here, over the two warpgroups through shared memory
+      float la = l_a.x + l_a.y, lb = l_b.x + l_b.y;
 #pragma unroll
-            for (int n = 0; n < 16; ++n) {
-              const float p0 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 0]), c2, -m_a));
-              const float p1 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 1]), c2, -m_a));
-              const float p2 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 2]), c2, -m_b));
-              const float p3 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 3]), c2, -m_b));
-              l_a += p0 + p1;
-              l_b += p2 + p3;
-              const uint32_t wa = pack_bf16x2(p0, p1), wb = pack_bf16x2(p2, p3);
-              r_a += __uint_as_float(wa << 16) + __uint_as_float(wa & 0xffff0000u);
-              r_b += __uint_as_float(wb << 16) + __uint_as_float(wb & 0xffff0000u);
-              pk[2 * n] = wa;
-              pk[2 * n + 1] = wb;
-            }
-          } else {
-#pragma unroll
-            for (int n = 0; n < 16; ++n) {
-              const unsigned m = (n < 8 ? ma : mb) >> (2 * (n & 7));
-              float p0 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 0]), c2, -m_a));
-              float p1 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 1]), c2, -m_a));
-              float p2 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 2]), c2, -m_b));
-              float p3 = ex2_approx(fmaf(__uint_as_float(sv[4 * n + 3]), c2, -m_b));
-              if (!(m & 1u)) { p0 = 0.f; p2 = 0.f; }
-              if (!(m & 2u)) { p1 = 0.f; p3 = 0.f; }
-              l_a += p0 + p1;
-              l_b += p2 + p3;
-              const uint32_t wa = pack_bf16x2(p0, p1), wb = pack_bf16x2(p2, p3);
-              r_a += __uint_as_float(wa << 16) + __uint_as_float(wa & 0xffff0000u);
-              r_b += __uint_as_float(wb << 16) + __uint_as_float(wb & 0xffff0000u);
-              pk[2 * n] = wa;
-              pk[2 * n + 1] = wb;
-            }
-          }
-          VSA2_WAIT(&misc->p_free[buf], ((tgt >> 1) & 1) ^ 1);
-          tc::tmem_st_16x128b_x16(lane_addr + C::TM_P + buf * 64, pk);
-          tc::tmem_st_wait();
-          tc::tc_fence_before();
-          tc::mbar_arrive(&misc->p_ready[buf]);
-        }
-        tg += nt;
-        // row sums: over the four threads of a row here, over the two warpgroups through shared memory
-        l_a += __shfl_xor_sync(0xffffffffu, l_a, 1);
-        l_b += __shfl_xor_sync(0xffffffffu, l_b, 1);
-        r_a += __shfl_xor_sync(0xffffffffu, r_a, 1);
-        r_b += __shfl_xor_sync(0xffffffffu, r_b, 1);
-        l_a += __shfl_xor_sync(0xffffffffu, l_a, 2);
-        l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
-        r_a += __shfl_xor_sync(0xffffffffu, r_a, 2);
-        r_b += __shfl_xor_sync(0xffffffffu, r_b, 2);
-        if (cq == 0) {
-          misc->red[wg][0][row_a] = l_a;
-          misc->red[wg][0][row_b] = l_b;
-          misc->red[wg][1][row_a] = r_a;
-          misc->red[wg][1][row_b] = r_b;
-        }
+      for (int o = 1; o <= 2; o <<= 1) {
+        la += __shfl_xor_sync(0xffffffffu, la, o);
+        lb += __shfl_xor_sync(0xffffffffu, lb, o);
+        r_a += __shfl_xor_sync(0xffffffffu, r_a, o);
+        r_b += __shfl_xor_sync(0xffffffffu, r_b, o);
       }
-      VSA2_GROUP_SYNC(&misc->all_sync, all_phase);
+      if (cq == 0) {
+        misc->red[tb][wg][0][row_a] = la;
+        misc->red[tb][wg][0][row_b] = lb;
+        misc->red[tb][wg][1][row_a] = r_a;
+        misc->red[tb][wg][1][row_b] = r_b;
+      }
+      tc::mbar_arrive(&misc->sums_full[tb]);
+      tc::mbar_arrive(&misc->tab_free[tb]);
+    }
+  } else {
+    // ------------------------------------------------------------------ Q into tensor memory, one block ahead, and epilogue (128 threads)
+    const int quad = warp & 3;
+    const int cq = lane & 3;
+    const int row_a = quad * 16 + (lane >> 2), row_b = row_a + 8;     // the two query rows of this thread
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+    uint32_t n_staged = 0, n_items = 0;
+    // the next item's Q tile, if the item keeps anything (word 4 n + cq of a row is word cq of its 16-byte chunk n); its number
+    auto next_item = [&](uint32_t seq) -> int {
+      int item = 0;
+      if (lane == 0) item = item_get(&misc->items, seq, &misc->abort_flag);
+      item = __shfl_sync(0xffffffffu, item, 0);
+      if (item < 0) return item;
+      int i, bhq;
+      item_block(g, item, bhq, i);
+      if (a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] == a.row_ptr[(size_t)bhq * (g.N + 1) + i]) return item;
+      const uint32_t qb = n_staged & 1;
+      if (!tc::mbar_wait_parked(&misc->q_full, n_staged & 1, &misc->abort_flag)) return -2;
+      if (!tc::mbar_wait_parked(&misc->qt_empty[qb], ((n_staged >> 1) & 1) ^ 1, &misc->abort_flag)) return -2;
+      tc::tc_fence_after();
+#pragma unroll 1
+      for (int h = 0; h < C::DH; ++h) {
+        uint32_t w[16];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+          const unsigned char* at = q_tile + h * kSlab + ((n ^ (row_a & 7)) << 4) + 4 * cq;      // (row_b & 7 is the same)
+          w[2 * n] = *reinterpret_cast<const uint32_t*>(at + row_a * 128);
+          w[2 * n + 1] = *reinterpret_cast<const uint32_t*>(at + row_b * 128);
+        }
+        tc::tmem_st_16x128b_x8(lane_addr + C::TM_Q + qb * 64 + 32 * h, w);
+      }
+      tc::mbar_arrive(&misc->q_empty);
+      tc::tmem_st_wait();
+      tc::tc_fence_before();
+      tc::mbar_arrive(&misc->qt_full[qb]);
+      ++n_staged;
+      return item;
+    };
+    int item = next_item(0);
+    for (uint32_t n_all = 0;; ++n_all) {
+      if (item == -2) goto done;
+      if (item < 0) break;
+      const int item_next = next_item(n_all + 1);
+      int i, bhq;
+      item_block(g, item, bhq, i);
+      const int tb = n_all & 1;
+      VSA2_WAIT_PARKED(&misc->tab_full[tb], (n_all >> 1) & 1);
+      const int k = misc->list_k[tb];
+      VSA2_WAIT_PARKED(&misc->sums_full[tb], (n_all >> 1) & 1);
+      const uint32_t ob_ = n_items & 1;
       float inv_a = 0.f, inv_b = 0.f;
       if (k > 0) {
-        const float la = misc->red[0][0][row_a] + misc->red[1][0][row_a], lb = misc->red[0][0][row_b] + misc->red[1][0][row_b];
-        const float ra = misc->red[0][1][row_a] + misc->red[1][1][row_a], rb = misc->red[0][1][row_b] + misc->red[1][1][row_b];
+        const float la = misc->red[tb][0][0][row_a] + misc->red[tb][1][0][row_a], lb = misc->red[tb][0][0][row_b] + misc->red[tb][1][0][row_b];
+        const float ra = misc->red[tb][0][1][row_a] + misc->red[tb][1][1][row_a], rb = misc->red[tb][0][1][row_b] + misc->red[tb][1][1][row_b];
         inv_a = 1.f / ra;
         inv_b = 1.f / rb;
-        if (wg == 0 && cq == 0) {
-          // sums outside the safe range (overflow, NaN or total underflow): hand the block to the exact kernel
-          if (!(la > 1e-30f && la < 1e30f && ra > 1e-30f) || !(lb > 1e-30f && lb < 1e30f && rb > 1e-30f)) misc->rescue_flag = 1;
+        if (cq == 0) {
           const int ta = misc->tok[tb][row_a], tk_b = misc->tok[tb][row_b];
-          if (ta >= 0) a.lse[(size_t)bhq * g.S + ta] = (m_a + __log2f(la)) * 0.6931471805599453f;
-          if (tk_b >= 0) a.lse[(size_t)bhq * g.S + tk_b] = (m_b + __log2f(lb)) * 0.6931471805599453f;
+          if (ta >= 0) a.lse[(size_t)bhq * g.S + ta] = (misc->m_ref[tb][row_a] + __log2f(la)) * 0.6931471805599453f;
+          if (tk_b >= 0) a.lse[(size_t)bhq * g.S + tk_b] = (misc->m_ref[tb][row_b] + __log2f(lb)) * 0.6931471805599453f;
         }
-        VSA2_WAIT(&misc->o_full, n_items & 1);
+        // sums outside the safe range (overflow, NaN or total underflow): hand the block to the exact kernel, once
+        const bool bad = !(la > 1e-30f && la < 1e30f && ra > 1e-30f) || !(lb > 1e-30f && lb < 1e30f && rb > 1e-30f);
+        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued, n_all + 1) != n_all + 1) {
+          const int slot = atomicAdd(a.rescue_count, 1);
+          if (slot < a.rescue_cap) a.rescue_items[slot] = item;
+          else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);
+        }
+        VSA2_WAIT_PARKED(&misc->o_full[ob_], (n_items >> 1) & 1);
         tc::tc_fence_after();
-      } else if (wg == 0 && cq == 0) {
+      } else if (cq == 0) {
         const int ta = misc->tok[tb][row_a], tk_b = misc->tok[tb][row_b];
         if (ta >= 0) a.lse[(size_t)bhq * g.S + ta] = -INFINITY;
         if (tk_b >= 0) a.lse[(size_t)bhq * g.S + tk_b] = -INFINITY;
       }
 
-      // O[l, d] = O_acc[q, d] / (rounded row sum) + gate[q] * O_c[d]; this warpgroup owns COLS output columns
+      // O[l, d] = O_acc[q, d] / (rounded row sum) + gate[q] * O_c[d]
       {
         // The accumulator is read in slices of 32 columns inside a rolled loop: what runs once per query block is fetched
         // from the instruction cache once per query block (the tile loop has evicted it by then).
         const float ga = misc->gate[tb][row_a], gb = misc->gate[tb][row_b];
         const int ta = misc->tok[tb][row_a], tk_b = misc->tok[tb][row_b];
         bf16* ob = reinterpret_cast<bf16*>(a.o);
-        const size_t base_a = ((size_t)bhq * g.S + (ta >= 0 ? ta : 0)) * D + wg * COLS, base_b = ((size_t)bhq * g.S + (tk_b >= 0 ? tk_b : 0)) * D + wg * COLS;
+        const size_t base_a = ((size_t)bhq * g.S + (ta >= 0 ? ta : 0)) * D, base_b = ((size_t)bhq * g.S + (tk_b >= 0 ? tk_b : 0)) * D;
 #pragma unroll 1
-        for (int n0 = 0; n0 < COLS / 8; n0 += 4) {
+        for (int n0 = 0; n0 < D / 8; n0 += 4) {
           uint32_t acc[16];
           if (k > 0) {
-            tc::tmem_ld_16x256b_x4(lane_addr + C::TM_O + wg * COLS + 8 * n0, acc);
+            tc::tmem_ld_16x256b_x4(lane_addr + C::TM_O + ob_ * 128 + 8 * n0, acc);
             tc::tmem_ld_wait();
-            if (n0 + 4 >= COLS / 8) {
+            if (n0 + 4 >= D / 8) {
               tc::tc_fence_before();
-              tc::mbar_arrive(&misc->o_empty);
+              tc::mbar_arrive(&misc->o_empty[ob_]);
             }
           } else {
 #pragma unroll
@@ -558,7 +602,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
           float v[16];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const float2 oc2 = *reinterpret_cast<const float2*>(&misc->oc[tb][wg * COLS + 8 * (n0 + u) + 2 * cq]);
+            const float2 oc2 = *reinterpret_cast<const float2*>(&misc->oc[tb][8 * (n0 + u) + 2 * cq]);
             v[4 * u] = fmaf(ga, oc2.x, __uint_as_float(acc[4 * u]) * inv_a);
             v[4 * u + 1] = fmaf(ga, oc2.y, __uint_as_float(acc[4 * u + 1]) * inv_a);
             v[4 * u + 2] = fmaf(gb, oc2.x, __uint_as_float(acc[4 * u + 2]) * inv_b);
@@ -598,12 +642,8 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         }
       }
       tc::mbar_arrive(&misc->tab_free[tb]);
-      if (k > 0 && wg == 0 && sm_tid == 0 && misc->rescue_flag) {
-        int slot = atomicAdd(a.rescue_count, 1);
-        if (slot < a.rescue_cap) a.rescue_items[slot] = item;
-        else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);
-      }
       if (k > 0) ++n_items;
+      item = item_next;
     }
   }
 
@@ -655,12 +695,12 @@ cudaError_t launch_fine_fwd_rows_tc(const Geo& g, const bf16* q, const bf16* k, 
   if (g.D == 128) {
     const size_t smb = FwdRows<128>::smem_bytes(g.N);
     static KernelAttr attr;
-    if ((e = prepare_kernel((const void*)fine_fwd_rows_tc_kernel<128>, attr, smb, kFrThreads, 256 * 56 + 256 * 200))) return e;
+    if ((e = prepare_kernel((const void*)fine_fwd_rows_tc_kernel<128>, attr, smb, kFrThreads, kFrRegs))) return e;
     launch_kernel(fine_fwd_rows_tc_kernel<128>, grid, kFrThreads, smb, st, tq, tk, tv, tqt, tkt, tvt, g, a);
   } else {
     const size_t smb = FwdRows<64>::smem_bytes(g.N);
     static KernelAttr attr;
-    if ((e = prepare_kernel((const void*)fine_fwd_rows_tc_kernel<64>, attr, smb, kFrThreads, 256 * 56 + 256 * 200))) return e;
+    if ((e = prepare_kernel((const void*)fine_fwd_rows_tc_kernel<64>, attr, smb, kFrThreads, kFrRegs))) return e;
     launch_kernel(fine_fwd_rows_tc_kernel<64>, grid, kFrThreads, smb, st, tq, tk, tv, tqt, tkt, tvt, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
