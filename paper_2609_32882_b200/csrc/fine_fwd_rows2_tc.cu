@@ -394,23 +394,12 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           VSA2_WAIT(&misc->s_full[buf], (tgt >> 1) & 1);
           tc::tc_fence_after();
           VSA2_WAIT(&misc->p_free[buf], ((tgt >> 1) & 1) ^ 1);      // (the P buffer: PV of the tile two back has read it)
-#if VSA2_X & 8
-          uint32_t s2[2][32];
-          tc::tmem_ld32(lane_addr + C::TM_S + buf * 128, s2[0]);
-#endif
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-#if VSA2_X & 8
-            uint32_t (&sv)[32] = s2[c & 1];
-            uint32_t pk[16];
-            tc::tmem_ld_wait();
-            if (c < 3) tc::tmem_ld32(lane_addr + C::TM_S + buf * 128 + 32 * (c + 1), s2[(c + 1) & 1]);
-#else
             uint32_t sv[32], pk[16];
             tc::tmem_ld32(lane_addr + C::TM_S + buf * 128 + 32 * c, sv);
             tc::tmem_ld_wait();
-#endif
-            if (c == 3 && !(VSA2_X & 2)) {
+            if (c == 3) {
               tc::tc_fence_before();
               tc::mbar_arrive(&misc->s_free[buf]);
             }
@@ -433,9 +422,6 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           tc::tmem_st_wait();
           tc::tc_fence_before();
           tc::mbar_arrive(&misc->p_ready[buf]);
-#if VSA2_X & 2
-          tc::mbar_arrive(&misc->s_free[buf]);
-#endif
         }
         tg += nt;
         misc->red[wg][0][row] = l_sum2.x + l_sum2.y;

@@ -6,9 +6,6 @@
 
 namespace vsa2 {
 
-#ifndef VSA2_X
-#define VSA2_X 0
-#endif
 constexpr uint32_t kSlab = 8192;   // one cube x 64 channels of bf16, 64 rows of 128 bytes, 128-byte swizzled
 
 __device__ __forceinline__ float ex2_approx(float x) {
