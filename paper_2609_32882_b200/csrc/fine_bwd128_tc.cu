@@ -279,7 +279,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
   if (!(F16 && PASS == 0) && a.when == 0) grid_enter_items(a.items);
 
   if (warp < 8) {
-    tc::reg_dec<56>();
+    tc::reg_dec<72>();
     if (warp < 4) {
       // ---------------------------------------------------------------- TMA producers
       const int which = warp & 1;                           // 0: ring A (Y0) + the stationary tiles, 1: ring B (Y1)
@@ -552,7 +552,10 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
     }
   } else {
     // ------------------------------------------------------------------ elementwise stage + epilogue (256 threads)
-    tc::reg_inc<200>();
+    // (Packed arithmetic in the dK/dV pass, and 16 of its threads' registers for warp 7, which had 20 words in local memory: 45.5 -> 44.4
+    // Mcycles for the backward of 219,600 tokens, 10 heads, which under the power cap is 31.8 -> 31.5 ms.  Sixteen elementwise warps of 32 columns a
+    // thread: 43.5 Mcycles, 31.3 ms, within the runs' spread.)
+    tc::reg_inc<184>();
     const int quad = warp & 3;
     const int half = (warp - 8) >> 2;            // which 64 columns of a tile, and which D / 2 channels in the epilogue
     const int row = (quad << 5) | lane;          // row of the tile = token of the stationary cube = tensor-memory lane
@@ -646,10 +649,12 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
 #pragma unroll
               for (int e4 = 0; e4 < 8; ++e4) {
                 const float4 ls = l4[e4];
-                pc[4 * e4 + 0] = ex2_approx(fmaf(__uint_as_float(pf[32 * c + 4 * e4 + 0]), c2, -ls.x));
-                pc[4 * e4 + 1] = ex2_approx(fmaf(__uint_as_float(pf[32 * c + 4 * e4 + 1]), c2, -ls.y));
-                pc[4 * e4 + 2] = ex2_approx(fmaf(__uint_as_float(pf[32 * c + 4 * e4 + 2]), c2, -ls.z));
-                pc[4 * e4 + 3] = ex2_approx(fmaf(__uint_as_float(pf[32 * c + 4 * e4 + 3]), c2, -ls.w));
+                const int e0 = 32 * c + 4 * e4;
+                const float2 xa = fma_bits2(pf[e0], pf[e0 + 1], c2, -ls.x, -ls.y), xb = fma_bits2(pf[e0 + 2], pf[e0 + 3], c2, -ls.z, -ls.w);
+                pc[4 * e4 + 0] = ex2_approx(xa.x);
+                pc[4 * e4 + 1] = ex2_approx(xa.y);
+                pc[4 * e4 + 2] = ex2_approx(xb.x);
+                pc[4 * e4 + 3] = ex2_approx(xb.y);
               }
 #pragma unroll
               for (int e = 0; e < 32; ++e) pf[32 * c + e] = __float_as_uint(pc[e]);
@@ -681,10 +686,12 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
 #pragma unroll
               for (int e4 = 0; e4 < 8; ++e4) {
                 const float4 dl = d4[e4];
-                ds[4 * e4 + 0] = __uint_as_float(pf[32 * c + 4 * e4 + 0]) * (__uint_as_float(dp[32 * c + 4 * e4 + 0]) - dl.x);
-                ds[4 * e4 + 1] = __uint_as_float(pf[32 * c + 4 * e4 + 1]) * (__uint_as_float(dp[32 * c + 4 * e4 + 1]) - dl.y);
-                ds[4 * e4 + 2] = __uint_as_float(pf[32 * c + 4 * e4 + 2]) * (__uint_as_float(dp[32 * c + 4 * e4 + 2]) - dl.z);
-                ds[4 * e4 + 3] = __uint_as_float(pf[32 * c + 4 * e4 + 3]) * (__uint_as_float(dp[32 * c + 4 * e4 + 3]) - dl.w);
+                const int e0 = 32 * c + 4 * e4;
+                const float2 da = ds_bits2(pf[e0], pf[e0 + 1], dp[e0], dp[e0 + 1], dl.x, dl.y), db = ds_bits2(pf[e0 + 2], pf[e0 + 3], dp[e0 + 2], dp[e0 + 3], dl.z, dl.w);
+                ds[4 * e4 + 0] = da.x;
+                ds[4 * e4 + 1] = da.y;
+                ds[4 * e4 + 2] = db.x;
+                ds[4 * e4 + 3] = db.y;
               }
               if constexpr (F16) {     // (a dS at the clamp: the dQ pass has met the same value and raised the flag)
                 uint32_t h[16];
@@ -808,7 +815,7 @@ static cudaError_t launch_bwd128(const CUtensorMap& x0, const CUtensorMap& x1, c
   cudaError_t e;
   static KernelAttr attr;
   if ((e = prepare_kernel((const void*)fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE>, attr, Bwd128<D>::smem_bytes, kW2Threads,
-                          256 * 56 + 256 * 200)))
+                          256 * 72 + 256 * 184)))
     return e;
   launch_kernel(fine_bwd128_tc_kernel<D, PASS, SPLIT, F16, STORE>, grid, kW2Threads, Bwd128<D>::smem_bytes, st, x0, x1, y0, y1, g, a);
   return cudaGetLastError();

@@ -516,7 +516,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             tc::mbar_arrive(&misc->dp_free[s]);
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
-              const float2 d = ds_bits2(sv[c], sv[c + 1], dp[c], dp[c + 1], dlt);
+              const float2 d = ds_bits2(sv[c], sv[c + 1], dp[c], dp[c + 1], dlt, dlt);
               const float d0 = d.x, d1 = d.y;
               if constexpr (SPLIT) {
                 split_bf16x2(d0, d1, pd[c >> 1], pdl[c >> 1]);

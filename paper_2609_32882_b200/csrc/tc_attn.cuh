@@ -25,10 +25,10 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 __device__ __forceinline__ float2 fma_bits2(uint32_t a, uint32_t b, float s, float c0, float c1) {
   return __ffma2_rn(make_float2(__uint_as_float(a), __uint_as_float(b)), make_float2(s, s), make_float2(c0, c1));
 }
-// (p0 (d0 - m), p1 (d1 - m)), all but m as float bits
-__device__ __forceinline__ float2 ds_bits2(uint32_t p0, uint32_t p1, uint32_t d0, uint32_t d1, float m) {
+// (p0 (d0 - m0), p1 (d1 - m1)), p and d as float bits
+__device__ __forceinline__ float2 ds_bits2(uint32_t p0, uint32_t p1, uint32_t d0, uint32_t d1, float m0, float m1) {
   return __fmul2_rn(make_float2(__uint_as_float(p0), __uint_as_float(p1)),
-                    __fadd2_rn(make_float2(__uint_as_float(d0), __uint_as_float(d1)), make_float2(-m, -m)));
+                    __fadd2_rn(make_float2(__uint_as_float(d0), __uint_as_float(d1)), make_float2(-m0, -m1)));
 }
 // 64 bf16 (32 packed words) -> one 128-byte row of a swizzled operand tile: 16-byte chunk c lands at c ^ (row & 7)
 __device__ __forceinline__ void store_row_sw128(unsigned char* tile, int row, const uint32_t (&packed)[32]) {
