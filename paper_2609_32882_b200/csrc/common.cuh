@@ -86,10 +86,9 @@ __device__ __forceinline__ void grid_enter(bool early = true) {
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
-// Persistent kernels with many items per CTA keep the SMs to themselves until they end.  Successors let in by all / up to eight items per
-// CTA / none, us: 2048-token clip, training 188 / 187 / 177; ragged clip 724 / 703 / 709; 13 x 27 x 47 tokens, 16 heads 1506 / 1520 / 1507;
-// 480p, 12 heads on 3 6276 / 6265 / 6228; from 720p on the same.  (The line is the ragged clip's; the training clip would do better
-// below it.)
+// The attention kernels let their successor in when they end: beside them it finds no room or takes issue slots from them (all kernels early up to
+// eight items per CTA / the router alone, us: 2048-token clip, training 176 / 168; toy grid, as a graph 72 / 62; 480p, 12 heads on 3 6093 / 6039;
+// ragged clip 624 / 623; 13 x 27 x 47 tokens, 16 heads 1335 / 1331).  The router lets it in up to eight items per CTA (without: ragged clip 624 / 628).
 __device__ __forceinline__ void grid_enter_items(int items) { grid_enter(items <= 8 * (int)gridDim.x); }
 
 // Brackets the launches of one kernel group with the caller's timing events.

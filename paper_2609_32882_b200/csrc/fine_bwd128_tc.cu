@@ -276,7 +276,7 @@ fine_bwd128_tc_kernel(const __grid_constant__ CUtensorMap tm_x0, const __grid_co
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
-  if (!(F16 && PASS == 0) && a.when == 0) grid_enter_items(a.items);
+  if (!(F16 && PASS == 0) && a.when == 0) grid_enter(false);
 
   if (warp < 8) {
     tc::reg_dec<72>();

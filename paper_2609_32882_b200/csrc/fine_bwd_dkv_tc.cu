@@ -179,7 +179,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     grid_enter(false);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   } else if (!second && !fallback) {
-    grid_enter_items(a.items);
+    grid_enter(false);
   }
   if (a.when == 1 && __syncthreads_or(tid == 0 && *a.range_flag != 0)) {
     if (warp == 2) tc::tmem_dealloc(tmem_base, 512);

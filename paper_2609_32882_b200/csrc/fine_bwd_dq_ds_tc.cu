@@ -73,7 +73,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
-  grid_enter_items(a.items);
+  grid_enter(false);
   if (__syncthreads_or(tid == 0 && *a.range_flag != 0)) {       // the fallback computes dQ
     if (warp == 3) tc::tmem_dealloc(tmem_base, 64 * kDsSets);
     return;

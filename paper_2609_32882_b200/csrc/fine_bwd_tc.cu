@@ -213,7 +213,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
-  if (!F16 && a.when == 0) grid_enter_items(total_items);
+  if (!F16 && a.when == 0) grid_enter(false);
   // tensor-memory columns: S^T buffers 0, 64; dP^T buffers 128, 192; dQ^T 256 (SPLIT: its low-order part at 320)
 
   if (warp < 2) {

@@ -195,7 +195,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
-  grid_enter_items(g.batch * g.Hq * g.N);
+  grid_enter(false);
 
   if (warp < 8) {
     tc::reg_dec<kFrServiceRegs>();
