@@ -5,7 +5,7 @@
 
 #include <atomic>
 
-#include "common.cuh"
+#include "pooled_inputs.cuh"
 
 using namespace vsa2;
 
@@ -740,24 +740,14 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   const bf16* o_res = (saved != nullptr && !g.out_f32) ? reinterpret_cast<const bf16*>(saved->o_res) : nullptr;
   // (V is copied to fp16 for GQA groups only; O is of V's size or, a mean of up to a few thousand rows, well below it)
   const DsScale scale{at<float2>(workspace, lay.absmax), at<int>(workspace, lay.ds_exp), dkv_pass_gqa_f16(g) ? pow2i(-16) : 0.f};
+  unsigned char* pooled_ws = at<unsigned char>(cube_ws, cl.pooled);
+  const PooledInputs pooled = coarse && !wide ? pooled_bwd_inputs(g, saved->qc, saved->kc, saved->vc, nullptr, pooled_ws) : PooledInputs{};
   {
     ProfScope ps(VSA2_KERNEL_BWD_PRE, st);
     VSA2_CUDA(launch_bwd_preprocess(fx, dob, o, o_res, coarse ? gate : nullptr, oc_hat, delta, coarse ? dgate : nullptr,
-                                    d_oc_hat, dq_pass_f16(g) ? at<float2>(workspace, lay.absmax) : nullptr,
+                                    wide ? d_oc_hat : nullptr, coarse && !wide ? pooled.y[3] : nullptr, coarse && !wide ? pooled_bwd_delta(g, pooled_ws) : nullptr,
+                                    dq_pass_f16(g) ? at<float2>(workspace, lay.absmax) : nullptr,
                                     reinterpret_cast<StatusBlock*>(workspace), st));
-  }
-  if (coarse) {
-    // pooled grid: the bf16 copies with the dense map, the pooled preprocess, dQ, dK/dV (+ two group spreads)
-    ProfScope ps(VSA2_KERNEL_COARSE_BWD, st);
-    if (wide) VSA2_CUDA(launch_fold_sum(n, n.Hq, d_oc_hat, d_oc_hat_cube, st));
-    VSA2_CUDA(launch_coarse_bwd_pooled(g, saved->qc, saved->kc, saved->vc, saved->oc_hat, saved->lse_c, d_oc_hat_cube,
-                                       dqc_cube, dkc_cube, dvc_cube, at<unsigned char>(cube_ws, cl.pooled),
-                                       reinterpret_cast<StatusBlock*>(workspace), st));
-    if (wide) {
-      VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dqc_cube, dqc, st));
-      VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dkc_cube, dkc, st));
-      VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dvc_cube, dvc, st));
-    }
   }
   // dS kept from the dK/dV pass for the dQ pass, which then runs inside it; otherwise the dQ pass recomputes dS and runs first
   const DsLayout dl = ds_layout(g, scratch != nullptr ? scratch_bytes : 0, false);
@@ -774,17 +764,34 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   // cubes of 128 tokens: both passes on 128 x 128 tiles
   const bool wide128 = wide && g.Lt == 0 && fine_bwd128_supported(n);
   {
+    // what the passes below read beside the tensors (cubes of 128 tokens: the inputs of the coarse backward come from its own launches)
+    ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st);
+    const PrepLists lists{sd.row_ptr, sd.col_idx, wide ? map->col_ptr : col_ptr, wide ? map->row_idx : row_idx, at<int>(scratch, dl.pos), sd.counters,
+                          2 * g.batch * g.Hkv, pk.shift > 0 ? at<int>(workspace, lay.full) : nullptr, pk.first, dkv_order};
+    const bool pooled_here = coarse && !wide;
+    if (ds_groups > 0 || pooled_here)
+      VSA2_CUDA(launch_bwd_prep(ds_groups > 0 ? &fx : nullptr, qb, at<unsigned char>(workspace, bwd_f16_offset(g)), kb,
+                                at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale,
+                                &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], ds_groups > 0 ? &dg : nullptr, lists,
+                                pooled_here ? &pooled : nullptr, st));
+  }
+  if (coarse) {
+    // pooled grid: dQ, dK/dV (+ two group spreads); cubes of 128 tokens: first the bf16 copies with the dense map and the pooled preprocess
+    ProfScope ps(VSA2_KERNEL_COARSE_BWD, st);
+    if (wide) VSA2_CUDA(launch_fold_sum(n, n.Hq, d_oc_hat, d_oc_hat_cube, st));
+    VSA2_CUDA(launch_coarse_bwd_pooled(g, saved->qc, saved->kc, saved->vc, saved->oc_hat, saved->lse_c, wide ? d_oc_hat_cube : nullptr,
+                                       dqc_cube, dkc_cube, dvc_cube, pooled_ws,
+                                       reinterpret_cast<StatusBlock*>(workspace), st));
+    if (wide) {
+      VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dqc_cube, dqc, st));
+      VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dkc_cube, dkc, st));
+      VSA2_CUDA(launch_expand_rows(n, n.Hq, true, dvc_cube, dvc, st));
+    }
+  }
+  if (ds_groups == 0) {
     const bool f16 = dq_pass_f16(g);     // the copy, the fp16 form, the (idle) fallback
     ProfScope ps(VSA2_KERNEL_FINE_BWD_DQ, st);
-    if (ds_groups > 0) {
-      VSA2_CUDA(launch_cast_qk(fx, qb, at<unsigned char>(workspace, bwd_f16_offset(g)), kb,
-                               at<unsigned char>(workspace, bwd_f16_offset(g) + bwd_q16_bytes(g)), scale,
-                               &reinterpret_cast<StatusBlock*>(workspace)->pad[kRangeFlagSlot], st));
-      VSA2_CUDA(launch_ds_positions(dg, sd.row_ptr, sd.col_idx, wide ? map->col_ptr : col_ptr, wide ? map->row_idx : row_idx,
-                                    at<int>(scratch, dl.pos), sd.counters, 2 * g.batch * g.Hkv, st));
-      if (pk.shift > 0) VSA2_CUDA(launch_full_counts(fx, pk, col_ptr, row_idx, at<int>(workspace, lay.full), st));
-      if (dkv_order != nullptr) VSA2_CUDA(launch_dkv_order(dg, wide ? map->col_ptr : col_ptr, dkv_order, st));
-    } else if (wide128)
+    if (wide128)
       VSA2_CUDA(launch_fine_bwd128_dq_tc(n, qb, kb, vb, dob, lse, delta, row_ptr, col_idx, coarse ? dqc : nullptr, dq,
                                          reinterpret_cast<StatusBlock*>(workspace), st,
                                          f16 ? at<unsigned char>(workspace, bwd_f16_offset(g)) : nullptr,

@@ -1,6 +1,6 @@
 // First step of the backward pass: the per-token quantities of the gated merge (paper Eq. 14) and of the fine softmax
 // (Eq. 12) that the dQ and dK/dV passes (fine_bwd_tc.cu) and the coarse backward read:
-//   delta = rowsum(dO * O_f), dGate = rowsum(dO * O_c), dO_c_hat[n] = sum_{l in n} gate_l dO_l
+//   delta = rowsum(dO * O_f), dGate = rowsum(dO * O_c), dO_c_hat[n] = sum_{l in n} gate_l dO_l (in fp32, or in bf16 with its row sum against O_c)
 // and, for the scale of dS in the fp16 passes (DsScale in common.cuh), the largest |dO| and |O| of every block.
 // HBM-bound: one pass over dO, O (and the bf16 rounding residual of O).
 #include "common.cuh"
@@ -19,8 +19,8 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
                                                              const float* gate,
                                                              const float* oc_hat, Geo g,
                                                              float* __restrict__ delta, float* __restrict__ dgate,
-                                                             float* __restrict__ d_oc_hat, float2* __restrict__ absmax,
-                                                             StatusBlock* clear) {
+                                                             float* __restrict__ d_oc_hat, bf16* __restrict__ do_c, float* __restrict__ delta_c,
+                                                             float2* __restrict__ absmax, StatusBlock* clear) {
   grid_enter();
   constexpr int CH = D / 8;                // threads per token = 16-byte chunks of a token row
   constexpr int PAR = 256 / CH;            // tokens at a time
@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
   __shared__ __align__(16) bf16 rows[kBlockTokens * D];
   __shared__ float gates[kBlockTokens];
   __shared__ unsigned warp_max[2][8];
+  __shared__ float row_sum[D / 32];
   if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(StatusBlock) / 4)
     reinterpret_cast<int*>(clear)[threadIdx.x] = 0;      // (for the kernels behind this one)
   const int i = blockIdx.x, ch = threadIdx.x % CH, hq = blockIdx.y, b = blockIdx.z;
@@ -135,18 +136,36 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
     float acc = 0.f;
 #pragma unroll 16
     for (int p = 0; p < kBlockTokens; ++p) acc = fmaf(gates[p], __bfloat162float(rows[p * D + threadIdx.x]), acc);
-    d_oc_hat[(bhq * g.Nvid + i) * D + threadIdx.x] = acc;
+    const size_t at = (bhq * g.Nvid + i) * D + threadIdx.x;
+    if (d_oc_hat != nullptr) d_oc_hat[at] = acc;
+    if (do_c != nullptr) {
+      // the coarse branch's backward reads dO_c_hat in bf16 and rowsum(dO_c_hat * O_c) of that
+      const bf16 h = __float2bfloat16_rn(acc);
+      do_c[at] = h;
+      float s = __bfloat162float(h) * oc_hat[at];
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      if (lane == 0) row_sum[threadIdx.x >> 5] = s;
+    }
+  }
+  if (do_c == nullptr) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < D / 32; ++w) s += row_sum[w];
+    delta_c[bhq * g.Nvid + i] = s;
   }
 }
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
-                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, float2* absmax,
-                                  StatusBlock* clear, cudaStream_t st) {
+                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, bf16* do_c, float* delta_c,
+                                  float2* absmax, StatusBlock* clear, cudaStream_t st) {
   dim3 grid(g.N, g.Hq, g.batch);
-  if (g.D == 128 && g.out_f32) launch_kernel(bwd_preprocess_kernel<128, true>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
-  else if (g.D == 128) launch_kernel(bwd_preprocess_kernel<128, false>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
-  else if (g.out_f32) launch_kernel(bwd_preprocess_kernel<64, true>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
-  else launch_kernel(bwd_preprocess_kernel<64, false>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, absmax, clear);
+  if (g.D == 128 && g.out_f32) launch_kernel(bwd_preprocess_kernel<128, true>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, do_c, delta_c, absmax, clear);
+  else if (g.D == 128) launch_kernel(bwd_preprocess_kernel<128, false>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, do_c, delta_c, absmax, clear);
+  else if (g.out_f32) launch_kernel(bwd_preprocess_kernel<64, true>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, do_c, delta_c, absmax, clear);
+  else launch_kernel(bwd_preprocess_kernel<64, false>, grid, 256, 0, st, d_o, o, o_res, gate, oc_hat, g, delta, dgate, d_oc_hat, do_c, delta_c, absmax, clear);
   return cudaGetLastError();
 }
 

@@ -3,7 +3,7 @@
 // and dense attention over them is block-sparse attention with every block selected.  The pooled fp32 means are
 // rounded to bf16 (the precision of the model's other attention operands), the outputs stay fp32.
 // This file holds the glue: the pooled problem's geometry, the dense block map, the casts and the launch sequence.
-#include "common.cuh"
+#include "pooled_inputs.cuh"
 
 namespace vsa2 {
 
@@ -47,48 +47,15 @@ PooledLayout pooled_layout(const Geo& g, bool backward) {
   return r;
 }
 
-// dense map of np blocks for `heads` lists: ptr[h][i] = i * np, idx[h][i * np + j] = j (its transpose is the same map)
-__device__ __forceinline__ void dense_map_entry(int* ptr, int* idx, int np, size_t e) {
-  const size_t per = (size_t)np * np + np + 1, h = e / per;
-  const int r = (int)(e - h * per);
-  if (r <= np) ptr[h * (np + 1) + r] = r * np;
-  else idx[h * np * np + r - np - 1] = (r - np - 1) % np;
-}
-// What the pooled kernels read, in one launch: bf16 copies of up to four fp32 tensors, the dense map, a cleared status block
-struct PooledInputs {
-  const float* x[4];
-  bf16* y[4];
-  size_t n4[4];            // 16-byte groups of each tensor
-  int* ptr;
-  int* idx;
-  int np;
-  size_t map_words;        // heads * (np * np + np + 1)
-  StatusBlock* status;
-};
 __global__ void __launch_bounds__(256) pooled_inputs_kernel(PooledInputs p) {
   grid_enter();
-  if (blockIdx.x == 0 && threadIdx.x < sizeof(StatusBlock) / 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
-  const size_t stride = (size_t)gridDim.x * blockDim.x, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-#pragma unroll
-  for (int t = 0; t < 4; ++t)
-    for (size_t i = first; i < p.n4[t]; i += stride) {
-      const float4 v = reinterpret_cast<const float4*>(p.x[t])[i];
-      __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-      uint2 o;
-      o.x = *reinterpret_cast<uint32_t*>(&a);
-      o.y = *reinterpret_cast<uint32_t*>(&b);
-      reinterpret_cast<uint2*>(p.y[t])[i] = o;
-    }
-  for (size_t i = first; i < p.map_words; i += stride) dense_map_entry(p.ptr, p.idx, p.np, i);
+  pooled_inputs(p, blockIdx.x, gridDim.x);
 }
 static cudaError_t launch_pooled_inputs(const PooledInputs& p, cudaStream_t st) {
-  size_t most = p.map_words;
-  for (size_t n : p.n4) most = n > most ? n : most;
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  const size_t blocks = (most + 255) / 256;
-  launch_kernel(pooled_inputs_kernel, (unsigned)(blocks < (size_t)sms * 8 ? blocks : (size_t)sms * 8), 256, 0, st, p);
+  launch_kernel(pooled_inputs_kernel, pooled_inputs_blocks(p, sms), 256, 0, st, p);
   return cudaGetLastError();
 }
 
@@ -105,9 +72,9 @@ __global__ void spread_to_group_kernel(const float* x_kv, float* __restrict__ x_
   reinterpret_cast<float4*>(x_q)[(size_t)hq * per_head4 + i] = v;
 }
 
-// The pooled passes count their work items in a status block of their own (inside the scratch region); a non-zero
-// status word there (a bounded wait that ran out, a rescue list that overflowed) is copied into the caller's status word,
-// which is the one vsa2_device_status reads.
+// The pooled passes count their work items in a status block of their own (inside the scratch region).  The backward ones report to the
+// caller's block; a non-zero status word that the forward leaves there (a bounded wait that ran out, a rescue list that overflowed) is copied
+// into the caller's status word, which is the one vsa2_device_status reads.
 __global__ void merge_status_kernel(const StatusBlock* from, StatusBlock* into) {
   grid_enter();
   const int s = from->status;
@@ -136,34 +103,45 @@ cudaError_t launch_coarse_fwd_pooled(const Geo& g, const float* qc, const float*
   return cudaGetLastError();
 }
 
+PooledInputs pooled_bwd_inputs(const Geo& g, const float* qc, const float* kc, const float* vc, const float* d_oc_hat, void* workspace) {
+  const PooledLayout lay = pooled_layout(g, true);
+  unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
+  const int np = pooled_geo(g).N;
+  const size_t BHq = (size_t)g.batch * g.Hq, nq = BHq * g.N * g.D / 4, nk = (size_t)g.batch * g.Hkv * g.N * g.D / 4;      // (multiples of the head dimension)
+  auto b16 = [&](size_t off) { return reinterpret_cast<bf16*>(ws + off); };
+  return PooledInputs{{qc, kc, vc, d_oc_hat}, {b16(lay.q16), b16(lay.k16), b16(lay.v16), b16(lay.do16)}, {nq, nk, nk, d_oc_hat != nullptr ? nq : 0},
+                      reinterpret_cast<int*>(ws + lay.ptr), reinterpret_cast<int*>(ws + lay.idx), np, BHq * ((size_t)np * np + np + 1),
+                      reinterpret_cast<StatusBlock*>(ws + lay.status)};
+}
+float* pooled_bwd_delta(const Geo& g, void* workspace) { return reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + pooled_layout(g, true).delta); }
+
 cudaError_t launch_coarse_bwd_pooled(const Geo& g, const float* qc, const float* kc, const float* vc, const float* oc_hat,
                                      const float* lse_c, const float* d_oc_hat, float* dqc, float* dkc, float* dvc,
                                      void* workspace, StatusBlock* caller_status, cudaStream_t st) {
   const Geo p = pooled_geo(g);
   const PooledLayout lay = pooled_layout(g, true);
+  const PooledInputs in = pooled_bwd_inputs(g, qc, kc, vc, d_oc_hat, workspace);
   unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
-  const size_t BHq = (size_t)g.batch * g.Hq, BHk = (size_t)g.batch * g.Hkv;
-  bf16* q16 = reinterpret_cast<bf16*>(ws + lay.q16);
-  bf16* k16 = reinterpret_cast<bf16*>(ws + lay.k16);
-  bf16* v16 = reinterpret_cast<bf16*>(ws + lay.v16);
-  bf16* do16 = reinterpret_cast<bf16*>(ws + lay.do16);
-  int* ptr = reinterpret_cast<int*>(ws + lay.ptr);
-  int* idx = reinterpret_cast<int*>(ws + lay.idx);
-  float* delta = reinterpret_cast<float*>(ws + lay.delta);
+  const size_t BHq = (size_t)g.batch * g.Hq;
+  const bf16 *q16 = in.y[0], *k16 = in.y[1], *v16 = in.y[2], *do16 = in.y[3];
+  const int *ptr = in.ptr, *idx = in.idx;
+  float* delta = pooled_bwd_delta(g, workspace);
   float* dk_kv = reinterpret_cast<float*>(ws + lay.dk_kv);
   float* dv_kv = reinterpret_cast<float*>(ws + lay.dv_kv);
-  StatusBlock* status = reinterpret_cast<StatusBlock*>(ws + lay.status);
+  StatusBlock* status = in.status;
   cudaError_t e;
-  const size_t nq = BHq * g.N * g.D / 4, nk = BHk * g.N * g.D / 4;      // (multiples of the head dimension)
-  const PooledInputs in{{qc, kc, vc, d_oc_hat}, {q16, k16, v16, do16}, {nq, nk, nk, nq},
-                        ptr, idx, p.N, BHq * ((size_t)p.N * p.N + p.N + 1), status};
-  if ((e = launch_pooled_inputs(in, st)) != cudaSuccess) return e;
-  // delta_c = rowsum(dO_c * O_c) through the preprocess kernel of the pooled problem (no gate: only delta is written)
-  if ((e = launch_bwd_preprocess(p, do16, oc_hat, nullptr, nullptr, nullptr, delta, nullptr, nullptr, nullptr, nullptr, st)) != cudaSuccess) return e;
-  if ((e = launch_fine_bwd_dq_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, dqc, status, st, nullptr, nullptr, nullptr)) != cudaSuccess) return e;
+  if (d_oc_hat != nullptr) {
+    if ((e = launch_pooled_inputs(in, st)) != cudaSuccess) return e;
+    // delta_c = rowsum(dO_c * O_c) through the preprocess kernel of the pooled problem (no gate: only delta is written)
+    if ((e = launch_bwd_preprocess(p, do16, oc_hat, nullptr, nullptr, nullptr, delta, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, st)) != cudaSuccess) return e;
+  }
+  if ((e = launch_fine_bwd_dq_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, dqc, status, st, nullptr, nullptr, nullptr,
+                                 caller_status)) != cudaSuccess)
+    return e;
   const bool grouped = g.rep > 1;
   if ((e = launch_fine_bwd_dkv_tc(p, q16, k16, v16, do16, lse_c, delta, ptr, idx, nullptr, nullptr, grouped ? dk_kv : dkc,
-                                  grouped ? dv_kv : dvc, status, st, false, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr)) != cudaSuccess)
+                                  grouped ? dv_kv : dvc, status, st, false, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, PackedCubes{},
+                                  caller_status)) != cudaSuccess)
     return e;
   if (grouped) {
     const size_t per_head4 = (size_t)g.N * g.D / 4;
@@ -172,7 +150,6 @@ cudaError_t launch_coarse_bwd_pooled(const Geo& g, const float* qc, const float*
     launch_kernel(spread_to_group_kernel, grid, 256, 0, st, dv_kv, dvc, g.rep, per_head4, (int)BHq);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  launch_kernel(merge_status_kernel, 1, 1, 0, st, status, caller_status);
   return cudaGetLastError();
 }
 

@@ -364,7 +364,7 @@ cudaError_t launch_fine_fwd_rows2_tc(const Geo& g, bool pair_heads, const bf16* 
 // (lse, or delta where dO itself is a scaled copy) and taken out again by the epilogues, both exact.
 struct DsScale {
   const float2* absmax;   // [B, Hq, N of the block problem]: max |dO|, max |O| of each block (launch_bwd_preprocess)
-  int* exp;               // [B, Hkv], written by launch_cast_qk
+  int* exp;               // [B, Hkv], written by launch_bwd_prep or launch_cast_qk
   // 0, or (where dP is formed from an fp16 copy of V) the max |O| below which a group's V counts as too small for that copy and
   // the range flag goes up: an element of it is then good to 2^-9 of V's size at worst
   float least_o;
@@ -390,7 +390,7 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
 cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                   const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
                                   const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
-                                     const DsScale* scale);
+                                  const DsScale* scale, StatusBlock* report = nullptr);      // (report: the status block written to, if not `status`)
 bool fine_bwd_dq_uses_f16(const Geo& g);
 // Slot of StatusBlock.pad that holds the range flag of the fp16 dQ passes (the slot behind it: the fallback launch's counter)
 constexpr int kRangeFlagSlot = 8;
@@ -409,23 +409,33 @@ struct PackedCubes {
   const int* full;    // [B, Hq, N]: entries of a column list in front of them
 };
 PackedCubes packed_cubes(const Geo& g, const int* full);
-cudaError_t launch_full_counts(const Geo& g, const PackedCubes& pk, const int* ptr, const int* idx, int* full, cudaStream_t st);
 // dS kept between the two backward passes (fine_bwd_dq_ds_tc.cu, fine_bwd128_dq_ds_tc.cu): scratch for the pairs of `chunk_groups`
 // KV groups at a time.  On 128 x 128 tiles every size and list below is that of the cube map.
 struct StoredDs {
   void* scratch;        // chunk_groups * rep * nnz_cap tiles of 8 KB (64 queries x 64 keys, fp16), or of 32 KB (128 x 128)
-  const int* pos;       // [B, Hq, nnz_cap], filled by launch_ds_positions
-  int* counters;        // two words per chunk, cleared by launch_ds_positions
-  int* order;           // null, or [B, Hkv, N]: items of the dK/dV pass, longest lists of a group first (launch_dkv_order)
+  const int* pos;       // [B, Hq, nnz_cap], filled by launch_bwd_prep
+  int* counters;        // two words per chunk, cleared by launch_bwd_prep
+  int* order;           // null, or [B, Hkv, N]: items of the dK/dV pass, longest lists of a group first (launch_bwd_prep)
   int chunk_groups;
   const int* row_ptr;
   const int* col_idx;
   const float* dqc;
   void* dq;
 };
-cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col_idx, const int* col_ptr, const int* row_idx, int* pos,
-                                int* counters, int n_counters, cudaStream_t st);
-cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st);
+// The backward's preparation in one launch (bwd_prep.cu), each part where its pointer is given: the fp16 copies of Q and K (`fine`: geometry of
+// the fine passes) as launch_cast_qk makes them; the lists of the dS tiles; the inputs of the coarse backward.
+struct PrepLists {
+  const int *row_ptr, *col_idx, *col_ptr, *row_idx;
+  int* pos;             // StoredDs::pos and counters
+  int* counters;
+  int n_counters;
+  int* full;            // null, or PackedCubes::full, with the first cube of the layer
+  int first;
+  int* order;           // null, or StoredDs::order
+};
+struct PooledInputs;
+cudaError_t launch_bwd_prep(const Geo* fine, const bf16* q, void* q16, const bf16* k, void* k16, const DsScale& scale, int* range_flag,
+                            const Geo* lists_geo, const PrepLists& lists, const PooledInputs* pooled, cudaStream_t st);
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,
                                   int* item_counter, bool swizzled, const int* ds_exp, const PackedCubes& pk, cudaStream_t st);
@@ -445,11 +455,11 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
                                    const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp,
-                                   const PackedCubes& pk = PackedCubes{});
+                                   const PackedCubes& pk = PackedCubes{}, StatusBlock* report = nullptr);
 bool fine_bwd_dkv_gqa_uses_f16(const Geo& g);
 bool fine_bwd_dkv_splits_long_columns(const Geo& g, bool split_long_columns);
 
 cudaError_t launch_bwd_preprocess(const Geo& g, const bf16* d_o, const void* o, const bf16* o_res, const float* gate,
-                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, float2* absmax,
-                                  StatusBlock* clear, cudaStream_t st);
+                                  const float* oc_hat, float* delta, float* dgate, float* d_oc_hat, bf16* do_c, float* delta_c,
+                                  float2* absmax, StatusBlock* clear, cudaStream_t st);
 }  // namespace vsa2

@@ -672,7 +672,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
                                    const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp,
-                                   const PackedCubes& pk) {
+                                   const PackedCubes& pk, StatusBlock* report) {
   if (g.rep > kMaxRep) return cudaErrorInvalidValue;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16;
   // GQA groups without a precision flag take the all-fp16 form when they are given scratch for fp16 copies of V and dO as
@@ -722,7 +722,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   auto launch = [&](bool split, int* counter, int k_lo, int k_hi, int when, int group0, int groups,
                     bool ds, int overlap = 0) -> cudaError_t {
     const int items = groups * g.N, grid = items < sms ? items : sms;
-    DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
+    DkvArgs a{counter, lse, delta, col_ptr, row_idx, dkc, dvc, dk, dv, report != nullptr ? report : status, k_lo, k_hi, &status->pad[kRangeFlagSlot], when,
               group0 * g.N, items, ds ? reinterpret_cast<unsigned char*>(sd->scratch) : nullptr, ds ? sd->pos : nullptr,
               group0 * g.rep, when == 1 || ds ? ds_exp : nullptr, ds ? sd->order : nullptr, pk, overlap};
     if (ds && pack) {
@@ -801,31 +801,6 @@ PackedCubes packed_cubes(const Geo& g, const int* full) {
   const int rows = (g.T - (g.Nt - 1) * g.Bt) * g.Bh * g.Bw;
   const int shift = rows == kBlockTokens / 4 ? 2 : rows == kBlockTokens / 2 ? 1 : 0;
   return PackedCubes{g.Nvid >= 128 && g.Nt > 1 ? shift : 0, (g.Nt - 1) * g.Nh * g.Nw, full};
-}
-
-// One warp per list: the entries in front of the cubes of the last layer -- or, of a list that does not have them at its end, all
-// but the text blocks (nothing of it is packed then)
-__global__ void __launch_bounds__(256) full_counts_kernel(int N, int Nvid, int first, long long cap, const int* ptr,
-                                                          const int* idx, int* __restrict__ full) {
-  grid_enter();
-  const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (j >= N) return;
-  const size_t bh = blockIdx.y;
-  const int beg = ptr[bh * (N + 1) + j], k = ptr[bh * (N + 1) + j + 1] - beg - (N - Nvid);
-  const int* list = idx + bh * cap + beg;
-  int n = 0, last = -1;                      // entries before the layer, and the last of them
-  for (int e = lane; e < k; e += 32)
-    if (list[e] < first) {
-      ++n;
-      last = e;
-    }
-  n = __reduce_add_sync(0xffffffffu, n);
-  last = __reduce_max_sync(0xffffffffu, last);
-  if (lane == 0) full[bh * N + j] = last + 1 == n ? n : k;
-}
-cudaError_t launch_full_counts(const Geo& g, const PackedCubes& pk, const int* ptr, const int* idx, int* full, cudaStream_t st) {
-  launch_kernel(full_counts_kernel, dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st, g.N, g.Nvid, pk.first, g.nnz_cap, ptr, idx, full);
-  return cudaGetLastError();
 }
 
 // Whether the dK/dV pass of a GQA problem takes its all-fp16 form when it is given the scratch for the four copies.  Rows that

@@ -234,88 +234,6 @@ done:
   if (warp == 3) tc::tmem_dealloc(tmem_base, 64 * kDsSets);
 }
 
-// place of every entry of the column lists in the row lists of its head: pos[bh][e] for entry e of row_idx (both kinds of lists
-// ascend).  One warp per column; `counters`: n words to clear for the launches behind this one
-__global__ void __launch_bounds__(256) ds_positions_kernel(int N, long long cap, const int* row_ptr,
-                                                           const int* col_idx, const int* col_ptr,
-                                                           const int* row_idx, int* __restrict__ pos,
-                                                           int* __restrict__ counters, int n_counters) {
-  grid_enter();
-  if (blockIdx.x == 0 && blockIdx.y == 0)
-    for (int c = threadIdx.x; c < n_counters; c += blockDim.x) counters[c] = 0;
-  const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (j >= N) return;
-  const size_t bh = blockIdx.y;
-  const int* rp = row_ptr + bh * (N + 1);
-  const int* ci = col_idx + bh * cap;
-  const int beg = col_ptr[bh * (N + 1) + j], end = col_ptr[bh * (N + 1) + j + 1];
-  for (int e = beg + lane; e < end; e += 32) {
-    const int i = row_idx[bh * cap + e];
-    int lo = rp[i], hi = rp[i + 1] - 1;       // the entry j is in [lo, hi]
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (ci[mid] < j) lo = mid + 1;
-      else hi = mid;
-    }
-    pos[bh * cap + e] = min(lo, (int)cap - 1);      // (column lists that are not the row lists' transpose stay inside the scratch)
-  }
-}
-
-cudaError_t launch_ds_positions(const Geo& g, const int* row_ptr, const int* col_idx, const int* col_ptr, const int* row_idx, int* pos,
-                                int* counters, int n_counters, cudaStream_t st) {
-  launch_kernel(ds_positions_kernel, dim3((g.N + 7) / 8, g.batch * g.Hq), 256, 0, st, g.N, g.nnz_cap, row_ptr, col_idx, col_ptr, row_idx, pos,
-                                                                         counters, n_counters);
-  return cudaGetLastError();
-}
-
-// Items of the dK/dV pass in the order of their list lengths, longest first, group by group (groups stay in order: the CTAs work on
-// one group's tensors at a time, which L2 holds).  A KV block's list can be ten times the mean, and a launch that draws such
-// items last ends with most SMs idle (720p, budget of 16..256 cubes, four heads a group: 0.7 ms for the mean item of a
-// 6 ms launch).  Counting sort by one block per group; the order of equal lengths depends on the run, the results do not.
-__global__ void __launch_bounds__(1024) dkv_order_kernel(Geo g, const int* col_ptr, int* __restrict__ order) {
-  grid_enter();
-  __shared__ int hist[1024], warp_sums[32], longest;
-  const int bhk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  auto length = [&](int r) {
-    int bh, j, k = 0;
-    item_block(g, bhk * g.N + r, bh, j);
-    for (int hh = 0; hh < g.rep; ++hh) {
-      const int* c = col_ptr + ((size_t)bhk * g.rep + hh) * (g.N + 1) + j;
-      k += c[1] - c[0];
-    }
-    return k;
-  };
-  hist[tid] = 0;
-  if (tid == 0) longest = 0;
-  __syncthreads();
-  int m = 0;
-  for (int r = tid; r < g.N; r += 1024) m = max(m, length(r));
-  m = __reduce_max_sync(0xffffffffu, m);
-  if (lane == 0) atomicMax(&longest, m);
-  __syncthreads();
-  const int shift = max(0, 22 - __clz(longest));          // bins of 2^shift entries: longest >> shift < 1024
-  for (int r = tid; r < g.N; r += 1024) atomicAdd(&hist[1023 - (length(r) >> shift)], 1);
-  __syncthreads();
-  const int mine = hist[tid];
-  int incl = mine;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  if (lane == 31) warp_sums[warp] = incl;
-  __syncthreads();
-  int before = 0;
-  for (int w = 0; w < warp; ++w) before += warp_sums[w];
-  hist[tid] = before + incl - mine;
-  __syncthreads();
-  for (int r = tid; r < g.N; r += 1024) order[bhk * g.N + atomicAdd(&hist[1023 - (length(r) >> shift)], 1)] = bhk * g.N + r;
-}
-
-cudaError_t launch_dkv_order(const Geo& g, const int* col_ptr, int* order, cudaStream_t st) {
-  launch_kernel(dkv_order_kernel, g.batch * g.Hkv, 1024, 0, st, g, col_ptr, order);
-  return cudaGetLastError();
-}
-
 // dQ of the heads head0 .. head0 + heads - 1 (index batch * Hq) from their dS tiles
 cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds, int head0, int heads, const int* row_ptr,
                                   const int* col_idx, const float* dqc, void* dq, StatusBlock* status, int* range_flag,

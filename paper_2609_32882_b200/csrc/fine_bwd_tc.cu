@@ -43,119 +43,14 @@ struct DqArgs {
   const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale)
 };
 
-// An exponent of max|dO| max|O| from which on a dS is taken to leave the fp16 range: a weight of 2^-8 in the row of the largest dO is
-// enough.  The flag then goes up before the fp16 passes have run for nothing (720p, 8 heads, dO of 3e6: 14.6 -> 7 ms).
-constexpr int kBeyondF16 = 22;
-// DsScale::exp of the groups blockIdx.x, blockIdx.x + step, ... (the whole block calls it); true if the fp16 forms are not to run:
-// O below least_o, or dS beyond the fp16 range
-__device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int per_group, int step) {
-  __shared__ unsigned red[2][8];
-  bool bad = false;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int grp = blockIdx.x; grp < groups; grp += step) {
-    const uint2* m = reinterpret_cast<const uint2*>(s.absmax) + (size_t)grp * per_group;      // (bit patterns order like the numbers)
-    unsigned d = 0u, o = 0u;
-    for (int i = threadIdx.x; i < per_group; i += 256) {
-      const uint2 v = m[i];
-      d = max(d, v.x);
-      o = max(o, v.y);
-    }
-    d = __reduce_max_sync(0xffffffffu, d);
-    o = __reduce_max_sync(0xffffffffu, o);
-    if (lane == 0) {
-      red[0][warp] = d;
-      red[1][warp] = o;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < 8; ++w) {
-        d = max(d, red[0][w]);
-        o = max(o, red[1][w]);
-      }
-      const int e = (int)(d >> 23) - 127 + (int)(o >> 23) - 127;
-      s.exp[grp] = d == 0u || o == 0u ? 0 : max(0, min(-3 - e, 100));
-      bad |= o != 0u && (__uint_as_float(o) < s.least_o || (d != 0u && e >= kBeyondF16));
-    }
-    __syncthreads();
-  }
-  return bad;
-}
-
-// Copies of two bf16 tensors in fp16 (8 elements per thread and step), b times 2^b_exp[its group of `b_group` steps] if there is one.
-// A finite bf16 below 65520 in magnitude has an exact fp16 image if it is a multiple of 2^-24 (all of 2^-17 and more are: fp16
-// keeps more mantissa bits), and one within 2^-25 otherwise; a finite value beyond that range sets `range_flag` and the caller's
-// fp16 kernels stand back.  The first `reducers` blocks form the exponents of dS meanwhile.
-// SCALED: there is a b_exp.  (Without it the magnitudes are compared as the integers they are; a thread walks its groups by adding
-// quotient and remainder of its stride: a division per step and products of 1 made the copies of 480p 30 us longer.)
 template <bool SCALED>
-__global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(const uint4* xa, uint4* __restrict__ ya, size_t na,
-                                                               const uint4* xb, uint4* __restrict__ yb, size_t nb,
-                                                               const int* b_exp, unsigned b_group, int* range_flag,
-                                                               DsScale scale, int groups, int per_group, int reducers) {
+__global__ void __launch_bounds__(256) cast_bf16_to_f16_kernel(CastJob job, DsScale scale, int groups, int per_group, int reducers) {
   grid_enter();
-  const size_t stride = (size_t)(gridDim.x - reducers) * blockDim.x, n = na + nb;
-  bool bad = false;
   if ((int)blockIdx.x < reducers) {
-    if (form_ds_exp(scale, groups, per_group, reducers)) atomicExch(range_flag, 1);
+    if (form_ds_exp(scale, groups, per_group, blockIdx.x, reducers)) atomicExch(job.range_flag, 1);
     return;
   }
-  constexpr int U = 4;      // 16-byte loads in flight per thread (a pure streaming kernel)
-  const size_t first = (size_t)(blockIdx.x - reducers) * blockDim.x + threadIdx.x;
-  unsigned grp = 0u, in_grp = 0u, step_q = 0u, step_r = 0u;      // SCALED: group of element group i of b, place in it; the same of a stride
-  if (SCALED) {
-    step_q = (unsigned)(stride / b_group);
-    step_r = (unsigned)(stride % b_group);
-  }
-  bool in_b = false;
-  for (size_t i0 = first; i0 < n; i0 += U * stride) {
-    uint4 v[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const size_t i = i0 + u * stride;
-      v[u] = i < n ? (i < na ? xa[i] : xb[i - na]) : make_uint4(0, 0, 0, 0);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const size_t i = i0 + u * stride;
-      if (i >= n) break;
-      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-      float f = 1.f;
-      if (SCALED && i >= na) {
-        if (!in_b) {
-          in_b = true;
-          grp = (unsigned)((i - na) / b_group);
-          in_grp = (unsigned)((i - na) % b_group);
-        } else {
-          grp += step_q;
-          in_grp += step_r;
-          if (in_grp >= b_group) {
-            in_grp -= b_group;
-            ++grp;
-          }
-        }
-        // (a scaled value stays finite: the exponent takes the largest of a group to 2^-2 / max |O| at most)
-        f = pow2i(b_exp[grp]);
-      }
-      uint32_t r[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float x0 = __uint_as_float(w[e] << 16), x1 = __uint_as_float(w[e] & 0xffff0000u);
-        if (SCALED) {
-          x0 *= f;
-          x1 *= f;
-        }
-        // magnitudes as bit patterns (65536 <= |x| < infinity)
-        const uint32_t m0 = __float_as_uint(x0) & 0x7fffffffu, m1 = __float_as_uint(x1) & 0x7fffffffu;
-        bad |= m0 - 0x47800000u < 0x38000000u || m1 - 0x47800000u < 0x38000000u;
-        const __half2 h = __floats2half2_rn(x0, x1);
-        r[e] = *reinterpret_cast<const uint32_t*>(&h);
-      }
-      const uint4 o = make_uint4(r[0], r[1], r[2], r[3]);
-      if (i < na) ya[i] = o;
-      else yb[i - na] = o;
-    }
-  }
-  if (bad) atomicExch(range_flag, 1);
+  cast_bf16_to_f16<SCALED>(job, blockIdx.x - reducers, gridDim.x - reducers);
 }
 
 // Roles: warp 0 = TMA producer of the K pairs (ring A; a slot is held until the dQ^T product of its tile is done) and of
@@ -543,7 +438,7 @@ done:
 cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                   const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
                                   const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
-                                  const DsScale* scale) {
+                                  const DsScale* scale, StatusBlock* report) {
   const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr && scale != nullptr;
   const bf16* qa = f16 ? reinterpret_cast<const bf16*>(q16) : q;      // (same element size and layout: the maps only move bytes)
   const bf16* ka = f16 ? reinterpret_cast<const bf16*>(k16) : k;
@@ -556,7 +451,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
-  DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, status, flag, 0, f16 ? scale->exp : nullptr};
+  DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, report != nullptr ? report : status, flag, 0, f16 ? scale->exp : nullptr};
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
   const bool split = !(g.flags & VSA2_FLAG_FAST_BWD);
@@ -613,9 +508,7 @@ static cudaError_t launch_cast(const bf16* a, void* a16, size_t na, const bf16* 
   // (element counts are multiples of the head dimension)
   const int reducers = groups < sms ? groups : sms;
   auto* kernel = b_exp != nullptr ? cast_bf16_to_f16_kernel<true> : cast_bf16_to_f16_kernel<false>;
-  launch_kernel(kernel, sms * 16 + reducers, 256, 0, st, reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8,
-                                                     reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16), nb / 8, b_exp,
-                                                     (unsigned)(b_group / 8), range_flag, scale, groups, per_group, reducers);
+  launch_kernel(kernel, sms * kCastBlocksPerSm + reducers, 256, 0, st, cast_job(a, a16, na, b, b16, nb, b_exp, b_group, range_flag), scale, groups, per_group, reducers);
   return cudaGetLastError();
 }
 

@@ -255,4 +255,127 @@ __device__ __forceinline__ void bwd_init_barriers(BwdMisc* misc) {
                       (lane >> 1) * 64, (CW), (CH), (CT), (BH));                                                  \
   } while (0)
 
+// An exponent of max|dO| max|O| from which on a dS is taken to leave the fp16 range: a weight of 2^-8 in the row of the largest dO is
+// enough.  The flag then goes up before the fp16 passes have run for nothing (720p, 8 heads, dO of 3e6: 14.6 -> 7 ms).
+constexpr int kBeyondF16 = 22;
+// DsScale::exp of the groups first, first + step, ... (the whole block calls it); true if the fp16 forms are not to run:
+// O below least_o, or dS beyond the fp16 range
+__device__ __forceinline__ bool form_ds_exp(const DsScale& s, int groups, int per_group, int first, int step) {
+  __shared__ unsigned red[2][8];
+  bool bad = false;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int grp = first; grp < groups; grp += step) {
+    const uint2* m = reinterpret_cast<const uint2*>(s.absmax) + (size_t)grp * per_group;      // (bit patterns order like the numbers)
+    unsigned d = 0u, o = 0u;
+    for (int i = threadIdx.x; i < per_group; i += 256) {
+      const uint2 v = m[i];
+      d = max(d, v.x);
+      o = max(o, v.y);
+    }
+    d = __reduce_max_sync(0xffffffffu, d);
+    o = __reduce_max_sync(0xffffffffu, o);
+    if (lane == 0) {
+      red[0][warp] = d;
+      red[1][warp] = o;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) {
+        d = max(d, red[0][w]);
+        o = max(o, red[1][w]);
+      }
+      const int e = (int)(d >> 23) - 127 + (int)(o >> 23) - 127;
+      s.exp[grp] = d == 0u || o == 0u ? 0 : max(0, min(-3 - e, 100));
+      bad |= o != 0u && (__uint_as_float(o) < s.least_o || (d != 0u && e >= kBeyondF16));
+    }
+    __syncthreads();
+  }
+  return bad;
+}
+
+struct CastJob {
+  const uint4* xa;
+  uint4* ya;
+  size_t na;
+  const uint4* xb;
+  uint4* yb;
+  size_t nb;
+  const int* b_exp;
+  unsigned b_group;
+  int* range_flag;
+};
+constexpr int kCastBlocksPerSm = 16;
+// (na, nb, b_group: elements, multiples of 8)
+inline CastJob cast_job(const bf16* a, void* a16, size_t na, const bf16* b, void* b16, size_t nb, const int* b_exp, size_t b_group, int* range_flag) {
+  return CastJob{reinterpret_cast<const uint4*>(a), reinterpret_cast<uint4*>(a16), na / 8, reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(b16),
+                 nb / 8, b_exp, (unsigned)(b_group / 8), range_flag};
+}
+// Copies of two bf16 tensors in fp16 (8 elements per thread and step), b times 2^b_exp[its group of `b_group` steps] if there is one.
+// A finite bf16 below 65520 in magnitude has an exact fp16 image if it is a multiple of 2^-24 (all of 2^-17 and more are: fp16
+// keeps more mantissa bits), and one within 2^-25 otherwise; a finite value beyond that range sets `range_flag` and the caller's
+// fp16 kernels stand back.
+// SCALED: there is a b_exp.  (Without it the magnitudes are compared as the integers they are; a thread walks its groups by adding
+// quotient and remainder of its stride: a division per step and products of 1 made the copies of 480p 30 us longer.)
+template <bool SCALED>
+__device__ __forceinline__ void cast_bf16_to_f16(const CastJob& job, unsigned block, unsigned blocks) {
+  const size_t stride = (size_t)blocks * blockDim.x, n = job.na + job.nb, first = (size_t)block * blockDim.x + threadIdx.x;
+  bool bad = false;
+  constexpr int U = 4;      // 16-byte loads in flight per thread (a pure streaming kernel)
+  unsigned grp = 0u, in_grp = 0u, step_q = 0u, step_r = 0u;      // SCALED: group of element group i of b, place in it; the same of a stride
+  if (SCALED) {
+    step_q = (unsigned)(stride / job.b_group);
+    step_r = (unsigned)(stride % job.b_group);
+  }
+  bool in_b = false;
+  for (size_t i0 = first; i0 < n; i0 += U * stride) {
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const size_t i = i0 + u * stride;
+      v[u] = i < n ? (i < job.na ? job.xa[i] : job.xb[i - job.na]) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const size_t i = i0 + u * stride;
+      if (i >= n) break;
+      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+      float f = 1.f;
+      if (SCALED && i >= job.na) {
+        if (!in_b) {
+          in_b = true;
+          grp = (unsigned)((i - job.na) / job.b_group);
+          in_grp = (unsigned)((i - job.na) % job.b_group);
+        } else {
+          grp += step_q;
+          in_grp += step_r;
+          if (in_grp >= job.b_group) {
+            in_grp -= job.b_group;
+            ++grp;
+          }
+        }
+        // (a scaled value stays finite: the exponent takes the largest of a group to 2^-2 / max |O| at most)
+        f = pow2i(job.b_exp[grp]);
+      }
+      uint32_t r[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float x0 = __uint_as_float(w[e] << 16), x1 = __uint_as_float(w[e] & 0xffff0000u);
+        if (SCALED) {
+          x0 *= f;
+          x1 *= f;
+        }
+        // magnitudes as bit patterns (65536 <= |x| < infinity)
+        const uint32_t m0 = __float_as_uint(x0) & 0x7fffffffu, m1 = __float_as_uint(x1) & 0x7fffffffu;
+        bad |= m0 - 0x47800000u < 0x38000000u || m1 - 0x47800000u < 0x38000000u;
+        const __half2 h = __floats2half2_rn(x0, x1);
+        r[e] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      const uint4 o = make_uint4(r[0], r[1], r[2], r[3]);
+      if (i < job.na) job.ya[i] = o;
+      else job.yb[i - job.na] = o;
+    }
+  }
+  if (bad) atomicExch(job.range_flag, 1);
+}
+
 }  // namespace vsa2
