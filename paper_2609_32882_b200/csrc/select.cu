@@ -271,6 +271,28 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
   }
 }
 
+// The k-th largest (1 <= k <= entries) of a row that a warp holds in registers, U a lane (0 where there is none), by bisection over the bits
+template <int U>
+__device__ __forceinline__ unsigned row_threshold(const unsigned (&v)[U], int k) {
+  unsigned tau = 0u;            // the largest value with at least k entries >= it
+  for (int bit = 31; bit >= 0; --bit) {
+    const unsigned cand = tau | (1u << bit);
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) c += v[u] >= cand;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (c >= k) tau = cand;
+    if (c == k) {               // exactly the kept entries: the threshold is the smallest of them
+      unsigned m = 0xffffffffu;
+#pragma unroll
+      for (int u = 0; u < U; ++u) m = v[u] >= cand ? min(m, v[u]) : m;
+      tau = __reduce_min_sync(0xffffffffu, m);
+      break;
+    }
+  }
+  return tau;
+}
+
 // per-row modes: the k_i-th largest of row i by bisection over the bits of the threshold, a warp per row with the row in registers
 // (U a lane): rounds of U compares and a warp sum until the kept entries are apart from the others (about 20; 32 with ties), no
 // shared memory, no atomics, no block barrier.  grid (ceil(N / 8), BH)
@@ -298,22 +320,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* pr,
     if (lane == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
     return;
   }
-  unsigned tau = 0u;            // the largest value with at least k entries >= it
-  for (int bit = 31; bit >= 0; --bit) {
-    const unsigned cand = tau | (1u << bit);
-    int c = 0;
-#pragma unroll
-    for (int u = 0; u < U; ++u) c += v[u] >= cand;
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (c >= k) tau = cand;
-    if (c == k) {               // exactly the kept entries: the threshold is the smallest of them
-      unsigned m = 0xffffffffu;
-#pragma unroll
-      for (int u = 0; u < U; ++u) m = v[u] >= cand ? min(m, v[u]) : m;
-      tau = __reduce_min_sync(0xffffffffu, m);
-      break;
-    }
-  }
+  const unsigned tau = row_threshold<U>(v, k);
   int gt = 0;
 #pragma unroll
   for (int u = 0; u < U; ++u) gt += v[u] > tau;
@@ -667,18 +674,19 @@ __global__ void __launch_bounds__(1024) sel_settle_kernel(const float* pr, int N
   }
 }
 
-// Up to kSelOneBlockN cubes: everything behind the counts of the kept entries in one launch, a block per head with both bitmaps in
+// Up to kSelOneBlockN cubes, per-row modes: the selection in one launch (row_tau: null, or the thresholds are there), or everything behind the counts of the kept entries, a block per head with both bitmaps in
 // shared memory (the six launches below take 2 us and a gap each and keep a few SMs busy).  Same rules: rows in order, ties at the
 // threshold to the lower column, both maps cut at the capacity.
 __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, int words, int per_sequence,
                                                         const unsigned* state, const int* row_gt,
                                                         const int* row_eq, const float* row_tau,
                                                         const int* row_eq_take, const int* row_cnt,
-                                                        const unsigned* bits_gt, const unsigned* bits_eq,
+                                                        const unsigned* bits_gt, const unsigned* bits_eq, int K, const int* budgets,
                                                         int* row_ptr, int* col_idx, int* col_ptr, int* row_idx, long long nnz_cap,
                                                         StatusBlock* status) {
   grid_enter();
   constexpr int W = kSelOneBlockN / 32;
+  __shared__ unsigned tau_s[kSelOneBlockN];
   __shared__ unsigned bm[kSelOneBlockN * W], bt[kSelOneBlockN * W];
   __shared__ int take_s[kSelOneBlockN], ptr_s[kSelOneBlockN], ws[33];
   const int bh = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -691,9 +699,36 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, 
       take = max(0, min(eq, (int)state[bh * 8 + 4] - before));
       cnt = row_gt[base + tid] + take;
     }
-  } else if (tid < N) {
-    take = row_eq_take[base + tid];
-    cnt = row_cnt[base + tid];
+  } else if (row_tau != nullptr) {
+    if (tid < N) {
+      take = row_eq_take[base + tid];
+      cnt = row_cnt[base + tid];
+      tau_s[tid] = __float_as_uint(row_tau[base + tid]);
+    }
+  } else {
+    // the thresholds as well (as sel_row_topk_warp_kernel): a launch less, and its wait
+    for (int i = warp; i < N; i += 32) {
+      const unsigned* src = reinterpret_cast<const unsigned*>(pr) + (base + i) * N;
+      unsigned v[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) v[w] = w * 32 + lane < N ? src[w * 32 + lane] : 0u;
+      const int k = max(0, min(budgets ? budgets[base + i] : K, N));
+      const unsigned tau = k > 0 ? row_threshold<W>(v, k) : 0x7f800000u;
+      int gt = 0;
+#pragma unroll
+      for (int w = 0; w < W; ++w) gt += v[w] > tau;
+      gt = __reduce_add_sync(0xffffffffu, gt);
+      if (lane == 0) {
+        tau_s[i] = tau;
+        take_s[i] = k > 0 ? k - gt : 0;
+        ptr_s[i] = k;
+      }
+    }
+    __syncthreads();
+    if (tid < N) {
+      take = take_s[tid];
+      cnt = ptr_s[tid];
+    }
   }
   int pre = block_excl_scan(cnt, ws, tot);
   if (tid < N) {
@@ -710,7 +745,7 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, 
   const unsigned lt = (1u << lane) - 1u;
   for (int i = warp; i < N; i += 32) {
     const unsigned* src = reinterpret_cast<const unsigned*>(pr) + (base + i) * N;
-    const unsigned tau = per_sequence ? 0u : __float_as_uint(row_tau[base + i]);
+    const unsigned tau = per_sequence ? 0u : tau_s[i];
     int pos = (int)min((long long)ptr_s[i], nnz_cap), left = take_s[i];
     // (the whole row is read first: a row's words one after another waited for memory every time)
     unsigned v[W], gw = 0u, ew = 0u;
@@ -792,7 +827,7 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, 
 // Route calls, us, the launches above / this: 180 cubes, 12 heads 84 / 59; 288 cubes, 2 heads 79 / 64, 24 heads 183 / 158; 336 cubes, 16
 // heads 180 / 163, 32 heads behind the one-pass router 270 / 229; 384 cubes, 16 heads 204 / 184; 480 cubes, 2 heads 99.6 / 96.3, 32
 // heads 409 / 407; 528 cubes, 2 heads 109 / 111, 32 heads 475 / 481: eight CTAs a head are too few from there on, hence kSelHeadN.
-// (One to 128 cubes have sel_maps_kernel.  For the maps of the per-row modes, and from bitmaps, a cluster was slower: 480p, 12 heads 264 / 279.)
+// (Below 129 cubes the launches above are nine.  For the maps of the per-row modes, and from bitmaps, a cluster was slower: 480p, 12 heads 264 / 279.)
 // MAPS: the maps are written.  Without: bitmaps, counts and threshold as sel_row_bits_kernel leaves them, for one-pass scores (BAND: as there).
 constexpr int kSelParts = 8, kSelHeadThreads = 512, kSelHeadN = 480;
 struct SelHead {
@@ -1106,7 +1141,7 @@ static void launch_row_topk(const Geo& g, const float* pr, const int* budgets, c
 
 // whether the selection of a head runs in a cluster
 static bool sel_head_runs(const Geo& g) {
-  return g.mode == VSA2_PER_SEQUENCE && g.N > kSelOneBlockN && g.N <= kSelHeadN;
+  return g.mode == VSA2_PER_SEQUENCE && g.N <= kSelHeadN;
 }
 template <bool BAND, bool MAPS>
 static cudaError_t launch_sel_head(const Geo& g, const float* pr, const SelectScratch& s, int* row_ptr, int* col_idx, int* col_ptr, int* row_idx,
@@ -1167,12 +1202,14 @@ cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, con
   se.redo = const_cast<int*>(redo);
   if (redo == nullptr && sel_head_runs(g))
     return launch_sel_head<false, true>(g, pr, s, row_ptr, col_idx, col_ptr, row_idx, status, se, st);
+  const bool per_sequence = g.mode == VSA2_PER_SEQUENCE, small = N <= kSelOneBlockN;
+  const bool with_thresholds = small && !per_sequence && redo == nullptr;      // (the block per head finds them itself)
   cudaError_t e;
-  if ((e = launch_thresholds<false>(g, pr, budgets, s, se, st)) != cudaSuccess) return e;
-  if (N <= kSelOneBlockN) {
-    launch_kernel(sel_maps_kernel, BH, 1024, 0, st, pr, N, s.words, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
-                                         s.row_eq_take, s.row_cnt, s.bitmap, s.bitmap_t, row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap,
-                                         status);
+  if (!with_thresholds && (e = launch_thresholds<false>(g, pr, budgets, s, se, st)) != cudaSuccess) return e;
+  if (small) {
+    launch_kernel(sel_maps_kernel, BH, 1024, 0, st, pr, N, s.words, per_sequence, s.state, s.row_gt, s.row_eq, with_thresholds ? nullptr : s.row_tau,
+                  s.row_eq_take, s.row_cnt, s.bitmap, s.bitmap_t, g.K, g.mode == VSA2_PER_QUERY_BUDGET ? budgets : nullptr, row_ptr, col_idx,
+                  col_ptr, row_idx, g.nnz_cap, status);
     return cudaGetLastError();
   }
   launch_kernel(sel_scan_rows_kernel, BH, 1024, 0, st, N, g.mode == VSA2_PER_SEQUENCE, s.state, s.row_gt, s.row_eq, s.row_tau,
