@@ -69,6 +69,12 @@ __device__ __forceinline__ int dkv_entry(const Geo& g, const DkvArgs& a, int rep
   return kind;
 }
 
+// Slots of the Q ring and of the dO ring.  With 64 channels a slot is 16 KB, half of what the plan is made for, and a short list's pass waits
+// for its loads, so there are more of them.  Backward of 13 x 27 x 47 tokens, 16 heads of 64 channels, us: 3 + 2 slots 816, 4 + 3 767, 5 + 4 769,
+// 6 + 4 777.
+__host__ __device__ constexpr int dkv_ring_a(int D, bool split) { return D == 64 ? 4 : split ? 2 : kRingA; }
+__host__ __device__ constexpr int dkv_ring_b(int D) { return D == 64 ? 3 : kRingB; }
+
 // Roles: warp 0 = TMA producer of the Q pairs (ring A) and of the stationary K and V tiles, warp 1 = TMA producer of the
 // dO pairs (ring B), warp 2 = issuer of S = Q_pair K^T, warp 3 = issuer of dP = dO_pair V^T, warp 16 = issuer of
 // dV^T += dO_pair^T P (frees the dO slot), warp 17 = issuer of dK^T += Q_pair^T dS (frees the Q slot), warps 4..11 =
@@ -122,10 +128,10 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                        const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_dot,
                        const __grid_constant__ CUtensorMap tm_qe, const __grid_constant__ CUtensorMap tm_doe, Geo g,
                        DkvArgs a) {
-  constexpr int RA = SPLIT ? 2 : kRingA;                   // slots of the Q ring
+  constexpr int RA = dkv_ring_a(D, SPLIT), RB = dkv_ring_b(D);      // slots of the Q ring and of the dO ring
   // accumulators: without SPLIT two sets of dK^T, dV^T (64 columns each), used by item parity
   constexpr uint32_t TM_DK = 256, TM_DV = SPLIT ? 384 : 320, TM_SET = 128, SETS = SPLIT ? 1 : 2;
-  using C = BwdTc<D, RA, SPLIT ? 4 : 2>;
+  using C = BwdTc<D, RA, SPLIT ? 4 : 2, RB>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* k_tile = smem + C::OFF_ST0;
@@ -133,6 +139,10 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   unsigned char* p_tile = smem + C::OFF_P;                                  // P  [128 q, 64 kv] (SPLIT: followed by its low part)
   unsigned char* ds_tile = smem + C::OFF_P + (SPLIT ? 2 : 1) * C::PBYTES;   // dS [128 q, 64 kv] (SPLIT: followed by its low part)
   BwdMisc* misc = reinterpret_cast<BwdMisc*>(smem + C::OFF_MISC);
+
+  BwdRings* rings = reinterpret_cast<BwdRings*>(smem + C::OFF_MISC + 2048);      // (D = 64)
+  uint64_t *ring_a_full = D == 64 ? rings->a_full : misc->a_full, *ring_a_empty = D == 64 ? rings->a_empty : misc->a_empty;
+  uint64_t *ring_b_full = D == 64 ? rings->b_full : misc->b_full, *ring_b_empty = D == 64 ? rings->b_empty : misc->b_empty;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float c2 = g.scale * 1.4426950408889634f;
@@ -160,7 +170,14 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
     bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4 + (STORES_DS && !SPLIT && a.ds != nullptr ? 1 : 0));
     if (STORES_DS && !SPLIT && a.ds != nullptr) tc::mbar_init(&misc->ds_free[0], 2);     // read by the dK product and by the copy
-    for (int s = 0; s < kRingB; ++s) tc::mbar_init(&misc->b_empty[s], 2);     // a dO slot is read by dP and by dV^T
+    if (D == 64) {
+      for (int s = 0; s < RA; ++s) {
+        tc::mbar_init(&ring_a_full[s], 1);
+        tc::mbar_init(&ring_a_empty[s], 1);
+      }
+      for (int s = 0; s < RB; ++s) tc::mbar_init(&ring_b_full[s], 1);
+    }
+    for (int s = 0; s < RB; ++s) tc::mbar_init(&ring_b_empty[s], 2);     // a dO slot is read by dP and by dV^T
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_k);
@@ -267,11 +284,11 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           kind_l = dkv_entry<false, PACK>(g, a, rep, b, hk, cnt_prefix, col_beg, (my_blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2, bhq_l, i_l, nullptr,
                                           my_sub, col_full, col_cnt);
         if constexpr (PACK) {
-          const uint32_t nslots = which == 0 ? RA : kRingB, slot = tg % nslots, par = (tg / nslots) & 1;
-          uint64_t* full = which == 0 ? &misc->a_full[slot] : &misc->b_full[slot];
+          const uint32_t nslots = which == 0 ? RA : RB, slot = tg % nslots, par = (tg / nslots) & 1;
+          uint64_t* full = which == 0 ? &ring_a_full[slot] : &ring_b_full[slot];
           int ok = 1;
           if (lane == 0) {
-            ok = tc::mbar_wait_parked(which == 0 ? &misc->a_empty[slot] : &misc->b_empty[slot], par ^ 1, &misc->abort_flag);
+            ok = tc::mbar_wait_parked(which == 0 ? &ring_a_empty[slot] : &ring_b_empty[slot], par ^ 1, &misc->abort_flag);
             if (ok) tc::mbar_expect_tx(full, C::SLOT);
           }
           if (!__shfl_sync(0xffffffffu, ok, 0)) goto done;
@@ -280,8 +297,8 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                                 (kind_t > 0 ? my_sub * (kSlab >> a.pk.shift) : 0),
                             tm_i, full, my_h * 64, c1, c2, c3, bhq_t);
         } else {
-          if (which == 0) VSA2_RING_LOAD(misc->a_full, misc->a_empty, RA, smem, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
-          else VSA2_RING_LOAD(misc->b_full, misc->b_empty, kRingB, smem + C::OFF_RING_B, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
+          if (which == 0) VSA2_RING_LOAD(ring_a_full, ring_a_empty, RA, smem, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
+          else VSA2_RING_LOAD(ring_b_full, ring_b_empty, RB, smem + C::OFF_RING_B, tm_i, tg, c3, c2, c1, bhq_t, {}, mbar_wait_parked);
         }
       }
     }
@@ -301,7 +318,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const uint32_t sb = tg & 1, pb = (tg >> 1) & 1;
           if (is_s) {
             const uint32_t sa = tg % RA, pa = (tg / RA) & 1;
-            VSA2_WAIT_PARKED(&misc->a_full[sa], pa);
+            VSA2_WAIT_PARKED(&ring_a_full[sa], pa);
             VSA2_WAIT_PARKED(&misc->s_free[sb], pb ^ 1);
             tc::tc_fence_after();
             if (tc::elect_one()) {
@@ -310,13 +327,14 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               if (t == nt - 1) tc::mma_commit(&misc->st_empty);
             }
           } else {
-            VSA2_WAIT_PARKED(&misc->b_full[sb], pb);
+            const uint32_t so = tg % RB;
+            VSA2_WAIT_PARKED(&ring_b_full[so], (tg / RB) & 1);
             VSA2_WAIT_PARKED(&misc->dp_free[sb], pb ^ 1);
             tc::tc_fence_after();
             if (tc::elect_one()) {
-              mma_pair_kmajor<D, F16 >= 2>(tmem_base + 128 + sb * 64, base + C::OFF_RING_B + sb * C::SLOT, b_addr);
+              mma_pair_kmajor<D, F16 >= 2>(tmem_base + 128 + sb * 64, base + C::OFF_RING_B + so * C::SLOT, b_addr);
               tc::mma_commit(&misc->dp_full[sb]);
-              tc::mma_commit(&misc->b_empty[sb]);
+              tc::mma_commit(&ring_b_empty[so]);
               if (t == nt - 1) tc::mma_commit(&misc->st_empty);
             }
           }
@@ -377,14 +395,14 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         for (int t = 0; t < nt; ++t, ++tg) {
           if (is_v) {
             // P depends on S only, so it can be ready before the dO pair of the tile has landed: wait for that too
-            const uint32_t sv = tg & 1;
-            VSA2_WAIT_PARKED(&misc->b_full[sv], (tg >> 1) & 1);
+            const uint32_t sv = tg % RB;
+            VSA2_WAIT_PARKED(&ring_b_full[sv], (tg / RB) & 1);
             VSA2_WAIT_PARKED(&misc->p_ready, tg & 1);
             tc::tc_fence_after();
             if (tc::elect_one()) {
               if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, C::PBYTES, t > 0);
               else mma_pairT_mnmajor<D, F16 >= 2>(acc, base + C::OFF_RING_B + sv * C::SLOT, b_addr, t > 0);
-              tc::mma_commit(&misc->b_empty[sv]);
+              tc::mma_commit(&ring_b_empty[sv]);
               tc::mma_commit(&misc->p_free);
               if (t == nt - 1) tc::mma_commit(&misc->o_full[set]);
             }
@@ -395,7 +413,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             if (tc::elect_one()) {
               if constexpr (SPLIT) mma_pairT_mnmajor_n128<D>(acc, base + sa * C::SLOT, b_addr, C::PBYTES, t > 0);
               else mma_pairT_mnmajor<D, F16 != 0>(acc, base + sa * C::SLOT, b_addr, t > 0);
-              tc::mma_commit(&misc->a_empty[sa]);
+              tc::mma_commit(&ring_a_empty[sa]);
               tc::mma_commit(&misc->ds_free[0]);
               if (t == nt - 1) tc::mma_commit(&misc->o_full[set]);
             }
@@ -708,7 +726,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   }
 #define VSA2_LAUNCH_DKV(DD, SP, MH, F, PK, TQ, TK, TQT, TKT, TV, TDO, TVT, TDOT)                                                                         \
   do {                                                                                                                           \
-    using L_ = BwdTc<DD, SP ? 2 : kRingA, SP ? 4 : 2>;                                                                           \
+    using L_ = BwdTc<DD, dkv_ring_a(DD, SP), SP ? 4 : 2, dkv_ring_b(DD)>;                                                         \
     static KernelAttr attr_;                                                                                                     \
     if ((e = prepare_kernel((const void*)fine_bwd_dkv_tc_kernel<DD, SP, MH, F, PK>, attr_, L_::smem_bytes, kDkvThreads,               \
                             128 * (48 + 2 * 120 + 2 * 48 + 96))))                                                                \

@@ -12,23 +12,28 @@ constexpr int kRingA = 3;          // slots of the ring whose tiles are also an 
 constexpr int kRingB = 2;          // (the ring-B slot of a tile is also the index of its tensor-memory buffers)
 static_assert(kRingB == 2, "ring B shares its slot index with the two accumulator buffers");
 
+// Barriers of the dK/dV pass's rings where they have more slots than BwdMisc holds (behind it)
+struct BwdRings {
+  uint64_t a_full[6], a_empty[6], b_full[6], b_empty[6];
+};
+
 // Shared-memory plan of both passes (D = 128: 5 x 32 KB ring slots, 2 x 16 KB stationary tiles, 2 x 16 KB operand
 // buffers, 2 KB of barriers and per-block vectors: exactly the 227 KB a block may use).  Ring A has 3 slots, ring B 2;
 // each ring has one producing warp and fixed consuming roles.
 // RA: slots of ring A; NP: 16 KB operand buffers (the dK/dV pass in its split mode trades one ring-A slot for the two
 // buffers that hold the low-order parts of P and dS).
-template <int D, int RA = kRingA, int NP = 2>
+template <int D, int RA = kRingA, int NP = 2, int RB = kRingB>
 struct BwdTc {
   static constexpr int DH = D / 64;
   static constexpr uint32_t SLOT = 2 * DH * kSlab;   // a pair of cube tiles, [half][A | B]
   static constexpr uint32_t TILE = DH * kSlab;       // one cube tile, [half]
   static constexpr uint32_t PBYTES = 128 * 128;      // 128 rows x 64 bf16
   static constexpr uint32_t OFF_RING_B = RA * SLOT;
-  static constexpr uint32_t OFF_ST0 = (RA + kRingB) * SLOT;       // stationary tile 0 (Q or K)
+  static constexpr uint32_t OFF_ST0 = (RA + RB) * SLOT;       // stationary tile 0 (Q or K)
   static constexpr uint32_t OFF_ST1 = OFF_ST0 + TILE;             // stationary tile 1 (dO or V)
   static constexpr uint32_t OFF_P = OFF_ST1 + TILE;               // the 16 KB operand buffers
   static constexpr uint32_t OFF_MISC = OFF_P + NP * PBYTES;
-  static constexpr uint32_t MISC_BYTES = 2048;
+  static constexpr uint32_t MISC_BYTES = D == 64 ? 2048 + sizeof(BwdRings) : 2048;
   static constexpr size_t smem_bytes = OFF_MISC + MISC_BYTES + 1024;
 };
 

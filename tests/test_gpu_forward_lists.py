@@ -1,4 +1,4 @@
-"""The 64-row forward on lists of every small length: empty, one block, odd and even, all of them, one after the other, with more items than
+"""The 64-row kernels, forward and backward, on lists of every small length: empty, one block, odd and even, all of them, one after the other, with more items than
 SMs (several items per CTA: its double buffers change over, empty items between them) on a grid that cuts cubes in every dimension."""
 import numpy as np
 import pytest
@@ -34,3 +34,9 @@ def test_lists_of_every_small_length(dim, out_dtype, grid):
     want, want_lse = orc.forward(to_f64(q), to_f64(k), to_f64(v), to_f64(gate), mask, geo, 1.0 / np.sqrt(dim))
     assert_close("O", to_f64(o), want, bf16_storage=out_dtype == vb.BF16)
     assert_lse_close(to_f64(lse), want_lse)
+    d_o = torch.randn_like(q)
+    got = attn.backward(q, k, v, gate, o, lse, d_o)
+    attn.check_status()
+    ref = orc.backward(to_f64(q), to_f64(k), to_f64(v), to_f64(gate), mask, geo, 1.0 / np.sqrt(dim), to_f64(d_o))
+    for name, x, y in zip(("dQ", "dK", "dV", "dgate"), got, ref):
+        assert_close(name, to_f64(x), y, bf16_storage=x.dtype == torch.bfloat16)
