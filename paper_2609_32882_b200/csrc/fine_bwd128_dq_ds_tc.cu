@@ -165,7 +165,7 @@ fine_bwd128_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, Geo g, long l
           tc::tmem_ld32(lane_addr + set * 128 + col0, acc);
           tc::tmem_ld_wait();
           // a dS that left the fp16 range is an infinity and has made every channel of its query non-finite
-          if (__any_sync(0xffffffffu, any_non_finite32(acc)) && lane == 0) *a.range_flag = 1;
+          if (__any_sync(0xffffffffu, any_non_finite(acc)) && lane == 0) *a.range_flag = 1;
         } else {
 #pragma unroll
           for (int e = 0; e < 32; ++e) acc[e] = 0u;

@@ -359,13 +359,14 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         for (int t = 0; t < nt; ++t, ++tg) {
           VSA2_WAIT_PARKED(&misc->ds_ready[0], tg & 1);
           if (lane == 0) {
-#pragma unroll
+#pragma unroll 1
             for (int h = 0; h < 2; ++h) {
               const int* at = misc->ds_slot[tg % 3][h];
               if (!PACK || at[1] == kWholeBlock) {
                 if (at[0] >= 0) tc::bulk_store(a.ds + (size_t)at[0] * kSlab, ds_tile + h * kSlab, kSlab, policy);
               } else {
                 const uint32_t bytes = kSlab >> a.pk.shift;
+#pragma unroll 1
                 for (int c = 0; c < 1 << a.pk.shift; ++c)
                   if (at[c] >= 0) tc::bulk_store(a.ds + (size_t)at[c] * kSlab, ds_tile + h * kSlab + c * bytes, bytes, policy);
               }
@@ -600,6 +601,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const float inv_scale = a.ds_exp != nullptr ? pow2i(-a.ds_exp[bhk]) : 1.f, k_scale = g.scale * inv_scale;
       const size_t head = (size_t)bhk * g.S;
       if (k == 0) {                            // nothing kept: the coarse gradients only
+#pragma unroll 1
         for (int c = 0; c < 64; ++c) {
           const int l = __shfl_sync(0xffffffffu, c < 32 ? tok0 : tok1, c & 31);
           if (l < 0 || row >= D) continue;
@@ -619,32 +621,27 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       tok[32 + lane] = tok1;
       __syncwarp();
 #pragma unroll 1
-      for (int part = 0; part < 4; ++part) {   // dK tokens 0..31, 32..63, dV the same
-        const bool is_v = part >= 2;
-        float v[32];
-        {
-          const uint32_t addr = lane_addr + set * TM_SET + (is_v ? TM_DV : TM_DK) + (part & 1) * 32;
-          uint32_t x[32];
-          tc::tmem_ld32(addr, x);
-          tc::tmem_ld_wait();
-#pragma unroll
-          for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(x[c]);
-          if constexpr (SPLIT) {
-            tc::tmem_ld32(addr + 64, x);
-            tc::tmem_ld_wait();
-#pragma unroll
-            for (int c = 0; c < 32; ++c) v[c] += __uint_as_float(x[c]);
-            if (part == 3) {                   // everything has been read: the accumulators are free
-              tc::tc_fence_before();
-              __syncwarp();
-              if (lane == 0) tc::mbar_arrive(&misc->o_empty[0]);
-            }
-          }
+      for (int part = 0; part < 8; ++part) {   // dK tokens 0..15, .., 48..63, dV the same
+        const bool is_v = part >= 4;
+        const uint32_t addr = lane_addr + set * TM_SET + (is_v ? TM_DV : TM_DK) + (part & 3) * 16;
+        uint32_t x[16], lo[SPLIT ? 16 : 1];
+        tc::tmem_ld16(addr, x);
+        if constexpr (SPLIT) tc::tmem_ld16(addr + 64, lo);
+        tc::tmem_ld_wait();
+        if (SPLIT && part == 7) {              // everything has been read: the accumulators are free
+          tc::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&misc->o_empty[0]);
         }
-        const float add = is_v ? coarse[1] : coarse[0];
+        const float add = is_v ? coarse[1] : coarse[0], factor = is_v ? inv_scale : k_scale;
+        float v[16];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) v[c] = fmaf(v[c], is_v ? inv_scale : k_scale, add);
-        if (row < D) store_channels<D>(is_v ? a.dv : a.dk, g.out_f32, head, tok + (part & 1) * 32, v, row);
+        for (int c = 0; c < 16; ++c) {
+          v[c] = __uint_as_float(x[c]);
+          if constexpr (SPLIT) v[c] += __uint_as_float(lo[c]);
+          v[c] = fmaf(v[c], factor, add);
+        }
+        if (row < D) store_channels<D>(is_v ? a.dv : a.dk, g.out_f32, head, tok + (part & 3) * 16, v, row);
       }
       if constexpr (!SPLIT) {
         tc::tc_fence_before();

@@ -177,6 +177,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       const float out_scale = g.scale * pow2i(-a.ds_exp[rec.y / g.rep]);      // (rec.y / rep: batch * Hkv + KV head)
       const size_t head = (size_t)rec.y * g.S;
       if (k == 0) {                            // nothing kept: the coarse gradient only
+#pragma unroll 1
         for (int c = 0; c < 64; ++c) {
           const int l = __shfl_sync(0xffffffffu, c < 32 ? tok0 : tok1, c & 31);
           if (l >= 0 && row < D) store_out(a.dq, (head + l) * D + row, coarse_d, g.out_f32);
@@ -192,22 +193,20 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       tok[lane] = tok0;
       tok[32 + lane] = tok1;
       __syncwarp();
+      const int rows_in = packed_query(g, a.pk, i) ? 64 >> a.pk.shift : 64;       // (what lies behind a packed cube's rows is nobody's dS)
 #pragma unroll 1
-      for (int part = 0; part < 2; ++part) {
-        uint32_t x[32];
-        tc::tmem_ld32(lane_addr + set * 64 + part * 32, x);
+      for (int part = 0; part < 4; ++part) {
+        uint32_t x[16];
+        tc::tmem_ld16(lane_addr + set * 64 + part * 16, x);
         tc::tmem_ld_wait();
         // a dS that left the fp16 range is an infinity and has made every channel of its query column non-finite (one store per
         // warp: with all rows out of range one per thread took 2.7 ms for 8 heads of 720p)
-        if (packed_query(g, a.pk, i)) {       // (what lies behind a packed cube's rows is nobody's dS)
+        if (part * 16 >= rows_in) break;       // (a quarter or half of the rows)
+        if (__any_sync(0xffffffffu, row < D && any_non_finite(x)) && lane == 0) *a.range_flag = 1;
+        float v[16];
 #pragma unroll
-          for (int c = 0; c < 32; ++c) x[c] = part * 32 + c < 64 >> a.pk.shift ? x[c] : 0u;
-        }
-        if (__any_sync(0xffffffffu, row < D && any_non_finite32(x)) && lane == 0) *a.range_flag = 1;
-        float v[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) v[c] = fmaf(__uint_as_float(x[c]), out_scale, coarse_d);
-        if (row < D) store_channels<D>(a.dq, g.out_f32, head, tok + part * 32, v, row);
+        for (int c = 0; c < 16; ++c) v[c] = fmaf(__uint_as_float(x[c]), out_scale, coarse_d);
+        if (row < D) store_channels<D>(a.dq, g.out_f32, head, tok + part * 16, v, row);
       }
       tc::tc_fence_before();
       __syncwarp();

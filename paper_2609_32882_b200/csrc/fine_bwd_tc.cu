@@ -375,7 +375,7 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
           // F16: a dS that left the fp16 range went into the product as an infinity and has made every channel of its query
           // column non-finite: the result of this launch is not to be used, the fallback launch redoes it
           if constexpr (F16) {
-            if (row < D && any_non_finite32(o0)) atomicExch(a.range_flag, 1);
+            if (row < D && any_non_finite(o0)) atomicExch(a.range_flag, 1);
           }
         } else {
 #pragma unroll

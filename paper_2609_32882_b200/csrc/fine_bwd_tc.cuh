@@ -142,23 +142,25 @@ __device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int firs
   }
 }
 
-// Stores 32 values per thread -- channel `row` of 32 tokens, the warp's lanes being 32 neighbouring channels -- to the token
-// rows named by tok[0 .. 31] (shared memory, -1 = no token).  No exchange between lanes: shuffles and a transpose in shared
+// Stores 16 values per thread -- channel `row` of 16 tokens, the warp's lanes being 32 neighbouring channels -- to the token
+// rows named by tok[0 .. 15] (shared memory, -1 = no token).  No exchange between lanes: shuffles and a transpose in shared
 // memory both use the data pipe that bounds the passes, and a chain of them took the epilogue warps three times as long as
-// storing 64 bytes per warp and token.
+// storing 64 bytes per warp and token.  Sixteen tokens at a time in a rolled loop, because an epilogue's code passes through the
+// instruction cache once per item (kernels of 52 and 29 KB instead of 70 and 40 with 32 tokens): backward, us, 13 x 27 x 47 tokens, 16 heads of
+// 64 channels 728 -> 679; 8 heads on 2 with budgets 14135 -> 13693.
 template <int D>
-__device__ __forceinline__ void store_channels(void* out, int out_f32, size_t head, const int* tok, const float (&v)[32], int row) {
+__device__ __forceinline__ void store_channels(void* out, int out_f32, size_t head, const int* tok, const float (&v)[16], int row) {
   if (out_f32) {
     float* base = reinterpret_cast<float*>(out) + head * D + row;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) {
+    for (int c = 0; c < 16; ++c) {
       const int l = tok[c];
       if (l >= 0) base[(size_t)l * D] = v[c];
     }
   } else {
     bf16* base = reinterpret_cast<bf16*>(out) + head * D + row;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) {
+    for (int c = 0; c < 16; ++c) {
       const int l = tok[c];
       if (l >= 0) base[(size_t)l * D] = __float2bfloat16_rn(v[c]);
     }

@@ -109,11 +109,12 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
   asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
-// whether one of 32 accumulator values (float bits) is an infinity or not a number: x * 0 is 0 for every finite x
-__device__ __forceinline__ bool any_non_finite32(const uint32_t (&v)[32]) {
+// whether one of N accumulator values (float bits) is an infinity or not a number: x * 0 is 0 for every finite x
+template <int N>
+__device__ __forceinline__ bool any_non_finite(const uint32_t (&v)[N]) {
   float t = 0.f;
 #pragma unroll
-  for (int e = 0; e < 32; ++e) t = fmaf(__uint_as_float(v[e]), 0.f, t);
+  for (int e = 0; e < N; ++e) t = fmaf(__uint_as_float(v[e]), 0.f, t);
   return t != t;
 }
 // x -> (bf16(x), bf16(x - bf16(x))) for two values, packed like pack_bf16x2
