@@ -390,7 +390,8 @@ cudaError_t launch_fine_bwd128_dkv_tc(const Geo& g, const bf16* q, const bf16* k
 cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                   const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
                                   const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
-                                  const DsScale* scale, StatusBlock* report = nullptr);      // (report: the status block written to, if not `status`)
+                                  const DsScale* scale, StatusBlock* report = nullptr,       // (report: the status block written to, if not `status`)
+                                  bool beside = false);      // the launch that comes next is a dK/dV pass with `beside`
 bool fine_bwd_dq_uses_f16(const Geo& g);
 // Slot of StatusBlock.pad that holds the range flag of the fp16 dQ passes (the slot behind it: the fallback launch's counter)
 constexpr int kRangeFlagSlot = 8;
@@ -455,7 +456,8 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
                                    const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp,
-                                   const PackedCubes& pk = PackedCubes{}, StatusBlock* report = nullptr);
+                                   const PackedCubes& pk = PackedCubes{}, StatusBlock* report = nullptr,
+                                   bool beside = false);     // it may run beside the dQ pass launched just before it with `beside` (same inputs)
 bool fine_bwd_dkv_gqa_uses_f16(const Geo& g);
 bool fine_bwd_dkv_splits_long_columns(const Geo& g, bool split_long_columns);
 

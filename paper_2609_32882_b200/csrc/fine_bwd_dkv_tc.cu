@@ -149,7 +149,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int rep = MHA ? 1 : g.rep;
   constexpr bool STORES_DS = F16 == 1 || F16 == 2 || (SPLIT && !MHA);
   static_assert(F16 == 0 || !SPLIT, "the fp16 forms carry no pairs");
-  // The launch of the few long lists (overlap 1) lets the launch of the others (2; disjoint outputs, nothing read from the first) take
+  // The launch of the few long lists (overlap 1), or the dQ pass of the pooled problem, lets the launch of the others (2; disjoint outputs, nothing read from the first) take
   // the SMs as its CTAs leave them, once what both read is there; the second waits for the first at its end, so that what
   // follows waits for both.
   const bool second = !SPLIT && F16 == 0 && a.overlap == 2;
@@ -687,7 +687,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
                                    const float* dkc, const float* dvc, void* dk, void* dv, StatusBlock* status,
                                    cudaStream_t st, bool split_long_columns, const void* q16,
                                    const void* k16, void* v16, void* do16, const StoredDs* sd, const int* ds_exp,
-                                   const PackedCubes& pk, StatusBlock* report) {
+                                   const PackedCubes& pk, StatusBlock* report, bool beside) {
   if (g.rep > kMaxRep) return cudaErrorInvalidValue;
   CUtensorMap tq, tk, tv, tdo, tqt, tkt, tvt, tdot, tq16, tk16, tqt16, tkt16, tv16, tdo16, tvt16, tdot16;
   // GQA groups without a precision flag take the all-fp16 form when they are given scratch for fp16 copies of V and dO as
@@ -796,7 +796,7 @@ cudaError_t launch_fine_bwd_dkv_tc(const Geo& g, const bf16* q, const bf16* k, c
   }
   if (fine_bwd_dkv_wants_pair(g)) return main_pass(true, 0);
   if (!fine_bwd_dkv_splits_long_columns(g, split_long_columns))
-    return launch(false, &status->pad[3], 0, kAll, 0, 0, all, false);
+    return launch(false, &status->pad[3], 0, kAll, 0, 0, all, false, beside ? 2 : 0);
   // With the fp16 copies of Q and K: one launch in the fp16 form; the two launches below then run only if the range flag
   // came up (in the dQ pass or in this launch), on counters of their own.
   int when = 0, slot_plain = 3;

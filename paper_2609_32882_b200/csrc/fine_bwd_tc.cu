@@ -41,6 +41,7 @@ struct DqArgs {
   int* range_flag;
   int when;
   const int* ds_exp;    // null, or the exponent of the scale of dS per KV group (DsScale)
+  bool beside;          // the launch behind this one may start while this one runs (when = 0; it reads nothing of this one's)
 };
 
 template <bool SCALED>
@@ -108,7 +109,10 @@ fine_bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = misc->tmem_base;
-  if (!F16 && a.when == 0) grid_enter(false);
+  if (!F16 && a.when == 0) {
+    grid_enter(false);
+    if (a.beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   // tensor-memory columns: S^T buffers 0, 64; dP^T buffers 128, 192; dQ^T 256 (SPLIT: its low-order part at 320)
 
   if (warp < 2) {
@@ -438,7 +442,7 @@ done:
 cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, const bf16* v, const bf16* d_o,
                                   const float* lse, const float* delta, const int* row_ptr, const int* col_idx,
                                   const float* dqc, void* dq, StatusBlock* status, cudaStream_t st, void* q16, void* k16,
-                                  const DsScale* scale, StatusBlock* report) {
+                                  const DsScale* scale, StatusBlock* report, bool beside) {
   const bool f16 = fine_bwd_dq_uses_f16(g) && q16 != nullptr && k16 != nullptr && scale != nullptr;
   const bf16* qa = f16 ? reinterpret_cast<const bf16*>(q16) : q;      // (same element size and layout: the maps only move bytes)
   const bf16* ka = f16 ? reinterpret_cast<const bf16*>(k16) : k;
@@ -451,7 +455,7 @@ cudaError_t launch_fine_bwd_dq_tc(const Geo& g, const bf16* q, const bf16* k, co
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
   int* flag = &status->pad[kRangeFlagSlot];
-  DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, report != nullptr ? report : status, flag, 0, f16 ? scale->exp : nullptr};
+  DqArgs a{&status->pad[2], lse, delta, row_ptr, col_idx, dqc, dq, report != nullptr ? report : status, flag, 0, f16 ? scale->exp : nullptr, beside};
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
   const bool split = !(g.flags & VSA2_FLAG_FAST_BWD);
@@ -491,7 +495,7 @@ cudaError_t launch_fine_bwd_dq_fallback(const Geo& g, const bf16* q, const bf16*
   int sms = 0;
   cudaError_t e;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  DqArgs a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, dq, status, &status->pad[kRangeFlagSlot], 2, nullptr};
+  DqArgs a{&status->pad[kRangeFlagSlot + 1], lse, delta, row_ptr, col_idx, dqc, dq, status, &status->pad[kRangeFlagSlot], 2, nullptr, false};
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
   if (g.D == 128) VSA2_LAUNCH_DQ(128, true, false, tq, tk, tqt, tkt);
