@@ -73,7 +73,7 @@ struct FwdRowsMisc {
   uint64_t s_full[2], s_free[2];
   uint64_t p_ready[2], p_free[2];
   ItemQueue items;
-  uint64_t all_sync;               // group barrier of the 256 softmax threads
+  uint64_t m_full[2];              // reference exponents of the item with that parity
   uint32_t tmem_base;
   int abort_flag;
   uint32_t rescued;                // 1 + number of the last item that was handed to the exact kernel
@@ -157,6 +157,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       tc::mbar_init(&misc->qt_empty[s], 1);
       tc::mbar_init(&misc->o_full[s], 1);
       tc::mbar_init(&misc->o_empty[s], 128);
+      tc::mbar_init(&misc->m_full[s], 128);    // the warpgroup of tile 0
       tc::mbar_init(&misc->sums_full[s], 256);
       tc::mbar_init(&misc->tab_full[s], 32);
       tc::mbar_init(&misc->tab_free[s], 256 + 128);
@@ -175,7 +176,6 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       tc::mbar_init(&misc->p_ready[s], 128);
       tc::mbar_init(&misc->p_free[s], 1);
     }
-    tc::mbar_init(&misc->all_sync, 256);
     item_queue_init(&misc->items, 4 + 2 + 1 + 256 + 4); // lane 0 of the producers, of the issuers, of the table loader and of the epilogue warps; the softmax threads
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
@@ -391,7 +391,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     const int cq = lane & 3;
     const int row_a = quad * 16 + (lane >> 2), row_b = row_a + 8;     // the two query rows of this thread
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    uint32_t tg = 0, all_phase = 0;
+    uint32_t tg = 0;
     for (uint32_t n_all = 0;; ++n_all) {
       VSA2_NEXT_ITEM(item, n_all);
       int i, bhq;
@@ -405,14 +405,15 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       const int nt = (k + 1) >> 1;
       const uint32_t tg0 = tg;
       // Tiles with (global tile index & 1) == wg.  The owner of tile 0 takes the exact row maximum of that tile as the reference exponent of
-      // every query row; both warpgroups pick it up in front of their first tile's weights.
+      // every query row; the other waits for it in front of its first tile's weights.  (One way only: with a barrier of all 256 threads the owner
+      // waited for the other's last tile of the item before: 13 x 27 x 47 tokens, 16 heads of 64 channels 371 us against 356.)
       float2 l_a = make_float2(0.f, 0.f), l_b = l_a;       // exact sums of the two rows, even and odd columns apart
       float r_a = 0.f, r_b = 0.f;                          // and sums of the bf16 roundings
       float m_a = 0.f, m_b = 0.f;
       const int t_first = (tg0 & 1) == (uint32_t)wg ? 0 : 1;
       // KV blocks of this warpgroup's tiles: the first from the item's table, the others fetched one own tile ahead
       int ja = head[2 * t_first < k ? 2 * t_first : 0], jb = head[2 * t_first + 1 < k ? 2 * t_first + 1 : 0];
-      if (t_first >= nt) VSA2_GROUP_SYNC(&misc->all_sync, all_phase);      // (no tile of its own)
+      if (nt == 0 && t_first == 0) tc::mbar_arrive(&misc->m_full[tb]);     // (one phase per item)
       for (int t = t_first; t < nt; t += 2) {
         const uint32_t tgt = tg0 + t, buf = tgt & 1;
         const int fa = edge[ja], fb = 2 * t + 1 >= k ? kFrNone : edge[jb];
@@ -442,24 +443,26 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             }
           }
         }
-        if (t == t_first) {
-          if (t == 0) {
-            float mx_a = -INFINITY, mx_b = -INFINITY;
+        if (t == 0) {
+          float mx_a = -INFINITY, mx_b = -INFINITY;
 #pragma unroll
-            for (int n = 0; n < 16; ++n) {
-              mx_a = fmaxf(mx_a, fmaxf(__uint_as_float(sv[4 * n]), __uint_as_float(sv[4 * n + 1])));
-              mx_b = fmaxf(mx_b, fmaxf(__uint_as_float(sv[4 * n + 2]), __uint_as_float(sv[4 * n + 3])));
-            }
-            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 1));
-            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 1));
-            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 2));
-            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 2));
-            if (cq == 0) {
-              misc->m_ref[tb][row_a] = (mx_a > -INFINITY) ? mx_a * c2 : 0.f;
-              misc->m_ref[tb][row_b] = (mx_b > -INFINITY) ? mx_b * c2 : 0.f;
-            }
+          for (int n = 0; n < 16; ++n) {
+            mx_a = fmaxf(mx_a, fmaxf(__uint_as_float(sv[4 * n]), __uint_as_float(sv[4 * n + 1])));
+            mx_b = fmaxf(mx_b, fmaxf(__uint_as_float(sv[4 * n + 2]), __uint_as_float(sv[4 * n + 3])));
           }
-          VSA2_GROUP_SYNC(&misc->all_sync, all_phase);
+          mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 1));
+          mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 1));
+          mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 2));
+          mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 2));
+          m_a = (mx_a > -INFINITY) ? mx_a * c2 : 0.f;
+          m_b = (mx_b > -INFINITY) ? mx_b * c2 : 0.f;
+          if (cq == 0) {
+            misc->m_ref[tb][row_a] = m_a;
+            misc->m_ref[tb][row_b] = m_b;
+          }
+          tc::mbar_arrive(&misc->m_full[tb]);
+        } else if (t == 1) {
+          VSA2_WAIT(&misc->m_full[tb], (n_all >> 1) & 1);
           m_a = misc->m_ref[tb][row_a];
           m_b = misc->m_ref[tb][row_b];
         }
