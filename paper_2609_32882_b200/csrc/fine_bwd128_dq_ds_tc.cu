@@ -30,7 +30,7 @@ struct DqDs128 {
 struct DqDs128Misc {
   uint64_t full[4], empty[4];
   uint64_t o_full[kW2DsSets], o_empty[kW2DsSets];
-  BwdQueue queue;
+  ListQueue queue;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -56,7 +56,7 @@ fine_bwd128_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, Geo g, long l
       tc::mbar_init(&misc->o_full[s], 1);
       tc::mbar_init(&misc->o_empty[s], 4);
     }
-    bwd_queue_init(&misc->queue, 8);
+    list_queue_init(&misc->queue, 8);
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_k);
   }
@@ -210,7 +210,7 @@ fine_bwd128_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, Geo g, long l
   } else {
     Geo cubes = g;
     cubes.N = g.N / 2;
-    if (!bwd_schedule(&misc->queue, cubes, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, false,
+    if (!schedule_lists(&misc->queue, cubes, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, false,
                       a.range_flag, lane, &misc->abort_flag))
       goto done;
   }

@@ -81,7 +81,7 @@ __host__ __device__ constexpr int dkv_ring_b(int D) { return D == 64 ? 3 : kRing
 // elementwise stage (each half of the key columns): P is handed to the dV^T product before dS is formed;
 // warps 12..15 = one thread per query row of the tile: they look up the row's (head, block, token) and fetch its lse and
 // delta one tile ahead, so that the elementwise warps, which bound the pass, touch no global memory inside a tile; warp 18 =
-// scheduler (BwdQueue); warps 20..23 = epilogue.  The accumulators of dK^T and dV^T exist twice (without SPLIT), so the
+// scheduler (ListQueue); warps 20..23 = epilogue.  The accumulators of dK^T and dV^T exist twice (without SPLIT), so the
 // elementwise warps go from one KV block to the next while the epilogue warps read out and store the last one: with
 // the epilogue on the elementwise warps, 9200 of 85000 cycles of a 720p item (top-64) went by between its last tile and the
 // first of the next item (clock64 trace: 3900 epilogue, 3200 fetching the next item's record and lists, 2100 waits).
@@ -168,7 +168,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       tc::mbar_init(&misc->o_full[s], 2);                                     // two last-stage issuers
       tc::mbar_init(&misc->o_empty[s], 4);                                    // the epilogue warps
     }
-    bwd_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4 + (STORES_DS && !SPLIT && a.ds != nullptr ? 1 : 0));
+    list_queue_init(&misc->queue, 2 + 4 + 8 + 4 + 4 + (STORES_DS && !SPLIT && a.ds != nullptr ? 1 : 0));
     if (STORES_DS && !SPLIT && a.ds != nullptr) tc::mbar_init(&misc->ds_free[0], 2);     // read by the dK product and by the copy
     if (D == 64) {
       for (int s = 0; s < RA; ++s) {
@@ -346,7 +346,7 @@ fine_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   } else if (warp >= 16 && warp < 20) {
     tc::reg_dec<48>();
-    if (warp == 18 && !bwd_schedule<PACK>(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
+    if (warp == 18 && !schedule_lists<PACK>(&misc->queue, g, a.first_item, a.items, rep, a.col_ptr, a.item_counter, a.order, a.k_lo,
                                     a.k_hi, SPLIT && MHA && a.k_lo > 1, nullptr, lane, &misc->abort_flag, a.pk))
       goto done;
     if (STORES_DS && !SPLIT && warp == 19 && a.ds != nullptr) {

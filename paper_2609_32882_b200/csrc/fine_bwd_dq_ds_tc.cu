@@ -32,7 +32,7 @@ struct DqDs {
 struct DqDsMisc {
   uint64_t full[6], empty[6];
   uint64_t o_full[kDsSets], o_empty[kDsSets];
-  BwdQueue queue;
+  ListQueue queue;
   uint32_t tmem_base;
   int abort_flag;
   int tok[2][2][64];                  // raster tokens of an item's rows: per epilogue warpgroup, by parity of its items
@@ -61,7 +61,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       tc::mbar_init(&misc->o_full[s], 1);
       tc::mbar_init(&misc->o_empty[s], 4);
     }
-    bwd_queue_init(&misc->queue, 4 + 8);
+    list_queue_init(&misc->queue, 4 + 8);
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_k);
   }
@@ -213,7 +213,7 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       if (lane == 0) tc::mbar_arrive(&misc->o_empty[set]);
     }
   } else {
-    if (!bwd_schedule(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, false, a.range_flag, lane,
+    if (!schedule_lists(&misc->queue, g, a.first_item, a.items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, false, a.range_flag, lane,
                       &misc->abort_flag))
       goto done;
   }

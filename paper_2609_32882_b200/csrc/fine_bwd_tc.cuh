@@ -37,111 +37,6 @@ struct BwdTc {
   static constexpr size_t smem_bytes = OFF_MISC + MISC_BYTES + 1024;
 };
 
-// Work items of a persistent CTA with everything a role needs to know about one: {block, batch * heads index, entries of its
-// list, start of the list}, block -1 at the end.  A warp of its own (the scheduler) draws the items and looks the lists up, one
-// item ahead of the first producer: nothing of that -- an atomic and two dependent loads -- lies on another role's path,
-// and a CTA does not claim items that a CTA with less to do could start sooner.
-struct BwdQueue {
-  uint64_t full[kItemSlots], empty[kItemSlots], taken;
-  int4 rec[kItemSlots];
-};
-// `consumers`: warps that call bwd_queue_get for every item
-__device__ __forceinline__ void bwd_queue_init(BwdQueue* q, int consumers) {
-  for (int s = 0; s < kItemSlots; ++s) {
-    tc::mbar_init(&q->full[s], 1);
-    tc::mbar_init(&q->empty[s], consumers);
-  }
-  tc::mbar_init(&q->taken, 1);
-}
-// whole warp: record of the item with sequence number seq; false on a timed-out wait
-__device__ __forceinline__ bool bwd_queue_get(BwdQueue* q, uint32_t seq, int lane, int4& rec, volatile int* abort_flag) {
-  const uint32_t slot = seq % kItemSlots;
-  const bool ok = tc::mbar_wait_parked(&q->full[slot], (seq / kItemSlots) & 1, abort_flag);
-  rec = q->rec[slot];
-  __syncwarp();
-  if (lane == 0) tc::mbar_arrive(&q->empty[slot]);
-  return ok;
-}
-#define VSA2_NEXT_REC(REC, SEQ)                                                          \
-  int4 REC;                                                                              \
-  if (!bwd_queue_get(&misc->queue, (SEQ), lane, REC, &misc->abort_flag)) goto done;      \
-  if (REC.x < 0) break
-// scheduler warp: draws the items first_item .. first_item + items - 1 (in the order of `order`, if there is one) until the
-// counter runs out or `stop` (null, or a flag in global memory, looked at every fourth draw) is up.  `ptr`, `rep`: start pointers of the lists, an item has those of
-// `rep` consecutive heads; items with fewer than k_lo or more than k_hi entries are left out.
-// `sparse`: few items are in that range.  A draw then stands for 32 of them, one per lane and far apart (their lists tend to be long
-// side by side), so that passing over the others costs a 32nd of the draws.
-// PACK: the entries counted are tiles of 64 rows (a list's cubes of the cut layer are packed).
-template <bool PACK = false>
-__device__ __forceinline__ bool bwd_schedule(BwdQueue* q, const Geo& g, int first_item, int items, int rep, const int* ptr,
-                                             int* counter, const int* order, int k_lo, int k_hi, bool sparse, const int* stop, int lane,
-                                             volatile int* abort_flag, const PackedCubes& pk = PackedCubes{}) {
-  const int draws = sparse ? (items + 31) / 32 : items;
-  uint32_t drawn = 0;
-  unsigned left = 0u;             // sparse: lanes of the current draw whose items are still to be handed out
-  int4 mine;
-  for (uint32_t p = 0;; ++p) {
-    const uint32_t slot = p % kItemSlots;
-    if (p > 0 && !tc::mbar_wait_parked(&q->taken, (p - 1) & 1, abort_flag)) return false;
-    if (!tc::mbar_wait_parked(&q->empty[slot], ((p / kItemSlots) & 1) ^ 1, abort_flag)) return false;
-    int4 rec;
-    for (;;) {
-      rec = make_int4(-1, 0, 0, 0);
-      if (left != 0u) {
-        const int src = __ffs(left) - 1;
-        left &= left - 1u;
-        rec.x = __shfl_sync(0xffffffffu, mine.x, src);
-        rec.y = __shfl_sync(0xffffffffu, mine.y, src);
-        rec.z = __shfl_sync(0xffffffffu, mine.z, src);
-        rec.w = __shfl_sync(0xffffffffu, mine.w, src);
-        break;
-      }
-      int n = 0;
-      if (lane == 0) {
-        n = item_draw(drawn, counter);
-        if ((drawn & 3u) == 1u && stop != nullptr && *reinterpret_cast<const volatile int*>(stop) != 0) n = draws;
-      }
-      n = __shfl_sync(0xffffffffu, n, 0);
-      ++drawn;
-      if (n >= draws) break;
-      if (sparse) {
-        const int item = n + lane * draws;
-        mine = make_int4(-1, 0, 0, 0);
-        if (item < items) {
-          item_block(g, first_item + item, mine.y, mine.x);
-          for (int hh = 0; hh < rep; ++hh) {
-            const int* c = ptr + ((size_t)mine.y * rep + hh) * (g.N + 1) + mine.x;
-            const int beg = c[0];
-            if (hh == 0) mine.w = beg;
-            mine.z += c[1] - beg;
-          }
-        }
-        left = __ballot_sync(0xffffffffu, item < items && mine.z >= k_lo && mine.z <= k_hi);
-        continue;
-      }
-      item_block(g, order != nullptr ? order[first_item + n] : first_item + n, rec.y, rec.x);
-      int beg = 0, k = 0;
-      if (lane < rep) {      // (heads of a group are neighbours: b * Hq + hk * rep + hh)
-        const int* c = ptr + ((size_t)rec.y * rep + lane) * (g.N + 1) + rec.x;
-        beg = c[0];
-        k = c[1] - beg;
-        if (PACK) {
-          const int full = pk.full[((size_t)rec.y * rep + lane) * g.N + rec.x], text = g.N - g.Nvid;
-          k = full + text + (k - text - full + (1 << pk.shift) - 1 >> pk.shift);
-        }
-      }
-      rec.z = __reduce_add_sync(0xffffffffu, k);
-      rec.w = __shfl_sync(0xffffffffu, beg, 0);
-      if (rec.z >= k_lo && rec.z <= k_hi) break;
-    }
-    if (lane == 0) {
-      q->rec[slot] = rec;
-      tc::mbar_arrive(&q->full[slot]);
-    }
-    if (rec.x < 0) return true;
-  }
-}
-
 // Stores 16 values per thread -- channel `row` of 16 tokens, the warp's lanes being 32 neighbouring channels -- to the token
 // rows named by tok[0 .. 15] (shared memory, -1 = no token).  No exchange between lanes: shuffles and a transpose in shared
 // memory both use the data pipe that bounds the passes, and a chain of them took the epilogue warps three times as long as
@@ -194,7 +89,7 @@ struct BwdMisc {
   uint64_t stat_full, stat_free;                            // dK/dV pass: the per-row statistics of a tile
   union {                                                   // work items of this CTA
     ItemQueue items;                                        // dQ pass (see tc_attn.cuh)
-    BwdQueue queue;                                         // dK/dV pass
+    ListQueue queue;                                         // dK/dV pass
   };
   uint32_t tmem_base;
   int abort_flag;

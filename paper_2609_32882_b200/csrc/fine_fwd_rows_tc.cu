@@ -26,7 +26,7 @@
 // 2^-9 relative, reached the backward through delta = rowsum(dO * O) and was its largest error on sharply peaked rows).
 //
 // Roles (640 threads): warps 0..3 = TMA producers (K / V ring x first / second block of a pair; warp 0 also brings the Q
-// tile and schedules the CTA's work items), warp 4 = issuer of S, warp 5 = issuer of O, warp 6 = per-item tables, warps 8..15 = two
+// tile), warp 4 = issuer of S, warp 5 = issuer of O, warp 6 = per-item tables, warp 7 = scheduler (ListQueue), warps 8..15 = two
 // softmax warpgroups that alternate tiles, warps 16..19 = Q of the next block into tensor memory, then the epilogue of the present one
 // while the softmax warps are at the next.  Persistent CTAs draw query blocks from a global counter.  Every wait is bounded.
 //
@@ -36,6 +36,9 @@
 // in the softmax warps, selects in a masked copy of the loop, Q from shared memory) -> after: 9 x 30 x 45 tokens, 24 heads, top-16 514 -> 436;
 // 13 x 27 x 47, 16 heads of 64 channels, top-24 484 -> 362; 480p, 12 heads on 3, top-78 1688 -> 1573; 720p, 5 heads with text 1899 -> 1772;
 // 10 heads, top-128 4958 -> 4654.  (Epilogue and Q alone: 573, 481, 1602, 1877, 4789: more code beside the loop.)
+// And nobody looks up an item: with the item's number alone, and row pointers read by every role, 2700 cycles went by between the last product
+// of a block and the first of the next.  The same calls, before -> with the scheduler's records: 406 -> 365, 356 -> 340, 1571 -> 1532, 1777 -> 1736,
+// 4692 -> 4665.
 #include "tc_attn.cuh"
 
 namespace vsa2 {
@@ -72,7 +75,7 @@ struct FwdRowsMisc {
   uint64_t v_full[kFrVSlots], v_empty[kFrVSlots];
   uint64_t s_full[2], s_free[2];
   uint64_t p_ready[2], p_free[2];
-  ItemQueue items;
+  ListQueue queue;
   uint64_t m_full[2];              // reference exponents of the item with that parity
   uint32_t tmem_base;
   int abort_flag;
@@ -85,7 +88,6 @@ struct FwdRowsMisc {
   alignas(16) float oc[2][128];    // coarse output row of the query cube, by item parity
   int tok[2][64];                  // raster token of each query row (-1 = padding), by item parity
   float gate[2][64];
-  int list_k[2], list_beg[2];      // length and start of the item's list of KV blocks
   int list_head[2][4];             // its first four entries (tiles 0 and 1)
 };
 static_assert(sizeof(FwdRowsMisc) <= 10240, "misc region too small");
@@ -176,7 +178,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       tc::mbar_init(&misc->p_ready[s], 128);
       tc::mbar_init(&misc->p_free[s], 1);
     }
-    item_queue_init(&misc->items, 4 + 2 + 1 + 256 + 4); // lane 0 of the producers, of the issuers, of the table loader and of the epilogue warps; the softmax threads
+    list_queue_init(&misc->queue, 4 + 2 + 1 + 8 + 4);   // producers, issuers, table loader, softmax warps, epilogue warps
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_k);
@@ -213,24 +215,14 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       unsigned char* ring = smem + (which == 0 ? 0 : kFrKSlots * C::SLOT);
       const int my_h = lane;
       const bool issuer = lane < C::DH;
-      uint32_t tg = 0, n_items = 0, published = 0;
+      uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        // warp 0, lane 0 is the CTA's scheduler
-        int item = 0;
-        if (lane == 0) {
-          if (warp == 0 && !item_publish_ahead(&misc->items, seq, published, a.item_counter, total_items, &misc->abort_flag)) item = -2;
-          else item = item_get(&misc->items, seq, &misc->abort_flag);
-        }
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item == -2) goto done;
-        if (item < 0) break;
-        int i, bhq;
-        item_block(g, item, bhq, i);
-        const int b = bhq / g.Hq, hq = bhq % g.Hq, bhk = b * g.Hkv + hq / g.rep;
-        const int beg = a.row_ptr[(size_t)bhq * (g.N + 1) + i], end = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1];
-        const int k = end - beg;
+        VSA2_NEXT_REC(rec, seq);
+        if (warp == 0 && lane == 0) tc::mbar_arrive(&misc->queue.taken);
+        const int i = rec.x, bhq = rec.y, k = rec.z;
         if (k == 0) continue;
-        const int* cols = a.col_idx + (size_t)bhq * g.nnz_cap + beg;
+        const int b = bhq / g.Hq, hq = bhq % g.Hq, bhk = b * g.Hkv + hq / g.rep;
+        const int* cols = a.col_idx + (size_t)bhq * g.nnz_cap + rec.w;
         if (warp == 0) {
           int c1, c2, c3;
           block_box(g, i, c1, c2, c3);
@@ -270,16 +262,9 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       const uint32_t slot0 = tc::smem_u32(smem);
       uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        int item = 0;
-        if (lane == 0) item = item_get(&misc->items, seq, &misc->abort_flag);
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item == -2) goto done;
-        if (item < 0) break;
-        int i, bhq;
-        item_block(g, item, bhq, i);
-        const int k = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] - a.row_ptr[(size_t)bhq * (g.N + 1) + i];
-        if (k == 0) continue;
-        const int nt = (k + 1) >> 1;
+        VSA2_NEXT_REC(rec, seq);
+        const int nt = (rec.z + 1) >> 1;
+        if (nt == 0) continue;
         const uint32_t qb = n_items & 1, tm_q_op = tmem_base + C::TM_Q + qb * 64;
         VSA2_WAIT(&misc->qt_full[qb], (n_items >> 1) & 1);
         for (int t = 0; t < nt; ++t, ++tg) {
@@ -309,16 +294,9 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       const uint32_t slot0 = tc::smem_u32(smem) + kFrKSlots * C::SLOT;
       uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        int item = 0;
-        if (lane == 0) item = item_get(&misc->items, seq, &misc->abort_flag);
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item == -2) goto done;
-        if (item < 0) break;
-        int i, bhq;
-        item_block(g, item, bhq, i);
-        const int k = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] - a.row_ptr[(size_t)bhq * (g.N + 1) + i];
-        if (k == 0) continue;
-        const int nt = (k + 1) >> 1;
+        VSA2_NEXT_REC(rec, seq);
+        const int nt = (rec.z + 1) >> 1;
+        if (nt == 0) continue;
         const uint32_t ob_ = n_items & 1, acc = tmem_base + C::TM_O + ob_ * 128;
         VSA2_WAIT(&misc->o_empty[ob_], ((n_items >> 1) & 1) ^ 1);      // the accumulator of the block before the last was read out
         for (int t = 0; t < nt; ++t, ++tg) {
@@ -346,17 +324,11 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       // raster token and gate of every query row, coarse output row of the cube (global loads kept off their critical path)
       const bool coarse = !(g.flags & VSA2_FLAG_NO_COARSE) && a.gate != nullptr;
       for (uint32_t seq = 0;; ++seq) {
-        int item = 0;
-        if (lane == 0) item = item_get(&misc->items, seq, &misc->abort_flag);
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item == -2) goto done;
-        if (item < 0) break;
-        int i, bhq;
-        item_block(g, item, bhq, i);
+        VSA2_NEXT_REC(rec, seq);
+        const int i = rec.x, bhq = rec.y;
         const uint32_t tb = seq & 1;
         const bool video = !block_is_text(g, i);      // text queries take no part in the coarse branch or the gate
-        const int beg_ = a.row_ptr[(size_t)bhq * (g.N + 1) + i], k_ = a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] - beg_;
-        const int head_ = (lane < 4 && lane < k_) ? a.col_idx[(size_t)bhq * g.nnz_cap + beg_ + lane] : 0;
+        const int head_ = (lane < 4 && lane < rec.z) ? a.col_idx[(size_t)bhq * g.nnz_cap + rec.w + lane] : 0;
         int l2[2];
         float g2[2], oc4[4];
 #pragma unroll
@@ -376,12 +348,11 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
 #pragma unroll
         for (int r = 0; r < 4; ++r) misc->oc[tb][lane + 32 * r] = oc4[r];
         if (lane < 4) misc->list_head[tb][lane] = head_;
-        if (lane == 0) {
-          misc->list_k[tb] = k_;
-          misc->list_beg[tb] = beg_;
-        }
         tc::mbar_arrive(&misc->tab_full[tb]);
       }
+    } else if (!schedule_lists(&misc->queue, g, 0, total_items, 1, a.row_ptr, a.item_counter, nullptr, 0, 0x7fffffff, false, nullptr, lane,
+                               &misc->abort_flag)) {      // warp 7
+      goto done;
     }
   } else if (warp < 16) {
     // ------------------------------------------------------------------ softmax (2 x 128 threads)
@@ -393,15 +364,12 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     uint32_t tg = 0;
     for (uint32_t n_all = 0;; ++n_all) {
-      VSA2_NEXT_ITEM(item, n_all);
-      int i, bhq;
-      item_block(g, item, bhq, i);
+      VSA2_NEXT_REC(rec, n_all);
       const int tb = n_all & 1;
       VSA2_WAIT(&misc->tab_full[tb], (n_all >> 1) & 1);  // the item's tables (loaded one item ahead by warp 6)
-      const int k = misc->list_k[tb];
-      const int* cols = a.col_idx + (size_t)bhq * g.nnz_cap + misc->list_beg[tb];
+      const int k = rec.z;
+      const int* cols = a.col_idx + (size_t)rec.y * g.nnz_cap + rec.w;
       const int* head = misc->list_head[tb];
-      (void)i;
       const int nt = (k + 1) >> 1;
       const uint32_t tg0 = tg;
       // Tiles with (global tile index & 1) == wg.  The owner of tile 0 takes the exact row maximum of that tile as the reference exponent of
@@ -511,18 +479,14 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
     const int row_a = quad * 16 + (lane >> 2), row_b = row_a + 8;     // the two query rows of this thread
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     uint32_t n_staged = 0, n_items = 0;
-    // the next item's Q tile, if the item keeps anything (word 4 n + cq of a row is word cq of its 16-byte chunk n); its number
-    auto next_item = [&](uint32_t seq) -> int {
-      int item = 0;
-      if (lane == 0) item = item_get(&misc->items, seq, &misc->abort_flag);
-      item = __shfl_sync(0xffffffffu, item, 0);
-      if (item < 0) return item;
-      int i, bhq;
-      item_block(g, item, bhq, i);
-      if (a.row_ptr[(size_t)bhq * (g.N + 1) + i + 1] == a.row_ptr[(size_t)bhq * (g.N + 1) + i]) return item;
+    // the next item's record, and its Q tile, if the item keeps anything (word 4 n + cq of a row is word cq of its 16-byte chunk n); false on a
+    // timed-out wait
+    auto next_item = [&](uint32_t seq, int4& rec) -> bool {
+      if (!list_queue_get(&misc->queue, seq, lane, rec, &misc->abort_flag)) return false;
+      if (rec.x < 0 || rec.z == 0) return true;
       const uint32_t qb = n_staged & 1;
-      if (!tc::mbar_wait_parked(&misc->q_full, n_staged & 1, &misc->abort_flag)) return -2;
-      if (!tc::mbar_wait_parked(&misc->qt_empty[qb], ((n_staged >> 1) & 1) ^ 1, &misc->abort_flag)) return -2;
+      if (!tc::mbar_wait_parked(&misc->q_full, n_staged & 1, &misc->abort_flag)) return false;
+      if (!tc::mbar_wait_parked(&misc->qt_empty[qb], ((n_staged >> 1) & 1) ^ 1, &misc->abort_flag)) return false;
       tc::tc_fence_after();
 #pragma unroll 1
       for (int h = 0; h < C::DH; ++h) {
@@ -540,18 +504,15 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       tc::tc_fence_before();
       tc::mbar_arrive(&misc->qt_full[qb]);
       ++n_staged;
-      return item;
+      return true;
     };
-    int item = next_item(0);
-    for (uint32_t n_all = 0;; ++n_all) {
-      if (item == -2) goto done;
-      if (item < 0) break;
-      const int item_next = next_item(n_all + 1);
-      int i, bhq;
-      item_block(g, item, bhq, i);
+    int4 rec, rec_next;
+    if (!next_item(0, rec)) goto done;
+    for (uint32_t n_all = 0; rec.x >= 0; ++n_all) {
+      if (!next_item(n_all + 1, rec_next)) goto done;
+      const int bhq = rec.y, k = rec.z;
       const int tb = n_all & 1;
       VSA2_WAIT_PARKED(&misc->tab_full[tb], (n_all >> 1) & 1);
-      const int k = misc->list_k[tb];
       VSA2_WAIT_PARKED(&misc->sums_full[tb], (n_all >> 1) & 1);
       const uint32_t ob_ = n_items & 1;
       float inv_a = 0.f, inv_b = 0.f;
@@ -569,7 +530,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const bool bad = !(la > 1e-30f && la < 1e30f && ra > 1e-30f) || !(lb > 1e-30f && lb < 1e30f && rb > 1e-30f);
         if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued, n_all + 1) != n_all + 1) {
           const int slot = atomicAdd(a.rescue_count, 1);
-          if (slot < a.rescue_cap) a.rescue_items[slot] = item;
+          if (slot < a.rescue_cap) a.rescue_items[slot] = block_item(g, bhq, rec.x);
           else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);
         }
         VSA2_WAIT_PARKED(&misc->o_full[ob_], (n_items >> 1) & 1);
@@ -646,7 +607,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       }
       tc::mbar_arrive(&misc->tab_free[tb]);
       if (k > 0) ++n_items;
-      item = item_next;
+      rec = rec_next;
     }
   }
 
