@@ -20,9 +20,51 @@ struct BwdPrepArgs {
   int lists_per_head;                                            // blocks of 8 columns
 };
 
+// Places of the entries e0, e0 + 32, .. of column j of a head: U searches at once
+template <int U>
+__device__ __forceinline__ void find_places(const Geo& g, const int* rp, const int* ci, const int* list, int j, int e0, int end, int (&row)[U], int (&place)[U]) {
+  int lo[U], hi[U], open = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) row[u] = e0 + 32 * u < end ? list[e0 + 32 * u] : -1;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    lo[u] = hi[u] = 0;
+    if (row[u] >= 0) {                          // the entry j is in [lo, hi]
+      lo[u] = rp[row[u]];
+      hi[u] = rp[row[u] + 1] - 1;
+    }
+  }
+  if (j >= g.Nvid) {                            // a text block: the last ones of every list
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int at = hi[u] + 1 - (g.N - j);
+      if (row[u] >= 0 && at >= lo[u] && ci[at] == j) lo[u] = hi[u] = at;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) open |= lo[u] < hi[u];
+  while (open) {
+    open = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (lo[u] < hi[u]) {
+        const int mid = (lo[u] + hi[u]) >> 1;
+        if (ci[mid] < j) lo[u] = mid + 1;
+        else hi[u] = mid;
+      }
+      open |= lo[u] < hi[u];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) place[u] = lo[u];
+}
+
 // One warp per column of the block map.  Place of every entry of the column's list in the row lists of its head: pos[bh][e] for entry
 // e of row_idx (both kinds of lists ascend); and the entries in front of the cubes of a cut last layer -- or, of a list that does not have
 // them at its end, all but the text blocks (nothing of it is packed then).
+// A search is a chain of loads and a column can hold every query (the text blocks' do), so a lane has four under way at once where there are more
+// than 32 entries, and text blocks are looked for where they lie.  The launch, us, one search at a time / this: 720p, 5 heads with text
+// 182 / 71; 480p, 12 heads on 3 71 / 56; 8 heads on 2 with budgets 150 / 125.
 __device__ __forceinline__ void prep_lists(const BwdPrepArgs& a, int block) {
   const Geo& g = a.g;
   const PrepLists& l = a.lists;
@@ -36,18 +78,24 @@ __device__ __forceinline__ void prep_lists(const BwdPrepArgs& a, int block) {
   const int* list = l.row_idx + (size_t)bh * cap;
   const int beg = l.col_ptr[(size_t)bh * (g.N + 1) + j], end = l.col_ptr[(size_t)bh * (g.N + 1) + j + 1], video_end = end - (g.N - g.Nvid);
   int n = 0, last = -1;                       // entries before the layer, and the last of them
-  for (int e = beg + lane; e < end; e += 32) {
-    const int i = list[e];
-    int lo = rp[i], hi = rp[i + 1] - 1;       // the entry j is in [lo, hi]
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (ci[mid] < j) lo = mid + 1;
-      else hi = mid;
-    }
-    l.pos[(size_t)bh * cap + e] = min(lo, (int)cap - 1);      // (column lists that are not the row lists' transpose stay inside the scratch)
+  auto store = [&](int e, int i, int place) {
+    if (e >= end) return;
+    l.pos[(size_t)bh * cap + e] = min(place, (int)cap - 1);      // (column lists that are not the row lists' transpose stay inside the scratch)
     if (e < video_end && i < l.first) {
       ++n;
       last = e - beg;
+    }
+  };
+  if (end - beg <= 32) {
+    int row[1], place[1];
+    find_places(g, rp, ci, list, j, beg + lane, end, row, place);
+    store(beg + lane, row[0], place[0]);
+  } else {
+    for (int e0 = beg + lane; e0 < end; e0 += 128) {
+      int row[4], place[4];
+      find_places(g, rp, ci, list, j, e0, end, row, place);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) store(e0 + 32 * u, row[u], place[u]);
     }
   }
   if (l.full == nullptr) return;
