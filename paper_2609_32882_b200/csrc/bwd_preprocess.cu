@@ -8,13 +8,18 @@
 namespace vsa2 {
 
 // One CTA of 256 threads per 64-token block: a thread has a 16-byte channel chunk of one token in 256 / (D / 8), two tokens at a time
-// (six loads in flight; four CTAs per SM); the D / 8 threads of a token reduce its two row sums with shuffles.  The sum
-// gate_l dO_l runs over the tokens in order, so the dO rows are left in shared memory for one thread per channel.  (With
+// (six loads in flight; four CTAs per SM, five with 64 channels); the D / 8 threads of a token reduce its two row sums with shuffles.  The sum
+// gate_l dO_l runs over the tokens in PARTS parts side by side, so the dO rows are left in shared memory.  (With
 // one thread per chunk walking the block's tokens a small problem waited for sixteen rounds of loads, 21 us.)
+// Issue slots (78 %) bound it before memory, so sums and products go two values at a time, and all warps take part in the sum over the tokens (one
+// thread per channel walked 64 of them while half the CTA waited).  us, before -> after: 720p, 40 heads 685 -> 647; 480p, 12 heads 82 -> 78; 13 x 27 x 47
+// tokens, 16 heads of 64 channels 34.5 -> 29.1 (four CTAs: 32); 2048-token clip 7.1 -> 6.5.  Five CTAs with 128 channels: 688, 84.
 // F32: the type of O.  (As a branch in the loop it cost the loads of a token their place ahead of the first use: 720p, 40 heads, 646 us
 // against 533 = 4.5 TB/s.)
+__device__ __forceinline__ uint32_t word(const uint4& v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
+__device__ __forceinline__ float2 bf16_pair(uint32_t x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
 template <int D, bool F32>
-__global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o, const void* o,
+__global__ void __launch_bounds__(256, D == 64 ? 5 : 4) bwd_preprocess_kernel(const bf16* d_o, const void* o,
                                                              const bf16* o_res,
                                                              const float* gate,
                                                              const float* oc_hat, Geo g,
@@ -26,7 +31,9 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
   constexpr int PAR = 256 / CH;            // tokens at a time
   constexpr int TOK = 2;                   // tokens in flight per thread
   __shared__ __align__(16) bf16 rows[kBlockTokens * D];
-  __shared__ float gates[kBlockTokens];
+  __shared__ __align__(16) float gates[kBlockTokens];
+  constexpr int PARTS = 512 / D;           // parts of a block's tokens in the sum of gate * dO
+  __shared__ __align__(8) float part_sum[PARTS][D];
   __shared__ unsigned warp_max[2][8];
   __shared__ float row_sum[D / 32];
   if (clear != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < sizeof(StatusBlock) / 4)
@@ -80,35 +87,18 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
       const unsigned d2_max = __vmaxu2(__vmaxu2(dv[u].x & 0x7fff7fffu, dv[u].y & 0x7fff7fffu),
                                        __vmaxu2(dv[u].z & 0x7fff7fffu, dv[u].w & 0x7fff7fffu));
       unsigned o_max = 0u;
-      float ov[8], dd[8];
-      const __nv_bfloat162* d2 = reinterpret_cast<const __nv_bfloat162*>(&dv[u]);
+      float2 oo = make_float2(0.f, 0.f), oc = oo;      // even and odd channels apart
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(d2[e]);
-        dd[2 * e] = f.x; dd[2 * e + 1] = f.y;
+        const float2 dd = bf16_pair(word(dv[u], e));
+        float2 ov;
+        if constexpr (F32) ov = make_float2(__uint_as_float(word(ov4[u][e >> 1], 2 * (e & 1))), __uint_as_float(word(ov4[u][e >> 1], 2 * (e & 1) + 1)));
+        else ov = __fadd2_rn(bf16_pair(word(ov4[u][0], e)), bf16_pair(word(ov4[u][1], e)));     // (no residual: zero)
+        oo = __ffma2_rn(dd, ov, oo);
+        oc = __ffma2_rn(dd, make_float2(ocv[2 * e], ocv[2 * e + 1]), oc);
+        o_max = max(max(o_max, __float_as_uint(ov.x) & 0x7fff0000u), __float_as_uint(ov.y) & 0x7fff0000u);
       }
-      if constexpr (F32) {
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          ov[4 * e] = __uint_as_float(ov4[u][e].x); ov[4 * e + 1] = __uint_as_float(ov4[u][e].y);
-          ov[4 * e + 2] = __uint_as_float(ov4[u][e].z); ov[4 * e + 3] = __uint_as_float(ov4[u][e].w);
-        }
-      } else {
-        const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&ov4[u][0]);
-        const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(&ov4[u][1]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 f = __bfloat1622float2(o2[e]), r = __bfloat1622float2(r2[e]);     // (no residual: zero)
-          ov[2 * e] = f.x + r.x; ov[2 * e + 1] = f.y + r.y;
-        }
-      }
-      float s_oo = 0.f, s_oc = 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        s_oo = fmaf(dd[e], ov[e], s_oo);
-        s_oc = fmaf(dd[e], ocv[e], s_oc);
-        o_max = max(o_max, __float_as_uint(ov[e]) & 0x7fff0000u);
-      }
+      float s_oo = oo.x + oo.y, s_oc = oc.x + oc.y;
       most = __vmaxu2(most, o_max | max(d2_max >> 16, d2_max & 0xffffu));
 #pragma unroll
       for (int off = CH / 2; off >= 1; off >>= 1) {
@@ -132,10 +122,26 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_kernel(const bf16* d_o,
     if (threadIdx.x == 0) absmax[bhq * g.N + i] = make_float2(__uint_as_float(dm), __uint_as_float(om));
   }
   if (!coarse) return;
+  {
+    constexpr int PT = kBlockTokens / PARTS;
+    const int c = threadIdx.x % (D / 2), part = threadIdx.x / (D / 2);
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int p = 0; p < PT; p += 4) {
+      const float4 g4 = *reinterpret_cast<const float4*>(gates + part * PT + p);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float w = u == 0 ? g4.x : u == 1 ? g4.y : u == 2 ? g4.z : g4.w;
+        acc = __ffma2_rn(make_float2(w, w), bf16_pair(*reinterpret_cast<const uint32_t*>(rows + (part * PT + p + u) * D + 2 * c)), acc);
+      }
+    }
+    *reinterpret_cast<float2*>(&part_sum[part][2 * c]) = acc;
+  }
+  __syncthreads();
   if (threadIdx.x < D) {
-    float acc = 0.f;
-#pragma unroll 16
-    for (int p = 0; p < kBlockTokens; ++p) acc = fmaf(gates[p], __bfloat162float(rows[p * D + threadIdx.x]), acc);
+    float acc = part_sum[0][threadIdx.x];
+#pragma unroll
+    for (int q = 1; q < PARTS; ++q) acc += part_sum[q][threadIdx.x];
     const size_t at = (bhq * g.Nvid + i) * D + threadIdx.x;
     if (d_oc_hat != nullptr) d_oc_hat[at] = acc;
     if (do_c != nullptr) {
