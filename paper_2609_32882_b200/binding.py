@@ -143,10 +143,18 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _current_stream():
+    """Handle of the calling thread's current stream, without the Stream object (0.3 us instead of 3.2; a toy grid's calls wait for the host)."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
@@ -352,27 +360,42 @@ class Vsa2Attention:
                    scratch=self._scratch("route_scratch_bytes", q.device, stream))
 
     def forward(self, q, k, v, gate, o=None, lse=None, stream=None):
-        torch, p = self.torch, self.p
+        p = self.p
         if o is None:
-            o = torch.empty(q.shape, dtype=self.out_torch_dtype, device=q.device)
+            o = self._empty_like(q, q.device)
         if lse is None:
-            lse = torch.empty(q.shape[:-1], dtype=torch.float32, device=q.device)
+            lse = self._empty_f32(q, q.shape[:-1])
         vsa2_attn_fwd(p, q, k, v, gate, self.map, o, lse, self.saved, self.ws_fwd, stream=stream)
         return o, lse
 
     def backward(self, q, k, v, gate, o, lse, d_o, dq=None, dk=None, dv=None, dgate=None, stream=None):
-        torch, p = self.torch, self.p
+        p = self.p
         if dq is None:
-            dq = torch.empty(q.shape, dtype=self.out_torch_dtype, device=q.device)
+            dq = self._empty_like(q, q.device)
         if dk is None:
-            dk = torch.empty(k.shape, dtype=self.out_torch_dtype, device=q.device)
+            dk = self._empty_like(k, q.device)
         if dv is None:
-            dv = torch.empty(v.shape, dtype=self.out_torch_dtype, device=q.device)
+            dv = self._empty_like(v, q.device)
         if dgate is None:      # video tokens only (text tokens have no gate)
-            dgate = torch.empty(q.shape[:-2] + (self.sizes.seq_len,), dtype=torch.float32, device=q.device)
+            dgate = self._empty_f32(q, q.shape[:-2] + (self.sizes.seq_len,))
         vsa2_attn_bwd(p, q, k, v, gate, self.map, o, lse, self.saved, d_o, dq, dk, dv, dgate, self.ws_bwd, stream=stream,
                       scratch=self._scratch("bwd_scratch_bytes", q.device, stream))
         return dq, dk, dv, dgate
+
+    # A toy grid's calls wait for the host, and torch.empty takes 3.3 us: empty_like takes 1.5 (and lays out alike what is contiguous), new_empty
+    # 2.4.  With the stream's plain handle (_current_stream) a training pass of 256 tokens takes 79 us instead of 93, of 2048 tokens 141 instead of 152.
+    def _empty_f32(self, x, shape):
+        torch = self.torch
+        if type(x) is torch.Tensor:
+            return x.new_empty(shape, dtype=torch.float32)
+        return torch.empty(shape, dtype=torch.float32, device=x.device)
+
+    def _empty_like(self, x, device):
+        """An output tensor (contiguous, in the output type) of the shape of x."""
+        torch = self.torch
+        if type(x) is torch.Tensor and x.is_contiguous() and x.device == device:
+            return torch.empty_like(x, dtype=self.out_torch_dtype)
+        return torch.empty(x.shape, dtype=self.out_torch_dtype, device=device)
 
     def _scratch(self, size, device, stream):
         """Scratch for one call of the bytes in attribute `size`, allocated on the stream the call runs on (its memory is then reused in
