@@ -11,15 +11,22 @@
 // fine_fwd_rows_tc.cu) are thread-local scalars.
 //
 // Tensor memory (512 columns): two S buffers (2 x 128), two P buffers (2 x 64 columns of bf16 pairs), O (D columns).
-// Roles (512 threads): warps 0..3 = TMA producers (K / V ring x first / second block of a pair; warp 0 also brings the Q
-// pair and schedules the CTA's work items), warp 4 = issuer of S, warp 5 = issuer of O, warp 6 = loader of the per-item
-// tables, warps 8..15 = two softmax + epilogue warpgroups that alternate tiles (thread r of a warpgroup owns query row r).
+// Roles (640 threads): warps 0..3 = TMA producers (K / V ring x first / second block of a pair; warp 0 also brings the Q
+// pair), warp 4 = issuer of S, warp 5 = issuer of O, warp 6 = loader of the per-item
+// tables, warp 7 = scheduler (ListQueue), warps 8..15 = two softmax warpgroups that alternate tiles (thread r of a warpgroup owns query
+// row r), warps 16..19 = epilogue, while the softmax warps are at the next item.
 // Persistent CTAs draw items from a global counter.  Every wait is bounded.
+// (With the epilogue on the softmax warps, three barriers of both warpgroups and a lookup of the list by every role, the tensor pipe waited some
+// 4000 cycles an item.  Forward calls, us, that / this: 480p with one map for 4 heads 1094 / 1061; 219,600 tokens, 10 heads 10673 / 10411;
+// 435,600 tokens 21131 / 20670.)
 #include "tc_attn.cuh"
 
 namespace vsa2 {
 
-constexpr int kF2Threads = 512;
+constexpr int kF2Threads = 640;
+// registers a thread: the launch allocates 96; the softmax warps take what the service warps leave
+constexpr int kF2ServiceRegs = 48, kF2SoftmaxRegs = 144, kF2Regs = 256 * kF2ServiceRegs + 256 * kF2SoftmaxRegs + 128 * 96;
+static_assert(kF2Regs == kF2Threads * 96, "the shares have to fit the launch");
 constexpr int kF2KSlots = 3;
 constexpr int kF2VSlots = 2;
 constexpr int kF2MaxCubes = 8192;
@@ -30,33 +37,32 @@ struct FwdRows2 {
   static constexpr uint32_t SLOT = 2 * DH * kSlab;     // a K, V or Q pair: [channel half][block A | block B]
   static constexpr uint32_t OFF_Q = (kF2KSlots + kF2VSlots) * SLOT;
   static constexpr uint32_t OFF_MISC = OFF_Q + SLOT;
-  static constexpr uint32_t MISC_BYTES = 8192;
+  static constexpr uint32_t MISC_BYTES = 10240;
   static constexpr uint32_t TM_S = 0, TM_P = 256, TM_O = 384;
   static size_t smem_bytes(int n_blocks) { return OFF_MISC + MISC_BYTES + ((size_t)n_blocks + 15) / 16 * 16 + 1024; }
 };
 
 struct FwdRows2Misc {
   uint64_t q_full, q_empty, o_full, o_empty;
-  uint64_t tab_full[2], tab_free[2];
+  uint64_t tab_full[2], tab_free[2];   // per-item tables (tok, gate, oc, first list entries) of the item with that parity
+  uint64_t m_full[2], sums_full[2];    // its reference exponents, its row sums
   uint64_t k_full[kF2KSlots], k_empty[kF2KSlots];
   uint64_t v_full[kF2VSlots], v_empty[kF2VSlots];
   uint64_t s_full[2], s_free[2];
   uint64_t p_ready[2], p_free[2];
-  ItemQueue items;
-  uint64_t all_sync;               // group barrier of the 256 softmax threads
+  ListQueue queue;
   uint32_t tmem_base;
   int abort_flag;
-  int rescue_flag[2];              // per member of the item
+  uint32_t rescued[2];             // per member: 1 + number of the last item that was handed to the exact kernel
   unsigned long long vmask[17];    // [table row of a block]: which of its 64 positions hold tokens
-  alignas(16) float m_ref[128];    // per query row: reference exponent (log2 units)
-  float red[2][2][128];            // [warpgroup][exact sum | sum of the bf16 roundings][query row]
+  float m_ref[2][128];             // by item parity, per query row: reference exponent (log2 units)
+  float red[2][2][2][128];         // [item parity][warpgroup][exact sum | sum of the bf16 roundings][query row]
   alignas(16) float oc[2][2][128]; // [item parity][member][channel]: coarse output row of the member's cube
   int tok[2][128];                 // [item parity][query row]: row of the token tensors (-1 = padding)
   float gate[2][128];
-  int list_k[2], list_beg[2];
   int list_head[2][4];
 };
-static_assert(sizeof(FwdRows2Misc) <= 8192, "misc region too small");
+static_assert(sizeof(FwdRows2Misc) <= 10240, "misc region too small");
 
 struct FwdRows2Args {
   int pair_heads;       // 0: an item is a query cube of 128 tokens (two half-cubes of one head); 1: an item is one query
@@ -110,6 +116,7 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int total_items = g.batch * g.Hq * g.N / 2;
   const float c2 = g.scale * 1.4426950408889634f;
+  const int dh = a.pair_heads ? 1 : 0, di = 1 - dh;              // (PairItem)
 
   for (int n = tid; n < g.N; n += blockDim.x) edge[n] = (unsigned char)cube_edge_flags(g, n);
   if (tid < 16) {
@@ -124,13 +131,16 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   if (tid == 0) {
     misc->abort_flag = 0;
     misc->vmask[16] = 0ull;
+    misc->rescued[0] = misc->rescued[1] = 0;
     tc::mbar_init(&misc->q_full, 1);
     tc::mbar_init(&misc->q_empty, 1);
     tc::mbar_init(&misc->o_full, 1);
-    tc::mbar_init(&misc->o_empty, 256);
+    tc::mbar_init(&misc->o_empty, 128);
     for (int s = 0; s < 2; ++s) {
       tc::mbar_init(&misc->tab_full[s], 32);
-      tc::mbar_init(&misc->tab_free[s], 256);
+      tc::mbar_init(&misc->tab_free[s], 256 + 128);
+      tc::mbar_init(&misc->m_full[s], 128);    // the warpgroup of tile 0
+      tc::mbar_init(&misc->sums_full[s], 256);
       tc::mbar_init(&misc->s_full[s], 1);
       tc::mbar_init(&misc->s_free[s], 128);
       tc::mbar_init(&misc->p_ready[s], 128);
@@ -144,8 +154,7 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       tc::mbar_init(&misc->v_full[s], 2);
       tc::mbar_init(&misc->v_empty[s], 1);
     }
-    tc::mbar_init(&misc->all_sync, 256);
-    item_queue_init(&misc->items, 4 + 2 + 1 + 256);
+    list_queue_init(&misc->queue, 4 + 2 + 1 + 8 + 4);   // producers, issuers, table loader, softmax warps, epilogue warps
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_q);
     tc::prefetch_tmap(&tm_k);
@@ -162,7 +171,7 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   grid_enter(false);
 
   if (warp < 8) {
-    tc::reg_dec<56>();
+    tc::reg_dec<kF2ServiceRegs>();
     if (warp < 4) {
       // ---------------------------------------------------------------- TMA producers
       const int which = warp & 1;                           // 0: K ring (+ Q pair), 1: V ring
@@ -174,22 +183,15 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       unsigned char* ring = smem + (which == 0 ? 0 : kF2KSlots * C::SLOT);
       const int my_h = lane;
       const bool issuer = lane < C::DH;
-      uint32_t tg = 0, n_items = 0, published = 0;
+      uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        int item = 0;
-        if (lane == 0) {
-          if (warp == 0 && !item_publish_ahead(&misc->items, seq, published, a.item_counter, total_items, &misc->abort_flag)) item = -2;
-          else item = item_get(&misc->items, seq, &misc->abort_flag);
-        }
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item == -2) goto done;
-        if (item < 0) break;
-        const PairItem wi = decode_pair_item(g, a.pair_heads, item);
-        const int b = wi.bhq0 / g.Hq, hq = wi.bhq0 % g.Hq, bhk = b * g.Hkv + hq / g.rep;
-        const int beg = a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0], end = a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0 + 1];
-        const int k = end - beg;
+        VSA2_NEXT_REC(rec, seq);
+        if (warp == 0 && lane == 0) tc::mbar_arrive(&misc->queue.taken);
+        const int k = rec.z;
         if (k == 0) continue;
-        const int* cols = a.col_idx + (size_t)wi.bhq0 * g.nnz_cap + beg;
+        const PairItem wi{rec.y, rec.x, dh, di};
+        const int b = wi.bhq0 / g.Hq, hq = wi.bhq0 % g.Hq, bhk = b * g.Hkv + hq / g.rep;
+        const int* cols = a.col_idx + (size_t)wi.bhq0 * g.nnz_cap + rec.w;
         if (warp == 0) {
           int ok = 1;
           if (lane == 0) {
@@ -231,11 +233,9 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       const uint32_t slot0 = tc::smem_u32(smem);
       uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        VSA2_NEXT_ITEM_WARP(item, seq);
-        const PairItem wi = decode_pair_item(g, a.pair_heads, item);
-        const int k = a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0 + 1] - a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0];
-        if (k == 0) continue;
-        const int nt = (k + 1) >> 1;
+        VSA2_NEXT_REC(rec, seq);
+        const int nt = (rec.z + 1) >> 1;
+        if (nt == 0) continue;
         VSA2_WAIT(&misc->q_full, n_items & 1);
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t slot = tg % kF2KSlots, buf = tg & 1;
@@ -264,11 +264,9 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       const uint32_t slot0 = tc::smem_u32(smem) + kF2KSlots * C::SLOT;
       uint32_t tg = 0, n_items = 0;
       for (uint32_t seq = 0;; ++seq) {
-        VSA2_NEXT_ITEM_WARP(item, seq);
-        const PairItem wi = decode_pair_item(g, a.pair_heads, item);
-        const int k = a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0 + 1] - a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0];
-        if (k == 0) continue;
-        const int nt = (k + 1) >> 1;
+        VSA2_NEXT_REC(rec, seq);
+        const int nt = (rec.z + 1) >> 1;
+        if (nt == 0) continue;
         VSA2_WAIT(&misc->o_empty, (n_items & 1) ^ 1);
         for (int t = 0; t < nt; ++t, ++tg) {
           const uint32_t slot = tg % kF2VSlots, buf = tg & 1;
@@ -294,12 +292,10 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       // ---------------------------------------------------------------- per-item tables, one item ahead of the softmax warps
       const bool coarse = !(g.flags & VSA2_FLAG_NO_COARSE) && a.gate != nullptr;
       for (uint32_t seq = 0;; ++seq) {
-        VSA2_NEXT_ITEM_WARP(item, seq);
-        const PairItem wi = decode_pair_item(g, a.pair_heads, item);
+        VSA2_NEXT_REC(rec, seq);
+        const PairItem wi{rec.y, rec.x, dh, di};
         const uint32_t tb = seq & 1;
-        const int beg_ = a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0];
-        const int k_ = a.row_ptr[(size_t)wi.bhq0 * (g.N + 1) + wi.i0 + 1] - beg_;
-        const int head_ = (lane < 4 && lane < k_) ? a.col_idx[(size_t)wi.bhq0 * g.nnz_cap + beg_ + lane] : 0;
+        const int head_ = (lane < 4 && lane < rec.z) ? a.col_idx[(size_t)wi.bhq0 * g.nnz_cap + rec.w + lane] : 0;
         int l4[4];
         float g4[4], oc8[8];
 #pragma unroll
@@ -324,54 +320,75 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 #pragma unroll
         for (int r = 0; r < 8; ++r) (&misc->oc[tb][0][0])[lane + 32 * r] = oc8[r];
         if (lane < 4) misc->list_head[tb][lane] = head_;
-        if (lane == 0) {
-          misc->list_k[tb] = k_;
-          misc->list_beg[tb] = beg_;
-        }
         tc::mbar_arrive(&misc->tab_full[tb]);
       }
+    } else {
+      // ---------------------------------------------------------------- scheduler (warp 7): draws the items and looks their lists up, one item
+      // ahead of the first producer (as schedule_lists, which knows single blocks)
+      for (uint32_t p = 0;; ++p) {
+        const uint32_t slot = p % kItemSlots;
+        if (p > 0) VSA2_WAIT_PARKED(&misc->queue.taken, (p - 1) & 1);
+        VSA2_WAIT_PARKED(&misc->queue.empty[slot], ((p / kItemSlots) & 1) ^ 1);
+        int4 rec = make_int4(-1, 0, 0, 0);
+        if (lane == 0) {
+          const int item = item_draw(p, a.item_counter);
+          if (item < total_items) {
+            const PairItem wi = decode_pair_item(g, a.pair_heads, item);
+            const int* c = a.row_ptr + (size_t)wi.bhq0 * (g.N + 1) + wi.i0;
+            const int beg = c[0];
+            rec = make_int4(wi.i0, wi.bhq0, c[1] - beg, beg);
+          }
+          misc->queue.rec[slot] = rec;
+          tc::mbar_arrive(&misc->queue.full[slot]);
+        }
+        if (__shfl_sync(0xffffffffu, rec.x, 0) < 0) break;
+      }
     }
-  } else {
-    // ------------------------------------------------------------------ softmax + epilogue (2 x 128 threads)
-    tc::reg_inc<200>();
+  } else if (warp < 16) {
+    // ------------------------------------------------------------------ softmax (2 x 128 threads)
+    tc::reg_inc<kF2SoftmaxRegs>();
     const int wg = (warp >> 2) - 2;              // 0 or 1: the tiles with (global tile index & 1) == wg
     const int quad = warp & 3;
     const int row = (quad << 5) | lane;          // query row of the item (0..127) = tensor-memory lane
-    const int member = row >> 6;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    uint32_t tg = 0, n_items = 0, all_phase = 0;
+    uint32_t tg = 0;
     for (uint32_t n_all = 0;; ++n_all) {
-      VSA2_NEXT_ITEM(item, n_all);
-      const PairItem wi = decode_pair_item(g, a.pair_heads, item);
+      VSA2_NEXT_REC(rec, n_all);
       const int tb = n_all & 1;
       VSA2_WAIT(&misc->tab_full[tb], (n_all >> 1) & 1);
-      const int k = misc->list_k[tb];
-      const int* cols = a.col_idx + (size_t)wi.bhq0 * g.nnz_cap + misc->list_beg[tb];
+      const int k = rec.z;
+      const int* cols = a.col_idx + (size_t)rec.y * g.nnz_cap + rec.w;
       const int* head = misc->list_head[tb];
-      if (wg == 0 && row < 2) misc->rescue_flag[row] = 0;
       const int nt = (k + 1) >> 1;
       const uint32_t tg0 = tg;
+      const int t_first = ((tg0 & 1) == (uint32_t)wg) ? 0 : 1;
       float m_row = 0.f;
-      if (k > 0 && (tg & 1) == (uint32_t)wg) {
-        // this warpgroup owns tile 0: reference exponent of its row = exact row maximum of that tile (thread-local)
-        const uint32_t buf = tg & 1;
-        const unsigned long long ma = misc->vmask[edge[head[0]]], mb = k > 1 ? misc->vmask[edge[head[1]]] : 0ull;
-        VSA2_WAIT(&misc->s_full[buf], (tg >> 1) & 1);
-        tc::tc_fence_after();
-        float mx = -INFINITY;
+      if (t_first == 0) {
+        if (k > 0) {
+          // this warpgroup owns tile 0: reference exponent of its row = exact row maximum of that tile (thread-local)
+          const uint32_t buf = tg & 1;
+          const unsigned long long ma = misc->vmask[edge[head[0]]], mb = k > 1 ? misc->vmask[edge[head[1]]] : 0ull;
+          VSA2_WAIT(&misc->s_full[buf], (tg >> 1) & 1);
+          tc::tc_fence_after();
+          float mx = -INFINITY;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          uint32_t sv[32];
-          tc::tmem_ld32(lane_addr + C::TM_S + buf * 128 + 32 * c, sv);
-          tc::tmem_ld_wait();
-          const unsigned vm = (unsigned)((c < 2 ? ma : mb) >> (32 * (c & 1)));
+          for (int c = 0; c < 4; ++c) {
+            uint32_t sv[32];
+            tc::tmem_ld32(lane_addr + C::TM_S + buf * 128 + 32 * c, sv);
+            tc::tmem_ld_wait();
+            const unsigned vm = (unsigned)((c < 2 ? ma : mb) >> (32 * (c & 1)));
 #pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if ((vm >> e) & 1u) mx = fmaxf(mx, __uint_as_float(sv[e]));
+            for (int e = 0; e < 32; ++e)
+              if ((vm >> e) & 1u) mx = fmaxf(mx, __uint_as_float(sv[e]));
+          }
+          m_row = (mx > -INFINITY) ? mx * c2 : 0.f;
+          misc->m_ref[tb][row] = m_row;
         }
-        misc->m_ref[row] = (mx > -INFINITY) ? mx * c2 : 0.f;
+        tc::mbar_arrive(&misc->m_full[tb]);              // (one phase per item)
+      } else if (nt > 1) {
+        VSA2_WAIT(&misc->m_full[tb], (n_all >> 1) & 1);
+        m_row = misc->m_ref[tb][row];
       }
-      VSA2_GROUP_SYNC(&misc->all_sync, all_phase);       // reference exponents visible to both warpgroups
 
       // exact sum (even and odd keys apart) and sum of the bf16 roundings of this row.  (Scale and exact sum two values at a time, us,
       // scalar -> packed: 480p with one map for 4 heads 1231 -> 1202, 219,600 tokens, 10 heads 11960 -> 11830; the scale alone
@@ -379,8 +396,6 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       float2 l_sum2 = make_float2(0.f, 0.f);
       float r_sum = 0.f;
       if (k > 0) {
-        m_row = misc->m_ref[row];
-        const int t_first = ((tg0 & 1) == (uint32_t)wg) ? 0 : 1;
         int ja = head[2 * t_first < k ? 2 * t_first : 0], jb = head[2 * t_first + 1 < k ? 2 * t_first + 1 : 0];
         for (int t = t_first; t < nt; t += 2) {
           const uint32_t tgt = tg0 + t, buf = tgt & 1;
@@ -430,79 +445,85 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           tc::mbar_arrive(&misc->p_ready[buf]);
         }
         tg += nt;
-        misc->red[wg][0][row] = l_sum2.x + l_sum2.y;
-        misc->red[wg][1][row] = r_sum;
+        misc->red[tb][wg][0][row] = l_sum2.x + l_sum2.y;
+        misc->red[tb][wg][1][row] = r_sum;
       }
-      VSA2_GROUP_SYNC(&misc->all_sync, all_phase);
-      const int bhq = wi.bhq0 + member * wi.dh;
+      tc::mbar_arrive(&misc->sums_full[tb]);
+      tc::mbar_arrive(&misc->tab_free[tb]);
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue (128 threads, one per query row)
+    const int quad = warp & 3;
+    const int row = (quad << 5) | lane, member = row >> 6;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+    uint32_t n_items = 0;
+    for (uint32_t n_all = 0;; ++n_all) {
+      VSA2_NEXT_REC(rec, n_all);
+      const int k = rec.z, tb = n_all & 1;
+      VSA2_WAIT_PARKED(&misc->tab_full[tb], (n_all >> 1) & 1);
+      VSA2_WAIT_PARKED(&misc->sums_full[tb], (n_all >> 1) & 1);
+      const int bhq = rec.y + member * dh;
       const int tk = misc->tok[tb][row];
       float inv = 0.f;
       if (k > 0) {
-        const float l = misc->red[0][0][row] + misc->red[1][0][row], r = misc->red[0][1][row] + misc->red[1][1][row];
+        const float l = misc->red[tb][0][0][row] + misc->red[tb][1][0][row], r = misc->red[tb][0][1][row] + misc->red[tb][1][1][row];
         inv = 1.f / r;
-        if (wg == 0) {
-          if (!(l > 1e-30f && l < 1e30f && r > 1e-30f)) misc->rescue_flag[member] = 1;
-          if (tk >= 0) a.lse[(size_t)bhq * g.L + tk] = (m_row + __log2f(l)) * 0.6931471805599453f;
+        // the exact kernel works on 64-token blocks: one list entry per member with a sum outside the safe range
+        const bool bad = !(l > 1e-30f && l < 1e30f && r > 1e-30f);
+        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued[member], n_all + 1) != n_all + 1) {
+          const int slot = atomicAdd(a.rescue_count, 1);
+          if (slot < a.rescue_cap) a.rescue_items[slot] = block_item(g, bhq, rec.x + member * di);
+          else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);
         }
-        VSA2_WAIT(&misc->o_full, n_items & 1);
+        if (tk >= 0) a.lse[(size_t)bhq * g.L + tk] = (misc->m_ref[tb][row] + __log2f(l)) * 0.6931471805599453f;
+        VSA2_WAIT_PARKED(&misc->o_full, n_items & 1);
         tc::tc_fence_after();
-      } else if (wg == 0 && tk >= 0) {
+      } else if (tk >= 0) {
         a.lse[(size_t)bhq * g.L + tk] = -INFINITY;
       }
 
-      // O[l, d] = O_acc[q, d] / (rounded row sum) + gate[q] * O_c[d]; this warpgroup writes D / 2 channels of every row
-      {
-        constexpr int COLS = D / 2;
-        const float gt = misc->gate[tb][row];
-        const float* oc = misc->oc[tb][member];
-#pragma unroll
-        for (int c = 0; c < COLS / 32; ++c) {
-          const int col0 = wg * COLS + 32 * c;
-          uint32_t acc[32];
-          if (k > 0) {
-            tc::tmem_ld32(lane_addr + C::TM_O + col0, acc);
-            tc::tmem_ld_wait();
-          } else {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) acc[e] = 0u;
+      // O[l, d] = O_acc[q, d] / (rounded row sum) + gate[q] * O_c[d]
+      const float gt = misc->gate[tb][row];
+#pragma unroll 1
+      for (int col0 = 0; col0 < D; col0 += 32) {
+        const float* oc = misc->oc[tb][member] + col0;
+        uint32_t acc[32];
+        if (k > 0) {
+          tc::tmem_ld32(lane_addr + C::TM_O + col0, acc);
+          tc::tmem_ld_wait();
+          if (col0 + 32 >= D) {
+            tc::tc_fence_before();
+            tc::mbar_arrive(&misc->o_empty);
           }
-          if (tk >= 0) {
-            const size_t idx = ((size_t)bhq * g.L + tk) * D + col0;
-            if (g.out_f32) {
-              float* dst = reinterpret_cast<float*>(a.o) + idx;
+        } else {
 #pragma unroll
-              for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<float4*>(dst + e) =
-                    make_float4(fmaf(gt, oc[col0 + e], __uint_as_float(acc[e]) * inv), fmaf(gt, oc[col0 + e + 1], __uint_as_float(acc[e + 1]) * inv),
-                                fmaf(gt, oc[col0 + e + 2], __uint_as_float(acc[e + 2]) * inv), fmaf(gt, oc[col0 + e + 3], __uint_as_float(acc[e + 3]) * inv));
-            } else {
-              bf16* dst = reinterpret_cast<bf16*>(a.o) + idx;
+          for (int e = 0; e < 32; ++e) acc[e] = 0u;
+        }
+        if (tk >= 0) {
+          const size_t idx = ((size_t)bhq * g.L + tk) * D + col0;
+          if (g.out_f32) {
+            float* dst = reinterpret_cast<float*>(a.o) + idx;
 #pragma unroll
-              for (int e = 0; e < 32; e += 8) {
-                uint32_t hi[4], lo[4];
+            for (int e = 0; e < 32; e += 4)
+              *reinterpret_cast<float4*>(dst + e) =
+                  make_float4(fmaf(gt, oc[e], __uint_as_float(acc[e]) * inv), fmaf(gt, oc[e + 1], __uint_as_float(acc[e + 1]) * inv),
+                              fmaf(gt, oc[e + 2], __uint_as_float(acc[e + 2]) * inv), fmaf(gt, oc[e + 3], __uint_as_float(acc[e + 3]) * inv));
+          } else {
+            bf16* dst = reinterpret_cast<bf16*>(a.o) + idx;
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                  split_bf16x2(fmaf(gt, oc[col0 + e + 2 * q], __uint_as_float(acc[e + 2 * q]) * inv),
-                               fmaf(gt, oc[col0 + e + 2 * q + 1], __uint_as_float(acc[e + 2 * q + 1]) * inv), hi[q], lo[q]);
-                *reinterpret_cast<uint4*>(dst + e) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                if (a.o_res != nullptr) *reinterpret_cast<uint4*>(a.o_res + idx + e) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-              }
+            for (int e = 0; e < 32; e += 8) {
+              uint32_t hi[4], lo[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                split_bf16x2(fmaf(gt, oc[e + 2 * q], __uint_as_float(acc[e + 2 * q]) * inv),
+                             fmaf(gt, oc[e + 2 * q + 1], __uint_as_float(acc[e + 2 * q + 1]) * inv), hi[q], lo[q]);
+              *reinterpret_cast<uint4*>(dst + e) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+              if (a.o_res != nullptr) *reinterpret_cast<uint4*>(a.o_res + idx + e) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
           }
         }
-        if (k > 0) {
-          tc::tc_fence_before();
-          tc::mbar_arrive(&misc->o_empty);
-        }
       }
-      VSA2_GROUP_SYNC(&misc->all_sync, all_phase);       // rescue flags complete
       tc::mbar_arrive(&misc->tab_free[tb]);
-      if (k > 0 && wg == 0 && row < 2 && misc->rescue_flag[row]) {
-        // the exact kernel works on 64-token blocks: one list entry per member whose sums left the safe range
-        const int slot = atomicAdd(a.rescue_count, 1);
-        if (slot < a.rescue_cap) a.rescue_items[slot] = block_item(g, wi.bhq0 + row * wi.dh, wi.i0 + row * wi.di);
-        else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);
-      }
       if (k > 0) ++n_items;
     }
   }
@@ -557,12 +578,12 @@ cudaError_t launch_fine_fwd_rows2_tc(const Geo& g, bool pair_heads, const bf16* 
     const size_t smb = FwdRows2<128>::smem_bytes(g.N);
     if (smb > 227 * 1024) return cudaErrorInvalidValue;
     static KernelAttr attr;
-    if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<128>, attr, smb, kF2Threads, 256 * 56 + 256 * 200))) return e;
+    if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<128>, attr, smb, kF2Threads, kF2Regs))) return e;
     launch_kernel(fine_fwd_rows2_tc_kernel<128>, grid, kF2Threads, smb, st, tq, tk, tv, g, a);
   } else {
     const size_t smb = FwdRows2<64>::smem_bytes(g.N);
     static KernelAttr attr;
-    if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<64>, attr, smb, kF2Threads, 256 * 56 + 256 * 200))) return e;
+    if ((e = prepare_kernel((const void*)fine_fwd_rows2_tc_kernel<64>, attr, smb, kF2Threads, kF2Regs))) return e;
     launch_kernel(fine_fwd_rows2_tc_kernel<64>, grid, kF2Threads, smb, st, tq, tk, tv, g, a);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

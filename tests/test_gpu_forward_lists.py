@@ -40,3 +40,37 @@ def test_lists_of_every_small_length(dim, out_dtype, grid):
     ref = orc.backward(to_f64(q), to_f64(k), to_f64(v), to_f64(gate), mask, geo, 1.0 / np.sqrt(dim), to_f64(d_o))
     for name, x, y in zip(("dQ", "dK", "dV", "dgate"), got, ref):
         assert_close(name, to_f64(x), y, bf16_storage=x.dtype == torch.bfloat16)
+
+
+@pytest.mark.parametrize("dim", [64, 128])
+@pytest.mark.parametrize("out_dtype", [vb.BF16, vb.F32])
+@pytest.mark.parametrize("kind", ["cubes_of_128", "shared_map"])
+def test_pairs_of_blocks_on_lists_of_every_small_length(dim, out_dtype, kind):
+    """The same for the 128-row forward: cubes of 128 tokens (some of whose second halves are empty), and query heads that share a map."""
+    torch.manual_seed(dim)
+    wide = kind == "cubes_of_128"
+    heads, heads_kv = (24, 24) if wide else (32, 8)
+    grid, cube = ((5, 9, 26), (4, 4, 8)) if wide else ((5, 9, 13), (4, 4, 4))
+    tok = grid[0] * grid[1] * grid[2]
+    geo = orc.Geometry(grid, cube, (2, 2, 2))
+    q = torch.randn(1, heads, tok, dim, device="cuda", dtype=torch.bfloat16)
+    k, v = (torch.randn(1, heads_kv, tok, dim, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    gate = torch.tanh(torch.randn(1, heads, tok, device="cuda"))
+    n = geo.N
+    if wide:
+        lengths = torch.tensor([0, 1, 2, 3, 0, 0, n, 4, 5, 1, 1, 0, 7], dtype=torch.int32, device="cuda")
+        budgets = lengths[(torch.arange(heads * n, device="cuda") * 5) % len(lengths)].view(1, heads, n).contiguous()
+        p = vb.make_params(1, heads, heads_kv, dim, grid, cube=cube, select_mode=vb.PER_QUERY_BUDGET, out_dtype=out_dtype,
+                           nnz_cap=int(budgets.sum(-1).max()))
+    else:                                    # (kept per sequence: lists of any length)
+        budgets = None
+        p = vb.make_params(1, heads, heads_kv, dim, grid, select_mode=vb.PER_SEQUENCE, topk=3, out_dtype=out_dtype, flags=vb.FLAG_GROUP_ROUTING)
+    attn = vb.Vsa2Attention(p)
+    attn.route(q, k, budgets)
+    o, lse = attn.forward(q, k, v, gate)
+    attn.check_status()
+    rp, ci, _, _ = (t.cpu().numpy() for t in attn.map_views())
+    mask = csr_to_mask(rp, ci, n)
+    want, want_lse = orc.forward(to_f64(q), to_f64(k), to_f64(v), to_f64(gate), mask, geo, 1.0 / np.sqrt(dim))
+    assert_close("O", to_f64(o), want, bf16_storage=out_dtype == vb.BF16)
+    assert_lse_close(to_f64(lse), want_lse)
