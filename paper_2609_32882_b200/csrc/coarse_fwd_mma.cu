@@ -11,7 +11,7 @@
 // GROUPS = 2: a second group of four warps takes every other tile of keys, and the two results of a row are put together at the end.  For problems
 // whose row blocks are no more than the SMs: one warp per scheduler, which waits for itself (issue slots 39 %), becomes two.  Forward
 // calls, us, one group -> two: 9 x 30 x 45 tokens, 24 heads 371 -> 358; 13 x 27 x 47, 16 heads of 64 channels 350 -> 330; 480p, 12 heads 1548 -> 1512,
-// with a shared map 1198 -> 1169.
+// with a shared map 1198 -> 1169.  The result is no further from 64 bits (288 cubes, 128 channels: 2.53e-4 of its norm against 2.55e-4).
 #include "common.cuh"
 
 namespace vsa2 {
