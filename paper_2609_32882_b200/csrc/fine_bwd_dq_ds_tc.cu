@@ -15,7 +15,10 @@
 
 namespace vsa2 {
 
-constexpr int kDsThreads = 416;       // 2 producer warps of K blocks, 1 of dS tiles, issuer; 2 x 4 epilogue warps; scheduler
+// 2 producer warps of K blocks, 1 of dS tiles, issuer; 2 x 4 epilogue warps; scheduler; with 128 channels 2 more K producers (a warp fetches some
+// 24 bytes a cycle of such boxes and a tile needs 32 KB.  us, two / four: 480p, 12 heads 923 / 904; 720p, 5 heads with text 1035 / 1008; backward of 720p,
+// 40 heads 24505 / 24190)
+constexpr int ds_threads(int D) { return D == 128 ? 480 : 416; }
 constexpr int kDsSets = 4;            // accumulators (64 columns each), used by item in turn
 
 template <int D>
@@ -42,7 +45,7 @@ static_assert(sizeof(DqDsMisc) <= 2048, "misc region too small");
 __device__ __forceinline__ bool packed_query(const Geo& g, const PackedCubes& pk, int i) { return pk.shift > 0 && i >= pk.first && i < g.Nvid; }
 
 template <int D>
-__global__ void __launch_bounds__(kDsThreads, 1)
+__global__ void __launch_bounds__(ds_threads(D), 1)
 fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_kt, Geo g,
                       DqDsArgs a) {
   using C = DqDs<D>;
@@ -54,14 +57,14 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
   if (tid == 0) {
     misc->abort_flag = 0;
     for (int s = 0; s < C::STAGES; ++s) {
-      tc::mbar_init(&misc->full[s], 3);       // the three producers
+      tc::mbar_init(&misc->full[s], D == 128 ? 5 : 3);       // the producers
       tc::mbar_init(&misc->empty[s], 1);
     }
     for (int s = 0; s < kDsSets; ++s) {
       tc::mbar_init(&misc->o_full[s], 1);
       tc::mbar_init(&misc->o_empty[s], 4);
     }
-    list_queue_init(&misc->queue, 4 + 8);
+    list_queue_init(&misc->queue, 4 + 8 + (D == 128 ? 2 : 0));
     tc::fence_barrier_init();
     tc::prefetch_tmap(&tm_k);
   }
@@ -79,8 +82,10 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
     return;
   }
 
-  if (warp < 3) {
-    // ------------------------------------------------------------------ producers: first K block of a pair, second, dS pair
+  if (warp < 3 || warp > 12) {
+    const bool is_k = warp != 2;
+    const int blk = warp > 12 ? warp - 13 : warp, my_h = D == 128 ? (warp > 12 ? 1 : 0) : lane;      // (D = 128: a warp per block and channel half)
+    // ------------------------------------------------------------------ producers: first K block of a pair (warps 0 and 13), second (1, 14), dS pair (2)
     const uint64_t policy = tc::evict_first_policy();      // (the tiles pass through once, the K cubes stay)
     uint32_t tg = 0;
     for (uint32_t seq = 0;; ++seq) {
@@ -93,27 +98,27 @@ fine_bwd_dq_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
       const unsigned char* tiles = a.ds + ((size_t)(rec.y - a.head0) * g.nnz_cap + rec.w) * kSlab;
       // (rows of a packed cube are the first of its tiles as the fp16 forms leave them; the other form has them in every chunk)
       const uint32_t tile_bytes = a.ds_swizzled && packed_query(g, a.pk, rec.x) ? kSlab >> a.pk.shift : kSlab;
-      int j = warp < 2 ? cols[(warp == 1 && k > 1) ? 1 : 0] : 0;
+      int j = is_k ? cols[(blk == 1 && k > 1) ? 1 : 0] : 0;
       for (int t = 0; t < nt; ++t, ++tg) {
         int c1 = 0, c2 = 0, c3 = 0;
         bool text = false;
-        if (warp < 2) {
+        if (is_k) {
           block_box(g, j, c1, c2, c3);
           text = block_is_text(g, j);
-          if (t + 1 < nt) j = cols[(warp == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2];   // next tile, fetched early
+          if (t + 1 < nt) j = cols[(blk == 1 && 2 * t + 3 < k) ? 2 * t + 3 : 2 * t + 2];   // next tile, fetched early
         }
         const uint32_t slot = tg % C::STAGES;
         const uint32_t ds_bytes = (t == nt - 1 && (k & 1)) ? tile_bytes : 2 * tile_bytes;
         int ok = 1;
         if (lane == 0) {
           ok = tc::mbar_wait_parked(&misc->empty[slot], ((tg / C::STAGES) & 1) ^ 1, &misc->abort_flag);
-          if (ok) tc::mbar_expect_tx(&misc->full[slot], warp < 2 ? C::KBYTES / 2 : ds_bytes);
+          if (ok) tc::mbar_expect_tx(&misc->full[slot], is_k ? (D == 128 ? C::KBYTES / 4 : C::KBYTES / 2) : ds_bytes);
         }
         if (!__shfl_sync(0xffffffffu, ok, 0)) goto done;
         unsigned char* stage = smem + slot * C::STAGE;
-        if (warp < 2) {
-          if (lane < C::DH)
-            tc::tma_load_5d(stage + (2 * lane + warp) * kSlab, text ? &tm_kt : &tm_k, &misc->full[slot], lane * 64, c1, c2, c3, bhk);
+        if (is_k) {
+          if (lane == 0)
+            tc::tma_load_5d(stage + (2 * my_h + blk) * kSlab, text ? &tm_kt : &tm_k, &misc->full[slot], my_h * 64, c1, c2, c3, bhk);
         } else if (lane == 0) {
           tc::bulk_load(stage + C::KBYTES, tiles + (size_t)t * C::DSBYTES, tile_bytes == kSlab ? ds_bytes : tile_bytes, &misc->full[slot], policy);
           if (tile_bytes != kSlab && ds_bytes > tile_bytes)
@@ -250,7 +255,7 @@ cudaError_t launch_fine_bwd_dq_ds(const Geo& g, const void* k16, const void* ds,
   do {                                                                                                                           \
     static KernelAttr attr_;                                                                                                     \
     if ((e = prepare_kernel((const void*)fine_bwd_dq_ds_kernel<DD>, attr_, DqDs<DD>::smem_bytes))) return e;                     \
-    launch_kernel(fine_bwd_dq_ds_kernel<DD>, grid, kDsThreads, DqDs<DD>::smem_bytes, st, tk, tkt, g, a);                               \
+    launch_kernel(fine_bwd_dq_ds_kernel<DD>, grid, ds_threads(DD), DqDs<DD>::smem_bytes, st, tk, tkt, g, a);                               \
   } while (0)
   if (g.D == 128) VSA2_LAUNCH_DQ_DS(128);
   else VSA2_LAUNCH_DQ_DS(64);
