@@ -448,6 +448,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
           pk[2 * n + 1] = wb;
         }
         VSA2_WAIT(&misc->p_free[buf], ((tgt >> 1) & 1) ^ 1);
+        tc::tc_fence_after();                     // (the store is not to run ahead of the product that has read the buffer)
         tc::tmem_st_16x128b_x16(lane_addr + C::TM_P + buf * 64, pk);
         tc::tmem_st_wait();
         tc::tc_fence_before();

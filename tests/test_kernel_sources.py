@@ -31,3 +31,29 @@ def test_every_kernel_is_launched_to_overlap_and_waits_for_the_one_before_it():
         kernels = re.findall(r"__global__[^;{]*?\b(\w+_kernel)\s*\([^{;]*\)\s*\{(.*?)\n\}", code, re.S)
         for name, body in kernels:
             assert "grid_enter" in body, (path, name)
+
+
+def test_tensor_memory_is_touched_behind_a_fence_after_every_wait():
+    """A tcgen05 operation (load, store, product) behind a wait for tcgen05 work of other threads needs tcgen05.fence::after_thread_sync between the
+    two: without it the operation may run ahead of what was waited for.  In the order of the source, from each wait to the next operation; waits on
+    vectors in shared memory (`stat_full`) and barriers of a group of threads (VSA2_GROUP_SYNC) stand behind a fence of their own."""
+    token = re.compile(r"(?P<wait>\bVSA2_WAIT\w*\s*\(\s*(?!&misc->stat_full)|\bmbar_wait\w*\s*\()|(?P<fence>\btc_fence_after\s*\()"
+                       r"|(?P<op>\btc::(?:tmem_ld_?\d\w*|tmem_st_\d\w*|mma_ts|mma_ss\w*)\s*\(|\bmma_pair\w*)")
+    operations = 0
+    for path in glob.glob(os.path.join(CSRC, "fine_*.cu")) + [os.path.join(CSRC, "router_tc.cu")]:
+        pending = None
+        for number, line in enumerate(_code_lines(path), 1):
+            for m in token.finditer(line):
+                if m.group("wait"):
+                    pending = number
+                elif m.group("fence"):
+                    pending = None
+                else:
+                    assert pending is None, (path, f"line {number} follows the wait in line {pending} without a fence")
+                    operations += 1
+    assert operations > 50
+
+
+def _code_lines(path):
+    with open(path) as f:
+        return [re.sub(r"//.*", "", line) for line in f]
