@@ -7,11 +7,7 @@
 // 16 x D output accumulators live in registers; a CTA of four warps (64 query rows) shares key / value tiles of 32 pooled
 // tokens, double-buffered with cp.async; P goes from the score accumulators to the A operand of the second product through
 // a warp-private strip of shared memory (the TF32 fragment layouts of C and A differ).  Two CTAs fit an SM.
-//
-// GROUPS = 2: a second group of four warps takes every other tile of keys, and the two results of a row are put together at the end.  For problems
-// whose row blocks are no more than the SMs: one warp per scheduler, which waits for itself (issue slots 39 %), becomes two.  Forward
-// calls, us, one group -> two: 9 x 30 x 45 tokens, 24 heads 371 -> 358; 13 x 27 x 47, 16 heads of 64 channels 350 -> 330; 480p, 12 heads 1548 -> 1512,
-// with a shared map 1198 -> 1169.  The result is no further from 64 bits (288 cubes, 128 channels: 2.53e-4 of its norm against 2.55e-4).
+// A row's operations and their order depend on N alone, so a head's result is the same to the bit whatever other heads and batches are in the call.
 #include "common.cuh"
 
 namespace vsa2 {
@@ -20,7 +16,8 @@ namespace {
 
 constexpr int kCfRows = 64;      // query rows per CTA (16 per warp)
 constexpr int kCfKeys = 32;      // keys per tile
-constexpr int kCfThreads = 128;  // per group of warps
+constexpr int kCfThreads = 128;
+constexpr size_t kCfAlone = 116 * 1024;      // two CTAs of this size do not fit the 228 KB of an SM
 
 template <int D>
 struct CoarseFwdSmem {
@@ -30,10 +27,7 @@ struct CoarseFwdSmem {
   static constexpr size_t k_tile = (size_t)kCfKeys * LDK * sizeof(float);
   static constexpr size_t v_tile = (size_t)kCfKeys * LDV * sizeof(float);
   static constexpr size_t p_strip = (size_t)16 * LDP * sizeof(float);
-  static constexpr size_t bytes = 2 * (k_tile + v_tile) + 4 * p_strip;      // per group of warps
-  // results of the second group's warps, in its tile buffers: [16 rows][D], then maximum and sum of the rows
-  static constexpr int LDO = D + 8;
-  static_assert(4 * 16 * (LDO + 2) * sizeof(float) <= 2 * (k_tile + v_tile), "the result strips lie in the tile buffers");
+  static constexpr size_t bytes = 2 * (k_tile + v_tile) + 4 * p_strip;
 };
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -52,19 +46,12 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// barrier of one group of warps
-template <int GROUPS>
-__device__ __forceinline__ void group_sync(int group) {
-  if constexpr (GROUPS == 1) __syncthreads();
-  else asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kCfThreads) : "memory");
-}
-
 // rows j0 .. j0 + 31 of K_c and V_c (rows beyond the last pooled token repeat it; their scores are masked)
 template <int D>
-__device__ __forceinline__ void issue_tile(float* ks, float* vs, const float* kc, const float* vc, int j0, int N, int tid) {
+__device__ __forceinline__ void issue_tile(float* ks, float* vs, const float* kc, const float* vc, int j0, int N) {
   using S = CoarseFwdSmem<D>;
   constexpr int CH = D / 4;                       // 16-byte chunks per row
-  for (int e = tid; e < kCfKeys * CH; e += kCfThreads) {
+  for (int e = threadIdx.x; e < kCfKeys * CH; e += kCfThreads) {
     const int r = e / CH, c = e % CH;
     const int row = min(j0 + r, N - 1);
     cp_async16(ks + r * S::LDK + c * 4, kc + (size_t)row * D + c * 4);
@@ -72,19 +59,18 @@ __device__ __forceinline__ void issue_tile(float* ks, float* vs, const float* kc
   }
 }
 
-// grid (ceil(N / 64), Hq, batch), 128 threads per group
-template <int D, int GROUPS>
-__global__ void __launch_bounds__(kCfThreads * GROUPS, 2 / GROUPS)
+// grid (ceil(N / 64), Hq, batch), 128 threads
+template <int D>
+__global__ void __launch_bounds__(kCfThreads, 2)
 coarse_fwd_mma_kernel(const float* qc, const float* kc, const float* vc, Geo g,
                       float* __restrict__ oc_hat, float* __restrict__ lse_c) {
   grid_enter();
   using S = CoarseFwdSmem<D>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int group = GROUPS > 1 ? threadIdx.x / kCfThreads : 0, tid = threadIdx.x - group * kCfThreads;
-  float* kbuf = reinterpret_cast<float*>(smem_raw + group * S::bytes);    // [2][32][LDK]
+  float* kbuf = reinterpret_cast<float*>(smem_raw);                       // [2][32][LDK]
   float* vbuf = kbuf + 2 * kCfKeys * S::LDK;                              // [2][32][LDV]
   float* pbuf = vbuf + 2 * kCfKeys * S::LDV;                              // [4 warps][16][LDP]
-  const int warp = tid >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gq = lane >> 2, tq = lane & 3;                                // fragment coordinates of this lane
   const int hq = blockIdx.y, b = blockIdx.z, hk = hq / g.rep;
   const int N = g.N;
@@ -94,8 +80,7 @@ coarse_fwd_mma_kernel(const float* qc, const float* kc, const float* vc, Geo g,
   const int row_lo = blockIdx.x * kCfRows + warp * 16 + gq, row_hi = row_lo + 8;   // this lane's two query rows
   const float sl2 = g.scale * 1.4426950408889634f;                        // scores in log2 units
 
-  const int n_tiles = (N + kCfKeys - 1) / kCfKeys;
-  if (group < n_tiles) issue_tile<D>(kbuf, vbuf, kbase, vbase, group * kCfKeys, N, tid);
+  issue_tile<D>(kbuf, vbuf, kbase, vbase, 0, N);
   cp_async_commit();
 
   // Q fragments of the warp's 16 rows, all D / 8 contraction steps, converted once
@@ -117,19 +102,20 @@ coarse_fwd_mma_kernel(const float* qc, const float* kc, const float* vc, Geo g,
   float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;       // running maximum (log2 units) and sum
   float* pw = pbuf + warp * 16 * S::LDP;
 
-  for (int t = group, n = 0; t < n_tiles; t += GROUPS, ++n) {
+  const int n_tiles = (N + kCfKeys - 1) / kCfKeys;
+  for (int t = 0; t < n_tiles; ++t) {
     const int j0 = t * kCfKeys;
-    const float* ks_ = kbuf + (n & 1) * kCfKeys * S::LDK;
-    const float* vs_ = vbuf + (n & 1) * kCfKeys * S::LDV;
-    if (t + GROUPS < n_tiles) {
-      issue_tile<D>(kbuf + ((n + 1) & 1) * kCfKeys * S::LDK, vbuf + ((n + 1) & 1) * kCfKeys * S::LDV, kbase, vbase,
-                    j0 + GROUPS * kCfKeys, N, tid);
+    const float* ks_ = kbuf + (t & 1) * kCfKeys * S::LDK;
+    const float* vs_ = vbuf + (t & 1) * kCfKeys * S::LDV;
+    if (t + 1 < n_tiles) {
+      issue_tile<D>(kbuf + ((t + 1) & 1) * kCfKeys * S::LDK, vbuf + ((t + 1) & 1) * kCfKeys * S::LDV, kbase, vbase,
+                    j0 + kCfKeys, N);
       cp_async_commit();
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
     }
-    group_sync<GROUPS>(group);               // tile t has landed for every thread
+    __syncthreads();                         // tile t has landed for every thread
 
     // S[16, 32] = Q K^T
     float s[kCfKeys / 8][4];
@@ -200,43 +186,7 @@ coarse_fwd_mma_kernel(const float* qc, const float* kc, const float* vc, Geo g,
         mma_tf32(o[n], pf, to_tf32(vp[0]), to_tf32(vp[4 * S::LDV]));
       }
     }
-    group_sync<GROUPS>(group);               // everyone is done with tile t before its buffer is refilled
-  }
-
-  if constexpr (GROUPS > 1) {                // the second group's maxima, sums and accumulators go through its tile buffers
-    float* strip = reinterpret_cast<float*>(smem_raw + S::bytes) + warp * 16 * (S::LDO + 2);
-    float* stat = strip + 16 * S::LDO;
-    if (group == 1) {
-#pragma unroll
-      for (int n = 0; n < D / 8; ++n) {
-        *reinterpret_cast<float2*>(strip + gq * S::LDO + n * 8 + 2 * tq) = make_float2(o[n][0], o[n][1]);
-        *reinterpret_cast<float2*>(strip + (gq + 8) * S::LDO + n * 8 + 2 * tq) = make_float2(o[n][2], o[n][3]);
-      }
-      if (tq == 0) {
-        stat[gq] = m_lo;
-        stat[gq + 8] = m_hi;
-        stat[16 + gq] = l_lo;
-        stat[16 + gq + 8] = l_hi;
-      }
-    }
-    __syncthreads();
-    if (group == 1) return;
-    const float n_lo = stat[gq], n_hi = stat[gq + 8];                     // (both groups have a tile: more than 32 keys)
-    const float mn_lo = fmaxf(m_lo, n_lo), mn_hi = fmaxf(m_hi, n_hi);
-    const float a_lo = exp2f(m_lo - mn_lo), a_hi = exp2f(m_hi - mn_hi), b_lo = exp2f(n_lo - mn_lo), b_hi = exp2f(n_hi - mn_hi);
-    l_lo = l_lo * a_lo + stat[16 + gq] * b_lo;
-    l_hi = l_hi * a_hi + stat[16 + gq + 8] * b_hi;
-    m_lo = mn_lo;
-    m_hi = mn_hi;
-#pragma unroll
-    for (int n = 0; n < D / 8; ++n) {
-      const float2 x = *reinterpret_cast<const float2*>(strip + gq * S::LDO + n * 8 + 2 * tq);
-      const float2 y = *reinterpret_cast<const float2*>(strip + (gq + 8) * S::LDO + n * 8 + 2 * tq);
-      o[n][0] = o[n][0] * a_lo + x.x * b_lo;
-      o[n][1] = o[n][1] * a_lo + x.y * b_lo;
-      o[n][2] = o[n][2] * a_hi + y.x * b_hi;
-      o[n][3] = o[n][3] * a_hi + y.y * b_hi;
-    }
+    __syncthreads();                         // everyone is done with tile t before its buffer is refilled
   }
 
   const float inv_lo = 1.f / l_lo, inv_hi = 1.f / l_hi;
@@ -264,22 +214,20 @@ cudaError_t launch_coarse_fwd_mma(const Geo& g, const float* qc, const float* kc
   cudaError_t e;
   int sms = 0;
   if ((e = sm_count(&sms)) != cudaSuccess) return e;
-  // a second group of warps where every row block has an SM to itself, and there are keys for it
-  const bool two = (long long)grid.x * grid.y * grid.z <= sms && g.N > kCfKeys;
-#define VSA2_LAUNCH_CF(DD, GG)                                                                                               \
-  do {                                                                                                                       \
-    const size_t smb = GG * CoarseFwdSmem<DD>::bytes;                                                                        \
-    static KernelAttr attr;                                                                                                  \
-    if ((e = prepare_kernel((const void*)coarse_fwd_mma_kernel<DD, GG>, attr, smb))) return e;                               \
-    launch_kernel(coarse_fwd_mma_kernel<DD, GG>, grid, GG * kCfThreads, smb, st, qc, kc, vc, g, oc_hat, lse_c);              \
+  // No more row blocks than SMs: each asks for more than half of an SM's shared memory and so gets an SM to itself.  (CTAs are placed while the
+  // kernel before this one leaves its SMs; two of them came to lie on one SM while others stayed empty.  Forward calls, us, as placed / apart:
+  // 9 x 30 x 45 tokens, 24 heads 363 / 352; 13 x 27 x 47, 16 heads of 64 channels 338 / 321; 480p, 12 heads 1538 / 1511, with a shared map
+  // 1135 / 1120; 720p, 5 heads with text 1732 / 1678.)
+  const size_t least = (long long)grid.x * grid.y * grid.z <= sms ? kCfAlone : 0;
+#define VSA2_LAUNCH_CF(DD)                                                                                       \
+  do {                                                                                                           \
+    const size_t smb = least > CoarseFwdSmem<DD>::bytes ? least : CoarseFwdSmem<DD>::bytes;                      \
+    static KernelAttr attr;                                                                                      \
+    if ((e = prepare_kernel((const void*)coarse_fwd_mma_kernel<DD>, attr, smb))) return e;                       \
+    launch_kernel(coarse_fwd_mma_kernel<DD>, grid, kCfThreads, smb, st, qc, kc, vc, g, oc_hat, lse_c);           \
   } while (0)
-  if (g.D == 128) {
-    if (two) VSA2_LAUNCH_CF(128, 2);
-    else VSA2_LAUNCH_CF(128, 1);
-  } else {
-    if (two) VSA2_LAUNCH_CF(64, 2);
-    else VSA2_LAUNCH_CF(64, 1);
-  }
+  if (g.D == 128) VSA2_LAUNCH_CF(128);
+  else VSA2_LAUNCH_CF(64);
 #undef VSA2_LAUNCH_CF
   return cudaGetLastError();
 }
