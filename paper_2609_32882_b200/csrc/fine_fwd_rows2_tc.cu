@@ -53,7 +53,7 @@ struct FwdRows2Misc {
   ListQueue queue;
   uint32_t tmem_base;
   int abort_flag;
-  uint32_t rescued[2];             // per member: 1 + number of the last item that was handed to the exact kernel
+  uint32_t rescued[2][2];          // by item parity (as in the 64-row kernel), per member: 1 + number of the last item handed to the exact kernel
   unsigned long long vmask[17];    // [table row of a block]: which of its 64 positions hold tokens
   float m_ref[2][128];             // by item parity, per query row: reference exponent (log2 units)
   float red[2][2][2][128];         // [item parity][warpgroup][exact sum | sum of the bf16 roundings][query row]
@@ -131,7 +131,7 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   if (tid == 0) {
     misc->abort_flag = 0;
     misc->vmask[16] = 0ull;
-    misc->rescued[0] = misc->rescued[1] = 0;
+    misc->rescued[0][0] = misc->rescued[0][1] = misc->rescued[1][0] = misc->rescued[1][1] = 0;
     tc::mbar_init(&misc->q_full, 1);
     tc::mbar_init(&misc->q_empty, 1);
     tc::mbar_init(&misc->o_full, 1);
@@ -470,7 +470,7 @@ fine_fwd_rows2_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         inv = 1.f / r;
         // the exact kernel works on 64-token blocks: one list entry per member with a sum outside the safe range
         const bool bad = !(l > 1e-30f && l < 1e30f && r > 1e-30f);
-        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued[member], n_all + 1) != n_all + 1) {
+        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued[tb][member], n_all + 1) != n_all + 1) {
           const int slot = atomicAdd(a.rescue_count, 1);
           if (slot < a.rescue_cap) a.rescue_items[slot] = block_item(g, bhq, rec.x + member * di);
           else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);

@@ -79,7 +79,8 @@ struct FwdRowsMisc {
   uint64_t m_full[2];              // reference exponents of the item with that parity
   uint32_t tmem_base;
   int abort_flag;
-  uint32_t rescued;                // 1 + number of the last item that was handed to the exact kernel
+  // by item parity (the warps are less than two items apart, tab_free sees to that): 1 + number of the last item handed to the exact kernel
+  uint32_t rescued[2];
   // [validity row of a block][lane % 4]: 0 for key columns 8n + 2c + e (n = 0..7, e = 0, 1) that hold tokens, -infinity for the others; added
   // to the exponents.  Row 0 is not looked at; kFrTail: the last text block if it is cut, kFrNone: no token (the block that an odd list repeats)
   alignas(16) float2 bias[18][4][8];
@@ -151,7 +152,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
   }
   if (tid == 0) {
     misc->abort_flag = 0;
-    misc->rescued = 0;
+    misc->rescued[0] = misc->rescued[1] = 0;
     tc::mbar_init(&misc->q_full, 1);
     tc::mbar_init(&misc->q_empty, 128);
     for (int s = 0; s < 2; ++s) {
@@ -529,7 +530,7 @@ fine_fwd_rows_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         }
         // sums outside the safe range (overflow, NaN or total underflow): hand the block to the exact kernel, once
         const bool bad = !(la > 1e-30f && la < 1e30f && ra > 1e-30f) || !(lb > 1e-30f && lb < 1e30f && rb > 1e-30f);
-        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued, n_all + 1) != n_all + 1) {
+        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(&misc->rescued[tb], n_all + 1) != n_all + 1) {
           const int slot = atomicAdd(a.rescue_count, 1);
           if (slot < a.rescue_cap) a.rescue_items[slot] = block_item(g, bhq, rec.x);
           else atomicExch(&a.status->status, VSA2_ERR_UNSUPPORTED);

@@ -54,6 +54,15 @@ def test_tensor_memory_is_touched_behind_a_fence_after_every_wait():
     assert operations > 50
 
 
+def test_forward_kernels_keep_what_their_warps_share_of_an_item_by_its_parity():
+    """Epilogue and softmax warps of the forward kernels are up to one item apart, so nothing that belongs to an item may lie in a single place."""
+    for name in ("fine_fwd_rows_tc.cu", "fine_fwd_rows2_tc.cu"):
+        code = "".join(_code_lines(os.path.join(CSRC, name)))
+        uses = re.findall(r"misc->(m_ref|red|oc|tok|gate|list_head|rescued|tab_full|tab_free|m_full|sums_full)\b(\[\w+\])?", code)
+        assert {u[0] for u in uses} >= {"m_ref", "red", "tok", "rescued"}
+        assert all(index in ("[tb]", "[0]", "[1]", "[s]") for _, index in uses), (name, [u for u in uses if u[1] not in ("[tb]", "[0]", "[1]", "[s]")])
+
+
 def _code_lines(path):
     with open(path) as f:
         return [re.sub(r"//.*", "", line) for line in f]
