@@ -57,7 +57,7 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint64_t* bar, uint32_t par
       : "memory");
   return ok != 0;
 }
-// Bounded waits: they give up after a given time (two seconds at 2 GHz), or as soon as another thread of the CTA has raised *abort_flag, and
+// Bounded waits: they give up after a given time (two seconds), or as soon as another thread of the CTA has raised *abort_flag, and
 // return false then, after raising the flag themselves.
 __device__ __forceinline__ unsigned long long global_timer_ns() {
   unsigned long long t;
@@ -78,21 +78,24 @@ __device__ __forceinline__ bool mbar_wait_ns(uint64_t* bar, uint32_t parity, vol
   *abort_flag = 1;
   return false;
 }
-__device__ __forceinline__ uint32_t clock_lo() {
+// Its low half: 4.3 seconds round.  (Not the SM's clock: a thread that is preempted may go on on another SM, whose counter can be behind.)
+__device__ __forceinline__ uint32_t timer_lo_ns() {
   uint32_t t;
-  asm volatile("mov.u32 %0, %%clock;" : "=r"(t));
+  asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
   return t;
 }
 // The wait of every role, some 45 copies of it in a kernel: what it does not need it does not have.  With a limit in nanoseconds (64 bits), polls
 // counted and the flag looked at now and then, the copies were 4 to 8 KB of a kernel's code, and short lists, whose warps change from
 // one stretch of code to another, wait for the instruction cache.  Whole passes, us, that form / this one: 9 x 30 x 45 tokens, 24 heads 597 / 569;
 // 13 x 27 x 47, 16 heads 1290 / 1248; 480p, 12 heads on 3 5994 / 5911; 720p, 40 heads 38360 / 37990; 219,600 tokens, 10 heads 46860 / 45940.
-constexpr uint32_t kWaitLimitCycles = 0xf0000000u;      // (of a 32-bit clock; polls come far more often than it goes round)
+// (By the SM's clock instead of the timer's low half, us: ragged clip 518 / 521, 13 x 27 x 47 1182 / 1188, 480p 5917 / 5918, 720p 37890 / 37440, 219,600 tokens
+// 46520 / 46760: no difference.)
+constexpr uint32_t kWaitLimitNs = 2000000000u;      // (polls come far more often than the timer's low half goes round)
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   if (mbar_try_wait(bar, parity)) return true;
-  const uint32_t t0 = clock_lo();
+  const uint32_t t0 = timer_lo_ns();
   while (!mbar_try_wait(bar, parity)) {
-    if (*abort_flag || clock_lo() - t0 > kWaitLimitCycles) {
+    if (*abort_flag || timer_lo_ns() - t0 > kWaitLimitNs) {
       *abort_flag = 1;
       return false;
     }
@@ -102,9 +105,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // The same for roles with slack: parked between polls (a slightly later wake-up, no issue slots spent spinning).
 __device__ __forceinline__ bool mbar_wait_parked(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   if (mbar_try_wait(bar, parity)) return true;
-  const uint32_t t0 = clock_lo();
+  const uint32_t t0 = timer_lo_ns();
   while (!mbar_try_wait_parked(bar, parity)) {
-    if (*abort_flag || clock_lo() - t0 > kWaitLimitCycles) {
+    if (*abort_flag || timer_lo_ns() - t0 > kWaitLimitNs) {
       *abort_flag = 1;
       return false;
     }

@@ -63,6 +63,12 @@ def test_forward_kernels_keep_what_their_warps_share_of_an_item_by_its_parity():
         assert all(index in ("[tb]", "[0]", "[1]", "[s]") for _, index in uses), (name, [u for u in uses if u[1] not in ("[tb]", "[0]", "[1]", "[s]")])
 
 
+def test_waits_are_limited_by_a_timer_that_all_sms_share():
+    """%clock counts on one SM; a thread that was preempted may go on on another one, whose count can be behind, and its wait would seem to have run out."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        assert not re.search(r"%clock|\bclock(64)?\s*\(", _code(path)), path
+
+
 def _code_lines(path):
     with open(path) as f:
         return [re.sub(r"//.*", "", line) for line in f]
