@@ -356,11 +356,12 @@ int vsa2_selftest_umma(const vsa2_params* p, const void* q, const void* k, const
 
 /* Diagnostic of the bounded-wait discipline (the paper has no counterpart).  Every device-side wait of the attention
  * kernels gives up after a time limit: the CTA raises an abort flag, all its roles leave, the status word becomes
- * VSA2_ERR_DEVICE_TIMEOUT and tensor memory is released.  This call runs that path alone, in one CTA: one thread waits
- * `limit_us` microseconds (1 .. 100000) on a barrier nothing arrives at, a second thread waits on another barrier with the
- * kernels' own 2 s limit and must be released by the first one's abort flag.  `status` (device int32, caller-zeroed)
- * receives VSA2_ERR_DEVICE_TIMEOUT; `waited_ns` (device uint64, may be NULL) the time the first wait took.  No GPU fault,
- * trap or hang is involved and the context stays usable. */
+ * VSA2_ERR_DEVICE_TIMEOUT and tensor memory is released.  This call runs that path alone, in one CTA, once for each of the
+ * two kinds of waits that the kernels use: one thread waits `limit_us` microseconds (1 .. 100000) on a barrier nothing
+ * arrives at, a second thread waits on another barrier with the kernels' own 2 s limit and must be released by the first
+ * one's abort flag.  `status` (device int32, caller-zeroed) receives VSA2_ERR_DEVICE_TIMEOUT; `waited_ns` (device uint64, may
+ * be NULL) the time the first thread waited, the shorter of the two.  No GPU fault, trap or hang is involved and the context
+ * stays usable. */
 int vsa2_selftest_timeout(uint32_t limit_us, int32_t* status, uint64_t* waited_ns, void* cuda_stream);
 
 /* Host-only diagnostic (no GPU, no CUDA call; the paper has no counterpart): the kernels decode cube and token indices with

@@ -110,11 +110,12 @@ __global__ void __launch_bounds__(128) selftest_kernel(const __grid_constant__ C
 }
 
 // The give-up path of the attention kernels in isolation: a CTA allocates tensor memory, one role waits on an mbarrier
-// that no role ever arrives at, with a limit of `limit_us` microseconds instead of the kernels' 2 s; the wait runs out,
+// that no role ever arrives at -- the kernels' own wait, polling or parked (PARKED) -- with a limit of `limit_us` microseconds instead of 2 s; the wait runs out,
 // the role raises the CTA's abort flag, every thread leaves through the common exit, the status word receives
 // VSA2_ERR_DEVICE_TIMEOUT and the tensor memory is released.  Nothing faults or hangs; the context stays usable.
+template <bool PARKED>
 __global__ void __launch_bounds__(128) selftest_timeout_kernel(unsigned limit_us, int* __restrict__ status,
-                                                               unsigned long long* __restrict__ waited_ns) {
+                                                               unsigned long long* waited_ns) {
   __shared__ __align__(8) uint64_t never, other;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
@@ -136,17 +137,20 @@ __global__ void __launch_bounds__(128) selftest_timeout_kernel(unsigned limit_us
   if (tid == 32) {
     // the role whose producer never shows up
     const unsigned long long t0 = tc::global_timer_ns();
-    const bool ok = tc::mbar_wait_ns(&never, 0, &abort_flag, (unsigned long long)limit_us * 1000ull);
-    if (waited_ns != nullptr) *waited_ns = tc::global_timer_ns() - t0;
+    const uint32_t limit_ns = limit_us * 1000u;
+    const bool ok = PARKED ? tc::mbar_wait_parked(&never, 0, &abort_flag, limit_ns) : tc::mbar_wait(&never, 0, &abort_flag, limit_ns);
+    const unsigned long long waited = tc::global_timer_ns() - t0;
+    if (waited_ns != nullptr) *waited_ns = PARKED && *waited_ns < waited ? *waited_ns : waited;      // (the shorter of the two launches' waits)
     if (ok) atomicExch(status, VSA2_ERR_INVALID_ARG);      // cannot happen: nothing arrives on that barrier
   } else if (tid == 64) {
-    // a second role parked on another barrier: it must leave as soon as the first one has given up (shared abort flag),
+    // a second role on another barrier, in the other kind of wait: it must leave as soon as the first one has given up (shared abort flag),
     // long before its own 2 s limit
-    tc::mbar_wait(&other, 0, &abort_flag);
+    if (PARKED) tc::mbar_wait(&other, 0, &abort_flag);
+    else tc::mbar_wait_parked(&other, 0, &abort_flag);
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (abort_flag && tid == 0) atomicExch(status, VSA2_ERR_DEVICE_TIMEOUT);
+  if (abort_flag && tid == 0) atomicCAS(status, 0, VSA2_ERR_DEVICE_TIMEOUT);      // (what is there already stays)
   if (warp == 0) tc::tmem_dealloc(tmem_base, 128);
 }
 
@@ -176,8 +180,10 @@ extern "C" int64_t vsa2_selftest_divmod(int32_t n_max, int32_t d_min, int32_t d_
 
 extern "C" int vsa2_selftest_timeout(uint32_t limit_us, int32_t* status, uint64_t* waited_ns, void* cuda_stream) {
   if (status == nullptr || limit_us == 0 || limit_us > 100000u) return VSA2_ERR_INVALID_ARG;
-  selftest_timeout_kernel<<<1, 128, 0, reinterpret_cast<cudaStream_t>(cuda_stream)>>>(
-      limit_us, status, reinterpret_cast<unsigned long long*>(waited_ns));
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  unsigned long long* waited = reinterpret_cast<unsigned long long*>(waited_ns);
+  selftest_timeout_kernel<false><<<1, 128, 0, st>>>(limit_us, status, waited);
+  selftest_timeout_kernel<true><<<1, 128, 0, st>>>(limit_us, status, waited);
   return cudaGetLastError() == cudaSuccess ? VSA2_OK : VSA2_ERR_CUDA;
 }
 

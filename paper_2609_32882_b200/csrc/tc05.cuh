@@ -64,38 +64,24 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-__device__ __forceinline__ bool mbar_wait_ns(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                             unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 0u) {
-      if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > limit_ns) break;
-    }
-  }
-  *abort_flag = 1;
-  return false;
-}
 // Its low half: 4.3 seconds round.  (Not the SM's clock: a thread that is preempted may go on on another SM, whose counter can be behind.)
 __device__ __forceinline__ uint32_t timer_lo_ns() {
   uint32_t t;
   asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
   return t;
 }
-// The wait of every role, some 45 copies of it in a kernel: what it does not need it does not have.  With a limit in nanoseconds (64 bits), polls
+// The wait of every role (`limit_ns`: for the self-test, which runs it out), some 45 copies of it in a kernel: what it does not need it does not have.  With a limit in nanoseconds (64 bits), polls
 // counted and the flag looked at now and then, the copies were 4 to 8 KB of a kernel's code, and short lists, whose warps change from
 // one stretch of code to another, wait for the instruction cache.  Whole passes, us, that form / this one: 9 x 30 x 45 tokens, 24 heads 597 / 569;
 // 13 x 27 x 47, 16 heads 1290 / 1248; 480p, 12 heads on 3 5994 / 5911; 720p, 40 heads 38360 / 37990; 219,600 tokens, 10 heads 46860 / 45940.
 // (By the SM's clock instead of the timer's low half, us: ragged clip 518 / 521, 13 x 27 x 47 1182 / 1188, 480p 5917 / 5918, 720p 37890 / 37440, 219,600 tokens
 // 46520 / 46760: no difference.)
 constexpr uint32_t kWaitLimitNs = 2000000000u;      // (polls come far more often than the timer's low half goes round)
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint32_t t0 = timer_lo_ns();
   while (!mbar_try_wait(bar, parity)) {
-    if (*abort_flag || timer_lo_ns() - t0 > kWaitLimitNs) {
+    if (*abort_flag || timer_lo_ns() - t0 > limit_ns) {
       *abort_flag = 1;
       return false;
     }
@@ -103,11 +89,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 // The same for roles with slack: parked between polls (a slightly later wake-up, no issue slots spent spinning).
-__device__ __forceinline__ bool mbar_wait_parked(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool mbar_wait_parked(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint32_t t0 = timer_lo_ns();
   while (!mbar_try_wait_parked(bar, parity)) {
-    if (*abort_flag || timer_lo_ns() - t0 > kWaitLimitNs) {
+    if (*abort_flag || timer_lo_ns() - t0 > limit_ns) {
       *abort_flag = 1;
       return false;
     }

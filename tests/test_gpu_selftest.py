@@ -72,8 +72,8 @@ def test_tma_cube_tiles_and_tcgen05_products(wl, cubes):
 
 
 def test_a_wait_that_runs_out_reports_a_timeout_and_leaves_the_context_usable():
-    """The give-up path of the attention kernels, driven without any fault: a wait on a barrier nothing arrives at runs out
-    after 1 ms, the CTA's second waiting role is released by the shared abort flag, the status word reads
+    """The give-up path of the attention kernels, driven without any fault, in two launches for their two kinds of waits: a wait on a
+    barrier nothing arrives at runs out after 1 ms, the CTA's second waiting role is released by the shared abort flag, the status word reads
     VSA2_ERR_DEVICE_TIMEOUT, tensor memory is handed back -- and an ordinary route + forward right after it succeeds (it
     allocates all 512 tensor-memory columns, so a leaked allocation would make it wait and time out as well)."""
     import time

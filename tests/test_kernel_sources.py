@@ -69,6 +69,15 @@ def test_waits_are_limited_by_a_timer_that_all_sms_share():
         assert not re.search(r"%clock|\bclock(64)?\s*\(", _code(path)), path
 
 
+def test_the_self_test_runs_out_every_wait_that_the_kernels_use():
+    with open(os.path.join(CSRC, "tc05.cuh")) as f:
+        waits = re.findall(r"bool (mbar_wait\w*)\(", f.read())
+    code = _code(os.path.join(CSRC, "selftest.cu"))
+    assert sorted(waits) == ["mbar_wait", "mbar_wait_parked"]
+    for name in waits:
+        assert re.search(rf"\b{name}\(&never, 0, &abort_flag, limit_ns\)", code), name
+
+
 def _code_lines(path):
     with open(path) as f:
         return [re.sub(r"//.*", "", line) for line in f]
