@@ -95,6 +95,8 @@ enum { VSA2_FLAG_FAST_BWD = 4 };      /* round P and dS once to bf16 everywhere,
 enum { VSA2_FLAG_PRECISE_BWD = 8 };   /* bf16 pairs in the dQ pass and in the dK/dV pass, for MHA as well (dQ pass about 15 %, dK/dV
                                          pass about 35 % slower): for maps that keep only a few blocks per row, where the softmax is
                                          sharply peaked and P itself needs the extra bits */
+enum { VSA2_FLAG_SELECT_NO_CLUSTERS = 512 }; /* validation aid for vsa2_route: the selection as it runs in a part of a GPU that has no room
+                                         for a cluster of eight CTAs (the maps are the same) */
 enum { VSA2_FLAG_GROUP_ROUTING = 256 };/* vsa2_route: the query heads of one KV group share one block map ("group head", Sec. 4
                                          ablation): the block scores of the group's heads are added before the TopK, so
                                          the maps written for those heads are identical.  Not with VSA2_PER_QUERY_BUDGET

@@ -23,6 +23,7 @@ FLAG_FAST_BWD = 4
 FLAG_PRECISE_BWD = 8
 FLAG_BF16_COARSE_FWD = 64
 FLAG_GROUP_ROUTING = 256
+FLAG_SELECT_NO_CLUSTERS = 512
 
 OK = 0
 ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE_TOO_SMALL, ERR_MISALIGNED = -1, -2, -3, -4

@@ -382,6 +382,37 @@ cudaError_t prepare_kernel(const void* kernel, KernelAttr& attr, size_t smem, in
   return cudaSuccess;
 }
 
+cudaError_t cluster_room(const void* kernel, ClusterRoom& room, int ctas, int threads, size_t smem, bool* fits) {
+  int dev = 0, clusters = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  const unsigned long long ctx = dev < kMaxDevices ? context_id() : 0;
+  if (ctx != 0) {
+    const unsigned long long k = room.known[dev].load(std::memory_order_relaxed);
+    if (k >> 1 == ctx) {
+      *fits = k & 1;
+      return cudaSuccess;
+    }
+  }
+  if ((e = prepare_kernel(kernel, room.attr, smem)) != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = ctas;
+  cfg.blockDim = threads;
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {(unsigned)ctas, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) {      // (as good as no room; the error is not left behind)
+    clusters = 0;
+    cudaGetLastError();
+  }
+  *fits = clusters > 0;
+  if (ctx != 0) room.known[dev].store(ctx << 1 | (unsigned long long)*fits, std::memory_order_relaxed);
+  return cudaSuccess;
+}
+
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 ProfScope::ProfScope(int kernel_id, cudaStream_t stream) : id(kernel_id), st(stream) {

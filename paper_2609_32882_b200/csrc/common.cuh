@@ -111,6 +111,13 @@ struct KernelAttr {
 // `least_registers`: registers the launch has to allocate over all its threads (kernels that redistribute them wait for ever
 // otherwise), checked with `threads` on the first call
 cudaError_t prepare_kernel(const void* kernel, KernelAttr& attr, size_t smem, int threads = 0, int least_registers = 0);
+// Whether the current context has room for a cluster of `ctas` CTAs of the kernel (a MIG slice or a green context may not have the SMs in one GPC):
+// asked once per context, of the kernel's largest need `smem`, which is allowed it by this
+struct ClusterRoom {
+  KernelAttr attr;
+  std::atomic<unsigned long long> known[kMaxDevices] = {};      // context id << 1 | answer
+};
+cudaError_t cluster_room(const void* kernel, ClusterRoom& room, int ctas, int threads, size_t smem, bool* fits);
 // number of SMs of the current device (looked up once per device)
 cudaError_t sm_count(int* sms);
 

@@ -827,6 +827,7 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, 
 // Route calls, us, the launches above / this: 180 cubes, 12 heads 84 / 59; 288 cubes, 2 heads 79 / 64, 24 heads 183 / 158; 336 cubes, 16
 // heads 180 / 163, 32 heads behind the one-pass router 270 / 229; 384 cubes, 16 heads 204 / 184; 480 cubes, 2 heads 99.6 / 96.3, 32
 // heads 409 / 407; 528 cubes, 2 heads 109 / 111, 32 heads 475 / 481: eight CTAs a head are too few from there on, hence kSelHeadN.
+// Where a context has no room for a cluster (cluster_room) the launches over all heads run at every size.
 // (Below 129 cubes the launches above are nine.  For the maps of the per-row modes, and from bitmaps, a cluster was slower: 480p, 12 heads 264 / 279.)
 // MAPS: the maps are written.  Without: bitmaps, counts and threshold as sel_row_bits_kernel leaves them, for one-pass scores (BAND: as there).
 constexpr int kSelParts = 8, kSelHeadThreads = 512, kSelHeadN = 480;
@@ -1139,20 +1140,20 @@ static void launch_row_topk(const Geo& g, const float* pr, const int* budgets, c
 #undef VSA2_ROW_TOPK
 }
 
-// whether the selection of a head runs in a cluster
-static bool sel_head_runs(const Geo& g) {
-  return g.mode == VSA2_PER_SEQUENCE && g.N <= kSelHeadN;
-}
+// Per sequence, up to kSelHeadN cubes: the selection of the heads in clusters, if the context has room for one of the largest; *done: it was launched
 template <bool BAND, bool MAPS>
 static cudaError_t launch_sel_head(const Geo& g, const float* pr, const SelectScratch& s, int* row_ptr, int* col_idx, int* col_ptr, int* row_idx,
-                                   StatusBlock* status, const Settle& se, cudaStream_t st) {
-  static KernelAttr attr;
-  const size_t smem = (size_t)SelHeadSmem(g.N, s.words).total * 4;
+                                   StatusBlock* status, const Settle& se, cudaStream_t st, bool* done) {
+  *done = false;
+  if (g.mode != VSA2_PER_SEQUENCE || g.N > kSelHeadN || (g.flags & VSA2_FLAG_SELECT_NO_CLUSTERS)) return cudaSuccess;
+  static ClusterRoom room;
   cudaError_t e;
-  if ((e = prepare_kernel((const void*)sel_head_kernel<BAND, MAPS>, attr, smem))) return e;
+  if ((e = cluster_room((const void*)sel_head_kernel<BAND, MAPS>, room, kSelParts, kSelHeadThreads,
+                        (size_t)SelHeadSmem(kSelHeadN, (kSelHeadN + 31) / 32).total * 4, done)) != cudaSuccess || !*done)
+    return e;
   const SelHead a{pr, g.N, s.words, (unsigned)((long long)g.N * g.K), s.state, s.bitmap, s.bitmap_t, s.row_gt, s.row_eq,
                   row_ptr, col_idx, col_ptr, row_idx, g.nnz_cap, status};
-  return launch_kernel(sel_head_kernel<BAND, MAPS>, kSelParts * g.batch * g.Hq, kSelHeadThreads, smem, st, a, se);
+  return launch_kernel(sel_head_kernel<BAND, MAPS>, kSelParts * g.batch * g.Hq, kSelHeadThreads, (size_t)SelHeadSmem(g.N, s.words).total * 4, st, a, se);
 }
 
 // thresholds, counts and (per sequence) bitmaps of all heads; `se.redo`: null, or the flag without which nothing happens
@@ -1163,8 +1164,11 @@ static cudaError_t launch_thresholds(const Geo& g, const float* pr, const int* b
     const long long n_elems = (long long)N * N;
     const unsigned keep = (unsigned)((long long)N * g.K);
     const int* redo = BAND ? nullptr : se.redo;
-    if ((BAND || redo != nullptr) && sel_head_runs(g))
-      return launch_sel_head<BAND, false>(g, pr, s, nullptr, nullptr, nullptr, nullptr, nullptr, se, st);
+    if (BAND || redo != nullptr) {
+      bool done;
+      const cudaError_t e = launch_sel_head<BAND, false>(g, pr, s, nullptr, nullptr, nullptr, nullptr, nullptr, se, st, &done);
+      if (e != cudaSuccess || done) return e;
+    }
     int init_n = BH * 3 * kHistBins;
     launch_kernel(sel_init_kernel, (init_n + 255) / 256, 256, 0, st, s.state, s.hist, BH, keep, redo);
     int chunks = (int)((n_elems + 256 * 16 - 1) / (256 * 16));
@@ -1200,11 +1204,13 @@ cudaError_t launch_select(const Geo& g, const float* pr, const int* budgets, con
   const int BH = g.batch * g.Hq, N = g.N;
   Settle se{};
   se.redo = const_cast<int*>(redo);
-  if (redo == nullptr && sel_head_runs(g))
-    return launch_sel_head<false, true>(g, pr, s, row_ptr, col_idx, col_ptr, row_idx, status, se, st);
+  cudaError_t e;
+  if (redo == nullptr) {
+    bool done;
+    if ((e = launch_sel_head<false, true>(g, pr, s, row_ptr, col_idx, col_ptr, row_idx, status, se, st, &done)) != cudaSuccess || done) return e;
+  }
   const bool per_sequence = g.mode == VSA2_PER_SEQUENCE, small = N <= kSelOneBlockN;
   const bool with_thresholds = small && !per_sequence && redo == nullptr;      // (the block per head finds them itself)
-  cudaError_t e;
   if (!with_thresholds && (e = launch_thresholds<false>(g, pr, budgets, s, se, st)) != cudaSuccess) return e;
   if (small) {
     launch_kernel(sel_maps_kernel, BH, 1024, 0, st, pr, N, s.words, per_sequence, s.state, s.row_gt, s.row_eq, with_thresholds ? nullptr : s.row_tau,

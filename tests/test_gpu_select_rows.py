@@ -110,3 +110,32 @@ def test_heads_whose_selection_runs_in_a_cluster(n, ties):
         vb.vsa2_route(p, q, kk, None, one.map, one.ws_route, scratch=scratch)
         for a, b in zip(maps, one.map_views()):
             assert np.array_equal(a[:, :keep], b[0].cpu().numpy()[:, :keep])
+
+
+@pytest.mark.parametrize("n", [1, 128, 129, 288, 480])
+@pytest.mark.parametrize("ties", [False, True])
+def test_selection_without_room_for_clusters(n, ties):
+    """Contexts without room for a cluster of eight CTAs take the launches over all heads: the same maps, from two-pass and one-pass scores, and
+    within the capacity or not.  (An ordinary context has the room: it needs fewer launches.)"""
+    torch.manual_seed(n)
+    heads, k = 3, min(9, n)
+    q = torch.randn(1, heads, 64 * n, 64, device="cuda", dtype=torch.bfloat16)
+    kk = torch.randn_like(q)
+    if ties:
+        kk[:, 0, : 32 * n] = 0.0
+        q[:, 1] = 0.0
+    scratch = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    for cap in (0, max(1, n * k - 4 * n - 3)):
+        for extra in (None, scratch):
+            maps, launches, status = [], [], []
+            for flags in (0, vb.FLAG_SELECT_NO_CLUSTERS):
+                p = vb.make_params(1, heads, heads, 64, (4, 4, 4 * n), select_mode=vb.PER_SEQUENCE, topk=k, nnz_cap=cap, flags=flags)
+                attn = vb.Vsa2Attention(p)
+                before = vb.vsa2_launch_count()
+                vb.vsa2_route(p, q, kk, None, attn.map, attn.ws_route, scratch=extra)
+                launches.append(vb.vsa2_launch_count() - before)
+                status.append(vb.vsa2_device_status(attn.ws_route))
+                keep = int(attn.map_views()[0].max())
+                maps.append([t[..., : keep if i % 2 else None].clone() for i, t in enumerate(attn.map_views())])
+            assert launches[0] < launches[1] and status[0] == status[1]
+            assert all(torch.equal(a, b) for a, b in zip(*maps))
