@@ -20,7 +20,7 @@ struct RouteLayout {
   int words;
 };
 struct BwdLayout {
-  size_t status, delta, absmax, ds_exp, full, d_oc_hat, delta_c, dqc, dkc, dvc, pooled, total;
+  size_t status, delta, absmax, ds_exp, full, d_oc_hat, dqc, dkc, dvc, pooled, total;
 };
 
 struct Carver {
@@ -140,7 +140,8 @@ RouteLayout route_layout(const Geo& g, bool folded = false) {
   return r;
 }
 
-BwdLayout bwd_layout(const Geo& g) {
+// `of_wide`: a level of a 128-token-cube problem, where dO_c_hat goes through memory in fp32 (else the preprocess leaves it in the pooled region)
+BwdLayout bwd_layout(const Geo& g, bool of_wide) {
   BwdLayout r;
   Carver c;
   const size_t BHq = (size_t)g.batch * g.Hq;
@@ -149,8 +150,7 @@ BwdLayout bwd_layout(const Geo& g) {
   r.absmax = c.take(BHq * (g.N + text_blocks(g)) * sizeof(float2));
   r.ds_exp = c.take((size_t)g.batch * g.Hkv * sizeof(int));
   r.full = c.take(packed_cubes(g, nullptr).shift > 0 ? BHq * (g.N + text_blocks(g)) * sizeof(int) : 0);
-  r.d_oc_hat = c.take(BHq * g.N * g.D * sizeof(float));
-  r.delta_c = c.take(BHq * g.N * sizeof(float));
+  r.d_oc_hat = c.take(of_wide ? BHq * g.N * g.D * sizeof(float) : 0);
   r.dqc = c.take(BHq * g.N * g.D * sizeof(float));
   r.dkc = c.take(BHq * g.N * g.D * sizeof(float));
   r.dvc = c.take(BHq * g.N * g.D * sizeof(float));
@@ -198,15 +198,15 @@ WideFwdLayout wide_fwd_layout(const Geo& g) {
   return r;
 }
 struct WideBwdLayout {
-  BwdLayout narrow;        // status, delta, d_oc_hat, dqc, dkc, dvc at half-cube level (delta_c and pooled unused)
-  BwdLayout cube;          // d_oc_hat, delta_c, dqc, dkc, dvc, pooled at cube level, offsets relative to `cube_base`
+  BwdLayout narrow;        // status, delta, absmax, ds_exp, d_oc_hat, dqc, dkc, dvc at half-cube level (pooled unused)
+  BwdLayout cube;          // d_oc_hat, dqc, dkc, dvc, pooled at cube level, offsets relative to `cube_base`
   size_t cube_base, oc_hat64, ptr64, idx64, cptr64, ridx64, total;
 };
 WideBwdLayout wide_bwd_layout(const Geo& g) {
   const Geo n = narrow_geo(g);
   WideBwdLayout r;
-  r.narrow = bwd_layout(n);
-  r.cube = bwd_layout(g);
+  r.narrow = bwd_layout(n, true);
+  r.cube = bwd_layout(g, true);
   r.cube_base = align_up(r.narrow.pooled, 256);
   Carver c;
   c.off = r.cube_base + r.cube.total;
@@ -245,7 +245,7 @@ size_t route_workspace_bytes(const Geo& g) { return wide_cube(g) ? wide_route_la
 size_t fwd_base_bytes(const Geo& g) {
   return wide_cube(g) ? wide_fwd_layout(g).total : align_up(fwd_pooled_offset() + pooled_layout(g, false).total, 256);
 }
-size_t bwd_base_bytes(const Geo& g) { return wide_cube(g) ? wide_bwd_layout(g).total : align_up(bwd_layout(g).total, 256); }
+size_t bwd_base_bytes(const Geo& g) { return wide_cube(g) ? wide_bwd_layout(g).total : align_up(bwd_layout(g, false).total, 256); }
 size_t fwd_workspace_bytes(const Geo& g) { return fwd_base_bytes(g) + text_map_layout(g, false).total; }
 // fp16 copies of Q and K for the dQ pass (behind the other regions of the backward's workspace)
 bool dq_pass_f16(const Geo& g) { return fine_bwd_dq_uses_f16(g); }
@@ -719,7 +719,7 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   const bool wide = wide_cube(g);
   const Geo n = wide ? narrow_geo(g) : g;
   const WideBwdLayout wl = wide ? wide_bwd_layout(g) : WideBwdLayout();
-  const BwdLayout lay = wide ? wl.narrow : bwd_layout(g);
+  const BwdLayout lay = wide ? wl.narrow : bwd_layout(g, false);
   const BwdLayout cl = wide ? wl.cube : lay;
   void* cube_ws = wide ? at<unsigned char>(workspace, wl.cube_base) : workspace;
   const bf16* qb = reinterpret_cast<const bf16*>(q);
@@ -727,7 +727,7 @@ int vsa2_attn_bwd_scratch(const vsa2_params* p, const void* q, const void* k, co
   const bf16* vb = reinterpret_cast<const bf16*>(v);
   const bf16* dob = reinterpret_cast<const bf16*>(d_o);
   float* delta = at<float>(workspace, lay.delta);
-  float* d_oc_hat = at<float>(workspace, lay.d_oc_hat);
+  float* d_oc_hat = at<float>(workspace, lay.d_oc_hat);      // (128-token cubes)
   float* dqc = at<float>(workspace, lay.dqc);
   float* dkc = at<float>(workspace, lay.dkc);
   float* dvc = at<float>(workspace, lay.dvc);

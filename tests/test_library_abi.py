@@ -73,6 +73,19 @@ def test_backward_workspace_holds_the_fp16_copies_of_the_default_forms():
     assert bwd_bytes(wl, topk=4) == up(plain) + q16 + k16  # rows that keep few blocks: the dK/dV pass stays with its pairs
 
 
+def test_backward_workspace_of_64_token_cubes_is_what_the_kernels_use():
+    """Status, delta, the blocks' maxima, the exponents, three coarse gradients, and the pooled problem's status, inputs and outputs: nothing else (whole cubes, no
+    fp16 copies)."""
+    batch, heads, heads_kv, dim, grid = 2, 6, 3, 64, (8, 12, 20)
+    p = vb.make_params(batch, heads, heads_kv, dim, grid, select_mode=vb.PER_QUERY, topk=4, flags=vb.FLAG_FAST_BWD)
+    n, rows, bq, bk = 30, 8 * 12 * 20, batch * heads, batch * heads_kv
+    pooled_n = (n + 63) // 64                              # blocks of 64 pooled tokens
+    regions = [256, bq * rows * 4, bq * n * 8, bk * 4] + 3 * [bq * n * dim * 4]
+    regions += [256 + 4 * 16384, bq * n * dim * 2] + 2 * [bk * n * dim * 2] + [bq * (pooled_n + 1) * 4, bq * pooled_n ** 2 * 4]
+    regions += [bq * n * dim * 2, bq * n * 4] + 2 * [bk * n * dim * 4]
+    assert vb.vsa2_query_sizes(p).bwd_workspace_bytes == sum((x + 255) // 256 * 256 for x in regions)
+
+
 def test_backward_scratch_is_checked_and_bounded():
     lib = vb._lib()
     p = vb.params_from_workload(syn.CONFIGS[3])                       # 720p, 40 heads, top-64
