@@ -258,3 +258,17 @@ def test_scratch_is_asked_for_again_after_a_shortage():
     got = [take() for _ in range(70)]
     assert attn.route_scratch_bytes == 4096 and all(x.numel() == 4096 for x in got)
     assert take("bwd_scratch_bytes") is None                       # (0 from the start: none is wanted)
+
+
+def test_outputs_have_the_strides_of_a_new_tensor():
+    """Also where an input that counts as contiguous has other strides in its dimensions of size one."""
+    torch = pytest.importorskip("torch")
+    attn = object.__new__(vb.Vsa2Attention)
+    attn.torch, attn.out_torch_dtype = torch, torch.bfloat16
+    plain = torch.zeros(1, 3, 8, 4)
+    for x in (plain, torch.zeros(3, 1, 8, 4).transpose(0, 1), torch.zeros(2, 1, 8, 4).to(memory_format=torch.channels_last),
+              plain.transpose(2, 3), plain.as_subclass(torch.nn.Parameter)):
+        out = attn._empty_like(x, x.device)
+        assert out.stride() == torch.empty(x.shape).stride() and out.dtype == torch.bfloat16 and type(out) is torch.Tensor
+        out = attn._empty_f32(x, x.shape[:-1])
+        assert out.stride() == torch.empty(x.shape[:-1]).stride() and out.dtype == torch.float32 and type(out) is torch.Tensor
