@@ -272,3 +272,20 @@ def test_outputs_have_the_strides_of_a_new_tensor():
         assert out.stride() == torch.empty(x.shape).stride() and out.dtype == torch.bfloat16 and type(out) is torch.Tensor
         out = attn._empty_f32(x, x.shape[:-1])
         assert out.stride() == torch.empty(x.shape[:-1]).stride() and out.dtype == torch.float32 and type(out) is torch.Tensor
+
+
+@pytest.mark.parametrize("missing", [(), ("_cuda_getCurrentRawStream",), ("_cuda_getDevice",)])
+def test_current_stream_without_torchs_private_names(monkeypatch, missing):
+    """The handle comes from torch's internals where both names are there, and from the public call where one is not."""
+    torch = pytest.importorskip("torch")
+
+    class Stream:
+        cuda_stream = 7
+
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 100 + device, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 3, raising=False)
+    for name in missing:
+        monkeypatch.delattr(torch._C, name)
+    assert vb._stream(None) == (7 if missing else 103)
