@@ -82,7 +82,7 @@ struct FwdRowsMisc {
   // by item parity (the warps are less than two items apart, tab_free sees to that): 1 + number of the last item handed to the exact kernel
   uint32_t rescued[2];
   // [validity row of a block][lane % 4]: 0 for key columns 8n + 2c + e (n = 0..7, e = 0, 1) that hold tokens, -infinity for the others; added
-  // to the exponents.  Row 0 is not looked at; kFrTail: the last text block if it is cut, kFrNone: no token (the block that an odd list repeats)
+  // to the scores.  Row 0 is all zeros (read for the whole block of a pair whose other block is cut); kFrTail: the last text block if it is cut, kFrNone: no token (the block that an odd list repeats)
   alignas(16) float2 bias[18][4][8];
   float m_ref[2][64];              // by item parity, per query row: reference exponent (log2 units)
   float red[2][2][2][64];          // [item parity][warpgroup][exact sum | sum of the bf16 roundings][query row]
@@ -656,8 +656,8 @@ cudaError_t launch_fine_fwd_rows_tc(const Geo& g, const bf16* q, const bf16* k, 
   a.rescue_cap = fwd_rescue_capacity();
   const int total = g.batch * g.Hq * g.N;
   const int grid = total < sms ? total : sms;
-  // The softmax warpgroups raise their register count to 200 with the registers the service warpgroups give up
-  // (setmaxnreg); that request would block for ever if the launch allocation were smaller than 128 per thread.
+  // The softmax warpgroups raise their register count to kFrSoftmaxRegs with the registers the service warpgroups give up (setmaxnreg); that request
+  // would block for ever if the launch allocated fewer than kFrRegs, which prepare_kernel checks.
   if (g.D == 128) {
     const size_t smb = FwdRows<128>::smem_bytes(g.N);
     static KernelAttr attr;
