@@ -38,24 +38,21 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the 720p top-64 launch with 40 heads: an
 # 8-head ncu capture of the same kernel times 5 (every head streams its own tensors, so the traffic grows in
 # proportion to the heads; the 40-head launch is too large for a full-set capture).
-NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.505465e9 + 0.293843e9),
-                                # copies of Q and K + dK/dV with the stored dS + dQ from it
-                                "fine_bwd": 5 * ((0.309827e9 + 0.264207e9) + (1.562046e9 + 5.232290e9) + (5.133052e9 + 0.135355e9)),
+NCU_TRAFFIC_BYTES_720P_TOP64 = {"fine_fwd": 5 * (0.499201e9 + 0.293479e9),
+                                # preparation (copies of Q and K) + dK/dV with the stored dS + dQ from it
+                                "fine_bwd": 5 * ((0.333500e9 + 0.273135e9) + (1.552499e9 + 5.231945e9) + (5.133017e9 + 0.134821e9)),
                                 # one-pass router: the parked scores are written and read once
-                                "router_pool": 5 * (0.532343e9 + 0.564607e9)}
+                                "router_pool": 5 * (0.537678e9 + 0.565744e9)}
 
 
 # What ncu shows as the busiest unit of each tensor kernel at 64-token cubes (8-head capture, profiles/): the roofline
 # below is quoted against the tensor peak as the contract asks, these say what actually holds the kernel there.
 NCU_LIMITER = {
-    "fine_fwd": "L2 -> SM read rate: 12.9 TB/s against 11.8 TB/s sustained peak (tensor pipe 82 % active at the half rate of M = 64)",
-    "fine_bwd": "dK/dV: shared-memory data pipe 88 % (tensor-core operand fetches 61 % + thread loads/stores 27 %; tensor pipe 41 %); "
-                "dQ from the stored dS: DRAM 54 % (tensor pipe 33 %)",
-    "router_pool": "instruction issue 71 %, exponential unit 66 % (one ex2 per score)",
+    "fine_fwd": "tensor pipe 95 % active at the half rate of M = 64 (64 query rows per block); the power cap in long runs",
+    "fine_bwd": "dK/dV: shared-memory data pipe 96 % (tensor-core operand fetches 66 % + thread loads/stores 30 %; tensor pipe 44 %); "
+                "dQ from the stored dS: 62 of the 63 bytes a cycle that an SM takes in (DRAM 55 %, tensor pipe 34 %); the power cap in long runs",
+    "router_pool": "instruction issue 67 %, exponential unit 63 % (one ex2 per score)",
 }
-# L2 -> SM read rate that ncu reports as the sustained peak of this part (derived__lts__lts2xbar_bytes.sum.peak_sustained
-# in the 8-head capture of profiles/kernels_720p_8heads_ncu_full.md, where the fine forward itself reads 12.0 TB/s).
-NCU_L2_TO_SM_PEAK_TBS = 11.776
 
 
 def workload(config: int, heads: int = 0, topk: int = 0, grid=None, cube=None, text_len: int = 0) -> syn.Workload:
@@ -515,11 +512,8 @@ def run_ours(args):
         "actual_tflops": executed / (ms_step * 1e-3) / 1e12 * world,
         "fine_fwd": {"ms": kernel_ms["fine_fwd"], "tflops": fine_fwd_tf, "frac_of_sustained_peak": fine_fwd_tf / peak_tf,
                      "frac_of_burst_peak": fine_fwd_tf / pk["bf16_tflops"], "frac_of_nominal_2250": fine_fwd_tf / 2250.0,
-                     "l2_to_sm": {"bytes_per_launch": fwd_tile_bytes, "achieved_tbs": fwd_l2_tbs, "peak_tbs": NCU_L2_TO_SM_PEAK_TBS,
-                                  "frac": fwd_l2_tbs / NCU_L2_TO_SM_PEAK_TBS,
-                                  "what": "K and V tiles of every selected block pair (64 FLOP per byte at D = 128 with 64 query rows per tile); "
-                                          "peak = the sustained L2 -> SM rate ncu reports (at the profiled clock, so a run at a higher "
-                                          "clock can read above 1); with 64-token cubes this rate, not the tensor pipe, bounds the kernel"}},
+                     "l2_to_sm": {"bytes_per_launch": fwd_tile_bytes, "achieved_tbs": fwd_l2_tbs,
+                                  "what": "K and V tiles of every selected block pair (64 FLOP per byte at D = 128 with 64 query rows per tile)"}},
         "kernel_ms": kernel_ms,
         "gate": gate_info,
         "paper_context": "paper reports 8.9x attention speed-up over FlashAttention-3 on one H800 at 220K tokens (not comparable)",
