@@ -271,6 +271,9 @@ __global__ void __launch_bounds__(256) sel_emit_rows_bits_kernel(int N, int word
   }
 }
 
+// Threshold of a row that keeps nothing: above every score as a bit pattern, also one that is not a number.  (Infinity is not: a row of NaNs that
+// keeps nothing then wrote its columns over the lists of the rows behind it.)
+constexpr unsigned kNoEntry = 0xffffffffu;
 // The k-th largest (1 <= k <= entries) of a row that a warp holds in registers, U a lane (0 where there is none), by bisection over the bits
 template <int U>
 __device__ __forceinline__ unsigned row_threshold(const unsigned (&v)[U], int k) {
@@ -317,7 +320,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_warp_kernel(const float* pr,
   for (int u = 0; u < U; ++u) v[u] = u * 32 + lane < N ? src[u * 32 + lane] : 0u;      // (0 is never above a candidate)
   const int asked = budgets ? budgets[o] : K, k = max(0, min(asked, N));
   if (k == 0) {
-    if (lane == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
+    if (lane == 0) { row_tau[o] = __uint_as_float(kNoEntry); row_eq_take[o] = 0; row_cnt[o] = 0; }
     return;
   }
   const unsigned tau = row_threshold<U>(v, k);
@@ -364,7 +367,7 @@ __global__ void __launch_bounds__(256) sel_row_topk_kernel(const float* pr, int 
   const unsigned* src = reinterpret_cast<const unsigned*>(pr) + o * N;
   const int asked = budgets ? budgets[o] : K, k = max(0, min(asked, N));
   if (k == 0) {
-    if (threadIdx.x == 0) { row_tau[o] = INFINITY; row_eq_take[o] = 0; row_cnt[o] = 0; }
+    if (threadIdx.x == 0) { row_tau[o] = __uint_as_float(kNoEntry); row_eq_take[o] = 0; row_cnt[o] = 0; }
     continue;
   }
   if (threadIdx.x == 0) { s_prefix = 0u; s_mask = 0u; s_remaining = (unsigned)k; }
@@ -713,7 +716,7 @@ __global__ void __launch_bounds__(1024) sel_maps_kernel(const float* pr, int N, 
 #pragma unroll
       for (int w = 0; w < W; ++w) v[w] = w * 32 + lane < N ? src[w * 32 + lane] : 0u;
       const int k = max(0, min(budgets ? budgets[base + i] : K, N));
-      const unsigned tau = k > 0 ? row_threshold<W>(v, k) : 0x7f800000u;
+      const unsigned tau = k > 0 ? row_threshold<W>(v, k) : kNoEntry;
       int gt = 0;
 #pragma unroll
       for (int w = 0; w < W; ++w) gt += v[w] > tau;

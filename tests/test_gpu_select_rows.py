@@ -139,3 +139,28 @@ def test_selection_without_room_for_clusters(n, ties):
                 maps.append([t[..., : keep if i % 2 else None].clone() for i, t in enumerate(attn.map_views())])
             assert launches[0] < launches[1] and status[0] == status[1]
             assert all(torch.equal(a, b) for a, b in zip(*maps))
+
+
+@pytest.mark.parametrize("n", [40, 128, 129, 300, 1100, 2100])
+@pytest.mark.parametrize("one_pass", [False, True])
+def test_rows_that_keep_nothing_whatever_their_scores(n, one_pass):
+    """Rows with a budget of none stay empty where their scores are not numbers, and leave the other rows' lists alone."""
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    q, k = (torch.randn(1, 1, 64 * n, 64, device="cuda", generator=gen).bfloat16() for _ in range(2))
+    none = torch.rand(n, device="cuda", generator=gen) < 0.3
+    none[:2] = torch.tensor([True, False], device="cuda")
+    budgets = torch.randint(1, 9, (1, 1, n), device="cuda", generator=gen, dtype=torch.int32)
+    budgets[0, 0, none] = 0
+    cap = int(budgets.sum())
+    p = vb.make_params(1, 1, 1, 64, (4, 4, 4 * n), select_mode=vb.PER_QUERY_BUDGET, nnz_cap=cap)
+    scratch = torch.empty(1 << 29, dtype=torch.uint8, device="cuda") if one_pass else None
+    maps = []
+    for value in (None, float("nan")):
+        if value is not None:
+            q.view(4, 4, n, 4, 64)[:, :, none] = value
+        attn = vb.Vsa2Attention(p)
+        vb.vsa2_route(p, q, k, budgets, attn.map, attn.ws_route, scratch=scratch)
+        assert vb.vsa2_device_status(attn.ws_route) == vb.OK
+        maps.append([t.clone() for t in attn.map_views()])
+    assert int(maps[0][0][0, 0, n]) == cap and int(maps[0][2][0, 0, n]) == cap
+    assert all(torch.equal(a, b) for a, b in zip(*maps))
